@@ -220,3 +220,108 @@ def tolerance(case):
     if kind == "head":          # seen: 2.9e-4 and 7.8e-3
         return {"rel": 1.2e-3, "max": 0.032}
     return {"rel": 1.5e-3, "max": 0.15}     # seen: 3.7e-4 and 3.8e-2
+
+
+# ---- the same results in 64 bits: the chain of products, functions and storage formats, in plain torch
+
+_BF, _C = torch.bfloat16, math.sqrt(0.5)      # both residual coefficients (tau = 1/2)
+
+
+def _q(v, dtype):
+    """The values of v in a storage format (FP8 casts saturate)."""
+    most = {E4: 448.0, E5: 57344.0}.get(dtype)
+    return (v if most is None else v.clamp(-most, most)).to(dtype).double()
+
+
+def _phi_pdf(z):
+    return 0.5 * torch.erfc(-z * math.sqrt(0.5)), torch.exp(-0.5 * z * z) / math.sqrt(2 * math.pi)
+
+
+def _ffn64(X, W1, W2, G, act, grad):
+    T, (d, f) = X.shape[0], W1.shape
+    Xq, W1q, W2q = _q(X, act), _q(W1, act), _q(W2, act)
+    H = d ** -0.5 * (Xq @ W1q)
+    A = _q(1.7009262 * H * _phi_pdf(H)[0], act)
+    R = _q(_C * X + _C * f ** -0.5 * (A @ W2q), _BF)
+    if G is None:
+        return {"R": R}
+    H, Gq = _q(H, _BF), _q(G, grad)
+    P, p = _phi_pdf(H)
+    dH = _q(1.4811144 * (P + H * p) * d ** -0.5 * (Gq @ W2q.T), grad)
+    return {"R": R, "dX": _q(_C * G + _C * f ** -0.5 * (dH @ W1q.T), _BF), "dW1": T ** -0.5 * (Xq.T @ dH), "dW2": T ** -0.5 * (A.T @ Gq)}
+
+
+def _norm64(U, w, c):
+    m = U.mean(1, keepdim=True)
+    s = ((U - m).square().mean(1, keepdim=True) + 1e-5).sqrt()
+    return _q((U - m) / s * w + c, _BF), (U - m) / s, s
+
+
+def _norm_bwd64(xh, s, w, g):
+    gw, b = g * w, g.shape[0] ** -0.5
+    dx = (gw - gw.mean(1, keepdim=True) - xh * (gw * xh).mean(1, keepdim=True)) / s
+    return _q(dx, _BF), b * (g * xh).sum(0), b * g.sum(0)
+
+
+def _encoder64(case, X, Wqkv, Wo, W1, W2, G, ln):
+    ns, s, nh, fused = case["nseq"], case["slen"], case["nhead"], case["fused"]
+    T, d, hd = X.shape[0], X.shape[1], 64
+    act, grad, wide = (E4, E5, _BF) if case["attention"] == "fp8" else (OUTPUTS[case["attention"]],) * 3
+    mid = (lambda v, dt: v) if fused else _q       # the fused kernels keep scores and their gradient unrounded
+
+    def heads(M):
+        return M.reshape(ns, s, nh, hd).transpose(1, 2)
+
+    def rows(H):
+        return H.transpose(1, 2).reshape(T, nh * hd)
+    Xq, Wqkv_q, Wo_q = _q(X, E4), _q(Wqkv, E4), _q(Wo, E4)
+    Q, K, V = (heads(m) for m in _q(d ** -0.5 * (Xq @ Wqkv_q), act).split(d, 1))
+    P = _q(s * torch.softmax(mid(hd ** -0.5 * (Q @ K.transpose(2, 3)), wide), -1), act)
+    C = _q(rows(s ** -0.5 * (P @ V)), E4)
+    U1 = R1 = _q(_C * X + _C * d ** -0.5 * (C @ Wo_q), _BF)
+    if ln:
+        R1, xh1, s1 = _norm64(U1, ln[0], ln[1])
+        F = _ffn64(R1, W1, W2, None, E4, E5)["R"]
+        R, xh2, s2 = _norm64(F, ln[2], ln[3])
+        g2, dw2, dc2 = _norm_bwd64(xh2, s2, ln[2], G)
+        f = _ffn64(R1, W1, W2, g2, E4, E5)
+        g1, dw1, dc1 = _norm_bwd64(xh1, s1, ln[0], f["dX"])
+    else:
+        f = _ffn64(R1, W1, W2, G, E4, E5)
+        R, g1 = f["R"], f["dX"]
+    g1q = _q(g1, E5)
+    dC = heads(_q(d ** -0.5 * (g1q @ Wo_q.T), grad))
+    dP = mid(hd ** -0.5 * (dC @ V.transpose(2, 3)), wide)
+    p = P / s
+    dS = _q(s * p * (dP - (p * dP).sum(-1, keepdim=True)), grad)
+    dQKV = torch.cat([rows(hd ** -0.5 * (dS @ K)), rows(hd ** -0.5 * (dS.transpose(2, 3) @ Q)), rows(s ** -0.5 * (P.transpose(2, 3) @ dC))], 1)
+    dQKV = _q(dQKV if fused else _q(dQKV, grad), E5)
+    out = {"dX": _q(_C * g1 + _C * (3 * d) ** -0.5 * (dQKV @ Wqkv_q.T), _BF), "R": R, "dWqkv": T ** -0.5 * (Xq.T @ dQKV),
+           "dWo": T ** -0.5 * (C.T @ g1q), "dW1": f["dW1"], "dW2": f["dW2"]}
+    if ln:
+        out["dln"] = [dw1, dc1, dw2, dc2]
+    return out
+
+
+def exact(case, seed):
+    """What `run` returns for these inputs, computed in float64 with the path's storage formats between the steps."""
+    kind = case["kind"]
+    s = prepare(dict(case, graph=False), seed)
+    if kind in ("step", "forward"):
+        X, W1, W2, G = (t.double() for t in s["x"])
+        return _ffn64(X, W1, W2, G if kind == "step" else None, *OPERANDS[case["operand"]])
+    if kind == "encoder":
+        return _encoder64(case, *(t.double() for t in s["x"]), [v.double() for v in s["ln"]] if "ln" in s else None)
+    if kind == "linear":
+        b, m, n = case["b"], case["m"], case["n"]
+        x, w, g = (s[k].double() for k in "xwg")
+        out = OUTPUTS[case["out"]]
+        return {"y": _q(m ** -0.5 * (x @ w), out), "dx": _q(n ** -0.5 * (g @ w.T), out), "dw": b ** -0.5 * (x.T @ g)}
+    T, d, v = case["tokens"], case["d"], case["classes"]
+    xq, wq, t = _q(s["x"], E4), _q(s["w"], E4), s["t"].long()[:, None]
+    logits = _q(d ** -0.5 * (xq @ wq), _BF)
+    logp = torch.log_softmax(logits, 1)
+    g = -logp.exp()
+    g.scatter_add_(1, t, torch.ones_like(t, dtype=torch.float64))
+    g = _q(s["beta"] * g, E5)
+    return {"logits": logits, "loss": logp.gather(1, t)[:, 0], "dx": _q(v ** -0.5 * (g @ wq.T), _BF), "dw": T ** -0.5 * (xq.T @ g)}
