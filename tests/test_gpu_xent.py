@@ -62,3 +62,24 @@ def test_softmax_xent_unit_scale_and_bad_targets():
     with pytest.raises(L.UnitScaleError) as e:
         L.us_softmax_xent_bwd(X, t, None, 1.0, torch.empty((rows, s + 8), device="cuda"))
     assert e.value.status == 1
+
+
+# Class counts at the edges of the row kernel's choices: a warp per row up to 512, then 128 ... 1024 threads with 1 to 8
+# (float32: 4) chunks of eight per thread, then rows that are re-read; row ends inside a chunk, with and without an
+# aligned row pitch.
+@pytest.mark.parametrize("cols", [512, 513, 1023, 1025, 4097, 8192, 8193, 16391, 30522, 32768, 32769, 65536, 65541])
+@pytest.mark.parametrize("in_fmt,out_fmt,pad", [("bf16", "e5m2", True), ("fp16", "f32", False), ("f32", "bf16", True)])
+def test_softmax_xent_row_kernel_edges(cols, in_fmt, out_fmt, pad):
+    L, synth = _mods()
+    rows, ld = 3, ((cols + 15) // 16 * 16 if pad else None)
+    x = synth.normal(33, cols, (rows, cols), 2.0)
+    x[1, 5:9] = -np.inf                                               # masked classes
+    t = np.array([0, cols - 1, cols // 2], np.int32)
+    Xt, xv = U.to_device(x, in_fmt, ld), U.values_of(x, in_fmt)
+    tt = torch.from_numpy(t).cuda()
+    out, dX = torch.empty(rows, device="cuda"), U.empty(rows, cols, out_fmt, ld)
+    L.us_softmax_xent_fwd(Xt, tt, out)
+    ref = O.softmax_xent_fwd(xv, t)
+    assert np.abs(out.cpu().numpy() - ref).max() <= 4e-6 * (1 + np.abs(ref).max())
+    L.us_softmax_xent_bwd(Xt, tt, None, 8.0, dX)
+    U.assert_close_stored(dX, O.softmax_xent_bwd(xv, t, np.ones(rows), 8.0), out_fmt, 3e-6 * 8.0, "xent bwd")
