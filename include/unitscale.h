@@ -182,6 +182,10 @@ typedef struct {
   us_mat out;
 } us_linear_call;
 us_status us_linear_group(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, void* stream);
+/* The same launch without those limits, for a training step that issues its GEMMs this way at every size: 16-bit operands
+ * (all calls of a launch the same operand width) and outputs of any size are covered too; US_ERR_UNSUPPORTED remains for a
+ * fused activation, mixed widths and more tiles than the work list holds (2048). */
+us_status us_linear_group_any(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, void* stream);
 
 /*
  * us_ffn_hidden: both GEMMs that end in the hidden layer of the FFN block, as ONE kernel launch.
@@ -209,6 +213,10 @@ us_status us_linear_group(int count, const us_linear_call* calls, void* ws, size
 us_status us_ffn_hidden(const us_mat* X, const us_mat* W1, float alpha, const us_mat* G, const us_mat* W2, float beta_x,
                         float act_in_scale, float act_out_scale, float grad_out_scale, int32_t h_dtype, const us_mat* H,
                         const us_mat* A, const us_mat* dH, void* ws, size_t ws_bytes, void* stream);
+/* The same launch for 16-bit operands too (X, W1, G, W2, A and dH all US_BF16 or all US_F16) and for any b and f. */
+us_status us_ffn_hidden_any(const us_mat* X, const us_mat* W1, float alpha, const us_mat* G, const us_mat* W2, float beta_x,
+                            float act_in_scale, float act_out_scale, float grad_out_scale, int32_t h_dtype, const us_mat* H,
+                            const us_mat* A, const us_mat* dH, void* ws, size_t ws_bytes, void* stream);
 
 /* us_test_ffn_hidden_starved: us_test_linear_fwd_starved for the kernel of us_ffn_hidden (no operand loads, every
  * device-side wait gives up after `wait_limit` polls, 1 .. 65536): the kernel raises the status word, frees its
@@ -310,6 +318,8 @@ typedef enum { US_FN_GELU = 0, US_FN_RELU = 1, US_FN_TANH = 2, US_FN_SIGMOID = 3
  *                  elements.  Every tensor must be free of row padding (ld == cols) and start
  *                  on a 16-byte boundary: US_ERR_UNSUPPORTED / US_ERR_ALIGNMENT otherwise, and
  *                  nothing is launched.  Tensors must not overlap.
+ * us_cast_multi    the same launch with BF16 / F16 destinations allowed (the 16-bit alternative of a step's operands):
+ *                  one rounding of scale[i] * src[i], as us_residual_add with tau = 0 rounds it.
  *
  * Inputs may be F32, BF16 or F16 (us_weighted_add also takes E4M3 / E5M2 inputs: partial results that travelled
  * in 8 bits); outputs any us_dtype (us_cast_fp8, us_cast_fp8_multi: E4M3 or E5M2 only).  0 <= tau <= 1.
@@ -327,6 +337,7 @@ us_status us_weighted_add(int count, const us_mat* src, const float* gamma, floa
 us_status us_cast_fp8(const us_mat* src, float scale, const us_mat* dst, void* stream);
 us_status us_cast_fp8_multi(int count, const us_mat* src, const float* scale, const us_mat* dst,
                             void* stream);
+us_status us_cast_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, void* stream);
 
 /* ------------------------------------------------------------ fused scaled dot-product attention (forward)
  *

@@ -110,14 +110,20 @@ __device__ __forceinline__ MultiChunk multi_locate(const MultiCastArgs& p, int64
   m.e0 = (c - (t ? p.chunk_end[t - 1] : 0)) * kVec;
   m.sdt = p.src_dt[t]; m.ddt = p.dst_dt[t];
   m.src = static_cast<const char*>(p.src[t]) + m.e0 * dtype_size(m.sdt);
-  m.dst = static_cast<char*>(p.dst[t]) + m.e0;                          // FP8: one byte per element
+  m.dst = static_cast<char*>(p.dst[t]) + m.e0 * dtype_size(m.ddt);
   m.scale = p.scale[t];
   m.full = m.e0 + kVec <= p.elems[t];
   return m;
 }
+// The value that is rounded: scale * x; for a 16-bit destination x + 0 x of that product, what us_residual_add with
+// tau = 0 rounds (an infinite x gives NaN there, too).
+__device__ __forceinline__ float multi_value(float x, float scale, int ddt) {
+  const float v = scale * x;
+  return ddt == US_BF16 || ddt == US_F16 ? fmaf(0.f, v, v) : v;
+}
 __device__ __forceinline__ void multi_tail(const MultiCastArgs& p, const MultiChunk& m) {
   for (int64_t i = 0; m.e0 + i < p.elems[m.t]; ++i)
-    store_one(p.dst[m.t], m.ddt, m.e0 + i, m.scale * load_one(p.src[m.t], m.sdt, m.e0 + i));
+    store_one(p.dst[m.t], m.ddt, m.e0 + i, multi_value(load_one(p.src[m.t], m.sdt, m.e0 + i), m.scale, m.ddt));
 }
 
 // Two chunks per thread and iteration, both loaded before either is stored, to keep more loads in flight.
@@ -133,7 +139,7 @@ __global__ void __launch_bounds__(kThreads) multi_cast_kernel(const MultiCastArg
     if (two && m1.full) load_vec<kVec>(m1.src, m1.sdt, b);
     if (m0.full) {
 #pragma unroll
-      for (int i = 0; i < kVec; ++i) a[i] *= m0.scale;
+      for (int i = 0; i < kVec; ++i) a[i] = multi_value(a[i], m0.scale, m0.ddt);
       store_vec<kVec>(m0.dst, m0.ddt, a);
     } else {
       multi_tail(p, m0);
@@ -141,7 +147,7 @@ __global__ void __launch_bounds__(kThreads) multi_cast_kernel(const MultiCastArg
     if (two) {
       if (m1.full) {
 #pragma unroll
-        for (int i = 0; i < kVec; ++i) b[i] *= m1.scale;
+        for (int i = 0; i < kVec; ++i) b[i] = multi_value(b[i], m1.scale, m1.ddt);
         store_vec<kVec>(m1.dst, m1.ddt, b);
       } else {
         multi_tail(p, m1);
@@ -250,7 +256,7 @@ extern "C" us_status us_cast_fp8(const us_mat* src, float scale, const us_mat* d
   return ew_launch<kCast>(src, nullptr, dst, scale, 0.f, stream);
 }
 
-extern "C" us_status us_cast_fp8_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, void* stream) {
+static us_status cast_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, bool to16, void* stream) {
   if (count < 1 || count > kMultiMax || !src || !scale || !dst) return US_ERR_INVALID_ARG;
   MultiCastArgs p{};
   int64_t chunks = 0;
@@ -258,7 +264,8 @@ extern "C" us_status us_cast_fp8_multi(int count, const us_mat* src, const float
   for (int i = 0; i < count; ++i) {
     us_status s = check_ew(&src[i], nullptr, &dst[i]);
     if (s != US_OK) return s;
-    if (dst[i].dtype != US_E4M3 && dst[i].dtype != US_E5M2) return US_ERR_UNSUPPORTED;
+    if (dst[i].dtype != US_E4M3 && dst[i].dtype != US_E5M2 && !(to16 && (dst[i].dtype == US_BF16 || dst[i].dtype == US_F16)))
+      return US_ERR_UNSUPPORTED;
     const int64_t n = src[i].rows * src[i].cols;
     if (n == 0) continue;
     const bool dense = (src[i].ld == src[i].cols && dst[i].ld == dst[i].cols) || src[i].rows == 1;
@@ -278,6 +285,13 @@ extern "C" us_status us_cast_fp8_multi(int count, const us_mat* src, const float
   const int64_t cap = (int64_t)sms * 8;
   multi_cast_kernel<<<(int)(want < cap ? want : cap), kThreads, 0, static_cast<cudaStream_t>(stream)>>>(p);
   return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
+}
+
+extern "C" us_status us_cast_fp8_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, void* stream) {
+  return cast_multi(count, src, scale, dst, false, stream);
+}
+extern "C" us_status us_cast_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, void* stream) {
+  return cast_multi(count, src, scale, dst, true, stream);
 }
 
 extern "C" us_status us_weighted_add(int count, const us_mat* src, const float* gamma, float alpha, const us_mat* out,

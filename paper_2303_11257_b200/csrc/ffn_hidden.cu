@@ -1,22 +1,28 @@
 // us_ffn_hidden: the two GEMMs that end in the hidden layer of the FFN block as ONE launch.
 //
 //   H  = alpha  * X W1                                   (first forward GEMM,          K = d_model)
-//   A  = round_fp8(act_out * gelu(act_in * H))
+//   A  = round(act_out * gelu(act_in * H))               (to FP8, or to the 16-bit operand format)
 //   dA = beta_x * G W2^T                                 (second layer's input gradient, K = d_model)
-//   dH = round_fp8(grad_out * act_in * gelu'(act_in * round16(H)) * dA)
+//   dH = round(grad_out * act_in * gelu'(act_in * round16(H)) * dA)
 //
 // Both GEMMs produce a [tokens x d_ff] matrix and the GELU gradient needs, element for element, the
 // pre-activation H the forward GEMM has just produced.  Launched separately, H travels to memory in
 // 16 bits and back (2 x 2 bytes per element of the largest tensor of the block), and both kernels'
 // stores compete with their operand loads for the SM's memory path.  Here a CTA pair computes, for
 // one 256 x 256 output tile, first X W1 into accumulator 0 and then G W2^T into accumulator 1 of
-// tensor memory.  The sixteen epilogue warps turn accumulator 0 into A (stored as FP8) while the MMAs
-// of accumulator 1 run, keep H -- rounded to the 16-bit format the unfused path stores it in -- in
+// tensor memory.  The sixteen epilogue warps turn accumulator 0 into A while the MMAs
+// of accumulator 1 run (stored as FP8 or in the 16-bit operand format), keep H -- rounded to the 16-bit format the unfused path stores it in -- in
 // registers, and turn accumulator 1 into dH while the next tile's X W1 runs: the two
 // accumulators alternate exactly as two consecutive tiles of gemm_kernel do, and H never leaves the SM
 // (unless the caller asks for a copy).  Results are bit-identical to us_linear_fwd + GELU epilogue
 // followed by us_linear_bwd_x + GELU-gradient epilogue.
+//
+// Bound: tensor pipe, in a long run the power cap.  Measured, separate launches -> this one, us:
+// FP8 8192 x 1024 x 4096: 86 -> 67;  BF16 8192 x 1024 x 4096 (H copy kept): 171 -> 138;  FP8 16384 x 2048 x 8192:
+// 550 -> 507;  FP8 256 x 128 x 512 on 128 x 128 tiles: 12.3 + a launch gap -> 7.2.
 #include <cuda.h>
+
+#include <type_traits>
 
 #include "gemm_kernel.cuh"
 #include "host.h"
@@ -26,13 +32,15 @@ namespace {
 
 constexpr int kHidEW = 16;
 // Shared-memory plan: 32 KB operand stages (this CTA's 128 rows of A and 128 rows of B, 128 bytes of K each) and one
-// 32-row x 64-byte output box per epilogue warp.  The kept pre-activation lives in registers, which leaves room for
-// six stages.
+// output box of 32 rows per epilogue warp, BN / 4 columns of OES bytes.  The kept pre-activation lives in registers,
+// which leaves room for six stages (five with 16-bit outputs and 256-column tiles).
+template <int BN, int OES>
 struct HidSmem {
   static constexpr int kABytes = kBM * kStageKBytes;
   static constexpr int kBBytes = 128 * kStageKBytes;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kEpiWarpBytes = 2048;
+  static constexpr int kRowBytes = BN / 4 * OES;                     // of an output box: 32, 64 or 128
+  static constexpr int kEpiWarpBytes = 32 * kRowBytes;
   static constexpr int kEpiBytes = kHidEW * kEpiWarpBytes;
   static constexpr int kStages = (229376 - kEpiBytes) / kStageBytes;
   static constexpr int kBarrierBytes = 512;
@@ -52,15 +60,22 @@ struct HiddenParams {
   int no_loads;                     // test hook: no operand loads are issued, so that the waits run out
 };
 
-template <bool A_E5, bool D_E5, bool H_BF16>
+// ES: operand bytes per element (1 = FP8, 2 = BF16 / F16).  BN, CG: tiles of 256 x 256 per CTA pair (256, 2), or of
+// 128 x 128 per CTA (128, 1) where the large ones would leave more than half of the pairs idle (hidden_impl).
+// OUT_A, OUT_D: output formats of A and dH (us_dtype).  H_BF16: pre-activation rounded to BF16 (else F16).
+template <int ES, int BN, int CG, int OUT_A, int OUT_D, bool H_BF16>
 __global__ void __launch_bounds__(gemm_threads(kHidEW), 1)
 ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w1,
                   const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_w2,
                   const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_dh,
                   const HiddenParams p) {
-  using S = HidSmem;
-  constexpr int BN = 256, kBK = 128;
-  constexpr uint32_t kChunkBytes = kBK * 128;       // an MN-major operand tile: 128 rows of K x 128 bytes
+  constexpr int kOes = OUT_A == US_E4M3 || OUT_A == US_E5M2 ? 1 : 2;
+  using S = HidSmem<BN, kOes>;
+  static_assert(BN / CG == 128, "128 rows of B per CTA");
+  constexpr int kBK = 128 / ES;                     // K elements per stage
+  constexpr int kTileM = kBM * CG;
+  constexpr int kWarpCols = BN / 4, kSlices = kWarpCols / 32;   // columns of a tile one epilogue warp handles
+  constexpr uint32_t kChunkBytes = kBK * 128;       // a box of an MN-major operand tile: kBK rows of K x 128 bytes
   constexpr uint32_t kTmemCols = 2 * BN;
 
   extern __shared__ uint8_t smem_raw[];
@@ -79,8 +94,8 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 4);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rank = (int)ptx::cluster_ctarank();
-  const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
+  const int rank = CG == 2 ? (int)ptx::cluster_ctarank() : 0;
+  const int pair = blockIdx.x / CG, num_pairs = gridDim.x / CG;      // tile-walking unit: CTA pair or CTA
   const int num_tiles = p.tiles_m * p.tiles_n;
   const int kb1 = (p.K1 + kBK - 1) / kBK, kb2 = (p.K2 + kBK - 1) / kBK;
   // column-major over the tiles: pairs that run side by side share a panel of W1 and of W2
@@ -88,7 +103,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S::kStages; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
-    for (int a = 0; a < 2; ++a) { ptx::mbar_init(acc_full_bar(a), 1); ptx::mbar_init(acc_empty_bar(a), 2 * kHidEW); }
+    for (int a = 0; a < 2; ++a) { ptx::mbar_init(acc_full_bar(a), 1); ptx::mbar_init(acc_empty_bar(a), CG * kHidEW); }
     ptx::mbar_init(drained_bar, 1);
     *abort_flag = 0;
     ptx::mbar_init_fence();
@@ -97,15 +112,18 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     ptx::prefetch_tensormap(&tm_g);
     ptx::prefetch_tensormap(&tm_w2);
   }
-  if (warp == 1) { ptx::tmem_alloc_pair(ptx::smem_addr(const_cast<uint32_t*>(tmem_slot)), kTmemCols); ptx::tmem_relinquish_pair(); }
+  if (warp == 1) {
+    if (CG == 2) { ptx::tmem_alloc_pair(ptx::smem_addr(const_cast<uint32_t*>(tmem_slot)), kTmemCols); ptx::tmem_relinquish_pair(); }
+    else { ptx::tmem_alloc(ptx::smem_addr(const_cast<uint32_t*>(tmem_slot)), kTmemCols); ptx::tmem_relinquish(); }
+  }
   ptx::tc_fence_before_sync();
   __syncthreads();
-  ptx::cluster_sync();
+  if (CG == 2) ptx::cluster_sync();
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer (both CTAs of the pair)
+    // ------------------------------------------------------------ TMA producer (every CTA)
     if (lane == 0) {
       uint32_t issued = 0;
       int stage = 0; uint32_t phase = 0;
@@ -113,7 +131,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       for (int tile = pair; ok && !p.no_loads && tile < num_tiles; tile += num_pairs) {
         int tm, tn;
         tile_mn2(tile, tm, tn);
-        const int m0 = tm * 256 + rank * 128, n0 = tn * 256 + rank * 128;
+        const int m0 = tm * kTileM + rank * 128, n0 = tn * BN + rank * 128;
         for (int sub = 0; ok && sub < 2; ++sub) {
           const int num_kb = sub ? kb2 : kb1;
           for (int kb = 0; kb < num_kb; ++kb) {
@@ -121,14 +139,18 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             if (!ok) break;
             const uint32_t a_dst = smem_base + stage * S::kStageBytes, b_dst = a_dst + S::kABytes;
             const int k0 = kb * kBK;
-            const uint32_t fb = ptx::in_even_cta(full_bar(stage));
-            if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), 2 * S::kStageBytes);
+            const uint32_t fb = CG == 2 ? ptx::in_even_cta(full_bar(stage)) : full_bar(stage);
+            if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), CG * S::kStageBytes);
+            auto load = [&](uint32_t dst, const void* tmap, int x, int y) {
+              if (CG == 2) ptx::tma_load_2d_pair(dst, tmap, fb, x, y); else ptx::tma_load_2d(dst, tmap, fb, x, y);
+            };
             if (sub == 0) {
-              ptx::tma_load_2d_pair(a_dst, &tm_x, fb, k0, m0);      // X  [M x K1], K-major
-              ptx::tma_load_2d_pair(b_dst, &tm_w1, fb, n0, k0);     // W1 [K1 x N], N-major
+              load(a_dst, &tm_x, k0, m0);                           // X  [M x K1], K-major
+#pragma unroll
+              for (int c = 0; c < ES; ++c) load(b_dst + c * kChunkBytes, &tm_w1, n0 + c * kBK, k0);   // W1 [K1 x N], N-major, 128 / ES columns per box
             } else {
-              ptx::tma_load_2d_pair(a_dst, &tm_g, fb, k0, m0);      // G  [M x K2], K-major
-              ptx::tma_load_2d_pair(b_dst, &tm_w2, fb, k0, n0);     // W2 [N x K2], K-major
+              load(a_dst, &tm_g, k0, m0);                           // G  [M x K2], K-major
+              load(b_dst, &tm_w2, k0, n0);                          // W2 [N x K2], K-major
             }
             ++issued;
             if (++stage == S::kStages) { stage = 0; phase ^= 1u; }
@@ -146,7 +168,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer (even CTA)
+    // ------------------------------------------------------------ MMA issuer (even CTA of a pair only)
     if (lane == 0 && rank == 0) {
       int stage = 0; uint32_t phase = 0, local = 0;
       bool ok = true;
@@ -179,37 +201,57 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             for (int k = 0; k < kKSteps; ++k) {
               const uint64_t adesc = ((uint64_t)a_hi << 32) | (a_lo + k * 2u);
               const uint64_t bdesc = ((uint64_t)b_hi << 32) | (b_lo + k * b_step);
-              ptx::mma_ss_pair<true>(d_tmem, adesc, bdesc, idesc, accumulate);
+              if (CG == 2) ptx::mma_ss_pair<ES == 1>(d_tmem, adesc, bdesc, idesc, accumulate);
+              else ptx::mma_ss<ES == 1>(d_tmem, adesc, bdesc, idesc, accumulate);
               accumulate = 1;
             }
-            ptx::mma_commit_pair(empty_bar(stage), 3);
+            if (CG == 2) ptx::mma_commit_pair(empty_bar(stage), 3); else ptx::mma_commit(empty_bar(stage));
             if (++stage == S::kStages) { stage = 0; phase ^= 1u; }
           }
-          if (ok) ptx::mma_commit_pair(acc_full_bar(sub), 3);
+          if (ok) { if (CG == 2) ptx::mma_commit_pair(acc_full_bar(sub), 3); else ptx::mma_commit(acc_full_bar(sub)); }
         }
       }
       if (*abort_flag) {
-        ptx::mma_commit_pair(drained_bar, 1);
+        if (CG == 2) ptx::mma_commit_pair(drained_bar, 1); else ptx::mma_commit(drained_bar);
         for (uint32_t it = 0; it < p.wait_limit && !ptx::mbar_try_wait(drained_bar, 0); ++it) {}
       }
     }
   } else {
     // ------------------------------------------------------------ epilogue warps
-    // Warp (lane quarter q, part) owns 32 rows x 64 columns of the tile; a lane holds one row of them.  The rounded
-    // pre-activation of a tile stays in 32 registers of packed 16-bit pairs (hst) between the two phases; staging
-    // is one FP8 output box of 32 rows x 64 bytes (64-byte swizzle) per warp.
+    // Warp (lane quarter q, part) owns 32 rows x kWarpCols columns of the tile; a lane holds one row of them.  The
+    // rounded pre-activation of a tile stays in registers as packed 16-bit pairs (hst) between the two phases; staging
+    // is one output box of 32 rows per warp, swizzled with the pattern of its row width (32-byte rows: none).
     const int q = warp & 3, part = (warp - 2) >> 2;
     const uint32_t buf_out = epi_base + (warp - 2) * S::kEpiWarpBytes;
-    const uint32_t row64 = (uint32_t)lane * 64u, sw64 = (uint32_t)((lane >> 1) & 3);
+    const uint32_t box_row = (uint32_t)lane * S::kRowBytes;
+    const uint32_t box_sw = S::kRowBytes == 128 ? (uint32_t)(lane & 7) : S::kRowBytes == 64 ? (uint32_t)((lane >> 1) & 3) : 0u;
     const f32x2 s1 = splat2(p.scale1), s2 = splat2(p.scale2), in2 = splat2(p.act_in), os2 = splat2(p.grad_out * p.act_in);
     const float tail_k = fabsf(p.act_in) * (1.0f / kTailRange), act_oi = p.act_out * p.act_in;
 
     auto release_acc = [&](int a) {
       ptx::tc_fence_before_sync();
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive_cluster(ptx::in_even_cta(acc_empty_bar(a)));
+      if (lane == 0) {
+        if (CG == 2) ptx::mbar_arrive_cluster(ptx::in_even_cta(acc_empty_bar(a)));
+        else ptx::mbar_arrive(acc_empty_bar(a));
+      }
     };
-    uint32_t hst[32];
+    // Eight outputs of this lane's row, group g of slice s, into the box: 16-byte chunk c at c ^ box_sw.
+    auto stage_out = [&](auto fmt, const float (&y)[8], uint32_t (&held)[2], int s, int g) {
+      constexpr int F = decltype(fmt)::value;
+      if constexpr (F == US_E4M3 || F == US_E5M2) {
+        const uint32_t lo = cvt_fp8x4<F == US_E5M2>(y[0], y[1], y[2], y[3]);
+        const uint32_t hi = cvt_fp8x4<F == US_E5M2>(y[4], y[5], y[6], y[7]);
+        if ((g & 1) == 0) { held[0] = lo; held[1] = hi; }
+        else ptx::sts128(buf_out + box_row + ((((uint32_t)(2 * s + (g >> 1))) ^ box_sw) << 4), make_uint4(held[0], held[1], lo, hi));
+      } else {
+        uint32_t w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] = F == US_BF16 ? pack_bf16x2(y[2 * k], y[2 * k + 1]) : pack_f16x2(y[2 * k], y[2 * k + 1]);
+        ptx::sts128(buf_out + box_row + ((((uint32_t)(4 * s + g)) ^ box_sw) << 4), make_uint4(w[0], w[1], w[2], w[3]));
+      }
+    };
+    uint32_t hst[16 * kSlices];
     // One 32-column slice s of accumulator 0: scale, keep round16(H), GELU, round, stage.
     auto slice_fwd = [&](const uint32_t (&r)[32], int s) {
       uint32_t held[2];
@@ -225,11 +267,8 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
           hst[16 * s + 4 * g + k] = H_BF16 ? pack_bf16x2(a, b) : pack_f16x2(a, b);
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) gelu_scaled2<true>(x[k], tail_k, act_oi, y[2 * k], y[2 * k + 1]);
-        const uint32_t lo = cvt_fp8x4<A_E5>(y[0], y[1], y[2], y[3]);
-        const uint32_t hi = cvt_fp8x4<A_E5>(y[4], y[5], y[6], y[7]);
-        if ((g & 1) == 0) { held[0] = lo; held[1] = hi; }
-        else ptx::sts128(buf_out + row64 + ((((uint32_t)(2 * s + (g >> 1))) ^ sw64) << 4), make_uint4(held[0], held[1], lo, hi));
+        for (int k = 0; k < 4; ++k) gelu_scaled2<kOes == 1>(x[k], tail_k, act_oi, y[2 * k], y[2 * k + 1]);   // the form the separate launch takes for this output
+        stage_out(std::integral_constant<int, OUT_A>(), y, held, s, g);
       }
     };
     // The same slice of accumulator 1: scale, GELU gradient from the kept pre-activation, round, stage.
@@ -244,10 +283,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
           const float2 h = H_BF16 ? unpack_bf16x2(hst[16 * s + 4 * g + k]) : unpack_f16x2(hst[16 * s + 4 * g + k]);
           unpack2(gelu_grad_scaled2(pack2(h.x, h.y), x, in2, os2), y[2 * k], y[2 * k + 1]);
         }
-        const uint32_t lo = cvt_fp8x4<D_E5>(y[0], y[1], y[2], y[3]);
-        const uint32_t hi = cvt_fp8x4<D_E5>(y[4], y[5], y[6], y[7]);
-        if ((g & 1) == 0) { held[0] = lo; held[1] = hi; }
-        else ptx::sts128(buf_out + row64 + ((((uint32_t)(2 * s + (g >> 1))) ^ sw64) << 4), make_uint4(held[0], held[1], lo, hi));
+        stage_out(std::integral_constant<int, OUT_D>(), y, held, s, g);
       }
     };
 
@@ -256,7 +292,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     for (int tile = pair; ok && tile < num_tiles; tile += num_pairs, ++local) {
       int tm, tn;
       tile_mn2(tile, tm, tn);
-      const int row0 = tm * 256 + rank * 128 + q * 32, n_w = tn * BN + part * 64;
+      const int row0 = tm * kTileM + rank * 128 + q * 32, n_w = tn * BN + part * kWarpCols;
       const bool active = n_w < p.N;                            // warp-uniform
       const uint32_t acc_phase = local & 1u;
 #pragma unroll
@@ -265,25 +301,28 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         ptx::tc_fence_after_sync();
-        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + sub * BN + part * 64;
+        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + sub * BN + part * kWarpCols;
         uint32_t r0[32], r1[32];
         if (active) {
           ptx::tmem_ld_32x32_issue(t_row, r0);
           if (lane == 0) ptx::bulk_wait_group_read<0>();        // earlier stores have read the staging boxes
           __syncwarp();
           ptx::tmem_ld_fence(r0);
-          ptx::tmem_ld_32x32_issue(t_row + 32, r1);
-          if (sub == 0) slice_fwd(r0, 0); else slice_bwd(r0, 0);
-          ptx::tmem_ld_fence(r1);
+          if (kSlices == 2) {
+            ptx::tmem_ld_32x32_issue(t_row + 32, r1);
+            if (sub == 0) slice_fwd(r0, 0); else slice_bwd(r0, 0);
+            ptx::tmem_ld_fence(r1);
+          }
         }
         release_acc(sub);                                       // the values are in registers
         if (active) {
-          if (sub == 0) slice_fwd(r1, 1); else slice_bwd(r1, 1);
+          if (kSlices == 2) { if (sub == 0) slice_fwd(r1, 1); else slice_bwd(r1, 1); }
+          else { if (sub == 0) slice_fwd(r0, 0); else slice_bwd(r0, 0); }
           if (sub == 0 && p.h_ptr != nullptr && row0 + lane < p.M) {
-            // the copy of the rounded pre-activation: this lane's 64 columns, 8 at a time (16 aligned bytes)
+            // the copy of the rounded pre-activation: this lane's columns, 8 at a time (16 aligned bytes)
             uint8_t* dst = p.h_ptr + ((long long)(row0 + lane) * p.h_ld + n_w) * 2;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
+            for (int c = 0; c < 4 * kSlices; ++c) {
               const int col = n_w + 8 * c;
               if (col + 8 <= p.N) {
                 *reinterpret_cast<uint4*>(dst + 16 * c) = make_uint4(hst[4 * c], hst[4 * c + 1], hst[4 * c + 2], hst[4 * c + 3]);
@@ -317,10 +356,10 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 
   ptx::tc_fence_before_sync();
   __syncthreads();
-  ptx::cluster_sync();
+  if (CG == 2) ptx::cluster_sync();
   if (warp == 1) {
     ptx::tc_fence_after_sync();
-    ptx::tmem_dealloc_pair(tmem_base, kTmemCols);
+    if (CG == 2) ptx::tmem_dealloc_pair(tmem_base, kTmemCols); else ptx::tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 
@@ -335,7 +374,7 @@ bool make_tmap(CUtensorMap* tm, const us_mat* m, int es, int box_rows, int box_b
   cuuint32_t box[2] = {(cuuint32_t)(box_bytes / es), (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
   return fn(tm, type, 2, m->ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+            box_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_NONE : box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -348,28 +387,34 @@ bool valid_mat(const us_mat* m) {
 }
 bool is_fp8(int dt) { return dt == US_E4M3 || dt == US_E5M2; }
 
-template <bool A_E5, bool D_E5, bool H_BF16>
-us_status launch_hidden(const CUtensorMap* t, const HiddenParams& p, int grid, cudaStream_t stream) {
-  auto kern = ffn_hidden_kernel<A_E5, D_E5, H_BF16>;
-  constexpr int smem = HidSmem::kTotal;
+template <int ES, int BN, int CG, int OUT_A, int OUT_D, bool H_BF16>
+us_status launch_hidden(const CUtensorMap* t, const HiddenParams& p, int units, cudaStream_t stream) {
+  auto kern = ffn_hidden_kernel<ES, BN, CG, OUT_A, OUT_D, H_BF16>;
+  constexpr int smem = HidSmem<BN, OUT_A == US_E4M3 || OUT_A == US_E5M2 ? 1 : 2>::kTotal;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return US_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = dim3(CG * units);
   cfg.blockDim = dim3(gemm_threads(kHidEW));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[0].val.clusterDim.x = CG; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, t[0], t[1], t[2], t[3], t[4], t[5], p) == cudaSuccess ? US_OK : US_ERR_CUDA;
 }
+template <int ES, int OUT_A, int OUT_D>
+us_status pick_hidden(bool pair, bool h_bf16, const CUtensorMap* t, const HiddenParams& p, int units, cudaStream_t st) {
+  if (pair) return h_bf16 ? launch_hidden<ES, 256, 2, OUT_A, OUT_D, true>(t, p, units, st) : launch_hidden<ES, 256, 2, OUT_A, OUT_D, false>(t, p, units, st);
+  return h_bf16 ? launch_hidden<ES, 128, 1, OUT_A, OUT_D, true>(t, p, units, st) : launch_hidden<ES, 128, 1, OUT_A, OUT_D, false>(t, p, units, st);
+}
 
+// any: 16-bit operands (outputs in the same format) and any size are covered too.
 us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_mat* G, const us_mat* W2, float beta_x,
                       float act_in_scale, float act_out_scale, float grad_out_scale, int h_dtype, const us_mat* H,
                       const us_mat* A, const us_mat* dH, void* ws, size_t ws_bytes, void* stream, uint32_t wait_limit,
-                      int no_loads) {
+                      int no_loads, bool any) {
   if (!valid_mat(X) || !valid_mat(W1) || !valid_mat(G) || !valid_mat(W2) || !valid_mat(A) || !valid_mat(dH)) return US_ERR_INVALID_ARG;
   const bool keep_h = H && H->ptr;
   if (keep_h && !valid_mat(H)) return US_ERR_INVALID_ARG;
@@ -383,17 +428,25 @@ us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_m
   if (!aligned16(X) || !aligned16(W1) || !aligned16(G) || !aligned16(W2) || !aligned16(A) || !aligned16(dH) ||
       (keep_h && !aligned16(H)))
     return US_ERR_ALIGNMENT;
-  if (!(is_fp8(X->dtype) && is_fp8(W1->dtype) && is_fp8(G->dtype) && is_fp8(W2->dtype) && is_fp8(A->dtype) && is_fp8(dH->dtype)))
-    return US_ERR_UNSUPPORTED;
-  if (M <= 128 || N <= 128) return US_ERR_UNSUPPORTED;          // tiles of 256 x 256 only
+  const us_mat* ms[6] = {X, W1, G, W2, A, dH};
+  bool f8 = true, h16 = X->dtype == US_BF16 || X->dtype == US_F16;
+  for (const us_mat* m : ms) { f8 = f8 && is_fp8(m->dtype); h16 = h16 && m->dtype == X->dtype; }
+  if (!f8 && !(any && h16)) return US_ERR_UNSUPPORTED;
+  if (!any && (M <= 128 || N <= 128)) return US_ERR_UNSUPPORTED;
+  const int sms = host::sm_count();
+  if (sms <= 0) return US_ERR_CUDA;
 
+  // The rule of the single launches: 256 x 256 tiles per CTA pair unless they would leave more than half of the pairs idle
+  // (1000 x 528 x 2096, 36 such tiles: 13.0 us with them, 9.5 us with 128 x 128).
+  const bool pair = 4 * ((M + 255) / 256) * ((N + 255) / 256) >= sms;
+  const int tile = pair ? 256 : 128, es = f8 ? 1 : 2, one = f8 ? US_E5M2 : US_BF16;
   HiddenParams p{};
   p.M = (int)M; p.N = (int)N; p.K1 = (int)K1; p.K2 = (int)K2;
-  p.tiles_m = (int)((M + 255) / 256); p.tiles_n = (int)((N + 255) / 256);
+  p.tiles_m = (int)((M + tile - 1) / tile); p.tiles_n = (int)((N + tile - 1) / tile);
   if ((int64_t)p.tiles_m * p.tiles_n >= (1ll << 30)) return US_ERR_UNSUPPORTED;
   p.d_tiles_m = make_fast_div(p.tiles_m);
-  p.idesc1 = make_idesc(X->dtype == US_E5M2, W1->dtype == US_E5M2, false, true, 256, 256);
-  p.idesc2 = make_idesc(G->dtype == US_E5M2, W2->dtype == US_E5M2, false, false, 256, 256);
+  p.idesc1 = make_idesc(X->dtype == one, W1->dtype == one, false, true, tile, tile);
+  p.idesc2 = make_idesc(G->dtype == one, W2->dtype == one, false, false, tile, tile);
   p.scale1 = alpha; p.scale2 = beta_x;
   p.act_in = act_in_scale; p.act_out = act_out_scale; p.grad_out = grad_out_scale;
   p.h_ptr = keep_h ? static_cast<uint8_t*>(H->ptr) : nullptr;
@@ -403,20 +456,21 @@ us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_m
   p.no_loads = no_loads;
 
   CUtensorMap t[6];
-  if (!make_tmap(&t[0], X, 1, 128, 128) || !make_tmap(&t[1], W1, 1, 128, 128) || !make_tmap(&t[2], G, 1, 128, 128) ||
-      !make_tmap(&t[3], W2, 1, 128, 128) || !make_tmap(&t[4], A, 1, 32, 64) || !make_tmap(&t[5], dH, 1, 32, 64))
+  const int out_box = tile / 4 * es;                             // bytes per row of an epilogue warp's output box
+  if (!make_tmap(&t[0], X, es, 128, 128) || !make_tmap(&t[1], W1, es, 128 / es, 128) || !make_tmap(&t[2], G, es, 128, 128) ||
+      !make_tmap(&t[3], W2, es, 128, 128) || !make_tmap(&t[4], A, es, 32, out_box) || !make_tmap(&t[5], dH, es, 32, out_box))
     return US_ERR_CUDA;
 
-  const int sms = host::sm_count();
-  if (sms <= 0) return US_ERR_CUDA;
-  const int tiles = p.tiles_m * p.tiles_n, pairs = sms / 2;
-  const int grid = 2 * (tiles < pairs ? tiles : pairs);
+  const int tiles = p.tiles_m * p.tiles_n, most = pair ? sms / 2 : sms;
+  const int units = tiles < most ? tiles : most;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const bool a5 = A->dtype == US_E5M2, d5 = dH->dtype == US_E5M2, bf = h_dtype == US_BF16;
-  if (!a5 && d5) return bf ? launch_hidden<false, true, true>(t, p, grid, st) : launch_hidden<false, true, false>(t, p, grid, st);
-  if (!a5 && !d5) return bf ? launch_hidden<false, false, true>(t, p, grid, st) : launch_hidden<false, false, false>(t, p, grid, st);
-  if (a5 && d5) return bf ? launch_hidden<true, true, true>(t, p, grid, st) : launch_hidden<true, true, false>(t, p, grid, st);
-  return bf ? launch_hidden<true, false, true>(t, p, grid, st) : launch_hidden<true, false, false>(t, p, grid, st);
+  const bool bf = h_dtype == US_BF16;
+  if (!f8) return X->dtype == US_BF16 ? pick_hidden<2, US_BF16, US_BF16>(pair, bf, t, p, units, st) : pick_hidden<2, US_F16, US_F16>(pair, bf, t, p, units, st);
+  const bool a5 = A->dtype == US_E5M2, d5 = dH->dtype == US_E5M2;
+  if (!a5 && d5) return pick_hidden<1, US_E4M3, US_E5M2>(pair, bf, t, p, units, st);
+  if (!a5 && !d5) return pick_hidden<1, US_E4M3, US_E4M3>(pair, bf, t, p, units, st);
+  if (a5 && d5) return pick_hidden<1, US_E5M2, US_E5M2>(pair, bf, t, p, units, st);
+  return pick_hidden<1, US_E5M2, US_E4M3>(pair, bf, t, p, units, st);
 }
 
 }  // namespace
@@ -427,12 +481,20 @@ extern "C" us_status us_ffn_hidden(const us_mat* X, const us_mat* W1, float alph
                                    int32_t h_dtype, const us_mat* H, const us_mat* A, const us_mat* dH, void* ws,
                                    size_t ws_bytes, void* stream) {
   return us::hidden_impl(X, W1, alpha, G, W2, beta_x, act_in_scale, act_out_scale, grad_out_scale, h_dtype, H, A, dH, ws,
-                         ws_bytes, stream, us::kWaitLimit, 0);
+                         ws_bytes, stream, us::kWaitLimit, 0, false);
+}
+
+extern "C" us_status us_ffn_hidden_any(const us_mat* X, const us_mat* W1, float alpha, const us_mat* G, const us_mat* W2,
+                                       float beta_x, float act_in_scale, float act_out_scale, float grad_out_scale,
+                                       int32_t h_dtype, const us_mat* H, const us_mat* A, const us_mat* dH, void* ws,
+                                       size_t ws_bytes, void* stream) {
+  return us::hidden_impl(X, W1, alpha, G, W2, beta_x, act_in_scale, act_out_scale, grad_out_scale, h_dtype, H, A, dH, ws,
+                         ws_bytes, stream, us::kWaitLimit, 0, true);
 }
 
 extern "C" us_status us_test_ffn_hidden_starved(const us_mat* X, const us_mat* W1, const us_mat* G, const us_mat* W2,
                                                 const us_mat* A, const us_mat* dH, void* ws, size_t ws_bytes,
                                                 uint32_t wait_limit, void* stream) {
   if (wait_limit == 0 || wait_limit > (1u << 16)) return US_ERR_INVALID_ARG;
-  return us::hidden_impl(X, W1, 1.f, G, W2, 1.f, 1.f, 1.f, 1.f, US_BF16, nullptr, A, dH, ws, ws_bytes, stream, wait_limit, 1);
+  return us::hidden_impl(X, W1, 1.f, G, W2, 1.f, 1.f, 1.f, 1.f, US_BF16, nullptr, A, dH, ws, ws_bytes, stream, wait_limit, 1, false);
 }

@@ -2,7 +2,6 @@
 #include <cuda.h>
 
 #include <algorithm>
-#include <vector>
 
 #include "gemm_group.cuh"
 #include "host.h"
@@ -36,7 +35,8 @@ bool is_fp8(int dt) { return dt == US_E4M3 || dt == US_E5M2; }
 struct Shape { int64_t M, N, K; };
 
 // Host checks of one call of the group; US_ERR_UNSUPPORTED for a valid call this launch form does not cover.
-us_status check_call(const us_linear_call* c, Shape* sh) {
+// any: 16-bit operands and outputs of any size are covered too.
+us_status check_call(const us_linear_call* c, bool any, Shape* sh) {
   if (c->op < US_OP_FWD || c->op > US_OP_BWD_W) return US_ERR_INVALID_ARG;
   if (!valid_mat(&c->a) || !valid_mat(&c->b) || !valid_mat(&c->out)) return US_ERR_INVALID_ARG;
   int64_t M, N, K;
@@ -50,7 +50,7 @@ us_status check_call(const us_linear_call* c, Shape* sh) {
   if (!aligned16(&c->a) || !aligned16(&c->b) || !aligned16(&c->out)) return US_ERR_ALIGNMENT;
   if (!(is_fp8(c->a.dtype) && is_fp8(c->b.dtype))) {
     const bool h16 = (c->a.dtype == US_BF16 || c->a.dtype == US_F16) && c->a.dtype == c->b.dtype;
-    return h16 ? US_ERR_UNSUPPORTED : US_ERR_UNSUPPORTED;
+    if (!h16 || !any) return US_ERR_UNSUPPORTED;
   }
   if (c->ep.act != US_ACT_NONE) return c->ep.act < US_ACT_NONE || c->ep.act > US_ACT_SIGMOID_GRAD ? US_ERR_INVALID_ARG : US_ERR_UNSUPPORTED;
   if (c->ep.skip.ptr) {
@@ -59,88 +59,132 @@ us_status check_call(const us_linear_call* c, Shape* sh) {
     if (s->dtype != US_F32 && s->dtype != US_BF16 && s->dtype != US_F16) return US_ERR_UNSUPPORTED;
     if (!aligned16(s)) return US_ERR_ALIGNMENT;
   }
-  if (M <= 128 || N <= 128) return US_ERR_UNSUPPORTED;       // tiles of 256 x 256 only
+  if (!any && (M <= 128 || N <= 128)) return US_ERR_UNSUPPORTED;
   if (M > 4095ll * 256 || N > 4095ll * 256) return US_ERR_UNSUPPORTED;
   sh->M = M; sh->N = N; sh->K = K;
   return US_OK;
 }
 
-struct Item { int prob, tm, tn; int64_t kb; };
+// Deals the tiles of all problems to the units, longest contraction first, each tile to the unit with the least work
+// so far (ties: lowest unit), in a fixed order: the same arguments always give the same work list, and a tile's result
+// never depends on it anyway (one unit, one accumulator).  False if a unit would get more than max_rounds tiles.
+bool deal(GroupParams& g, int es, int tile_m, int bn, int units, int max_rounds) {
+  int order[kGroupMaxProblems];
+  for (int i = 0; i < g.count; ++i) order[i] = i;
+  std::stable_sort(order, order + g.count, [&](int x, int y) { return g.prob[x].K > g.prob[y].K; });
+  uint32_t heap[kGroupMaxUnits];                        // load << 8 | unit, a binary heap with the least on top
+  int filled[kGroupMaxUnits] = {0};
+  for (int u = 0; u < units; ++u) heap[u] = (uint32_t)u;
+  std::fill(g.table, g.table + kGroupMaxItems, -1);
+  const auto more = [](uint32_t x, uint32_t y) { return x > y; };
+  int rounds = 0;
+  const int kbk = 128 / es;
+  for (int o = 0; o < g.count; ++o) {
+    const GroupProblem& P = g.prob[order[o]];
+    const int tiles_m = (P.M + tile_m - 1) / tile_m, tiles_n = (P.N + bn - 1) / bn;
+    const uint32_t cost = (uint32_t)((P.K + kbk - 1) / kbk) + 4;            // K blocks plus a change-over
+    // column-major over the tiles of a problem (neighbours in the list share a B panel) while A stays in L2, bands of
+    // eight tile rows beyond that, as for the single launches
+    const int band = (int64_t)P.M * P.K * es <= (80ll << 20) ? tiles_m : 8;
+    for (int m0 = 0; m0 < tiles_m; m0 += band)
+      for (int tn = 0; tn < tiles_n; ++tn)
+        for (int tm = m0; tm < m0 + band && tm < tiles_m; ++tm) {
+          std::pop_heap(heap, heap + units, more);
+          const uint32_t top = heap[units - 1], unit = top & 0xffu;
+          const int slot = filled[unit] * units + (int)unit;
+          if (filled[unit] >= max_rounds || slot >= kGroupMaxItems || (top >> 8) + cost >= (1u << 24)) return false;
+          g.table[slot] = (order[o] << 28) | (tm << 14) | tn;
+          rounds = std::max(rounds, ++filled[unit]);
+          heap[units - 1] = (((top >> 8) + cost) << 8) | unit;
+          std::push_heap(heap, heap + units, more);
+        }
+  }
+  if (rounds * units > kGroupMaxItems) return false;
+  g.rounds = rounds; g.units = units;
+  return true;
+}
 
-}  // namespace
-}  // namespace us
+template <int ES, int BN, int CG>
+us_status launch_group(const GroupParams& g, cudaStream_t stream) {
+  auto kern = gemm_group_kernel<ES, BN, CG>;
+  constexpr int smem = GemmSmem<BN, CG, kGroupEW>::kTotal;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return US_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CG * g.units);
+  cfg.blockDim = dim3(gemm_threads(kGroupEW));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CG; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, g) == cudaSuccess ? US_OK : US_ERR_CUDA;
+}
 
-using namespace us;
-
-extern "C" us_status us_linear_group(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, void* stream) {
+us_status group_impl(int count, const us_linear_call* calls, bool any, void* ws, size_t ws_bytes, void* stream) {
   if (count < 1 || count > kGroupMaxProblems || !calls) return count >= 1 && calls ? US_ERR_UNSUPPORTED : US_ERR_INVALID_ARG;
   if (!ws || ws_bytes < us_workspace_bytes()) return US_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(ws) % 16) return US_ERR_ALIGNMENT;
   static_assert(sizeof(GroupParams) < 32000, "kernel parameter limit");
-  GroupParams g{};
-  std::vector<Item> items;
+  Shape sh[kGroupMaxProblems];
+  int64_t pair_tiles = 0;
+  bool fp8_out = false;
   for (int i = 0; i < count; ++i) {
-    Shape sh;
-    us_status s = check_call(&calls[i], &sh);
+    us_status s = check_call(&calls[i], any, &sh[i]);
     if (s != US_OK) return s;
+    if (dtype_size(calls[i].a.dtype) != dtype_size(calls[0].a.dtype)) return US_ERR_UNSUPPORTED;   // one operand width per launch
+    pair_tiles += ((sh[i].M + 255) / 256) * ((sh[i].N + 255) / 256);
+    fp8_out = fp8_out || is_fp8(calls[i].out.dtype);
+  }
+  const int sms = host::sm_count();
+  if (sms <= 0) return US_ERR_CUDA;
+  const int es = dtype_size(calls[0].a.dtype);
+  // The rule of the single launches: 256 x 256 tiles per CTA pair unless they would leave more than half of the pairs
+  // idle.  (The 64 columns an epilogue warp of a 128 x 128 tile owns do not fill an FP8 output box, so such calls keep
+  // pair tiles.)
+  const bool pair = fp8_out || 4 * pair_tiles >= sms;
+  const int tile_m = pair ? 256 : 128, bn = pair ? 256 : 128;
+  GroupParams g;
+  g.count = count;
+  for (int i = 0; i < count; ++i) {
     GroupProblem& P = g.prob[i];
     const us_linear_call& c = calls[i];
-    P.M = (int)sh.M; P.N = (int)sh.N; P.K = (int)sh.K;
+    P.M = (int)sh[i].M; P.N = (int)sh[i].N; P.K = (int)sh[i].K;
     P.a_mn = c.op == US_OP_BWD_W; P.b_mn = c.op != US_OP_BWD_X;
-    P.idesc = make_idesc(c.a.dtype == US_E5M2, c.b.dtype == US_E5M2, P.a_mn != 0, P.b_mn != 0, 256, 256);
+    const int one = es == 1 ? US_E5M2 : US_BF16;         // the format the descriptor numbers 1
+    P.idesc = make_idesc(c.a.dtype == one, c.b.dtype == one, P.a_mn != 0, P.b_mn != 0, tile_m, bn);
     P.scale = c.scale;
     P.out_dt = c.out.dtype;
     P.has_skip = c.ep.skip.ptr != nullptr;
     P.skip_dt = P.has_skip ? c.ep.skip.dtype : US_F32;
     P.skip_coef = P.has_skip ? c.ep.skip_coef : 0.f;
     P.out_coef = P.has_skip ? c.ep.out_coef : 1.f;
-    // operand tiles are 128-row x 128-byte boxes in either layout (FP8: 128 elements of K, or of M / N, per row)
-    if (!make_tmap(&P.ta, &c.a, 1, 128) || !make_tmap(&P.tb, &c.b, 1, 128)) return US_ERR_CUDA;
+    if (!make_tmap(&P.ta, &c.a, es, P.a_mn ? 128 / es : 128) || !make_tmap(&P.tb, &c.b, es, P.b_mn ? 128 / es : 128)) return US_ERR_CUDA;
     if (!make_tmap(&P.tout, &c.out, dtype_size(c.out.dtype), 32)) return US_ERR_CUDA;
     P.tskip = P.tout;
     if (P.has_skip && !make_tmap(&P.tskip, &c.ep.skip, dtype_size(c.ep.skip.dtype), 32)) return US_ERR_CUDA;
-    const int tiles_m = (int)((sh.M + 255) / 256), tiles_n = (int)((sh.N + 255) / 256);
-    const int64_t kb = (sh.K + 127) / 128;
-    // column-major over the tiles of a problem: neighbours in the list share a B panel
-    for (int tn = 0; tn < tiles_n; ++tn)
-      for (int tm = 0; tm < tiles_m; ++tm) items.push_back({i, tm, tn, kb});
   }
-  const int sms = host::sm_count();
-  if (sms <= 0) return US_ERR_CUDA;
-  int pairs = sms / 2;
-  if (pairs > kGroupMaxPairs) pairs = kGroupMaxPairs;
-  if ((int)items.size() < pairs) pairs = (int)items.size();
-  // Longest first, each tile to the pair with the least work so far (ties: lowest pair), in a fixed order: the same
-  // arguments always give the same work list, and a tile's result never depends on it anyway (one pair, one accumulator).
-  std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return a.kb > b.kb; });
-  std::vector<int64_t> load(pairs, 0);
-  std::vector<int> filled(pairs, 0);
-  for (int i = 0; i < kGroupMaxRounds * kGroupMaxPairs; ++i) g.table[i] = -1;
-  int rounds = 0;
-  for (const Item& it : items) {
-    int best = 0;
-    for (int p = 1; p < pairs; ++p)
-      if (load[p] < load[best]) best = p;
-    if (filled[best] >= kGroupMaxRounds) return US_ERR_UNSUPPORTED;      // too many tiles per pair for the work list
-    g.table[filled[best] * pairs + best] = (it.prob << 24) | (it.tm << 12) | it.tn;
-    load[best] += it.kb + 4;                                            // a tile costs its K blocks plus a change-over
-    rounds = std::max(rounds, ++filled[best]);
+  int units = std::min(pair ? sms / 2 : sms, kGroupMaxUnits);
+  if (!pair || pair_tiles < units) {
+    int64_t tiles = 0;
+    for (int i = 0; i < count; ++i) tiles += ((sh[i].M + tile_m - 1) / tile_m) * ((sh[i].N + bn - 1) / bn);
+    units = (int)std::min<int64_t>(units, tiles);
   }
-  g.count = count; g.rounds = rounds; g.pairs = pairs;
+  if (!deal(g, es, tile_m, bn, units, any ? kGroupMaxItems : 12)) return US_ERR_UNSUPPORTED;      // too many tiles per unit for the work list
   g.status = static_cast<unsigned int*>(ws);
   g.wait_limit = kWaitLimit;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (es == 1) return pair ? launch_group<1, 256, 2>(g, st) : launch_group<1, 128, 1>(g, st);
+  return pair ? launch_group<2, 256, 2>(g, st) : launch_group<2, 128, 1>(g, st);
+}
 
-  constexpr int smem = GroupSmem::kTotal;
-  if (cudaFuncSetAttribute(gemm_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return US_ERR_CUDA;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * pairs);
-  cfg.blockDim = dim3(gemm_threads(kGroupEW));
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = static_cast<cudaStream_t>(stream);
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, gemm_group_kernel, g) == cudaSuccess ? US_OK : US_ERR_CUDA;
+}  // namespace
+}  // namespace us
+
+extern "C" us_status us_linear_group(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, void* stream) {
+  return us::group_impl(count, calls, false, ws, ws_bytes, stream);
+}
+extern "C" us_status us_linear_group_any(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, void* stream) {
+  return us::group_impl(count, calls, true, ws, ws_bytes, stream);
 }

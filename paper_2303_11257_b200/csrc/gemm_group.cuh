@@ -9,11 +9,14 @@
 // eight epilogue warps), and the main loop of a pair's next tile runs while its previous tile's
 // epilogue drains, across problem boundaries too.
 //
-// Scope: FP8 operands (either layout each), CTA-pair tiles of 256 x 256 (cta_group::2), plain
-// or residual (skip) epilogue, any output dtype, up to kGroupMaxProblems problems.  Everything that
-// differs between problems is run-time data here: tensor maps, operand layouts (a K-major and an
-// MN-major FP8 tile are both one 128-row x 128-byte box, only the coordinate order and the
-// descriptor strides differ), instruction descriptor, scale, epilogue kind.
+// Scope: FP8 or 16-bit operands (all problems of a launch the same width; either layout each), plain
+// or residual (skip) epilogue, any output dtype, up to kGroupMaxProblems problems.  CTA-pair tiles of
+// 256 x 256 (cta_group::2), or, when those would leave more than half of the pairs idle, single-CTA tiles
+// of 128 x 128.  Everything that differs between problems is run-time data here: tensor maps, operand
+// layouts (a K-major tile is one box of 128 rows x 128 bytes; an MN-major one has 128 / ES rows of K per
+// box, one box of 128 bytes for FP8 and two for 16-bit elements), instruction descriptor, scale, epilogue kind.
+// Measured, four separate launches -> this one, us: FP8 8192 x 1024 x 4096 122 -> 101; BF16 216 -> 199;
+// FP8 16384 x 2048 x 8192 (21 tiles per pair) 912 of kernel time, partly side by side, -> 809; FP8 256 x 128 x 512 26 -> 7.
 #pragma once
 
 #include "gemm_kernel.cuh"
@@ -21,11 +24,11 @@
 namespace us {
 
 constexpr int kGroupMaxProblems = 4;
-constexpr int kGroupMaxRounds = 12;
-constexpr int kGroupMaxPairs = 80;
+constexpr int kGroupMaxItems = 2048;    // entries of the work list (a kernel parameter: 8 KB)
+constexpr int kGroupMaxUnits = 160;     // CTA pairs or CTAs that share the list
 
 struct GroupProblem {
-  CUtensorMap ta, tb, tout, tskip;      // A and B: 128-row x 128-byte boxes; out / skip: 32-row x 128-byte boxes
+  CUtensorMap ta, tb, tout, tskip;      // A and B: operand boxes (above); out / skip: 32-row x 128-byte boxes
   int M, N, K;
   int a_mn, b_mn;                       // operand stored MN-major ([K x M] resp. [K x N] row-major)
   uint32_t idesc;
@@ -37,25 +40,28 @@ struct GroupProblem {
 
 struct GroupParams {
   GroupProblem prob[kGroupMaxProblems];
-  int count, rounds, pairs;
+  int count, rounds, units;             // units: CTA pairs, or CTAs with single-CTA tiles
   unsigned int* status;
   uint32_t wait_limit;
-  // work list: entry [round * pairs + pair] = problem << 24 | tile row << 12 | tile column, or -1
-  int32_t table[kGroupMaxRounds * kGroupMaxPairs];
+  // work list: entry [round * units + unit] = problem << 28 | tile row << 14 | tile column, or -1
+  int32_t table[kGroupMaxItems];
 };
 
 __device__ __forceinline__ void group_decode(int32_t e, int& prob, int& tm, int& tn) {
-  prob = e >> 24; tm = (e >> 12) & 0xfff; tn = e & 0xfff;
+  prob = e >> 28; tm = (e >> 14) & 0x3fff; tn = e & 0x3fff;
 }
 
 constexpr int kGroupEW = 8;
-using GroupSmem = GemmSmem<256, 2, kGroupEW>;
 
+template <int ES, int BN, int CG>
 __global__ void __launch_bounds__(gemm_threads(kGroupEW), 1)
 gemm_group_kernel(const __grid_constant__ GroupParams g) {
-  using S = GroupSmem;
-  constexpr int BN = 256, kBK = 128;
-  constexpr uint32_t kChunkBytes = kBK * 128;       // an MN-major operand tile: 128 rows of K x 128 bytes
+  using S = GemmSmem<BN, CG, kGroupEW>;
+  static_assert(BN / CG == 128, "128 rows of B per CTA");
+  constexpr int kBK = 128 / ES;                     // K elements per stage
+  constexpr int kTileM = kBM * CG;
+  constexpr int kWarpCols = BN / 2;                 // columns of a tile one epilogue warp handles
+  constexpr uint32_t kChunkBytes = kBK * 128;       // a box of an MN-major operand tile: kBK rows of K x 128 bytes
   constexpr uint32_t kTmemCols = 2 * BN;
 
   extern __shared__ uint8_t smem_raw[];
@@ -74,27 +80,30 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 4);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rank = (int)ptx::cluster_ctarank();
-  const int pair = blockIdx.x >> 1;
-  auto entry = [&](int r) { return g.table[r * g.pairs + pair]; };
+  const int rank = CG == 2 ? (int)ptx::cluster_ctarank() : 0;
+  const int unit = blockIdx.x / CG;
+  auto entry = [&](int r) { return g.table[r * g.units + unit]; };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S::kStages; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
-    for (int a = 0; a < 2; ++a) { ptx::mbar_init(acc_full_bar(a), 1); ptx::mbar_init(acc_empty_bar(a), 2 * 4 * (BN / 128)); }
+    for (int a = 0; a < 2; ++a) { ptx::mbar_init(acc_full_bar(a), 1); ptx::mbar_init(acc_empty_bar(a), CG * kGroupEW); }
     ptx::mbar_init(drained_bar, 1);
     for (int w = 0; w < kGroupEW; ++w) ptx::mbar_init(epi_in_bar(w), 1);
     *abort_flag = 0;
     ptx::mbar_init_fence();
   }
-  if (warp == 1) { ptx::tmem_alloc_pair(ptx::smem_addr(const_cast<uint32_t*>(tmem_slot)), kTmemCols); ptx::tmem_relinquish_pair(); }
+  if (warp == 1) {
+    if (CG == 2) { ptx::tmem_alloc_pair(ptx::smem_addr(const_cast<uint32_t*>(tmem_slot)), kTmemCols); ptx::tmem_relinquish_pair(); }
+    else { ptx::tmem_alloc(ptx::smem_addr(const_cast<uint32_t*>(tmem_slot)), kTmemCols); ptx::tmem_relinquish(); }
+  }
   ptx::tc_fence_before_sync();
   __syncthreads();
-  ptx::cluster_sync();
+  if (CG == 2) ptx::cluster_sync();
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer (both CTAs of the pair)
+    // ------------------------------------------------------------ TMA producer (every CTA)
     if (lane == 0) {
       uint32_t issued = 0;
       int stage = 0; uint32_t phase = 0;
@@ -105,17 +114,28 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
         int pi, tm, tn;
         group_decode(e, pi, tm, tn);
         const GroupProblem& P = g.prob[pi];
-        const int m0 = tm * 256 + rank * 128, n0 = tn * 256 + rank * 128;
+        const int m0 = tm * kTileM + rank * 128, n0 = tn * BN + rank * 128;
         const int num_kb = (P.K + kBK - 1) / kBK;
         for (int kb = 0; kb < num_kb; ++kb) {
           ok = wait_bounded(empty_bar(stage), phase ^ 1u, abort_flag, g.status, g.wait_limit);
           if (!ok) break;
           const uint32_t a_dst = smem_base + stage * S::kStageBytes, b_dst = a_dst + S::kABytes;
           const int k0 = kb * kBK;
-          const uint32_t fb = ptx::in_even_cta(full_bar(stage));
-          if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), 2 * S::kStageBytes);
-          if (P.a_mn) ptx::tma_load_2d_pair(a_dst, &P.ta, fb, m0, k0); else ptx::tma_load_2d_pair(a_dst, &P.ta, fb, k0, m0);
-          if (P.b_mn) ptx::tma_load_2d_pair(b_dst, &P.tb, fb, n0, k0); else ptx::tma_load_2d_pair(b_dst, &P.tb, fb, k0, n0);
+          const uint32_t fb = CG == 2 ? ptx::in_even_cta(full_bar(stage)) : full_bar(stage);
+          if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), CG * S::kStageBytes);
+          auto load = [&](uint32_t dst, const void* tmap, int x, int y) {
+            if (CG == 2) ptx::tma_load_2d_pair(dst, tmap, fb, x, y); else ptx::tma_load_2d(dst, tmap, fb, x, y);
+          };
+          auto operand = [&](uint32_t dst, const void* tmap, int mn, int mn0) {
+            if (mn) {
+#pragma unroll
+              for (int c = 0; c < ES; ++c) load(dst + c * kChunkBytes, tmap, mn0 + c * kBK, k0);   // 128 / ES elements per box
+            } else {
+              load(dst, tmap, k0, mn0);
+            }
+          };
+          operand(a_dst, &P.ta, P.a_mn, m0);
+          operand(b_dst, &P.tb, P.b_mn, n0);
           ++issued;
           if (++stage == S::kStages) { stage = 0; phase ^= 1u; }
         }
@@ -130,7 +150,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer (even CTA)
+    // ------------------------------------------------------------ MMA issuer (even CTA of a pair only)
     if (lane == 0 && rank == 0) {
       int stage = 0; uint32_t phase = 0, local = 0;
       bool ok = true;
@@ -167,22 +187,23 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
           for (int k = 0; k < kKSteps; ++k) {
             const uint64_t adesc = ((uint64_t)a_hi << 32) | (a_lo + k * a_step);
             const uint64_t bdesc = ((uint64_t)b_hi << 32) | (b_lo + k * b_step);
-            ptx::mma_ss_pair<true>(d_tmem, adesc, bdesc, idesc, accumulate);
+            if (CG == 2) ptx::mma_ss_pair<ES == 1>(d_tmem, adesc, bdesc, idesc, accumulate);
+            else ptx::mma_ss<ES == 1>(d_tmem, adesc, bdesc, idesc, accumulate);
             accumulate = 1;
           }
-          ptx::mma_commit_pair(empty_bar(stage), 3);
+          if (CG == 2) ptx::mma_commit_pair(empty_bar(stage), 3); else ptx::mma_commit(empty_bar(stage));
           if (++stage == S::kStages) { stage = 0; phase ^= 1u; }
         }
-        if (ok) ptx::mma_commit_pair(acc_full_bar(acc), 3);
+        if (ok) { if (CG == 2) ptx::mma_commit_pair(acc_full_bar(acc), 3); else ptx::mma_commit(acc_full_bar(acc)); }
       }
       if (*abort_flag) {
-        ptx::mma_commit_pair(drained_bar, 1);
+        if (CG == 2) ptx::mma_commit_pair(drained_bar, 1); else ptx::mma_commit(drained_bar);
         for (uint32_t it = 0; it < g.wait_limit && !ptx::mbar_try_wait(drained_bar, 0); ++it) {}
       }
     }
   } else {
     // ------------------------------------------------------------ epilogue warps
-    // Warp (quarter q, half) owns 32 rows x 128 columns of a tile, worked in 32-column slices.  Staging: box 0
+    // Warp (quarter q, half) owns 32 rows x half of the columns of a tile, worked in 32-column slices.  Staging: box 0
     // (4 KB) receives the skip tensor's boxes by TMA, box 1 (4 KB) collects output and leaves by TMA store.
     const int q = warp & 3, half = (warp - 2) >> 2;
     const uint32_t buf_in = epi_base + (warp - 2) * epi_warp_bytes(kGroupEW), buf_out = buf_in + 4096u;
@@ -206,8 +227,8 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
         int pi, tm, tn;
         group_decode(e, pi, tm, tn);
         const GroupProblem& P = g.prob[pi];
-        const int n_w = tn * BN + half * 128;
-        if (P.has_skip && n_w < P.N) issue_in(P, n_w, tm * 256 + rank * 128 + q * 32);
+        const int n_w = tn * BN + half * kWarpCols;
+        if (P.has_skip && n_w < P.N) issue_in(P, n_w, tm * kTileM + rank * 128 + q * 32);
         return;                                                // only the very next tile is looked at
       }
     };
@@ -221,7 +242,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
       const GroupProblem& P = g.prob[pi];
       const uint32_t acc = local & 1u, acc_phase = (local >> 1) & 1u;
       ++local;
-      const int row0 = tm * 256 + rank * 128 + q * 32, n_w = tn * BN + half * 128;
+      const int row0 = tm * kTileM + rank * 128 + q * 32, n_w = tn * BN + half * kWarpCols;
       const bool skip = P.has_skip != 0;
       const int in_es = dtype_size(P.skip_dt), out_es = dtype_size(P.out_dt);
       const int in_box_cols = 128 / in_es, out_box_cols = 128 / out_es;
@@ -229,20 +250,23 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       ptx::tc_fence_after_sync();
-      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + half * 128;
+      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + half * kWarpCols;
       auto release_acc = [&]() {
         ptx::tc_fence_before_sync();
         __syncwarp();
-        if (lane == 0) ptx::mbar_arrive_cluster(ptx::in_even_cta(acc_empty_bar(acc)));
+        if (lane == 0) {
+          if (CG == 2) ptx::mbar_arrive_cluster(ptx::in_even_cta(acc_empty_bar(acc)));
+          else ptx::mbar_arrive(acc_empty_bar(acc));
+        }
       };
       bool released = false, looked_ahead = false;
       if (n_w < P.N) {
         const f32x2 scale2 = splat2(P.scale), skip2 = splat2(P.skip_coef), oc2 = splat2(P.out_coef);
 #pragma unroll 1
-        for (int sl = 0; sl < 4; ++sl) {
+        for (int sl = 0; sl < kWarpCols / 32; ++sl) {
           const int col = n_w + 32 * sl;
           if (col >= P.N) break;
-          const bool last_slice = sl == 3 || col + 32 >= P.N;
+          const bool last_slice = sl == kWarpCols / 32 - 1 || col + 32 >= P.N;
           uint4 raw[8];
           if (skip) {
             const int off = (32 * sl) & (in_box_cols - 1);
@@ -341,10 +365,10 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
 
   ptx::tc_fence_before_sync();
   __syncthreads();
-  ptx::cluster_sync();
+  if (CG == 2) ptx::cluster_sync();
   if (warp == 1) {
     ptx::tc_fence_after_sync();
-    ptx::tmem_dealloc_pair(tmem_base, kTmemCols);
+    if (CG == 2) ptx::tmem_dealloc_pair(tmem_base, kTmemCols); else ptx::tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 

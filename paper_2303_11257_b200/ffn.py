@@ -17,9 +17,10 @@ Backward, G = dL/dR (the branch output receives G unscaled):
 q is E4M3 for activations / weights and E5M2 for gradients in "fp8" mode; in "bf16" / "fp16"
 mode the matmul inputs are rounded to that format instead (no loss scale, same fixed scales).
 
-step() knows G when it starts.  In FP8 mode it therefore issues the two GEMMs that end in the hidden layer (H, A and
-dH above) as one us_ffn_hidden launch, in which H stays on the SM, and the other four GEMMs as one us_linear_group
-launch: three launches per step with the fused cast.  self.H is then written only with keep_h = True.
+step() knows G when it starts.  It therefore issues the two GEMMs that end in the hidden layer (H, A and dH above) as
+one us_ffn_hidden launch, in which H stays on the SM, and the other four GEMMs as one us_linear_group launch (the
+"_any" forms of both, which take 16-bit operands and small shapes): three launches per step with the fused cast.  In
+FP8 mode self.H is then written only with keep_h = True.
 """
 from __future__ import annotations
 
@@ -81,22 +82,22 @@ class UnitScaledFFN:
         self.ws = L.new_workspace(device)
         c_skip, c_branch = L.us_scales_residual(self.sc.tau)
         self._c = (c_skip, c_branch)
-        # step() has all four tensors to quantise at hand when it starts, so in FP8 mode it casts them
+        # step() has all four tensors to quantise at hand when it starts, so it casts them
         # with one launch; forward() / backward() on their own cast what they are given.
-        self.fused_casts = operand == "fp8"
+        self.fused_casts = True
         # After the first GEMM, the second forward GEMM, the GELU-gradient GEMM and the first weight-gradient GEMM
         # depend on nothing but it, and the last two GEMMs only on the GELU-gradient one.  step() issues them on
         # three streams, so that the CTAs of one kernel fill the SMs another leaves idle in its last wave (64 or
         # 128 tiles on 74 CTA pairs); measured 6 % faster than one stream once the power cap holds the clock.
-        self.concurrent = self.fused_casts
+        self.concurrent = operand == "fp8"
         self._side = None
-        # FP8 operands: the four GEMMs that remain after the GELU-gradient GEMM are independent of one another and
+        # The four GEMMs that remain after the GELU-gradient GEMM are independent of one another and
         # go out as one us_linear_group launch (4 launches per step instead of 7).
-        self.grouped = operand == "fp8"
-        # FP8 operands and G known up front: the first GEMM + GELU and the GELU-gradient GEMM are one us_ffn_hidden
-        # launch that keeps the pre-activation on the SM; keep_h = True also writes its 16-bit copy to self.H (the
-        # separate launches always do, the backward one reads it from there).
-        self.fused_hidden = operand == "fp8"
+        self.grouped = True
+        # G known up front: the first GEMM + GELU and the GELU-gradient GEMM are one us_ffn_hidden launch that keeps
+        # the pre-activation on the SM; keep_h = True also writes its 16-bit copy to self.H (the separate launches,
+        # 16-bit operand mode and blocks with a dimension of at most 128 always do; backward() reads it from there).
+        self.fused_hidden = operand == "fp8" or h_dtype in (torch.bfloat16, torch.float16)
         self.keep_h = keep_h
 
     @property
@@ -106,7 +107,7 @@ class UnitScaledFFN:
 
     @property
     def launches_per_step(self) -> int:
-        """Kernel launches of step(): the cast(s) plus gemm_launches in FP8 mode."""
+        """Kernel launches of step(): the cast(s) plus gemm_launches."""
         if self.fused_casts:
             return 1 + self.gemm_launches
         return 10
@@ -117,6 +118,15 @@ class UnitScaledFFN:
         else:
             # 16-bit operand mode: rounding fp32 -> bf16/fp16 is the residual kernel with tau = 0
             L.us_residual_add(src, src, 0.0, dst, stream)
+
+    def _cast_all(self, X, W1, W2, G, stream):
+        try:
+            L.us_cast_multi([W1, W2, X, G], [1.0] * 4, [self.W1q, self.W2q, self.Xq, self.Gq], stream)
+        except L.UnitScaleError as e:
+            if self.operand == "fp8" or e.status not in (L.US_ERR_UNSUPPORTED, L.US_ERR_ALIGNMENT):
+                raise
+            for src, dst in ((W1, self.W1q), (W2, self.W2q), (X, self.Xq), (G, self.Gq)):    # padded or unaligned rows
+                self._cast(src, dst, stream)
 
     def stages(self, X, W1, W2, G, fused_casts: bool | None = None):
         """The launches of one pass, in order, as (name, kind, callable(stream)) triples.
@@ -132,8 +142,7 @@ class UnitScaledFFN:
         ep5 = L.epilogue(skip=G, skip_coef=c_skip, out_coef=c_branch)
         ws = self.ws
         if fused:
-            casts = [("cast_all", "cast", lambda st=None: L.us_cast_fp8_multi(
-                [W1, W2, X, G], [1.0] * 4, [self.W1q, self.W2q, self.Xq, self.Gq], st))]
+            casts = [("cast_all", "cast", lambda st=None: self._cast_all(X, W1, W2, G, st))]
             cast_g = []
         else:
             casts = [("cast_W1", "cast", lambda st=None: self._cast(W1, self.W1q, st)),
@@ -161,7 +170,7 @@ class UnitScaledFFN:
         if self.fused_hidden:
             head = head[:1] + [("hidden_fwd1_gelu_bwd_x2_gelu_grad", "group", 2, lambda stream=None: self._hidden(stream))]
         return head + [("group_fwd2_bwd_w2_bwd_x1_bwd_w1", "group", 4,
-                        lambda stream=None: L.us_linear_group(self.group_calls(X, G), self.ws, stream))]
+                        lambda stream=None: L.us_linear_group_any(self.group_calls(X, G), self.ws, stream))]
 
     def group_calls(self, X, G):
         """The four GEMMs that follow the GELU-gradient GEMM, as the entries of one us_linear_group launch
@@ -177,8 +186,9 @@ class UnitScaledFFN:
     def _hidden(self, stream=None):
         """H, A and dH in one launch (us_ffn_hidden) from the quantised operands."""
         sc = self.sc
-        L.us_ffn_hidden(self.Xq, self.W1q, sc.alpha1, self.Gq, self.W2q, sc.beta_x2, sc.s_in, sc.alpha_g, sc.beta_g,
-                        self.Aq, self.dHq, self.ws, H=self.H if self.keep_h else None, h_dtype=self.H.dtype, stream=stream)
+        keep = self.keep_h or self.operand != "fp8" or min(self.T, self.d, self.f) <= 128     # small blocks always keep it
+        L.us_ffn_hidden_any(self.Xq, self.W1q, sc.alpha1, self.Gq, self.W2q, sc.beta_x2, sc.s_in, sc.alpha_g, sc.beta_g,
+                            self.Aq, self.dHq, self.ws, H=self.H if keep else None, h_dtype=self.H.dtype, stream=stream)
 
     def cast_weights(self, W1, W2, stream=None):
         self._cast(W1, self.W1q, stream)
@@ -255,7 +265,7 @@ class UnitScaledFFN:
         return self.dX, self.dW1, self.dW2
 
     def step_from_casts(self, X, G, stream=None):
-        """The GEMMs of one pass when self.Xq, W1q, W2q, Gq already hold the quantised operands (FP8 mode): two
+        """The GEMMs of one pass when self.Xq, W1q, W2q, Gq already hold the quantised operands: two
         launches -- the hidden layer's two GEMMs with GELU and GELU gradient, the other four as one group -- or their
         separate forms where a shape is not covered.  X and G are the unquantised skip inputs of the two residual
         epilogues."""
@@ -267,19 +277,19 @@ class UnitScaledFFN:
             except L.UnitScaleError as e:
                 if e.status != L.US_ERR_UNSUPPORTED:
                     raise
-                fused = self.fused_hidden = False            # at most 128 tokens or hidden units: nothing was launched
+                fused = self.fused_hidden = False            # a shape this form does not cover: nothing was launched
         if not fused:
             by["fwd1_gelu"](stream)
             by["bwd_x2_gelu_grad"](stream)
         if self.grouped:
             try:
-                L.us_linear_group(self.group_calls(X, G), self.ws, stream)
+                L.us_linear_group_any(self.group_calls(X, G), self.ws, stream)
                 return self.dX, self.dW1, self.dW2
             except L.UnitScaleError as e:
                 if e.status != L.US_ERR_UNSUPPORTED:
                     raise
-                # a shape the grouped form does not cover (an output of at most 128 rows or columns): nothing was
-                # launched; the four GEMMs go out one by one, now and in later steps
+                # more tiles than the work list of the grouped form holds: nothing was launched; the four GEMMs go out
+                # one by one, now and in later steps
                 self.grouped = False
         for name in ("fwd2_residual", "bwd_w2", "bwd_x1_residual", "bwd_w1"):
             by[name](stream)

@@ -96,9 +96,11 @@ def _load() -> C.CDLL:
     lib.us_test_linear_fwd_starved.argtypes = [MP, MP, F, MP, V, SZ, C.c_uint, V]
     lib.us_test_linear_fwd_starved.restype = C.c_int
     lib.us_linear_group.argtypes = [C.c_int, C.POINTER(us_linear_call), V, SZ, V]
-    lib.us_linear_group.restype = C.c_int
+    lib.us_linear_group_any.argtypes = lib.us_linear_group.argtypes
+    lib.us_linear_group.restype = lib.us_linear_group_any.restype = C.c_int
     lib.us_ffn_hidden.argtypes = [MP, MP, F, MP, MP, F, F, F, F, C.c_int32, MP, MP, MP, V, SZ, V]
-    lib.us_ffn_hidden.restype = C.c_int
+    lib.us_ffn_hidden_any.argtypes = lib.us_ffn_hidden.argtypes
+    lib.us_ffn_hidden.restype = lib.us_ffn_hidden_any.restype = C.c_int
     lib.us_test_ffn_hidden_starved.argtypes = [MP, MP, MP, MP, MP, MP, V, SZ, C.c_uint, V]
     lib.us_test_ffn_hidden_starved.restype = C.c_int
     lib.us_workspace_bytes.argtypes = []
@@ -112,7 +114,7 @@ def _load() -> C.CDLL:
     lib.us_activation_fwd.argtypes = [C.c_int, MP, F, F, MP, V]
     lib.us_activation_bwd.argtypes = [C.c_int, MP, MP, F, F, MP, V]
     lib.us_activation_fwd.restype = lib.us_activation_bwd.restype = C.c_int
-    lib.us_cast_fp8_multi.argtypes = [C.c_int, MP, C.POINTER(C.c_float), MP, V]
+    lib.us_cast_fp8_multi.argtypes = lib.us_cast_multi.argtypes = [C.c_int, MP, C.POINTER(C.c_float), MP, V]
     lib.us_weighted_add.argtypes = [C.c_int, MP, C.POINTER(C.c_float), F, MP, V]
     lib.us_weighted_add.restype = C.c_int
     lib.us_softmax_fwd.argtypes = [MP, F, MP, V]
@@ -129,7 +131,7 @@ def _load() -> C.CDLL:
     lib.us_quant_stats_workspace_bytes.restype = SZ
     lib.us_quant_stats.argtypes = [MP, F, C.c_int, C.c_int, C.c_int, V, V, V, SZ, V]
     lib.us_quant_stats.restype = C.c_int
-    for name in ("us_gelu_fwd", "us_gelu_bwd", "us_residual_add", "us_cast_fp8", "us_cast_fp8_multi", "us_softmax_fwd", "us_softmax_bwd"):
+    for name in ("us_gelu_fwd", "us_gelu_bwd", "us_residual_add", "us_cast_fp8", "us_cast_fp8_multi", "us_cast_multi", "us_softmax_fwd", "us_softmax_bwd"):
         getattr(lib, name).restype = C.c_int
     FP = C.POINTER(C.c_float)
     lib.us_scales_linear.argtypes = [C.c_int64, C.c_int64, C.c_int64, C.c_int, FP, FP, FP]
@@ -235,10 +237,15 @@ def linear_call(op: int, a, b, scale: float, out, ep=None) -> us_linear_call:
     return c
 
 
-def us_linear_group(calls, ws, stream=None):
+def us_linear_group(calls, ws, stream=None, name="us_linear_group"):
     """Several independent linear ops in one launch (see the header for what this form covers)."""
     arr = (us_linear_call * len(calls))(*calls)
-    _check("us_linear_group", _lib.us_linear_group(len(calls), arr, ws.data_ptr(), ws.numel() * ws.element_size(), _stream(stream)))
+    _check(name, getattr(_lib, name)(len(calls), arr, ws.data_ptr(), ws.numel() * ws.element_size(), _stream(stream)))
+
+
+def us_linear_group_any(calls, ws, stream=None):
+    """us_linear_group for 16-bit operands and outputs of any size, too."""
+    us_linear_group(calls, ws, stream, "us_linear_group_any")
 
 
 def batch(count, a_stride, b_stride, out_stride) -> us_batch:
@@ -334,15 +341,20 @@ def us_test_linear_fwd_starved(X, W, alpha, Y, ws, wait_limit: int, stream=None)
 
 
 def us_ffn_hidden(X, W1, alpha, G, W2, beta_x, act_in_scale, act_out_scale, grad_out_scale, A, dH, ws,
-                  H=None, h_dtype=torch.bfloat16, stream=None):
+                  H=None, h_dtype=torch.bfloat16, stream=None, name="us_ffn_hidden"):
     """Hidden layer of the FFN block, forward and backward, in one launch (see the header): A and dH are written,
     H (optional) receives the pre-activation rounded to h_dtype."""
     hp = C.byref(mat(H)) if H is not None else None
-    _check("us_ffn_hidden",
-           _lib.us_ffn_hidden(C.byref(mat(X)), C.byref(mat(W1)), alpha, C.byref(mat(G)), C.byref(mat(W2)), beta_x,
-                              act_in_scale, act_out_scale, grad_out_scale, _TORCH_DTYPES[h_dtype], hp, C.byref(mat(A)),
-                              C.byref(mat(dH)), ws.data_ptr(), ws.numel() * ws.element_size(), _stream(stream)))
+    _check(name,
+           getattr(_lib, name)(C.byref(mat(X)), C.byref(mat(W1)), alpha, C.byref(mat(G)), C.byref(mat(W2)), beta_x,
+                               act_in_scale, act_out_scale, grad_out_scale, _TORCH_DTYPES[h_dtype], hp, C.byref(mat(A)),
+                               C.byref(mat(dH)), ws.data_ptr(), ws.numel() * ws.element_size(), _stream(stream)))
     return A, dH
+
+
+def us_ffn_hidden_any(*args, **kwargs):
+    """us_ffn_hidden for 16-bit operands and any number of rows and hidden units, too."""
+    return us_ffn_hidden(*args, **kwargs, name="us_ffn_hidden_any")
 
 
 def us_test_ffn_hidden_starved(X, W1, G, W2, A, dH, ws, wait_limit: int, stream=None):
@@ -403,14 +415,19 @@ def us_weighted_add(srcs, gammas, alpha, out, stream=None):
     return out
 
 
-def us_cast_fp8_multi(srcs, scales, dsts, stream=None):
+def us_cast_fp8_multi(srcs, scales, dsts, stream=None, name="us_cast_fp8_multi"):
     """One launch for len(srcs) casts; scales: one float per tensor."""
     n = len(srcs)
     sm = (us_mat * n)(*[mat(t) for t in srcs])
     dm = (us_mat * n)(*[mat(t) for t in dsts])
     sc = (C.c_float * n)(*[float(x) for x in scales])
-    _check("us_cast_fp8_multi", _lib.us_cast_fp8_multi(n, sm, sc, dm, _stream(stream)))
+    _check(name, getattr(_lib, name)(n, sm, sc, dm, _stream(stream)))
     return dsts
+
+
+def us_cast_multi(srcs, scales, dsts, stream=None):
+    """us_cast_fp8_multi with BF16 / F16 destinations allowed."""
+    return us_cast_fp8_multi(srcs, scales, dsts, stream, "us_cast_multi")
 
 
 def us_softmax_fwd(S, alpha, P, stream=None):

@@ -163,3 +163,23 @@ def test_ffn_hidden_starved_launch_times_out_and_the_next_call_is_correct():
         with pytest.raises(L.UnitScaleError) as err:
             L.us_test_ffn_hidden_starved(Xt, W1t, Gt, W2t, A, dH, ws, wait_limit=bad)
         assert err.value.status == US_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("b,m,f,n", [(1, 16, 16, 16), (48, 128, 512, 128), (129, 80, 136, 208), (128, 64, 128, 1040), (300, 144, 400, 80),
+                                     (2304, 256, 4864, 256)])
+@pytest.mark.parametrize("act,grad,h_fmt", [("bf16", "bf16", "bf16"), ("fp16", "fp16", "bf16"), ("bf16", "bf16", "fp16"), ("e4m3", "e5m2", "bf16")])
+def test_ffn_hidden_any_equals_the_separate_calls(b, m, f, n, act, grad, h_fmt):
+    """Every operand width and both tile sizes, down to single rows: A, dH and the kept copy bit for bit."""
+    L, synth = _mods()
+    ws = L.new_workspace()
+    X, W1 = U.to_device(synth.normal(7, 0, (b, m)), act, (m + 15) // 16 * 16), U.to_device(synth.normal(7, 1, (m, f)), act, (f + 15) // 16 * 16)
+    G, W2 = U.to_device(synth.normal(7, 2, (b, n)), grad), U.to_device(synth.normal(7, 3, (f, n)), act)
+    out = lambda fmt: U.empty(b, f, fmt, (f + 15) // 16 * 16)
+    A, dH, H = out(act), out(grad), out(h_fmt)
+    L.us_ffn_hidden_any(X, W1, m ** -0.5, G, W2, n ** -0.5, 0.75, 1.7, 1.48, A, dH, ws, H=H, h_dtype=H.dtype)
+    A1, dH1, H1 = out(act), out(grad), out(h_fmt)
+    L.us_linear_fwd(X, W1, m ** -0.5, A1, ws, L.epilogue(act=L.US_ACT_GELU, act_in_scale=0.75, act_out_scale=1.7, aux=H1))
+    L.us_linear_bwd_x(G, W2, n ** -0.5, dH1, ws, L.epilogue(act=L.US_ACT_GELU_GRAD, act_in_scale=0.75, act_out_scale=1.48, aux=H1))
+    assert L.us_workspace_status(ws) == 0
+    for a, r in ((H, H1), (A, A1), (dH, dH1)):
+        assert np.array_equal(U.codes_of(a), U.codes_of(r))

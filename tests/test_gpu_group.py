@@ -105,3 +105,27 @@ def test_ffn_step_with_the_grouped_launch_equals_the_seven_launch_step():
         outs.append([t.clone() for t in (blk.R, blk.dX, blk.dW1, blk.dW2)])
     for a, b in zip(*outs):
         assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
+
+
+@pytest.mark.parametrize("fmt", ["bf16", "fp16", "e4m3"])
+@pytest.mark.parametrize("b,m,n", [(1, 16, 16), (48, 128, 512), (129, 80, 136), (2000, 528, 272), (4352, 1040, 2048)])
+def test_group_any_equals_single_calls(fmt, b, m, n):
+    """16-bit operands, outputs of one tile or less, both tile sizes and a work list of more than twelve rounds: the
+    grouped launch without the size limits against the single entry points."""
+    L, synth = _mods()
+    ws = L.new_workspace()
+    dev = lambda i, shape: U.to_device(synth.normal(40 + i, 0, shape), fmt, (shape[1] + 15) // 16 * 16)
+    X, W, G, skip = dev(0, (b, m)), dev(1, (m, n)), dev(2, (b, n)), U.to_device(synth.normal(44, 0, (b, m)), "f32")
+    ep = lambda: L.epilogue(skip=skip, skip_coef=0.8, out_coef=0.6)
+    outs = [[U.empty(b, n, "bf16", (n + 7) // 8 * 8), U.empty(b, m, "bf16"), U.empty(m, n, "f32"), U.empty(m, n, "fp16", (n + 7) // 8 * 8)] for _ in range(2)]
+    o = outs[0]
+    L.us_linear_group_any([L.linear_call(L.US_OP_BWD_W, X, G, 0.1, o[2]), L.linear_call(L.US_OP_FWD, X, W, 0.2, o[0]),
+                           L.linear_call(L.US_OP_BWD_X, G, W, 0.3, o[1], ep()), L.linear_call(L.US_OP_BWD_W, X, G, 0.4, o[3])], ws)
+    o = outs[1]
+    L.us_linear_bwd_w(X, G, 0.1, o[2], ws)
+    L.us_linear_fwd(X, W, 0.2, o[0], ws)
+    L.us_linear_bwd_x(G, W, 0.3, o[1], ws, ep())
+    L.us_linear_bwd_w(X, G, 0.4, o[3], ws)
+    assert L.us_workspace_status(ws) == 0
+    for a, r in zip(*outs):
+        assert torch.equal(a.contiguous().view(torch.uint8), r.contiguous().view(torch.uint8))
