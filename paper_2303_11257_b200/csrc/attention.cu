@@ -83,6 +83,7 @@ template <bool F8>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_fwd_kernel(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CUtensorMap tk,
                      const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap tp, const AttnParams a) {
+  ptx::grid_release_next();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - ptx::smem_addr(smem_raw));
@@ -118,6 +119,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tq, const __grid_consta
   __syncthreads();
   ptx::tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  ptx::grid_wait_previous();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -397,6 +399,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_bwd_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_constant__ CUtensorMap tv,
                      const __grid_constant__ CUtensorMap tk, const __grid_constant__ CUtensorMap tp,
                      const __grid_constant__ CUtensorMap tds, const AttnBwdParams a) {
+  ptx::grid_release_next();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - ptx::smem_addr(smem_raw));
@@ -431,6 +434,7 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_const
   __syncthreads();
   ptx::tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  ptx::grid_wait_previous();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -720,16 +724,14 @@ extern "C" us_status us_attention_fwd(const us_mat* Q, const us_mat* K, const us
   a.wait_limit = kWaitLimit;
 
   auto kern = f8 ? attention_fwd_kernel<true> : attention_fwd_kernel<false>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAttnSmem) != cudaSuccess)
-    return US_ERR_CUDA;
+  static std::atomic<uint64_t> smem_set[2];
   a.q_tiles = (int)((s_q + 127) / 128); a.nb1 = (int)cnt[1]; a.nb0 = (int)cnt[0];
   const int64_t tiles = (int64_t)a.q_tiles * cnt[1] * cnt[0];
   if (tiles > 0x7fffffff) return US_ERR_INVALID_ARG;
   const int sms = host::sm_count();
   if (sms <= 0) return US_ERR_CUDA;
   const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);    // persistent: one CTA per SM walks the tiles
-  kern<<<grid, kAttnThreads, kAttnSmem, static_cast<cudaStream_t>(stream)>>>(tq, tk, tv, tp, a);
-  return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
+  return host::launch(kern, &smem_set[f8], (int)grid, kAttnThreads, kAttnSmem, 1, static_cast<cudaStream_t>(stream), tq, tk, tv, tp, a);
 }
 
 extern "C" us_status us_attention_bwd(const us_mat* dC, const us_mat* P, const us_mat* K, const us_mat* V, float beta_p,
@@ -796,9 +798,7 @@ extern "C" us_status us_attention_bwd(const us_mat* dC, const us_mat* P, const u
   const int sms = host::sm_count();
   if (sms <= 0) return US_ERR_CUDA;
   auto kern = f8 ? attention_bwd_kernel<true> : attention_bwd_kernel<false>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAttnBwdSmem) != cudaSuccess)
-    return US_ERR_CUDA;
+  static std::atomic<uint64_t> smem_set[2];
   const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
-  kern<<<grid, kAttnThreads, kAttnBwdSmem, static_cast<cudaStream_t>(stream)>>>(tdc, tv, tk, tp, tds, a);
-  return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
+  return host::launch(kern, &smem_set[f8], (int)grid, kAttnThreads, kAttnBwdSmem, 1, static_cast<cudaStream_t>(stream), tdc, tv, tk, tp, tds, a);
 }

@@ -4,6 +4,7 @@
 // the SM count and strides over the tensor.
 #include "common.cuh"
 #include "host.h"
+#include "sm100.cuh"
 
 namespace us {
 
@@ -51,7 +52,7 @@ template <int OP>
 __global__ void __launch_bounds__(kThreads) ew_kernel(const EwArgs p) {
   constexpr bool kTwoInputs = (OP == kGeluBwd || OP == kResidual || OP == kActBwd);
   const int64_t total = p.rows * p.chunks_per_row;
-  for (int64_t c = blockIdx.x * (int64_t)kThreads + threadIdx.x; c < total;
+  for (int64_t c = blockIdx.x * (int64_t)kThreads + threadIdx.x + ptx::grid_sync_previous(); c < total;
        c += (int64_t)gridDim.x * kThreads) {
     const int64_t row = p.rows == 1 ? 0 : c / p.chunks_per_row;      // tensors without row padding arrive as one long row
     const int64_t col = (c - row * p.chunks_per_row) * kVec;
@@ -130,7 +131,7 @@ __device__ __forceinline__ void multi_tail(const MultiCastArgs& p, const MultiCh
 __global__ void __launch_bounds__(kThreads) multi_cast_kernel(const MultiCastArgs p) {
   const int64_t total = p.chunk_end[p.count - 1];
   const int64_t stride = (int64_t)gridDim.x * kThreads;
-  for (int64_t c = blockIdx.x * (int64_t)kThreads + threadIdx.x; c < total; c += 2 * stride) {
+  for (int64_t c = blockIdx.x * (int64_t)kThreads + threadIdx.x + ptx::grid_sync_previous(); c < total; c += 2 * stride) {
     const MultiChunk m0 = multi_locate(p, c);
     const bool two = c + stride < total;
     const MultiChunk m1 = two ? multi_locate(p, c + stride) : m0;
@@ -224,8 +225,7 @@ static us_status ew_launch(const us_mat* in0, const us_mat* in1, const us_mat* o
   const int64_t want = (total + kThreads - 1) / kThreads;
   const int64_t cap = (int64_t)sms * 8;                 // 8 resident CTAs of 256 threads per SM
   const int grid = (int)(want < cap ? want : cap);
-  ew_kernel<OP><<<grid, kThreads, 0, static_cast<cudaStream_t>(stream)>>>(p);
-  return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
+  return host::launch(ew_kernel<OP>, nullptr, grid, kThreads, 0, 1, static_cast<cudaStream_t>(stream), p);
 }
 
 }  // namespace us
@@ -283,8 +283,7 @@ static us_status cast_multi(int count, const us_mat* src, const float* scale, co
   if (sms <= 0) return US_ERR_CUDA;
   const int64_t want = (chunks + kThreads - 1) / kThreads;
   const int64_t cap = (int64_t)sms * 8;
-  multi_cast_kernel<<<(int)(want < cap ? want : cap), kThreads, 0, static_cast<cudaStream_t>(stream)>>>(p);
-  return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
+  return host::launch(multi_cast_kernel, nullptr, (int)(want < cap ? want : cap), kThreads, 0, 1, static_cast<cudaStream_t>(stream), p);
 }
 
 extern "C" us_status us_cast_fp8_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, void* stream) {

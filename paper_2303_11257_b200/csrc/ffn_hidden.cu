@@ -78,6 +78,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   constexpr uint32_t kChunkBytes = kBK * 128;       // a box of an MN-major operand tile: kBK rows of K x 128 bytes
   constexpr uint32_t kTmemCols = 2 * BN;
 
+  ptx::grid_release_next();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
@@ -121,6 +122,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   if (CG == 2) ptx::cluster_sync();
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  ptx::grid_wait_previous();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (every CTA)
@@ -391,18 +393,8 @@ template <int ES, int BN, int CG, int OUT_A, int OUT_D, bool H_BF16>
 us_status launch_hidden(const CUtensorMap* t, const HiddenParams& p, int units, cudaStream_t stream) {
   auto kern = ffn_hidden_kernel<ES, BN, CG, OUT_A, OUT_D, H_BF16>;
   constexpr int smem = HidSmem<BN, OUT_A == US_E4M3 || OUT_A == US_E5M2 ? 1 : 2>::kTotal;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return US_ERR_CUDA;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CG * units);
-  cfg.blockDim = dim3(gemm_threads(kHidEW));
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CG; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, t[0], t[1], t[2], t[3], t[4], t[5], p) == cudaSuccess ? US_OK : US_ERR_CUDA;
+  static std::atomic<uint64_t> smem_set{0};
+  return host::launch(kern, &smem_set, CG * units, gemm_threads(kHidEW), smem, CG, stream, t[0], t[1], t[2], t[3], t[4], t[5], p);
 }
 template <int ES, int OUT_A, int OUT_D>
 us_status pick_hidden(bool pair, bool h_bf16, const CUtensorMap* t, const HiddenParams& p, int units, cudaStream_t st) {

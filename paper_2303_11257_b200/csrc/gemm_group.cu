@@ -108,18 +108,8 @@ template <int ES, int BN, int CG>
 us_status launch_group(const GroupParams& g, cudaStream_t stream) {
   auto kern = gemm_group_kernel<ES, BN, CG>;
   constexpr int smem = GemmSmem<BN, CG, kGroupEW>::kTotal;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return US_ERR_CUDA;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CG * g.units);
-  cfg.blockDim = dim3(gemm_threads(kGroupEW));
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CG; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, g) == cudaSuccess ? US_OK : US_ERR_CUDA;
+  static std::atomic<uint64_t> smem_set{0};
+  return host::launch(kern, &smem_set, CG * g.units, gemm_threads(kGroupEW), smem, CG, stream, g);
 }
 
 us_status group_impl(int count, const us_linear_call* calls, bool any, void* ws, size_t ws_bytes, void* stream) {

@@ -64,6 +64,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
   constexpr uint32_t kChunkBytes = kBK * 128;       // a box of an MN-major operand tile: kBK rows of K x 128 bytes
   constexpr uint32_t kTmemCols = 2 * BN;
 
+  ptx::grid_release_next();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
@@ -101,6 +102,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
   if (CG == 2) ptx::cluster_sync();
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  ptx::grid_wait_previous();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (every CTA)

@@ -59,23 +59,13 @@ static us_status launch(const us_mat* A, const us_mat* B, const GemmParams& p, c
   if (EPI != kEpiLegacy && em.skip && !make_tmap(&t_skip, em.skip, dtype_size(em.skip->dtype), 32)) return US_ERR_CUDA;
   auto kern = gemm_kernel<ES, A_MN, B_MN, BN, CG, EPI, EW, BATCHED>;
   constexpr int smem = GemmSmem<BN, CG, EW>::kTotal;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return US_ERR_CUDA;
   const int sms = host::sm_count();
   if (sms <= 0) return US_ERR_CUDA;
   const int tiles = p.tiles_m * p.tiles_n * p.nb0 * p.nb1;
   const int groups = sms / CG;                        // one CTA per SM; pairs share a TPC
   const int grid = CG * (tiles < groups ? tiles : groups);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(gemm_threads(EW));
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CG; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, ta, tb, t_out, t_aux, t_skip, p) == cudaSuccess ? US_OK : US_ERR_CUDA;
+  static std::atomic<uint64_t> smem_set{0};
+  return host::launch(kern, &smem_set, grid, gemm_threads(EW), smem, CG, stream, ta, tb, t_out, t_aux, t_skip, p);
 }
 
 template <int ES, bool A_MN, bool B_MN, int BN, int CG>

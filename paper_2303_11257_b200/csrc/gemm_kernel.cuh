@@ -679,6 +679,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   constexpr int kBRows = BN / CG;                   // B rows (N indices) this CTA loads
   static_assert(CG == 1 || (kBRows % kChunkElems) == 0, "pair tiles need whole 128-byte chunks of N per CTA");
 
+  ptx::grid_release_next();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
@@ -723,6 +724,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   if (CG == 2) ptx::cluster_sync();                  // the partner's barriers and TMEM are ready too
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  const int zero = ptx::grid_wait_previous();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (every CTA)
@@ -858,7 +860,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
       const uint32_t acc = local & 1u, acc_phase = (local >> 1) & 1u;
       const int m0 = tile_m(p, tile) * (kBM * CG) + rank * kBM;
       const int n0 = tile_n(p, tile) * BN;
-      const int64_t row = m0 + q * 32 + lane;
+      const int64_t row = m0 + q * 32 + lane + zero;
       const bool row_ok = row < p.M;
       EpiloguePrefetch pf;
       const int c_first = 32 * half;

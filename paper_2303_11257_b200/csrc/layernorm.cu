@@ -248,11 +248,12 @@ __global__ void __launch_bounds__(kLnThreads, 2) ln_fwd16_kernel(const LnArgs a)
   extern __shared__ __align__(16) float ln_smem[];                         // w[cols], c[cols] as float32
   float* w_s = ln_smem;
   float* c_s = ln_smem + a.cols;
-  for (int j = threadIdx.x; j < a.cols; j += blockDim.x) { w_s[j] = load_one(a.w, a.w_dt, j); c_s[j] = load_one(a.c, a.c_dt, j); }
+  const int zero = ptx::grid_sync_previous();
+  for (int j = threadIdx.x + zero; j < a.cols; j += blockDim.x) { w_s[j] = load_one(a.w, a.w_dt, j); c_s[j] = load_one(a.c, a.c_dt, j); }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int64_t stride = (int64_t)gridDim.x * nw;
-  int64_t row = (int64_t)blockIdx.x * nw + warp;
+  int64_t row = (int64_t)blockIdx.x * nw + warp + zero;
   uint4 cur[NCH], nxt[NCH];
   if (row < a.rows) load_row16<NCH>(a.x, row * a.x_ld, lane, a.cols, cur);
   for (; row < a.rows; row += stride) {
@@ -314,7 +315,8 @@ __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
   // (columns 8 q .. 8 q + 7) are split into a low and a high half; low halves at [4 q, 4 q + 4), high halves
   // kLnHi floats further.
   const int kLnHi = NCH * 32 * 4;
-  for (int j = threadIdx.x; j < a.cols; j += blockDim.x)
+  const int zero = ptx::grid_sync_previous();
+  for (int j = threadIdx.x + zero; j < a.cols; j += blockDim.x)
     w_s[(j >> 3) * 4 + (j & 3) + ((j & 4) ? kLnHi : 0)] = load_one(a.w, a.w_dt, j);
   __syncthreads();
   const int64_t stride = (int64_t)gridDim.x * nw;
@@ -324,7 +326,7 @@ __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
   for (int c = 0; c < NCH; ++c)
 #pragma unroll
     for (int j = 0; j < 4; ++j) { sw[c][j] = pack2(0.f, 0.f); sc[c][j] = pack2(0.f, 0.f); }
-  int64_t row = (int64_t)blockIdx.x * nw + warp;
+  int64_t row = (int64_t)blockIdx.x * nw + warp + zero;
   auto issue = [&](int64_t r, int st) {                        // lane 0
     const uint32_t bar = bars + 8u * st;
     ptx::mbar_expect_tx(bar, slot);
@@ -522,8 +524,9 @@ __global__ void __launch_bounds__(32 * kLnReduceGroups) ln_bwd_reduce_kernel(con
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int j = blockIdx.x * 32 + tx;               // index into [2][cols]
   float s4[4] = {0.f, 0.f, 0.f, 0.f};
+  const int zero = ptx::grid_sync_previous();
   if (j < 2 * cols) {
-    int p = ty;
+    int p = ty + zero;
     for (; p + 3 * kLnReduceGroups < nparts; p += 4 * kLnReduceGroups) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) s4[u] += partial[(size_t)(p + u * kLnReduceGroups) * 2 * cols + j];
@@ -605,11 +608,10 @@ extern "C" us_status us_layer_norm_fwd(const us_mat* X, const us_mat* w, const u
     if (sms <= 0) return US_ERR_CUDA;
     const int pgrid = grid < 2 * sms ? grid : 2 * sms;       // two resident CTAs per SM, warps walk the rows
     const size_t smem = (size_t)2 * a.cols * sizeof(float);
-    if (nch <= 1) ln_fwd16_kernel<1><<<pgrid, kLnThreads, smem, st>>>(a);
-    else if (nch <= 2) ln_fwd16_kernel<2><<<pgrid, kLnThreads, smem, st>>>(a);
-    else if (nch <= 4) ln_fwd16_kernel<4><<<pgrid, kLnThreads, smem, st>>>(a);
-    else ln_fwd16_kernel<8><<<pgrid, kLnThreads, smem, st>>>(a);
-    return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
+    if (nch <= 1) return host::launch(ln_fwd16_kernel<1>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
+    if (nch <= 2) return host::launch(ln_fwd16_kernel<2>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
+    if (nch <= 4) return host::launch(ln_fwd16_kernel<4>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
+    return host::launch(ln_fwd16_kernel<8>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
   }
   if (nch <= 1) ln_fwd_kernel<1><<<grid, kLnThreads, 0, st>>>(a);
   else if (nch <= 2) ln_fwd_kernel<2><<<grid, kLnThreads, 0, st>>>(a);
@@ -673,7 +675,8 @@ extern "C" us_status us_layer_norm_bwd(const us_mat* X, const us_mat* w, const u
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return US_ERR_CUDA;
-    fn<<<nparts, 32 * kLnFastWarps, smem, st>>>(a);
+    const us_status launched = host::launch(fn, nullptr, nparts, 32 * kLnFastWarps, smem, 1, st, a);
+    if (launched != US_OK) return launched;
   } else if (nch <= 4) {
     const size_t smem = (size_t)kLnWarps * a.cols * sizeof(float);
     if (nch <= 1) ln_bwd_kernel<1><<<grid, kLnThreads, smem, st>>>(a);
@@ -687,6 +690,6 @@ extern "C" us_status us_layer_norm_bwd(const us_mat* X, const us_mat* w, const u
   }
   if (cudaGetLastError() != cudaSuccess) return US_ERR_CUDA;
   const int rgrid = (2 * a.cols + 31) / 32;
-  ln_bwd_reduce_kernel<<<rgrid, 32 * kLnReduceGroups, 0, st>>>(a.partial, nparts, a.cols, beta_wc, dw->ptr, dw->dtype, dc->ptr, dc->dtype);
-  return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
+  return host::launch(ln_bwd_reduce_kernel, nullptr, rgrid, 32 * kLnReduceGroups, 0, 1, st, a.partial, nparts, a.cols, beta_wc, dw->ptr,
+                      dw->dtype, dc->ptr, dc->dtype);
 }

@@ -47,6 +47,23 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// ------------------------------------------------------------------ overlap with neighbouring kernels of the stream
+// grid_release_next lets the next kernel of the stream take free SMs from now on (it waits, in its own
+// grid_wait_previous, until this grid has finished); grid_wait_previous returns once the previous kernel has finished
+// and its writes are visible.  Every kernel launched through host::launch calls both, and touches no global memory
+// before the second.  The returned zero goes into the index of the first read, so that no read-only load can be
+// scheduled ahead of the wait.
+__device__ __forceinline__ void grid_release_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ int grid_wait_previous() {
+  int zero;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero)::"memory");
+  return zero;
+}
+__device__ __forceinline__ int grid_sync_previous() {
+  grid_release_next();
+  return grid_wait_previous();
+}
+
 // ------------------------------------------------------------------ TMA (tile mode, 2-D)
 __device__ __forceinline__ void prefetch_tensormap(const void* tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");

@@ -5,6 +5,7 @@
 #include "common.cuh"
 #include "host.h"
 #include "rowwise.cuh"
+#include "sm100.cuh"
 
 namespace us {
 
@@ -140,7 +141,7 @@ template <int NCH>
 __global__ void __launch_bounds__(kSmThreads, 2) softmax_fwd16_kernel(const SmArgs a) {
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int64_t stride = (int64_t)gridDim.x * nw;
-  int64_t row = (int64_t)blockIdx.x * nw + (threadIdx.x >> 5);
+  int64_t row = (int64_t)blockIdx.x * nw + (threadIdx.x >> 5) + ptx::grid_sync_previous();
   uint4 cur[NCH], nxt[NCH];
   if (row < a.rows) load_row16<NCH>(a.in0, row * a.in0_ld, lane, a.cols, cur);
   for (; row < a.rows; row += stride) {
@@ -189,7 +190,7 @@ __global__ void __launch_bounds__(kSmThreads, 2) softmax_bwd16_kernel(const SmAr
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int64_t stride = (int64_t)gridDim.x * nw;
   const float inv_alpha = 1.0f / a.alpha;
-  int64_t row = (int64_t)blockIdx.x * nw + (threadIdx.x >> 5);
+  int64_t row = (int64_t)blockIdx.x * nw + (threadIdx.x >> 5) + ptx::grid_sync_previous();
   uint4 cp[P8 ? 1 : NCH], cg[NCH], np_[P8 ? 1 : NCH], ng[NCH];
   uint2 cp8[P8 ? NCH : 1], np8[P8 ? NCH : 1];
   if (row < a.rows) {
@@ -438,15 +439,14 @@ static us_status launch_softmax(const SmArgs& a, cudaStream_t st) {
     const int pgrid = grid < 2 * sms ? grid : 2 * sms;        // two resident CTAs per SM, warps walk the rows
 #define US_SM16(N)                                                                   \
   do {                                                                               \
-    if (BWD && p8) softmax_bwd16_kernel<N, true><<<pgrid, kSmThreads, 0, st>>>(a);   \
-    else if (BWD) softmax_bwd16_kernel<N, false><<<pgrid, kSmThreads, 0, st>>>(a);   \
-    else softmax_fwd16_kernel<N><<<pgrid, kSmThreads, 0, st>>>(a);                   \
+    if (BWD && p8) return host::launch(softmax_bwd16_kernel<N, true>, nullptr, pgrid, kSmThreads, 0, 1, st, a);  \
+    if (BWD) return host::launch(softmax_bwd16_kernel<N, false>, nullptr, pgrid, kSmThreads, 0, 1, st, a);       \
+    return host::launch(softmax_fwd16_kernel<N>, nullptr, pgrid, kSmThreads, 0, 1, st, a);                       \
   } while (0)
     if (nch <= 1) US_SM16(1);
     else if (nch <= 2) US_SM16(2);
     else US_SM16(4);
 #undef US_SM16
-    return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
   }
 #define US_SM_LAUNCH(N)                                                          \
   do {                                                                           \
