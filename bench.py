@@ -698,7 +698,7 @@ def run_encoder(args, rank, world, local, torch, dev, peaks):
         windows.append((w0, time.time()))
         layer.check()
         ms = e0.elapsed_time(e1) / args.steps
-        results[name] = {"ms_per_step": ms, "tflops": layer.flops() / (ms * 1e-3) / 1e12, "launches": layer.launches_per_step,
+        results[name] = {"ms_per_step": ms, "tflops": layer.flops() / (ms * 1e-3) / 1e12, "launches": layer.kernel_launches,
                               "tokens_per_s": T / (ms * 1e-3)}
         flops = layer.flops()
         del layer, g

@@ -9,17 +9,18 @@
 namespace us {
 namespace {
 
-// Row-major [rows x cols] matrix of es-byte elements, boxes of box_rows rows x 128 bytes, 128-byte swizzle, zero fill.
-bool make_tmap(CUtensorMap* tm, const us_mat* m, int es, int box_rows) {
+// Row-major [rows x cols] matrix of es-byte elements, boxes of box_rows rows x 128 (or 64) bytes, swizzled with that width's pattern, zero fill.
+bool make_tmap(CUtensorMap* tm, const us_mat* m, int es, int box_rows, int box_bytes = 128) {
   host::EncodeTiledFn fn = host::encode_tiled_fn();
   if (!fn) return false;
   const CUtensorMapDataType type = es == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8
                                  : es == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_UINT32;
   cuuint64_t dims[2] = {(cuuint64_t)m->cols, (cuuint64_t)m->rows};
   cuuint64_t strides[1] = {(cuuint64_t)m->ld * es};
-  cuuint32_t box[2] = {(cuuint32_t)(128 / es), (cuuint32_t)box_rows};
+  cuuint32_t box[2] = {(cuuint32_t)(box_bytes / es), (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
-  return fn(tm, type, 2, m->ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+  return fn(tm, type, 2, m->ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -119,21 +120,18 @@ us_status group_impl(int count, const us_linear_call* calls, bool any, void* ws,
   static_assert(sizeof(GroupParams) < 32000, "kernel parameter limit");
   Shape sh[kGroupMaxProblems];
   int64_t pair_tiles = 0;
-  bool fp8_out = false;
   for (int i = 0; i < count; ++i) {
     us_status s = check_call(&calls[i], any, &sh[i]);
     if (s != US_OK) return s;
     if (dtype_size(calls[i].a.dtype) != dtype_size(calls[0].a.dtype)) return US_ERR_UNSUPPORTED;   // one operand width per launch
     pair_tiles += ((sh[i].M + 255) / 256) * ((sh[i].N + 255) / 256);
-    fp8_out = fp8_out || is_fp8(calls[i].out.dtype);
   }
   const int sms = host::sm_count();
   if (sms <= 0) return US_ERR_CUDA;
   const int es = dtype_size(calls[0].a.dtype);
-  // The rule of the single launches: 256 x 256 tiles per CTA pair unless they would leave more than half of the pairs
-  // idle.  (The 64 columns an epilogue warp of a 128 x 128 tile owns do not fill an FP8 output box, so such calls keep
-  // pair tiles.)
-  const bool pair = fp8_out || 4 * pair_tiles >= sms;
+  // 256 x 256 tiles per CTA pair unless they would leave a quarter of the pairs idle (measured over FFN steps, FP8 / BF16,
+  // us: 48 such tiles 14.3 / 19.2 against 10.7 / 17.1 with 128 x 128 tiles, 64 tiles 14.9 / 20.0 against 16.3 / 27.3).
+  const bool pair = 8 * pair_tiles >= 3 * sms;
   const int tile_m = pair ? 256 : 128, bn = pair ? 256 : 128;
   GroupParams g;
   g.count = count;
@@ -151,7 +149,7 @@ us_status group_impl(int count, const us_linear_call* calls, bool any, void* ws,
     P.skip_coef = P.has_skip ? c.ep.skip_coef : 0.f;
     P.out_coef = P.has_skip ? c.ep.out_coef : 1.f;
     if (!make_tmap(&P.ta, &c.a, es, P.a_mn ? 128 / es : 128) || !make_tmap(&P.tb, &c.b, es, P.b_mn ? 128 / es : 128)) return US_ERR_CUDA;
-    if (!make_tmap(&P.tout, &c.out, dtype_size(c.out.dtype), 32)) return US_ERR_CUDA;
+    if (!make_tmap(&P.tout, &c.out, dtype_size(c.out.dtype), 32, !pair && is_fp8(c.out.dtype) ? 64 : 128)) return US_ERR_CUDA;
     P.tskip = P.tout;
     if (P.has_skip && !make_tmap(&P.tskip, &c.ep.skip, dtype_size(c.ep.skip.dtype), 32)) return US_ERR_CUDA;
   }

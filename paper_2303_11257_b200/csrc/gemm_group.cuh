@@ -11,8 +11,7 @@
 //
 // Scope: FP8 or 16-bit operands (all problems of a launch the same width; either layout each), plain
 // or residual (skip) epilogue, any output dtype, up to kGroupMaxProblems problems.  CTA-pair tiles of
-// 256 x 256 (cta_group::2), or, when those would leave more than half of the pairs idle, single-CTA tiles
-// of 128 x 128.  Everything that differs between problems is run-time data here: tensor maps, operand
+// 256 x 256 (cta_group::2), or, when those would leave too many pairs idle, single-CTA tiles of 128 x 128.  Everything that differs between problems is run-time data here: tensor maps, operand
 // layouts (a K-major tile is one box of 128 rows x 128 bytes; an MN-major one has 128 / ES rows of K per
 // box, one box of 128 bytes for FP8 and two for 16-bit elements), instruction descriptor, scale, epilogue kind.
 // Measured, four separate launches -> this one, us: FP8 8192 x 1024 x 4096 122 -> 101; BF16 216 -> 199;
@@ -247,7 +246,10 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
       const int row0 = tm * kTileM + rank * 128 + q * 32, n_w = tn * BN + half * kWarpCols;
       const bool skip = P.has_skip != 0;
       const int in_es = dtype_size(P.skip_dt), out_es = dtype_size(P.out_dt);
-      const int in_box_cols = 128 / in_es, out_box_cols = 128 / out_es;
+      // an output box holds 128-byte rows, or the 64 bytes a warp's 64 columns of FP8 codes are
+      const bool narrow = kWarpCols == 64 && out_es == 1;
+      const int in_box_cols = 128 / in_es, out_box_cols = (narrow ? 64 : 128) / out_es;
+      const uint32_t out_sw = narrow ? (uint32_t)((lane >> 1) & 3) : sw;
       ok = wait_bounded(acc_full_bar(acc), acc_phase, abort_flag, g.status, g.wait_limit);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
@@ -299,7 +301,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
           ptx::tmem_ld_32x32(t_row + 32 * sl, v);
           if (last_slice) { release_acc(); released = true; }
           const uint32_t out_cb = (uint32_t)(out_off * out_es) >> 4;
-          const uint32_t dst = buf_out + row_off;
+          const uint32_t dst = buf_out + (narrow ? (uint32_t)lane * 64u : row_off);
           uint32_t held[2];
 #pragma unroll
           for (int gi = 0; gi < 4; ++gi) {
@@ -330,21 +332,21 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
               for (int k = 0; k < 4; ++k) unpack2(x[k], y[2 * k], y[2 * k + 1]);
             }
             if (P.out_dt == US_F32) {
-              ptx::sts128(dst + (((out_cb + 2 * gi) ^ sw) << 4),
+              ptx::sts128(dst + (((out_cb + 2 * gi) ^ out_sw) << 4),
                           make_uint4(__float_as_uint(y[0]), __float_as_uint(y[1]), __float_as_uint(y[2]), __float_as_uint(y[3])));
-              ptx::sts128(dst + (((out_cb + 2 * gi + 1) ^ sw) << 4),
+              ptx::sts128(dst + (((out_cb + 2 * gi + 1) ^ out_sw) << 4),
                           make_uint4(__float_as_uint(y[4]), __float_as_uint(y[5]), __float_as_uint(y[6]), __float_as_uint(y[7])));
             } else if (P.out_dt == US_BF16 || P.out_dt == US_F16) {
               uint32_t w[4];
 #pragma unroll
               for (int k = 0; k < 4; ++k)
                 w[k] = P.out_dt == US_BF16 ? pack_bf16x2(y[2 * k], y[2 * k + 1]) : pack_f16x2(y[2 * k], y[2 * k + 1]);
-              ptx::sts128(dst + (((out_cb + gi) ^ sw) << 4), make_uint4(w[0], w[1], w[2], w[3]));
+              ptx::sts128(dst + (((out_cb + gi) ^ out_sw) << 4), make_uint4(w[0], w[1], w[2], w[3]));
             } else {
               const uint32_t lo = P.out_dt == US_E5M2 ? cvt_fp8x4<true>(y[0], y[1], y[2], y[3]) : cvt_fp8x4<false>(y[0], y[1], y[2], y[3]);
               const uint32_t hi = P.out_dt == US_E5M2 ? cvt_fp8x4<true>(y[4], y[5], y[6], y[7]) : cvt_fp8x4<false>(y[4], y[5], y[6], y[7]);
               if ((gi & 1) == 0) { held[0] = lo; held[1] = hi; }
-              else ptx::sts128(dst + (((out_cb + (gi >> 1)) ^ sw) << 4), make_uint4(held[0], held[1], lo, hi));
+              else ptx::sts128(dst + (((out_cb + (gi >> 1)) ^ out_sw) << 4), make_uint4(held[0], held[1], lo, hi));
             }
           }
           if (out_off + 32 == out_box_cols || last_slice) {

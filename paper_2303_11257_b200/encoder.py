@@ -97,9 +97,15 @@ class UnitScaledEncoderLayer:
 
     @property
     def launches_per_step(self) -> int:
-        """Kernel launches of one step (without layer norms the FFN block's six GEMMs go out in its grouped forms, as
-        two or three launches, while those cover the shape)."""
+        """Launches of one step with the two gradient GEMMs of a projection counted singly (without layer norms the FFN
+        block's six GEMMs go out in its grouped forms, as two or three launches, while those cover the shape)."""
         return self._launches - (6 - self.ffn.gemm_launches if self.norm is None else 0)
+
+    @property
+    def kernel_launches(self) -> int:
+        """Kernel launches of one step: launches_per_step less one for each projection, and with layer norms the three
+        GEMMs that end the FFN block's backward pass as one."""
+        return self.launches_per_step - 2 - (2 if self.norm is not None and self.ffn.grouped else 0)
 
     def _heads(self, M, which):
         """Problem (0, 0) of a [T x 3d] matrix: rows of the first sequence, columns of head 0 of Q / K / V."""
@@ -147,8 +153,9 @@ class UnitScaledEncoderLayer:
         else:
             f.backward(G, stream, cast_g=False)                     # f.dX = dL/dR1
             g1 = f.dX
-        # The weight-gradient GEMMs and one GEMM of each attention pair depend only on tensors that exist
-        # already; with no explicit stream they go to a side stream (parallel branches under graph capture).
+        # The two gradient GEMMs of a projection are independent of one another and go out as one launch, the weight
+        # gradient's long contractions dealt out first.  One GEMM of each attention pair depends only on tensors that
+        # exist already; with no explicit stream it goes to a side stream (a parallel branch under graph capture).
         par = stream is None and f.concurrent
         cur = torch.cuda.current_stream() if par else stream
         side = f._side_streams()[0] if par else stream
@@ -162,8 +169,8 @@ class UnitScaledEncoderLayer:
             fn(side)
 
         L.us_cast_fp8(g1, 1.0, self.g1q, cur)
-        beside(lambda st: L.us_linear_bwd_w(self.Cq, self.g1q, sc["beta_w"], self.dWo, ws, None, st))
-        L.us_linear_bwd_x(self.g1q, self.Wo_q, sc["beta_o"], self.dC, ws, None, cur)
+        L.linear_together([L.linear_call(L.US_OP_BWD_W, self.Cq, self.g1q, sc["beta_w"], self.dWo),
+                           L.linear_call(L.US_OP_BWD_X, self.g1q, self.Wo_q, sc["beta_o"], self.dC)], ws, cur)
         dC_h = self.dC[:s, : self.hd]
         beside(lambda st: L.us_linear_bwd_w_batched(self.P[:s], dC_h, sc["beta_V"], self._heads(self.dQKV, 2), self.bt["dV"], ws, st))
         if self.fused_attention:
@@ -179,11 +186,9 @@ class UnitScaledEncoderLayer:
             cur.wait_stream(side)                                   # dQ, dK, dV all written
         if self.dQKV is not self.dQKVq:
             L.us_cast_fp8(self.dQKV, 1.0, self.dQKVq, cur)
-        beside(lambda st: L.us_linear_bwd_w(self.Xq, self.dQKVq, sc["beta_w"], self.dWqkv, ws, None, st))
         ep = L.epilogue(skip=g1, skip_coef=self.c_skip, out_coef=self.c_branch)
-        L.us_linear_bwd_x(self.dQKVq, self.Wqkv_q, sc["beta_qkv"], self.dX, ws, ep, cur)
-        if par:
-            cur.wait_stream(side)
+        L.linear_together([L.linear_call(L.US_OP_BWD_W, self.Xq, self.dQKVq, sc["beta_w"], self.dWqkv),
+                           L.linear_call(L.US_OP_BWD_X, self.dQKVq, self.Wqkv_q, sc["beta_qkv"], self.dX, ep)], ws, cur)
         return self.dX
 
     def check(self) -> None:

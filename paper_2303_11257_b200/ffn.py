@@ -175,12 +175,16 @@ class UnitScaledFFN:
     def group_calls(self, X, G):
         """The four GEMMs that follow the GELU-gradient GEMM, as the entries of one us_linear_group launch
         (same operands, scales and epilogues as the stages fwd2_residual, bwd_w2, bwd_x1_residual, bwd_w1)."""
-        sc, (c_skip, c_branch) = self.sc, self._c
-        ep2 = L.epilogue(skip=X, skip_coef=c_skip, out_coef=c_branch)
-        ep5 = L.epilogue(skip=G, skip_coef=c_skip, out_coef=c_branch)
+        ep2 = L.epilogue(skip=X, skip_coef=self._c[0], out_coef=self._c[1])
+        w2, w1, x1 = self.backward_calls(G)
+        return [w2, w1, L.linear_call(L.US_OP_FWD, self.Aq, self.W2q, self.sc.alpha2, self.R, ep2), x1]
+
+    def backward_calls(self, G):
+        """The GEMMs that follow the GELU-gradient GEMM in a backward pass of its own: bwd_w2, bwd_w1, bwd_x1_residual."""
+        sc = self.sc
+        ep5 = L.epilogue(skip=G, skip_coef=self._c[0], out_coef=self._c[1])
         return [L.linear_call(L.US_OP_BWD_W, self.Aq, self.Gq, sc.beta_w, self.dW2),
                 L.linear_call(L.US_OP_BWD_W, self.Xq, self.dHq, sc.beta_w, self.dW1),
-                L.linear_call(L.US_OP_FWD, self.Aq, self.W2q, sc.alpha2, self.R, ep2),
                 L.linear_call(L.US_OP_BWD_X, self.dHq, self.W1q, sc.beta_x1, self.dX, ep5)]
 
     def _hidden(self, stream=None):
@@ -206,9 +210,16 @@ class UnitScaledFFN:
 
     def backward(self, G, stream=None, cast_g: bool = True):
         """Backward pass from G = dL/dR.  cast_g=False: self.Gq already holds q(G) (a caller that
-        quantised G together with other tensors in one us_cast_fp8_multi launch).  With self.concurrent and
-        no explicit stream the two weight-gradient GEMMs run on side streams beside the input-gradient ones."""
+        quantised G together with other tensors in one us_cast_fp8_multi launch).  The three GEMMs that remain once
+        the hidden layer's gradient is there go out as one launch while self.grouped is set; without it, with
+        self.concurrent and no explicit stream, the weight-gradient GEMMs run on side streams."""
         st = self.stages(None, None, None, G, fused_casts=False)[5 if cast_g else 6:]
+        if self.grouped:
+            for name, _, fn in st:
+                if name in ("cast_G", "bwd_x2_gelu_grad"):
+                    fn(stream)
+            L.linear_together(self.backward_calls(G), self.ws, stream)
+            return self.dX, self.dW1, self.dW2
         if not (self.concurrent and stream is None):
             for name, _, fn in st:
                 fn(stream)

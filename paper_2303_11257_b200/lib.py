@@ -248,6 +248,24 @@ def us_linear_group_any(calls, ws, stream=None):
     us_linear_group(calls, ws, stream, "us_linear_group_any")
 
 
+def linear_each(calls, ws, stream=None):
+    """The same ops as single launches, in order (for a group with more tiles than the grouped form's work list holds)."""
+    for c in calls:
+        name = ("us_linear_fwd", "us_linear_bwd_x", "us_linear_bwd_w")[c.op]
+        _check(name, getattr(_lib, name)(C.byref(c.a), C.byref(c.b), c.scale, C.byref(c.ep), C.byref(c.out), ws.data_ptr(),
+                                         ws.numel() * ws.element_size(), _stream(stream)))
+
+
+def linear_together(calls, ws, stream=None):
+    """The ops as one launch, or one by one where the grouped form does not cover them."""
+    try:
+        us_linear_group_any(calls, ws, stream)
+    except UnitScaleError as e:
+        if e.status != US_ERR_UNSUPPORTED:
+            raise
+        linear_each(calls, ws, stream)
+
+
 def batch(count, a_stride, b_stride, out_stride) -> us_batch:
     """us_batch from (outer, inner) pairs of counts and element strides."""
     b = us_batch()

@@ -90,7 +90,7 @@ def encoder_step(nseq=16, slen=512, d=1024, nhead=16, d_ff=4096, iters=10, atten
     layer.check()
     t = e0.elapsed_time(e1) * 1e-3 / iters
     return {"workload": f"encoder layer fwd+bwd 16x512 tokens, d=1024, 16 heads, d_ff=4096, {attention} attention operands" + (", post-norm" if norm else ""), "ms_per_step": t * 1e3,
-            "tflops": layer.flops() / t / 1e12, "tokens_per_s": T / t, "launches": layer.launches_per_step}
+            "tflops": layer.flops() / t / 1e12, "tokens_per_s": T / t, "launches": layer.kernel_launches}
 
 
 if __name__ == "__main__":

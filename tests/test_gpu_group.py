@@ -129,3 +129,17 @@ def test_group_any_equals_single_calls(fmt, b, m, n):
     assert L.us_workspace_status(ws) == 0
     for a, r in zip(*outs):
         assert torch.equal(a.contiguous().view(torch.uint8), r.contiguous().view(torch.uint8))
+
+
+@pytest.mark.parametrize("out_fmt", ["e5m2", "e4m3"])
+def test_group_any_fp8_outputs_of_small_tiles(out_fmt):
+    """FP8 results of 128 x 128 tiles leave by 64-byte boxes: ragged columns and a second tile."""
+    L, synth = _mods()
+    ws = L.new_workspace()
+    for b, m, n in ((40, 208, 80), (200, 64, 176)):
+        G, W = U.to_device(synth.normal(50, 0, (b, n)), "e5m2"), U.to_device(synth.normal(50, 1, (m, n)), "e4m3")
+        o, r = U.empty(b, m, out_fmt), U.empty(b, m, out_fmt)
+        L.us_linear_group_any([L.linear_call(L.US_OP_BWD_X, G, W, n ** -0.5, o)], ws)
+        L.us_linear_bwd_x(G, W, n ** -0.5, r, ws)
+        assert np.array_equal(U.codes_of(o), U.codes_of(r))
+    assert L.us_workspace_status(ws) == 0
