@@ -72,6 +72,7 @@ class UnitScaledEncoderLayer:
         self.dX = e(T, d, torch.bfloat16)
         self.dWqkv, self.dWo = e(d, 3 * d, torch.float32), e(d, d, torch.float32)
         self.ws = L.new_workspace(device)
+        self._plan, self._fork, self._join = None, torch.cuda.Event(), torch.cuda.Event()
         if norm == "post":
             # post-norm (appendix "Model architectures"): a scaled layer norm after each residual sum
             self.U1, self.R2 = e(T, d, torch.bfloat16), e(T, d, torch.bfloat16)
@@ -112,9 +113,125 @@ class UnitScaledEncoderLayer:
         o = which * self.d
         return M[: self.slen, o:o + self.hd]
 
+    # ---- a step as calls laid out once over the layer's buffers (L.Plan), in the order of _step_each.  An entry is
+    # (where, call): on the main stream; on the side stream once all that was issued before has finished; or (JOIN, None),
+    # after which the main stream waits for the side stream.
+    MAIN, SIDE, JOIN = range(3)
+
+    def _owned(self):
+        own = (self.Xq, self.Wqkv_q, self.Wo_q, self.QKV, self.P, self.Cq, self.R1, self.g1q, self.dC, self.dS, self.dQKVq, self.dQKV,
+               self.dX, self.dWqkv, self.dWo, self.ws) + self.ffn._owned()
+        if not self.fused_attention:
+            own += (self.S, self.dP)
+        if self.norm == "post":
+            own += (self.U1, self.R2, self.dU1, self.dU2, self.ln_ws, *self.dln)
+        return own
+
+    def _state(self):
+        return (*self.sc.values(), self.c_skip, self.c_branch, self.eps, self.beta_ln if self.norm else 0.0) + self.ffn._state()
+
+    def _lay_out(self, p):
+        sc, ws, s, f = self.sc, self.ws, self.slen, self.ffn
+        post, fused = self.norm == "post", self.fused_attention
+        coef = (self.c_skip, self.c_branch)
+        Q, K, V = (self._heads(self.QKV, i) for i in range(3))
+        dQ, dK, dV = (self._heads(self.dQKV, i) for i in range(3))
+        P, dS, C_h, dC_h = self.P[:s], self.dS[:s], self.Cq[:s, : self.hd], self.dC[:s, : self.hd]
+        tail = (ws.data_ptr(), ws.numel())
+        MAIN = self.MAIN
+
+        def norm_bwd(X, w, G, dX, dw, dc):
+            g = p.slot(G) if isinstance(G, str) else L.mat(G)
+            return L.Call("us_layer_norm_bwd", L.mat(X), p.slot(w), g, self.eps, 1.0, self.beta_ln, L.mat(dX), L._vec(dw), L._vec(dc),
+                          self.ln_ws.data_ptr(), self.ln_ws.numel())
+
+        yield MAIN, p.cast_multi(["Wqkv", "Wo", "X", "W1", "W2"] + ([] if post else ["G"]),
+                                 [self.Wqkv_q, self.Wo_q, self.Xq, f.W1q, f.W2q] + ([] if post else [f.Gq]))
+        yield MAIN, p.linear("us_linear_fwd", self.Xq, self.Wqkv_q, sc["alpha_qkv"], self.QKV, ws)
+        if fused:
+            yield MAIN, L.Call("us_attention_fwd", L.mat(Q), L.mat(K), L.mat(V), sc["alpha_s"], sc["sm"], sc["alpha_c"], L.mat(C_h), L.mat(P),
+                               self.bt_fused, *tail)
+        else:
+            yield MAIN, p.batched("us_linear_bwd_x_batched", Q, K, sc["alpha_s"], self.S[:s], self.bt["scores"], ws)
+            yield MAIN, L.Call("us_softmax_fwd", L.mat(self.S), sc["sm"], L.mat(self.P))
+            yield MAIN, p.batched("us_linear_fwd_batched", P, V, sc["alpha_c"], C_h, self.bt["ctx"], ws)
+        yield MAIN, p.linear("us_linear_fwd", self.Cq, self.Wo_q, sc["alpha_o"], self.U1 if post else self.R1, ws, p.residual("X", coef))
+        if post:
+            yield MAIN, L.Call("us_layer_norm_fwd", L.mat(self.U1), p.slot("w1"), p.slot("c1"), self.eps, L.mat(self.R1))
+            for c in f.plan_forward(p, self.R1):
+                yield MAIN, c
+            yield MAIN, L.Call("us_layer_norm_fwd", L.mat(f.R), p.slot("w2"), p.slot("c2"), self.eps, L.mat(self.R2))
+            yield MAIN, norm_bwd(f.R, "w2", "G", self.dU2, self.dln[2], self.dln[3])
+            for c in f.plan_backward(p, self.dU2):
+                yield MAIN, c
+            yield MAIN, norm_bwd(self.U1, "w1", f.dX, self.dU1, self.dln[0], self.dln[1])
+            g1 = self.dU1
+        else:
+            yield MAIN, f._plan_cast(p, self.R1, f.Xq)
+            for c in f.plan_gemms(p, self.R1, "G"):
+                yield MAIN, c
+            g1 = f.dX
+        yield MAIN, L.Call("us_cast_fp8", L.mat(g1), 1.0, L.mat(self.g1q))
+        yield MAIN, p.group([(L.US_OP_BWD_W, self.Cq, self.g1q, sc["beta_w"], self.dWo, None, None),
+                             (L.US_OP_BWD_X, self.g1q, self.Wo_q, sc["beta_o"], self.dC, None, None)], ws)
+        yield self.SIDE, p.batched("us_linear_bwd_w_batched", P, dC_h, sc["beta_V"], dV, self.bt["dV"], ws)
+        gemm_dk = p.batched("us_linear_bwd_w_batched", dS, Q, sc["beta_K"], dK, self.bt["dK"], ws)
+        if fused:
+            yield MAIN, L.Call("us_attention_bwd", L.mat(dC_h), L.mat(P), L.mat(K), L.mat(V), sc["beta_P"], sc["sm"], sc["sm"], sc["beta_Q"],
+                               L.mat(dS), L.mat(dQ), self.bt_fused_bwd, *tail)
+            yield self.SIDE, gemm_dk
+        else:
+            yield MAIN, p.batched("us_linear_bwd_x_batched", dC_h, V, sc["beta_P"], self.dP[:s], self.bt["dP"], ws)
+            yield MAIN, L.Call("us_softmax_bwd", L.mat(self.P), L.mat(self.dP), sc["sm"], sc["sm"], L.mat(self.dS))
+            yield self.SIDE, gemm_dk
+            yield MAIN, p.batched("us_linear_fwd_batched", dS, K, sc["beta_Q"], dQ, self.bt["dQ"], ws)
+        yield self.JOIN, None                                       # dQ, dK, dV all written
+        if self.dQKV is not self.dQKVq:
+            yield MAIN, L.Call("us_cast_fp8", L.mat(self.dQKV), 1.0, L.mat(self.dQKVq))
+        yield MAIN, p.group([(L.US_OP_BWD_W, self.Xq, self.dQKVq, sc["beta_w"], self.dWqkv, None, None),
+                             (L.US_OP_BWD_X, self.dQKVq, self.Wqkv_q, sc["beta_qkv"], self.dX, g1, coef)], ws)
+
+    def _run(self, stream, **inputs):
+        owned, state = self._owned(), self._state()
+        p = self._plan
+        if p is None or not p.same(owned, state):
+            p = self._plan = L.Plan(owned, state)
+        for name, t in inputs.items():
+            p.put(name, t)
+        if not (stream is None and self.ffn.concurrent):
+            st = L._stream(stream)
+            for where, call in p.calls(self._lay_out):
+                if call is not None:
+                    call(st)
+            return
+        cur, side = torch.cuda.current_stream(), self.ffn._side_streams()[0]
+        st, side_st = cur.cuda_stream, side.cuda_stream
+        for where, call in p.calls(self._lay_out):
+            if where == self.MAIN:
+                call(st)
+            elif where == self.SIDE:
+                self._fork.record(cur)
+                side.wait_event(self._fork)
+                call(side_st)
+            else:
+                self._join.record(side)
+                cur.wait_event(self._join)
+
     def step(self, X, Wqkv, Wo, W1, W2, G, stream=None, ln=None):
         """One forward + backward pass.  G is the gradient of the layer output; with norm = "post",
         ln = (w1, c1, w2, c2) are the weights and biases of the two layer norms ([d] each)."""
+        if self.ffn.grouped and self.ffn.fused_hidden:
+            norm = dict(zip(("w1", "c1", "w2", "c2"), (t.view(1, -1) for t in ln))) if self.norm == "post" else {}
+            try:
+                self._run(stream, X=X, Wqkv=Wqkv, Wo=Wo, W1=W1, W2=W2, G=G, **norm)
+                return self.dX
+            except L.UnitScaleError as e:
+                if e.status != L.US_ERR_UNSUPPORTED:
+                    raise                                           # else: what a grouped form does not cover goes out singly
+        return self._step_each(X, Wqkv, Wo, W1, W2, G, stream, ln)
+
+    def _step_each(self, X, Wqkv, Wo, W1, W2, G, stream, ln):
+        """step() call by call."""
         sc, ws, s = self.sc, self.ws, self.slen
         post = self.norm == "post"
         # ---- forward

@@ -99,6 +99,77 @@ class UnitScaledFFN:
         # 16-bit operand mode and blocks with a dimension of at most 128 always do; backward() reads it from there).
         self.fused_hidden = operand == "fp8" or h_dtype in (torch.bfloat16, torch.float16)
         self.keep_h = keep_h
+        self._plans = {}
+
+    # ---- the calls of a pass over this block's buffers, laid out once (L.Plan): a step's host time is then its three C
+    # calls.  They are used while the block issues the launches it issues by default; stages() is the general form.
+    def _owned(self):
+        return (self.Xq, self.W1q, self.W2q, self.Gq, self.H, self.Aq, self.dHq, self.R, self.dX, self.dW1, self.dW2, self.ws)
+
+    def _state(self):
+        sc = self.sc
+        return (sc.alpha1, sc.alpha2, sc.beta_x1, sc.beta_x2, sc.beta_w, sc.alpha_g, sc.beta_g, sc.s_in, self._c, self.keep_h, self.operand)
+
+    def _run(self, kind, stream, **inputs):
+        owned, state = self._owned(), self._state()
+        p = self._plans.get(kind)
+        if p is None or not p.same(owned, state):
+            p = self._plans[kind] = L.Plan(owned, state)
+        for name, t in inputs.items():
+            p.put(name, t)
+        st = L._stream(stream)
+        for call in p.calls(getattr(self, "_plan_" + kind)):
+            call(st)
+
+    def _plan_cast(self, p, src, dst):
+        m = p.slot(src) if isinstance(src, str) else L.mat(src)
+        return L.Call("us_cast_fp8", m, 1.0, L.mat(dst)) if self.operand == "fp8" else L.Call("us_residual_add", m, m, 0.0, L.mat(dst))
+
+    def _plan_step(self, p):
+        yield p.cast_multi(["W1", "W2", "X", "G"], [self.W1q, self.W2q, self.Xq, self.Gq])
+        yield from self.plan_gemms(p, "X", "G")
+
+    def _plan_forward(self, p):
+        return self.plan_forward(p, "X")
+
+    def _plan_backward(self, p):
+        return self.plan_backward(p, "G")
+
+    def _plan_backward_from_cast(self, p):
+        return self.plan_backward(p, "G", cast_g=False)
+
+    def plan_gemms(self, p, X, G):
+        """step_from_casts() as prepared calls; X, G: the skip inputs, tensors or names of inputs."""
+        sc = self.sc
+        keep = self.keep_h or self.operand != "fp8" or min(self.T, self.d, self.f) <= 128
+        yield L.Call("us_ffn_hidden_any", L.mat(self.Xq), L.mat(self.W1q), sc.alpha1, L.mat(self.Gq), L.mat(self.W2q), sc.beta_x2,
+                     sc.s_in, sc.alpha_g, sc.beta_g, L._TORCH_DTYPES[self.H.dtype], L.mat(self.H) if keep else None,
+                     L.mat(self.Aq), L.mat(self.dHq), self.ws.data_ptr(), self.ws.numel())
+        w2, w1, x1 = self._plan_backward_entries(G)
+        yield p.group([w2, w1, (L.US_OP_FWD, self.Aq, self.W2q, sc.alpha2, self.R, X, self._c), x1], self.ws)
+
+    def plan_forward(self, p, X):
+        """forward() as prepared calls."""
+        sc = self.sc
+        ep1 = L.epilogue(act=L.US_ACT_GELU, act_in_scale=sc.s_in, act_out_scale=sc.alpha_g, aux=self.H)
+        yield self._plan_cast(p, X, self.Xq)
+        yield p.linear("us_linear_fwd", self.Xq, self.W1q, sc.alpha1, self.Aq, self.ws, ep1)
+        yield p.linear("us_linear_fwd", self.Aq, self.W2q, sc.alpha2, self.R, self.ws, p.residual(X, self._c))
+
+    def plan_backward(self, p, G, cast_g=True):
+        """backward() as prepared calls."""
+        sc = self.sc
+        ep3 = L.epilogue(act=L.US_ACT_GELU_GRAD, act_in_scale=sc.s_in, act_out_scale=sc.beta_g, aux=self.H)
+        if cast_g:
+            yield self._plan_cast(p, G, self.Gq)
+        yield p.linear("us_linear_bwd_x", self.Gq, self.W2q, sc.beta_x2, self.dHq, self.ws, ep3)
+        yield p.group(self._plan_backward_entries(G), self.ws)
+
+    def _plan_backward_entries(self, G):
+        sc = self.sc
+        return [(L.US_OP_BWD_W, self.Aq, self.Gq, sc.beta_w, self.dW2, None, None),
+                (L.US_OP_BWD_W, self.Xq, self.dHq, sc.beta_w, self.dW1, None, None),
+                (L.US_OP_BWD_X, self.dHq, self.W1q, sc.beta_x1, self.dX, G, self._c)]
 
     @property
     def gemm_launches(self) -> int:
@@ -199,8 +270,7 @@ class UnitScaledFFN:
         self._cast(W2, self.W2q, stream)
 
     def forward(self, X, stream=None):
-        for name, _, fn in self.stages(X, None, None, None, fused_casts=False)[2:5]:
-            fn(stream)
+        self._run("forward", stream, X=X)
         return self.R
 
     def _side_streams(self):
@@ -213,13 +283,15 @@ class UnitScaledFFN:
         quantised G together with other tensors in one us_cast_fp8_multi launch).  The three GEMMs that remain once
         the hidden layer's gradient is there go out as one launch while self.grouped is set; without it, with
         self.concurrent and no explicit stream, the weight-gradient GEMMs run on side streams."""
-        st = self.stages(None, None, None, G, fused_casts=False)[5 if cast_g else 6:]
         if self.grouped:
-            for name, _, fn in st:
-                if name in ("cast_G", "bwd_x2_gelu_grad"):
-                    fn(stream)
-            L.linear_together(self.backward_calls(G), self.ws, stream)
-            return self.dX, self.dW1, self.dW2
+            try:
+                self._run("backward" if cast_g else "backward_from_cast", stream, G=G)
+                return self.dX, self.dW1, self.dW2
+            except L.UnitScaleError as e:
+                if e.status != L.US_ERR_UNSUPPORTED:
+                    raise
+                self.grouped = False                            # more tiles than the grouped form's work list holds
+        st = self.stages(None, None, None, G, fused_casts=False)[5 if cast_g else 6:]
         if not (self.concurrent and stream is None):
             for name, _, fn in st:
                 fn(stream)
@@ -247,6 +319,13 @@ class UnitScaledFFN:
 
         With self.concurrent and no explicit stream, independent GEMMs go to two side streams that fork from
         and join back into the current stream (this also records as parallel branches under graph capture)."""
+        if self.grouped and self.fused_casts and self.fused_hidden:
+            try:
+                self._run("step", stream, X=X, W1=W1, W2=W2, G=G)
+                return self.dX, self.dW1, self.dW2
+            except L.UnitScaleError as e:
+                if e.status not in (L.US_ERR_UNSUPPORTED, L.US_ERR_ALIGNMENT):
+                    raise                                       # else: what is not covered goes out in its general form
         st = self.stages(X, W1, W2, G)
         if self.grouped and self.fused_casts:
             cast_all = next(fn for name, _, fn in st if name == "cast_all")

@@ -7,6 +7,7 @@ compiled library: there is no fallback of any kind.
 from __future__ import annotations
 
 import ctypes as C
+import operator
 import os
 
 import torch
@@ -159,18 +160,125 @@ def raw() -> C.CDLL:
     return _lib
 
 
+def describe(t: torch.Tensor) -> tuple:
+    """The fields of a us_mat for a 2-D row-major torch tensor (last stride 1)."""
+    shape, stride = t.shape, t.stride()
+    if len(shape) != 2 or (shape[1] > 1 and stride[1] != 1):
+        raise ValueError("expected a 2-D tensor with unit column stride")
+    rows, cols = shape
+    return t.data_ptr(), _TORCH_DTYPES[t.dtype], rows, cols, stride[0] if rows > 1 else max(cols, stride[0])
+
+
 def mat(t: torch.Tensor) -> us_mat:
     """Describe a 2-D row-major torch tensor (last stride 1) without copying it."""
-    if t.dim() != 2 or (t.shape[1] > 1 and t.stride(1) != 1):
-        raise ValueError("expected a 2-D tensor with unit column stride")
-    ld = t.stride(0) if t.shape[0] > 1 else max(t.shape[1], t.stride(0))
-    return us_mat(t.data_ptr(), _TORCH_DTYPES[t.dtype], t.shape[0], t.shape[1], ld)
+    return us_mat(*describe(t))
+
+
+def current_stream() -> int:
+    """Handle of the current device's current stream.  Asks torch's C layer for the handle itself (0.4 us, against 3.4 us
+    for making a Stream object of it); every launch asks."""
+    if torch.cuda.is_initialized():
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
+
+
+class Call:
+    """A library call whose arguments are laid out once: calling it costs the C call and little else.  It points into
+    tensors that the caller keeps (a block's own buffers); descriptions that change from call to call -- the tensors a
+    user passes to a step -- are written into its us_mat slots before each call (Plan.put)."""
+    __slots__ = ("name", "fn", "args", "keep")
+
+    def __init__(self, name, *args):
+        self.name, self.fn, self.keep = name, getattr(_lib, name), args
+        self.args = tuple(C.byref(a) if isinstance(a, C.Structure) else a for a in args)
+
+    def __call__(self, stream: int) -> None:
+        status = self.fn(*self.args, stream)
+        if status != US_OK:
+            raise UnitScaleError(self.name, status)
+
+
+class Plan:
+    """The calls of one pass over an object's own buffers, and the slots its inputs go to.  `owned` are those buffers,
+    `state` every other value the calls were laid out for: same() says whether both are still what they were.
+    calls(lay_out): lay_out(plan) yields the calls in order; the first pass issues each as soon as it is laid out."""
+
+    def __init__(self, owned, state):
+        self.owned, self.state, self.ptrs = owned, state, [t.data_ptr() for t in owned]
+        self.slots, self.inputs, self.done = {}, {}, None
+
+    def same(self, owned, state) -> bool:
+        return self.state == state and all(map(operator.is_, owned, self.owned)) and [t.data_ptr() for t in owned] == self.ptrs
+
+    def slot(self, name: str, m: us_mat = None) -> us_mat:
+        """A us_mat (m, or a new one) that put() fills for the input `name`."""
+        m = us_mat() if m is None else m
+        self.slots.setdefault(name, []).append(m)
+        m.ptr, m.dtype, m.rows, m.cols, m.ld = self.inputs[name]
+        return m
+
+    def put(self, name: str, t: torch.Tensor) -> None:
+        d = self.inputs[name] = describe(t)
+        for m in self.slots.get(name, ()):
+            m.ptr, m.dtype, m.rows, m.cols, m.ld = d
+
+    def calls(self, lay_out):
+        """The calls of a pass whose inputs have been put."""
+        return self.done if self.done is not None else self._first(lay_out)
+
+    def _first(self, lay_out):
+        self.slots, made = {}, []
+        for c in lay_out(self):
+            made.append(c)
+            yield c
+        self.done = made                                        # a pass that ended early is laid out again
+
+    def cast_multi(self, srcs, dsts):
+        """us_cast_multi at scale 1; an entry of srcs is a tensor or the name of an input."""
+        n = len(srcs)
+        sm = (us_mat * n)()
+        for i, s in enumerate(srcs):
+            if isinstance(s, str):
+                self.slot(s, sm[i])
+            else:
+                sm[i] = mat(s)
+        return Call("us_cast_multi", n, sm, (C.c_float * n)(*[1.0] * n), (us_mat * n)(*[mat(t) for t in dsts]))
+
+    def residual(self, skip, coef):
+        """The fixed(tau) residual epilogue; skip is a tensor or the name of an input."""
+        ep = us_epilogue()
+        ep.act, ep.act_in_scale, ep.act_out_scale, ep.skip_coef, ep.out_coef = US_ACT_NONE, 1.0, 1.0, *coef
+        if isinstance(skip, str):
+            self.slot(skip, ep.skip)
+        else:
+            ep.skip = mat(skip)
+        return ep
+
+    def group(self, entries, ws):
+        """us_linear_group_any over (op, a, b, scale, out, skip or None, (skip_coef, out_coef))."""
+        arr = (us_linear_call * len(entries))()
+        for c, (op, a, b, scale, out, skip, coef) in zip(arr, entries):
+            c.op, c.a, c.b, c.scale, c.out, c.ep.out_coef = op, mat(a), mat(b), scale, mat(out), 1.0
+            if skip is not None:
+                c.ep.act_in_scale = c.ep.act_out_scale = 1.0
+                c.ep.skip_coef, c.ep.out_coef = coef
+                if isinstance(skip, str):
+                    self.slot(skip, c.ep.skip)
+                else:
+                    c.ep.skip = mat(skip)
+        return Call("us_linear_group_any", len(entries), arr, ws.data_ptr(), ws.numel())
+
+    def linear(self, name, a, b, scale, out, ws, ep=None):
+        return Call(name, mat(a), mat(b), scale, ep, mat(out), ws.data_ptr(), ws.numel())
+
+    def batched(self, name, a, b, scale, out, bt, ws):
+        return Call(name, mat(a), mat(b), scale, mat(out), bt, ws.data_ptr(), ws.numel())
 
 
 def _check(fn: str, status: int) -> None:
