@@ -141,26 +141,26 @@ class UnitScaledEncoderLayer:
         MAIN = self.MAIN
 
         def norm_bwd(X, w, G, dX, dw, dc):
-            g = p.slot(G) if isinstance(G, str) else L.mat(G)
-            return L.Call("us_layer_norm_bwd", L.mat(X), p.slot(w), g, self.eps, 1.0, self.beta_ln, L.mat(dX), L._vec(dw), L._vec(dc),
+            g = p.slot(G) if isinstance(G, str) else p.mat(G)
+            return L.Call("us_layer_norm_bwd", p.mat(X), p.slot(w), g, self.eps, 1.0, self.beta_ln, p.mat(dX), L._vec(dw), L._vec(dc),
                           self.ln_ws.data_ptr(), self.ln_ws.numel())
 
         yield MAIN, p.cast_multi(["Wqkv", "Wo", "X", "W1", "W2"] + ([] if post else ["G"]),
                                  [self.Wqkv_q, self.Wo_q, self.Xq, f.W1q, f.W2q] + ([] if post else [f.Gq]))
         yield MAIN, p.linear("us_linear_fwd", self.Xq, self.Wqkv_q, sc["alpha_qkv"], self.QKV, ws)
         if fused:
-            yield MAIN, L.Call("us_attention_fwd", L.mat(Q), L.mat(K), L.mat(V), sc["alpha_s"], sc["sm"], sc["alpha_c"], L.mat(C_h), L.mat(P),
+            yield MAIN, L.Call("us_attention_fwd", p.mat(Q), p.mat(K), p.mat(V), sc["alpha_s"], sc["sm"], sc["alpha_c"], p.mat(C_h), p.mat(P),
                                self.bt_fused, *tail)
         else:
             yield MAIN, p.batched("us_linear_bwd_x_batched", Q, K, sc["alpha_s"], self.S[:s], self.bt["scores"], ws)
-            yield MAIN, L.Call("us_softmax_fwd", L.mat(self.S), sc["sm"], L.mat(self.P))
+            yield MAIN, L.Call("us_softmax_fwd", p.mat(self.S), sc["sm"], p.mat(self.P))
             yield MAIN, p.batched("us_linear_fwd_batched", P, V, sc["alpha_c"], C_h, self.bt["ctx"], ws)
         yield MAIN, p.linear("us_linear_fwd", self.Cq, self.Wo_q, sc["alpha_o"], self.U1 if post else self.R1, ws, p.residual("X", coef))
         if post:
-            yield MAIN, L.Call("us_layer_norm_fwd", L.mat(self.U1), p.slot("w1"), p.slot("c1"), self.eps, L.mat(self.R1))
+            yield MAIN, L.Call("us_layer_norm_fwd", p.mat(self.U1), p.slot("w1"), p.slot("c1"), self.eps, p.mat(self.R1))
             for c in f.plan_forward(p, self.R1):
                 yield MAIN, c
-            yield MAIN, L.Call("us_layer_norm_fwd", L.mat(f.R), p.slot("w2"), p.slot("c2"), self.eps, L.mat(self.R2))
+            yield MAIN, L.Call("us_layer_norm_fwd", p.mat(f.R), p.slot("w2"), p.slot("c2"), self.eps, p.mat(self.R2))
             yield MAIN, norm_bwd(f.R, "w2", "G", self.dU2, self.dln[2], self.dln[3])
             for c in f.plan_backward(p, self.dU2):
                 yield MAIN, c
@@ -171,23 +171,23 @@ class UnitScaledEncoderLayer:
             for c in f.plan_gemms(p, self.R1, "G"):
                 yield MAIN, c
             g1 = f.dX
-        yield MAIN, L.Call("us_cast_fp8", L.mat(g1), 1.0, L.mat(self.g1q))
+        yield MAIN, L.Call("us_cast_fp8", p.mat(g1), 1.0, p.mat(self.g1q))
         yield MAIN, p.group([(L.US_OP_BWD_W, self.Cq, self.g1q, sc["beta_w"], self.dWo, None, None),
                              (L.US_OP_BWD_X, self.g1q, self.Wo_q, sc["beta_o"], self.dC, None, None)], ws)
         yield self.SIDE, p.batched("us_linear_bwd_w_batched", P, dC_h, sc["beta_V"], dV, self.bt["dV"], ws)
         gemm_dk = p.batched("us_linear_bwd_w_batched", dS, Q, sc["beta_K"], dK, self.bt["dK"], ws)
         if fused:
-            yield MAIN, L.Call("us_attention_bwd", L.mat(dC_h), L.mat(P), L.mat(K), L.mat(V), sc["beta_P"], sc["sm"], sc["sm"], sc["beta_Q"],
-                               L.mat(dS), L.mat(dQ), self.bt_fused_bwd, *tail)
+            yield MAIN, L.Call("us_attention_bwd", p.mat(dC_h), p.mat(P), p.mat(K), p.mat(V), sc["beta_P"], sc["sm"], sc["sm"], sc["beta_Q"],
+                               p.mat(dS), p.mat(dQ), self.bt_fused_bwd, *tail)
             yield self.SIDE, gemm_dk
         else:
             yield MAIN, p.batched("us_linear_bwd_x_batched", dC_h, V, sc["beta_P"], self.dP[:s], self.bt["dP"], ws)
-            yield MAIN, L.Call("us_softmax_bwd", L.mat(self.P), L.mat(self.dP), sc["sm"], sc["sm"], L.mat(self.dS))
+            yield MAIN, L.Call("us_softmax_bwd", p.mat(self.P), p.mat(self.dP), sc["sm"], sc["sm"], p.mat(self.dS))
             yield self.SIDE, gemm_dk
             yield MAIN, p.batched("us_linear_fwd_batched", dS, K, sc["beta_Q"], dQ, self.bt["dQ"], ws)
         yield self.JOIN, None                                       # dQ, dK, dV all written
         if self.dQKV is not self.dQKVq:
-            yield MAIN, L.Call("us_cast_fp8", L.mat(self.dQKV), 1.0, L.mat(self.dQKVq))
+            yield MAIN, L.Call("us_cast_fp8", p.mat(self.dQKV), 1.0, p.mat(self.dQKVq))
         yield MAIN, p.group([(L.US_OP_BWD_W, self.Xq, self.dQKVq, sc["beta_w"], self.dWqkv, None, None),
                              (L.US_OP_BWD_X, self.dQKVq, self.Wqkv_q, sc["beta_qkv"], self.dX, g1, coef)], ws)
 

@@ -122,8 +122,8 @@ class UnitScaledFFN:
             call(st)
 
     def _plan_cast(self, p, src, dst):
-        m = p.slot(src) if isinstance(src, str) else L.mat(src)
-        return L.Call("us_cast_fp8", m, 1.0, L.mat(dst)) if self.operand == "fp8" else L.Call("us_residual_add", m, m, 0.0, L.mat(dst))
+        m = p.slot(src) if isinstance(src, str) else p.mat(src)
+        return L.Call("us_cast_fp8", m, 1.0, p.mat(dst)) if self.operand == "fp8" else L.Call("us_residual_add", m, m, 0.0, p.mat(dst))
 
     def _plan_step(self, p):
         yield p.cast_multi(["W1", "W2", "X", "G"], [self.W1q, self.W2q, self.Xq, self.Gq])
@@ -142,9 +142,9 @@ class UnitScaledFFN:
         """step_from_casts() as prepared calls; X, G: the skip inputs, tensors or names of inputs."""
         sc = self.sc
         keep = self.keep_h or self.operand != "fp8" or min(self.T, self.d, self.f) <= 128
-        yield L.Call("us_ffn_hidden_any", L.mat(self.Xq), L.mat(self.W1q), sc.alpha1, L.mat(self.Gq), L.mat(self.W2q), sc.beta_x2,
-                     sc.s_in, sc.alpha_g, sc.beta_g, L._TORCH_DTYPES[self.H.dtype], L.mat(self.H) if keep else None,
-                     L.mat(self.Aq), L.mat(self.dHq), self.ws.data_ptr(), self.ws.numel())
+        yield L.Call("us_ffn_hidden_any", p.mat(self.Xq), p.mat(self.W1q), sc.alpha1, p.mat(self.Gq), p.mat(self.W2q), sc.beta_x2,
+                     sc.s_in, sc.alpha_g, sc.beta_g, L._TORCH_DTYPES[self.H.dtype], p.mat(self.H) if keep else None,
+                     p.mat(self.Aq), p.mat(self.dHq), self.ws.data_ptr(), self.ws.numel())
         w2, w1, x1 = self._plan_backward_entries(G)
         yield p.group([w2, w1, (L.US_OP_FWD, self.Aq, self.W2q, sc.alpha2, self.R, X, self._c), x1], self.ws)
 

@@ -211,10 +211,17 @@ class Plan:
 
     def __init__(self, owned, state):
         self.owned, self.state, self.ptrs = owned, state, [t.data_ptr() for t in owned]
-        self.slots, self.inputs, self.done = {}, {}, None
+        self.slots, self.inputs, self.done, self.mats = {}, {}, None, {}
 
     def same(self, owned, state) -> bool:
         return self.state == state and all(map(operator.is_, owned, self.owned)) and [t.data_ptr() for t in owned] == self.ptrs
+
+    def mat(self, t: torch.Tensor) -> us_mat:
+        """mat(t), made once for all calls of the pass that is being laid out."""
+        known = self.mats.get(id(t))
+        if known is None:
+            known = self.mats[id(t)] = (t, mat(t))              # t is held: its id stays its own
+        return known[1]
 
     def slot(self, name: str, m: us_mat = None) -> us_mat:
         """A us_mat (m, or a new one) that put() fills for the input `name`."""
@@ -233,11 +240,11 @@ class Plan:
         return self.done if self.done is not None else self._first(lay_out)
 
     def _first(self, lay_out):
-        self.slots, made = {}, []
+        self.slots, self.mats, made = {}, {}, []
         for c in lay_out(self):
             made.append(c)
             yield c
-        self.done = made                                        # a pass that ended early is laid out again
+        self.done, self.mats = made, {}                         # a pass that ended early is laid out again
 
     def cast_multi(self, srcs, dsts):
         """us_cast_multi at scale 1; an entry of srcs is a tensor or the name of an input."""
@@ -247,8 +254,8 @@ class Plan:
             if isinstance(s, str):
                 self.slot(s, sm[i])
             else:
-                sm[i] = mat(s)
-        return Call("us_cast_multi", n, sm, (C.c_float * n)(*[1.0] * n), (us_mat * n)(*[mat(t) for t in dsts]))
+                sm[i] = self.mat(s)
+        return Call("us_cast_multi", n, sm, (C.c_float * n)(*[1.0] * n), (us_mat * n)(*[self.mat(t) for t in dsts]))
 
     def residual(self, skip, coef):
         """The fixed(tau) residual epilogue; skip is a tensor or the name of an input."""
@@ -257,28 +264,28 @@ class Plan:
         if isinstance(skip, str):
             self.slot(skip, ep.skip)
         else:
-            ep.skip = mat(skip)
+            ep.skip = self.mat(skip)
         return ep
 
     def group(self, entries, ws):
         """us_linear_group_any over (op, a, b, scale, out, skip or None, (skip_coef, out_coef))."""
         arr = (us_linear_call * len(entries))()
         for c, (op, a, b, scale, out, skip, coef) in zip(arr, entries):
-            c.op, c.a, c.b, c.scale, c.out, c.ep.out_coef = op, mat(a), mat(b), scale, mat(out), 1.0
+            c.op, c.a, c.b, c.scale, c.out, c.ep.out_coef = op, self.mat(a), self.mat(b), scale, self.mat(out), 1.0
             if skip is not None:
                 c.ep.act_in_scale = c.ep.act_out_scale = 1.0
                 c.ep.skip_coef, c.ep.out_coef = coef
                 if isinstance(skip, str):
                     self.slot(skip, c.ep.skip)
                 else:
-                    c.ep.skip = mat(skip)
+                    c.ep.skip = self.mat(skip)
         return Call("us_linear_group_any", len(entries), arr, ws.data_ptr(), ws.numel())
 
     def linear(self, name, a, b, scale, out, ws, ep=None):
-        return Call(name, mat(a), mat(b), scale, ep, mat(out), ws.data_ptr(), ws.numel())
+        return Call(name, self.mat(a), self.mat(b), scale, ep, self.mat(out), ws.data_ptr(), ws.numel())
 
     def batched(self, name, a, b, scale, out, bt, ws):
-        return Call(name, mat(a), mat(b), scale, mat(out), bt, ws.data_ptr(), ws.numel())
+        return Call(name, self.mat(a), self.mat(b), scale, self.mat(out), bt, ws.data_ptr(), ws.numel())
 
 
 def _check(fn: str, status: int) -> None:
