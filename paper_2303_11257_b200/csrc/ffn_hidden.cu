@@ -19,7 +19,8 @@
 //
 // Bound: tensor pipe, in a long run the power cap.  Measured, separate launches -> this one, us:
 // FP8 8192 x 1024 x 4096: 86 -> 67;  BF16 8192 x 1024 x 4096 (H copy kept): 171 -> 138;  FP8 16384 x 2048 x 8192:
-// 550 -> 507;  FP8 256 x 128 x 512 on 128 x 128 tiles: 12.3 + a launch gap -> 7.2.
+// 550 -> 507;  FP8 256 x 128 x 512 on 128 x 128 tiles: 12.3 + a launch gap -> 7.2, with the columns of a tile split over four CTAs
+// (and the grouped launch over two) the whole three-launch step 16.4 -> 12.3.
 #include <cuda.h>
 
 #include <type_traits>
@@ -55,6 +56,7 @@ struct HiddenParams {
   float scale1, scale2;             // alpha, beta_x
   float act_in, act_out, grad_out;  // s_in, alpha_g, beta_g
   uint8_t* h_ptr; long long h_ld;   // optional copy of the rounded pre-activation (NULL: none); ld in elements
+  uint8_t *a_ptr, *d_ptr; long long a_ld, d_ld;   // A and dH, for SPLIT > 1 (otherwise reached by TMA)
   unsigned int* status;
   uint32_t wait_limit;
   int no_loads;                     // test hook: no operand loads are issued, so that the waits run out
@@ -62,8 +64,11 @@ struct HiddenParams {
 
 // ES: operand bytes per element (1 = FP8, 2 = BF16 / F16).  BN, CG: tiles of 256 x 256 per CTA pair (256, 2), or of
 // 128 x 128 per CTA (128, 1) where the large ones would leave more than half of the pairs idle (hidden_impl).
+// SPLIT (128 x 128 tiles): CTAs that compute the same tile, each turning 128 / SPLIT of its columns into outputs.  In a
+// small problem the arithmetic of the epilogue (3700 + 2800 cycles of one SM's issue slots for a tile) is the longest part of
+// the launch while most SMs are idle; repeating the short main loop costs less than it.
 // OUT_A, OUT_D: output formats of A and dH (us_dtype).  H_BF16: pre-activation rounded to BF16 (else F16).
-template <int ES, int BN, int CG, int OUT_A, int OUT_D, bool H_BF16>
+template <int ES, int BN, int CG, int SPLIT, int OUT_A, int OUT_D, bool H_BF16>
 __global__ void __launch_bounds__(gemm_threads(kHidEW), 1)
 ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w1,
                   const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_w2,
@@ -74,7 +79,10 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   static_assert(BN / CG == 128, "128 rows of B per CTA");
   constexpr int kBK = 128 / ES;                     // K elements per stage
   constexpr int kTileM = kBM * CG;
-  constexpr int kWarpCols = BN / 4, kSlices = kWarpCols / 32;   // columns of a tile one epilogue warp handles
+  static_assert(SPLIT == 1 || (CG == 1 && BN == 128 && (SPLIT == 2 || SPLIT == 4)), "split tiles are 128 x 128");
+  constexpr int kWarpCols = SPLIT > 1 ? 16 : BN / 4;            // columns of a tile one epilogue warp handles,
+  constexpr int kSliceCols = SPLIT > 1 ? 16 : 32, kSlices = kWarpCols / kSliceCols;   // worked in slices
+  constexpr int kWarpsUsed = SPLIT > 1 ? 4 * (BN / SPLIT / kWarpCols) : kHidEW;
   constexpr uint32_t kChunkBytes = kBK * 128;       // a box of an MN-major operand tile: kBK rows of K x 128 bytes
   constexpr uint32_t kTmemCols = 2 * BN;
 
@@ -96,7 +104,8 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = CG == 2 ? (int)ptx::cluster_ctarank() : 0;
-  const int pair = blockIdx.x / CG, num_pairs = gridDim.x / CG;      // tile-walking unit: CTA pair or CTA
+  const int pair = blockIdx.x / (CG * SPLIT), num_pairs = gridDim.x / (CG * SPLIT);      // tile-walking unit: CTA pair or CTA(s)
+  const int split_col = SPLIT > 1 ? (int)(blockIdx.x % SPLIT) * (BN / SPLIT) : 0;        // this CTA's columns of the tile
   const int num_tiles = p.tiles_m * p.tiles_n;
   const int kb1 = (p.K1 + kBK - 1) / kBK, kb2 = (p.K2 + kBK - 1) / kBK;
   // column-major over the tiles: pairs that run side by side share a panel of W1 and of W2
@@ -104,7 +113,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S::kStages; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
-    for (int a = 0; a < 2; ++a) { ptx::mbar_init(acc_full_bar(a), 1); ptx::mbar_init(acc_empty_bar(a), CG * kHidEW); }
+    for (int a = 0; a < 2; ++a) { ptx::mbar_init(acc_full_bar(a), 1); ptx::mbar_init(acc_empty_bar(a), CG * kWarpsUsed); }
     ptx::mbar_init(drained_bar, 1);
     *abort_flag = 0;
     ptx::mbar_init_fence();
@@ -122,7 +131,6 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   if (CG == 2) ptx::cluster_sync();
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  ptx::grid_wait_previous();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (every CTA)
@@ -141,6 +149,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             if (!ok) break;
             const uint32_t a_dst = smem_base + stage * S::kStageBytes, b_dst = a_dst + S::kABytes;
             const int k0 = kb * kBK;
+            if (issued == 0) ptx::grid_wait_previous();       // coordinates and barriers are ready: only the loads wait
             const uint32_t fb = CG == 2 ? ptx::in_even_cta(full_bar(stage)) : full_bar(stage);
             if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), CG * S::kStageBytes);
             auto load = [&](uint32_t dst, const void* tmap, int x, int y) {
@@ -218,8 +227,9 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         for (uint32_t it = 0; it < p.wait_limit && !ptx::mbar_try_wait(drained_bar, 0); ++it) {}
       }
     }
-  } else {
+  } else if (warp - 2 < kWarpsUsed) {
     // ------------------------------------------------------------ epilogue warps
+    ptx::grid_wait_previous();
     // Warp (lane quarter q, part) owns 32 rows x kWarpCols columns of the tile; a lane holds one row of them.  The
     // rounded pre-activation of a tile stays in registers as packed 16-bit pairs (hst) between the two phases; staging
     // is one output box of 32 rows per warp, swizzled with the pattern of its row width (32-byte rows: none).
@@ -239,26 +249,45 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       }
     };
     // Eight outputs of this lane's row, group g of slice s, into the box: 16-byte chunk c at c ^ box_sw.
+    // (SPLIT > 1: straight to memory, the 16-byte pieces of this lane's row.)
+    uint8_t* direct = nullptr;
+    int direct_cols = 0;                                        // columns of the lane's part that exist
+    auto put = [&](uint32_t c, uint4 v, int es) {               // 16 / es values from column c * 16 / es of the warp's part
+      if constexpr (SPLIT == 1) {
+        ptx::sts128(buf_out + box_row + ((c ^ box_sw) << 4), v);
+      } else {
+        const int per = 16 / es, col = (int)c * per;
+        if (col + per <= direct_cols) {
+          *reinterpret_cast<uint4*>(direct + c * 16u) = v;
+        } else {
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+          for (int i = 0; i < per && col + i < direct_cols; ++i) {
+            if (es == 1) direct[c * 16u + i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
+            else reinterpret_cast<uint16_t*>(direct + c * 16u)[i] = (uint16_t)(w[i >> 1] >> (16 * (i & 1)));
+          }
+        }
+      }
+    };
     auto stage_out = [&](auto fmt, const float (&y)[8], uint32_t (&held)[2], int s, int g) {
       constexpr int F = decltype(fmt)::value;
       if constexpr (F == US_E4M3 || F == US_E5M2) {
         const uint32_t lo = cvt_fp8x4<F == US_E5M2>(y[0], y[1], y[2], y[3]);
         const uint32_t hi = cvt_fp8x4<F == US_E5M2>(y[4], y[5], y[6], y[7]);
         if ((g & 1) == 0) { held[0] = lo; held[1] = hi; }
-        else ptx::sts128(buf_out + box_row + ((((uint32_t)(2 * s + (g >> 1))) ^ box_sw) << 4), make_uint4(held[0], held[1], lo, hi));
+        else put((uint32_t)(2 * s + (g >> 1)), make_uint4(held[0], held[1], lo, hi), 1);
       } else {
         uint32_t w[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) w[k] = F == US_BF16 ? pack_bf16x2(y[2 * k], y[2 * k + 1]) : pack_f16x2(y[2 * k], y[2 * k + 1]);
-        ptx::sts128(buf_out + box_row + ((((uint32_t)(4 * s + g)) ^ box_sw) << 4), make_uint4(w[0], w[1], w[2], w[3]));
+        put((uint32_t)(4 * s + g), make_uint4(w[0], w[1], w[2], w[3]), 2);
       }
     };
-    uint32_t hst[16 * kSlices];
+    uint32_t hst[kSliceCols / 2 * kSlices];
     // One 32-column slice s of accumulator 0: scale, keep round16(H), GELU, round, stage.
-    auto slice_fwd = [&](const uint32_t (&r)[32], int s) {
+    auto slice_fwd = [&](const uint32_t (&r)[kSliceCols], int s) {
       uint32_t held[2];
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
+      for (int g = 0; g < kSliceCols / 8; ++g) {
         f32x2 x[4];
         float y[8];
 #pragma unroll
@@ -266,7 +295,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
           x[k] = mul2(pack2(__uint_as_float(r[8 * g + 2 * k]), __uint_as_float(r[8 * g + 2 * k + 1])), s1);
           float a, b;
           unpack2(x[k], a, b);
-          hst[16 * s + 4 * g + k] = H_BF16 ? pack_bf16x2(a, b) : pack_f16x2(a, b);
+          hst[kSliceCols / 2 * s + 4 * g + k] = H_BF16 ? pack_bf16x2(a, b) : pack_f16x2(a, b);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) gelu_scaled2<kOes == 1>(x[k], tail_k, act_oi, y[2 * k], y[2 * k + 1]);   // the form the separate launch takes for this output
@@ -274,15 +303,15 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       }
     };
     // The same slice of accumulator 1: scale, GELU gradient from the kept pre-activation, round, stage.
-    auto slice_bwd = [&](const uint32_t (&r)[32], int s) {
+    auto slice_bwd = [&](const uint32_t (&r)[kSliceCols], int s) {
       uint32_t held[2];
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
+      for (int g = 0; g < kSliceCols / 8; ++g) {
         float y[8];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const f32x2 x = mul2(pack2(__uint_as_float(r[8 * g + 2 * k]), __uint_as_float(r[8 * g + 2 * k + 1])), s2);
-          const float2 h = H_BF16 ? unpack_bf16x2(hst[16 * s + 4 * g + k]) : unpack_f16x2(hst[16 * s + 4 * g + k]);
+          const float2 h = H_BF16 ? unpack_bf16x2(hst[kSliceCols / 2 * s + 4 * g + k]) : unpack_f16x2(hst[kSliceCols / 2 * s + 4 * g + k]);
           unpack2(gelu_grad_scaled2(pack2(h.x, h.y), x, in2, os2), y[2 * k], y[2 * k + 1]);
         }
         stage_out(std::integral_constant<int, OUT_D>(), y, held, s, g);
@@ -294,7 +323,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     for (int tile = pair; ok && tile < num_tiles; tile += num_pairs, ++local) {
       int tm, tn;
       tile_mn2(tile, tm, tn);
-      const int row0 = tm * kTileM + rank * 128 + q * 32, n_w = tn * BN + part * kWarpCols;
+      const int row0 = tm * kTileM + rank * 128 + q * 32, n_w = tn * BN + split_col + part * kWarpCols;
       const bool active = n_w < p.N;                            // warp-uniform
       const uint32_t acc_phase = local & 1u;
 #pragma unroll
@@ -303,12 +332,19 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         ptx::tc_fence_after_sync();
-        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + sub * BN + part * kWarpCols;
-        uint32_t r0[32], r1[32];
+        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + sub * BN + split_col + part * kWarpCols;
+        uint32_t r0[kSliceCols], r1[kSliceCols];
+        if (SPLIT > 1) {
+          const long long at = sub == 0 ? (long long)(row0 + lane) * p.a_ld : (long long)(row0 + lane) * p.d_ld;
+          direct = (sub == 0 ? p.a_ptr : p.d_ptr) + (at + n_w) * kOes;
+          direct_cols = row0 + lane < p.M ? p.N - n_w : 0;
+        }
         if (active) {
           ptx::tmem_ld_32x32_issue(t_row, r0);
-          if (lane == 0) ptx::bulk_wait_group_read<0>();        // earlier stores have read the staging boxes
-          __syncwarp();
+          if (SPLIT == 1) {
+            if (lane == 0) ptx::bulk_wait_group_read<0>();      // earlier stores have read the staging boxes
+            __syncwarp();
+          }
           ptx::tmem_ld_fence(r0);
           if (kSlices == 2) {
             ptx::tmem_ld_32x32_issue(t_row + 32, r1);
@@ -324,7 +360,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             // the copy of the rounded pre-activation: this lane's columns, 8 at a time (16 aligned bytes)
             uint8_t* dst = p.h_ptr + ((long long)(row0 + lane) * p.h_ld + n_w) * 2;
 #pragma unroll
-            for (int c = 0; c < 4 * kSlices; ++c) {
+            for (int c = 0; c < kWarpCols / 8; ++c) {
               const int col = n_w + 8 * c;
               if (col + 8 <= p.N) {
                 *reinterpret_cast<uint4*>(dst + 16 * c) = make_uint4(hst[4 * c], hst[4 * c + 1], hst[4 * c + 2], hst[4 * c + 3]);
@@ -336,15 +372,17 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
               }
             }
           }
-          ptx::fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) {
-            if (sub == 0) {
-              ptx::tma_store_2d(&tm_a, buf_out, n_w, row0);
-            } else {
-              ptx::tma_store_2d(&tm_dh, buf_out, n_w, row0);
+          if (SPLIT == 1) {
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+              if (sub == 0) {
+                ptx::tma_store_2d(&tm_a, buf_out, n_w, row0);
+              } else {
+                ptx::tma_store_2d(&tm_dh, buf_out, n_w, row0);
+              }
+              ptx::bulk_commit_group();
             }
-            ptx::bulk_commit_group();
           }
         }
       }
@@ -389,17 +427,23 @@ bool valid_mat(const us_mat* m) {
 }
 bool is_fp8(int dt) { return dt == US_E4M3 || dt == US_E5M2; }
 
-template <int ES, int BN, int CG, int OUT_A, int OUT_D, bool H_BF16>
+template <int ES, int BN, int CG, int SPLIT, int OUT_A, int OUT_D, bool H_BF16>
 us_status launch_hidden(const CUtensorMap* t, const HiddenParams& p, int units, cudaStream_t stream) {
-  auto kern = ffn_hidden_kernel<ES, BN, CG, OUT_A, OUT_D, H_BF16>;
+  auto kern = ffn_hidden_kernel<ES, BN, CG, SPLIT, OUT_A, OUT_D, H_BF16>;
   constexpr int smem = HidSmem<BN, OUT_A == US_E4M3 || OUT_A == US_E5M2 ? 1 : 2>::kTotal;
   static std::atomic<uint64_t> smem_set{0};
-  return host::launch(kern, &smem_set, CG * units, gemm_threads(kHidEW), smem, CG, stream, t[0], t[1], t[2], t[3], t[4], t[5], p);
+  return host::launch(kern, &smem_set, CG * SPLIT * units, gemm_threads(kHidEW), smem, CG, stream, t[0], t[1], t[2], t[3], t[4], t[5], p);
+}
+template <int ES, int OUT_A, int OUT_D, bool H_BF16>
+us_status pick_tile(bool pair, int split, const CUtensorMap* t, const HiddenParams& p, int units, cudaStream_t st) {
+  if (pair) return launch_hidden<ES, 256, 2, 1, OUT_A, OUT_D, H_BF16>(t, p, units, st);
+  if (split == 4) return launch_hidden<ES, 128, 1, 4, OUT_A, OUT_D, H_BF16>(t, p, units, st);
+  if (split == 2) return launch_hidden<ES, 128, 1, 2, OUT_A, OUT_D, H_BF16>(t, p, units, st);
+  return launch_hidden<ES, 128, 1, 1, OUT_A, OUT_D, H_BF16>(t, p, units, st);
 }
 template <int ES, int OUT_A, int OUT_D>
-us_status pick_hidden(bool pair, bool h_bf16, const CUtensorMap* t, const HiddenParams& p, int units, cudaStream_t st) {
-  if (pair) return h_bf16 ? launch_hidden<ES, 256, 2, OUT_A, OUT_D, true>(t, p, units, st) : launch_hidden<ES, 256, 2, OUT_A, OUT_D, false>(t, p, units, st);
-  return h_bf16 ? launch_hidden<ES, 128, 1, OUT_A, OUT_D, true>(t, p, units, st) : launch_hidden<ES, 128, 1, OUT_A, OUT_D, false>(t, p, units, st);
+us_status pick_hidden(bool pair, int split, bool h_bf16, const CUtensorMap* t, const HiddenParams& p, int units, cudaStream_t st) {
+  return h_bf16 ? pick_tile<ES, OUT_A, OUT_D, true>(pair, split, t, p, units, st) : pick_tile<ES, OUT_A, OUT_D, false>(pair, split, t, p, units, st);
 }
 
 // any: 16-bit operands (outputs in the same format) and any size are covered too.
@@ -443,6 +487,8 @@ us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_m
   p.act_in = act_in_scale; p.act_out = act_out_scale; p.grad_out = grad_out_scale;
   p.h_ptr = keep_h ? static_cast<uint8_t*>(H->ptr) : nullptr;
   p.h_ld = keep_h ? H->ld : 0;
+  p.a_ptr = static_cast<uint8_t*>(A->ptr); p.a_ld = A->ld;
+  p.d_ptr = static_cast<uint8_t*>(dH->ptr); p.d_ld = dH->ld;
   p.status = static_cast<unsigned int*>(ws);
   p.wait_limit = wait_limit;
   p.no_loads = no_loads;
@@ -455,14 +501,15 @@ us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_m
 
   const int tiles = p.tiles_m * p.tiles_n, most = pair ? sms / 2 : sms;
   const int units = tiles < most ? tiles : most;
+  const int split = pair || no_loads ? 1 : 4 * tiles <= sms ? 4 : 2 * tiles <= sms ? 2 : 1;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const bool bf = h_dtype == US_BF16;
-  if (!f8) return X->dtype == US_BF16 ? pick_hidden<2, US_BF16, US_BF16>(pair, bf, t, p, units, st) : pick_hidden<2, US_F16, US_F16>(pair, bf, t, p, units, st);
+  if (!f8) return X->dtype == US_BF16 ? pick_hidden<2, US_BF16, US_BF16>(pair, split, bf, t, p, units, st) : pick_hidden<2, US_F16, US_F16>(pair, split, bf, t, p, units, st);
   const bool a5 = A->dtype == US_E5M2, d5 = dH->dtype == US_E5M2;
-  if (!a5 && d5) return pick_hidden<1, US_E4M3, US_E5M2>(pair, bf, t, p, units, st);
-  if (!a5 && !d5) return pick_hidden<1, US_E4M3, US_E4M3>(pair, bf, t, p, units, st);
-  if (a5 && d5) return pick_hidden<1, US_E5M2, US_E5M2>(pair, bf, t, p, units, st);
-  return pick_hidden<1, US_E5M2, US_E4M3>(pair, bf, t, p, units, st);
+  if (!a5 && d5) return pick_hidden<1, US_E4M3, US_E5M2>(pair, split, bf, t, p, units, st);
+  if (!a5 && !d5) return pick_hidden<1, US_E4M3, US_E4M3>(pair, split, bf, t, p, units, st);
+  if (a5 && d5) return pick_hidden<1, US_E5M2, US_E5M2>(pair, split, bf, t, p, units, st);
+  return pick_hidden<1, US_E5M2, US_E4M3>(pair, split, bf, t, p, units, st);
 }
 
 }  // namespace

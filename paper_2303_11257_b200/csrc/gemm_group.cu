@@ -9,7 +9,8 @@
 namespace us {
 namespace {
 
-// Row-major [rows x cols] matrix of es-byte elements, boxes of box_rows rows x 128 (or 64) bytes, swizzled with that width's pattern, zero fill.
+// Row-major [rows x cols] matrix of es-byte elements, boxes of box_rows rows x 128 (64, 32) bytes, swizzled with that width's
+// pattern (32 bytes: not), zero fill.
 bool make_tmap(CUtensorMap* tm, const us_mat* m, int es, int box_rows, int box_bytes = 128) {
   host::EncodeTiledFn fn = host::encode_tiled_fn();
   if (!fn) return false;
@@ -20,7 +21,7 @@ bool make_tmap(CUtensorMap* tm, const us_mat* m, int es, int box_rows, int box_b
   cuuint32_t box[2] = {(cuuint32_t)(box_bytes / es), (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
   return fn(tm, type, 2, m->ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+            box_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_NONE : box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -69,7 +70,7 @@ us_status check_call(const us_linear_call* c, bool any, Shape* sh) {
 // Deals the tiles of all problems to the units, longest contraction first, each tile to the unit with the least work
 // so far (ties: lowest unit), in a fixed order: the same arguments always give the same work list, and a tile's result
 // never depends on it anyway (one unit, one accumulator).  False if a unit would get more than max_rounds tiles.
-bool deal(GroupParams& g, int es, int tile_m, int bn, int units, int max_rounds) {
+bool deal(GroupParams& g, int es, int tile_m, int bn, int split, int units, int max_rounds) {
   int order[kGroupMaxProblems];
   for (int i = 0; i < g.count; ++i) order[i] = i;
   std::stable_sort(order, order + g.count, [&](int x, int y) { return g.prob[x].K > g.prob[y].K; });
@@ -82,7 +83,7 @@ bool deal(GroupParams& g, int es, int tile_m, int bn, int units, int max_rounds)
   const int kbk = 128 / es;
   for (int o = 0; o < g.count; ++o) {
     const GroupProblem& P = g.prob[order[o]];
-    const int tiles_m = (P.M + tile_m - 1) / tile_m, tiles_n = (P.N + bn - 1) / bn;
+    const int tiles_m = (P.M + tile_m - 1) / tile_m, tiles_n = (P.N + bn - 1) / bn * split;      // split: entries per tile, one per part of its columns
     const uint32_t cost = (uint32_t)((P.K + kbk - 1) / kbk) + 4;            // K blocks plus a change-over
     // column-major over the tiles of a problem (neighbours in the list share a B panel) while A stays in L2, bands of
     // eight tile rows beyond that, as for the single launches
@@ -105,9 +106,9 @@ bool deal(GroupParams& g, int es, int tile_m, int bn, int units, int max_rounds)
   return true;
 }
 
-template <int ES, int BN, int CG>
+template <int ES, int BN, int CG, int SPLIT>
 us_status launch_group(const GroupParams& g, cudaStream_t stream) {
-  auto kern = gemm_group_kernel<ES, BN, CG>;
+  auto kern = gemm_group_kernel<ES, BN, CG, SPLIT>;
   constexpr int smem = GemmSmem<BN, CG, kGroupEW>::kTotal;
   static std::atomic<uint64_t> smem_set{0};
   return host::launch(kern, &smem_set, CG * g.units, gemm_threads(kGroupEW), smem, CG, stream, g);
@@ -133,6 +134,11 @@ us_status group_impl(int count, const us_linear_call* calls, bool any, void* ws,
   // us: 48 such tiles 14.3 / 19.2 against 10.7 / 17.1 with 128 x 128 tiles, 64 tiles 14.9 / 20.0 against 16.3 / 27.3).
   const bool pair = 8 * pair_tiles >= 3 * sms;
   const int tile_m = pair ? 256 : 128, bn = pair ? 256 : 128;
+  int64_t tiles = 0;
+  for (int i = 0; i < count; ++i) tiles += ((sh[i].M + tile_m - 1) / tile_m) * ((sh[i].N + bn - 1) / bn);
+  const int most = std::min(pair ? sms / 2 : sms, kGroupMaxUnits);
+  const int split = !pair && 2 * tiles <= most ? 2 : 1;
+  const int units = (int)std::min<int64_t>(most, tiles * split);
   GroupParams g;
   g.count = count;
   for (int i = 0; i < count; ++i) {
@@ -149,22 +155,17 @@ us_status group_impl(int count, const us_linear_call* calls, bool any, void* ws,
     P.skip_coef = P.has_skip ? c.ep.skip_coef : 0.f;
     P.out_coef = P.has_skip ? c.ep.out_coef : 1.f;
     if (!make_tmap(&P.ta, &c.a, es, P.a_mn ? 128 / es : 128) || !make_tmap(&P.tb, &c.b, es, P.b_mn ? 128 / es : 128)) return US_ERR_CUDA;
-    if (!make_tmap(&P.tout, &c.out, dtype_size(c.out.dtype), 32, !pair && is_fp8(c.out.dtype) ? 64 : 128)) return US_ERR_CUDA;
+    const int oes = dtype_size(c.out.dtype);
+    if (!make_tmap(&P.tout, &c.out, oes, 32, std::min(128, bn / 2 / split * oes))) return US_ERR_CUDA;
     P.tskip = P.tout;
     if (P.has_skip && !make_tmap(&P.tskip, &c.ep.skip, dtype_size(c.ep.skip.dtype), 32)) return US_ERR_CUDA;
   }
-  int units = std::min(pair ? sms / 2 : sms, kGroupMaxUnits);
-  if (!pair || pair_tiles < units) {
-    int64_t tiles = 0;
-    for (int i = 0; i < count; ++i) tiles += ((sh[i].M + tile_m - 1) / tile_m) * ((sh[i].N + bn - 1) / bn);
-    units = (int)std::min<int64_t>(units, tiles);
-  }
-  if (!deal(g, es, tile_m, bn, units, any ? kGroupMaxItems : 12)) return US_ERR_UNSUPPORTED;      // too many tiles per unit for the work list
+  if (!deal(g, es, tile_m, bn, split, units, any ? kGroupMaxItems : 12)) return US_ERR_UNSUPPORTED;      // too many tiles per unit for the work list
   g.status = static_cast<unsigned int*>(ws);
   g.wait_limit = kWaitLimit;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (es == 1) return pair ? launch_group<1, 256, 2>(g, st) : launch_group<1, 128, 1>(g, st);
-  return pair ? launch_group<2, 256, 2>(g, st) : launch_group<2, 128, 1>(g, st);
+  if (es == 1) return pair ? launch_group<1, 256, 2, 1>(g, st) : split == 2 ? launch_group<1, 128, 1, 2>(g, st) : launch_group<1, 128, 1, 1>(g, st);
+  return pair ? launch_group<2, 256, 2, 1>(g, st) : split == 2 ? launch_group<2, 128, 1, 2>(g, st) : launch_group<2, 128, 1, 1>(g, st);
 }
 
 }  // namespace

@@ -52,14 +52,19 @@ __device__ __forceinline__ void group_decode(int32_t e, int& prob, int& tm, int&
 
 constexpr int kGroupEW = 8;
 
-template <int ES, int BN, int CG>
+// SPLIT = 2 (128 x 128 tiles): two CTAs compute the same tile and each writes half of its columns, where the problems are so
+// small that half of the SMs would be idle: the epilogue of a tile takes longer than a short main loop.
+template <int ES, int BN, int CG, int SPLIT>
 __global__ void __launch_bounds__(gemm_threads(kGroupEW), 1)
 gemm_group_kernel(const __grid_constant__ GroupParams g) {
   using S = GemmSmem<BN, CG, kGroupEW>;
   static_assert(BN / CG == 128, "128 rows of B per CTA");
   constexpr int kBK = 128 / ES;                     // K elements per stage
   constexpr int kTileM = kBM * CG;
-  constexpr int kWarpCols = BN / 2;                 // columns of a tile one epilogue warp handles
+  static_assert(SPLIT == 1 || (BN == 128 && CG == 1), "split tiles are 128 x 128");
+  constexpr int kWarpCols = BN / 2 / SPLIT;         // columns of a tile one epilogue warp handles
+  // first column a warp handles, and its offset in the tile: a tile column of the work list is tn * SPLIT + part
+  auto warp_col = [](int tn, int half) { return tn * (BN / SPLIT) + half * kWarpCols; };
   constexpr uint32_t kChunkBytes = kBK * 128;       // a box of an MN-major operand tile: kBK rows of K x 128 bytes
   constexpr uint32_t kTmemCols = 2 * BN;
 
@@ -101,7 +106,6 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
   if (CG == 2) ptx::cluster_sync();
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  ptx::grid_wait_previous();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (every CTA)
@@ -115,13 +119,14 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
         int pi, tm, tn;
         group_decode(e, pi, tm, tn);
         const GroupProblem& P = g.prob[pi];
-        const int m0 = tm * kTileM + rank * 128, n0 = tn * BN + rank * 128;
+        const int m0 = tm * kTileM + rank * 128, n0 = tn / SPLIT * BN + rank * 128;
         const int num_kb = (P.K + kBK - 1) / kBK;
         for (int kb = 0; kb < num_kb; ++kb) {
           ok = wait_bounded(empty_bar(stage), phase ^ 1u, abort_flag, g.status, g.wait_limit);
           if (!ok) break;
           const uint32_t a_dst = smem_base + stage * S::kStageBytes, b_dst = a_dst + S::kABytes;
           const int k0 = kb * kBK;
+          if (issued == 0) ptx::grid_wait_previous();
           const uint32_t fb = CG == 2 ? ptx::in_even_cta(full_bar(stage)) : full_bar(stage);
           if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), CG * S::kStageBytes);
           auto load = [&](uint32_t dst, const void* tmap, int x, int y) {
@@ -207,6 +212,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
     // Warp (quarter q, half) owns 32 rows x half of the columns of a tile, worked in 32-column slices.  Staging: box 0
     // (4 KB) receives the skip tensor's boxes by TMA, box 1 (4 KB) collects output and leaves by TMA store.
     const int q = warp & 3, half = (warp - 2) >> 2;
+    ptx::grid_wait_previous();
     const uint32_t buf_in = epi_base + (warp - 2) * epi_warp_bytes(kGroupEW), buf_out = buf_in + 4096u;
     const uint32_t in_bar = epi_in_bar(warp - 2);
     const uint32_t row_off = (uint32_t)lane * 128u, sw = (uint32_t)(lane & 7);
@@ -228,7 +234,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
         int pi, tm, tn;
         group_decode(e, pi, tm, tn);
         const GroupProblem& P = g.prob[pi];
-        const int n_w = tn * BN + half * kWarpCols;
+        const int n_w = warp_col(tn, half);
         if (P.has_skip && n_w < P.N) issue_in(P, n_w, tm * kTileM + rank * 128 + q * 32);
         return;                                                // only the very next tile is looked at
       }
@@ -243,18 +249,18 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
       const GroupProblem& P = g.prob[pi];
       const uint32_t acc = local & 1u, acc_phase = (local >> 1) & 1u;
       ++local;
-      const int row0 = tm * kTileM + rank * 128 + q * 32, n_w = tn * BN + half * kWarpCols;
+      const int row0 = tm * kTileM + rank * 128 + q * 32, n_w = warp_col(tn, half);
       const bool skip = P.has_skip != 0;
       const int in_es = dtype_size(P.skip_dt), out_es = dtype_size(P.out_dt);
-      // an output box holds 128-byte rows, or the 64 bytes a warp's 64 columns of FP8 codes are
-      const bool narrow = kWarpCols == 64 && out_es == 1;
-      const int in_box_cols = 128 / in_es, out_box_cols = (narrow ? 64 : 128) / out_es;
-      const uint32_t out_sw = narrow ? (uint32_t)((lane >> 1) & 3) : sw;
+      // an output box holds 128-byte rows, or the fewer bytes that a warp's columns are (swizzled accordingly; 32-byte rows: not)
+      const int out_row = min(128, kWarpCols * out_es);
+      const int in_box_cols = 128 / in_es, out_box_cols = out_row / out_es;
+      const uint32_t out_sw = out_row == 128 ? sw : out_row == 64 ? (uint32_t)((lane >> 1) & 3) : 0u;
       ok = wait_bounded(acc_full_bar(acc), acc_phase, abort_flag, g.status, g.wait_limit);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       ptx::tc_fence_after_sync();
-      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + half * kWarpCols;
+      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + (tn % SPLIT) * (BN / SPLIT) + half * kWarpCols;
       auto release_acc = [&]() {
         ptx::tc_fence_before_sync();
         __syncwarp();
@@ -301,7 +307,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
           ptx::tmem_ld_32x32(t_row + 32 * sl, v);
           if (last_slice) { release_acc(); released = true; }
           const uint32_t out_cb = (uint32_t)(out_off * out_es) >> 4;
-          const uint32_t dst = buf_out + (narrow ? (uint32_t)lane * 64u : row_off);
+          const uint32_t dst = buf_out + (uint32_t)(lane * out_row);
           uint32_t held[2];
 #pragma unroll
           for (int gi = 0; gi < 4; ++gi) {

@@ -51,8 +51,9 @@ static us_status launch(const us_mat* A, const us_mat* B, const GemmParams& p, c
   const BatchDesc* b4 = BATCHED ? bd : nullptr;
   if (!make_tmap(&ta, A, ES, A_MN ? kBK : kBM, 128, b4, b4 ? bd->a : nullptr)) return US_ERR_CUDA;
   if (!make_tmap(&tb, B, ES, B_MN ? kBK : BN / CG, 128, b4, b4 ? bd->b : nullptr)) return US_ERR_CUDA;
-  // epilogue boxes: 32 rows x 128 bytes; unused maps alias the output's so that every parameter is valid
-  if (!make_tmap(&t_out, em.out, dtype_size(em.out->dtype), 32, EW == 16 ? 64 : 128, b4, b4 ? bd->out : nullptr)) return US_ERR_CUDA;
+  // epilogue boxes: 32 rows x 128 (or 64) bytes; unused maps alias the output's so that every parameter is valid
+  const bool narrow_out = EW == 16 || (BN == 128 && dtype_size(em.out->dtype) == 1);      // FP8 codes of a warp's 64 columns
+  if (!make_tmap(&t_out, em.out, dtype_size(em.out->dtype), 32, narrow_out ? 64 : 128, b4, b4 ? bd->out : nullptr)) return US_ERR_CUDA;
   t_aux = t_out; t_skip = t_out;
   // the 16-warp GELU-gradient epilogue reads the stored pre-activation as 32-row x 64-byte boxes (one per 32-column slice)
   if (EPI != kEpiLegacy && em.aux && !make_tmap(&t_aux, em.aux, dtype_size(em.aux->dtype), 32, (EW == 16 && EPI == kEpiGeluGrad) ? 64 : 128)) return US_ERR_CUDA;
