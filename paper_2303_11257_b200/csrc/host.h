@@ -49,5 +49,19 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn encode_tiled_fn();
+// A launch without that overlap, of a kernel that may take up to max_smem bytes of dynamic shared memory.
+template <class... P, class... A>
+us_status launch_plain(void (*kern)(P...), std::atomic<uint64_t>* smem_set, int grid, int threads, int max_smem, size_t smem,
+                       cudaStream_t stream, const A&... args) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return US_ERR_CUDA;
+  const uint64_t bit = 1ull << (dev & 63);
+  if (!(smem_set->load(std::memory_order_relaxed) & bit)) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess) return US_ERR_CUDA;
+    smem_set->fetch_or(bit, std::memory_order_relaxed);
+  }
+  kern<<<(unsigned)grid, (unsigned)threads, smem, stream>>>(P(args)...);
+  return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
+}
 }  // namespace host
 }  // namespace us

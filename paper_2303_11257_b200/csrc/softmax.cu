@@ -363,6 +363,82 @@ __global__ void __launch_bounds__(1024) softmax_xent_row_kernel(const XentArgs a
   });
 }
 
+// One CTA per row of 16-bit logits staged in shared memory by one bulk copy, for vocabularies whose rows the register form
+// holds with 512 threads: three CTAs per SM instead of two (40 registers a thread instead of 64), so that one row's load
+// runs under two others' reductions.  2048 rows of 30522 BF16 logits: forward 39 -> 31 us (4.1 TB/s), backward with an E5M2
+// gradient 66 -> 56 us (3.3 TB/s; two exponentials per class make 28 us of it).  A wait that runs out falls back to loads
+// from global memory.
+constexpr int kXentStagedThreads = 512;
+constexpr uint32_t kXentWaitLimit = 1u << 20;
+template <bool BWD, int DT>
+__global__ void __launch_bounds__(kXentStagedThreads, 3) softmax_xent_staged_kernel(const XentArgs a) {
+  extern __shared__ __align__(16) uint8_t xent_smem[];
+  __shared__ float slots[2][32];
+  __shared__ __align__(8) uint64_t bar_word;
+  const uint32_t data = ptx::smem_addr(xent_smem), bar = ptx::smem_addr(&bar_word);
+  const int64_t row = blockIdx.x, x_off = row * a.x_ld;
+  const int tid = (int)threadIdx.x;
+  const int full = a.cols / 8, tail = a.cols - 8 * full;      // whole chunks of eight; elements behind them
+  if (tid == 0) {
+    ptx::mbar_init(bar, 1);
+    ptx::mbar_init_fence();
+    ptx::mbar_expect_tx(bar, (uint32_t)full * 16u);
+    ptx::bulk_load_1d(data, static_cast<const char*>(a.x) + x_off * 2, (uint32_t)full * 16u, bar);
+  }
+  const int t = a.t[row];
+  const bool valid = t >= 0 && t < a.cols;                   // a target outside the row: NaN forward, no one-hot term backward
+  float xt = __int_as_float(0x7fc00000), gr = 1.0f;
+  if (!BWD && tid == 0 && valid) xt = load_one(a.x, DT, x_off + t);
+  if (BWD && a.g) gr = a.g[row];
+  const float last = tid < tail ? load_one(a.x, DT, x_off + 8 * full + tid) : -INFINITY;
+  __syncthreads();
+  bool staged = false;
+  for (uint32_t it = 0; it < kXentWaitLimit && !(staged = ptx::mbar_try_wait(bar, 0)); ++it) {}
+  auto for_chunks = [&](auto&& fn) {
+#pragma unroll 2
+    for (int c = tid; c < full; c += kXentStagedThreads) {
+      const uint4 raw = staged ? ptx::lds128(data + (uint32_t)c * 16u)
+                               : __ldg(reinterpret_cast<const uint4*>(static_cast<const char*>(a.x) + x_off * 2) + c);
+      float v[8];
+      unpack16x8(raw, DT, v);
+      fn(8 * c, v);
+    }
+  };
+  float m = last;
+  for_chunks([&](int, float (&v)[8]) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) m = fmaxf(m, v[i]);
+  });
+  m = cta_reduce<true>(m, slots[0]);
+  const float mb = m * kLog2e;
+  float sum = tid < tail ? ex2_approx(fmaf(last, kLog2e, -mb)) : 0.f;
+  for_chunks([&](int, float (&v)[8]) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sum += ex2_approx(fmaf(v[i], kLog2e, -mb));
+  });
+  sum = cta_reduce<false>(sum, slots[1]);
+  if (!BWD) {
+    if (tid == 0) static_cast<float*>(a.out)[row] = (xt - m) - 0.6931471805599453f * __log2f(sum);
+  } else {
+    const float k = a.beta * gr, inv = 1.0f / sum;
+    const int64_t out_off = row * a.out_ld;
+    for_chunks([&](int col, float (&v)[8]) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float p = ex2_approx(fmaf(v[i], kLog2e, -mb)) * inv;
+        v[i] = k * ((col + i == t ? 1.0f : 0.f) - p);
+      }
+      store8(a.out, a.out_dt, out_off, col, a.cols, true, v);
+    });
+    if (tid < tail) {
+      const int col = 8 * full + tid;
+      store_one(a.out, a.out_dt, out_off + col, k * ((col == t ? 1.0f : 0.f) - ex2_approx(fmaf(last, kLog2e, -mb)) * inv));
+    }
+  }
+  if (!staged && tid == 0)                                   // the copy lands before the CTA gives up its shared memory
+    for (uint32_t it = 0; it < kXentWaitLimit && !ptx::mbar_try_wait(bar, 0); ++it) {}
+}
+
 // One warp per row, for short rows: read twice (maximum, then sum of exponentials) and in the backward pass a third
 // time, from cache.
 template <bool BWD>
@@ -525,6 +601,13 @@ static us_status xent_launch_dt(const XentArgs& a, cudaStream_t st) {
   while (threads < 1024 && chunks > threads * kMaxCh) threads *= 2;
   const int nch = (chunks + threads - 1) / threads;
   const int rows = (int)a.rows;
+  if constexpr (DT != US_F32) {
+    // rows of 16385 to 36000 classes: three of them fit an SM's shared memory
+    if (a.vec_ok && (threads == 512 || (threads == 1024 && a.cols <= 36000))) {
+      static std::atomic<uint64_t> smem_set{0};
+      return host::launch_plain(softmax_xent_staged_kernel<BWD, DT>, &smem_set, rows, kXentStagedThreads, 72000, a.cols / 8 * 16, st, a);
+    }
+  }
   switch (nch > kMaxCh ? 0 : nch) {
     case 1: softmax_xent_row_kernel<BWD, DT, 1><<<rows, threads, 0, st>>>(a); break;
     case 2: softmax_xent_row_kernel<BWD, DT, 2><<<rows, threads, 0, st>>>(a); break;

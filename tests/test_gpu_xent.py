@@ -67,7 +67,7 @@ def test_softmax_xent_unit_scale_and_bad_targets():
 # Class counts at the edges of the row kernel's choices: a warp per row up to 512, then 128 ... 1024 threads with 1 to 8
 # (float32: 4) chunks of eight per thread, then rows that are re-read; row ends inside a chunk, with and without an
 # aligned row pitch.
-@pytest.mark.parametrize("cols", [512, 513, 1023, 1025, 4097, 8192, 8193, 16391, 30522, 32768, 32769, 65536, 65541])
+@pytest.mark.parametrize("cols", [512, 513, 1023, 1025, 4097, 8192, 8193, 16391, 30522, 30527, 32768, 32769, 36000, 36001, 65536, 65541])
 @pytest.mark.parametrize("in_fmt,out_fmt,pad", [("bf16", "e5m2", True), ("fp16", "f32", False), ("f32", "bf16", True)])
 def test_softmax_xent_row_kernel_edges(cols, in_fmt, out_fmt, pad):
     L, synth = _mods()
