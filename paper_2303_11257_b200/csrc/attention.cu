@@ -7,7 +7,7 @@
 //   * tcgen05.mma (kind::f16, M = 128, N = 256, twice) leaves the whole score block, 128 x 512
 //     float32, in tensor memory (all 512 columns): the scores never reach shared or global memory
 //     and are never rounded;
-//   * sixteen warps (four per TMEM lane quarter, one query row per lane, every fourth 32-column chunk each)
+//   * sixteen warps (four per TMEM lane quarter, one query row per lane)
 //     make three passes over their rows in tensor memory: maximum; exponentials, written back over the
 //     scores (tcgen05.st), and their sum; weights, scaled, rounded to the operand format and written
 //     to shared memory in the K-major swizzled layout of an MMA A operand, a key block (128 bytes of a
@@ -23,7 +23,8 @@
 // Bound: per tile of 128 queries x 512 keys the 65536 exponentials (4096 cycles of the ex2 unit) and the 128 KB of 16-bit
 // weights that leave through the SM's 32 bytes per clock (another 4096) run one after the other, because the scores fill
 // tensor memory.  16 x 512 tokens, 16 heads, 16-bit / FP8: 64.5 / 54.0 us with eight warps and two 32 KB buffers, 60.4 / 56.9
-// with four 16 KB buffers, 59.3 / 50.1 with sixteen warps as well (2.3 / 1.5 TB/s).
+// with four 16 KB buffers, 59.3 / 50.1 with sixteen warps as well; launches in a row 67.0 / 56.7 -> 60.4 / 50.9, that is 3.2 / 2.0
+// TB/s of Q, K, V, P and C (193 / 101 MB).
 // Every wait on an mbarrier is bounded; a wait that runs out raises the status word (as in the GEMM
 // kernels) and the CTA leaves after its own copies have landed and its tensor memory is freed.
 #include <cuda.h>
@@ -70,6 +71,16 @@ __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+
+// Sum of a row's terms, whose order is part of the result: eight chains, one for each (parity of the 32-key chunk, key
+// modulo 4), each in key order; then the four chains of a parity in pairs, then the two parities.  Warp (q, part) takes
+// parity part & 1 and, of every four keys, the two from 2 (part >> 1); it leaves the sum of its two chains in part's slot.
+// That order is the one of two warps per row, which sixteen warps keep at no cost in the forward kernel (a sum over every
+// fourth chunk instead takes as long) and for 77.5 / 64.5 against 76.2 / 61.6 us (16-bit / FP8) in the backward one, where
+// two warps then read each piece of P.
+__device__ __forceinline__ float row_total(const volatile float* part_sums, int r) {
+  return (part_sums[r] + part_sums[256 + r]) + (part_sums[128 + r] + part_sums[384 + r]);
 }
 
 // Tile n of a CTA: tiles blockIdx.x, blockIdx.x + gridDim.x, ... of q_tiles * nb1 * nb0, query tile fastest.
@@ -231,8 +242,8 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tq, const __grid_consta
   } else {
     // ------------------------------------------------------------------ softmax and output
     // kParts warps share each TMEM lane quarter (= 32 query rows, one per lane): warp (q, part) works on the
-    // 32-column chunks c = kParts i + part of its rows, and they exchange their partial row maxima and row
-    // sums through shared memory.
+    // 32-column chunks c = kParts i + part of its rows (the exponentials are dealt out as row_total says), and they
+    // exchange their partial row maxima and row sums through shared memory.
     const int q = warp & 3, part = (warp - 2) >> 2, r = q * 32 + lane;
     const uint32_t t_row = tmem + ((uint32_t)(q * 32) << 16);
     const int c_end = 4 * nq;                                  // 32-column chunks, whole quarters
@@ -273,28 +284,50 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tq, const __grid_consta
         for (int i = 0; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(x[i]));
       });
       row_max[part * 128 + r] = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+      ptx::tc_fence_before_sync();
       ptx::named_barrier_sync(1, 32 * kSoftmaxWarps);
+      ptx::tc_fence_after_sync();
       float rm = row_max[r];
 #pragma unroll
       for (int k = 1; k < kParts; ++k) rm = fmaxf(rm, row_max[k * 128 + r]);
       const float mk = rm * a.exp_scale;
-      float s4[4] = {0.f, 0.f, 0.f, 0.f};
-      sweep([&](int c, uint32_t (&x)[32]) {
-        mask(c, x);
+      // Exponentials and their row sum, the next chunk's columns loaded while this one's are worked on.
+      float s2[2] = {0.f, 0.f};
+      {
+        const uint32_t t_pair = t_row + 2u * (part >> 1);
+        uint32_t x[2][16];
+        auto exps = [&](int c, uint32_t (&v)[16]) {
+          if (32 * c + 32 > a.s_k) {
+            const int key0 = 32 * c + 2 * (part >> 1);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float e = ex2(fmaf(__uint_as_float(x[i]), a.exp_scale, -mk));
-          s4[i & 3] += e;
-          x[i] = __float_as_uint(e);
+            for (int i = 0; i < 16; ++i) if (key0 + 4 * (i >> 1) + (i & 1) >= a.s_k) v[i] = __float_as_uint(-3.0e38f);
+          }
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float e = ex2(fmaf(__uint_as_float(v[i]), a.exp_scale, -mk));
+            s2[i & 1] += e;
+            v[i] = __float_as_uint(e);
+          }
+          ptx::tmem_st_pairs(t_pair + 32u * c, v);             // the exponentials replace the scores
+        };
+        int c = part & 1;
+        ptx::tmem_ld_pairs_issue(t_pair + 32u * c, x[0]);
+#pragma unroll 1
+        for (; c < c_end; c += 4) {                            // c_end is a multiple of 4: two chunks of this parity
+          ptx::tmem_ld_fence(x[0]);
+          ptx::tmem_ld_pairs_issue(t_pair + 32u * (c + 2), x[1]);
+          exps(c, x[0]);
+          ptx::tmem_ld_fence(x[1]);
+          if (c + 4 < c_end) ptx::tmem_ld_pairs_issue(t_pair + 32u * (c + 4), x[0]);
+          exps(c + 2, x[1]);
         }
-        ptx::tmem_st_32x32_bits(t_row + 32u * c, x);           // the exponentials replace the scores
-      });
+      }
       ptx::tmem_st_wait();
-      row_sum[part * 128 + r] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+      row_sum[part * 128 + r] = s2[0] + s2[1];
+      ptx::tc_fence_before_sync();                             // the weights of a chunk are other warps' exponentials too
       ptx::named_barrier_sync(1, 32 * kSoftmaxWarps);
-      float rs = row_sum[r];
-#pragma unroll
-      for (int k = 1; k < kParts; ++k) rs += row_sum[k * 128 + r];
+      ptx::tc_fence_after_sync();
+      const float rs = row_total(row_sum, r);
       const float inv = a.softmax_scale / rs;
       const uint32_t row_off = (uint32_t)r * 128u, sw = (uint32_t)(r & 7);
       // weights, a 32-key chunk per warp at a time: chunk c belongs to key block c / 2 (16-bit) or c / 4 (FP8)
@@ -384,8 +417,8 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tq, const __grid_consta
 // 0..63; the tile of dS leaves by TMA store (the dK matmul reads it), eight of the warps scale and store dQ.
 // Bound: a 16-bit tile of P is one 128 KB buffer, so its load, the two passes (6000 of 18000 cycles) and the store of dS
 // follow one another; blocks are refilled one by one behind the store, from L2.  16 x 512 tokens, 16 heads, 16-bit / FP8:
-// 85.8 / 63.8 us before, 82.8 / 62.0 with the refill by blocks, 75.7 / 61.5 with sixteen warps, 74.6 / 60.1 with the L2 prefetch
-// (4.3 / 2.8 TB/s).
+// 85.8 / 63.8 us before, 82.8 / 62.0 with the refill by blocks, 75.7 / 61.5 with sixteen warps, 74.6 / 60.1 with the L2 prefetch;
+// launches in a row 89.6 / 67.2 -> 77.5 / 64.5 as it stands (row_total), that is 4.2 / 2.6 TB/s of dC, K, V, P, dS and dQ (327 / 168 MB).
 struct AttnBwdParams {
   int s_q, s_k;
   int q_tiles, nb1, nb0;
@@ -393,7 +426,6 @@ struct AttnBwdParams {
   float ds_scale;           // softmax_beta * beta_p / softmax_alpha
   float beta_q;
   void* dq; int dq_dt; int64_t dq_ld, dq_stride0, dq_stride1;
-  int op_bf16;
   uint32_t idesc_s, idesc_c;
   unsigned int* status;
   uint32_t wait_limit;
@@ -404,7 +436,8 @@ constexpr uint32_t kAttnBwdSmem = kQBytes + kKBytes + kTileBytes + 1024 + 128 + 
 
 // F8: dC and dS are E5M2 (gradients), P, K and V E4M3 (activations); layouts as in the forward kernel's FP8 form
 // (a 128-byte row of P / dS holds 128 keys; dC, V and K rows are 64 bytes in 128-byte boxes whose upper half is zero).
-template <bool F8>
+// BF16: 16-bit operands are BF16 (else F16); as a run-time flag it cost 2.7 us of a 16-bit pass.
+template <bool F8, bool BF16>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_bwd_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_constant__ CUtensorMap tv,
                      const __grid_constant__ CUtensorMap tk, const __grid_constant__ CUtensorMap tp,
@@ -594,7 +627,7 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_const
           const float2 lo = unpack_fp8x2((uint16_t)(w[j] & 0xffffu), false), hi = unpack_fp8x2((uint16_t)(w[j] >> 16), false);
           pv[4 * j] = lo.x; pv[4 * j + 1] = lo.y; pv[4 * j + 2] = hi.x; pv[4 * j + 3] = hi.y;
         } else {
-          const float2 f = a.op_bf16 ? unpack_bf16x2(w[j]) : unpack_f16x2(w[j]);
+          const float2 f = BF16 ? unpack_bf16x2(w[j]) : unpack_f16x2(w[j]);
           pv[2 * j] = f.x; pv[2 * j + 1] = f.y;
         }
       }
@@ -611,26 +644,38 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_const
       ptx::tc_fence_after_sync();
       int q0, b1, b0;
       coords(tile, q0, b1, b0);
-      // pass 1: sum_j P_j dP_j over this warp's chunks (columns beyond s_k hold zeros in both factors)
-      float s4[4] = {0.f, 0.f, 0.f, 0.f};
+      // pass 1: sum_j P_j dP_j (columns beyond s_k hold zeros in both factors) in the eight chains of row_total.  Register
+      // i of lo and hi is column i resp. 14 + i from this warp's first key: its keys are 4 k and 4 k + 1 from there.
+      float s2[2] = {0.f, 0.f};
+      const int odd = part >> 1;
 #pragma unroll 1
-      for (int c = part; c < c_end; c += kParts) {
-        float x[32];
-        ptx::tmem_ld_32x32(t_row + 32u * c, x);
+      for (int c = part & 1; c < c_end; c += 2) {
+        uint32_t lo[16], hi[16];
+        ptx::tmem_ld_32x32_issue(t_row + 32u * c + 2u * odd, lo);
+        ptx::tmem_ld_32x32_issue(t_row + 32u * c + 2u * odd + 14u, hi);
+        uint4 raw[kPieces];
 #pragma unroll
-        for (int g = 0; g < kPieces; ++g) {
-          float pv[16];
-          piece_values(ptx::lds128(p_addr(c, g)), pv);
+        for (int g = 0; g < kPieces; ++g) raw[g] = ptx::lds128(p_addr(c, g));
+        ptx::tmem_ld_fence(lo);
+        ptx::tmem_ld_fence(hi);
 #pragma unroll
-          for (int i = 0; i < kPieceVals; ++i) s4[i & 3] = fmaf(pv[i], x[kPieceVals * g + i], s4[i & 3]);
+        for (int k = 0; k < 8; ++k) {                          // keys 4 k .. 4 k + 3 of the chunk: this warp's two of them
+          const uint4 v = raw[k / (kPieceVals / 4)];
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+          float2 f;
+          if (F8) {
+            f = unpack_fp8x2((uint16_t)(w[k & 3] >> (16 * odd)), false);
+          } else {
+            const uint32_t u = odd ? w[2 * (k & 1) + 1] : w[2 * (k & 1)];
+            f = BF16 ? unpack_bf16x2(u) : unpack_f16x2(u);
+          }
+          s2[0] = fmaf(f.x, __uint_as_float(k < 4 ? lo[(4 * k) & 15] : hi[(4 * k - 14) & 15]), s2[0]);
+          s2[1] = fmaf(f.y, __uint_as_float(k < 4 ? lo[(4 * k + 1) & 15] : hi[(4 * k - 13) & 15]), s2[1]);
         }
       }
-      row_sum[part * 128 + r] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+      row_sum[part * 128 + r] = s2[0] + s2[1];
       ptx::named_barrier_sync(1, 32 * kSoftmaxWarps);
-      float rs = row_sum[r];
-#pragma unroll
-      for (int k = 1; k < kParts; ++k) rs += row_sum[k * 128 + r];
-      const float mean = rs * a.inv_alpha;                     // sum_j p_j dP_j in units of the raw accumulator
+      const float mean = row_total(row_sum, r) * a.inv_alpha;                     // sum_j p_j dP_j in units of the raw accumulator
       // pass 2: dS = ds_scale * P * (dP - mean), rounded, over P in place
 #pragma unroll 1
       for (int c = part; c < c_end; c += kParts) {
@@ -647,7 +692,7 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_const
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             if (F8) o[j] = cvt_fp8x4<true>(d[4 * j], d[4 * j + 1], d[4 * j + 2], d[4 * j + 3]);     // gradients: E5M2
-            else o[j] = a.op_bf16 ? pack_bf16x2(d[2 * j], d[2 * j + 1]) : pack_f16x2(d[2 * j], d[2 * j + 1]);
+            else o[j] = BF16 ? pack_bf16x2(d[2 * j], d[2 * j + 1]) : pack_f16x2(d[2 * j], d[2 * j + 1]);
           }
           ptx::sts128(addr, make_uint4(o[0], o[1], o[2], o[3]));
         }
@@ -832,8 +877,8 @@ extern "C" us_status us_attention_bwd(const us_mat* dC, const us_mat* P, const u
   a.beta_q = beta_q;
   a.dq = dQ->ptr; a.dq_dt = dQ->dtype; a.dq_ld = dQ->ld;
   a.dq_stride0 = cnt[0] > 1 ? batch->dq_stride[0] : 0; a.dq_stride1 = cnt[1] > 1 ? batch->dq_stride[1] : 0;
-  a.op_bf16 = dC->dtype == US_BF16;
-  const int fmt = a.op_bf16 ? 1 : 0;
+  const bool bf16 = dC->dtype == US_BF16;
+  const int fmt = bf16 ? 1 : 0;
   // FP8 (kind::f8f6f4: 0 = E4M3, 1 = E5M2): the A operands dC and dS are gradients, the B operands V and K activations
   a.idesc_s = f8 ? make_idesc(1, 0, false, false, 128, 256) : make_idesc(fmt, fmt, false, false, 128, 256);
   a.idesc_c = f8 ? make_idesc(1, 0, false, true, 128, 128) : make_idesc(fmt, fmt, false, true, 128, 64);
@@ -843,8 +888,8 @@ extern "C" us_status us_attention_bwd(const us_mat* dC, const us_mat* P, const u
   if (tiles > 0x7fffffff) return US_ERR_INVALID_ARG;
   const int sms = host::sm_count();
   if (sms <= 0) return US_ERR_CUDA;
-  auto kern = f8 ? attention_bwd_kernel<true> : attention_bwd_kernel<false>;
-  static std::atomic<uint64_t> smem_set[2];
+  auto kern = f8 ? attention_bwd_kernel<true, false> : bf16 ? attention_bwd_kernel<false, true> : attention_bwd_kernel<false, false>;
+  static std::atomic<uint64_t> smem_set[3];
   const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
-  return host::launch(kern, &smem_set[f8], (int)grid, kAttnThreads, kAttnBwdSmem, 1, static_cast<cudaStream_t>(stream), tdc, tv, tk, tp, tds, a);
+  return host::launch(kern, &smem_set[f8 ? 2 : fmt], (int)grid, kAttnThreads, kAttnBwdSmem, 1, static_cast<cudaStream_t>(stream), tdc, tv, tk, tp, tds, a);
 }

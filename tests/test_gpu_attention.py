@@ -343,3 +343,50 @@ def test_lengths_that_are_not_multiples_of_eight(s_q, s_k):
     assert (np.abs(got - ref) <= U.ulp_of(ref, "fp16") + 3e-6 * (np.abs(ref).max() + np.abs(dp).max())).all()
     ref_q = 0.125 * (got @ kv)
     assert np.abs(U.host_values(dQ) - ref_q).max() <= TOL * max(1.0, np.abs(ref_q).max())
+
+
+def _chain(k):
+    """The eight chains in which a row's 512 terms are summed: parity of the 32-key chunk, key modulo 4."""
+    return 4 * ((k // 32) & 1) + k % 4
+
+
+@pytest.mark.parametrize("s_k", [512, 200])
+@pytest.mark.parametrize("fmt", ["bf16", "fp16", "e4m3"])
+def test_row_sum_of_exponentials_is_taken_in_its_documented_order(fmt, s_k):
+    """One term of 1 opens a chain whose other terms are 2^-26: each addition rounds back to 1, so the sum of the row is
+    exactly 1 and the weight softmax_scale / 1 sits on the tie between two values of the format (to even: the upper one).
+    Any other split of that chain adds up some of the small terms first and lands below the tie."""
+    from paper_2303_11257_b200 import lib as L
+    key = np.arange(s_k)
+    K, first = np.full((s_k, 64), -96.0), [0] * 64
+    for row in range(64):                                      # Q is the identity: the scores of row r are column r of K
+        mine = np.flatnonzero(_chain(key) == row % 8)
+        K[mine, row] = -26.0
+        K[mine[0], row], first[row] = 0.0, mine[0]
+    Q, Kt = U.to_device(np.eye(64, dtype=np.float32), fmt), U.to_device(K, fmt)
+    P, Cx, ws = U.empty(64, s_k, fmt, (s_k + 15) // 16 * 16), U.empty(64, 64, "f32"), L.new_workspace()
+    step = 2.0 ** -F.FORMATS[fmt].M
+    L.us_attention_fwd(Q, Kt, Kt, float(np.log(2.0)), 1.0 + 1.5 * step, 1.0, Cx, P, L.attention_batch((1, 1), *[(0, 0)] * 5), ws)
+    assert L.us_workspace_status(ws) == 0
+    assert (U.host_values(P)[np.arange(64), first] == 1.0 + 2 * step).all()
+
+
+@pytest.mark.parametrize("s_k", [512, 208])
+@pytest.mark.parametrize("fmt", ["bf16", "fp16", "e4m3"])
+def test_row_sum_of_the_softmax_gradient_is_taken_in_its_documented_order(fmt, s_k):
+    """The same chains for sum P dP: a first term of big^2 that swallows the others' 2^-26 of it, so that the mean is exactly
+    that term's dP and its dS exactly zero."""
+    from paper_2303_11257_b200 import lib as L
+    big, small = (256.0, 2.0 ** -5) if fmt == "e4m3" else (1.0, 2.0 ** -13)
+    gfmt = "e5m2" if fmt == "e4m3" else fmt
+    key = np.arange(s_k)
+    P, V, first = np.zeros((64, s_k)), np.zeros((s_k, 64)), [0] * 64
+    for row in range(64):                                      # dC is the identity: dP of row r is column r of V
+        mine = np.flatnonzero(_chain(key) == row % 8)
+        P[row, mine], V[mine, row], first[row] = small, small, mine[0]
+        P[row, mine[0]], V[mine[0], row] = big, big
+    dC, Pt, Vt = U.to_device(np.eye(64, dtype=np.float32), gfmt), U.to_device(P, fmt), U.to_device(V, fmt)
+    dS, dQ, ws = U.empty(64, s_k, gfmt), U.empty(64, 64, "f32"), L.new_workspace()
+    L.us_attention_bwd(dC, Pt, Vt, Vt, 1.0, big, 1.0, 1.0, dS, dQ, L.attention_bwd_batch((1, 1), *[(0, 0)] * 6), ws)
+    assert L.us_workspace_status(ws) == 0
+    assert (U.host_values(dS)[np.arange(64), first] == 0.0).all()
