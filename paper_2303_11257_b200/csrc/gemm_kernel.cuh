@@ -785,6 +785,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA of a pair only)
     if (lane == 0 && rank == 0) {
+      ptx::grid_wait_previous();                       // no operand comes earlier: the bounded waits begin when the loads do
       int stage = 0; uint32_t phase = 0;
       uint32_t local = 0;
       bool ok = true;

@@ -11,8 +11,9 @@ namespace us {
 namespace host {
 // Launches a kernel that calls ptx::grid_wait_previous (programmatic dependent launch): its CTAs may take their
 // places and set up barriers and tensor memory while the previous kernel of the stream still drains, and wait there
-// for that kernel's completion before they touch memory.  Every thread of such a kernel waits, so that a grid never
-// completes ahead of its predecessors.  Worth its while where the grid is resident at once (the three launches of a
+// for that kernel's completion before they touch memory.  In such a kernel at least one thread of every CTA waits, so that
+// a grid never completes ahead of its predecessors, and so does every thread that touches global memory or makes bounded
+// waits (whose limit is then not spent on the predecessor).  Worth its while where the grid is resident at once (the three launches of a
 // 256 x 128 x 512 step 18.4 -> 16.4 us, of a 8192 x 1024 x 4096 one 199 -> 193 us); a grid of many waves pays for the wait
 // in every CTA (cross-entropy rows, 2048 CTAs: 39 -> 44 us) and is launched plainly.  cluster: CTAs per cluster (1: none).
 // smem_set: one static word per kernel, a bit per device on which its dynamic shared memory limit is set (nullptr: within 48 KB).

@@ -4,6 +4,8 @@ us_test_linear_fwd_starved launches the forward kernel with its operand loads wi
 wait limit: nothing is in flight, every role's wait runs out, the kernel raises the status word, frees its
 tensor memory and returns.  The context must stay usable: after clearing the word, an ordinary call
 on the same workspace has to match the oracle."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -57,3 +59,43 @@ def test_starved_launch_argument_checks():
             L.us_test_linear_fwd_starved(X, W, 1.0, Y, ws, wait_limit=bad)
         assert e.value.status == 1
     assert L.us_workspace_status(ws) == 0
+
+
+def _starve_linear(L, ws):
+    X, W, Y = U.empty(96, 64, "e4m3"), U.empty(64, 80, "e4m3"), U.empty(96, 80, "f32")
+    return lambda: L.us_test_linear_fwd_starved(X, W, 1.0, Y, ws, wait_limit=500)
+
+
+def _starve_hidden(L, ws):
+    X, W1, A = U.empty(200, 144, "e4m3"), U.empty(144, 336, "e4m3"), U.empty(200, 336, "e4m3")
+    G, W2, dH = U.empty(200, 144, "e5m2"), U.empty(336, 144, "e4m3"), U.empty(200, 336, "e5m2")
+    return lambda: L.us_test_ffn_hidden_starved(X, W1, G, W2, A, dH, ws, wait_limit=500)
+
+
+@pytest.mark.parametrize("make", [_starve_linear, _starve_hidden])
+def test_the_time_of_the_previous_kernel_is_not_counted_against_a_bounded_wait(make):
+    """A launch that overlaps a long predecessor (one tile, a contraction of 2^22) must begin to count its polls when that
+    has finished: half way through the predecessor its status word is still clear, although its limit is far shorter."""
+    from paper_2303_11257_b200 import lib as L
+    k = 1 << 22
+    X, W, Y = U.empty(16, k, "e4m3"), U.empty(k, 16, "e4m3"), U.empty(16, 16, "f32")
+    ws_long, ws, seen = L.new_workspace(), L.new_workspace(), torch.full((256,), 255, dtype=torch.uint8).pin_memory()
+    other, starve = torch.cuda.Stream(), make(L, ws)
+    L.us_linear_fwd(X, W, 1.0, Y, ws_long)
+    starve()                                              # kernels loaded, allocations made
+    torch.cuda.synchronize()
+    ws.zero_()
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    L.us_linear_fwd(X, W, 1.0, Y, ws_long)
+    torch.cuda.synchronize()
+    alone = time.perf_counter() - t0
+    assert alone > 2e-3                                        # far longer than 500 polls
+    L.us_linear_fwd(X, W, 1.0, Y, ws_long)
+    starve()
+    time.sleep(alone / 2)
+    with torch.cuda.stream(other):
+        seen.copy_(ws.view(torch.uint8)[:256], non_blocking=True)
+    other.synchronize()
+    assert not seen.any()
+    assert L.us_workspace_status(ws) == US_ERR_TIMEOUT and L.us_workspace_status(ws_long) == 0
