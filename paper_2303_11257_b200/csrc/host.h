@@ -9,6 +9,13 @@
 
 namespace us {
 namespace host {
+// The status of a failed runtime call.  The runtime also remembers the error; it is taken back here, or the next launch whose
+// status is read with cudaGetLastError would report it as its own.
+inline us_status failed() {
+  (void)cudaGetLastError();
+  return US_ERR_CUDA;
+}
+
 // Launches a kernel that calls ptx::grid_wait_previous (programmatic dependent launch): its CTAs may take their
 // places and set up barriers and tensor memory while the previous kernel of the stream still drains, and wait there
 // for that kernel's completion before they touch memory.  In such a kernel at least one thread of every CTA waits, so that
@@ -21,11 +28,11 @@ template <class... P, class... A>
 us_status launch(void (*kern)(P...), std::atomic<uint64_t>* smem_set, int grid, int threads, size_t smem, int cluster,
                  cudaStream_t stream, const A&... args) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return US_ERR_CUDA;
+  if (cudaGetDevice(&dev) != cudaSuccess) return failed();
   const uint64_t bit = 1ull << (dev & 63);
   const bool known = !smem_set || (smem_set->load(std::memory_order_relaxed) & bit);
   if (!known) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return US_ERR_CUDA;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return failed();
     smem_set->fetch_or(bit, std::memory_order_relaxed);
   }
   cudaLaunchConfig_t cfg = {};
@@ -40,7 +47,7 @@ us_status launch(void (*kern)(P...), std::atomic<uint64_t>* smem_set, int grid, 
   attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = cluster > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kern, P(args)...) == cudaSuccess ? US_OK : US_ERR_CUDA;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...) == cudaSuccess ? US_OK : failed();
 }
 
 // Number of SMs of the current device (cached per device), or -1 on error.
@@ -55,10 +62,10 @@ template <class... P, class... A>
 us_status launch_plain(void (*kern)(P...), std::atomic<uint64_t>* smem_set, int grid, int threads, int max_smem, size_t smem,
                        cudaStream_t stream, const A&... args) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return US_ERR_CUDA;
+  if (cudaGetDevice(&dev) != cudaSuccess) return failed();
   const uint64_t bit = 1ull << (dev & 63);
   if (!(smem_set->load(std::memory_order_relaxed) & bit)) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess) return US_ERR_CUDA;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess) return failed();
     smem_set->fetch_or(bit, std::memory_order_relaxed);
   }
   kern<<<(unsigned)grid, (unsigned)threads, smem, stream>>>(P(args)...);
