@@ -72,7 +72,7 @@ class UnitScaledEncoderLayer:
         self.dX = e(T, d, torch.bfloat16)
         self.dWqkv, self.dWo = e(d, 3 * d, torch.float32), e(d, d, torch.float32)
         self.ws = L.new_workspace(device)
-        self._plan, self._fork, self._join = None, torch.cuda.Event(), torch.cuda.Event()
+        self._plan = self._events = None
         if norm == "post":
             # post-norm (appendix "Model architectures"): a scaled layer norm after each residual sum
             self.U1, self.R2 = e(T, d, torch.bfloat16), e(T, d, torch.bfloat16)
@@ -191,6 +191,10 @@ class UnitScaledEncoderLayer:
         yield MAIN, p.group([(L.US_OP_BWD_W, self.Xq, self.dQKVq, sc["beta_w"], self.dWqkv, None, None),
                              (L.US_OP_BWD_X, self.dQKVq, self.Wqkv_q, sc["beta_qkv"], self.dX, g1, coef)], ws)
 
+    def __getstate__(self):
+        """A copy has buffers of its own: its plan is laid out, and its events are made, by its first step."""
+        return {**self.__dict__, "_plan": None, "_events": None}
+
     def _run(self, stream, **inputs):
         owned, state = self._owned(), self._state()
         p = self._plan
@@ -204,18 +208,20 @@ class UnitScaledEncoderLayer:
                 if call is not None:
                     call(st)
             return
-        cur, side = torch.cuda.current_stream(), self.ffn._side_streams()[0]
+        if self._events is None:
+            self._events = torch.cuda.Event(), torch.cuda.Event()
+        (fork, join), cur, side = self._events, torch.cuda.current_stream(), self.ffn._side_streams()[0]
         st, side_st = cur.cuda_stream, side.cuda_stream
         for where, call in p.calls(self._lay_out):
             if where == self.MAIN:
                 call(st)
             elif where == self.SIDE:
-                self._fork.record(cur)
-                side.wait_event(self._fork)
+                fork.record(cur)
+                side.wait_event(fork)
                 call(side_st)
             else:
-                self._join.record(side)
-                cur.wait_event(self._join)
+                join.record(side)
+                cur.wait_event(join)
 
     def step(self, X, Wqkv, Wo, W1, W2, G, stream=None, ln=None):
         """One forward + backward pass.  G is the gradient of the layer output; with norm = "post",

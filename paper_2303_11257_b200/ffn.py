@@ -110,6 +110,10 @@ class UnitScaledFFN:
         sc = self.sc
         return (sc.alpha1, sc.alpha2, sc.beta_x1, sc.beta_x2, sc.beta_w, sc.alpha_g, sc.beta_g, sc.s_in, self._c, self.keep_h, self.operand)
 
+    def __getstate__(self):
+        """A copy has buffers of its own: its plans are laid out, and its side streams are made, when it first needs them."""
+        return {**self.__dict__, "_plans": {}, "_side": None}
+
     def _run(self, kind, stream, **inputs):
         owned, state = self._owned(), self._state()
         p = self._plans.get(kind)

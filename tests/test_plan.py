@@ -1,10 +1,13 @@
 """The prepared calls of a block (lib.Plan): laid out once, their input slots refilled on every pass, laid out again when
 a buffer or a value they were made for changes.  No GPU: the calls are inspected, not issued."""
+import copy
 import gc
 import weakref
 
+import pytest
 import torch
 
+from paper_2303_11257_b200 import encoder, ffn
 from paper_2303_11257_b200 import lib as L
 
 
@@ -51,3 +54,50 @@ def test_a_pass_that_ends_early_is_laid_out_again_and_a_plan_keeps_nothing_but_i
         assert gone() is None
     finally:
         gc.enable()
+
+
+class _Recorder:
+    """Stands in for the library: notes every call (name, arguments) and returns a status for it."""
+
+    def __init__(self, status=lambda name, args: L.US_OK):
+        self.calls, self.status = [], status
+
+    def __getattr__(self, name):
+        def call(*args):
+            self.calls.append((name, args))
+            return self.status(name, args)
+        return call
+
+    def names(self):
+        return [n for n, _ in self.calls]
+
+
+def _ffn(**kw):
+    return ffn.UnitScaledFFN(64, 32, 64, device="cpu", **kw), [torch.zeros(s) for s in ((64, 32), (32, 64), (64, 32), (64, 32))]
+
+
+def _layer(**kw):
+    kw = {"fused_attention": True, **kw}
+    x = [torch.zeros(s) for s in ((128, 128), (128, 384), (128, 128), (128, 256), (256, 128), (128, 128))]
+    return encoder.UnitScaledEncoderLayer(2, 64, 128, 2, 256, device="cpu", **kw), x
+
+
+def _out_ptrs(rec):
+    return {a._obj.ptr for _, args in rec.calls for a in args if isinstance(getattr(a, "_obj", None), L.us_mat)}
+
+
+@pytest.mark.parametrize("make", [_ffn, _layer])
+def test_blocks_are_copied_before_and_after_a_step(make, monkeypatch):
+    """Prepared calls point into the object's buffers: they stay with it, and a copy lays out its own."""
+    block, x = make()
+    rec = _Recorder()
+    for stepped in (False, True):
+        if stepped:
+            monkeypatch.setattr(L, "_lib", rec)
+            block.step(*x, stream=0)
+        other = copy.deepcopy(block)
+        assert other.dX.data_ptr() != block.dX.data_ptr()
+    first, rec.calls = _out_ptrs(rec), []
+    other.step(*x, stream=0)
+    mine = {t.data_ptr() for t in block._owned()}
+    assert first & mine and not _out_ptrs(rec) & mine
