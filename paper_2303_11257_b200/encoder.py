@@ -228,16 +228,12 @@ class UnitScaledEncoderLayer:
         ln = (w1, c1, w2, c2) are the weights and biases of the two layer norms ([d] each)."""
         if self.ffn.grouped and self.ffn.fused_hidden:
             norm = dict(zip(("w1", "c1", "w2", "c2"), (t.view(1, -1) for t in ln))) if self.norm == "post" else {}
-            try:
-                self._run(stream, X=X, Wqkv=Wqkv, Wo=Wo, W1=W1, W2=W2, G=G, **norm)
-                return self.dX
-            except L.UnitScaleError as e:
-                if e.status != L.US_ERR_UNSUPPORTED:
-                    raise                                           # else: what a grouped form does not cover goes out singly
+            self._run(stream, X=X, Wqkv=Wqkv, Wo=Wo, W1=W1, W2=W2, G=G, **norm)
+            return self.dX
         return self._step_each(X, Wqkv, Wo, W1, W2, G, stream, ln)
 
     def _step_each(self, X, Wqkv, Wo, W1, W2, G, stream, ln):
-        """step() call by call."""
+        """step() call by call, for an FFN block whose grouped forms are switched off."""
         sc, ws, s = self.sc, self.ws, self.slen
         post = self.norm == "post"
         # ---- forward

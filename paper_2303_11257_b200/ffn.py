@@ -124,6 +124,7 @@ class UnitScaledFFN:
         st = L._stream(stream)
         for call in p.calls(getattr(self, "_plan_" + kind)):
             call(st)
+        return not call.refused                                 # the last call of a pass with gradients is its grouped launch
 
     def _plan_cast(self, p, src, dst):
         m = p.slot(src) if isinstance(src, str) else p.mat(src)
@@ -288,13 +289,9 @@ class UnitScaledFFN:
         the hidden layer's gradient is there go out as one launch while self.grouped is set; without it, with
         self.concurrent and no explicit stream, the weight-gradient GEMMs run on side streams."""
         if self.grouped:
-            try:
-                self._run("backward" if cast_g else "backward_from_cast", stream, G=G)
-                return self.dX, self.dW1, self.dW2
-            except L.UnitScaleError as e:
-                if e.status != L.US_ERR_UNSUPPORTED:
-                    raise
-                self.grouped = False                            # more tiles than the grouped form's work list holds
+            # False: more tiles than the grouped form's work list holds; this pass went out singly, later ones do so at once
+            self.grouped = self._run("backward" if cast_g else "backward_from_cast", stream, G=G)
+            return self.dX, self.dW1, self.dW2
         st = self.stages(None, None, None, G, fused_casts=False)[5 if cast_g else 6:]
         if not (self.concurrent and stream is None):
             for name, _, fn in st:
@@ -325,7 +322,7 @@ class UnitScaledFFN:
         and join back into the current stream (this also records as parallel branches under graph capture)."""
         if self.grouped and self.fused_casts and self.fused_hidden:
             try:
-                self._run("step", stream, X=X, W1=W1, W2=W2, G=G)
+                self.grouped = self._run("step", stream, X=X, W1=W1, W2=W2, G=G)
                 return self.dX, self.dW1, self.dW2
             except L.UnitScaleError as e:
                 if e.status not in (L.US_ERR_UNSUPPORTED, L.US_ERR_ALIGNMENT):

@@ -191,17 +191,21 @@ def _stream(stream) -> int:
 class Call:
     """A library call whose arguments are laid out once: calling it costs the C call and little else.  It points into
     tensors that the caller keeps (a block's own buffers); descriptions that change from call to call -- the tensors a
-    user passes to a step -- are written into its us_mat slots before each call (Plan.put)."""
-    __slots__ = ("name", "fn", "args", "keep")
+    user passes to a step -- are written into its us_mat slots before each call (Plan.put).  instead: (statuses, fn); a
+    call that the library refuses with one of those statuses, having launched nothing, issues fn(stream) in its place."""
+    __slots__ = ("name", "fn", "args", "keep", "instead", "refused")
 
-    def __init__(self, name, *args):
-        self.name, self.fn, self.keep = name, getattr(_lib, name), args
+    def __init__(self, name, *args, instead=((), None)):
+        self.name, self.fn, self.keep, self.instead, self.refused = name, getattr(_lib, name), args, instead, False
         self.args = tuple(C.byref(a) if isinstance(a, C.Structure) else a for a in args)
 
     def __call__(self, stream: int) -> None:
         status = self.fn(*self.args, stream)
         if status != US_OK:
-            raise UnitScaleError(self.name, status)
+            if status not in self.instead[0]:
+                raise UnitScaleError(self.name, status)
+            self.refused = True
+            self.instead[1](stream)
 
 
 class Plan:
@@ -268,7 +272,8 @@ class Plan:
         return ep
 
     def group(self, entries, ws):
-        """us_linear_group_any over (op, a, b, scale, out, skip or None, (skip_coef, out_coef))."""
+        """us_linear_group_any over (op, a, b, scale, out, skip or None, (skip_coef, out_coef)); as single launches where
+        there are more tiles than its work list holds."""
         arr = (us_linear_call * len(entries))()
         for c, (op, a, b, scale, out, skip, coef) in zip(arr, entries):
             c.op, c.a, c.b, c.scale, c.out, c.ep.out_coef = op, self.mat(a), self.mat(b), scale, self.mat(out), 1.0
@@ -279,7 +284,8 @@ class Plan:
                     self.slot(skip, c.ep.skip)
                 else:
                     c.ep.skip = self.mat(skip)
-        return Call("us_linear_group_any", len(entries), arr, ws.data_ptr(), ws.numel())
+        return Call("us_linear_group_any", len(entries), arr, ws.data_ptr(), ws.numel(),
+                    instead=((US_ERR_UNSUPPORTED,), lambda stream: linear_each(arr, ws, stream)))
 
     def linear(self, name, a, b, scale, out, ws, ep=None):
         return Call(name, self.mat(a), self.mat(b), scale, ep, self.mat(out), ws.data_ptr(), ws.numel())

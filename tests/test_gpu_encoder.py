@@ -144,3 +144,25 @@ def test_encoder_layer_post_norm(attention):
     # the layer output is normalised: per token, (R2 - c2) / w2 has zero mean and unit variance
     z = (layer.R2.float().cpu().numpy() - ln_host[3]) / ln_host[2]
     assert np.abs(z.mean(axis=1)).max() < 0.03 and np.abs(z.std(axis=1) - 1).max() < 0.03
+
+
+@pytest.mark.parametrize("attention,fused,norm", [("bf16", True, None), ("fp8", True, "post"), ("bf16", False, "post"), ("fp8", False, None)])
+def test_one_layer_stepped_with_other_tensors_equals_the_calls_one_by_one(attention, fused, norm):
+    """The prepared calls of a step take whatever tensors each pass is given (addresses, types), and do what the step does
+    call by call: every result bit for bit, on side streams and on a given one."""
+    from paper_2303_11257_b200 import encoder
+    nseq, slen, d, nhead, f = 3, 80, 128, 2, 272
+    T = nseq * slen
+    make = lambda: encoder.UnitScaledEncoderLayer(nseq, slen, d, nhead, f, attention=attention, fused_attention=fused, norm=norm)
+    planned, single = make(), make()
+    for seed, dtype, stream in ((0, torch.float32, None), (1, torch.bfloat16, None), (2, torch.float32, torch.cuda.current_stream())):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        x = [torch.randn(s, generator=g, device="cuda").to(dtype) for s in ((T, d), (d, 3 * d), (d, d), (d, f), (f, d), (T, d))]
+        ln = [torch.randn(d, generator=g, device="cuda") for _ in range(4)] if norm else None
+        planned.step(*x, stream=stream, ln=ln)
+        single._step_each(*x, stream, ln)
+        planned.check()
+        single.check()
+        out = lambda y: [y.dX, y.R2 if norm else y.ffn.R, y.dWqkv, y.dWo, y.ffn.dW1, y.ffn.dW2] + (y.dln if norm else [])
+        for a, b in zip(out(planned), out(single)):
+            assert torch.equal(a, b)

@@ -173,3 +173,25 @@ def test_step_on_three_streams_equals_step_on_one_stream():
         outs.append(eager)
     for a, b in zip(*outs):
         assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
+
+
+@pytest.mark.parametrize("operand", ["fp8", "bf16", "fp16"])
+def test_one_block_stepped_with_other_tensors_equals_new_blocks(operand):
+    """The prepared calls of a block take whatever tensors each pass is given: other addresses, types and (16-bit operands)
+    row pitches, against the single launches of a block of its own."""
+    from paper_2303_11257_b200 import ffn
+    T, d, f = 272, 144, 336
+    block = ffn.UnitScaledFFN(T, d, f, operand=operand)
+    for seed, dtype, pad in ((0, torch.float32, 0), (1, torch.bfloat16, 0), (2, torch.float32, 16 if operand != "fp8" else 0)):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        x = [torch.randn((r, c + pad), generator=g, device="cuda").to(dtype)[:, :c] for r, c in ((T, d), (d, f), (f, d), (T, d))]
+        block.step(*x)
+        other = ffn.UnitScaledFFN(T, d, f, operand=operand)
+        other.grouped = other.fused_casts = False
+        other.step(*x)
+        block.check()
+        other.check()
+        for a, b in zip((block.R, block.dX, block.dW1, block.dW2), (other.R, other.dX, other.dW1, other.dW2)):
+            assert torch.equal(a, b)
+        block.forward(x[0])                                    # evaluation with the weights of that step
+        assert torch.equal(block.R, other.R)

@@ -143,3 +143,25 @@ def test_group_any_fp8_outputs_of_small_tiles(out_fmt):
         L.us_linear_bwd_x(G, W, n ** -0.5, r, ws)
         assert np.array_equal(U.codes_of(o), U.codes_of(r))
     assert L.us_workspace_status(ws) == 0
+
+
+def test_more_tiles_than_the_work_list_holds_go_out_singly():
+    """46 x 46 tiles of 256 x 256 are more than the list's 2048 entries: the grouped call refuses them and launches nothing,
+    and a prepared pass issues the same GEMMs as single launches."""
+    L, synth = _mods()
+    n, k = 46 * 256, 16
+    X, W, G = (U.to_device(synth.normal(60, i, s), f) for i, s, f in ((0, (n, k), "e4m3"), (1, (k, n), "e4m3"), (2, (n, 64), "e5m2")))
+    ws = L.new_workspace()
+    big, dw, big1, dw1 = U.empty(n, n, "e4m3"), U.empty(k, 64, "f32"), U.empty(n, n, "e4m3"), U.empty(k, 64, "f32")
+    big.view(torch.uint8).fill_(0x55)
+    calls = [L.linear_call(L.US_OP_FWD, X, W, 0.25, big), L.linear_call(L.US_OP_BWD_W, X, G, 0.5, dw)]
+    with pytest.raises(L.UnitScaleError) as e:
+        L.us_linear_group_any(calls, ws)
+    assert e.value.status == L.US_ERR_UNSUPPORTED and bool((big.view(torch.uint8) == 0x55).all())
+    call = L.Plan((), ()).group([(L.US_OP_FWD, X, W, 0.25, big, None, None), (L.US_OP_BWD_W, X, G, 0.5, dw, None, None)], ws)
+    call(L.current_stream())
+    assert call.refused
+    L.us_linear_fwd(X, W, 0.25, big1, ws)
+    L.us_linear_bwd_w(X, G, 0.5, dw1, ws)
+    assert L.us_workspace_status(ws) == 0
+    assert torch.equal(big.view(torch.uint8), big1.view(torch.uint8)) and torch.equal(dw, dw1)

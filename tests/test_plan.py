@@ -101,3 +101,44 @@ def test_blocks_are_copied_before_and_after_a_step(make, monkeypatch):
     other.step(*x, stream=0)
     mine = {t.data_ptr() for t in block._owned()}
     assert first & mine and not _out_ptrs(rec) & mine
+
+
+GROUP, CAST = "us_linear_group_any", "us_cast_multi"
+
+
+def _refuse(name, status):
+    return lambda n, args: status if n == name else L.US_OK
+
+
+@pytest.mark.parametrize("norm", [None, "post"])
+def test_a_refused_group_goes_out_singly_and_nothing_is_issued_twice(norm, monkeypatch):
+    """More tiles than the work list of the grouped launch holds: the calls of that step are the others, each once, and the
+    group's GEMMs in its place -- in the first step and in later ones."""
+    ln = [torch.ones(128)] * 4 if norm else None
+    (layer, x), (other, _) = _layer(norm=norm), _layer(norm=norm)
+    rec = _Recorder()
+    monkeypatch.setattr(L, "_lib", rec)
+    layer.step(*x, stream=0, ln=ln)
+    want = []
+    for name, args in rec.calls:
+        want.append(name)
+        if name == GROUP:
+            want += [("us_linear_fwd", "us_linear_bwd_x", "us_linear_bwd_w")[c.op] for c in args[1]]
+    refusing = _Recorder(_refuse(GROUP, L.US_ERR_UNSUPPORTED))
+    monkeypatch.setattr(L, "_lib", refusing)
+    for _ in range(2):
+        other.step(*x, stream=0, ln=ln)
+        assert refusing.names() == want
+        refusing.calls.clear()
+
+
+def test_a_block_whose_group_is_refused_finishes_the_step_and_takes_the_general_form_from_then_on(monkeypatch):
+    block, x = _ffn()
+    rec = _Recorder(_refuse(GROUP, L.US_ERR_UNSUPPORTED))
+    monkeypatch.setattr(L, "_lib", rec)
+    block.step(*x, stream=0)
+    assert rec.names() == [CAST, "us_ffn_hidden_any", GROUP, "us_linear_bwd_w", "us_linear_bwd_w", "us_linear_fwd", "us_linear_bwd_x"]
+    assert not block.grouped
+    rec.calls.clear()
+    block.step(*x, stream=0)
+    assert GROUP not in rec.names() and rec.names().count("us_linear_bwd_w") == 2
