@@ -131,7 +131,7 @@ class UnitScaledFFN:
         return L.Call("us_cast_fp8", m, 1.0, p.mat(dst)) if self.operand == "fp8" else L.Call("us_residual_add", m, m, 0.0, p.mat(dst))
 
     def _plan_step(self, p):
-        yield p.cast_multi(["W1", "W2", "X", "G"], [self.W1q, self.W2q, self.Xq, self.Gq])
+        yield p.cast_multi(["W1", "W2", "X", "G"], [self.W1q, self.W2q, self.Xq, self.Gq], padded=self.operand != "fp8")
         yield from self.plan_gemms(p, "X", "G")
 
     def _plan_forward(self, p):
@@ -321,12 +321,8 @@ class UnitScaledFFN:
         With self.concurrent and no explicit stream, independent GEMMs go to two side streams that fork from
         and join back into the current stream (this also records as parallel branches under graph capture)."""
         if self.grouped and self.fused_casts and self.fused_hidden:
-            try:
-                self.grouped = self._run("step", stream, X=X, W1=W1, W2=W2, G=G)
-                return self.dX, self.dW1, self.dW2
-            except L.UnitScaleError as e:
-                if e.status not in (L.US_ERR_UNSUPPORTED, L.US_ERR_ALIGNMENT):
-                    raise                                       # else: what is not covered goes out in its general form
+            self.grouped = self._run("step", stream, X=X, W1=W1, W2=W2, G=G)
+            return self.dX, self.dW1, self.dW2
         st = self.stages(X, W1, W2, G)
         if self.grouped and self.fused_casts:
             cast_all = next(fn for name, _, fn in st if name == "cast_all")

@@ -250,8 +250,9 @@ class Plan:
             yield c
         self.done, self.mats = made, {}                         # a pass that ended early is laid out again
 
-    def cast_multi(self, srcs, dsts):
-        """us_cast_multi at scale 1; an entry of srcs is a tensor or the name of an input."""
+    def cast_multi(self, srcs, dsts, padded=False):
+        """us_cast_multi at scale 1; an entry of srcs is a tensor or the name of an input.  padded: rows that it does not
+        take (padded or unaligned ones) go out as one us_residual_add per tensor, for 16-bit destinations."""
         n = len(srcs)
         sm = (us_mat * n)()
         for i, s in enumerate(srcs):
@@ -259,7 +260,14 @@ class Plan:
                 self.slot(s, sm[i])
             else:
                 sm[i] = self.mat(s)
-        return Call("us_cast_multi", n, sm, (C.c_float * n)(*[1.0] * n), (us_mat * n)(*[self.mat(t) for t in dsts]))
+        dm = (us_mat * n)(*[self.mat(t) for t in dsts])
+
+        def each(stream):
+            for s, d in zip(sm, dm):
+                _check("us_residual_add", _lib.us_residual_add(C.byref(s), C.byref(s), 0.0, C.byref(d), stream))
+
+        return Call("us_cast_multi", n, sm, (C.c_float * n)(*[1.0] * n), dm,
+                    instead=((US_ERR_UNSUPPORTED, US_ERR_ALIGNMENT) if padded else (), each))
 
     def residual(self, skip, coef):
         """The fixed(tau) residual epilogue; skip is a tensor or the name of an input."""

@@ -142,3 +142,26 @@ def test_a_block_whose_group_is_refused_finishes_the_step_and_takes_the_general_
     rec.calls.clear()
     block.step(*x, stream=0)
     assert GROUP not in rec.names() and rec.names().count("us_linear_bwd_w") == 2
+
+
+def test_padded_inputs_of_a_16_bit_block_cost_one_refused_call_and_no_new_plan(monkeypatch):
+    block, x = _ffn(operand="bf16")
+    rec = _Recorder(_refuse(CAST, L.US_ERR_UNSUPPORTED))
+    monkeypatch.setattr(L, "_lib", rec)
+    block.step(*x, stream=0)
+    plan = block._plans["step"]
+    laid_out = plan.done
+    rec.calls.clear()
+    block.step(*x, stream=0)
+    assert rec.names() == [CAST] + 4 * ["us_residual_add"] + ["us_ffn_hidden_any", GROUP]
+    assert block._plans["step"] is plan and laid_out is not None and plan.done is laid_out
+
+
+def test_what_the_cast_of_an_fp8_block_refuses_stays_refused(monkeypatch):
+    for block, x in (_ffn(), _layer()):
+        rec = _Recorder(_refuse(CAST, L.US_ERR_UNSUPPORTED))
+        with monkeypatch.context() as m:
+            m.setattr(L, "_lib", rec)
+            with pytest.raises(L.UnitScaleError) as e:
+                block.step(*x, stream=0)
+        assert e.value.status == L.US_ERR_UNSUPPORTED and rec.names() == [CAST]
