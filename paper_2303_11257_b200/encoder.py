@@ -134,10 +134,6 @@ class UnitScaledEncoderLayer:
         sc, ws, s, f = self.sc, self.ws, self.slen, self.ffn
         post, fused = self.norm == "post", self.fused_attention
         coef = (self.c_skip, self.c_branch)
-        Q, K, V = (self._heads(self.QKV, i) for i in range(3))
-        dQ, dK, dV = (self._heads(self.dQKV, i) for i in range(3))
-        P, dS, C_h, dC_h = self.P[:s], self.dS[:s], self.Cq[:s, : self.hd], self.dC[:s, : self.hd]
-        tail = (ws.data_ptr(), ws.numel())
         MAIN = self.MAIN
 
         def norm_bwd(X, w, G, dX, dw, dc):
@@ -145,9 +141,13 @@ class UnitScaledEncoderLayer:
             return L.Call("us_layer_norm_bwd", p.mat(X), p.slot(w), g, self.eps, 1.0, self.beta_ln, p.mat(dX), L._vec(dw), L._vec(dc),
                           self.ln_ws.data_ptr(), self.ln_ws.numel())
 
+        # the first pass issues each call as it is laid out, so nothing is made before the call that needs it
         yield MAIN, p.cast_multi(["Wqkv", "Wo", "X", "W1", "W2"] + ([] if post else ["G"]),
                                  [self.Wqkv_q, self.Wo_q, self.Xq, f.W1q, f.W2q] + ([] if post else [f.Gq]))
         yield MAIN, p.linear("us_linear_fwd", self.Xq, self.Wqkv_q, sc["alpha_qkv"], self.QKV, ws)
+        Q, K, V = (self._heads(self.QKV, i) for i in range(3))
+        P, C_h = self.P[:s], self.Cq[:s, : self.hd]
+        tail = (ws.data_ptr(), ws.numel())
         if fused:
             yield MAIN, L.Call("us_attention_fwd", p.mat(Q), p.mat(K), p.mat(V), sc["alpha_s"], sc["sm"], sc["alpha_c"], p.mat(C_h), p.mat(P),
                                self.bt_fused, *tail)
@@ -174,6 +174,8 @@ class UnitScaledEncoderLayer:
         yield MAIN, L.Call("us_cast_fp8", p.mat(g1), 1.0, p.mat(self.g1q))
         yield MAIN, p.group([(L.US_OP_BWD_W, self.Cq, self.g1q, sc["beta_w"], self.dWo, None, None),
                              (L.US_OP_BWD_X, self.g1q, self.Wo_q, sc["beta_o"], self.dC, None, None)], ws)
+        dQ, dK, dV = (self._heads(self.dQKV, i) for i in range(3))
+        dS, dC_h = self.dS[:s], self.dC[:s, : self.hd]
         yield self.SIDE, p.batched("us_linear_bwd_w_batched", P, dC_h, sc["beta_V"], dV, self.bt["dV"], ws)
         gemm_dk = p.batched("us_linear_bwd_w_batched", dS, Q, sc["beta_K"], dK, self.bt["dK"], ws)
         if fused:

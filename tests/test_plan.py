@@ -165,3 +165,12 @@ def test_what_the_cast_of_an_fp8_block_refuses_stays_refused(monkeypatch):
             with pytest.raises(L.UnitScaleError) as e:
                 block.step(*x, stream=0)
         assert e.value.status == L.US_ERR_UNSUPPORTED and rec.names() == [CAST]
+
+
+def test_the_first_pass_issues_its_first_call_before_it_makes_what_later_ones_need(monkeypatch):
+    layer, x = _layer()
+    rec, heads, early = _Recorder(), layer._heads, []
+    monkeypatch.setattr(layer, "_heads", lambda *a: (early.append(len(rec.calls)), heads(*a))[1], raising=False)
+    monkeypatch.setattr(L, "_lib", rec)
+    layer.step(*x, stream=0)
+    assert early and min(early) >= 2 and rec.names()[:2] == [CAST, "us_linear_fwd"]
