@@ -512,7 +512,7 @@ us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_m
 
   const int tiles = p.tiles_m * p.tiles_n, most = pair ? sms / 2 : sms;
   const int units = tiles < most ? tiles : most;
-  const int split = pair || no_loads ? 1 : 4 * tiles <= sms ? 4 : 2 * tiles <= sms ? 2 : 1;
+  const int split = pair ? 1 : 4 * tiles <= sms ? 4 : 2 * tiles <= sms ? 2 : 1;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const bool bf = h_dtype == US_BF16;
   if (!f8) return X->dtype == US_BF16 ? pick_hidden<2, US_BF16, US_BF16>(pair, split, bf, t, p, units, st) : pick_hidden<2, US_F16, US_F16>(pair, split, bf, t, p, units, st);

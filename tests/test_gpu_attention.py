@@ -390,3 +390,50 @@ def test_row_sum_of_the_softmax_gradient_is_taken_in_its_documented_order(fmt, s
     L.us_attention_bwd(dC, Pt, Vt, Vt, 1.0, big, 1.0, 1.0, dS, dQ, L.attention_bwd_batch((1, 1), *[(0, 0)] * 6), ws)
     assert L.us_workspace_status(ws) == 0
     assert (U.host_values(dS)[np.arange(64), first] == 0.0).all()
+
+
+@pytest.mark.parametrize("fmt,s", [("bf16", 48), ("bf16", 136), ("bf16", 200), ("bf16", 328), ("bf16", 400), ("e4m3", 80), ("e4m3", 208), ("e4m3", 272)])
+def test_several_tiles_per_cta_with_every_number_of_key_blocks(fmt, s):
+    """More tiles than SMs, so that buffers, phases and refills carry over from tile to tile of a CTA, at numbers of key blocks
+    that the four weight buffers do not divide (1, 3, 4, 6 and 7; 1, 2 and 3): every problem bit for bit as in launches of one
+    sequence each (at most one tile per CTA), P stored and not, and sampled ones, the last among them, against the oracle."""
+    from paper_2303_11257_b200 import lib as L, synth
+    gfmt = "e5m2" if fmt == "e4m3" else fmt
+    nhead, q_tiles = 16, (s + 127) // 128
+    nseq = -(-2 * 160 // (nhead * q_tiles))                    # two or three tiles per CTA on 148 SMs
+    hd, d, T = 64, nhead * 64, nseq * s
+    qkv, dc = synth.normal(91, s, (T, 3 * d)), synth.normal(92, s, (T, d))
+    QKV, dC, ws = U.to_device(qkv, fmt), U.to_device(dc, gfmt), L.new_workspace()
+    a_s, sm, a_c = hd ** -0.5, float(s), s ** -0.5
+    st, td, sq = (s * 3 * d, hd), (s * d, hd), (nhead * s * s, s * s)
+
+    def run(first, count, store_p=True):
+        r, R = slice(first * s, first * s + s), slice(first * nhead * s, first * nhead * s + s)
+        Q, K, V = (QKV[r, o * d:o * d + hd] for o in range(3))
+        L.us_attention_fwd(Q, K, V, a_s, sm, a_c, Cx[r, :hd], P[R] if store_p else None, L.attention_batch((count, nhead), st, st, st, td, sq), ws)
+        if store_p:
+            L.us_attention_bwd(dC[r, :hd], P[R], K, V, a_s, sm, sm, a_s, dS[R], dQ[r, :hd], L.attention_bwd_batch((count, nhead), td, sq, st, st, sq, td), ws)
+
+    n = nseq * nhead * s
+    outs = []
+    for whole, store_p in ((True, True), (False, True), (True, False)):
+        Cx, P, dS, dQ = U.empty(T, d, "bf16"), U.empty(n, s, fmt), U.empty(n, s, gfmt), U.empty(T, d, "f32")
+        for first, count in ([(0, nseq)] if whole else [(i, 1) for i in range(nseq)]):
+            run(first, count, store_p)
+        assert L.us_workspace_status(ws) == 0
+        outs.append((Cx, P, dS, dQ))
+    for a, b in zip(outs[0], outs[1]):
+        assert torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
+    assert torch.equal(outs[0][0], outs[2][0])
+    Cx, P, dS, dQ = outs[0]
+    qv, dcv = U.values_of(qkv, fmt), U.values_of(dc, gfmt)
+    for i, j in ((0, 0), (nseq // 2, 7), (nseq - 1, nhead - 1)):
+        r, R = slice(i * s, (i + 1) * s), slice((i * nhead + j) * s, (i * nhead + j + 1) * s)
+        q, k, v = (qv[r, o * d + j * hd:o * d + (j + 1) * hd] for o in range(3))
+        p_ref, _ = O.attention_fwd(q, k, v, a_s, sm, a_c, "f64")
+        p_dev = U.host_values(P[R])
+        assert (np.abs(p_dev - F.quantise(p_ref, F.FORMATS[fmt])) <= U.ulp_of(p_ref, fmt) + 3e-6 * sm).all(), (i, j)
+        dp = np.float64(np.float32(a_s)) * (dcv[r, j * hd:(j + 1) * hd] @ v.T)
+        ref = O.softmax_bwd(p_dev, dp, sm, sm)
+        err = np.abs(U.host_values(dS[R]) - F.quantise(ref, F.FORMATS[gfmt]))
+        assert (err <= U.ulp_of(ref, gfmt) + 3e-6 * (np.abs(ref).max() + np.abs(dp).max())).all(), (i, j)

@@ -36,6 +36,10 @@ def _oracle(val, alpha, beta_x, s_in, ag, bg, h_fmt, a_fmt, d_fmt):
     return H, F.quantise_codes(A, F.FORMATS[a_fmt]), F.quantise_codes(dH, F.FORMATS[d_fmt])
 
 
+# One shape per form of the launch on 148 SMs, ragged in every dimension, K1 != K2 (b, m, f, n): 128 x 128 tiles computed by
+# four, two or one CTA each (6, 45 and 136 tiles), 256 x 256 tiles of CTA pairs (48).
+FORMS = {"four": (200, 144, 336, 208), "two": (520, 272, 1040, 400), "one": (1000, 528, 2096, 272), "pair": (1300, 272, 1808, 400)}
+
 CASES = [
     # b, m, f, n, h_fmt, a_fmt, d_fmt, s_in
     (256, 128, 512, 128, "bf16", "e4m3", "e5m2", 1.0),        # the small FFN configuration
@@ -139,11 +143,11 @@ def test_ffn_hidden_host_checks_launch_nothing():
     assert L.us_workspace_status(ws) == 0
 
 
-def test_ffn_hidden_starved_launch_times_out_and_the_next_call_is_correct():
+@pytest.mark.parametrize("b,m,f,n", [(520, 272, 1040, 272)] + [FORMS[k] for k in ("four", "one", "pair")])
+def test_ffn_hidden_starved_launch_times_out_and_the_next_call_is_correct(b, m, f, n):
     """The bounded waits of this kernel, exercised in the permitted form: no loads are issued, the waits of every role
-    run out, the status word is raised, tensor memory is freed and the kernel returns by itself."""
+    run out, the status word is raised, tensor memory is freed and the kernel returns by itself.  Every form of tile."""
     L, synth = _mods()
-    b, m, f, n = 520, 272, 1040, 272
     dev, val = _inputs(synth, b, m, f, n, 77)
     Xt, W1t, Gt, W2t = dev
     ws = L.new_workspace()
@@ -170,16 +174,30 @@ def test_ffn_hidden_starved_launch_times_out_and_the_next_call_is_correct():
 @pytest.mark.parametrize("act,grad,h_fmt", [("bf16", "bf16", "bf16"), ("fp16", "fp16", "bf16"), ("bf16", "bf16", "fp16"), ("e4m3", "e5m2", "bf16")])
 def test_ffn_hidden_any_equals_the_separate_calls(b, m, f, n, act, grad, h_fmt):
     """Every operand width and both tile sizes, down to single rows: A, dH and the kept copy bit for bit."""
+    _any_equals_separate(b, m, f, n, act, grad, h_fmt, lambda cols: (cols + 15) // 16 * 16)
+
+
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("act,grad,h_fmt", [("bf16", "bf16", "bf16"), ("fp16", "fp16", "fp16"), ("bf16", "bf16", "fp16"), ("e4m3", "e5m2", "fp16"),
+                                            ("e4m3", "e5m2", "bf16"), ("e5m2", "e4m3", "bf16"), ("e5m2", "e5m2", "fp16"), ("e4m3", "e4m3", "bf16")])
+@pytest.mark.parametrize("h_rows", ["sectors", "halves", None])
+def test_ffn_hidden_any_in_each_form(form, act, grad, h_fmt, h_rows):
+    """Every form of tile with every operand and output format; the kept copy with rows on 32-byte boundaries, with rows
+    that are only 16-byte aligned, and not kept."""
+    _any_equals_separate(*FORMS[form], act, grad, h_fmt, lambda cols: cols + (8 if h_rows == "halves" else 0), h_rows is not None)
+
+
+def _any_equals_separate(b, m, f, n, act, grad, h_fmt, h_ld, keep=True):
     L, synth = _mods()
     ws = L.new_workspace()
     X, W1 = U.to_device(synth.normal(7, 0, (b, m)), act, (m + 15) // 16 * 16), U.to_device(synth.normal(7, 1, (m, f)), act, (f + 15) // 16 * 16)
     G, W2 = U.to_device(synth.normal(7, 2, (b, n)), grad), U.to_device(synth.normal(7, 3, (f, n)), act)
     out = lambda fmt: U.empty(b, f, fmt, (f + 15) // 16 * 16)
-    A, dH, H = out(act), out(grad), out(h_fmt)
-    L.us_ffn_hidden_any(X, W1, m ** -0.5, G, W2, n ** -0.5, 0.75, 1.7, 1.48, A, dH, ws, H=H, h_dtype=H.dtype)
+    A, dH, H = out(act), out(grad), U.empty(b, f, h_fmt, h_ld(f))
+    L.us_ffn_hidden_any(X, W1, m ** -0.5, G, W2, n ** -0.5, 0.75, 1.7, 1.48, A, dH, ws, H=H if keep else None, h_dtype=H.dtype)
     A1, dH1, H1 = out(act), out(grad), out(h_fmt)
     L.us_linear_fwd(X, W1, m ** -0.5, A1, ws, L.epilogue(act=L.US_ACT_GELU, act_in_scale=0.75, act_out_scale=1.7, aux=H1))
     L.us_linear_bwd_x(G, W2, n ** -0.5, dH1, ws, L.epilogue(act=L.US_ACT_GELU_GRAD, act_in_scale=0.75, act_out_scale=1.48, aux=H1))
     assert L.us_workspace_status(ws) == 0
-    for a, r in ((H, H1), (A, A1), (dH, dH1)):
+    for a, r in ((A, A1), (dH, dH1)) + (((H, H1),) if keep else ()):
         assert np.array_equal(U.codes_of(a), U.codes_of(r))

@@ -133,10 +133,11 @@ def test_group_any_equals_single_calls(fmt, b, m, n):
 
 @pytest.mark.parametrize("out_fmt", ["e5m2", "e4m3"])
 def test_group_any_fp8_outputs_of_small_tiles(out_fmt):
-    """FP8 results of 128 x 128 tiles leave by 64-byte boxes: ragged columns and a second tile."""
+    """FP8 results of 128 x 128 tiles leave by 32-byte boxes where two CTAs share a tile, by 64-byte boxes otherwise (128
+    tiles): ragged columns and a second tile."""
     L, synth = _mods()
     ws = L.new_workspace()
-    for b, m, n in ((40, 208, 80), (200, 64, 176)):
+    for b, m, n in ((40, 208, 80), (200, 64, 176), (2000, 1008, 80)):
         G, W = U.to_device(synth.normal(50, 0, (b, n)), "e5m2"), U.to_device(synth.normal(50, 1, (m, n)), "e4m3")
         o, r = U.empty(b, m, out_fmt), U.empty(b, m, out_fmt)
         L.us_linear_group_any([L.linear_call(L.US_OP_BWD_X, G, W, n ** -0.5, o)], ws)
