@@ -237,8 +237,8 @@ __global__ void __launch_bounds__(kSmThreads, 2) softmax_bwd16_kernel(const SmAr
 
 // ---------------------------------------------------------------- softmax cross-entropy
 // softmax_xent(x, t) = log softmax(x)_t (table row "softmax_xent": alpha = 1, beta = s / sqrt(s - 1)).
-// Two kernels, chosen by the class count (xent_launch): one CTA per row for vocabulary-sized rows, one warp
-// per row for short ones.
+// Three kernels, chosen by the class count and the number of rows (xent_launch_dt): one CTA per row for vocabulary-sized
+// rows, held in registers or staged in shared memory, one warp per row for short ones.
 struct XentArgs {
   const void* x; int x_dt; int64_t x_ld;
   const int32_t* t;
@@ -585,14 +585,21 @@ extern "C" us_status us_softmax_bwd(const us_mat* P, const us_mat* dP, float alp
 
 template <bool BWD, int DT>
 static us_status xent_launch_dt(const XentArgs& a, cudaStream_t st) {
-  // A warp per row up to 512 classes (two chunks per lane); beyond, the smallest CTA whose threads hold the row in at
+  // A warp per row up to 512 classes (two chunks per lane), and in the forward pass up to 1280 where there are rows enough to
+  // fill the chip that way (16384 x 512 / 640 / 1024 / 1280 / 2048 BF16 logits, forward: a warp per row 9.4 / 9.9 / 12.2 / 14.5 /
+  // 23.8 us, a CTA per row 14.7 / 13.9 / 14.5 / 16.6 / 20.9; 2048 x 640 / 1024: 3.5 / 4.2 against 3.2 / 3.4; the forms are even at
+  // 2400 x 640, 3600 x 1024 and 5000 x 1280.  Backward 16384 x 512 / 640 / 1024: 14.7 / 17.8 / 22.9 against 17.2 / 18.2 / 20.8).
+  // Beyond, the smallest CTA whose threads hold the row in at
   // most 8 chunks of 16-bit or 4 chunks of float32 elements (32 registers of data each): few warps with many loads in
   // flight each and two or more CTAs per SM (30522 classes: 512 threads x 8 chunks 39 / 66 us forward / backward,
   // 1024 x 4 42 / 92 us, because one CTA then fills the SM and nothing overlaps its reductions).
   constexpr int kMaxCh = DT == US_F32 ? 4 : 8;
   const int64_t grid = (a.rows + kSmThreads / 32 - 1) / (kSmThreads / 32);
   if (grid > 0x7fffffff) return US_ERR_INVALID_ARG;
-  if (a.cols <= 512 || a.rows > 0x7fffffff) {
+  const int sms = host::sm_count();
+  if (sms <= 0) return US_ERR_CUDA;
+  const bool many_rows = !BWD && a.vec_ok && a.cols <= 1280 && a.rows >= 16 * sms && a.rows >= 4ll * a.cols;
+  if (a.cols <= 512 || many_rows || a.rows > 0x7fffffff) {
     softmax_xent_kernel<BWD><<<(int)grid, kSmThreads, 0, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
   }
@@ -602,7 +609,9 @@ static us_status xent_launch_dt(const XentArgs& a, cudaStream_t st) {
   const int nch = (chunks + threads - 1) / threads;
   const int rows = (int)a.rows;
   if constexpr (DT != US_F32) {
-    // rows of 16385 to 36000 classes: three of them fit an SM's shared memory
+    // Rows of 16385 to 36000 classes: three of them fit an SM's shared memory, and the register form needs 512 threads a row
+    // (2048 x 16384 / 16400 / 24576 BF16 logits, forward and backward: staged 20.9 + 37.3 / 20.8 + 37.6 / 25.5 + 48.8 us, in
+    // registers 18.7 + 35.2 / 21.0 + 43.5 / 33.1 + 56.0)
     if (a.vec_ok && (threads == 512 || (threads == 1024 && a.cols <= 36000))) {
       static std::atomic<uint64_t> smem_set{0};
       return host::launch_plain(softmax_xent_staged_kernel<BWD, DT>, &smem_set, rows, kXentStagedThreads, 72000, a.cols / 8 * 16, st, a);

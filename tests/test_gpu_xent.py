@@ -83,3 +83,17 @@ def test_softmax_xent_row_kernel_edges(cols, in_fmt, out_fmt, pad):
     assert np.abs(out.cpu().numpy() - ref).max() <= 4e-6 * (1 + np.abs(ref).max())
     L.us_softmax_xent_bwd(Xt, tt, None, 8.0, dX)
     U.assert_close_stored(dX, O.softmax_xent_bwd(xv, t, np.ones(rows), 8.0), out_fmt, 3e-6 * 8.0, "xent bwd")
+
+
+# The forward pass of many rows: a warp per row up to 1280 classes from 16 rows per SM and 4 rows per class on, and the row
+# kernel right beside that line.
+@pytest.mark.parametrize("rows,cols", [(2368, 513), (2367, 513), (2400, 595), (4096, 1024), (4095, 1024), (5120, 1280), (5121, 1275), (5124, 1281)])
+@pytest.mark.parametrize("in_fmt", ["bf16", "fp16", "f32"])
+def test_softmax_xent_forward_of_many_rows(rows, cols, in_fmt):
+    L, synth = _mods()
+    x = synth.normal(34, cols, (rows, cols), 2.0)
+    t = (np.arange(rows) * 7919 % cols).astype(np.int32)
+    out = torch.empty(rows, device="cuda")
+    L.us_softmax_xent_fwd(U.to_device(x, in_fmt, (cols + 15) // 16 * 16), torch.from_numpy(t).cuda(), out)
+    ref = O.softmax_xent_fwd(U.values_of(x, in_fmt), t)
+    assert np.abs(out.cpu().numpy() - ref).max() <= 4e-6 * (1 + np.abs(ref).max())
