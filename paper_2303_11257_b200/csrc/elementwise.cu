@@ -52,7 +52,7 @@ template <int OP>
 __global__ void __launch_bounds__(kThreads) ew_kernel(const EwArgs p) {
   constexpr bool kTwoInputs = (OP == kGeluBwd || OP == kResidual || OP == kActBwd);
   const int64_t total = p.rows * p.chunks_per_row;
-  for (int64_t c = blockIdx.x * (int64_t)kThreads + threadIdx.x + ptx::grid_sync_previous(); c < total;
+  for (int64_t c = blockIdx.x * (int64_t)kThreads + threadIdx.x + ptx::grid_wait_previous(); c < total;
        c += (int64_t)gridDim.x * kThreads) {
     const int64_t row = p.rows == 1 ? 0 : c / p.chunks_per_row;      // tensors without row padding arrive as one long row
     const int64_t col = (c - row * p.chunks_per_row) * kVec;

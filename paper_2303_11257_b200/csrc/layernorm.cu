@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kLnThreads, 2) ln_fwd16_kernel(const LnArgs a)
   extern __shared__ __align__(16) float ln_smem[];                         // w[cols], c[cols] as float32
   float* w_s = ln_smem;
   float* c_s = ln_smem + a.cols;
-  const int zero = ptx::grid_sync_previous();
+  const int zero = ptx::grid_wait_previous();
   for (int j = threadIdx.x + zero; j < a.cols; j += blockDim.x) { w_s[j] = load_one(a.w, a.w_dt, j); c_s[j] = load_one(a.c, a.c_dt, j); }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
   // (columns 8 q .. 8 q + 7) are split into a low and a high half; low halves at [4 q, 4 q + 4), high halves
   // kLnHi floats further.
   const int kLnHi = NCH * 32 * 4;
-  const int zero = ptx::grid_sync_previous();
+  const int zero = ptx::grid_wait_previous();
   for (int j = threadIdx.x + zero; j < a.cols; j += blockDim.x)
     w_s[(j >> 3) * 4 + (j & 3) + ((j & 4) ? kLnHi : 0)] = load_one(a.w, a.w_dt, j);
   __syncthreads();
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(32 * kLnReduceGroups) ln_bwd_reduce_kernel(con
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int j = blockIdx.x * 32 + tx;               // index into [2][cols]
   float s4[4] = {0.f, 0.f, 0.f, 0.f};
-  const int zero = ptx::grid_sync_previous();
+  const int zero = ptx::grid_wait_previous();
   if (j < 2 * cols) {
     int p = ty + zero;
     for (; p + 3 * kLnReduceGroups < nparts; p += 4 * kLnReduceGroups) {
@@ -674,7 +674,7 @@ extern "C" us_status us_layer_norm_bwd(const us_mat* X, const us_mat* w, const u
 #undef US_LN_PICK
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return US_ERR_CUDA;
+      return host::failed();
     const us_status launched = host::launch(fn, nullptr, nparts, 32 * kLnFastWarps, smem, 1, st, a);
     if (launched != US_OK) return launched;
   } else if (nch <= 4) {
@@ -685,7 +685,7 @@ extern "C" us_status us_layer_norm_bwd(const us_mat* X, const us_mat* w, const u
   } else {
     const size_t smem = (size_t)4 * 2 * a.cols * sizeof(float);
     if (cudaFuncSetAttribute(ln_bwd_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return US_ERR_CUDA;
+      return host::failed();
     ln_bwd_kernel<0><<<grid, 128, smem, st>>>(a);
   }
   if (cudaGetLastError() != cudaSuccess) return US_ERR_CUDA;

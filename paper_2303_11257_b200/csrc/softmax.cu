@@ -141,7 +141,7 @@ template <int NCH>
 __global__ void __launch_bounds__(kSmThreads, 2) softmax_fwd16_kernel(const SmArgs a) {
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int64_t stride = (int64_t)gridDim.x * nw;
-  int64_t row = (int64_t)blockIdx.x * nw + (threadIdx.x >> 5) + ptx::grid_sync_previous();
+  int64_t row = (int64_t)blockIdx.x * nw + (threadIdx.x >> 5) + ptx::grid_wait_previous();
   uint4 cur[NCH], nxt[NCH];
   if (row < a.rows) load_row16<NCH>(a.in0, row * a.in0_ld, lane, a.cols, cur);
   for (; row < a.rows; row += stride) {
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kSmThreads, 2) softmax_bwd16_kernel(const SmAr
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int64_t stride = (int64_t)gridDim.x * nw;
   const float inv_alpha = 1.0f / a.alpha;
-  int64_t row = (int64_t)blockIdx.x * nw + (threadIdx.x >> 5) + ptx::grid_sync_previous();
+  int64_t row = (int64_t)blockIdx.x * nw + (threadIdx.x >> 5) + ptx::grid_wait_previous();
   uint4 cp[P8 ? 1 : NCH], cg[NCH], np_[P8 ? 1 : NCH], ng[NCH];
   uint2 cp8[P8 ? NCH : 1], np8[P8 ? NCH : 1];
   if (row < a.rows) {
