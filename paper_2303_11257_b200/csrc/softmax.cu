@@ -441,7 +441,8 @@ __global__ void __launch_bounds__(kXentStagedThreads, 3) softmax_xent_staged_ker
 
 // One warp per row, for short rows: read twice (maximum, then sum of exponentials) and in the backward pass a third
 // time, from cache.
-template <bool BWD>
+// RAGGED: rows end inside a chunk of eight (the test costs 3 %).
+template <bool BWD, bool RAGGED>
 __global__ void __launch_bounds__(kSmThreads) softmax_xent_kernel(const XentArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * (kSmThreads / 32) + (threadIdx.x >> 5);
@@ -454,7 +455,7 @@ __global__ void __launch_bounds__(kSmThreads) softmax_xent_kernel(const XentArgs
     const int col = (c * 32 + lane) * 8;
     if (col >= a.cols) continue;
     float v[8];
-    load8(a.x, a.x_dt, x_off, col, a.cols, vec && col + 8 <= a.cols, -INFINITY, v);
+    load8(a.x, a.x_dt, x_off, col, a.cols, vec && (!RAGGED || col + 8 <= a.cols), -INFINITY, v);
 #pragma unroll
     for (int i = 0; i < 8; ++i) m = fmaxf(m, v[i]);
   }
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(kSmThreads) softmax_xent_kernel(const XentArgs
     const int col = (c * 32 + lane) * 8;
     if (col >= a.cols) continue;
     float v[8];
-    load8(a.x, a.x_dt, x_off, col, a.cols, vec && col + 8 <= a.cols, -INFINITY, v);
+    load8(a.x, a.x_dt, x_off, col, a.cols, vec && (!RAGGED || col + 8 <= a.cols), -INFINITY, v);
 #pragma unroll
     for (int i = 0; i < 8; ++i) sum += ex2_approx(fmaf(v[i], kLog2e, -mb));
   }
@@ -486,13 +487,13 @@ __global__ void __launch_bounds__(kSmThreads) softmax_xent_kernel(const XentArgs
     const int col = (c * 32 + lane) * 8;
     if (col >= a.cols) continue;
     float v[8];
-    load8(a.x, a.x_dt, x_off, col, a.cols, vec && col + 8 <= a.cols, -INFINITY, v);
+    load8(a.x, a.x_dt, x_off, col, a.cols, vec && (!RAGGED || col + 8 <= a.cols), -INFINITY, v);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const float p = ex2_approx(fmaf(v[i], kLog2e, -mb)) * inv;
       v[i] = k * ((col + i == t ? 1.0f : 0.f) - p);
     }
-    store8(a.out, a.out_dt, out_off, col, a.cols, vec && col + 8 <= a.cols, v);
+    store8(a.out, a.out_dt, out_off, col, a.cols, vec && (!RAGGED || col + 8 <= a.cols), v);
   }
 }
 
@@ -585,22 +586,25 @@ extern "C" us_status us_softmax_bwd(const us_mat* P, const us_mat* dP, float alp
 
 template <bool BWD, int DT>
 static us_status xent_launch_dt(const XentArgs& a, cudaStream_t st) {
-  // A warp per row up to 512 classes (two chunks per lane), and in the forward pass up to 1280 where there are rows enough to
-  // fill the chip that way (16384 x 512 / 640 / 1024 / 1280 / 2048 BF16 logits, forward: a warp per row 9.4 / 9.9 / 12.2 / 14.5 /
-  // 23.8 us, a CTA per row 14.7 / 13.9 / 14.5 / 16.6 / 20.9; 2048 x 640 / 1024: 3.5 / 4.2 against 3.2 / 3.4; the forms are even at
-  // 2400 x 640, 3600 x 1024 and 5000 x 1280.  Backward 16384 x 512 / 640 / 1024: 14.7 / 17.8 / 22.9 against 17.2 / 18.2 / 20.8).
-  // Beyond, the smallest CTA whose threads hold the row in at
-  // most 8 chunks of 16-bit or 4 chunks of float32 elements (32 registers of data each): few warps with many loads in
-  // flight each and two or more CTAs per SM (30522 classes: 512 threads x 8 chunks 39 / 66 us forward / backward,
-  // 1024 x 4 42 / 92 us, because one CTA then fills the SM and nothing overlaps its reductions).
+  // A warp per row up to 512 classes (two chunks per lane), and in the forward pass up to 1280 (16-bit: 1536) where there
+  // are rows enough to fill the chip that way.  BF16 logits, us, a warp per row against a CTA per row: forward 16384 x 512 /
+  // 640 / 1024 / 1280 / 2048: 9.4 / 9.6 / 12.2 / 14.1 / 23.8 against 14.7 / 13.9 / 14.5 / 16.6 / 20.9, 2048 x 640 / 1024: 3.5 / 4.2
+  // against 3.2 / 3.4, even at 2400 x 640, 3600 x 1024, 5000 x 1280 and 14000 x 1536, 65536 x 1536 63 against 75 (F32: 77, 72);
+  // backward 16384 x 512 / 640 / 1024: 14.7 / 17.8 / 22.9 against 17.2 / 18.2 / 20.8.
+  // Beyond, the smallest CTA whose threads hold the row in at most 8 chunks of 16-bit or 4 chunks of float32 elements (32
+  // registers of data each): few warps with many loads in flight each and two or more CTAs per SM (30522 classes: 512 threads
+  // x 8 chunks 39 / 66 us forward / backward, 1024 x 4 42 / 92 us, because one CTA then fills the SM and nothing overlaps its
+  // reductions).
   constexpr int kMaxCh = DT == US_F32 ? 4 : 8;
   const int64_t grid = (a.rows + kSmThreads / 32 - 1) / (kSmThreads / 32);
   if (grid > 0x7fffffff) return US_ERR_INVALID_ARG;
   const int sms = host::sm_count();
   if (sms <= 0) return US_ERR_CUDA;
-  const bool many_rows = !BWD && a.vec_ok && a.cols <= 1280 && a.rows >= 16 * sms && a.rows >= 4ll * a.cols;
+  const int limit = DT == US_F32 ? 1280 : 1536;
+  const bool many_rows = !BWD && a.vec_ok && a.cols <= limit && a.rows >= 16 * sms && a.rows >= (a.cols <= 1280 ? 4ll : 10ll) * a.cols;
   if (a.cols <= 512 || many_rows || a.rows > 0x7fffffff) {
-    softmax_xent_kernel<BWD><<<(int)grid, kSmThreads, 0, st>>>(a);
+    if (a.cols % 8 == 0) softmax_xent_kernel<BWD, false><<<(int)grid, kSmThreads, 0, st>>>(a);
+    else softmax_xent_kernel<BWD, true><<<(int)grid, kSmThreads, 0, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
   }
   const int chunks = (a.cols + 7) / 8;

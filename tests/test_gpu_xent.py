@@ -85,9 +85,9 @@ def test_softmax_xent_row_kernel_edges(cols, in_fmt, out_fmt, pad):
     U.assert_close_stored(dX, O.softmax_xent_bwd(xv, t, np.ones(rows), 8.0), out_fmt, 3e-6 * 8.0, "xent bwd")
 
 
-# The forward pass of many rows: a warp per row up to 1280 classes from 16 rows per SM and 4 rows per class on, and the row
+# The forward pass of many rows: a warp per row up to 1280 classes from 16 rows per SM and 4 rows per class on (16-bit: 1536 from 10 rows per class), and the row
 # kernel right beside that line.
-@pytest.mark.parametrize("rows,cols", [(2368, 513), (2367, 513), (2400, 595), (4096, 1024), (4095, 1024), (5120, 1280), (5121, 1275), (5124, 1281)])
+@pytest.mark.parametrize("rows,cols", [(2368, 513), (2367, 513), (2400, 595), (4096, 1024), (4095, 1024), (5120, 1280), (5121, 1275), (5124, 1281), (14060, 1406), (14059, 1406)])
 @pytest.mark.parametrize("in_fmt", ["bf16", "fp16", "f32"])
 def test_softmax_xent_forward_of_many_rows(rows, cols, in_fmt):
     L, synth = _mods()
