@@ -98,14 +98,15 @@ class UnitScaledEncoderLayer:
 
     @property
     def launches_per_step(self) -> int:
-        """Launches of one step with the two gradient GEMMs of a projection counted singly (without layer norms the FFN
-        block's six GEMMs go out in its grouped forms, as two or three launches, while those cover the shape)."""
+        """Library operations of one step with every GEMM of the layer itself counted (the FFN block's six GEMMs as its
+        gemm_launches, without layer norms).  The gradient GEMMs of a projection go out together: kernel_launches is the
+        number of kernels."""
         return self._launches - (6 - self.ffn.gemm_launches if self.norm is None else 0)
 
     @property
     def kernel_launches(self) -> int:
-        """Kernel launches of one step: launches_per_step less one for each projection, and with layer norms the three
-        GEMMs that end the FFN block's backward pass as one."""
+        """Kernel launches of one step while the grouped launches hold its tiles: launches_per_step less one for each
+        projection, and with layer norms the three GEMMs that end the FFN block's backward pass as one."""
         return self.launches_per_step - 2 - (2 if self.norm is not None and self.ffn.grouped else 0)
 
     def _heads(self, M, which):
@@ -113,7 +114,7 @@ class UnitScaledEncoderLayer:
         o = which * self.d
         return M[: self.slen, o:o + self.hd]
 
-    # ---- a step as calls laid out once over the layer's buffers (L.Plan), in the order of _step_each.  An entry is
+    # ---- a step as calls laid out once over the layer's buffers (L.Plan), the same ones as _step_each.  An entry is
     # (where, call): on the main stream; on the side stream once all that was issued before has finished; or (JOIN, None),
     # after which the main stream waits for the side stream.
     MAIN, SIDE, JOIN = range(3)

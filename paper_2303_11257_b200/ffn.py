@@ -19,8 +19,8 @@ mode the matmul inputs are rounded to that format instead (no loss scale, same f
 
 step() knows G when it starts.  It therefore issues the two GEMMs that end in the hidden layer (H, A and dH above) as
 one us_ffn_hidden launch, in which H stays on the SM, and the other four GEMMs as one us_linear_group launch (the
-"_any" forms of both, which take 16-bit operands and small shapes): three launches per step with the fused cast.  In
-FP8 mode self.H is then written only with keep_h = True.
+"_any" forms of both, which take 16-bit operands and small shapes): three launches per step with the fused cast.
+In FP8 mode self.H is then written only with keep_h = True (and in blocks with a dimension of at most 128).
 """
 from __future__ import annotations
 
@@ -85,18 +85,19 @@ class UnitScaledFFN:
         # step() has all four tensors to quantise at hand when it starts, so it casts them
         # with one launch; forward() / backward() on their own cast what they are given.
         self.fused_casts = True
-        # After the first GEMM, the second forward GEMM, the GELU-gradient GEMM and the first weight-gradient GEMM
-        # depend on nothing but it, and the last two GEMMs only on the GELU-gradient one.  step() issues them on
-        # three streams, so that the CTAs of one kernel fill the SMs another leaves idle in its last wave (64 or
-        # 128 tiles on 74 CTA pairs); measured 6 % faster than one stream once the power cap holds the clock.
+        # Without the grouped launch: after the first GEMM, the second forward GEMM, the GELU-gradient GEMM and the first
+        # weight-gradient GEMM depend on nothing but it, and the last two GEMMs only on the GELU-gradient one.  step()
+        # then issues them on three streams, so that the CTAs of one kernel fill the SMs another leaves idle in its last
+        # wave (64 or 128 tiles on 74 CTA pairs); measured 6 % faster than one stream once the power cap holds the clock.
+        # An encoder layer also puts one GEMM of each attention pair on a side stream while this is set.
         self.concurrent = operand == "fp8"
         self._side = None
         # The four GEMMs that remain after the GELU-gradient GEMM are independent of one another and
-        # go out as one us_linear_group launch (4 launches per step instead of 7).
+        # go out as one us_linear_group_any launch (3 launches per step with the one below, instead of 7).
         self.grouped = True
-        # G known up front: the first GEMM + GELU and the GELU-gradient GEMM are one us_ffn_hidden launch that keeps
-        # the pre-activation on the SM; keep_h = True also writes its 16-bit copy to self.H (the separate launches,
-        # 16-bit operand mode and blocks with a dimension of at most 128 always do; backward() reads it from there).
+        # G known up front: the first GEMM + GELU and the GELU-gradient GEMM are one us_ffn_hidden_any launch that keeps
+        # the pre-activation on the SM and writes its 16-bit copy to self.H as _writes_h() says (the separate launches
+        # always do; backward() reads it from there).
         self.fused_hidden = operand == "fp8" or h_dtype in (torch.bfloat16, torch.float16)
         self.keep_h = keep_h
         self._plans = {}
@@ -126,6 +127,11 @@ class UnitScaledFFN:
             call(st)
         return not call.refused                                 # the last call of a pass with gradients is its grouped launch
 
+    def _writes_h(self) -> bool:
+        """Whether step() leaves the pre-activation in self.H.  FP8 blocks write it on request.  16-bit blocks, and blocks with
+        a dimension of at most 128, have always had it there (their steps once went out as separate launches)."""
+        return self.keep_h or self.operand != "fp8" or min(self.T, self.d, self.f) <= 128
+
     def _plan_cast(self, p, src, dst):
         m = p.slot(src) if isinstance(src, str) else p.mat(src)
         return L.Call("us_cast_fp8", m, 1.0, p.mat(dst)) if self.operand == "fp8" else L.Call("us_residual_add", m, m, 0.0, p.mat(dst))
@@ -146,9 +152,8 @@ class UnitScaledFFN:
     def plan_gemms(self, p, X, G):
         """step_from_casts() as prepared calls; X, G: the skip inputs, tensors or names of inputs."""
         sc = self.sc
-        keep = self.keep_h or self.operand != "fp8" or min(self.T, self.d, self.f) <= 128
         yield L.Call("us_ffn_hidden_any", p.mat(self.Xq), p.mat(self.W1q), sc.alpha1, p.mat(self.Gq), p.mat(self.W2q), sc.beta_x2,
-                     sc.s_in, sc.alpha_g, sc.beta_g, L._TORCH_DTYPES[self.H.dtype], p.mat(self.H) if keep else None,
+                     sc.s_in, sc.alpha_g, sc.beta_g, L._TORCH_DTYPES[self.H.dtype], p.mat(self.H) if self._writes_h() else None,
                      p.mat(self.Aq), p.mat(self.dHq), self.ws.data_ptr(), self.ws.numel())
         w2, w1, x1 = self._plan_backward_entries(G)
         yield p.group([w2, w1, (L.US_OP_FWD, self.Aq, self.W2q, sc.alpha2, self.R, X, self._c), x1], self.ws)
@@ -207,9 +212,8 @@ class UnitScaledFFN:
     def stages(self, X, W1, W2, G, fused_casts: bool | None = None):
         """The launches of one pass, in order, as (name, kind, callable(stream)) triples.
 
-        kind is "cast" or "gemm".  These are the unfused launches: step() runs exactly these (seven with the casts
-        fused into one launch, ten otherwise) unless it takes the grouped forms (step_launches); forward() and
-        backward() run the ones they need."""
+        kind is "cast" or "gemm".  These are the unfused launches: seven with the casts fused into one launch, ten
+        otherwise.  step() and backward() run them where the grouped forms (step_launches) are switched off or refused."""
         sc, (c_skip, c_branch) = self.sc, self._c
         fused = self.fused_casts if fused_casts is None else fused_casts
         ep1 = L.epilogue(act=L.US_ACT_GELU, act_in_scale=sc.s_in, act_out_scale=sc.alpha_g, aux=self.H)
@@ -266,9 +270,8 @@ class UnitScaledFFN:
     def _hidden(self, stream=None):
         """H, A and dH in one launch (us_ffn_hidden) from the quantised operands."""
         sc = self.sc
-        keep = self.keep_h or self.operand != "fp8" or min(self.T, self.d, self.f) <= 128     # small blocks always keep it
         L.us_ffn_hidden_any(self.Xq, self.W1q, sc.alpha1, self.Gq, self.W2q, sc.beta_x2, sc.s_in, sc.alpha_g, sc.beta_g,
-                            self.Aq, self.dHq, self.ws, H=self.H if keep else None, h_dtype=self.H.dtype, stream=stream)
+                            self.Aq, self.dHq, self.ws, H=self.H if self._writes_h() else None, h_dtype=self.H.dtype, stream=stream)
 
     def cast_weights(self, W1, W2, stream=None):
         self._cast(W1, self.W1q, stream)
@@ -318,8 +321,9 @@ class UnitScaledFFN:
     def step(self, X, W1, W2, G, stream=None):
         """One pass of the whole path: casts, forward, backward (launches_per_step kernel launches).
 
-        With self.concurrent and no explicit stream, independent GEMMs go to two side streams that fork from
-        and join back into the current stream (this also records as parallel branches under graph capture)."""
+        With the grouped launches switched off (or refused: more tiles than their work list holds), self.concurrent set and
+        no explicit stream, independent GEMMs go to two side streams that fork from and join back into the current stream
+        (this also records as parallel branches under graph capture)."""
         if self.grouped and self.fused_casts and self.fused_hidden:
             self.grouped = self._run("step", stream, X=X, W1=W1, W2=W2, G=G)
             return self.dX, self.dW1, self.dW2
