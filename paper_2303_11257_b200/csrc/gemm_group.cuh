@@ -11,9 +11,10 @@
 //
 // Scope: FP8 or 16-bit operands (all problems of a launch the same width; either layout each), plain
 // or residual (skip) epilogue, any output dtype, up to kGroupMaxProblems problems.  CTA-pair tiles of
-// 256 x 256 (cta_group::2), or, when those would leave too many pairs idle, single-CTA tiles of 128 x 128.  Everything that differs between problems is run-time data here: tensor maps, operand
-// layouts (a K-major tile is one box of 128 rows x 128 bytes; an MN-major one has 128 / ES rows of K per
-// box, one box of 128 bytes for FP8 and two for 16-bit elements), instruction descriptor, scale, epilogue kind.
+// 256 x 256 (cta_group::2), or, when those would leave too many pairs idle, single-CTA tiles of 128 x 128.
+// Everything that differs between problems is run-time data here: tensor maps, operand layouts (a K-major
+// tile is one box of 128 rows x 128 bytes; an MN-major one has 128 / ES rows of K per box, one box of 128 bytes
+// for FP8 and two for 16-bit elements), instruction descriptor, scale, epilogue kind.
 // Measured, four separate launches -> this one, us: FP8 8192 x 1024 x 4096 122 -> 101; BF16 216 -> 199;
 // FP8 16384 x 2048 x 8192 (21 tiles per pair) 912 of kernel time, partly side by side, -> 809; FP8 256 x 128 x 512 26 -> 7.
 #pragma once
