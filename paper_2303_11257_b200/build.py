@@ -1,4 +1,4 @@
-"""Builds libunitscale.so in-tree with nvcc for sm_100a.
+"""Builds libunitscale.so (sm_100a) and its Python binding in-tree with nvcc.
 
     python -m paper_2303_11257_b200.build [--force]
 """
@@ -12,6 +12,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libunitscale.so")
+BINDING = os.path.join(HERE, "_binding.so")
 SOURCES = ["host.cu", "elementwise.cu", "softmax.cu", "layernorm.cu", "diagnostics.cu", "gemm.cu", "gemm_group.cu", "ffn_hidden.cu", "static_ws.cu", "attention.cu"]
 # (operand bytes, A MN-major, B MN-major): forward, backward-input, backward-weight for FP8 and 16-bit operands
 GEMM_PARTS = [(1, 0, 1), (1, 0, 0), (1, 1, 1), (2, 0, 1), (2, 0, 0), (2, 1, 1)]
@@ -26,10 +27,10 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(BINDING)):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [os.path.abspath(__file__)]
+    t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
+    deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS + ["binding.cpp"]] + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -38,6 +39,18 @@ def _compile(args):
     if res.returncode != 0:
         raise RuntimeError("nvcc failed:\n" + " ".join(args) + "\n" + res.stdout + res.stderr)
     return res.stderr
+
+
+def _binding_jobs(obj):
+    """Compiles and links the Python module (argument marshalling; torch's headers, and symbols of the torch that imports it)."""
+    import sysconfig
+    import torch
+    top = os.path.dirname(os.path.abspath(torch.__file__))
+    compile_ = [_nvcc(), "-std=c++17", "-O2", "-x", "c++", "-Xcompiler", f"-fPIC,-fvisibility=hidden,-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+                "-I", sysconfig.get_paths()["include"], "-I", os.path.join(top, "include"), "-c", "-o", obj, os.path.join(CSRC, "binding.cpp")]
+    link = [_nvcc(), "-shared", "-o", BINDING, obj, LIB, "-L", os.path.join(top, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lcudart",
+            "-Xlinker", "-rpath,$ORIGIN"]
+    return compile_, link
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -62,9 +75,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
         objs.append(o)
         jobs.append(common + [f"-DUS_INST_ES={es}", f"-DUS_INST_AMN={amn}", f"-DUS_INST_BMN={bmn}", "-o", o,
                               os.path.join(CSRC, "gemm_inst.cu")])
+    compile_binding, link_binding = _binding_jobs(os.path.join(objdir, "binding.o"))
     with ThreadPoolExecutor(max_workers=min(len(jobs), os.cpu_count() or 4)) as pool:
-        logs = list(pool.map(_compile, jobs))
-    _compile([_nvcc(), "-shared", "-o", LIB] + objs + ["-lcudart"])
+        logs = list(pool.map(_compile, [compile_binding] + jobs))
+    _compile([_nvcc(), "-shared", "-o", LIB, "-Xlinker", "-soname,libunitscale.so"] + objs + ["-lcudart"])
+    _compile(link_binding)
     if verbose:
         print("\n".join(logs))
     return LIB

@@ -114,10 +114,8 @@ class UnitScaledEncoderLayer:
         o = which * self.d
         return M[: self.slen, o:o + self.hd]
 
-    # ---- a step as calls laid out once over the layer's buffers (L.Plan), the same ones as _step_each.  An entry is
-    # (where, call): on the main stream; on the side stream once all that was issued before has finished; or (JOIN, None),
-    # after which the main stream waits for the side stream.
-    MAIN, SIDE, JOIN = range(3)
+    # ---- a step as calls laid out once over the layer's buffers (L.Plan), the same ones as _step_each, as (where, call) pairs
+    MAIN, SIDE, JOIN = L.Plan.MAIN, L.Plan.SIDE, L.Plan.JOIN
 
     def _owned(self):
         own = (self.Xq, self.Wqkv_q, self.Wo_q, self.QKV, self.P, self.Cq, self.R1, self.g1q, self.dC, self.dS, self.dQKVq, self.dQKV,
@@ -203,28 +201,15 @@ class UnitScaledEncoderLayer:
         p = self._plan
         if p is None or not p.same(owned, state):
             p = self._plan = L.Plan(owned, state)
-        for name, t in inputs.items():
-            p.put(name, t)
         if not (stream is None and self.ffn.concurrent):
-            st = L._stream(stream)
-            for where, call in p.calls(self._lay_out):
-                if call is not None:
-                    call(st)
+            p.issue(self._lay_out, inputs, L._stream(stream))
             return
+        cur = torch.cuda.current_stream()
         if self._events is None:
             self._events = torch.cuda.Event(), torch.cuda.Event()
-        (fork, join), cur, side = self._events, torch.cuda.current_stream(), self.ffn._side_streams()[0]
-        st, side_st = cur.cuda_stream, side.cuda_stream
-        for where, call in p.calls(self._lay_out):
-            if where == self.MAIN:
-                call(st)
-            elif where == self.SIDE:
-                fork.record(cur)
-                side.wait_event(fork)
-                call(side_st)
-            else:
-                join.record(side)
-                cur.wait_event(join)
+            for e in self._events:
+                e.record(cur)                                       # an event has a handle once it has been recorded
+        p.issue(self._lay_out, inputs, cur.cuda_stream, (self.ffn._side_streams()[0], *self._events))
 
     def step(self, X, Wqkv, Wo, W1, W2, G, stream=None, ln=None):
         """One forward + backward pass.  G is the gradient of the layer output; with norm = "post",

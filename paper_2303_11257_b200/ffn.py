@@ -120,12 +120,8 @@ class UnitScaledFFN:
         p = self._plans.get(kind)
         if p is None or not p.same(owned, state):
             p = self._plans[kind] = L.Plan(owned, state)
-        for name, t in inputs.items():
-            p.put(name, t)
-        st = L._stream(stream)
-        for call in p.calls(getattr(self, "_plan_" + kind)):
-            call(st)
-        return not call.refused                                 # the last call of a pass with gradients is its grouped launch
+        # the last call of a pass with gradients is its grouped launch
+        return not p.issue(getattr(self, "_plan_" + kind), inputs, L._stream(stream)).refused
 
     def _writes_h(self) -> bool:
         """Whether step() leaves the pre-activation in self.H.  FP8 blocks write it on request.  16-bit blocks, and blocks with

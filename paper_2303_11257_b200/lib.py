@@ -152,7 +152,13 @@ def _load() -> C.CDLL:
     return lib
 
 
-_lib = _load()
+_lib = _library = _load()
+from . import _binding                                        # noqa: E402  (links the library that has just been loaded)
+
+
+def _entry(name: str):
+    """The function of that name: through the binding, which takes tensors as they are."""
+    return _binding.calls[name] if _lib is _library else getattr(_lib, name)
 
 
 def raw() -> C.CDLL:
@@ -189,18 +195,20 @@ def _stream(stream) -> int:
 
 
 class Call:
-    """A library call whose arguments are laid out once: calling it costs the C call and little else.  It points into
-    tensors that the caller keeps (a block's own buffers); descriptions that change from call to call -- the tensors a
-    user passes to a step -- are written into its us_mat slots before each call (Plan.put).  instead: (statuses, fn); a
-    call that the library refuses with one of those statuses, having launched nothing, issues fn(stream) in its place."""
+    """A library call whose arguments are laid out once.  It points into tensors that the caller keeps (a block's own
+    buffers); descriptions that change from call to call -- the tensors a user passes to a step -- are written into its us_mat
+    slots before each call.  instead: (statuses, fn); a call that the library refuses with one of those statuses, having
+    launched nothing, issues fn(stream) in its place."""
     __slots__ = ("name", "fn", "args", "keep", "instead", "refused")
 
     def __init__(self, name, *args, instead=((), None)):
-        self.name, self.fn, self.keep, self.instead, self.refused = name, getattr(_lib, name), args, instead, False
-        self.args = tuple(C.byref(a) if isinstance(a, C.Structure) else a for a in args)
+        self.name, self.fn, self.keep, self.instead, self.refused = name, _entry(name), args, instead, False
+        self.args = args if _lib is _library else tuple(C.byref(a) if isinstance(a, C.Structure) else a for a in args)
 
     def __call__(self, stream: int) -> None:
-        status = self.fn(*self.args, stream)
+        self.finish(self.fn(*self.args, stream), stream)
+
+    def finish(self, status: int, stream: int) -> None:
         if status != US_OK:
             if status not in self.instead[0]:
                 raise UnitScaleError(self.name, status)
@@ -210,15 +218,20 @@ class Call:
 
 class Plan:
     """The calls of one pass over an object's own buffers, and the slots its inputs go to.  `owned` are those buffers,
-    `state` every other value the calls were laid out for: same() says whether both are still what they were.
-    calls(lay_out): lay_out(plan) yields the calls in order; the first pass issues each as soon as it is laid out."""
+    `state` every other value the calls were laid out for: same() says whether both are still what they were.  issue() makes
+    a pass: lay_out(plan) yields the calls in order, or (where, call) pairs (see MAIN); the first pass issues each as soon as
+    it is laid out, later ones go out as one call of the binding."""
+
+    # where a call goes: the main stream; the side stream, once all that was issued before has finished; or, without a call,
+    # the main stream waits for the side stream
+    MAIN, SIDE, JOIN = range(3)
 
     def __init__(self, owned, state):
-        self.owned, self.state, self.ptrs = owned, state, [t.data_ptr() for t in owned]
-        self.slots, self.inputs, self.done, self.mats = {}, {}, None, {}
+        self.owned, self.state, self.ptrs = owned, state, tuple(t.data_ptr() for t in owned)
+        self.slots, self.inputs, self.done, self.mats, self.program = {}, {}, None, {}, None
 
     def same(self, owned, state) -> bool:
-        return self.state == state and all(map(operator.is_, owned, self.owned)) and [t.data_ptr() for t in owned] == self.ptrs
+        return self.state == state and _binding.unchanged(owned, self.owned, self.ptrs)
 
     def mat(self, t: torch.Tensor) -> us_mat:
         """mat(t), made once for all calls of the pass that is being laid out."""
@@ -250,6 +263,48 @@ class Plan:
             yield c
         self.done, self.mats = made, {}                         # a pass that ended early is laid out again
 
+    def issue(self, lay_out, inputs: dict, main: int, side=None) -> Call:
+        """One pass with these inputs (tensors by name) on the stream `main`; side: (stream, fork event, join event) for the
+        calls that go to the side stream, which otherwise go to the main one.  Returns the pass's last call."""
+        if self.done is not None and _lib is _library:
+            if self.program is None:
+                self._compile(tuple(inputs))
+            names, program = self.program
+            values = tuple(inputs.values()) if tuple(inputs) == names else tuple(inputs[n] for n in names)
+            handles = (main, side[0].cuda_stream, side[1].cuda_event, side[2].cuda_event) if side else (main, 0, 0, 0)
+            r = _binding.run(program, 0, values, *handles)
+            while r >= 0:                                       # a call that was refused: what it has instead, then the rest
+                where, call = self._steps[r >> 8]
+                if call is None:
+                    raise UnitScaleError("join", r & 255)
+                call.finish(r & 255, handles[1] if where == self.SIDE and side else main)
+                r = _binding.run(program, (r >> 8) + 1, values, *handles)
+            return self._steps[-1][1]
+        for name, t in inputs.items():
+            self.put(name, t)
+        call = None
+        for entry in self.calls(lay_out):
+            where, this = entry if isinstance(entry, tuple) else (self.MAIN, entry)
+            if where == self.JOIN:
+                if side:
+                    side[2].record(side[0])
+                    torch.cuda.current_stream().wait_event(side[2])
+                continue
+            call = this
+            if where == self.SIDE and side:
+                side[1].record(torch.cuda.current_stream())
+                side[0].wait_event(side[1])
+                call(side[0].cuda_stream)
+            else:
+                call(main)
+        return call
+
+    def _compile(self, names):
+        self._steps = [e if isinstance(e, tuple) else (self.MAIN, e) for e in self.done]
+        steps = [(w, c if c is None else _binding.prepare(c.name, c.keep)) for w, c in self._steps]
+        slots = [(i, m) for i, n in enumerate(names) for m in self.slots.get(n, ())]
+        self.program = names, _binding.program(steps, slots)
+
     def cast_multi(self, srcs, dsts, padded=False):
         """us_cast_multi at scale 1; an entry of srcs is a tensor or the name of an input.  padded: rows that it does not
         take (padded or unaligned ones) go out as one us_residual_add per tensor, for 16-bit destinations."""
@@ -264,7 +319,7 @@ class Plan:
 
         def each(stream):
             for s, d in zip(sm, dm):
-                _check("us_residual_add", _lib.us_residual_add(C.byref(s), C.byref(s), 0.0, C.byref(d), stream))
+                _check("us_residual_add", _entry("us_residual_add")(s, s, 0.0, d, stream))
 
         return Call("us_cast_multi", n, sm, (C.c_float * n)(*[1.0] * n), dm,
                     instead=((US_ERR_UNSUPPORTED, US_ERR_ALIGNMENT) if padded else (), each))
@@ -335,10 +390,10 @@ def us_workspace_status(ws: torch.Tensor, stream=None) -> int:
 
 
 def _linear(name, a, b, scale, ep, out, ws, stream):
-    fn = getattr(_lib, name)
-    epp = C.byref(ep) if ep is not None else None
-    _check(name, fn(C.byref(mat(a)), C.byref(mat(b)), scale, epp, C.byref(mat(out)),
-                    ws.data_ptr(), ws.numel() * ws.element_size(), _stream(stream)))
+    fn = _entry(name)
+    epp = ep if ep is not None else None
+    _check(name, fn(a, b, scale, epp, out,
+                    ws, ws, _stream(stream)))
     return out
 
 
@@ -369,7 +424,7 @@ def linear_call(op: int, a, b, scale: float, out, ep=None) -> us_linear_call:
 def us_linear_group(calls, ws, stream=None, name="us_linear_group"):
     """Several independent linear ops in one launch (see the header for what this form covers)."""
     arr = (us_linear_call * len(calls))(*calls)
-    _check(name, getattr(_lib, name)(len(calls), arr, ws.data_ptr(), ws.numel() * ws.element_size(), _stream(stream)))
+    _check(name, _entry(name)(len(calls), arr, ws, ws, _stream(stream)))
 
 
 def us_linear_group_any(calls, ws, stream=None):
@@ -381,8 +436,7 @@ def linear_each(calls, ws, stream=None):
     """The same ops as single launches, in order (for a group with more tiles than the grouped form's work list holds)."""
     for c in calls:
         name = ("us_linear_fwd", "us_linear_bwd_x", "us_linear_bwd_w")[c.op]
-        _check(name, getattr(_lib, name)(C.byref(c.a), C.byref(c.b), c.scale, C.byref(c.ep), C.byref(c.out), ws.data_ptr(),
-                                         ws.numel() * ws.element_size(), _stream(stream)))
+        _check(name, _entry(name)(c.a, c.b, c.scale, c.ep, c.out, ws, ws, _stream(stream)))
 
 
 def linear_together(calls, ws, stream=None):
@@ -404,9 +458,9 @@ def batch(count, a_stride, b_stride, out_stride) -> us_batch:
 
 
 def _linear_batched(name, a, b, scale, out, bt, ws, stream):
-    fn = getattr(_lib, name)
-    _check(name, fn(C.byref(mat(a)), C.byref(mat(b)), scale, C.byref(mat(out)), C.byref(bt),
-                    ws.data_ptr(), ws.numel() * ws.element_size(), _stream(stream)))
+    fn = _entry(name)
+    _check(name, fn(a, b, scale, out, bt,
+                    ws, ws, _stream(stream)))
     return out
 
 
@@ -434,11 +488,7 @@ def attention_batch(count, q_stride, k_stride, v_stride, c_stride, p_stride=(0, 
 
 def us_attention_fwd(Q, K, V, alpha_scores, softmax_scale, alpha_context, Cx, P, bt, ws, stream=None):
     """Fused scaled dot-product attention forward; P may be None (weights not stored)."""
-    pp = C.byref(mat(P)) if P is not None else None
-    _check("us_attention_fwd",
-           _lib.us_attention_fwd(C.byref(mat(Q)), C.byref(mat(K)), C.byref(mat(V)), alpha_scores, softmax_scale,
-                                 alpha_context, C.byref(mat(Cx)), pp, C.byref(bt), ws.data_ptr(),
-                                 ws.numel() * ws.element_size(), _stream(stream)))
+    _check("us_attention_fwd", _entry("us_attention_fwd")(Q, K, V, alpha_scores, softmax_scale, alpha_context, Cx, P, bt, ws, ws, _stream(stream)))
     return Cx
 
 
@@ -453,10 +503,7 @@ def attention_bwd_batch(count, dc_stride, p_stride, k_stride, v_stride, ds_strid
 
 def us_attention_bwd(dC, P, K, V, beta_p, softmax_alpha, softmax_beta, beta_q, dS, dQ, bt, ws, stream=None):
     """Attention backward down to the queries: dS (for the dK matmul) and dQ from dC, the stored P, K and V."""
-    _check("us_attention_bwd",
-           _lib.us_attention_bwd(C.byref(mat(dC)), C.byref(mat(P)), C.byref(mat(K)), C.byref(mat(V)), beta_p, softmax_alpha,
-                                 softmax_beta, beta_q, C.byref(mat(dS)), C.byref(mat(dQ)), C.byref(bt), ws.data_ptr(),
-                                 ws.numel() * ws.element_size(), _stream(stream)))
+    _check("us_attention_bwd", _entry("us_attention_bwd")(dC, P, K, V, beta_p, softmax_alpha, softmax_beta, beta_q, dS, dQ, bt, ws, ws, _stream(stream)))
     return dQ
 
 
@@ -491,11 +538,8 @@ def us_ffn_hidden(X, W1, alpha, G, W2, beta_x, act_in_scale, act_out_scale, grad
                   H=None, h_dtype=torch.bfloat16, stream=None, name="us_ffn_hidden"):
     """Hidden layer of the FFN block, forward and backward, in one launch (see the header): A and dH are written,
     H (optional) receives the pre-activation rounded to h_dtype."""
-    hp = C.byref(mat(H)) if H is not None else None
-    _check(name,
-           getattr(_lib, name)(C.byref(mat(X)), C.byref(mat(W1)), alpha, C.byref(mat(G)), C.byref(mat(W2)), beta_x,
-                               act_in_scale, act_out_scale, grad_out_scale, _TORCH_DTYPES[h_dtype], hp, C.byref(mat(A)),
-                               C.byref(mat(dH)), ws.data_ptr(), ws.numel() * ws.element_size(), _stream(stream)))
+    _check(name, _entry(name)(X, W1, alpha, G, W2, beta_x, act_in_scale, act_out_scale, grad_out_scale, _TORCH_DTYPES[h_dtype], H, A, dH,
+                              ws, ws, _stream(stream)))
     return A, dH
 
 
@@ -518,23 +562,22 @@ def us_workspace_status_ptr(ws_ptr: int, stream=None) -> int:
 
 
 def us_gelu_fwd(H, s_in, alpha, A, stream=None):
-    _check("us_gelu_fwd", _lib.us_gelu_fwd(C.byref(mat(H)), s_in, alpha, C.byref(mat(A)), _stream(stream)))
+    _check("us_gelu_fwd", _entry("us_gelu_fwd")(H, s_in, alpha, A, _stream(stream)))
     return A
 
 
 def us_gelu_bwd(H, dA, s_in, beta, dH, stream=None):
-    _check("us_gelu_bwd", _lib.us_gelu_bwd(C.byref(mat(H)), C.byref(mat(dA)), s_in, beta, C.byref(mat(dH)), _stream(stream)))
+    _check("us_gelu_bwd", _entry("us_gelu_bwd")(H, dA, s_in, beta, dH, _stream(stream)))
     return dH
 
 
 def us_activation_fwd(fn, H, s_in, alpha, A, stream=None):
-    _check("us_activation_fwd", _lib.us_activation_fwd(FN_BY_NAME.get(fn, fn), C.byref(mat(H)), s_in, alpha, C.byref(mat(A)), _stream(stream)))
+    _check("us_activation_fwd", _entry("us_activation_fwd")(FN_BY_NAME.get(fn, fn), H, s_in, alpha, A, _stream(stream)))
     return A
 
 
 def us_activation_bwd(fn, H, dA, s_in, beta, dH, stream=None):
-    _check("us_activation_bwd", _lib.us_activation_bwd(FN_BY_NAME.get(fn, fn), C.byref(mat(H)), C.byref(mat(dA)), s_in, beta,
-                                                       C.byref(mat(dH)), _stream(stream)))
+    _check("us_activation_bwd", _entry("us_activation_bwd")(FN_BY_NAME.get(fn, fn), H, dA, s_in, beta, dH, _stream(stream)))
     return dH
 
 
@@ -545,12 +588,12 @@ def us_scales_activation(fn, constrained: bool = False):
 
 
 def us_residual_add(skip, branch, tau, out, stream=None):
-    _check("us_residual_add", _lib.us_residual_add(C.byref(mat(skip)), C.byref(mat(branch)), tau, C.byref(mat(out)), _stream(stream)))
+    _check("us_residual_add", _entry("us_residual_add")(skip, branch, tau, out, _stream(stream)))
     return out
 
 
 def us_cast_fp8(src, scale, dst, stream=None):
-    _check("us_cast_fp8", _lib.us_cast_fp8(C.byref(mat(src)), scale, C.byref(mat(dst)), _stream(stream)))
+    _check("us_cast_fp8", _entry("us_cast_fp8")(src, scale, dst, _stream(stream)))
     return dst
 
 
@@ -558,7 +601,7 @@ def us_weighted_add(srcs, gammas, alpha, out, stream=None):
     n = len(srcs)
     sm = (us_mat * n)(*[mat(t) for t in srcs])
     gm = (C.c_float * n)(*[float(g) for g in gammas])
-    _check("us_weighted_add", _lib.us_weighted_add(n, sm, gm, alpha, C.byref(mat(out)), _stream(stream)))
+    _check("us_weighted_add", _entry("us_weighted_add")(n, sm, gm, alpha, out, _stream(stream)))
     return out
 
 
@@ -568,7 +611,7 @@ def us_cast_fp8_multi(srcs, scales, dsts, stream=None, name="us_cast_fp8_multi")
     sm = (us_mat * n)(*[mat(t) for t in srcs])
     dm = (us_mat * n)(*[mat(t) for t in dsts])
     sc = (C.c_float * n)(*[float(x) for x in scales])
-    _check(name, getattr(_lib, name)(n, sm, sc, dm, _stream(stream)))
+    _check(name, _entry(name)(n, sm, sc, dm, _stream(stream)))
     return dsts
 
 
@@ -578,27 +621,26 @@ def us_cast_multi(srcs, scales, dsts, stream=None):
 
 
 def us_softmax_fwd(S, alpha, P, stream=None):
-    _check("us_softmax_fwd", _lib.us_softmax_fwd(C.byref(mat(S)), alpha, C.byref(mat(P)), _stream(stream)))
+    _check("us_softmax_fwd", _entry("us_softmax_fwd")(S, alpha, P, _stream(stream)))
     return P
 
 
 def us_softmax_bwd(P, dP, alpha, beta, dS, stream=None):
-    _check("us_softmax_bwd", _lib.us_softmax_bwd(C.byref(mat(P)), C.byref(mat(dP)), alpha, beta, C.byref(mat(dS)), _stream(stream)))
+    _check("us_softmax_bwd", _entry("us_softmax_bwd")(P, dP, alpha, beta, dS, _stream(stream)))
     return dS
 
 
 def us_softmax_xent_fwd(X, targets, out, stream=None):
     """targets: int32 CUDA tensor [rows]; out: float32 CUDA tensor [rows]."""
     assert targets.dtype == torch.int32 and out.dtype == torch.float32 and targets.is_contiguous() and out.is_contiguous()
-    _check("us_softmax_xent_fwd", _lib.us_softmax_xent_fwd(C.byref(mat(X)), targets.data_ptr(), out.data_ptr(), _stream(stream)))
+    _check("us_softmax_xent_fwd", _entry("us_softmax_xent_fwd")(X, targets.data_ptr(), out.data_ptr(), _stream(stream)))
     return out
 
 
 def us_softmax_xent_bwd(X, targets, g, beta, dX, stream=None):
     """g: float32 CUDA tensor [rows] or None (ones)."""
     assert targets.dtype == torch.int32 and targets.is_contiguous() and (g is None or (g.dtype == torch.float32 and g.is_contiguous()))
-    _check("us_softmax_xent_bwd", _lib.us_softmax_xent_bwd(C.byref(mat(X)), targets.data_ptr(), g.data_ptr() if g is not None else None,
-                                                           beta, C.byref(mat(dX)), _stream(stream)))
+    _check("us_softmax_xent_bwd", _entry("us_softmax_xent_bwd")(X, targets.data_ptr(), g.data_ptr() if g is not None else None, beta, dX, _stream(stream)))
     return dX
 
 
@@ -620,8 +662,7 @@ def _vec(t: torch.Tensor) -> us_mat:
 
 
 def us_layer_norm_fwd(X, w, c, eps, Y, stream=None):
-    _check("us_layer_norm_fwd", _lib.us_layer_norm_fwd(C.byref(mat(X)), C.byref(_vec(w)), C.byref(_vec(c)), eps,
-                                                       C.byref(mat(Y)), _stream(stream)))
+    _check("us_layer_norm_fwd", _entry("us_layer_norm_fwd")(X, w.view(1, -1), c.view(1, -1), eps, Y, _stream(stream)))
     return Y
 
 
@@ -631,9 +672,9 @@ def us_layer_norm_bwd_workspace_bytes(rows: int, cols: int) -> int:
 
 def us_layer_norm_bwd(X, w, G, eps, beta_x, beta_wc, dX, dw, dc, ws, stream=None):
     """ws: a uint8 CUDA tensor of at least us_layer_norm_bwd_workspace_bytes(rows, cols) bytes."""
-    _check("us_layer_norm_bwd", _lib.us_layer_norm_bwd(
-        C.byref(mat(X)), C.byref(_vec(w)), C.byref(mat(G)), eps, beta_x, beta_wc, C.byref(mat(dX)), C.byref(_vec(dw)),
-        C.byref(_vec(dc)), ws.data_ptr(), ws.numel() * ws.element_size(), _stream(stream)))
+    _check("us_layer_norm_bwd", _entry("us_layer_norm_bwd")(
+        X, w.view(1, -1), G, eps, beta_x, beta_wc, dX, dw.view(1, -1),
+        dc.view(1, -1), ws, ws, _stream(stream)))
     return dX, dw, dc
 
 
