@@ -97,3 +97,22 @@ def test_softmax_xent_forward_of_many_rows(rows, cols, in_fmt):
     L.us_softmax_xent_fwd(U.to_device(x, in_fmt, (cols + 15) // 16 * 16), torch.from_numpy(t).cuda(), out)
     ref = O.softmax_xent_fwd(U.values_of(x, in_fmt), t)
     assert np.abs(out.cpu().numpy() - ref).max() <= 4e-6 * (1 + np.abs(ref).max())
+
+
+@pytest.mark.parametrize("rows,cols", [(2400, 4104), (2400, 8192), (1300, 8201), (1000, 16384)])
+@pytest.mark.parametrize("in_fmt,out_fmt", [("bf16", "e5m2"), ("fp16", "bf16")])
+def test_softmax_xent_backward_of_rows_that_a_cta_walks(rows, cols, in_fmt, out_fmt):
+    """16-bit rows of 4097 to 16384 classes: CTAs that walk four or more rows through their ring of three, at both CTA sizes, with
+    targets outside the row and a gradient per row; every 37th row and the last ones against the oracle."""
+    L, synth = _mods()
+    ld = (cols + 15) // 16 * 16
+    x, g = synth.normal(35, cols, (rows, cols), 2.0), synth.normal(35, 1, (1, rows))[0]
+    t = (np.arange(rows) * 7919 % cols).astype(np.int32)
+    t[37], t[74] = -1, cols
+    Xt, xv, dX = U.to_device(x, in_fmt, ld), U.values_of(x, in_fmt), U.empty(rows, cols, out_fmt, ld)
+    L.us_softmax_xent_bwd(Xt, torch.from_numpy(t).cuda(), torch.from_numpy(g).cuda(), 8.0, dX)
+    pick = np.unique(np.concatenate([np.arange(0, rows, 37), np.arange(rows - 5, rows)]))
+    ref = O.softmax_xent_bwd(xv[pick], np.clip(t[pick], 0, cols - 1), g[pick].astype(np.float64), 8.0)
+    for i in np.flatnonzero((t[pick] < 0) | (t[pick] >= cols)):       # no one-hot term there
+        ref[i, np.clip(t[pick[i]], 0, cols - 1)] -= 8.0 * np.float64(g[pick[i]])
+    U.assert_close_stored(dX[torch.from_numpy(pick).cuda()], ref, out_fmt, 3e-6 * 8.0 * np.abs(g).max(), "xent bwd")
