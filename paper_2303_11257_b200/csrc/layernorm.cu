@@ -244,18 +244,18 @@ __device__ __forceinline__ void stats_regs(const float (&x)[NCH][8], int lane, i
 }
 
 template <int NCH>
-__global__ void __launch_bounds__(kLnThreads, 2) ln_fwd16_kernel(const LnArgs a) {
+__global__ void __launch_bounds__(kLnThreads, NCH <= 4 ? 3 : 2) ln_fwd16_kernel(const LnArgs a) {
   extern __shared__ __align__(16) float ln_smem[];                         // w[cols], c[cols] as float32
   float* w_s = ln_smem;
   float* c_s = ln_smem + a.cols;
   const int zero = ptx::grid_wait_previous();
-  for (int j = threadIdx.x + zero; j < a.cols; j += blockDim.x) { w_s[j] = load_one(a.w, a.w_dt, j); c_s[j] = load_one(a.c, a.c_dt, j); }
-  __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int64_t stride = (int64_t)gridDim.x * nw;
   int64_t row = (int64_t)blockIdx.x * nw + warp + zero;
   uint4 cur[NCH], nxt[NCH];
-  if (row < a.rows) load_row16<NCH>(a.x, row * a.x_ld, lane, a.cols, cur);
+  if (row < a.rows) load_row16<NCH>(a.x, row * a.x_ld, lane, a.cols, cur);   // the first row and w, c are on their way together
+  for (int j = threadIdx.x; j < a.cols; j += blockDim.x) { w_s[j] = load_one(a.w, a.w_dt, j + zero); c_s[j] = load_one(a.c, a.c_dt, j + zero); }
+  __syncthreads();
   for (; row < a.rows; row += stride) {
     if (row + stride < a.rows) load_row16<NCH>(a.x, (row + stride) * a.x_ld, lane, a.cols, nxt);
     float x[NCH][8];
@@ -606,7 +606,8 @@ extern "C" us_status us_layer_norm_fwd(const us_mat* X, const us_mat* w, const u
   if (a.vec_ok && (a.x_dt == US_BF16 || a.x_dt == US_F16) && nch <= 8) {
     const int sms = host::sm_count();
     if (sms <= 0) return US_ERR_CUDA;
-    const int pgrid = grid < 2 * sms ? grid : 2 * sms;       // two resident CTAs per SM, warps walk the rows
+    // resident CTAs, warps walk the rows; three an SM where their registers fit (8192 x 1024 BF16: 9.7 -> 9.2 us)
+    const int most = (nch <= 4 ? 3 : 2) * sms, pgrid = grid < most ? grid : most;
     const size_t smem = (size_t)2 * a.cols * sizeof(float);
     if (nch <= 1) return host::launch(ln_fwd16_kernel<1>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
     if (nch <= 2) return host::launch(ln_fwd16_kernel<2>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
