@@ -400,6 +400,29 @@ us_status us_attention_bwd(const us_mat* dC, const us_mat* P, const us_mat* K, c
                            float softmax_alpha, float softmax_beta, float beta_q, const us_mat* dS, const us_mat* dQ,
                            const us_attention_bwd_batch* batch, void* ws, size_t ws_bytes, void* stream);
 
+/*
+ * us_attention_bwd_all: the whole backward pass of scaled dot-product attention, per problem
+ *
+ *   dP = beta_p dC V^T,   dS = softmax_beta * p (dP - sum_j p_j dP_j),   p = P / softmax_alpha      (dP is not rounded)
+ *   dQ = beta_q dS K,     dK = beta_k dS^T Q,   dV = beta_v P^T dC     (from the rounded dS and the stored P)
+ *
+ * as ONE launch: what us_attention_bwd and two us_linear_bwd_w_batched calls compute, with P read and dS written once.  Row sums
+ * and the products of dQ are float32 sums in an order of their own (fixed: repeated calls give identical results).
+ * dC, Q, dQ [s_q x 64]; K, V, dK, dV [s_k x 64]; P, dS [s_q x s_k], s_k <= 512.  dS may be NULL (not stored).
+ * Formats as for us_attention_bwd (dC, P, Q, K, V and dS all BF16, all F16, or E5M2 gradients with E4M3 activations);
+ * dQ, dK, dV any us_dtype.  At least one query and one key (US_ERR_UNSUPPORTED otherwise); limits, alignment, strides,
+ * workspace and errors as for us_attention_bwd.
+ */
+typedef struct {
+  int64_t count[2];
+  int64_t dc_stride[2], p_stride[2], q_stride[2], k_stride[2], v_stride[2], ds_stride[2], dq_stride[2], dk_stride[2], dv_stride[2];
+} us_attention_bwd_all_batch;
+
+us_status us_attention_bwd_all(const us_mat* dC, const us_mat* P, const us_mat* Q, const us_mat* K, const us_mat* V, float beta_p,
+                               float softmax_alpha, float softmax_beta, float beta_q, float beta_k, float beta_v, const us_mat* dS,
+                               const us_mat* dQ, const us_mat* dK, const us_mat* dV, const us_attention_bwd_all_batch* batch,
+                               void* ws, size_t ws_bytes, void* stream);
+
 /* ------------------------------------------------------------ scaled softmax
  *
  * Row-wise scaled softmax and its gradient (table "Table of unit scaling factors", row softmax:

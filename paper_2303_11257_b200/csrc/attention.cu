@@ -33,6 +33,7 @@
 #include <cstdint>
 
 #include "../../include/unitscale.h"
+#include "attention_host.h"
 #include "common.cuh"
 #include "gemm_kernel.cuh"
 #include "host.h"
@@ -41,8 +42,7 @@
 namespace us {
 namespace {
 
-constexpr int kAttnD = 64;                 // head width
-constexpr int kAttnMaxKeys = 512;          // 128 x 512 float32 scores fill the 512 TMEM columns
+static_assert(kAttnMaxKeys == 512, "128 x 512 float32 scores fill the 512 TMEM columns");
 constexpr int kSoftmaxWarps = 16, kParts = kSoftmaxWarps / 4;   // warps per TMEM lane quarter
 constexpr int kAttnThreads = 64 + 32 * kSoftmaxWarps;   // warp 0: TMA + MMA issue; warp 1: TMEM owner; the rest: softmax
 constexpr uint32_t kQBytes = 128 * 128;    // 128 rows x 64 x 2 bytes
@@ -731,28 +731,6 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_const
   if (warp == 1) { ptx::tc_fence_after_sync(); ptx::tmem_dealloc(tmem, 512); }
 }
 
-// 4-d map (column, row, inner problem index, outer problem index) over elements of es bytes (2, or 1 for FP8); box of 128
-// bytes (128-byte swizzle) x box_rows rows of one problem; columns of a box beyond the matrix read as zeros.
-static bool attn_tmap(CUtensorMap* tm, const us_mat* m, const int64_t* stride, const int64_t* count, int box_rows, int es = 2) {
-  host::EncodeTiledFn fn = host::encode_tiled_fn();
-  if (!fn) return false;
-  cuuint64_t dims[4] = {(cuuint64_t)m->cols, (cuuint64_t)m->rows, (cuuint64_t)count[1], (cuuint64_t)count[0]};
-  // a dimension of extent 1 still needs a valid (multiple of 16 bytes) stride
-  const cuuint64_t s1 = count[1] > 1 ? (cuuint64_t)stride[1] * es : 16, s0 = count[0] > 1 ? (cuuint64_t)stride[0] * es : 16;
-  cuuint64_t strides[3] = {(cuuint64_t)m->ld * es, s1, s0};
-  cuuint32_t box[4] = {(cuuint32_t)(128 / es), (cuuint32_t)box_rows, 1, 1};
-  cuuint32_t estr[4] = {1, 1, 1, 1};
-  return fn(tm, es == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_UINT16, 4, m->ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-static bool ok16(const us_mat* m, const int64_t* stride, const int64_t* count, int es) {
-  if (reinterpret_cast<uintptr_t>(m->ptr) % 16 || (m->ld * es) % 16) return false;
-  for (int i = 0; i < 2; ++i)
-    if (count[i] > 1 && (stride[i] * es) % 16) return false;
-  return true;
-}
-
 }  // namespace
 }  // namespace us
 
@@ -788,8 +766,8 @@ extern "C" us_status us_attention_fwd(const us_mat* Q, const us_mat* K, const us
   if (!ws || ws_bytes < us_workspace_bytes()) return US_ERR_WORKSPACE;
   if (s_q == 0 || s_k == 0) return s_k == 0 && s_q > 0 ? US_ERR_INVALID_ARG : US_OK;   // a softmax over no keys is undefined
   const int c_es = (int)dtype_size(C->dtype);
-  if (!ok16(Q, batch->q_stride, cnt, es) || !ok16(K, batch->k_stride, cnt, es) || !ok16(V, batch->v_stride, cnt, es) ||
-      !ok16(C, batch->c_stride, cnt, c_es) || (P && !ok16(P, batch->p_stride, cnt, es)))
+  if (!attn_aligned(Q, batch->q_stride, cnt, es) || !attn_aligned(K, batch->k_stride, cnt, es) || !attn_aligned(V, batch->v_stride, cnt, es) ||
+      !attn_aligned(C, batch->c_stride, cnt, c_es) || (P && !attn_aligned(P, batch->p_stride, cnt, es)))
     return US_ERR_ALIGNMENT;
 
   CUtensorMap tq, tk, tv, tp;
@@ -860,8 +838,8 @@ extern "C" us_status us_attention_bwd(const us_mat* dC, const us_mat* P, const u
   if (s_q == 0 || s_k == 0) return US_OK;              // no queries: nothing to do; no keys: dS is empty and dQ is not written
   const int q_es = (int)dtype_size(dQ->dtype);
   for (int i = 0; i < 5; ++i)
-    if (!ok16(all[i], strides[i], cnt, es)) return US_ERR_ALIGNMENT;
-  if (!ok16(dQ, batch->dq_stride, cnt, q_es)) return US_ERR_ALIGNMENT;
+    if (!attn_aligned(all[i], strides[i], cnt, es)) return US_ERR_ALIGNMENT;
+  if (!attn_aligned(dQ, batch->dq_stride, cnt, q_es)) return US_ERR_ALIGNMENT;
 
   CUtensorMap tdc, tv, tk, tp, tds;
   if (!attn_tmap(&tdc, dC, batch->dc_stride, cnt, 128, es) || !attn_tmap(&tv, V, batch->v_stride, cnt, 256, es) ||

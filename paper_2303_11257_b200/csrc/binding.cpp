@@ -182,7 +182,7 @@ Prepared* keep(PyObject* const* o, Py_ssize_t n) { return decltype(entry_of(F)):
 const Known kKnown[] = {
     US_CALL(us_linear_fwd), US_CALL(us_linear_bwd_x), US_CALL(us_linear_bwd_w), US_CALL(us_linear_fwd_batched), US_CALL(us_linear_bwd_x_batched),
     US_CALL(us_linear_bwd_w_batched), US_CALL(us_linear_group), US_CALL(us_linear_group_any), US_CALL(us_ffn_hidden), US_CALL(us_ffn_hidden_any),
-    US_CALL(us_attention_fwd), US_CALL(us_attention_bwd), US_CALL(us_cast_fp8), US_CALL(us_cast_fp8_multi),
+    US_CALL(us_attention_fwd), US_CALL(us_attention_bwd), US_CALL(us_attention_bwd_all), US_CALL(us_cast_fp8), US_CALL(us_cast_fp8_multi),
     US_CALL(us_cast_multi), US_CALL(us_residual_add), US_CALL(us_gelu_fwd), US_CALL(us_gelu_bwd), US_CALL(us_activation_fwd),
     US_CALL(us_activation_bwd), US_CALL(us_weighted_add), US_CALL(us_softmax_fwd), US_CALL(us_softmax_bwd), US_CALL(us_softmax_xent_fwd),
     US_CALL(us_softmax_xent_bwd), US_CALL(us_layer_norm_fwd), US_CALL(us_layer_norm_bwd),

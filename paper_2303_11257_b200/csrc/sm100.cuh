@@ -163,6 +163,11 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+__device__ __forceinline__ uint32_t cluster_nctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -177,6 +182,24 @@ __device__ __forceinline__ uint32_t in_even_cta(uint32_t addr) {
 // Arrive on an mbarrier anywhere in the cluster (address in the shared::cluster window).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// A shared-memory address of this CTA re-addressed to the same offset in another CTA of the cluster.
+__device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// Asynchronous stores to a CTA's shared memory, counted in bytes on an mbarrier of that CTA (both shared::cluster addresses): the
+// data is there for whoever has seen the barrier's phase complete.  Only in kernels launched in clusters.  (An arrival with release
+// at cluster scope also waits for the thread's earlier stores to global memory: some 3000 cycles in a kernel that writes results all the time.)
+__device__ __forceinline__ void st_async128(uint32_t addr, const float* v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(addr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar) : "memory");
+}
+// An arrival on an mbarrier of the cluster that orders nothing.
+__device__ __forceinline__ void mbar_arrive_relaxed_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 // ------------------------------------------------------------------ tensor memory
@@ -354,6 +377,10 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr, uint32_t lbo_
   d |= (uint64_t)1 << 46;
   d |= (uint64_t)2 << 61;
   return d;
+}
+// The same for a 64-byte-swizzled tile (rows of 64 bytes, groups of eight rows 512 bytes long; layout type 4).
+__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
+  return (smem_desc_sw128(addr, lbo_bytes, sbo_bytes) & ~((uint64_t)7 << 61)) | ((uint64_t)4 << 61);
 }
 
 }  // namespace ptx

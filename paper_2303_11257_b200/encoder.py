@@ -41,9 +41,10 @@ class UnitScaledEncoderLayer:
                  fused_attention: bool = False):
         assert d % nhead == 0 and norm in (None, "post")
         self.attention, self.norm, self.eps = attention, norm, eps
-        # fused_attention: scores, scaled softmax and context of the forward pass as one us_attention_fwd launch, and
-        # dP, the softmax gradient and dQ of the backward pass as one us_attention_bwd launch (heads of 64, at most 512
-        # tokens per sequence; 16-bit or FP8 attention operands); the scores and the gradient dP are then never stored
+        # fused_attention: scores, scaled softmax and context of the forward pass as one us_attention_fwd launch, and the
+        # whole backward pass as one us_attention_bwd_all launch, or dP, the softmax gradient and dQ as one us_attention_bwd
+        # launch (heads of 64, at most 512 tokens per sequence; 16-bit or FP8 attention operands); the scores and the
+        # gradient dP are then never stored
         self.fused_attention = fused_attention
         if fused_attention and not (d // nhead == 64 and slen <= 512):
             raise ValueError("fused attention needs heads of 64 and sequences of at most 512 tokens")
@@ -95,19 +96,30 @@ class UnitScaledEncoderLayer:
         self._launches = 1 + (3 if fused_attention else 5) + 7 + ((10 if (attention == "fp8" or fused_attention) else 11) - (2 if fused_attention else 0)) + (7 if norm == "post" else 0)
         self.bt_fused = L.attention_batch(n, qkv, qkv, qkv, td, sq)
         self.bt_fused_bwd = L.attention_bwd_batch(n, td, sq, qkv, qkv, sq, qkv)
+        self.bt_fused_all = L.attention_bwd_all_batch(n, td, sq, qkv, qkv, qkv, sq, qkv, qkv, qkv)
+        # The whole backward pass of attention as one launch where that was the faster way, against three (us, 8192 tokens of
+        # 16 heads): 16-bit operands, sequences of 32: 83 against 135, 128: 32 / 56, 256: 66 / 84, 400 (12 heads): 111 / 103,
+        # 512: 117 / 132; FP8 operands, 256: 53 / 60, 400 (12 heads): 97 / 85, 512: 99 / 95.
+        self._whole = slen <= 256 or (slen > 448 and attention != "fp8")
+
+    @property
+    def whole_bwd(self) -> bool:
+        """Whether the backward pass of attention is one launch."""
+        return self.fused_attention and self._whole
 
     @property
     def launches_per_step(self) -> int:
         """Library operations of one step with every GEMM of the layer itself counted (the FFN block's six GEMMs as its
-        gemm_launches, without layer norms).  The gradient GEMMs of a projection go out together: kernel_launches is the
-        number of kernels."""
+        gemm_launches, without layer norms; the backward pass of fused attention as three operations: dQ, dK, dV).  The
+        gradient GEMMs of a projection go out together: kernel_launches is the number of kernels."""
         return self._launches - (6 - self.ffn.gemm_launches if self.norm is None else 0)
 
     @property
     def kernel_launches(self) -> int:
         """Kernel launches of one step while the grouped launches hold its tiles: launches_per_step less one for each
-        projection, and with layer norms the three GEMMs that end the FFN block's backward pass as one."""
-        return self.launches_per_step - 2 - (2 if self.norm is not None and self.ffn.grouped else 0)
+        projection, with layer norms the three GEMMs that end the FFN block's backward pass as one, and the fused backward pass of
+        attention as one."""
+        return self.launches_per_step - 2 - (2 if self.norm is not None and self.ffn.grouped else 0) - (2 if self.whole_bwd else 0)
 
     def _heads(self, M, which):
         """Problem (0, 0) of a [T x 3d] matrix: rows of the first sequence, columns of head 0 of Q / K / V."""
@@ -175,18 +187,22 @@ class UnitScaledEncoderLayer:
                              (L.US_OP_BWD_X, self.g1q, self.Wo_q, sc["beta_o"], self.dC, None, None)], ws)
         dQ, dK, dV = (self._heads(self.dQKV, i) for i in range(3))
         dS, dC_h = self.dS[:s], self.dC[:s, : self.hd]
-        yield self.SIDE, p.batched("us_linear_bwd_w_batched", P, dC_h, sc["beta_V"], dV, self.bt["dV"], ws)
-        gemm_dk = p.batched("us_linear_bwd_w_batched", dS, Q, sc["beta_K"], dK, self.bt["dK"], ws)
-        if fused:
-            yield MAIN, L.Call("us_attention_bwd", p.mat(dC_h), p.mat(P), p.mat(K), p.mat(V), sc["beta_P"], sc["sm"], sc["sm"], sc["beta_Q"],
-                               p.mat(dS), p.mat(dQ), self.bt_fused_bwd, *tail)
-            yield self.SIDE, gemm_dk
+        if self.whole_bwd:
+            yield MAIN, L.Call("us_attention_bwd_all", *(p.mat(t) for t in (dC_h, P, Q, K, V)), sc["beta_P"], sc["sm"], sc["sm"], sc["beta_Q"],
+                               sc["beta_K"], sc["beta_V"], *(p.mat(t) for t in (dS, dQ, dK, dV)), self.bt_fused_all, *tail)
         else:
-            yield MAIN, p.batched("us_linear_bwd_x_batched", dC_h, V, sc["beta_P"], self.dP[:s], self.bt["dP"], ws)
-            yield MAIN, L.Call("us_softmax_bwd", p.mat(self.P), p.mat(self.dP), sc["sm"], sc["sm"], p.mat(self.dS))
-            yield self.SIDE, gemm_dk
-            yield MAIN, p.batched("us_linear_fwd_batched", dS, K, sc["beta_Q"], dQ, self.bt["dQ"], ws)
-        yield self.JOIN, None                                       # dQ, dK, dV all written
+            yield self.SIDE, p.batched("us_linear_bwd_w_batched", P, dC_h, sc["beta_V"], dV, self.bt["dV"], ws)
+            gemm_dk = p.batched("us_linear_bwd_w_batched", dS, Q, sc["beta_K"], dK, self.bt["dK"], ws)
+            if fused:
+                yield MAIN, L.Call("us_attention_bwd", p.mat(dC_h), p.mat(P), p.mat(K), p.mat(V), sc["beta_P"], sc["sm"], sc["sm"], sc["beta_Q"],
+                                   p.mat(dS), p.mat(dQ), self.bt_fused_bwd, *tail)
+                yield self.SIDE, gemm_dk
+            else:
+                yield MAIN, p.batched("us_linear_bwd_x_batched", dC_h, V, sc["beta_P"], self.dP[:s], self.bt["dP"], ws)
+                yield MAIN, L.Call("us_softmax_bwd", p.mat(self.P), p.mat(self.dP), sc["sm"], sc["sm"], p.mat(self.dS))
+                yield self.SIDE, gemm_dk
+                yield MAIN, p.batched("us_linear_fwd_batched", dS, K, sc["beta_Q"], dQ, self.bt["dQ"], ws)
+            yield self.JOIN, None                                   # dQ, dK, dV all written
         if self.dQKV is not self.dQKVq:
             yield MAIN, L.Call("us_cast_fp8", p.mat(self.dQKV), 1.0, p.mat(self.dQKVq))
         yield MAIN, p.group([(L.US_OP_BWD_W, self.Xq, self.dQKVq, sc["beta_w"], self.dWqkv, None, None),
@@ -201,7 +217,7 @@ class UnitScaledEncoderLayer:
         p = self._plan
         if p is None or not p.same(owned, state):
             p = self._plan = L.Plan(owned, state)
-        if not (stream is None and self.ffn.concurrent):
+        if self.whole_bwd or not (stream is None and self.ffn.concurrent):
             p.issue(self._lay_out, inputs, L._stream(stream))
             return
         cur = torch.cuda.current_stream()
@@ -279,16 +295,21 @@ class UnitScaledEncoderLayer:
         L.linear_together([L.linear_call(L.US_OP_BWD_W, self.Cq, self.g1q, sc["beta_w"], self.dWo),
                            L.linear_call(L.US_OP_BWD_X, self.g1q, self.Wo_q, sc["beta_o"], self.dC)], ws, cur)
         dC_h = self.dC[:s, : self.hd]
-        beside(lambda st: L.us_linear_bwd_w_batched(self.P[:s], dC_h, sc["beta_V"], self._heads(self.dQKV, 2), self.bt["dV"], ws, st))
-        if self.fused_attention:
-            L.us_attention_bwd(dC_h, self.P[:s], K, V, sc["beta_P"], sc["sm"], sc["sm"], sc["beta_Q"], self.dS[:s],
-                               self._heads(self.dQKV, 0), self.bt_fused_bwd, ws, cur)
-            beside(lambda st: L.us_linear_bwd_w_batched(self.dS[:s], Q, sc["beta_K"], self._heads(self.dQKV, 1), self.bt["dK"], ws, st))
+        if self.whole_bwd:
+            L.us_attention_bwd_all(dC_h, self.P[:s], Q, K, V, sc["beta_P"], sc["sm"], sc["sm"], sc["beta_Q"], sc["beta_K"], sc["beta_V"],
+                                   self.dS[:s], *(self._heads(self.dQKV, i) for i in range(3)), self.bt_fused_all, ws, cur)
         else:
-            L.us_linear_bwd_x_batched(dC_h, V, sc["beta_P"], self.dP[:s], self.bt["dP"], ws, cur)
-            L.us_softmax_bwd(self.P, self.dP, sc["sm"], sc["sm"], self.dS, cur)
-            beside(lambda st: L.us_linear_bwd_w_batched(self.dS[:s], Q, sc["beta_K"], self._heads(self.dQKV, 1), self.bt["dK"], ws, st))
-            L.us_linear_fwd_batched(self.dS[:s], K, sc["beta_Q"], self._heads(self.dQKV, 0), self.bt["dQ"], ws, cur)
+            beside(lambda st: L.us_linear_bwd_w_batched(self.P[:s], dC_h, sc["beta_V"], self._heads(self.dQKV, 2), self.bt["dV"], ws, st))
+            gemm_dk = lambda st: L.us_linear_bwd_w_batched(self.dS[:s], Q, sc["beta_K"], self._heads(self.dQKV, 1), self.bt["dK"], ws, st)
+            if self.fused_attention:
+                L.us_attention_bwd(dC_h, self.P[:s], K, V, sc["beta_P"], sc["sm"], sc["sm"], sc["beta_Q"], self.dS[:s],
+                                   self._heads(self.dQKV, 0), self.bt_fused_bwd, ws, cur)
+                beside(gemm_dk)
+            else:
+                L.us_linear_bwd_x_batched(dC_h, V, sc["beta_P"], self.dP[:s], self.bt["dP"], ws, cur)
+                L.us_softmax_bwd(self.P, self.dP, sc["sm"], sc["sm"], self.dS, cur)
+                beside(gemm_dk)
+                L.us_linear_fwd_batched(self.dS[:s], K, sc["beta_Q"], self._heads(self.dQKV, 0), self.bt["dQ"], ws, cur)
         if par:
             cur.wait_stream(side)                                   # dQ, dK, dV all written
         if self.dQKV is not self.dQKVq:

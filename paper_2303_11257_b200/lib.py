@@ -53,6 +53,11 @@ class us_attention_bwd_batch(C.Structure):
                 ("v_stride", C.c_int64 * 2), ("ds_stride", C.c_int64 * 2), ("dq_stride", C.c_int64 * 2)]
 
 
+class us_attention_bwd_all_batch(C.Structure):
+    _fields_ = [(n, C.c_int64 * 2) for n in ("count", "dc_stride", "p_stride", "q_stride", "k_stride", "v_stride", "ds_stride",
+                                             "dq_stride", "dk_stride", "dv_stride")]
+
+
 class us_linear_call(C.Structure):
     _fields_ = [("op", C.c_int32), ("a", us_mat), ("b", us_mat), ("scale", C.c_float), ("ep", us_epilogue), ("out", us_mat)]
 
@@ -90,6 +95,8 @@ def _load() -> C.CDLL:
     lib.us_attention_fwd.restype = C.c_int
     lib.us_attention_bwd.argtypes = [MP, MP, MP, MP, F, F, F, F, MP, MP, C.POINTER(us_attention_bwd_batch), V, SZ, V]
     lib.us_attention_bwd.restype = C.c_int
+    lib.us_attention_bwd_all.argtypes = [MP] * 5 + [F] * 6 + [MP] * 4 + [C.POINTER(us_attention_bwd_all_batch), V, SZ, V]
+    lib.us_attention_bwd_all.restype = C.c_int
     lib.us_linear_fwd_static_ws.argtypes = [MP, MP, F, EP, MP, C.POINTER(C.c_void_p), V]
     lib.us_linear_fwd_static_ws.restype = C.c_int
     lib.us_linear_fwd_check.argtypes = [MP, MP, EP, MP, V, SZ]
@@ -505,6 +512,19 @@ def us_attention_bwd(dC, P, K, V, beta_p, softmax_alpha, softmax_beta, beta_q, d
     """Attention backward down to the queries: dS (for the dK matmul) and dQ from dC, the stored P, K and V."""
     _check("us_attention_bwd", _entry("us_attention_bwd")(dC, P, K, V, beta_p, softmax_alpha, softmax_beta, beta_q, dS, dQ, bt, ws, ws, _stream(stream)))
     return dQ
+
+
+def attention_bwd_all_batch(count, dc_stride, p_stride, q_stride, k_stride, v_stride, ds_stride, dq_stride, dk_stride, dv_stride) -> us_attention_bwd_all_batch:
+    b = us_attention_bwd_all_batch()
+    for (name, _), v in zip(b._fields_, (count, dc_stride, p_stride, q_stride, k_stride, v_stride, ds_stride, dq_stride, dk_stride, dv_stride)):
+        getattr(b, name)[:] = v
+    return b
+
+
+def us_attention_bwd_all(dC, P, Q, K, V, beta_p, softmax_alpha, softmax_beta, beta_q, beta_k, beta_v, dS, dQ, dK, dV, bt, ws, stream=None):
+    """The whole backward pass of attention in one launch; dS may be None (not stored)."""
+    _check("us_attention_bwd_all", _entry("us_attention_bwd_all")(dC, P, Q, K, V, beta_p, softmax_alpha, softmax_beta, beta_q, beta_k, beta_v, dS, dQ, dK, dV, bt, ws, ws, _stream(stream)))
+    return dQ, dK, dV
 
 
 def us_linear_fwd_static_ws(X, W, alpha, Y, ep=None, stream=None) -> int:
