@@ -86,6 +86,60 @@ __global__ void __launch_bounds__(kThreads) ew_kernel(const EwArgs p) {
   }
 }
 
+// One cast whose rows start on 16-byte boundaries (padded rows too); bound by HBM.  The row of a chunk comes from a multiply
+// instead of a 64-bit division, two chunks are in flight per thread, and all loads of a row's ragged last chunk are issued before
+// the first value is used.  Float32 to E4M3, against the general kernel: 16384 x 2048 29.1 -> 26.5 us (6.3 TB/s), 1024 x 30522 in
+// padded rows 28.8 -> 26.0, 128 x 1000 2.7 -> 2.3.
+struct CastArgs {
+  const char* src;
+  char* dst;
+  int src_dt, dst_dt;
+  int64_t src_ld, dst_ld, cols;
+  float scale;
+  int rows;                        // 1: the tensor is one long row
+  uint32_t chunks_per_row, total;
+  FastDiv d_row;                   // by chunks_per_row
+};
+
+__global__ void __launch_bounds__(kThreads) cast_kernel(const CastArgs p) {
+  const int zero = ptx::grid_wait_previous();
+  const uint32_t stride = gridDim.x * kThreads;
+  for (uint32_t c = blockIdx.x * kThreads + threadIdx.x + zero; c < p.total; c += 2 * stride) {
+    float v[2][kVec];
+    int64_t at[2];
+    int n[2];                                               // elements of the chunk that exist
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const uint32_t ck = c + k * stride;
+      n[k] = 0;
+      if (ck >= p.total) continue;
+      const uint32_t row = p.rows == 1 ? 0u : (uint32_t)p.d_row.div((int)ck);
+      const int64_t col = (int64_t)(ck - row * p.chunks_per_row) * kVec, i0 = (int64_t)row * p.src_ld + col;
+      at[k] = (int64_t)row * p.dst_ld + col;
+      n[k] = (int)min((int64_t)kVec, p.cols - col);
+      if (n[k] == kVec) {
+        load_vec<kVec>(p.src + i0 * dtype_size(p.src_dt), p.src_dt, v[k]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < kVec; ++i) v[k][i] = i < n[k] ? load_one(p.src, p.src_dt, i0 + i) : 0.f;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      if (n[k] == 0) continue;
+#pragma unroll
+      for (int i = 0; i < kVec; ++i) v[k][i] *= p.scale;
+      if (n[k] == kVec) {
+        store_vec<kVec>(p.dst + at[k], p.dst_dt, v[k]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < kVec; ++i)
+          if (i < n[k]) store_one(p.dst, p.dst_dt, at[k] + i, v[k][i]);
+      }
+    }
+  }
+}
+
 // Several casts in one launch: the chunks of all tensors are numbered consecutively and a thread finds
 // the tensor of its chunk by scanning the (at most kMultiMax) cumulative counts.  Tensors are contiguous
 // and 16-byte aligned (checked on the host), so every chunk but a tensor's last takes the vector path.
@@ -253,6 +307,21 @@ extern "C" us_status us_cast_fp8(const us_mat* src, float scale, const us_mat* d
   us_status s = check_ew(src, nullptr, dst);
   if (s != US_OK) return s;
   if (dst->dtype != US_E4M3 && dst->dtype != US_E5M2) return US_ERR_UNSUPPORTED;
+  // Rows on 16-byte boundaries and fewer than 2^31 chunks; anything else element by element through the general kernel.
+  const bool dense = src->ld == src->cols && dst->ld == dst->cols;
+  const int64_t rows = dense ? 1 : src->rows, cols = dense ? src->rows * src->cols : src->cols, cpr = (cols + kVec - 1) / kVec;
+  if (row_starts_aligned(src, dense) && row_starts_aligned(dst, dense) && rows > 0 && cpr > 0 && cpr < 0x7fffffffll / rows) {
+    CastArgs p{};
+    p.src = static_cast<const char*>(src->ptr); p.dst = static_cast<char*>(dst->ptr);
+    p.src_dt = src->dtype; p.dst_dt = dst->dtype; p.src_ld = src->ld; p.dst_ld = dst->ld;
+    p.cols = cols; p.rows = (int)rows; p.scale = scale;
+    p.chunks_per_row = (uint32_t)cpr; p.total = (uint32_t)(rows * cpr);
+    p.d_row = make_fast_div((int)cpr);
+    const int sms = host::sm_count();
+    if (sms <= 0) return US_ERR_CUDA;
+    const int64_t want = ((int64_t)p.total + kThreads - 1) / kThreads, cap = (int64_t)sms * 8;
+    return host::launch(cast_kernel, nullptr, (int)(want < cap ? want : cap), kThreads, 0, 1, static_cast<cudaStream_t>(stream), p);
+  }
   return ew_launch<kCast>(src, nullptr, dst, scale, 0.f, stream);
 }
 

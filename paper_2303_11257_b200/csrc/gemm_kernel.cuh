@@ -29,23 +29,6 @@
 
 namespace us {
 
-// Division of a non-negative int below 2^31 by a divisor fixed at launch: one multiply-high, one
-// add and one shift instead of the ~30-instruction sequence of a hardware-less integer divide, which
-// every epilogue warp would otherwise run several times per tile.  mul = floor(2^32 (2^shift - d) / d) + 1,
-// shift = ceil(log2 d); floor(n / d) = (mulhi(n, mul) + n) >> shift.
-struct FastDiv {
-  uint32_t mul, shift;
-  __device__ __forceinline__ int div(int n) const { return (int)((__umulhi((uint32_t)n, mul) + (uint32_t)n) >> shift); }
-};
-inline FastDiv make_fast_div(int d) {
-  FastDiv f;
-  uint32_t l = 0;
-  while ((1ll << l) < d) ++l;
-  f.shift = l;
-  f.mul = (uint32_t)((((1ull << l) - (uint64_t)d) << 32) / (uint64_t)d + 1ull);
-  return f;
-}
-
 struct GemmParams {
   int M, N, K;
   int tiles_m, tiles_n;

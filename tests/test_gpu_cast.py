@@ -70,6 +70,20 @@ def test_cast_shapes_scales_and_saturation(fmt, shape, ld):
             assert not full[:, shape[1]:].any()
 
 
+@pytest.mark.parametrize("shape,ld", [((2500, 2007), 2016), ((700, 16001), 16016), ((1, 4099), None)])
+@pytest.mark.parametrize("src", ["f32", "bf16"])
+def test_cast_of_padded_rows_with_several_chunks_per_thread(shape, ld, src):
+    """More chunks than resident threads, row ends inside a chunk, and nothing written behind a row's end."""
+    from paper_2303_11257_b200 import synth
+    L = _lib()
+    x = synth.normal(12, 0, shape)
+    dst = U.empty(*shape, "e4m3", ld)
+    L.us_cast_fp8(U.to_device(x, src, ld), 0.75, dst)
+    assert np.array_equal(U.codes_of(dst), F.scaled_cast(U.values_of(x, src).astype(np.float32), 0.75, F.E4M3))
+    if ld:
+        assert not dst.as_strided((shape[0], ld), (ld, 1)).view(torch.uint8)[:, shape[1]:].any()
+
+
 def test_cast_empty_and_errors():
     L = _lib()
     src = torch.zeros((0, 8), device="cuda")
