@@ -140,7 +140,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tq, const __grid_consta
   ptx::grid_wait_previous();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       // ---------------------------------------------------------------- TMA loads and both MMA chains
       auto load_qk = [&](int tile) {
         int q0, b1, b0;
@@ -216,7 +216,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tq, const __grid_consta
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       // ---------------------------------------------------------------- the stored weights leave by TMA store
       // A buffer is given back once the store after next has been issued and its own has been read (the softmax warps
       // are then at most two blocks ahead, never waiting for a buffer that this thread holds back).
@@ -480,7 +480,7 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_const
   ptx::grid_wait_previous();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       // ---------------------------------------------------------------- TMA loads and both MMA chains
       auto load_in = [&](int tile) {                           // dC tile and V
         int q0, b1, b0;
@@ -547,7 +547,7 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_const
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       // ---------------------------------------------------------------- the weight tile: P in by TMA load, dS out by TMA store
       auto load_p = [&](int tile) {                            // key block by key block
         int q0, b1, b0;

@@ -158,7 +158,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
   auto wait1 = [&](uint32_t bar, uint32_t parity) { return wait_bounded(bar, parity, abort_flag, a.status, a.wait_limit); };
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       // ---------------------------------------------------------------- MMA issue
       // dP and dV of tile n, before dQ and dK of tile n - 1
       auto opening = [&](int n) -> bool {
@@ -215,7 +215,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       // ---------------------------------------------------------------- loads, and dS out
       auto load = [&](uint32_t dst, const CUtensorMap* tm, uint32_t bar, int row, int n) {      // row < 0: the tile's query rows
         int q0, b1, b0;

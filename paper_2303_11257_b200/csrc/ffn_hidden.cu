@@ -135,7 +135,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (every CTA)
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       uint32_t issued = 0;
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
@@ -181,7 +181,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA of a pair only)
-    if (lane == 0 && rank == 0) {
+    if (ptx::elect_one() && rank == 0) {
       ptx::grid_wait_previous();                       // no operand comes earlier: the bounded waits begin when the loads do
       int stage = 0; uint32_t phase = 0, local = 0;
       bool ok = true;
@@ -344,7 +344,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         if (active) {
           ptx::tmem_ld_32x32_issue(t_row, r0);
           if (SPLIT == 1) {
-            if (lane == 0) ptx::bulk_wait_group_read<0>();      // earlier stores have read the staging boxes
+            if (ptx::elect_one()) ptx::bulk_wait_group_read<0>();      // earlier stores have read the staging boxes
             __syncwarp();
           }
           ptx::tmem_ld_fence(r0);
@@ -385,7 +385,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
           if (SPLIT == 1) {
             ptx::fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) {
+            if (ptx::elect_one()) {
               if (sub == 0) {
                 ptx::tma_store_2d(&tm_a, buf_out, n_w, row0);
               } else {
@@ -400,7 +400,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     // Leaving (early too, when a wait ran out somewhere in the CTA): tensor-memory loads have landed and
     // the stores have read shared memory before the CTA may give up its resources.
     ptx::tmem_ld_wait_all();
-    if (lane == 0) ptx::bulk_wait_group_read<0>();
+    if (ptx::elect_one()) ptx::bulk_wait_group_read<0>();
     __syncwarp();
   }
 

@@ -110,7 +110,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (every CTA)
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       uint32_t issued = 0;
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
@@ -158,7 +158,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA of a pair only)
-    if (lane == 0 && rank == 0) {
+    if (ptx::elect_one() && rank == 0) {
       ptx::grid_wait_previous();                       // no operand comes earlier: the bounded waits begin when the loads do
       int stage = 0; uint32_t phase = 0, local = 0;
       bool ok = true;
@@ -222,7 +222,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
     bool in_pending = false, ok = true;
 
     auto issue_in = [&](const GroupProblem& P, int col, int row0) {
-      if (lane == 0) {
+      if (ptx::elect_one()) {
         ptx::mbar_expect_tx(in_bar, 4096);
         ptx::tma_load_2d(buf_in, &P.tskip, in_bar, col, row0);
       }
@@ -302,7 +302,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
           }
           const int out_off = (32 * sl) & (out_box_cols - 1);
           if (out_off == 0) {                                  // the output box is about to be refilled
-            if (lane == 0) ptx::bulk_wait_group_read<0>();
+            if (ptx::elect_one()) ptx::bulk_wait_group_read<0>();
             __syncwarp();
           }
           float v[32];
@@ -360,7 +360,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
           if (out_off + 32 == out_box_cols || last_slice) {
             ptx::fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) { ptx::tma_store_2d(&P.tout, buf_out, col - out_off, row0); ptx::bulk_commit_group(); }
+            if (ptx::elect_one()) { ptx::tma_store_2d(&P.tout, buf_out, col - out_off, row0); ptx::bulk_commit_group(); }
           }
         }
       }
@@ -371,7 +371,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
     }
     if (in_pending && lane == 0)
       for (uint32_t it = 0; it < g.wait_limit && !ptx::mbar_try_wait(in_bar, in_phase); ++it) {}
-    if (lane == 0) ptx::bulk_wait_group_read<0>();
+    if (ptx::elect_one()) ptx::bulk_wait_group_read<0>();
     __syncwarp();
   }
 

@@ -269,7 +269,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
   };
   bool in_pending = false;                                   // an input box load has been issued and not yet waited for
   auto issue_in = [&](int col, int row0) {
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       ptx::mbar_expect_tx(c.in_bar, 4096);
       ptx::tma_load_2d(buf_in, tm_in, c.in_bar, col, row0);      // fused inputs exist for single problems only
     }
@@ -340,9 +340,9 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
           if (!in_kind && !aux_out) {                        // both boxes hold outputs, used alternately
             buf_out = c.buf0 + (plain_toggle ? 4096u : 0u);
             plain_toggle ^= 1;
-            if (lane == 0) ptx::bulk_wait_group_read<1>();
+            if (ptx::elect_one()) ptx::bulk_wait_group_read<1>();
           } else {
-            if (lane == 0) ptx::bulk_wait_group_read<0>();
+            if (ptx::elect_one()) ptx::bulk_wait_group_read<0>();
           }
           __syncwarp();
         }
@@ -445,12 +445,12 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
         if (aux_out && (aux_off == 32 || last_slice)) {
           ptx::fence_proxy_async_smem();
           __syncwarp();
-          if (lane == 0) { ptx::tma_store_2d(tm_aux, buf_aux, col - aux_off, row0); ptx::bulk_commit_group(); }
+          if (ptx::elect_one()) { ptx::tma_store_2d(tm_aux, buf_aux, col - aux_off, row0); ptx::bulk_commit_group(); }
         }
         if (out_off + 32 == out_box_cols || last_slice) {
           ptx::fence_proxy_async_smem();
           __syncwarp();
-          if (lane == 0) {
+          if (ptx::elect_one()) {
             if (BATCHED) { int b0, b1; tile_batch(p, tile, b0, b1); ptx::tma_store_4d(tm_out, buf_out, col - out_off, row0, b1, b0); }
             else ptx::tma_store_2d(tm_out, buf_out, col - out_off, row0);
             ptx::bulk_commit_group();
@@ -466,7 +466,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
   // land before the CTA may give up its shared memory.
   if (in_kind && in_pending && lane == 0)
     for (uint32_t it = 0; it < p.wait_limit && !ptx::mbar_try_wait(c.in_bar, in_phase); ++it) {}
-  if (lane == 0) ptx::bulk_wait_group_read<0>();             // stores have left shared memory before the CTA may exit
+  if (ptx::elect_one()) ptx::bulk_wait_group_read<0>();             // stores have left shared memory before the CTA may exit
   __syncwarp();
 }
 
@@ -506,7 +506,7 @@ __device__ __forceinline__ void epilogue_act16(const GemmParams& p, const CUtens
     row0 = tm * (kBM * CG) + c.rank * kBM + q * 32;
     n_w = tn * BN + part * 64;
   };
-  auto issue_in = [&](int half, int n_w, int row0) {          // lane 0 only; a box wholly outside the matrix reads zeros
+  auto issue_in = [&](int half, int n_w, int row0) {          // one elected lane; a box wholly outside the matrix reads zeros
     const uint32_t bar = half ? in_bar1 : c.in_bar;
     ptx::mbar_expect_tx(bar, 2048);
     ptx::tma_load_2d(buf_aux + 2048u * half, tm_aux, bar, n_w + 32 * half, row0);
@@ -566,7 +566,7 @@ __device__ __forceinline__ void epilogue_act16(const GemmParams& p, const CUtens
   if (tile < c.num_tiles) {
     coords(tile, row0, n_w);
     if (kIn) {
-      if (lane == 0) { issue_in(0, n_w, row0); issue_in(1, n_w, row0); }
+      if (ptx::elect_one()) { issue_in(0, n_w, row0); issue_in(1, n_w, row0); }
       pending[0] = pending[1] = true;
     }
   }
@@ -586,7 +586,7 @@ __device__ __forceinline__ void epilogue_act16(const GemmParams& p, const CUtens
     int next_row0 = 0, next_n_w = 0;
     if (next < c.num_tiles) coords(next, next_row0, next_n_w);
     if (active) {
-      if (lane == 0) ptx::bulk_wait_group_read<0>();          // the previous tile's stores have read the staging boxes
+      if (ptx::elect_one()) ptx::bulk_wait_group_read<0>();          // the previous tile's stores have read the staging boxes
       __syncwarp();
       ptx::tmem_ld_fence(r0);
       ptx::tmem_ld_32x32_issue(t_row + 32, r1);
@@ -602,7 +602,7 @@ __device__ __forceinline__ void epilogue_act16(const GemmParams& p, const CUtens
     if (kIn) {
       __syncwarp();                                           // every lane has read the first input box
       if (next < c.num_tiles) {
-        if (lane == 0) issue_in(0, next_n_w, next_row0);
+        if (ptx::elect_one()) issue_in(0, next_n_w, next_row0);
         pending[0] = true;
       }
     }
@@ -619,14 +619,14 @@ __device__ __forceinline__ void epilogue_act16(const GemmParams& p, const CUtens
     if (kIn) {
       __syncwarp();
       if (next < c.num_tiles) {
-        if (lane == 0) issue_in(1, next_n_w, next_row0);
+        if (ptx::elect_one()) issue_in(1, next_n_w, next_row0);
         pending[1] = true;
       }
     }
     if (active) {
       ptx::fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) {
+      if (ptx::elect_one()) {
         if (aux_out) ptx::tma_store_2d(tm_aux, buf_aux, n_w, row0);
         ptx::tma_store_2d(tm_out, buf_out, n_w, row0);
         ptx::bulk_commit_group();
@@ -641,7 +641,7 @@ __device__ __forceinline__ void epilogue_act16(const GemmParams& p, const CUtens
     if (pending[0]) for (uint32_t it = 0; it < p.wait_limit && !ptx::mbar_try_wait(c.in_bar, ph0); ++it) {}
     if (pending[1]) for (uint32_t it = 0; it < p.wait_limit && !ptx::mbar_try_wait(in_bar1, ph1); ++it) {}
   }
-  if (lane == 0) ptx::bulk_wait_group_read<0>();             // stores have left shared memory before the CTA may exit
+  if (ptx::elect_one()) ptx::bulk_wait_group_read<0>();             // stores have left shared memory before the CTA may exit
   __syncwarp();
 }
 
@@ -713,7 +713,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (every CTA)
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       uint32_t issued = 0;
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
@@ -767,7 +767,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA of a pair only)
-    if (lane == 0 && rank == 0) {
+    if (ptx::elect_one() && rank == 0) {
       ptx::grid_wait_previous();                       // no operand comes earlier: the bounded waits begin when the loads do
       int stage = 0; uint32_t phase = 0;
       uint32_t local = 0;

@@ -13,6 +13,9 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// True in one lane of a converged warp, always the same one.  A role of one thread, or a TMA copy, that begins with this instead of a
+// test of the lane index is known to have one active lane: tensor-core, copy and commit instructions, whose operands are uniform
+// registers, then take 10 to 20 cycles each instead of some 50 (four MMAs of a K block: 44 cycles instead of 200).
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred;
   asm volatile(
