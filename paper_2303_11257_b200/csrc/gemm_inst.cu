@@ -3,6 +3,8 @@
 // this file once per combination, in parallel.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "gemm_kernel.cuh"
 #include "gemm_launch.h"
 #include "host.h"
@@ -15,14 +17,14 @@ namespace us {
 namespace {
 
 // Tensor map over a row-major matrix [rows x cols] of ES-byte elements with a box of `box_rows` rows
-// and `box_bytes` (128, or 64) bytes per row, swizzled with the pattern of that width.  Out-of-range parts of a box read as zero.
+// and `box_bytes` (128, 64 or 32) bytes per row, swizzled with the pattern of that width (32: not).  Out-of-range parts of a box read as zero.
 static bool make_tmap(CUtensorMap* tm, const us_mat* m, int es, int box_rows, int box_bytes = 128,
                       const BatchDesc* bd = nullptr, const int64_t* bstride = nullptr) {
   host::EncodeTiledFn fn = host::encode_tiled_fn();
   if (!fn) return false;
   const CUtensorMapDataType type = es == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8
                                  : es == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_UINT32;
-  const CUtensorMapSwizzle swz = box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
+  const CUtensorMapSwizzle swz = box_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_NONE : box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
   CUresult r;
   if (!bd) {
     cuuint64_t dims[2] = {(cuuint64_t)m->cols, (cuuint64_t)m->rows};
@@ -49,14 +51,16 @@ static us_status launch(const us_mat* A, const us_mat* B, const GemmParams& p, c
   constexpr int kBK = kStageKBytes / ES;
   CUtensorMap ta, tb, t_out, t_aux, t_skip;
   const BatchDesc* b4 = BATCHED ? bd : nullptr;
-  if (!make_tmap(&ta, A, ES, A_MN ? kBK : kBM, 128, b4, b4 ? bd->a : nullptr)) return US_ERR_CUDA;
-  if (!make_tmap(&tb, B, ES, B_MN ? kBK : BN / CG, 128, b4, b4 ? bd->b : nullptr)) return US_ERR_CUDA;
-  // epilogue boxes: 32 rows x 128 (or 64) bytes; unused maps alias the output's so that every parameter is valid
-  const bool narrow_out = EW == 16 || (BN == 128 && dtype_size(em.out->dtype) == 1);      // FP8 codes of a warp's 64 columns
-  if (!make_tmap(&t_out, em.out, dtype_size(em.out->dtype), 32, narrow_out ? 64 : 128, b4, b4 ? bd->out : nullptr)) return US_ERR_CUDA;
+  if (!make_tmap(&ta, A, ES, A_MN ? kBK : BN == 64 ? (int)p.a_bytes / kStageKBytes : kBM, 128, b4, b4 ? bd->a : nullptr)) return US_ERR_CUDA;
+  if (!make_tmap(&tb, B, ES, B_MN ? kBK : BN / CG, B_MN && BN / CG * ES < 128 ? 64 : 128, b4, b4 ? bd->b : nullptr)) return US_ERR_CUDA;
+  // epilogue boxes: 32 rows x the bytes of a warp's columns, 128 at most (the 16-warp epilogue: 64 FP8 codes); unused maps alias the
+  // output's so that every parameter is valid
+  const int out_es = dtype_size(em.out->dtype);
+  if (!make_tmap(&t_out, em.out, out_es, 32, EW == 16 ? 64 : out_row_bytes(BN, out_es), b4, b4 ? bd->out : nullptr)) return US_ERR_CUDA;
   t_aux = t_out; t_skip = t_out;
   // the 16-warp GELU-gradient epilogue reads the stored pre-activation as 32-row x 64-byte boxes (one per 32-column slice)
-  if (EPI != kEpiLegacy && em.aux && !make_tmap(&t_aux, em.aux, dtype_size(em.aux->dtype), 32, (EW == 16 && EPI == kEpiGeluGrad) ? 64 : 128)) return US_ERR_CUDA;
+  const int aux_row = EPI == kEpiGeluGrad ? (EW == 16 ? 64 : 128) : out_row_bytes(BN, 2);
+  if (EPI != kEpiLegacy && em.aux && !make_tmap(&t_aux, em.aux, dtype_size(em.aux->dtype), 32, aux_row)) return US_ERR_CUDA;
   if (EPI != kEpiLegacy && em.skip && !make_tmap(&t_skip, em.skip, dtype_size(em.skip->dtype), 32)) return US_ERR_CUDA;
   auto kern = gemm_kernel<ES, A_MN, B_MN, BN, CG, EPI, EW, BATCHED>;
   constexpr int smem = GemmSmem<BN, CG, EW>::kTotal;
@@ -78,12 +82,14 @@ static us_status pick_epilogue(const us_mat* A, const us_mat* B, const GemmParam
   // The GELU epilogues with an FP8 output (the FFN's forward and backward hidden layer) are ALU
   // bound with eight epilogue warps; they run with sixteen.
   const bool fp8_out = (em.out->dtype == US_E4M3 || em.out->dtype == US_E5M2) && p.fn == US_FN_GELU;   // the 16-warp epilogue is the GELU pair's
+  if constexpr (BN != 64) {                            // (a warp has 32 columns of a narrow tile: eight are enough there)
+    if (fp8_out && epi == kEpiGelu) return launch<ES, A_MN, B_MN, BN, CG, kEpiGelu, 16>(A, B, p, em, stream);
+    if (fp8_out && epi == kEpiGeluGrad) return launch<ES, A_MN, B_MN, BN, CG, kEpiGeluGrad, 16>(A, B, p, em, stream);
+  }
   switch (epi) {
     case kEpiPlain:    return launch<ES, A_MN, B_MN, BN, CG, kEpiPlain, 8>(A, B, p, em, stream);
-    case kEpiGelu:     return fp8_out ? launch<ES, A_MN, B_MN, BN, CG, kEpiGelu, 16>(A, B, p, em, stream)
-                                      : launch<ES, A_MN, B_MN, BN, CG, kEpiGelu, 8>(A, B, p, em, stream);
-    case kEpiGeluGrad: return fp8_out ? launch<ES, A_MN, B_MN, BN, CG, kEpiGeluGrad, 16>(A, B, p, em, stream)
-                                      : launch<ES, A_MN, B_MN, BN, CG, kEpiGeluGrad, 8>(A, B, p, em, stream);
+    case kEpiGelu:     return launch<ES, A_MN, B_MN, BN, CG, kEpiGelu, 8>(A, B, p, em, stream);
+    case kEpiGeluGrad: return launch<ES, A_MN, B_MN, BN, CG, kEpiGeluGrad, 8>(A, B, p, em, stream);
     case kEpiSkip:     return launch<ES, A_MN, B_MN, BN, CG, kEpiSkip, 8>(A, B, p, em, stream);
     default:           return launch<ES, A_MN, B_MN, BN, CG, kEpiLegacy, 8>(A, B, p, em, stream);
   }
@@ -100,7 +106,14 @@ us_status launch_gemm(const us_mat* A, const us_mat* B, GemmParams& p, const Epi
   const int sms = host::sm_count();
   const long long pair_tiles = (long long)((p.M + 2 * kBM - 1) / (2 * kBM)) * ((p.N + 255) / 256) * bd.nb0 * bd.nb1;
   const bool pair = p.N > 128 && p.M > kBM && (sms <= 0 || 4 * pair_tiles >= sms);
-  const int bn = pair ? 256 : 128, cg = pair ? 2 : 1;
+  // 128 x 64 tiles where the machine has an SM for each of them (or, batched, where the outputs are no wider): half the operand
+  // bytes and epilogue of a 128 x 128 tile per CTA.
+  const long long narrow_tiles = (long long)((p.M + kBM - 1) / kBM) * ((p.N + 63) / 64);
+  const bool narrow = !pair && (bd.batched() ? p.N <= 64 : narrow_tiles <= sms);
+  const int bn = pair ? 256 : narrow ? 64 : 128, cg = pair ? 2 : 1;
+  using Narrow = GemmSmem<64, 1, 8>;
+  p.a_bytes = (A_MN || p.M >= kBM ? kBM : (p.M + 7) / 8 * 8) * kStageKBytes;
+  p.stages = std::min((uint32_t)Narrow::kMaxStages, (uint32_t)(Narrow::kStages * Narrow::kStageBytes) / (p.a_bytes + Narrow::kBBytes));
   p.tiles_m = (p.M + kBM * cg - 1) / (kBM * cg);
   p.tiles_n = (p.N + bn - 1) / bn;
   p.nb0 = (int)bd.nb0; p.nb1 = (int)bd.nb1;
@@ -115,7 +128,8 @@ us_status launch_gemm(const us_mat* A, const us_mat* B, GemmParams& p, const Epi
   p.d_nb1 = make_fast_div(p.nb1);
   p.idesc = (p.idesc & ~((0x3fu << 17) | (0x1fu << 24))) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)((kBM * cg) >> 4) << 24);
   return pair ? pick_epilogue<ES, A_MN, B_MN, 256, 2>(A, B, p, em, epi, bd, stream)
-              : pick_epilogue<ES, A_MN, B_MN, 128, 1>(A, B, p, em, epi, bd, stream);
+       : narrow ? pick_epilogue<ES, A_MN, B_MN, 64, 1>(A, B, p, em, epi, bd, stream)
+                : pick_epilogue<ES, A_MN, B_MN, 128, 1>(A, B, p, em, epi, bd, stream);
 }
 
 template us_status launch_gemm<US_INST_ES, (US_INST_AMN != 0), (US_INST_BMN != 0)>(const us_mat*, const us_mat*, GemmParams&,

@@ -46,6 +46,7 @@ struct GemmParams {
   unsigned int* status;
   uint32_t wait_limit;                      // polls a bounded wait makes before it gives up (kWaitLimit unless a test shortens it)
   int no_loads;                             // test hook: the producer issues no operand loads, so that the waits run out
+  uint32_t a_bytes, stages;                 // narrow tiles (BN = 64): bytes of A in a stage, and the stages that fit
 };
 
 constexpr int kBM = 128;                 // tile rows = TMEM lanes
@@ -79,6 +80,10 @@ struct GemmSmem {
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr int kEpiBytes = EW * epi_warp_bytes(EW);          // 64 KB (EW = 8) or 96 KB (EW = 16)
   static constexpr int kStages = (229376 - kEpiBytes) / kStageBytes; // 32 KB stages: 5 (EW = 8) or 4 (EW = 16)
+  // A narrow tile (BN = 64) of a short matrix holds only the rows of A that exist, in as many stages as fit: one such CTA is bound
+  // by the latency of its loads.  The MMA still reads 128 rows; what lies behind those of A ends up in rows that do not exist.
+  static constexpr bool kShortA = BN == 64;
+  static constexpr int kMaxStages = kShortA ? 16 : kStages;
   static constexpr int kBarrierBytes = 512;
   static constexpr int kTotal = kStages * kStageBytes + kEpiBytes + kBarrierBytes + 1024;  // + alignment slack
 };
@@ -226,6 +231,9 @@ struct EpiCtx {
   int warp, lane, rank, group, num_groups, num_tiles;
 };
 
+// Bytes per row of an output box of the eight-warp epilogue.
+__host__ __device__ constexpr int out_row_bytes(int bn, int es) { return bn / 2 * es < 128 ? bn / 2 * es : 128; }
+
 // Epilogue through shared memory.  Each warp owns 32 rows and half of the columns of the
 // tile and two private 32-row x 128-byte boxes (128-byte-swizzled, like the TMA maps).  A row of a
 // box is written / read by the lane that owns that row, 16-byte chunk c at chunk (c ^ (row & 7)),
@@ -238,9 +246,7 @@ struct EpiCtx {
 template <int BN, int CG, int EPI, int EW, bool BATCHED>
 __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUtensorMap* tm_out, const CUtensorMap* tm_aux,
                                                 const CUtensorMap* tm_skip, const EpiCtx& c) {
-  constexpr int kWarpCols = EW == 16 ? 64 : BN / 2;         // columns of the tile one warp handles
-  // 64 columns of FP8 codes are an output box of 64 bytes per row (64-byte swizzle)
-  const bool narrow_out = EW == 16 || (kWarpCols == 64 && dtype_size(p.out_dt) == 1);
+  constexpr int kWarpCols = BN / 2;                         // columns of the tile one warp handles
   const int q = c.warp & 3, half = (c.warp - 2) >> 2;       // lane quarter; which group of kWarpCols columns
   if (half >= BN / kWarpCols) return;                       // more warps than column groups: the rest sit out
   const int lane = c.lane;
@@ -250,13 +256,17 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
   const CUtensorMap* tm_in = in_kind == 1 ? tm_aux : tm_skip;
   const bool aux_out = EPI == kEpiGelu && p.aux != nullptr;
   const int out_es = dtype_size(p.out_dt);
-  const int in_box_cols = 128 / in_es, out_box_cols = narrow_out ? 64 : 128 / out_es;
+  // Boxes have rows of 128 bytes, or of the fewer bytes that a warp's columns are, swizzled with the pattern of that width (32-byte
+  // rows: not): 16-byte chunk c of row r sits at c ^ (r & 7), 64-byte rows c ^ ((r >> 1) & 3).
+  const int out_row = out_row_bytes(BN, out_es);
+  const int in_box_cols = 128 / in_es, out_box_cols = out_row / out_es;
+  constexpr int kAuxRow = kWarpCols * 2 < 128 ? kWarpCols * 2 : 128, kAuxCols = kAuxRow / 2;
   const uint32_t buf_in = c.buf0, buf_aux = c.buf0;          // first box: input, or the kept pre-activation
   const uint32_t row_off = (uint32_t)lane * 128u;
   const uint32_t sw = (uint32_t)(lane & 7);
-  // 64-byte output rows: pitch 64, 16-byte chunk c of row r at chunk c ^ ((r >> 1) & 3)
-  const uint32_t out_row_off = narrow_out ? (uint32_t)lane * 64u : row_off;
-  const uint32_t out_sw = narrow_out ? (uint32_t)((lane >> 1) & 3) : sw;
+  const uint32_t out_row_off = (uint32_t)(lane * out_row);
+  const uint32_t out_sw = out_row == 128 ? sw : out_row == 64 ? (uint32_t)((lane >> 1) & 3) : 0u;
+  const uint32_t aux_row_off = (uint32_t)(lane * kAuxRow), aux_sw = kAuxRow == 128 ? sw : (uint32_t)((lane >> 1) & 3);
   uint32_t in_phase = 0;
   int plain_toggle = 0;
   uint32_t buf_out = c.buf0 + 4096u;
@@ -335,7 +345,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
           }
         }
         // ---- staging boxes that start with this slice must have been read by their last TMA store
-        const int aux_off = (32 * sl) & 63, out_off = (32 * sl) & (out_box_cols - 1);
+        const int aux_off = (32 * sl) & (kAuxCols - 1), out_off = (32 * sl) & (out_box_cols - 1);
         if (out_off == 0 || (aux_out && aux_off == 0)) {
           if (!in_kind && !aux_out) {                        // both boxes hold outputs, used alternately
             buf_out = c.buf0 + (plain_toggle ? 4096u : 0u);
@@ -372,12 +382,14 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
                 unpack2(x[k], a, b);
                 w[k] = p.aux_dt == US_BF16 ? pack_bf16x2(a, b) : pack_f16x2(a, b);
               }
-              ptx::sts128(buf_aux + row_off + (((aux_cb + g) ^ sw) << 4), make_uint4(w[0], w[1], w[2], w[3]));
+              ptx::sts128(buf_aux + aux_row_off + (((aux_cb + g) ^ aux_sw) << 4), make_uint4(w[0], w[1], w[2], w[3]));
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              if (p.fn == US_FN_GELU) {
-                gelu_scaled2<EW == 16>(x[k], tail_k, act_oi, y[2 * k], y[2 * k + 1]);
+              if (BN == 64 && p.fn == US_FN_GELU && out_es == 1) {     // the form the 16-warp epilogue takes for FP8 outputs of larger tiles
+                gelu_scaled2<true>(x[k], tail_k, act_oi, y[2 * k], y[2 * k + 1]);
+              } else if (p.fn == US_FN_GELU) {
+                gelu_scaled2<false>(x[k], tail_k, act_oi, y[2 * k], y[2 * k + 1]);
               } else {                                          // relu, tanh, sigmoid (table section "Activations")
                 float a, b;
                 unpack2(x[k], a, b);
@@ -442,7 +454,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
           }
         }
         // ---- boxes completed by this slice go out
-        if (aux_out && (aux_off == 32 || last_slice)) {
+        if (aux_out && (aux_off + 32 == kAuxCols || last_slice)) {
           ptx::fence_proxy_async_smem();
           __syncwarp();
           if (ptx::elect_one()) { ptx::tma_store_2d(tm_aux, buf_aux, col - aux_off, row0); ptx::bulk_commit_group(); }
@@ -664,6 +676,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   constexpr uint32_t kTmemCols = 2 * BN;            // two accumulators
   constexpr int kBRows = BN / CG;                   // B rows (N indices) this CTA loads
   static_assert(CG == 1 || (kBRows % kChunkElems) == 0, "pair tiles need whole 128-byte chunks of N per CTA");
+  constexpr bool kHalfRowB = B_MN && kBRows < kChunkElems;      // an MN-major B of 64 FP8 columns: rows of 64 bytes, swizzled so
+  static_assert(BN != 64 || (CG == 1 && EW == 8), "narrow tiles: single CTAs, eight epilogue warps");
+  constexpr bool kShortA = S::kShortA && !A_MN;
+  const uint32_t a_bytes = kShortA ? p.a_bytes : (uint32_t)S::kABytes, stage_bytes = a_bytes + S::kBBytes;
+  const int stages = kShortA ? (int)p.stages : S::kStages;
 
   ptx::grid_release_next();
   extern __shared__ uint8_t smem_raw[];
@@ -673,13 +690,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   const uint32_t bars = epi_base + S::kEpiBytes;
   // barrier layout (8 bytes each): full[kStages], empty[kStages], acc_full[2], acc_empty[2], drained, epi_in[2 * EW]
   auto full_bar = [&](int s) { return bars + 8u * s; };
-  auto empty_bar = [&](int s) { return bars + 8u * (S::kStages + s); };
-  auto acc_full_bar = [&](int a) { return bars + 8u * (2 * S::kStages + a); };
-  auto acc_empty_bar = [&](int a) { return bars + 8u * (2 * S::kStages + 2 + a); };
-  const uint32_t drained_bar = bars + 8u * (2 * S::kStages + 4);
-  auto epi_in_bar = [&](int w) { return bars + 8u * (2 * S::kStages + 5 + w); };   // epilogue warp w owns 2 w and 2 w + 1
-  static_assert(8 * (2 * S::kStages + 5 + 2 * EW) + 8 <= S::kBarrierBytes, "barrier area too small");
-  uint8_t* tail = smem_gen + S::kStages * S::kStageBytes + S::kEpiBytes + 8 * (2 * S::kStages + 5 + 2 * EW);
+  auto empty_bar = [&](int s) { return bars + 8u * (S::kMaxStages + s); };
+  auto acc_full_bar = [&](int a) { return bars + 8u * (2 * S::kMaxStages + a); };
+  auto acc_empty_bar = [&](int a) { return bars + 8u * (2 * S::kMaxStages + 2 + a); };
+  const uint32_t drained_bar = bars + 8u * (2 * S::kMaxStages + 4);
+  auto epi_in_bar = [&](int w) { return bars + 8u * (2 * S::kMaxStages + 5 + w); };   // epilogue warp w owns 2 w and 2 w + 1
+  static_assert(8 * (2 * S::kMaxStages + 5 + 2 * EW) + 8 <= S::kBarrierBytes, "barrier area too small");
+  uint8_t* tail = smem_gen + S::kStages * S::kStageBytes + S::kEpiBytes + 8 * (2 * S::kMaxStages + 5 + 2 * EW);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(tail);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 4);
 
@@ -691,7 +708,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   const int num_kb = (p.K + kBK - 1) / kBK;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < S::kStages; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
+    for (int s = 0; s < stages; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
     const int epi_arrivals = EPI != kEpiLegacy ? EW == 16 ? CG * 4 * (BN / 64) : CG * kEpilogueWarps : CG * kEpilogueWarps;
     for (int a = 0; a < 2; ++a) { ptx::mbar_init(acc_full_bar(a), 1); ptx::mbar_init(acc_empty_bar(a), epi_arrivals); }
     ptx::mbar_init(drained_bar, 1);
@@ -725,13 +742,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
         for (int kb = 0; kb < num_kb; ++kb) {
           ok = wait_bounded(empty_bar(stage), phase ^ 1u, abort_flag, p.status, p.wait_limit);
           if (!ok) break;
-          const uint32_t a_dst = smem_base + stage * S::kStageBytes;
-          const uint32_t b_dst = a_dst + S::kABytes;
+          const uint32_t a_dst = smem_base + stage * stage_bytes;
+          const uint32_t b_dst = a_dst + a_bytes;
           const int k0 = kb * kBK;
           if (issued == 0) ptx::grid_wait_previous();        // coordinates and barriers are ready: only the loads wait
           // bytes of the whole tile stage are counted on the (even CTA's) full barrier
           const uint32_t fb = (CG == 2) ? ptx::in_even_cta(full_bar(stage)) : full_bar(stage);
-          if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), CG * S::kStageBytes);
+          if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), CG * stage_bytes);
           auto load = [&](uint32_t dst, const void* tm, int x, int y) {
             if (BATCHED) {
               if (CG == 2) ptx::tma_load_4d_pair(dst, tm, fb, x, y, b1, b0); else ptx::tma_load_4d(dst, tm, fb, x, y, b1, b0);
@@ -745,21 +762,23 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
           } else {
             load(a_dst, &tmap_a, k0, m0);
           }
-          if (B_MN) {
+          if (B_MN && !kHalfRowB) {
 #pragma unroll
             for (int c = 0; c < kBRows / kChunkElems; ++c) load(b_dst + c * kChunkBytes, &tmap_b, n0 + c * kChunkElems, k0);
+          } else if (kHalfRowB) {
+            load(b_dst, &tmap_b, n0, k0);
           } else {
             load(b_dst, &tmap_b, k0, n0);
           }
           ++issued;
-          if (++stage == S::kStages) { stage = 0; phase ^= 1u; }
+          if (++stage == stages) { stage = 0; phase ^= 1u; }
         }
       }
       if (*abort_flag && rank == 0) {
         // Let copies that are still in flight land before the CTA gives up its shared memory.
-        const uint32_t n = issued < (uint32_t)S::kStages ? issued : (uint32_t)S::kStages;
+        const uint32_t n = issued < (uint32_t)stages ? issued : (uint32_t)stages;
         for (uint32_t i = 0; i < n; ++i) {
-          if (stage == 0) { stage = S::kStages; phase ^= 1u; }
+          if (stage == 0) { stage = stages; phase ^= 1u; }
           --stage;
           for (uint32_t it = 0; it < p.wait_limit && !ptx::mbar_try_wait(full_bar(stage), phase); ++it) {}
         }
@@ -777,13 +796,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
       // k-step to k-step only in their 14-bit start-address field, i.e. by adding a constant to the
       // low word (no carry: shared memory addresses / 16 stay below 2^14).
       const uint64_t a_desc0 = A_MN ? ptx::smem_desc_sw128(smem_base, kChunkBytes, 1024) : ptx::smem_desc_sw128(smem_base, 16, 1024);
-      const uint64_t b_desc0 = B_MN ? ptx::smem_desc_sw128(smem_base + S::kABytes, kChunkBytes, 1024)
-                                    : ptx::smem_desc_sw128(smem_base + S::kABytes, 16, 1024);
+      const uint64_t b_desc0 = kHalfRowB ? ptx::smem_desc_sw64(smem_base + a_bytes, 16, 512)
+                               : B_MN    ? ptx::smem_desc_sw128(smem_base + a_bytes, kChunkBytes, 1024)
+                                         : ptx::smem_desc_sw128(smem_base + a_bytes, 16, 1024);
       const uint32_t a_hi = (uint32_t)(a_desc0 >> 32), b_hi = (uint32_t)(b_desc0 >> 32);
       const uint32_t a_lo0 = (uint32_t)a_desc0, b_lo0 = (uint32_t)b_desc0;
-      constexpr uint32_t kStageStep = S::kStageBytes >> 4;
+      const uint32_t stage_step = stage_bytes >> 4;
       constexpr uint32_t kAStep = (A_MN ? kChunkBytes / kKSteps : 32u) >> 4;   // K-major: 32 bytes along the row
-      constexpr uint32_t kBStep = (B_MN ? kChunkBytes / kKSteps : 32u) >> 4;   // MN-major: kBK/4 rows of 128 bytes
+      constexpr uint32_t kBStep = (kHalfRowB ? kChunkBytes / 2 / kKSteps : B_MN ? kChunkBytes / kKSteps : 32u) >> 4;   // MN-major: kBK/4 rows of 128 (64) bytes
       const uint32_t idesc = p.idesc;
       for (int tile = group; ok && tile < num_tiles; tile += num_groups, ++local) {
         const uint32_t acc = local & 1u, acc_phase = (local >> 1) & 1u;
@@ -798,7 +818,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
             if (!ok) break;
           }
           ptx::tc_fence_after_sync();
-          const uint32_t a_lo = a_lo0 + stage * kStageStep, b_lo = b_lo0 + stage * kStageStep;
+          const uint32_t a_lo = a_lo0 + stage * stage_step, b_lo = b_lo0 + stage * stage_step;
 #pragma unroll
           for (int k = 0; k < kKSteps; ++k) {
             const uint64_t adesc = ((uint64_t)a_hi << 32) | (a_lo + k * kAStep);
@@ -809,7 +829,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
           }
           // stage reusable (in both CTAs of a pair) once these MMAs have read it
           if (CG == 2) ptx::mma_commit_pair(empty_bar(stage), 3); else ptx::mma_commit(empty_bar(stage));
-          if (++stage == S::kStages) { stage = 0; phase ^= 1u; }
+          if (++stage == stages) { stage = 0; phase ^= 1u; }
         }
         if (ok) {                                     // accumulator complete
           if (CG == 2) ptx::mma_commit_pair(acc_full_bar(acc), 3); else ptx::mma_commit(acc_full_bar(acc));
