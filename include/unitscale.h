@@ -127,6 +127,12 @@ us_status us_linear_bwd_x(const us_mat* G, const us_mat* W, float beta_x, const 
 us_status us_linear_bwd_w(const us_mat* X, const us_mat* G, float beta_w, const us_epilogue* ep,
                           const us_mat* dW, void* ws, size_t ws_bytes, void* stream);
 
+/* us_linear_fwd with a residual epilogue (act NONE, a skip tensor), whose output is the input of a matmul too: Yq (US_E4M3 or
+ * US_E5M2, shape of Y, alignment as for Y) receives what us_cast_fp8 at scale 1 makes of Y (F32, BF16 or F16) as stored.
+ * US_ERR_UNSUPPORTED for other epilogues and formats. */
+us_status us_linear_fwd_cast(const us_mat* X, const us_mat* W, float alpha, const us_epilogue* ep, const us_mat* Y, const us_mat* Yq,
+                             void* ws, size_t ws_bytes, void* stream);
+
 /*
  * Batched forms: count[0] x count[1] independent problems of one shape in a single launch, e.g. the
  * (sequence, head) problems of scaled dot-product attention (appendix "Unit scaling and attention":
@@ -186,6 +192,9 @@ us_status us_linear_group(int count, const us_linear_call* calls, void* ws, size
  * (all calls of a launch the same operand width) and outputs of any size are covered too; US_ERR_UNSUPPORTED remains for a
  * fused activation, mixed widths and more tiles than the work list holds (2048). */
 us_status us_linear_group_any(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, void* stream);
+/* us_linear_group_any with FP8 copies as in us_linear_fwd_cast: copies[i] (ptr NULL: none) of the output of call i, which has a skip
+ * tensor. */
+us_status us_linear_group_cast(int count, const us_linear_call* calls, const us_mat* copies, void* ws, size_t ws_bytes, void* stream);
 
 /*
  * us_ffn_hidden: both GEMMs that end in the hidden layer of the FFN block, as ONE kernel launch.
@@ -477,10 +486,18 @@ us_status us_softmax_xent_bwd(const us_mat* X, const int32_t* targets, const flo
  */
 us_status us_layer_norm_fwd(const us_mat* X, const us_mat* w, const us_mat* c, float eps, const us_mat* Y,
                             void* stream);
+/* The same with Yq (US_E4M3 or US_E5M2, shape of Y), which receives what us_cast_fp8 at scale 1 makes of Y (F32, BF16 or F16). */
+us_status us_layer_norm_fwd_cast(const us_mat* X, const us_mat* w, const us_mat* c, float eps, const us_mat* Y, const us_mat* Yq,
+                                 void* stream);
 size_t us_layer_norm_bwd_workspace_bytes(int64_t rows, int64_t cols);
 us_status us_layer_norm_bwd(const us_mat* X, const us_mat* w, const us_mat* G, float eps, float beta_x,
                             float beta_wc, const us_mat* dX, const us_mat* dw, const us_mat* dc, void* ws,
                             size_t ws_bytes, void* stream);
+
+/* us_layer_norm_bwd with such a copy dXq of dX. */
+us_status us_layer_norm_bwd_cast(const us_mat* X, const us_mat* w, const us_mat* G, float eps, float beta_x,
+                                 float beta_wc, const us_mat* dX, const us_mat* dXq, const us_mat* dw, const us_mat* dc, void* ws,
+                                 size_t ws_bytes, void* stream);
 
 /* ------------------------------------------------------------ quantisation diagnostics
  *

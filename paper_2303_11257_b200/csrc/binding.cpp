@@ -185,7 +185,8 @@ const Known kKnown[] = {
     US_CALL(us_attention_fwd), US_CALL(us_attention_bwd), US_CALL(us_attention_bwd_all), US_CALL(us_cast_fp8), US_CALL(us_cast_fp8_multi),
     US_CALL(us_cast_multi), US_CALL(us_residual_add), US_CALL(us_gelu_fwd), US_CALL(us_gelu_bwd), US_CALL(us_activation_fwd),
     US_CALL(us_activation_bwd), US_CALL(us_weighted_add), US_CALL(us_softmax_fwd), US_CALL(us_softmax_bwd), US_CALL(us_softmax_xent_fwd),
-    US_CALL(us_softmax_xent_bwd), US_CALL(us_layer_norm_fwd), US_CALL(us_layer_norm_bwd),
+    US_CALL(us_softmax_xent_bwd), US_CALL(us_layer_norm_fwd), US_CALL(us_layer_norm_bwd), US_CALL(us_linear_fwd_cast), US_CALL(us_linear_group_cast),
+    US_CALL(us_layer_norm_fwd_cast), US_CALL(us_layer_norm_bwd_cast),
 };
 constexpr size_t kCount = sizeof(kKnown) / sizeof(kKnown[0]);
 PyMethodDef g_calls[kCount];

@@ -19,6 +19,13 @@ static bool is_fp8(int dt) { return dt == US_E4M3 || dt == US_E5M2; }
 
 enum Op { kFwd, kBwdX, kBwdW };
 
+// The FP8 copy of the output of a residual epilogue.
+us_status check_copy(const us_mat* q, const us_mat* out, bool residual) {
+  if (!valid_mat(q) || q->rows != out->rows || q->cols != out->cols) return US_ERR_INVALID_ARG;
+  if (!residual || !is_fp8(q->dtype) || is_fp8(out->dtype)) return US_ERR_UNSUPPORTED;
+  return aligned16(q) ? US_OK : US_ERR_ALIGNMENT;
+}
+
 // Failure-path test settings of one call: a short wait limit, and a producer that issues no loads.
 struct WaitTest {
   uint32_t wait_limit;
@@ -28,7 +35,7 @@ struct WaitTest {
 // A, B: the two operands in call order; out [M x N].
 static us_status linear(Op op, const us_mat* A, const us_mat* B, float scale, const us_epilogue* ep, const us_mat* out,
                         void* ws, size_t ws_bytes, void* stream, const us_batch* batch = nullptr,
-                        const WaitTest* wt = nullptr, bool validate_only = false) {
+                        const WaitTest* wt = nullptr, bool validate_only = false, const us_mat* copy = nullptr) {
   if (!valid_mat(A) || !valid_mat(B) || !valid_mat(out)) return US_ERR_INVALID_ARG;
   int64_t M, N, K;
   bool shapes_ok;
@@ -74,16 +81,22 @@ static us_status linear(Op op, const us_mat* A, const us_mat* B, float scale, co
       p.skip_coef = ep->skip_coef; p.out_coef = ep->out_coef;
     }
   }
+  if (copy) {
+    const us_status s = check_copy(copy, out, p.skip != nullptr && p.act == US_ACT_NONE);
+    if (s != US_OK) return s;
+    p.aux = copy->ptr; p.aux_dt = copy->dtype; p.aux_ld = copy->ld;
+    p.aux_sectors = reinterpret_cast<uintptr_t>(copy->ptr) % 32 == 0 && copy->ld % 32 == 0;
+  }
   if (!ws || ws_bytes < us_workspace_bytes()) return US_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(ws) % 16) return US_ERR_ALIGNMENT;
   p.status = static_cast<unsigned int*>(ws);
 
-  EpiMats em{out, p.aux ? &ep->aux : nullptr, p.skip ? &ep->skip : nullptr};
+  EpiMats em{out, p.aux && !copy ? &ep->aux : nullptr, p.skip ? &ep->skip : nullptr};
   // The specialised epilogues cover the combinations of the FFN path; anything else (an activation
   // together with a skip tensor) takes the general direct-access epilogue.
   int epi = kEpiLegacy;
   if (p.act == US_ACT_NONE && !p.skip) epi = kEpiPlain;
-  else if (p.act == US_ACT_NONE) epi = kEpiSkip;
+  else if (p.act == US_ACT_NONE) epi = copy ? kEpiSkipCopy : kEpiSkip;
   else if (p.act == US_ACT_GELU && !p.skip) epi = kEpiGelu;
   else if (p.act == US_ACT_GELU_GRAD && !p.skip) epi = kEpiGeluGrad;
   BatchDesc bd;
@@ -131,6 +144,10 @@ static us_status linear(Op op, const us_mat* A, const us_mat* B, float scale, co
 extern "C" us_status us_linear_fwd(const us_mat* X, const us_mat* W, float alpha, const us_epilogue* ep,
                                    const us_mat* Y, void* ws, size_t ws_bytes, void* stream) {
   return us::linear(us::kFwd, X, W, alpha, ep, Y, ws, ws_bytes, stream);
+}
+extern "C" us_status us_linear_fwd_cast(const us_mat* X, const us_mat* W, float alpha, const us_epilogue* ep, const us_mat* Y,
+                                        const us_mat* Yq, void* ws, size_t ws_bytes, void* stream) {
+  return Yq ? us::linear(us::kFwd, X, W, alpha, ep, Y, ws, ws_bytes, stream, nullptr, nullptr, false, Yq) : US_ERR_INVALID_ARG;
 }
 extern "C" us_status us_linear_bwd_x(const us_mat* G, const us_mat* W, float beta_x, const us_epilogue* ep,
                                      const us_mat* dX, void* ws, size_t ws_bytes, void* stream) {

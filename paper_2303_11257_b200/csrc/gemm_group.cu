@@ -4,6 +4,7 @@
 #include <algorithm>
 
 #include "gemm_group.cuh"
+#include "gemm_launch.h"
 #include "host.h"
 
 namespace us {
@@ -106,25 +107,36 @@ bool deal(GroupParams& g, int es, int tile_m, int bn, int split, int units, int 
   return true;
 }
 
-template <int ES, int BN, int CG, int SPLIT>
-us_status launch_group(const GroupParams& g, cudaStream_t stream) {
-  auto kern = gemm_group_kernel<ES, BN, CG, SPLIT>;
+template <int ES, int BN, int CG, int SPLIT, bool COPY>
+us_status launch_variant(const GroupParams& g, cudaStream_t stream) {
+  auto kern = gemm_group_kernel<ES, BN, CG, SPLIT, COPY>;
   constexpr int smem = GemmSmem<BN, CG, kGroupEW>::kTotal;
   static std::atomic<uint64_t> smem_set{0};
   return host::launch(kern, &smem_set, CG * g.units, gemm_threads(kGroupEW), smem, CG, stream, g);
 }
+template <int ES, int BN, int CG, int SPLIT>
+us_status launch_group(const GroupParams& g, bool copy, cudaStream_t stream) {
+  return copy ? launch_variant<ES, BN, CG, SPLIT, true>(g, stream) : launch_variant<ES, BN, CG, SPLIT, false>(g, stream);
+}
 
-us_status group_impl(int count, const us_linear_call* calls, bool any, void* ws, size_t ws_bytes, void* stream) {
+// copies: NULL, or for each call the FP8 copy of its output (ptr NULL: none).
+us_status group_impl(int count, const us_linear_call* calls, const us_mat* copies, bool any, void* ws, size_t ws_bytes, void* stream) {
   if (count < 1 || count > kGroupMaxProblems || !calls) return count >= 1 && calls ? US_ERR_UNSUPPORTED : US_ERR_INVALID_ARG;
   if (!ws || ws_bytes < us_workspace_bytes()) return US_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(ws) % 16) return US_ERR_ALIGNMENT;
   static_assert(sizeof(GroupParams) < 32000, "kernel parameter limit");
   Shape sh[kGroupMaxProblems];
   int64_t pair_tiles = 0;
+  bool copy = false;
   for (int i = 0; i < count; ++i) {
     us_status s = check_call(&calls[i], any, &sh[i]);
     if (s != US_OK) return s;
     if (dtype_size(calls[i].a.dtype) != dtype_size(calls[0].a.dtype)) return US_ERR_UNSUPPORTED;   // one operand width per launch
+    if (copies && copies[i].ptr) {
+      s = check_copy(&copies[i], &calls[i].out, calls[i].ep.skip.ptr != nullptr);
+      if (s != US_OK) return s;
+      copy = true;
+    }
     pair_tiles += ((sh[i].M + 255) / 256) * ((sh[i].N + 255) / 256);
   }
   const int sms = host::sm_count();
@@ -154,6 +166,10 @@ us_status group_impl(int count, const us_linear_call* calls, bool any, void* ws,
     P.skip_dt = P.has_skip ? c.ep.skip.dtype : US_F32;
     P.skip_coef = P.has_skip ? c.ep.skip_coef : 0.f;
     P.out_coef = P.has_skip ? c.ep.out_coef : 1.f;
+    P.copy = copies ? static_cast<uint8_t*>(copies[i].ptr) : nullptr;
+    P.copy_ld = P.copy ? copies[i].ld : 0;
+    P.copy_dt = P.copy ? copies[i].dtype : US_E4M3;
+    P.copy_sectors = reinterpret_cast<uintptr_t>(P.copy) % 32 == 0 && P.copy_ld % 32 == 0;
     if (!make_tmap(&P.ta, &c.a, es, P.a_mn ? 128 / es : 128) || !make_tmap(&P.tb, &c.b, es, P.b_mn ? 128 / es : 128)) return US_ERR_CUDA;
     const int oes = dtype_size(c.out.dtype);
     if (!make_tmap(&P.tout, &c.out, oes, 32, std::min(128, bn / 2 / split * oes))) return US_ERR_CUDA;
@@ -164,16 +180,19 @@ us_status group_impl(int count, const us_linear_call* calls, bool any, void* ws,
   g.status = static_cast<unsigned int*>(ws);
   g.wait_limit = kWaitLimit;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (es == 1) return pair ? launch_group<1, 256, 2, 1>(g, st) : split == 2 ? launch_group<1, 128, 1, 2>(g, st) : launch_group<1, 128, 1, 1>(g, st);
-  return pair ? launch_group<2, 256, 2, 1>(g, st) : split == 2 ? launch_group<2, 128, 1, 2>(g, st) : launch_group<2, 128, 1, 1>(g, st);
+  if (es == 1) return pair ? launch_group<1, 256, 2, 1>(g, copy, st) : split == 2 ? launch_group<1, 128, 1, 2>(g, copy, st) : launch_group<1, 128, 1, 1>(g, copy, st);
+  return pair ? launch_group<2, 256, 2, 1>(g, copy, st) : split == 2 ? launch_group<2, 128, 1, 2>(g, copy, st) : launch_group<2, 128, 1, 1>(g, copy, st);
 }
 
 }  // namespace
 }  // namespace us
 
 extern "C" us_status us_linear_group(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, void* stream) {
-  return us::group_impl(count, calls, false, ws, ws_bytes, stream);
+  return us::group_impl(count, calls, nullptr, false, ws, ws_bytes, stream);
 }
 extern "C" us_status us_linear_group_any(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, void* stream) {
-  return us::group_impl(count, calls, true, ws, ws_bytes, stream);
+  return us::group_impl(count, calls, nullptr, true, ws, ws_bytes, stream);
+}
+extern "C" us_status us_linear_group_cast(int count, const us_linear_call* calls, const us_mat* copies, void* ws, size_t ws_bytes, void* stream) {
+  return copies ? us::group_impl(count, calls, copies, true, ws, ws_bytes, stream) : US_ERR_INVALID_ARG;
 }

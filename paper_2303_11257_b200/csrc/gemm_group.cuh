@@ -36,6 +36,8 @@ struct GroupProblem {
   int out_dt;
   int has_skip, skip_dt;
   float skip_coef, out_coef;
+  uint8_t* copy; int64_t copy_ld;       // an FP8 copy of the output (null: none)
+  int copy_dt, copy_sectors;            // its rows start on 32-byte boundaries
 };
 
 struct GroupParams {
@@ -55,7 +57,10 @@ constexpr int kGroupEW = 8;
 
 // SPLIT = 2 (128 x 128 tiles): two CTAs compute the same tile and each writes half of its columns, where the problems are so
 // small that half of the SMs would be idle: the epilogue of a tile takes longer than a short main loop.
-template <int ES, int BN, int CG, int SPLIT>
+//
+// COPY: some problem's output is also written as FP8 codes.  A variant of its own, because the code of the copy, never taken,
+// cost the launches without one 3 to 4 % (1000 x 528 x 2096: 15.3 to 16.0 us).
+template <int ES, int BN, int CG, int SPLIT, bool COPY>
 __global__ void __launch_bounds__(gemm_threads(kGroupEW), 1)
 gemm_group_kernel(const __grid_constant__ GroupParams g) {
   using S = GemmSmem<BN, CG, kGroupEW>;
@@ -310,7 +315,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
           if (last_slice) { release_acc(); released = true; }
           const uint32_t out_cb = (uint32_t)(out_off * out_es) >> 4;
           const uint32_t dst = buf_out + (uint32_t)(lane * out_row);
-          uint32_t held[2];
+          uint32_t held[2], copy[8];
 #pragma unroll
           for (int gi = 0; gi < 4; ++gi) {
             f32x2 x[4];
@@ -335,6 +340,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
 #pragma unroll
               for (int k = 0; k < 4; ++k)
                 unpack2(fma2(skip2, pack2(sk[2 * k], sk[2 * k + 1]), mul2(oc2, x[k])), y[2 * k], y[2 * k + 1]);
+              if (COPY && P.copy) copy_codes(P.out_dt, P.copy_dt, y, &copy[2 * gi]);
             } else {
 #pragma unroll
               for (int k = 0; k < 4; ++k) unpack2(x[k], y[2 * k], y[2 * k + 1]);
@@ -357,6 +363,8 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
               else ptx::sts128(dst + (((out_cb + (gi >> 1)) ^ out_sw) << 4), make_uint4(held[0], held[1], lo, hi));
             }
           }
+          if (COPY && skip && P.copy && row0 + lane < P.M)
+            copy_store(P.copy + (int64_t)(row0 + lane) * P.copy_ld + col, copy, P.N - col, P.copy_sectors != 0);
           if (out_off + 32 == out_box_cols || last_slice) {
             ptx::fence_proxy_async_smem();
             __syncwarp();

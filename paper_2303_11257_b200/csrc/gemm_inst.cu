@@ -86,6 +86,9 @@ static us_status pick_epilogue(const us_mat* A, const us_mat* B, const GemmParam
     if (fp8_out && epi == kEpiGelu) return launch<ES, A_MN, B_MN, BN, CG, kEpiGelu, 16>(A, B, p, em, stream);
     if (fp8_out && epi == kEpiGeluGrad) return launch<ES, A_MN, B_MN, BN, CG, kEpiGeluGrad, 16>(A, B, p, em, stream);
   }
+  if constexpr (!A_MN && B_MN) {
+    if (epi == kEpiSkipCopy) return launch<ES, A_MN, B_MN, BN, CG, kEpiSkipCopy, 8>(A, B, p, em, stream);
+  }
   switch (epi) {
     case kEpiPlain:    return launch<ES, A_MN, B_MN, BN, CG, kEpiPlain, 8>(A, B, p, em, stream);
     case kEpiGelu:     return launch<ES, A_MN, B_MN, BN, CG, kEpiGelu, 8>(A, B, p, em, stream);

@@ -41,7 +41,8 @@ struct GemmParams {
   void* out; int out_dt; int64_t out_ld;
   int act; float act_in, act_out;          // act: US_ACT_NONE, or the forward / gradient class as US_ACT_GELU / US_ACT_GELU_GRAD
   int fn;                                   // us_fn of the activation (US_FN_GELU for the GELU pair)
-  void* aux; int aux_dt; int64_t aux_ld;
+  void* aux; int aux_dt; int64_t aux_ld;   // pre-activation; kEpiSkipCopy: the FP8 copy of the output
+  int aux_sectors;                          // the copy's rows start on 32-byte boundaries
   const void* skip; int skip_dt; int64_t skip_ld; float skip_coef, out_coef;
   unsigned int* status;
   uint32_t wait_limit;                      // polls a bounded wait makes before it gives up (kWaitLimit unless a test shortens it)
@@ -66,6 +67,7 @@ enum EpiKind {
   kEpiGelu = 1,      // + scaled GELU, optionally keeping the 16-bit pre-activation
   kEpiGeluGrad = 2,  // + scaled GELU gradient from the stored pre-activation
   kEpiSkip = 3,      // + weighted skip tensor (residual)
+  kEpiSkipCopy = 5,  // the same and an FP8 copy of the output (forward layout only: its code, never taken, costs kEpiSkip 3 %)
   kEpiLegacy = 4     // any other combination: direct global accesses, runtime switches
 };
 constexpr uint32_t kWaitLimit = 1u << 22;
@@ -231,6 +233,32 @@ struct EpiCtx {
   int warp, lane, rank, group, num_groups, num_tiles;
 };
 
+// Four more codes of a lane's FP8 copy: eight results as the output format dt stores them, rounded once more.
+__device__ __forceinline__ void copy_codes(int dt, int copy_dt, const float (&y)[8], uint32_t* codes) {
+  float r[8];
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) {
+    const float2 v = dt == US_BF16 ? unpack_bf16x2(pack_bf16x2(y[i], y[i + 1])) : dt == US_F16 ? unpack_f16x2(pack_f16x2(y[i], y[i + 1])) : make_float2(y[i], y[i + 1]);
+    r[i] = v.x; r[i + 1] = v.y;
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    codes[i] = copy_dt == US_E5M2 ? cvt_fp8x4<true>(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]) : cvt_fp8x4<false>(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+}
+// A lane's 32 codes to its row, of which cols columns exist.  The rows start on 16-byte boundaries (sectors: on 32-byte ones).
+__device__ __forceinline__ void copy_store(uint8_t* dst, const uint32_t (&codes)[8], int cols, bool sectors) {
+  if (cols >= 32 && sectors) {
+    ptx::stg256(dst, codes);
+  } else if (cols >= 32) {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(codes[0], codes[1], codes[2], codes[3]);
+    reinterpret_cast<uint4*>(dst)[1] = make_uint4(codes[4], codes[5], codes[6], codes[7]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      if (i < cols) dst[i] = (uint8_t)(codes[i >> 2] >> (8 * (i & 3)));
+  }
+}
+
 // Bytes per row of an output box of the eight-warp epilogue.
 __host__ __device__ constexpr int out_row_bytes(int bn, int es) { return bn / 2 * es < 128 ? bn / 2 * es : 128; }
 
@@ -250,7 +278,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
   const int q = c.warp & 3, half = (c.warp - 2) >> 2;       // lane quarter; which group of kWarpCols columns
   if (half >= BN / kWarpCols) return;                       // more warps than column groups: the rest sit out
   const int lane = c.lane;
-  constexpr int in_kind = EPI == kEpiGeluGrad ? 1 : (EPI == kEpiSkip ? 2 : 0);
+  constexpr int in_kind = EPI == kEpiGeluGrad ? 1 : (EPI == kEpiSkip || EPI == kEpiSkipCopy ? 2 : 0);
   const int in_dt = in_kind == 1 ? p.aux_dt : p.skip_dt;
   const int in_es = in_kind ? dtype_size(in_dt) : 4;
   const CUtensorMap* tm_in = in_kind == 1 ? tm_aux : tm_skip;
@@ -365,6 +393,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
         const uint32_t aux_cb = (uint32_t)(aux_off * 2) >> 4, out_cb = (uint32_t)(out_off * out_es) >> 4;
         const uint32_t dst = buf_out + out_row_off;
         uint32_t held[2];                                    // first half of a 16-byte chunk of FP8 codes
+        uint32_t copy[8];                                    // the FP8 copy of this lane's 32 columns
         // Eight values at a time run through the whole chain (scale, kept pre-activation, activation,
         // residual, rounding, staging store), so that the different execution pipes overlap.
 #pragma unroll
@@ -409,7 +438,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
                 y[2 * k] = act_grad_scaled(p.fn, h.x, a, p.act_in, p.act_out); y[2 * k + 1] = act_grad_scaled(p.fn, h.y, b, p.act_in, p.act_out);
               }
             }
-          } else if (EPI == kEpiSkip) {
+          } else if (in_kind == 2) {
             float sk[8];
             if (in_dt == US_F32) {
               sk[0] = __uint_as_float(raw[2 * g].x); sk[1] = __uint_as_float(raw[2 * g].y);
@@ -431,6 +460,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
 #pragma unroll
             for (int k = 0; k < 4; ++k) unpack2(x[k], y[2 * k], y[2 * k + 1]);
           }
+          if (EPI == kEpiSkipCopy) copy_codes(p.out_dt, p.aux_dt, y, &copy[2 * g]);
           // ---- rounding to the output format and staging store of these eight values
           if (p.out_dt == US_F32) {
             ptx::sts128(dst + (((out_cb + 2 * g) ^ out_sw) << 4),
@@ -453,6 +483,8 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
             }
           }
         }
+        if (EPI == kEpiSkipCopy && row0 + lane < p.M)
+          copy_store(static_cast<uint8_t*>(p.aux) + (int64_t)(row0 + lane) * p.aux_ld + col, copy, p.N - col, p.aux_sectors != 0);
         // ---- boxes completed by this slice go out
         if (aux_out && (aux_off + 32 == kAuxCols || last_slice)) {
           ptx::fence_proxy_async_smem();

@@ -16,6 +16,9 @@ struct EpiMats {
   const us_mat* skip;
 };
 
+// Whether q can take the FP8 copy of a residual epilogue's output.
+us_status check_copy(const us_mat* q, const us_mat* out, bool residual);
+
 // Batch description of one launch: nb0 x nb1 problems; element strides of each matrix between
 // consecutive problems of the outer (index 0) and inner (index 1) batch dimension.
 struct BatchDesc {

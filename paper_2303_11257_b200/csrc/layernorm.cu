@@ -28,11 +28,27 @@ struct LnArgs {
   const void* w; int w_dt;                  // [cols]
   const void* c; int c_dt;                  // [cols], forward only
   void* out; int out_dt; int64_t out_ld;    // Y (forward) or dX (backward)
+  void* q; int q_dt; int64_t q_ld;          // an FP8 copy of it (null: none)
   float* partial;                           // backward: [gridDim.x][2][cols]
   int64_t rows; int cols;
   int vec_ok;                               // all row starts 16-byte aligned and cols % 8 == 0
   float eps, beta_x;
 };
+
+// Eight results: stored, and the stored values once more in FP8 where the caller wants them as the operand of a matmul.
+__device__ __forceinline__ void ln_store8(const LnArgs& a, int64_t row, int col, bool vec, const float (&t)[8]) {
+  store8(a.out, a.out_dt, row * a.out_ld, col, a.cols, vec, t);
+  if (a.q) {
+    float r[8];
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+      const float2 v = a.out_dt == US_BF16 ? unpack_bf16x2(pack_bf16x2(t[i], t[i + 1])) : a.out_dt == US_F16 ? unpack_f16x2(pack_f16x2(t[i], t[i + 1]))
+                                                                                                        : make_float2(t[i], t[i + 1]);
+      r[i] = v.x; r[i + 1] = v.y;
+    }
+    store8(a.q, a.q_dt, row * a.q_ld, col, a.cols, vec, r);
+  }
+}
 
 // Mean and reciprocal standard deviation of a row given as nch chunks per lane.
 template <int NCH>
@@ -82,7 +98,7 @@ __global__ void __launch_bounds__(kLnThreads) ln_fwd_kernel(const LnArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * kLnWarps + (threadIdx.x >> 5);
   if (row >= a.rows) return;
-  const int64_t x_off = row * a.x_ld, out_off = row * a.out_ld;
+  const int64_t x_off = row * a.x_ld;
   const bool vec = a.vec_ok != 0;
   const int nch = NCH > 0 ? NCH : (a.cols + 255) / 256;
   float x[NCH > 0 ? NCH : 1][8];
@@ -103,7 +119,7 @@ __global__ void __launch_bounds__(kLnThreads) ln_fwd_kernel(const LnArgs a) {
     load8(a.c, a.c_dt, 0, col, a.cols, vec, 0.f, b);
 #pragma unroll
     for (int i = 0; i < 8; ++i) t[i] = fmaf(w[i], (t[i] - mu) * rstd, b[i]);
-    store8(a.out, a.out_dt, out_off, col, a.cols, vec, t);
+    ln_store8(a, row, col, vec, t);
   }
 }
 
@@ -129,7 +145,7 @@ __global__ void __launch_bounds__(kLnThreads) ln_bwd_kernel(const LnArgs a) {
     __syncwarp();
   }
   for (int64_t row = (int64_t)blockIdx.x * nw + warp; row < a.rows; row += (int64_t)gridDim.x * nw) {
-    const int64_t x_off = row * a.x_ld, g_off = row * a.g_ld, out_off = row * a.out_ld;
+    const int64_t x_off = row * a.x_ld, g_off = row * a.g_ld;
     float x[NCH > 0 ? NCH : 1][8], u[NCH > 0 ? NCH : 1][8];
     float mu, rstd;
     row_stats<NCH>(a, x_off, lane, nch, x, mu, rstd);
@@ -184,7 +200,7 @@ __global__ void __launch_bounds__(kLnThreads) ln_bwd_kernel(const LnArgs a) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) d[i] = k * (g[i] * w[i] - mean_u - (t[i] - mu) * rstd * mean_ux);
       }
-      store8(a.out, a.out_dt, out_off, col, a.cols, vec, d);
+      ln_store8(a, row, col, vec, d);
     }
   }
   // ---- combine the CTA's warps in warp order; one partial row (G xhat sums, then G sums) per CTA
@@ -263,7 +279,6 @@ __global__ void __launch_bounds__(kLnThreads, NCH <= 4 ? 3 : 2) ln_fwd16_kernel(
     for (int c = 0; c < NCH; ++c) unpack16x8(cur[c], a.x_dt, x[c]);
     float mu, rstd;
     stats_regs<NCH>(x, lane, a.cols, a.eps, mu, rstd);
-    const int64_t out_off = row * a.out_ld;
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
       const int col = (c * 32 + lane) * 8;
@@ -275,7 +290,7 @@ __global__ void __launch_bounds__(kLnThreads, NCH <= 4 ? 3 : 2) ln_fwd16_kernel(
         float t[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) t[i] = fmaf(w[i], (x[c][i] - mu) * rstd, b[i]);
-        store8(a.out, a.out_dt, out_off, col, a.cols, true, t);
+        ln_store8(a, row, col, true, t);
       }
     }
 #pragma unroll
@@ -466,7 +481,6 @@ __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
     const float mean_ux = warp_sum(lo + hi) * inv_n;
     const float k = a.beta_x * rstd;
     const f32x2 k2 = splat2(k), c0 = splat2(-k * mean_u), c1 = splat2(-k * mean_ux);
-    const int64_t out_off = row * a.out_ld;
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
       const int col = (c * 32 + lane) * 8;
@@ -480,7 +494,7 @@ __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
           const f32x2 t = fma2(mul2(g_pair(c, j), w2[j]), k2, c0);
           unpack2(fma2(xp[c][j], c1, t), d[2 * j], d[2 * j + 1]);
         }
-        store8(a.out, a.out_dt, out_off, col, a.cols, true, d);
+        ln_store8(a, row, col, true, d);
       }
     }
   }
@@ -550,6 +564,8 @@ __global__ void __launch_bounds__(32 * kLnReduceGroups) ln_bwd_reduce_kernel(con
 static bool ln_rows_aligned(const us_mat* m) {
   return reinterpret_cast<uintptr_t>(m->ptr) % 16 == 0 && (m->ld * dtype_size(m->dtype)) % 16 == 0;
 }
+// Eight codes of an FP8 copy are stored at once.
+static bool copy_rows_aligned(const us_mat* q) { return !q || (reinterpret_cast<uintptr_t>(q->ptr) % 8 == 0 && q->ld % 8 == 0); }
 static bool is_float_in(int dt) { return dt == US_F32 || dt == US_BF16 || dt == US_F16; }
 
 static us_status check_matrix(const us_mat* m, const us_mat* like, bool input) {
@@ -560,6 +576,13 @@ static us_status check_matrix(const us_mat* m, const us_mat* like, bool input) {
   if (input ? !is_float_in(m->dtype) : !(m->dtype >= US_F32 && m->dtype <= US_E5M2)) return US_ERR_UNSUPPORTED;
   if (m->ptr && reinterpret_cast<uintptr_t>(m->ptr) % dtype_size(m->dtype)) return US_ERR_ALIGNMENT;
   return US_OK;
+}
+// The FP8 copy of a result that is not FP8 itself.
+static us_status check_copy(const us_mat* q, const us_mat* of) {
+  if (!q) return US_OK;
+  const us_status s = check_matrix(q, of, false);
+  if (s != US_OK) return s;
+  return (q->dtype == US_E4M3 || q->dtype == US_E5M2) && is_float_in(of->dtype) ? US_OK : US_ERR_UNSUPPORTED;
 }
 // A parameter vector: 1 x cols.
 static us_status check_vector(const us_mat* v, int64_t cols, bool input) {
@@ -580,16 +603,12 @@ static int ln_bwd_grid(int64_t rows, int warps = kLnWarps, int per_sm = 2) {
 }
 constexpr int kLnFastWarps = 4, kLnFastPerSm = 3;   // the 16-bit backward kernel: three CTAs of four warps per SM
 
-}  // namespace us
-
-using namespace us;
-
-extern "C" us_status us_layer_norm_fwd(const us_mat* X, const us_mat* w, const us_mat* c, float eps, const us_mat* Y,
-                                       void* stream) {
+static us_status ln_fwd(const us_mat* X, const us_mat* w, const us_mat* c, float eps, const us_mat* Y, const us_mat* Yq, void* stream) {
   us_status s = check_matrix(X, nullptr, true);
   if (s == US_OK) s = check_matrix(Y, X, false);
   if (s == US_OK) s = check_vector(w, X->cols, true);
   if (s == US_OK) s = check_vector(c, X->cols, true);
+  if (s == US_OK) s = check_copy(Yq, Y);
   if (s != US_OK) return s;
   if (!(eps >= 0.f)) return US_ERR_INVALID_ARG;
   if (X->rows == 0 || X->cols == 0) return US_OK;
@@ -597,8 +616,9 @@ extern "C" us_status us_layer_norm_fwd(const us_mat* X, const us_mat* w, const u
   a.x = X->ptr; a.x_dt = X->dtype; a.x_ld = X->ld;
   a.w = w->ptr; a.w_dt = w->dtype; a.c = c->ptr; a.c_dt = c->dtype;
   a.out = Y->ptr; a.out_dt = Y->dtype; a.out_ld = Y->ld;
+  if (Yq) { a.q = Yq->ptr; a.q_dt = Yq->dtype; a.q_ld = Yq->ld; }
   a.rows = X->rows; a.cols = (int)X->cols; a.eps = eps; a.beta_x = 1.f;
-  a.vec_ok = ln_rows_aligned(X) && ln_rows_aligned(Y) && ln_rows_aligned(w) && ln_rows_aligned(c) && X->cols % 8 == 0;
+  a.vec_ok = ln_rows_aligned(X) && ln_rows_aligned(Y) && ln_rows_aligned(w) && ln_rows_aligned(c) && copy_rows_aligned(Yq) && X->cols % 8 == 0;
   const int64_t grid64 = (a.rows + kLnWarps - 1) / kLnWarps;
   if (grid64 > 0x7fffffff) return US_ERR_INVALID_ARG;
   const int grid = (int)grid64, nch = (a.cols + 255) / 256;
@@ -622,38 +642,33 @@ extern "C" us_status us_layer_norm_fwd(const us_mat* X, const us_mat* w, const u
   return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
 }
 
-extern "C" size_t us_layer_norm_bwd_workspace_bytes(int64_t rows, int64_t cols) {
-  if (rows <= 0 || cols <= 0) return 0;
-  const int g0 = ln_bwd_grid(rows), g1 = ln_bwd_grid(rows, kLnFastWarps, kLnFastPerSm);
-  const int grid = g0 > g1 ? g0 : g1;                // whichever kernel the call takes
-  return (size_t)(grid > 0 ? grid : 1) * 2 * (size_t)cols * sizeof(float);
-}
-
-extern "C" us_status us_layer_norm_bwd(const us_mat* X, const us_mat* w, const us_mat* G, float eps, float beta_x,
-                                       float beta_wc, const us_mat* dX, const us_mat* dw, const us_mat* dc, void* ws,
-                                       size_t ws_bytes, void* stream) {
+static us_status ln_bwd(const us_mat* X, const us_mat* w, const us_mat* G, float eps, float beta_x, float beta_wc, const us_mat* dX,
+                        const us_mat* dXq, const us_mat* dw, const us_mat* dc, void* ws, size_t ws_bytes, void* stream) {
   us_status s = check_matrix(X, nullptr, true);
   if (s == US_OK) s = check_matrix(G, X, true);
   if (s == US_OK) s = check_matrix(dX, X, false);
   if (s == US_OK) s = check_vector(w, X->cols, true);
   if (s == US_OK) s = check_vector(dw, X->cols, false);
   if (s == US_OK) s = check_vector(dc, X->cols, false);
+  if (s == US_OK) s = check_copy(dXq, dX);
   if (s != US_OK) return s;
   if (!(eps >= 0.f)) return US_ERR_INVALID_ARG;
   if (X->cols > kLnMaxBwdCols) return US_ERR_UNSUPPORTED;
   if (X->cols == 0) return US_OK;
   const int grid = ln_bwd_grid(X->rows > 0 ? X->rows : 1);
   if (grid <= 0) return US_ERR_CUDA;
-  if (!ws || ws_bytes < us_layer_norm_bwd_workspace_bytes(X->rows > 0 ? X->rows : 1, X->cols)) return US_ERR_WORKSPACE;
+  if (!ws || ws_bytes < ::us_layer_norm_bwd_workspace_bytes(X->rows > 0 ? X->rows : 1, X->cols)) return US_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(ws) % 16) return US_ERR_ALIGNMENT;
   LnArgs a{};
   a.x = X->ptr; a.x_dt = X->dtype; a.x_ld = X->ld;
   a.g = G->ptr; a.g_dt = G->dtype; a.g_ld = G->ld;
   a.w = w->ptr; a.w_dt = w->dtype;
   a.out = dX->ptr; a.out_dt = dX->dtype; a.out_ld = dX->ld;
+  if (dXq) { a.q = dXq->ptr; a.q_dt = dXq->dtype; a.q_ld = dXq->ld; }
   a.partial = static_cast<float*>(ws);
   a.rows = X->rows; a.cols = (int)X->cols; a.eps = eps; a.beta_x = beta_x;
-  a.vec_ok = ln_rows_aligned(X) && ln_rows_aligned(G) && ln_rows_aligned(dX) && ln_rows_aligned(w) && X->cols % 8 == 0;
+  a.vec_ok = ln_rows_aligned(X) && ln_rows_aligned(G) && ln_rows_aligned(dX) && ln_rows_aligned(w) &&
+             copy_rows_aligned(dXq) && X->cols % 8 == 0;
   const int nch = (a.cols + 255) / 256;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int nparts = grid;
@@ -693,4 +708,34 @@ extern "C" us_status us_layer_norm_bwd(const us_mat* X, const us_mat* w, const u
   const int rgrid = (2 * a.cols + 31) / 32;
   return host::launch(ln_bwd_reduce_kernel, nullptr, rgrid, 32 * kLnReduceGroups, 0, 1, st, a.partial, nparts, a.cols, beta_wc, dw->ptr,
                       dw->dtype, dc->ptr, dc->dtype);
+}
+
+}  // namespace us
+
+using namespace us;
+
+extern "C" size_t us_layer_norm_bwd_workspace_bytes(int64_t rows, int64_t cols) {
+  if (rows <= 0 || cols <= 0) return 0;
+  const int g0 = ln_bwd_grid(rows), g1 = ln_bwd_grid(rows, kLnFastWarps, kLnFastPerSm);
+  const int grid = g0 > g1 ? g0 : g1;                // whichever kernel the call takes
+  return (size_t)(grid > 0 ? grid : 1) * 2 * (size_t)cols * sizeof(float);
+}
+
+extern "C" us_status us_layer_norm_fwd(const us_mat* X, const us_mat* w, const us_mat* c, float eps, const us_mat* Y,
+                                       void* stream) {
+  return ln_fwd(X, w, c, eps, Y, nullptr, stream);
+}
+extern "C" us_status us_layer_norm_fwd_cast(const us_mat* X, const us_mat* w, const us_mat* c, float eps, const us_mat* Y,
+                                            const us_mat* Yq, void* stream) {
+  return Yq ? ln_fwd(X, w, c, eps, Y, Yq, stream) : US_ERR_INVALID_ARG;
+}
+extern "C" us_status us_layer_norm_bwd(const us_mat* X, const us_mat* w, const us_mat* G, float eps, float beta_x,
+                                       float beta_wc, const us_mat* dX, const us_mat* dw, const us_mat* dc, void* ws,
+                                       size_t ws_bytes, void* stream) {
+  return ln_bwd(X, w, G, eps, beta_x, beta_wc, dX, nullptr, dw, dc, ws, ws_bytes, stream);
+}
+extern "C" us_status us_layer_norm_bwd_cast(const us_mat* X, const us_mat* w, const us_mat* G, float eps, float beta_x,
+                                            float beta_wc, const us_mat* dX, const us_mat* dXq, const us_mat* dw, const us_mat* dc,
+                                            void* ws, size_t ws_bytes, void* stream) {
+  return dXq ? ln_bwd(X, w, G, eps, beta_x, beta_wc, dX, dXq, dw, dc, ws, ws_bytes, stream) : US_ERR_INVALID_ARG;
 }

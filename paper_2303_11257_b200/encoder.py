@@ -117,9 +117,9 @@ class UnitScaledEncoderLayer:
     @property
     def kernel_launches(self) -> int:
         """Kernel launches of one step while the grouped launches hold its tiles: launches_per_step less one for each
-        projection, with layer norms the three GEMMs that end the FFN block's backward pass as one, and the fused backward pass of
-        attention as one."""
-        return self.launches_per_step - 2 - (2 if self.norm is not None and self.ffn.grouped else 0) - (2 if self.whole_bwd else 0)
+        projection, with layer norms the three GEMMs that end the FFN block's backward pass as one, the fused backward pass of
+        attention as one, and the casts that their tensors' producers make."""
+        return self.launches_per_step - 2 - (2 if self.norm is not None and self.ffn.grouped else 0) - (2 if self.whole_bwd else 0) - (2 if self.norm is None else 3)
 
     def _heads(self, M, which):
         """Problem (0, 0) of a [T x 3d] matrix: rows of the first sequence, columns of head 0 of Q / K / V."""
@@ -147,9 +147,10 @@ class UnitScaledEncoderLayer:
         coef = (self.c_skip, self.c_branch)
         MAIN = self.MAIN
 
-        def norm_bwd(X, w, G, dX, dw, dc):
+        # a tensor that is the operand of a matmul too leaves its producer in FP8 as well
+        def norm_bwd(X, w, G, dX, dXq, dw, dc):
             g = p.slot(G) if isinstance(G, str) else p.mat(G)
-            return L.Call("us_layer_norm_bwd", p.mat(X), p.slot(w), g, self.eps, 1.0, self.beta_ln, p.mat(dX), L._vec(dw), L._vec(dc),
+            return L.Call("us_layer_norm_bwd_cast", p.mat(X), p.slot(w), g, self.eps, 1.0, self.beta_ln, p.mat(dX), p.mat(dXq), L._vec(dw), L._vec(dc),
                           self.ln_ws.data_ptr(), self.ln_ws.numel())
 
         # the first pass issues each call as it is laid out, so nothing is made before the call that needs it
@@ -166,23 +167,23 @@ class UnitScaledEncoderLayer:
             yield MAIN, p.batched("us_linear_bwd_x_batched", Q, K, sc["alpha_s"], self.S[:s], self.bt["scores"], ws)
             yield MAIN, L.Call("us_softmax_fwd", p.mat(self.S), sc["sm"], p.mat(self.P))
             yield MAIN, p.batched("us_linear_fwd_batched", P, V, sc["alpha_c"], C_h, self.bt["ctx"], ws)
-        yield MAIN, p.linear("us_linear_fwd", self.Cq, self.Wo_q, sc["alpha_o"], self.U1 if post else self.R1, ws, p.residual("X", coef))
         if post:
-            yield MAIN, L.Call("us_layer_norm_fwd", p.mat(self.U1), p.slot("w1"), p.slot("c1"), self.eps, p.mat(self.R1))
-            for c in f.plan_forward(p, self.R1):
+            yield MAIN, p.linear("us_linear_fwd", self.Cq, self.Wo_q, sc["alpha_o"], self.U1, ws, p.residual("X", coef))
+            yield MAIN, L.Call("us_layer_norm_fwd_cast", p.mat(self.U1), p.slot("w1"), p.slot("c1"), self.eps, p.mat(self.R1), p.mat(f.Xq))
+            for c in f.plan_forward(p, self.R1, cast_x=False):
                 yield MAIN, c
             yield MAIN, L.Call("us_layer_norm_fwd", p.mat(f.R), p.slot("w2"), p.slot("c2"), self.eps, p.mat(self.R2))
-            yield MAIN, norm_bwd(f.R, "w2", "G", self.dU2, self.dln[2], self.dln[3])
-            for c in f.plan_backward(p, self.dU2):
+            yield MAIN, norm_bwd(f.R, "w2", "G", self.dU2, f.Gq, self.dln[2], self.dln[3])
+            for c in f.plan_backward(p, self.dU2, cast_g=False):
                 yield MAIN, c
-            yield MAIN, norm_bwd(self.U1, "w1", f.dX, self.dU1, self.dln[0], self.dln[1])
+            yield MAIN, norm_bwd(self.U1, "w1", f.dX, self.dU1, self.g1q, self.dln[0], self.dln[1])
             g1 = self.dU1
         else:
-            yield MAIN, f._plan_cast(p, self.R1, f.Xq)
-            for c in f.plan_gemms(p, self.R1, "G"):
+            yield MAIN, L.Call("us_linear_fwd_cast", p.mat(self.Cq), p.mat(self.Wo_q), sc["alpha_o"], p.residual("X", coef), p.mat(self.R1),
+                               p.mat(f.Xq), *tail)
+            for c in f.plan_gemms(p, self.R1, "G", self.g1q):
                 yield MAIN, c
             g1 = f.dX
-        yield MAIN, L.Call("us_cast_fp8", p.mat(g1), 1.0, p.mat(self.g1q))
         yield MAIN, p.group([(L.US_OP_BWD_W, self.Cq, self.g1q, sc["beta_w"], self.dWo, None, None),
                              (L.US_OP_BWD_X, self.g1q, self.Wo_q, sc["beta_o"], self.dC, None, None)], ws)
         dQ, dK, dV = (self._heads(self.dQKV, i) for i in range(3))

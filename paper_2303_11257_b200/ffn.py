@@ -145,20 +145,21 @@ class UnitScaledFFN:
     def _plan_backward_from_cast(self, p):
         return self.plan_backward(p, "G", cast_g=False)
 
-    def plan_gemms(self, p, X, G):
-        """step_from_casts() as prepared calls; X, G: the skip inputs, tensors or names of inputs."""
+    def plan_gemms(self, p, X, G, dX_copy=None):
+        """step_from_casts() as prepared calls; X, G: the skip inputs, tensors or names of inputs; dX_copy: takes dX in FP8."""
         sc = self.sc
         yield L.Call("us_ffn_hidden_any", p.mat(self.Xq), p.mat(self.W1q), sc.alpha1, p.mat(self.Gq), p.mat(self.W2q), sc.beta_x2,
                      sc.s_in, sc.alpha_g, sc.beta_g, L._TORCH_DTYPES[self.H.dtype], p.mat(self.H) if self._writes_h() else None,
                      p.mat(self.Aq), p.mat(self.dHq), self.ws.data_ptr(), self.ws.numel())
         w2, w1, x1 = self._plan_backward_entries(G)
-        yield p.group([w2, w1, (L.US_OP_FWD, self.Aq, self.W2q, sc.alpha2, self.R, X, self._c), x1], self.ws)
+        yield p.group([w2, w1, (L.US_OP_FWD, self.Aq, self.W2q, sc.alpha2, self.R, X, self._c), x1], self.ws, {3: dX_copy} if dX_copy is not None else None)
 
-    def plan_forward(self, p, X):
-        """forward() as prepared calls."""
+    def plan_forward(self, p, X, cast_x=True):
+        """forward() as prepared calls.  cast_x = False: self.Xq already holds q(X)."""
         sc = self.sc
         ep1 = L.epilogue(act=L.US_ACT_GELU, act_in_scale=sc.s_in, act_out_scale=sc.alpha_g, aux=self.H)
-        yield self._plan_cast(p, X, self.Xq)
+        if cast_x:
+            yield self._plan_cast(p, X, self.Xq)
         yield p.linear("us_linear_fwd", self.Xq, self.W1q, sc.alpha1, self.Aq, self.ws, ep1)
         yield p.linear("us_linear_fwd", self.Aq, self.W2q, sc.alpha2, self.R, self.ws, p.residual(X, self._c))
 

@@ -106,6 +106,12 @@ def _load() -> C.CDLL:
     lib.us_linear_group.argtypes = [C.c_int, C.POINTER(us_linear_call), V, SZ, V]
     lib.us_linear_group_any.argtypes = lib.us_linear_group.argtypes
     lib.us_linear_group.restype = lib.us_linear_group_any.restype = C.c_int
+    lib.us_linear_fwd_cast.argtypes = [MP, MP, F, EP, MP, MP, V, SZ, V]
+    lib.us_linear_group_cast.argtypes = [C.c_int, C.POINTER(us_linear_call), MP, V, SZ, V]
+    lib.us_layer_norm_fwd_cast.argtypes = [MP, MP, MP, F, MP, MP, V]
+    lib.us_layer_norm_bwd_cast.argtypes = [MP, MP, MP, F, F, F, MP, MP, MP, MP, V, SZ, V]
+    for name in ("us_linear_fwd_cast", "us_linear_group_cast", "us_layer_norm_fwd_cast", "us_layer_norm_bwd_cast"):
+        getattr(lib, name).restype = C.c_int
     lib.us_ffn_hidden.argtypes = [MP, MP, F, MP, MP, F, F, F, F, C.c_int32, MP, MP, MP, V, SZ, V]
     lib.us_ffn_hidden_any.argtypes = lib.us_ffn_hidden.argtypes
     lib.us_ffn_hidden.restype = lib.us_ffn_hidden_any.restype = C.c_int
@@ -341,9 +347,9 @@ class Plan:
             ep.skip = self.mat(skip)
         return ep
 
-    def group(self, entries, ws):
+    def group(self, entries, ws, copies=None):
         """us_linear_group_any over (op, a, b, scale, out, skip or None, (skip_coef, out_coef)); as single launches where
-        there are more tiles than its work list holds."""
+        there are more tiles than its work list holds.  copies: FP8 copies of the outputs (us_linear_group_cast), by entry."""
         arr = (us_linear_call * len(entries))()
         for c, (op, a, b, scale, out, skip, coef) in zip(arr, entries):
             c.op, c.a, c.b, c.scale, c.out, c.ep.out_coef = op, self.mat(a), self.mat(b), scale, self.mat(out), 1.0
@@ -354,8 +360,19 @@ class Plan:
                     self.slot(skip, c.ep.skip)
                 else:
                     c.ep.skip = self.mat(skip)
-        return Call("us_linear_group_any", len(entries), arr, ws.data_ptr(), ws.numel(),
-                    instead=((US_ERR_UNSUPPORTED,), lambda stream: linear_each(arr, ws, stream)))
+        if not copies:
+            return Call("us_linear_group_any", len(entries), arr, ws.data_ptr(), ws.numel(),
+                        instead=((US_ERR_UNSUPPORTED,), lambda stream: linear_each(arr, ws, stream)))
+        cp = (us_mat * len(entries))()
+        for i, t in copies.items():
+            cp[i] = self.mat(t)
+
+        def each(stream):
+            linear_each(arr, ws, stream)
+            for i in copies:
+                _check("us_cast_fp8", _entry("us_cast_fp8")(arr[i].out, 1.0, cp[i], stream))
+
+        return Call("us_linear_group_cast", len(entries), arr, cp, ws.data_ptr(), ws.numel(), instead=((US_ERR_UNSUPPORTED,), each))
 
     def linear(self, name, a, b, scale, out, ws, ep=None):
         return Call(name, self.mat(a), self.mat(b), scale, ep, self.mat(out), ws.data_ptr(), ws.numel())

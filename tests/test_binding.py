@@ -53,3 +53,22 @@ def test_unchanged_compares_objects_and_addresses():
     at = tuple(t.data_ptr() for t in own)
     assert _binding.unchanged(own, own, at)
     assert not _binding.unchanged((F32, F8.clone()), own, at) and not _binding.unchanged(own, own, (at[0], at[1] + 16)) and not _binding.unchanged(own[:1], own, at)
+
+
+def test_fp8_copies_are_validated_before_any_launch():
+    """Statuses of the entry points that leave an FP8 copy (1 invalid argument, 2 unsupported, 3 alignment); fake device addresses."""
+    M = lambda addr, dt, r, c, ld=None: L.us_mat(addr, dt, r, c, ld or c)
+    X, W, Y = M(0x10000, L.US_E4M3, 64, 32), M(0x20000, L.US_E4M3, 32, 48), M(0x30000, L.US_BF16, 64, 48)
+    ep, no = L.us_epilogue(), L.us_epilogue()
+    ep.skip, ep.skip_coef, ep.out_coef = M(0x40000, L.US_BF16, 64, 48), 0.5, 0.5
+    fwd = lambda e, y, q: _binding.calls["us_linear_fwd_cast"](X, W, 1.0, e, y, q, 0x60000, 256, 0)
+    good = M(0x50000, L.US_E4M3, 64, 48)
+    assert fwd(ep, Y, None) == 1 and fwd(ep, Y, M(0x50000, L.US_E4M3, 64, 32)) == 1
+    assert fwd(no, Y, good) == 2 and fwd(None, Y, good) == 2                     # no skip tensor
+    assert fwd(ep, Y, M(0x50000, L.US_BF16, 64, 48)) == 2                        # the copy is FP8 ...
+    assert fwd(ep, M(0x30000, L.US_E5M2, 64, 48), good) == 2                     # ... of something that is not
+    assert fwd(ep, Y, M(0x50008, L.US_E4M3, 64, 48)) == 3
+    v = M(0x70000, L.US_F32, 1, 48)
+    norm = lambda y, q: _binding.calls["us_layer_norm_fwd_cast"](M(0x10000, L.US_BF16, 64, 48), v, v, 1e-5, y, q, 0)
+    assert norm(Y, None) == 1 and norm(Y, M(0x50000, L.US_E4M3, 64, 32)) == 1 and norm(Y, M(0x50000, L.US_BF16, 64, 48)) == 2
+    assert norm(M(0x30000, L.US_E5M2, 64, 48), good) == 2
