@@ -88,10 +88,11 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
   uint8_t* gen = smem_raw + (base - ptx::smem_addr(smem_raw));
   const uint32_t q_s = base + S::kQ, xch_s = base + S::kX, bars = base + S::kBars;
   // Tiles of the CTA's whole run are numbered n = 0, 1, ...; group n mod 2 works on tile n.  Barriers of tile n: per group
-  // (phase n / 2), row sums by n mod 4 (phase n / 4), slots by n mod kSlots; bar_q and bar_xfree once per tile; bar_v,
-  // bar_k and bar_acc by problem mod 2.
+  // (phase n / 2), row sums by n mod 4 (phase n / 4), slots by n mod kSlots; bar_q once per tile; bar_v, bar_k and bar_acc by
+  // problem mod 2.
   auto bar_at = [&](int i) { return bars + 8u * (uint32_t)i; };
-  const uint32_t bar_q = bar_at(0), bar_xfree = bar_at(1), bar_drained = bar_at(2);
+  const uint32_t bar_q = bar_at(0), bar_drained = bar_at(35);
+  auto bar_xfree = [&](int n) { return bar_at(1 + (n & 1)); };
   auto bar_v = [&](int i) { return bar_at(3 + (i & 1)); };
   auto bar_k = [&](int i) { return bar_at(5 + (i & 1)); };
   auto bar_acc = [&](int i) { return bar_at(7 + (i & 1)); };
@@ -139,7 +140,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
     }
     for (int i = 0; i < 4; ++i) ptx::mbar_init(bar_sum(i), kGrWarps);
     for (int i = 0; i < S::kSlots; ++i) ptx::mbar_init(bar_p(i), 1);
-    ptx::mbar_init(bar_xfree, (uint32_t)(cl * kGrParts));   // the cluster's warps that finish dQ have added up a tile
+    for (int i = 0; i < 2; ++i) ptx::mbar_init(bar_xfree(i), (uint32_t)(cl * kGrParts));   // the cluster's warps that finish dQ have added up a tile
     *abort_flag = 0;
     ptx::mbar_init_fence();
   }
@@ -301,7 +302,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
         }
         if (i == 4 / cl - 1) {
           __syncwarp();                                        // every lane has added what it read: the pieces may be overwritten
-          if (lane < cl) ptx::mbar_arrive_relaxed_cluster(ptx::in_cta(bar_xfree, (uint32_t)lane));
+          if (lane < cl) ptx::mbar_arrive_relaxed_cluster(ptx::in_cta(bar_xfree(n), (uint32_t)lane));
         }
         const int row = q0 + (rank + i * cl) * 32 + lane;
         if (row < a.s_q) {
@@ -434,7 +435,8 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
 #pragma unroll
           for (int i = 0; i < 32; ++i) v[i] = 0.f;
         }
-        if (n > 0 && !wait(bar_xfree, (uint32_t)(n - 1) & 1u)) break;
+        // (a wait by parity is sound only for a waiter that has seen every earlier phase: hence a barrier for the tiles of each group)
+        if (n > 0 && !wait(bar_xfree(n - 1), half_phase(n - 1))) break;
         const uint32_t owner = (uint32_t)(q % cl), bar = ptx::in_cta(bar_xch(n), owner);
         const uint32_t dst = ptx::in_cta(xch_s + (uint32_t)(((q / cl) * kGrParts + part) * cl + rank) * 4096u + (uint32_t)lane * 16u, owner);
 #pragma unroll

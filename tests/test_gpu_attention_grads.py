@@ -77,3 +77,31 @@ def test_gradients_do_not_depend_on_the_stored_scores_gradient_and_repeat(fmt):
     for other in runs[1:]:
         for a, b in zip(runs[0][1:], other[1:]):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("s_k", [200, 512])
+@pytest.mark.parametrize("fmt", ["bf16", "e4m3"])
+def test_long_runs_of_a_cluster(s_k, fmt):
+    """Every cluster of two (four) CTAs walks 16 to 50 tiles of 128 queries, so that the area its CTAs exchange parts of dQ in is reused
+    as often: dQ against the float64 product of the device's own dS and K, and the same bits from every launch."""
+    from paper_2303_11257_b200 import lib as L
+    n, s_q, gfmt = 320, 600, "e5m2" if fmt == "e4m3" else fmt
+    gen = torch.Generator(device="cuda").manual_seed(33)
+    ld = (s_k + 15) // 16 * 16
+    rand = lambda r, f: torch.randn(n * r, 64, generator=gen, device="cuda").to(U.TORCH_OF[f])
+    dC, Q, K, V = rand(s_q, gfmt), rand(s_q, fmt), rand(s_k, fmt), rand(s_k, fmt)
+    P = torch.zeros(n * s_q, ld, device="cuda")
+    P[:, :s_k] = s_k * torch.softmax(torch.randn(n * s_q, s_k, generator=gen, device="cuda"), 1)
+    P, dS = P.to(U.TORCH_OF[fmt])[:, :s_k], U.empty(n * s_q, s_k, gfmt, ld)
+    ws, first = L.new_workspace(), None
+    bt = L.attention_bwd_all_batch((1, n), (1, s_q * 64), (1, s_q * ld), (1, s_q * 64), (1, s_k * 64), (1, s_k * 64), (1, s_q * ld), (1, s_q * 64),
+                                   (1, s_k * 64), (1, s_k * 64))
+    for _ in range(6):
+        out = [torch.zeros(n * r, 64, device="cuda") for r in (s_q, s_k, s_k)]
+        L.us_attention_bwd_all(dC[:s_q], P[:s_q], Q[:s_q], K[:s_k], V[:s_k], 0.125, s_k, s_k, 0.25, 0.125, 0.5, dS[:s_q], *(t[:r] for t, r in zip(out, (s_q, s_k, s_k))), bt, ws)
+        assert L.us_workspace_status(ws) == 0
+        first = first or out
+        assert all(torch.equal(a, b) for a, b in zip(first, out))
+    wide = lambda t, r: t.float().double().reshape(n, r, -1)
+    ref = 0.25 * wide(dS, s_q) @ wide(K, s_k)
+    assert bool(((first[0].double().reshape(n, s_q, 64) - ref).abs() <= TOL * max(1.0, float(ref.abs().max()))).all())
