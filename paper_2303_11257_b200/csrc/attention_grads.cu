@@ -72,6 +72,7 @@ struct AttnGradParams {
   uint32_t idesc_dp, idesc_dv, idesc_dk, idesc_dq;
   unsigned int* status;
   uint32_t wait_limit;
+  uint32_t zero;            // 0; not a constant to the compiler (see the hand-over of the exchange area)
 };
 
 // BF16: 16-bit operands are BF16 (else F16).  CLUSTER: launched in clusters of two or four CTAs (more than 128 keys); without one the
@@ -157,6 +158,8 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
   auto head_desc = [&](uint32_t addr) { return F8 ? ptx::smem_desc_sw64(addr, 16, 512) : ptx::smem_desc_sw128(addr, 16, 1024); };
   constexpr uint32_t kHeadStep = 2048u >> 4;
   auto wait1 = [&](uint32_t bar, uint32_t parity) { return wait_bounded(bar, parity, abort_flag, a.status, a.wait_limit); };
+  // for what other CTAs of the cluster have written or handed back
+  auto wait1_cluster = [&](uint32_t bar, uint32_t parity) { return wait_bounded<CLUSTER>(bar, parity, abort_flag, a.status, a.wait_limit); };
 
   if (warp == 0) {
     if (ptx::elect_one()) {
@@ -285,7 +288,8 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
       int q0, b1, b0;
       coords(n, q0, b1, b0);
       if (part == 0 && lane == 0) ptx::mbar_expect_tx(bar_xch(n), 4u * kGrParts * 4096u);      // 4 / cl quarters x cl senders
-      if (!__all_sync(0xffffffffu, wait1(bar_xch(n), half_phase(n)))) break;
+      if (!__all_sync(0xffffffffu, wait1_cluster(bar_xch(n), half_phase(n)))) break;
+      uint32_t seen = 0;
       for (int i = 0; i < 4 / cl; ++i) {
         const uint32_t buf = xch_s + (uint32_t)((i * kGrParts + part) * cl) * 4096u + (uint32_t)lane * 16u;
         float v[32];
@@ -300,9 +304,15 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
             v[4 * j + 2] += __uint_as_float(o.z); v[4 * j + 3] += __uint_as_float(o.w);
           }
         }
+#pragma unroll
+        for (int j = 0; j < 32; ++j) seen |= __float_as_uint(v[j]);
         if (i == 4 / cl - 1) {
-          __syncwarp();                                        // every lane has added what it read: the pieces may be overwritten
-          if (lane < cl) ptx::mbar_arrive_relaxed_cluster(ptx::in_cta(bar_xfree(n), (uint32_t)lane));
+          // The pieces may be overwritten.  The arrivals are ordered behind the reads of all lanes by a dependency: their address
+          // contains every value that was read (and a zero that only the host knows to be one), so they cannot be made before the
+          // last of these has come, and the partners' stores follow from the arrivals.  A release at cluster scope orders the same and
+          // waits for the stores to global memory too: 104 -> 123 us at 16 x 16 x 512, 57 -> 63 at 32 x 16 x 256, 16 bits.
+          const uint32_t none = __reduce_or_sync(0xffffffffu, seen) & a.zero;
+          if (lane < cl) ptx::mbar_arrive_relaxed_cluster(ptx::in_cta(bar_xfree(n), (uint32_t)lane) + none);
         }
         const int row = q0 + (rank + i * cl) * 32 + lane;
         if (row < a.s_q) {
@@ -338,6 +348,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
       }
     };
     auto wait = [&](uint32_t bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, wait1(bar, parity)); };
+    auto wait_cluster = [&](uint32_t bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, wait1_cluster(bar, parity)); };
 #pragma unroll 1
     for (int n = group; n < steps; n += 2) {
       const uint32_t ph = half_phase(n);
@@ -390,7 +401,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
           ptx::mbar_arrive(bar_sum(n));
         }
       }
-      if (!wait(bar_sum(n), (uint32_t)(n >> 2) & 1u)) break;
+      if (!wait_cluster(bar_sum(n), (uint32_t)(n >> 2) & 1u)) break;
       const volatile float* sums = reinterpret_cast<const volatile float*>(gen + S::kS) + set + r;      // [rank][part][row]
       float total = 0.f;
       for (int k = 0; k < cl; ++k) total += sums[k * kGrParts * 128] + sums[k * kGrParts * 128 + 128];
@@ -436,7 +447,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
           for (int i = 0; i < 32; ++i) v[i] = 0.f;
         }
         // (a wait by parity is sound only for a waiter that has seen every earlier phase: hence a barrier for the tiles of each group)
-        if (n > 0 && !wait(bar_xfree(n - 1), half_phase(n - 1))) break;
+        if (n > 0 && !wait_cluster(bar_xfree(n - 1), half_phase(n - 1))) break;
         const uint32_t owner = (uint32_t)(q % cl), bar = ptx::in_cta(bar_xch(n), owner);
         const uint32_t dst = ptx::in_cta(xch_s + (uint32_t)(((q / cl) * kGrParts + part) * cl + rank) * 4096u + (uint32_t)lane * 16u, owner);
 #pragma unroll

@@ -117,11 +117,12 @@ __device__ __forceinline__ void tile_batch(const GemmParams& p, int tile, int& b
 
 // Bounded mbarrier wait.  Returns false if the CTA is aborting (this wait or another one timed out).
 // (Each attempt already suspends the thread in hardware for a while, so polling costs few issue
-// slots: pausing between attempts made no measurable difference.)
+// slots: pausing between attempts made no measurable difference.)  CLUSTER: also acquires what other CTAs of the cluster have released.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                              unsigned int* status, uint32_t limit) {
   for (uint32_t it = 0; it < limit; ++it) {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
+    if (CLUSTER ? ptx::mbar_try_wait_cluster(bar, parity) : ptx::mbar_try_wait(bar, parity)) return true;
     if ((it & 63u) == 63u && *abort_flag) return false;
   }
   *abort_flag = 1;

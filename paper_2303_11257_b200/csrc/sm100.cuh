@@ -50,6 +50,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// The same with acquire at cluster scope, for phases that other CTAs of the cluster complete.
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // ------------------------------------------------------------------ overlap with neighbouring kernels of the stream
 // grid_wait_previous returns once the previous kernel has finished and its writes are visible.  grid_release_next lets the
 // next kernel of the stream take free SMs from now on (it waits, in its own grid_wait_previous, until this grid has
@@ -194,13 +207,13 @@ __device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank) {
   return r;
 }
 // Asynchronous stores to a CTA's shared memory, counted in bytes on an mbarrier of that CTA (both shared::cluster addresses): the
-// data is there for whoever has seen the barrier's phase complete.  Only in kernels launched in clusters.  (An arrival with release
-// at cluster scope also waits for the thread's earlier stores to global memory: some 3000 cycles in a kernel that writes results all the time.)
+// data is there for whoever has seen the barrier's phase complete (mbar_try_wait_cluster).  Only in kernels launched in clusters.
 __device__ __forceinline__ void st_async128(uint32_t addr, const float* v, uint32_t bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
                ::"r"(addr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar) : "memory");
 }
-// An arrival on an mbarrier of the cluster that orders nothing.
+// An arrival on an mbarrier of the cluster that orders nothing but what its address depends on.  (One with release at cluster scope also
+// waits for the thread's earlier stores to global memory: some 3000 cycles in a kernel that writes results all the time.)
 __device__ __forceinline__ void mbar_arrive_relaxed_cluster(uint32_t bar) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
