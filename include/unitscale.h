@@ -432,6 +432,14 @@ us_status us_attention_bwd_all(const us_mat* dC, const us_mat* P, const us_mat* 
                                const us_mat* dQ, const us_mat* dK, const us_mat* dV, const us_attention_bwd_all_batch* batch,
                                void* ws, size_t ws_bytes, void* stream);
 
+/* us_test_attention_bwd_all_starved: us_test_linear_fwd_starved for the kernel of us_attention_bwd_all (all factors but
+ * softmax_alpha 1): CTA number `rank` of every cluster loads dC for its first `tile` tiles of 128 queries only, so that its waits and
+ * then those of its partners run out with the exchanges between them under way. */
+us_status us_test_attention_bwd_all_starved(const us_mat* dC, const us_mat* P, const us_mat* Q, const us_mat* K, const us_mat* V,
+                                            float softmax_alpha, const us_mat* dS, const us_mat* dQ, const us_mat* dK,
+                                            const us_mat* dV, const us_attention_bwd_all_batch* batch, void* ws, size_t ws_bytes,
+                                            unsigned int wait_limit, int rank, int tile, void* stream);
+
 /* ------------------------------------------------------------ scaled softmax
  *
  * Row-wise scaled softmax and its gradient (table "Table of unit scaling factors", row softmax:

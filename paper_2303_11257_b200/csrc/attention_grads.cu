@@ -25,7 +25,7 @@
 //
 // Every wait is on an mbarrier and bounded, remote arrivals included, and no role waits at a hardware barrier between the
 // start and the end, so a wait that runs out (in any CTA of a cluster) only makes the others' waits run out too; the
-// cluster then meets at its last barrier with all copies landed.
+// cluster then meets at its last barrier, its own copies landed, and a CTA that gave up waits for what its partners had sent it.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -41,8 +41,10 @@ namespace {
 constexpr int kGrWarps = 8, kGrParts = 2;                 // softmax warps of a group; per TMEM lane quarter
 // warp 0: MMA issue; warp 1: TMA and TMEM owner; two groups of softmax warps; in a cluster, two warps that finish dQ
 constexpr int gr_threads(bool cluster) { return 64 + 2 * 32 * kGrWarps + (cluster ? 64 : 0); }
+constexpr int kGrPieces = 4 * kGrParts;                      // parts of dQ that a CTA gets per tile: 4 / (cluster size) quarters from each CTA, by column half
 constexpr int kGrKeys = 128, kGrMaxCluster = kAttnMaxKeys / kGrKeys;
 constexpr uint32_t kGrBlock = 128 * 128;                  // 128 query rows x 128 bytes of P / dS
+constexpr unsigned int kStatusNotLanded = 2;              // beside kStatusTimeout: stores of a partner did not come in
 constexpr uint32_t kColAcc = 256, kColDk = 64;            // sums of problem i: columns 256 + 128 (i mod 2): dV, then dK
 
 // Shared memory.  A tile of P is one block of FP8 or two of 16 bits; a slot holds a tile.
@@ -55,7 +57,8 @@ struct GradSmem {
   static constexpr uint32_t kExchange = 32 * 1024;                      // parts of dQ: eight warp-sized pieces of 4 KB
   static constexpr uint32_t kSums = 4 * kGrMaxCluster * kGrParts * 128 * 4;   // row sums by tile mod 4, rank and part
   static constexpr uint32_t kV = 0, kK = kHead, kDc = 2 * kHead, kQ = 4 * kHead, kP = 5 * kHead, kX = kP + kSlots * kSlot,
-                            kS = kX + kExchange, kBars = kS + kSums, kTotal = kBars + 512 + 1024 /* alignment */;
+                            kS = kX + kExchange, kBars = kS + kSums, kSent = kBars + 512,
+                            kTotal = kSent + kGrMaxCluster * 2 * kGrWarps * 8 + 16 + 1024 /* alignment */;
   static_assert(kTotal <= 232448, "shared memory of an SM");
 };
 
@@ -72,6 +75,7 @@ struct AttnGradParams {
   uint32_t idesc_dp, idesc_dv, idesc_dk, idesc_dq;
   unsigned int* status;
   uint32_t wait_limit;
+  int stall_rank, stall_tile;   // test hook: this CTA of every cluster loads dC up to this tile only (-1: none), so that the waits run out
   uint32_t zero;            // 0; not a constant to the compiler (see the hand-over of the exchange area)
 };
 
@@ -113,6 +117,11 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
   auto half_phase = [&](int n) { return (uint32_t)(n >> 1) & 1u; };
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + S::kBars + 288);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gen + S::kBars + 292);
+  // What the cluster's softmax warps have sent this CTA, in tiles of their group: row sums and parts of dQ, [rank][warp][2]; behind it the
+  // tiles whose parts were expected.  Written at the end, for a CTA that gave up.
+  constexpr int kSenders = 2 * kGrWarps;
+  auto sent_at = [&](int from, int w) { return (uint32_t)((from * kSenders + w) * 8); };
+  constexpr uint32_t kExpected = kGrMaxCluster * kSenders * 8;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cl = CLUSTER ? (int)ptx::cluster_nctarank() : 1, rank = CLUSTER ? (int)ptx::cluster_ctarank() : 0;
@@ -235,13 +244,19 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
         if (!F8) ptx::tma_load_4d(slot(n) + kGrBlock, &tp, bar_p(n), key0 + kBlockKeys, q0, b1, b0);
       };
       int n_p = 0, n_dc = 0, n_q = 0, n_v = 0, n_k = 0;      // loads asked for
+      const int stall = rank == a.stall_rank ? a.stall_tile : 0x7fffffff;
+      auto load_dc = [&](int n) {
+        if (n >= stall) return;
+        load(dc_s(n), &tdc, bar_dc(n), -1, n);
+        ++n_dc;
+      };
       auto load_v = [&]() { load(v_s(n_v), &tv, bar_v(n_v), key0, n_v * a.q_tiles); ++n_v; };      // of the next problem
       auto load_k = [&]() { load(k_s(n_k), &tk, bar_k(n_k), key0, n_k * a.q_tiles); ++n_k; };
       if (steps > 0) {
-        load(dc_s(0), &tdc, bar_dc(0), -1, 0); ++n_dc;
+        load_dc(0);
         load_v();
         load_p(n_p++);
-        if (steps > 1) { load(dc_s(1), &tdc, bar_dc(1), -1, 1); ++n_dc; load_p(n_p++); }
+        if (steps > 1) { load_dc(1); load_p(n_p++); }
         load_k();
         load(q_s, &tq, bar_q, -1, 0); ++n_q;
         if (ahead == 2 && my_problems > 1) { load_v(); load_k(); }
@@ -254,7 +269,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
           load_v();
         }
         if (!wait1(bar_dv(n), half_phase(n))) break;         // ... and dC of this tile
-        if (n + 2 < steps) { load(dc_s(n), &tdc, bar_dc(n), -1, n + 2); ++n_dc; }
+        if (n + 2 < steps) load_dc(n + 2);
         if (!wait1(bar_ds(n), half_phase(n))) break;
         if (a.store_ds) {
           int q0, b1, b0;
@@ -284,10 +299,12 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
     // ------------------------------------------------------------------ dQ of this CTA's lane quarters (in a cluster)
     // The exchange area: by quarter, part and sender, pieces of 32 rows x 32 columns, a lane's 16-byte piece i at 512 i.
     const int part = warp - (2 + 2 * kGrWarps);
+    int expected = 0;
     for (int n = 0; n < steps; ++n) {
       int q0, b1, b0;
       coords(n, q0, b1, b0);
-      if (part == 0 && lane == 0) ptx::mbar_expect_tx(bar_xch(n), 4u * kGrParts * 4096u);      // 4 / cl quarters x cl senders
+      if (part == 0 && lane == 0) ptx::mbar_expect_tx(bar_xch(n), kGrPieces * 4096u);
+      ++expected;
       if (!__all_sync(0xffffffffu, wait1_cluster(bar_xch(n), half_phase(n)))) break;
       uint32_t seen = 0;
       for (int i = 0; i < 4 / cl; ++i) {
@@ -323,6 +340,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
         }
       }
     }
+    if (part == 0 && lane == 0) *reinterpret_cast<volatile int*>(gen + S::kSent + kExpected) = expected;
   } else {
     // ------------------------------------------------------------------ softmax gradient, dQ, dK, dV
     // Warp (group, q, part): query rows 32 q .. + 31 of a tile, one per lane; the 32-key chunks part and part + 2 of the CTA's
@@ -334,6 +352,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
     constexpr int kVals = F8 ? 16 : 8;
     const int c_end = blocks * kPerBlock;
     const uint32_t row_off = (uint32_t)r * 128u, sw = (uint32_t)(r & 7);
+    uint32_t sent_sums = 0, sent_dq = 0;
     auto values = [&](const uint4& raw, float (&pv)[16]) {
       const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
@@ -401,6 +420,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
           ptx::mbar_arrive(bar_sum(n));
         }
       }
+      ++sent_sums;
       if (!wait_cluster(bar_sum(n), (uint32_t)(n >> 2) & 1u)) break;
       const volatile float* sums = reinterpret_cast<const volatile float*>(gen + S::kS) + set + r;      // [rank][part][row]
       float total = 0.f;
@@ -452,6 +472,7 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
         const uint32_t dst = ptx::in_cta(xch_s + (uint32_t)(((q / cl) * kGrParts + part) * cl + rank) * 4096u + (uint32_t)lane * 16u, owner);
 #pragma unroll
         for (int i = 0; i < 8; ++i) ptx::st_async128(dst + 512u * i, &v[4 * i], bar);
+        ++sent_dq;
       } else if (q0 + r < a.s_q) {
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] *= a.beta_q;
@@ -486,12 +507,56 @@ attention_grads_kernel(const __grid_constant__ CUtensorMap tdc, const __grid_con
         }
       }
     }
+    if constexpr (CLUSTER) {
+      if (lane < cl) ptx::st_cluster_v2(ptx::in_cta(base + S::kSent + sent_at(rank, warp - 2), (uint32_t)lane), sent_sums, sent_dq);
+    }
   }
   ptx::tc_fence_before_sync();
   __syncthreads();
   if (CLUSTER) ptx::cluster_sync();                          // no CTA leaves while a partner may still signal it
-  if (CLUSTER && *abort_flag)                                // ... or has stores under way to it that nobody waited for: they land
-    for (const long long t = clock64(); clock64() - t < 50000;) {}
+  if constexpr (CLUSTER) {
+    if (*abort_flag && threadIdx.x == 0) {
+      // Stores that the partners had under way when this CTA gave up land before it leaves.  The senders of a group are at most one
+      // tile apart (each tile of one needs something of the tile before from all): of the first tile that not all have sent, what is
+      // missing is made up for here, so that its phase completes with the last of the stores that were issued.
+      const volatile uint32_t* sent = reinterpret_cast<const volatile uint32_t*>(gen + S::kSent);
+      const int begun = *reinterpret_cast<volatile int*>(gen + S::kSent + kExpected);
+      auto land = [&](uint32_t bar, int phase) {
+        uint32_t it = 0;
+        while (it < a.wait_limit && !ptx::mbar_try_wait_cluster(bar, (uint32_t)phase & 1u)) ++it;
+        if (it == a.wait_limit) atomicOr(a.status, kStatusNotLanded);
+      };
+      for (int g = 0; g < 2; ++g) {
+        for (int what = 0; what < 2; ++what) {                 // row sums, parts of dQ
+          auto for_senders = [&](auto&& f) {                   // from, tiles sent; of dQ those that send it to this CTA
+            for (int from = 0; from < cl; ++from)
+              for (int w = g * kGrWarps; w < (g + 1) * kGrWarps; ++w)
+                if (what == 0 || ((w + 2) & 3) % cl == rank) f(from, sent[sent_at(from, w) / 4 + what]);
+          };
+          uint32_t least = 0xffffffffu;
+          for_senders([&](int, uint32_t tiles) { least = min(least, tiles); });
+          int own = 0, others = 0;                             // that have sent tile number `least` of the group
+          for_senders([&](int from, uint32_t tiles) { if (tiles > least) ++(what == 0 && from == rank ? own : others); });
+          const int n = g + 2 * (int)least;                    // that tile
+          if (what == 0) {
+            if (least > 0) land(bar_sum(n - 2), (n - 2) >> 2);
+            if (others == 0) continue;
+            // the own warp that brings the bytes to expect is the one of quarter `rank`, part 0
+            if (sent[sent_at(rank, g * kGrWarps + ((rank + 2) & 3)) / 4] > least) ptx::mbar_complete_tx(bar_sum(n), (uint32_t)((cl - 1) * kGrWarps - others) * 128u);
+            else ptx::mbar_expect_only(bar_sum(n), (uint32_t)others * 128u);
+            for (; own < kGrWarps; ++own) ptx::mbar_arrive(bar_sum(n));
+            land(bar_sum(n), n >> 2);
+          } else {
+            const int last = others > 0 ? n : n - 2, parts = others > 0 ? others : kGrPieces;       // the last tile with parts under way
+            if (last < 0) continue;
+            if (last < begun) ptx::mbar_complete_tx(bar_xch(last), (uint32_t)(kGrPieces - parts) * 4096u);
+            else ptx::mbar_expect_tx(bar_xch(last), (uint32_t)parts * 4096u);
+            land(bar_xch(last), last >> 1);
+          }
+        }
+      }
+    }
+  }
   if (warp == 1) { ptx::tc_fence_after_sync(); ptx::tmem_dealloc(tmem, 512); }
 }
 
@@ -510,14 +575,15 @@ us_status pick_grads(const CUtensorMap* t, const AttnGradParams& a, cudaStream_t
   return a.s_k > kGrKeys ? launch_grads<F8, BF16, true>(t, a, stream) : launch_grads<F8, BF16, false>(t, a, stream);
 }
 
-}  // namespace
-}  // namespace us
+// Failure-path test settings of one call.
+struct Stall {
+  uint32_t wait_limit;
+  int rank, tile;
+};
 
-extern "C" us_status us_attention_bwd_all(const us_mat* dC, const us_mat* P, const us_mat* Q, const us_mat* K, const us_mat* V,
-                                          float beta_p, float softmax_alpha, float softmax_beta, float beta_q, float beta_k,
-                                          float beta_v, const us_mat* dS, const us_mat* dQ, const us_mat* dK, const us_mat* dV,
-                                          const us_attention_bwd_all_batch* batch, void* ws, size_t ws_bytes, void* stream) {
-  using namespace us;
+us_status bwd_all(const us_mat* dC, const us_mat* P, const us_mat* Q, const us_mat* K, const us_mat* V, float beta_p, float softmax_alpha,
+                  float softmax_beta, float beta_q, float beta_k, float beta_v, const us_mat* dS, const us_mat* dQ, const us_mat* dK,
+                  const us_mat* dV, const us_attention_bwd_all_batch* batch, void* ws, size_t ws_bytes, void* stream, const Stall& test) {
   if (!dC || !P || !Q || !K || !V || !dQ || !dK || !dV || !batch) return US_ERR_INVALID_ARG;
   if (dS && !dS->ptr) dS = nullptr;
   const int64_t* cnt = batch->count;
@@ -580,7 +646,7 @@ extern "C" us_status us_attention_bwd_all(const us_mat* dC, const us_mat* P, con
   a.idesc_dk = make_idesc(grad, act, true, true, 128, 64);
   a.idesc_dq = make_idesc(grad, act, false, true, 128, 64);
   a.status = static_cast<unsigned int*>(ws);
-  a.wait_limit = kWaitLimit;
+  a.wait_limit = test.wait_limit; a.stall_rank = test.rank; a.stall_tile = test.tile;
 
   CUtensorMap t[6];                                        // dC, Q, K, V, P, dS
   const int row = f8 ? 64 : 128;
@@ -592,4 +658,22 @@ extern "C" us_status us_attention_bwd_all(const us_mat* dC, const us_mat* P, con
   if (dS && !attn_tmap(&t[5], dS, batch->ds_stride, cnt, 128, es)) return US_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   return f8 ? pick_grads<true, false>(t, a, st) : bf16 ? pick_grads<false, true>(t, a, st) : pick_grads<false, false>(t, a, st);
+}
+
+}  // namespace
+}  // namespace us
+
+extern "C" us_status us_attention_bwd_all(const us_mat* dC, const us_mat* P, const us_mat* Q, const us_mat* K, const us_mat* V,
+                                          float beta_p, float softmax_alpha, float softmax_beta, float beta_q, float beta_k,
+                                          float beta_v, const us_mat* dS, const us_mat* dQ, const us_mat* dK, const us_mat* dV,
+                                          const us_attention_bwd_all_batch* batch, void* ws, size_t ws_bytes, void* stream) {
+  return us::bwd_all(dC, P, Q, K, V, beta_p, softmax_alpha, softmax_beta, beta_q, beta_k, beta_v, dS, dQ, dK, dV, batch, ws, ws_bytes, stream,
+                     {us::kWaitLimit, -1, 0});
+}
+extern "C" us_status us_test_attention_bwd_all_starved(const us_mat* dC, const us_mat* P, const us_mat* Q, const us_mat* K, const us_mat* V,
+                                                       float softmax_alpha, const us_mat* dS, const us_mat* dQ, const us_mat* dK,
+                                                       const us_mat* dV, const us_attention_bwd_all_batch* batch, void* ws, size_t ws_bytes,
+                                                       unsigned int wait_limit, int rank, int tile, void* stream) {
+  if (wait_limit < 1 || wait_limit > (1u << 16) || rank < 0 || tile < 0) return US_ERR_INVALID_ARG;
+  return us::bwd_all(dC, P, Q, K, V, 1.f, softmax_alpha, 1.f, 1.f, 1.f, 1.f, dS, dQ, dK, dV, batch, ws, ws_bytes, stream, {wait_limit, rank, tile});
 }

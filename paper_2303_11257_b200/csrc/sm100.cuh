@@ -218,6 +218,18 @@ __device__ __forceinline__ void mbar_arrive_relaxed_cluster(uint32_t bar) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// Two words to a CTA of the cluster (a shared::cluster address); ordered by the next cluster_sync.
+__device__ __forceinline__ void st_cluster_v2(uint32_t addr, uint32_t a, uint32_t b) {
+  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+// The bytes that the phase under way of one of this CTA's mbarriers waits for: more of them without an arrival, or some made up for.
+__device__ __forceinline__ void mbar_expect_only(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_complete_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
 // ------------------------------------------------------------------ tensor memory
 // Executed by one full warp.  Writes the base address of `cols` columns (power of two >= 32)
 // to the shared-memory word at `dst`.

@@ -96,7 +96,8 @@ def _load() -> C.CDLL:
     lib.us_attention_bwd.argtypes = [MP, MP, MP, MP, F, F, F, F, MP, MP, C.POINTER(us_attention_bwd_batch), V, SZ, V]
     lib.us_attention_bwd.restype = C.c_int
     lib.us_attention_bwd_all.argtypes = [MP] * 5 + [F] * 6 + [MP] * 4 + [C.POINTER(us_attention_bwd_all_batch), V, SZ, V]
-    lib.us_attention_bwd_all.restype = C.c_int
+    lib.us_test_attention_bwd_all_starved.argtypes = [MP] * 5 + [F] + [MP] * 4 + [C.POINTER(us_attention_bwd_all_batch), V, SZ, C.c_uint, C.c_int, C.c_int, V]
+    lib.us_attention_bwd_all.restype = lib.us_test_attention_bwd_all_starved.restype = C.c_int
     lib.us_linear_fwd_static_ws.argtypes = [MP, MP, F, EP, MP, C.POINTER(C.c_void_p), V]
     lib.us_linear_fwd_static_ws.restype = C.c_int
     lib.us_linear_fwd_check.argtypes = [MP, MP, EP, MP, V, SZ]
@@ -542,6 +543,13 @@ def us_attention_bwd_all(dC, P, Q, K, V, beta_p, softmax_alpha, softmax_beta, be
     """The whole backward pass of attention in one launch; dS may be None (not stored)."""
     _check("us_attention_bwd_all", _entry("us_attention_bwd_all")(dC, P, Q, K, V, beta_p, softmax_alpha, softmax_beta, beta_q, beta_k, beta_v, dS, dQ, dK, dV, bt, ws, ws, _stream(stream)))
     return dQ, dK, dV
+
+
+def us_test_attention_bwd_all_starved(dC, P, Q, K, V, softmax_alpha, dS, dQ, dK, dV, bt, ws, wait_limit: int, rank: int, tile: int, stream=None):
+    """us_test_linear_fwd_starved for the kernel of us_attention_bwd_all: CTA `rank` of a cluster gets dC for `tile` tiles only."""
+    _check("us_test_attention_bwd_all_starved",
+           _lib.us_test_attention_bwd_all_starved(*(C.byref(mat(t)) for t in (dC, P, Q, K, V)), softmax_alpha, *(C.byref(mat(t)) for t in (dS, dQ, dK, dV)),
+                                                  C.byref(bt), ws.data_ptr(), ws.numel() * ws.element_size(), wait_limit, rank, tile, _stream(stream)))
 
 
 def us_linear_fwd_static_ws(X, W, alpha, Y, ep=None, stream=None) -> int:

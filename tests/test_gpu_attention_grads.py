@@ -105,3 +105,30 @@ def test_long_runs_of_a_cluster(s_k, fmt):
     wide = lambda t, r: t.float().double().reshape(n, r, -1)
     ref = 0.25 * wide(dS, s_q) @ wide(K, s_k)
     assert bool(((first[0].double().reshape(n, s_q, 64) - ref).abs() <= TOL * max(1.0, float(ref.abs().max()))).all())
+
+
+@pytest.mark.parametrize("fmt,s_k,cl", [("bf16", 100, 1), ("bf16", 200, 2), ("e4m3", 256, 2), ("fp16", 400, 4), ("e4m3", 512, 4)])
+def test_a_cluster_that_gives_up_drains_what_its_ctas_send_each_other(fmt, s_k, cl):
+    """One CTA of the cluster gets dC for some tiles only: every wait runs out, the status word says so and, with one cluster in the
+    launch, nothing else (2 would be stores of a partner that did not come in); the same call without the stall is right afterwards."""
+    from paper_2303_11257_b200 import lib as L, synth
+    s_q, gfmt, ld = 900, "e5m2" if fmt == "e4m3" else fmt, (s_k + 15) // 16 * 16
+    t = lambda i, r, f: U.to_device(synth.normal(34, i, (r, 64)), f)
+    dC, Q, K, V = t(0, s_q, gfmt), t(1, s_q, fmt), t(2, s_k, fmt), t(3, s_k, fmt)
+    P, dS = U.to_device(np.abs(synth.normal(34, 4, (s_q, s_k))), fmt, ld), U.empty(s_q, s_k, gfmt, ld)
+    ws, bt = L.new_workspace(), L.attention_bwd_all_batch((1, 1), *[(1, 1)] * 9)
+    call = lambda: [U.empty(r, 64, "f32") for r in (s_q, s_k, s_k)]
+    good = call()
+    L.us_attention_bwd_all(dC, P, Q, K, V, 1.0, s_k, 1.0, 1.0, 1.0, 1.0, dS, *good, bt, ws)
+    assert L.us_workspace_status(ws) == 0
+    for rank in range(cl):
+        for tile in (0, 1, 2, 3, 5):
+            L.us_test_attention_bwd_all_starved(dC, P, Q, K, V, s_k, dS, *call(), bt, ws, wait_limit=2000, rank=rank, tile=tile)
+            assert L.us_workspace_status(ws) == 6 and int(ws[:4].view(torch.int32)[0]) == 1, (rank, tile)
+            ws.zero_()
+    again = call()
+    L.us_attention_bwd_all(dC, P, Q, K, V, 1.0, s_k, 1.0, 1.0, 1.0, 1.0, dS, *again, bt, ws)
+    assert L.us_workspace_status(ws) == 0 and all(torch.equal(a, b) for a, b in zip(good, again))
+    with pytest.raises(L.UnitScaleError) as e:
+        L.us_test_attention_bwd_all_starved(dC, P, Q, K, V, s_k, dS, *again, bt, ws, wait_limit=0, rank=0, tile=0)
+    assert e.value.status == 1
