@@ -63,22 +63,38 @@ struct Args {
   }
 };
 
-PyTypeObject* g_ctypes_data = nullptr;                        // the base of ctypes structures and arrays
-void* buffer(PyObject* o) {                                  // the memory of one
-  if (!PyObject_TypeCheck(o, g_ctypes_data)) fail(PyExc_TypeError, "expected a tensor, a ctypes structure or array, an address or None");
+// ctypes types of the structures (and of host numbers), as register_types() was given them
+template <class T>
+PyTypeObject* g_type = nullptr;
+PyTypeObject* g_ctypes_array = nullptr;
+
+// The memory of a ctypes object of T's type, or of an array of them, that holds `count` at least.
+template <class T>
+T* structure(PyObject* o, size_t count) {
+  bool right = g_type<T> && PyObject_TypeCheck(o, g_type<T>);
+  if (!right && PyObject_TypeCheck(o, g_ctypes_array)) {
+    PyObject* of = PyObject_GetAttrString(reinterpret_cast<PyObject*>(Py_TYPE(o)), "_type_");
+    if (!of) throw Failed();
+    right = reinterpret_cast<PyTypeObject*>(of) == g_type<T>;
+    Py_DECREF(of);
+  }
+  if (!right) fail(PyExc_TypeError, "expected a tensor, a ctypes structure or array of the parameter's type, an address or None");
   Py_buffer b;
   if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) throw Failed();
   void* p = b.buf;
+  const bool enough = (size_t)b.len / sizeof(T) >= count;
   PyBuffer_Release(&b);
-  return p;
+  if (!enough) fail(PyExc_ValueError, "an array is shorter than the count");
+  return static_cast<T*>(p);
 }
 
-// Pointers to device memory (and handles) may be given as addresses or tensors; those to structures may not.
+// Pointers to device memory (and handles) are given as addresses or tensors, those to structures and to arrays on the host are not.
 template <class T>
 constexpr bool kAddress = std::is_same_v<T, void*> || std::is_same_v<T, float*> || std::is_same_v<T, const float*> || std::is_same_v<T, const int32_t*>;
 
-template <class T>
-T convert(PyObject* o, Args& a) {
+// ARRAY: a pointer to `count` elements in host memory.
+template <class T, bool ARRAY>
+T convert(PyObject* o, Args& a, size_t count) {
   if constexpr (std::is_same_v<T, float>) {
     const double v = PyFloat_AsDouble(o);
     if (v == -1.0 && PyErr_Occurred()) throw Failed();
@@ -86,19 +102,20 @@ T convert(PyObject* o, Args& a) {
   } else if constexpr (std::is_pointer_v<T>) {
     if (o == Py_None) return nullptr;
     if constexpr (std::is_same_v<T, const us_mat*>) {
-      if (THPVariable_Check(o)) return a.add(o);
-      return (T)buffer(o);
+      if (THPVariable_Check(o) && count <= 1) return a.add(o);
     }
-    if (PyLong_Check(o) && kAddress<T>) {
+    if constexpr (kAddress<T> && !ARRAY) {
+      if (THPVariable_Check(o)) {
+        if (!a.immediate) fail(PyExc_TypeError, "a prepared call takes addresses");
+        return (T)THPVariable_Unpack(o).data_ptr();
+      }
+      if (!PyLong_Check(o)) fail(PyExc_TypeError, "expected a tensor, an address or None");
       void* p = PyLong_AsVoidPtr(o);
       if (!p && PyErr_Occurred()) throw Failed();
       return (T)p;
+    } else {
+      return structure<std::remove_const_t<std::remove_pointer_t<T>>>(o, count);
     }
-    if (THPVariable_Check(o) && kAddress<T>) {
-      if (!a.immediate) fail(PyExc_TypeError, "a prepared call takes addresses");
-      return (T)THPVariable_Unpack(o).data_ptr();
-    }
-    return (T)buffer(o);
   } else if constexpr (std::is_same_v<T, size_t>) {
     if (THPVariable_Check(o)) return THPVariable_Unpack(o).nbytes();
     const size_t v = PyLong_AsSize_t(o);
@@ -128,15 +145,26 @@ struct Prepared {
   virtual int run(void* stream) = 0;
 };
 
-template <class... A>
+// ARRAYS: parameters 1 .. ARRAYS are arrays of as many elements as parameter 0 says.
+template <size_t ARRAYS, class... A>
 struct Entry {
   using Fn = us_status (*)(A...);
   static constexpr size_t kArgs = sizeof...(A);
   using Tuple = std::tuple<A...>;
   template <size_t... I>
   static Tuple read(PyObject* const* o, Args& a, std::index_sequence<I...>) {
-    return Tuple{convert<A>(o[I], a)...};                     // braces: left to right
+    size_t count = 1;
+    if constexpr (ARRAYS > 0) {
+      const long n = PyLong_AsLong(o[0]);
+      if (n == -1 && PyErr_Occurred()) throw Failed();
+      count = n > 0 ? (size_t)n : 0;                          // the library refuses fewer than one
+    }
+    // a workspace is given twice, for its address and for its size, which one number cannot be
+    for (size_t i = 0; a.immediate && i + 1 < kArgs; ++i)
+      if (o[i] == o[i + 1] && kSize[i + 1] && !THPVariable_Check(o[i])) fail(PyExc_TypeError, "a workspace is a tensor");
+    return Tuple{convert<A, (I >= 1 && I <= ARRAYS)>(o[I], a, I >= 1 && I <= ARRAYS ? count : 1)...};      // braces: left to right
   }
+  static constexpr bool kSize[] = {std::is_same_v<A, size_t>...};
   struct Kept : Prepared {
     Fn fn;
     Tuple t;
@@ -168,24 +196,25 @@ struct Entry {
     return k.release();
   }
 };
-template <class... A>
-Entry<A...> entry_of(us_status (*)(A...));
+template <size_t ARRAYS, class... A>
+Entry<ARRAYS, A...> entry_of(us_status (*)(A...));
 
 using Keep = Prepared* (*)(PyObject* const*, Py_ssize_t);
 struct Known { const char* name; PyCFunction now; Keep keep; };
 
-template <auto F>
-PyObject* now(PyObject*, PyObject* const* o, Py_ssize_t n) { return decltype(entry_of(F))::now(F, o, n); }
-template <auto F>
-Prepared* keep(PyObject* const* o, Py_ssize_t n) { return decltype(entry_of(F))::keep(F, o, n); }
-#define US_CALL(f) {#f, (PyCFunction)(void (*)(void))now<f>, keep<f>}
+template <auto F, size_t ARRAYS>
+PyObject* now(PyObject*, PyObject* const* o, Py_ssize_t n) { return decltype(entry_of<ARRAYS>(F))::now(F, o, n); }
+template <auto F, size_t ARRAYS>
+Prepared* keep(PyObject* const* o, Py_ssize_t n) { return decltype(entry_of<ARRAYS>(F))::keep(F, o, n); }
+#define US_ARRAYS(f, n) {#f, (PyCFunction)(void (*)(void))now<f, n>, keep<f, n>}
+#define US_CALL(f) US_ARRAYS(f, 0)
 const Known kKnown[] = {
     US_CALL(us_linear_fwd), US_CALL(us_linear_bwd_x), US_CALL(us_linear_bwd_w), US_CALL(us_linear_fwd_batched), US_CALL(us_linear_bwd_x_batched),
-    US_CALL(us_linear_bwd_w_batched), US_CALL(us_linear_group), US_CALL(us_linear_group_any), US_CALL(us_ffn_hidden), US_CALL(us_ffn_hidden_any),
-    US_CALL(us_attention_fwd), US_CALL(us_attention_bwd), US_CALL(us_attention_bwd_all), US_CALL(us_cast_fp8), US_CALL(us_cast_fp8_multi),
-    US_CALL(us_cast_multi), US_CALL(us_residual_add), US_CALL(us_gelu_fwd), US_CALL(us_gelu_bwd), US_CALL(us_activation_fwd),
-    US_CALL(us_activation_bwd), US_CALL(us_weighted_add), US_CALL(us_softmax_fwd), US_CALL(us_softmax_bwd), US_CALL(us_softmax_xent_fwd),
-    US_CALL(us_softmax_xent_bwd), US_CALL(us_layer_norm_fwd), US_CALL(us_layer_norm_bwd), US_CALL(us_linear_fwd_cast), US_CALL(us_linear_group_cast),
+    US_CALL(us_linear_bwd_w_batched), US_ARRAYS(us_linear_group, 1), US_ARRAYS(us_linear_group_any, 1), US_CALL(us_ffn_hidden), US_CALL(us_ffn_hidden_any),
+    US_CALL(us_attention_fwd), US_CALL(us_attention_bwd), US_CALL(us_attention_bwd_all), US_CALL(us_cast_fp8), US_ARRAYS(us_cast_fp8_multi, 3),
+    US_ARRAYS(us_cast_multi, 3), US_CALL(us_residual_add), US_CALL(us_gelu_fwd), US_CALL(us_gelu_bwd), US_CALL(us_activation_fwd),
+    US_CALL(us_activation_bwd), US_ARRAYS(us_weighted_add, 2), US_CALL(us_softmax_fwd), US_CALL(us_softmax_bwd), US_CALL(us_softmax_xent_fwd),
+    US_CALL(us_softmax_xent_bwd), US_CALL(us_layer_norm_fwd), US_CALL(us_layer_norm_bwd), US_CALL(us_linear_fwd_cast), US_ARRAYS(us_linear_group_cast, 2),
     US_CALL(us_layer_norm_fwd_cast), US_CALL(us_layer_norm_bwd_cast),
 };
 constexpr size_t kCount = sizeof(kKnown) / sizeof(kKnown[0]);
@@ -242,7 +271,7 @@ PyObject* program(PyObject*, PyObject* const* o, Py_ssize_t n) {
         if (first == -1 && PyErr_Occurred()) throw Failed();
         second = PyTuple_GET_ITEM(e, 1);
         if (which == 1) {
-          p->slots.emplace_back((int)first, static_cast<us_mat*>(buffer(second)));
+          p->slots.emplace_back((int)first, structure<us_mat>(second, 1));
         } else if (second == Py_None) {
           p->steps.push_back({(int)first, nullptr});
         } else {
@@ -325,7 +354,25 @@ PyObject* unchanged(PyObject*, PyObject* const* o, Py_ssize_t n) {
   });
 }
 
+// register_types((us_mat, us_epilogue, us_batch, us_attention_batch, us_attention_bwd_batch, us_attention_bwd_all_batch, us_linear_call,
+// c_float)): the ctypes types of the parameters; every argument is checked against its own
+template <class... T>
+void keep_types(PyObject* types) {
+  Py_ssize_t i = 0;
+  for (Py_ssize_t k = 0; k < (Py_ssize_t)sizeof...(T); ++k)
+    if (!PyType_Check(PyTuple_GET_ITEM(types, k))) fail(PyExc_TypeError, "types");
+  (void(g_type<T> = reinterpret_cast<PyTypeObject*>(Py_NewRef(PyTuple_GET_ITEM(types, i++)))), ...);
+}
+PyObject* register_types(PyObject*, PyObject* const* o, Py_ssize_t n) {
+  return guarded([&]() -> PyObject* {
+    if (n != 1 || !PyTuple_Check(o[0]) || PyTuple_GET_SIZE(o[0]) != 8) fail(PyExc_TypeError, "register_types((eight types))");
+    keep_types<us_mat, us_epilogue, us_batch, us_attention_batch, us_attention_bwd_batch, us_attention_bwd_all_batch, us_linear_call, float>(o[0]);
+    Py_RETURN_NONE;
+  });
+}
+
 PyMethodDef g_methods[] = {
+    {"register_types", (PyCFunction)(void (*)(void))register_types, METH_FASTCALL, nullptr},
     {"unchanged", (PyCFunction)(void (*)(void))unchanged, METH_FASTCALL, nullptr},
     {"prepare", (PyCFunction)(void (*)(void))prepare, METH_FASTCALL, nullptr},
     {"program", (PyCFunction)(void (*)(void))program, METH_FASTCALL, nullptr},
@@ -337,10 +384,10 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, g_method
 
 PyMODINIT_FUNC PyInit__binding(void) {
   PyObject* ct = PyImport_ImportModule("ctypes");
-  PyObject* st = ct ? PyObject_GetAttrString(ct, "Structure") : nullptr;
+  PyObject* array = ct ? PyObject_GetAttrString(ct, "Array") : nullptr;      // kept: lives as long as this module
   Py_XDECREF(ct);
-  if (!st) return nullptr;
-  g_ctypes_data = reinterpret_cast<PyTypeObject*>(st)->tp_base;   // Structure lives as long as its module
+  if (!array) return nullptr;
+  g_ctypes_array = reinterpret_cast<PyTypeObject*>(array);
   PyObject* m = PyModule_Create(&g_module);
   PyObject* d = m ? PyDict_New() : nullptr;
   if (!d) { Py_XDECREF(m); return nullptr; }

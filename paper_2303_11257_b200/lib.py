@@ -169,6 +169,8 @@ def _load() -> C.CDLL:
 _lib = _library = _load()
 from . import _binding                                        # noqa: E402  (links the library that has just been loaded)
 
+_binding.register_types((us_mat, us_epilogue, us_batch, us_attention_batch, us_attention_bwd_batch, us_attention_bwd_all_batch, us_linear_call, C.c_float))
+
 
 def _entry(name: str):
     """The function of that name: through the binding, which takes tensors as they are."""

@@ -72,3 +72,51 @@ def test_fp8_copies_are_validated_before_any_launch():
     norm = lambda y, q: _binding.calls["us_layer_norm_fwd_cast"](M(0x10000, L.US_BF16, 64, 48), v, v, 1e-5, y, q, 0)
     assert norm(Y, None) == 1 and norm(Y, M(0x50000, L.US_E4M3, 64, 32)) == 1 and norm(Y, M(0x50000, L.US_BF16, 64, 48)) == 2
     assert norm(M(0x30000, L.US_E5M2, 64, 48), good) == 2
+
+
+ROWS = torch.zeros(4, 64, dtype=torch.bfloat16)
+WS = torch.zeros(256, dtype=torch.uint8)
+ONE, TWO = L.us_mat(0x10000, L.US_F32, 4, 16, 16), (L.us_mat * 2)()
+WRONG = [L.us_mat(), L.us_epilogue(), L.us_batch(), L.us_attention_batch(), L.us_attention_bwd_batch(), L.us_attention_bwd_all_batch(), C.c_float(1.0),
+         C.c_void_p(0x10000), C.pointer(L.us_mat()), C.byref(L.us_mat()), (C.c_uint8 * 4096)(), (L.us_epilogue * 2)(), b"x" * 4096, np.zeros(4096, np.uint8)]
+
+
+@pytest.mark.parametrize("call,own", [
+    (lambda x: L.us_attention_fwd(ROWS, ROWS, ROWS, 1.0, 1.0, 1.0, ROWS, None, x, WS, 0), L.us_attention_batch),
+    (lambda x: L.us_attention_bwd(ROWS, ROWS, ROWS, ROWS, 1.0, 1.0, 1.0, 1.0, ROWS, ROWS, x, WS, 0), L.us_attention_bwd_batch),
+    (lambda x: L.us_attention_bwd_all(ROWS, ROWS, ROWS, ROWS, ROWS, *[1.0] * 6, ROWS, ROWS, ROWS, ROWS, x, WS, 0), L.us_attention_bwd_all_batch),
+    (lambda x: L.us_linear_fwd_batched(ROWS, ROWS, 1.0, ROWS, x, WS, 0), L.us_batch),
+    (lambda x: L.us_linear_fwd(F32, F32, 1.0, F32, WS, x, 0), L.us_epilogue),
+    (lambda x: cast(x, 1.0, F8, 0), L.us_mat),
+    (lambda x: L.us_linear_fwd(F32, F32, 1.0, F32, x, None, 0), None),                      # the workspace
+    (lambda x: _binding.program([], [(0, x)]), L.us_mat)])
+def test_a_structure_of_another_kind_is_refused(call, own):
+    for x in WRONG:
+        if own is not None and type(x) in (own, own * 2):
+            continue
+        with pytest.raises((TypeError, AttributeError, KeyError)):
+            call(x)
+
+
+def test_arrays_hold_as_many_elements_as_the_count():
+    calls, factors = (L.us_linear_call * 2)(), (C.c_float * 2)(1.0, 1.0)
+    for args in [("us_linear_group", 3, calls, WS, WS), ("us_linear_group_any", 2, calls[0], WS, WS), ("us_linear_group_cast", 2, calls, ONE, WS, WS),
+                 ("us_cast_fp8_multi", 3, (L.us_mat * 3)(), factors, (L.us_mat * 3)()), ("us_cast_multi", 2, TWO, factors, ONE), ("us_weighted_add", 2, ONE, factors, 1.0, ONE)]:
+        with pytest.raises(ValueError):
+            _binding.calls[args[0]](*args[1:], 0)
+        with pytest.raises(ValueError):
+            _binding.prepare(args[0], tuple(a if a is not WS else 256 for a in args[1:]))
+    for factor in (0x10000, F32):                                                           # numbers on the host, not an address
+        with pytest.raises(TypeError):
+            _binding.calls["us_weighted_add"](2, TWO, factor, 1.0, ONE, 0)
+    assert _binding.calls["us_weighted_add"](2, TWO, factors, 1.0, ONE, 0) == L.US_ERR_INVALID_ARG
+    assert _binding.calls["us_linear_group"](0, calls, WS, WS, 0) == L.US_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("ws", [0x10000, 4096, None, np.zeros(256, np.uint8)])
+def test_a_workspace_is_a_tensor(ws):
+    """An address alone says nothing about the size; it is not taken for one."""
+    with pytest.raises(TypeError):
+        L.us_linear_fwd(F32, F32, 1.0, F32, ws, None, 0)
+    with pytest.raises(TypeError):
+        L.us_linear_group([L.us_linear_call()], ws, 0)
