@@ -566,7 +566,8 @@ us_status launch_grads(const CUtensorMap* t, const AttnGradParams& a, cudaStream
   constexpr int smem = GradSmem<F8>::kTotal;
   static std::atomic<uint64_t> smem_set{0};
   const int cl = !CLUSTER ? 1 : a.s_k > 2 * kGrKeys ? 4 : 2;
-  const int fit = host::resident_clusters(reinterpret_cast<const void*>(kern), gr_threads(CLUSTER), smem, cl);
+  static host::ClusterCount count;
+  const int fit = host::resident_clusters(reinterpret_cast<const void*>(kern), gr_threads(CLUSTER), smem, cl, count);
   if (fit <= 0) return US_ERR_CUDA;
   return host::launch(kern, &smem_set, cl * (a.problems < fit ? a.problems : fit), gr_threads(CLUSTER), smem, cl, stream, t[0], t[1], t[2], t[3], t[4], t[5], a);
 }

@@ -17,12 +17,11 @@ int sm_count() {
   return cached[dev];
 }
 
-int resident_clusters(const void* kern, int threads, size_t smem, int cluster) {
-  static std::atomic<int> cached[64][9];
+int resident_clusters(const void* kern, int threads, size_t smem, int cluster, ClusterCount& count) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || cluster < 1 || cluster > 8) return -1;
   if (cluster == 1) return sm_count();
-  int n = cached[dev][cluster].load(std::memory_order_relaxed);
+  int n = count.cached[dev][cluster].load(std::memory_order_relaxed);
   if (n > 0) return n;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) { (void)failed(); return -1; }
   cudaLaunchConfig_t cfg = {};
@@ -34,7 +33,7 @@ int resident_clusters(const void* kern, int threads, size_t smem, int cluster) {
   attr[0].val.clusterDim.x = (unsigned)cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
   if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) { (void)failed(); return -1; }
-  cached[dev][cluster].store(n, std::memory_order_relaxed);
+  count.cached[dev][cluster].store(n, std::memory_order_relaxed);
   return n;
 }
 

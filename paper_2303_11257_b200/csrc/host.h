@@ -53,8 +53,10 @@ us_status launch(void (*kern)(P...), std::atomic<uint64_t>* smem_set, int grid, 
 // Number of SMs of the current device (cached per device), or -1 on error.
 int sm_count();
 // Clusters of `cluster` CTAs (1 .. 8) of a kernel of one CTA per SM that run at once on the current device: a cluster stays within
-// one group of SMs, whose number need not be a multiple of the cluster's.  Cached per device and size; -1 on error.
-int resident_clusters(const void* kern, int threads, size_t smem, int cluster);
+// one group of SMs, whose number need not be a multiple of the cluster's.  Cached per device and size in `count`, a static of the
+// kernel's own (another kernel's threads and shared memory fit another number); -1 on error.
+struct ClusterCount { std::atomic<int> cached[64][9]; };
+int resident_clusters(const void* kern, int threads, size_t smem, int cluster, ClusterCount& count);
 // cuTensorMapEncodeTiled, looked up through the runtime (the library does not link against libcuda); nullptr if unavailable.
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
