@@ -26,9 +26,18 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
+def built_for() -> str:
+    """The Python and torch whose headers and libraries the binding is built with; it holds this text (built_for in binding.cpp)."""
+    import torch
+    return f"us-binding-for python {sys.version_info[0]}.{sys.version_info[1]} torch {torch.__version__};"
+
+
 def _stale() -> bool:
     if not (os.path.exists(LIB) and os.path.exists(BINDING)):
         return True
+    with open(BINDING, "rb") as f:                              # it cannot be imported to be asked: another torch may lack its symbols
+        if built_for().encode() not in f.read():
+            return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS + ["binding.cpp"]] + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
@@ -46,7 +55,7 @@ def _binding_jobs(obj):
     import sysconfig
     import torch
     top = os.path.dirname(os.path.abspath(torch.__file__))
-    compile_ = [_nvcc(), "-std=c++17", "-O2", "-x", "c++", "-Xcompiler", f"-fPIC,-fvisibility=hidden,-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+    compile_ = [_nvcc(), "-std=c++17", "-O2", "-x", "c++", f'-DUS_BUILT_FOR="{built_for()}"', "-Xcompiler", f"-fPIC,-fvisibility=hidden,-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
                 "-I", sysconfig.get_paths()["include"], "-I", os.path.join(top, "include"), "-c", "-o", obj, os.path.join(CSRC, "binding.cpp")]
     link = [_nvcc(), "-shared", "-o", BINDING, obj, LIB, "-L", os.path.join(top, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lcudart",
             "-Xlinker", "-rpath,$ORIGIN"]
@@ -54,7 +63,8 @@ def _binding_jobs(obj):
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile the library if it is missing or older than its sources; returns its path.
+    """Compile the library and the binding if one is missing, older than its sources or built for another Python or torch; returns
+    the library's path.
 
     Every translation unit is compiled to an object in parallel (gemm_inst.cu once per operand
     width and layout), then linked into libunitscale.so next to this file."""

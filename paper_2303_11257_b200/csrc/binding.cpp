@@ -378,6 +378,7 @@ PyMethodDef g_methods[] = {
     {"program", (PyCFunction)(void (*)(void))program, METH_FASTCALL, nullptr},
     {"run", (PyCFunction)(void (*)(void))run, METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
+const char built_for[] = US_BUILT_FOR;                       // what build.py looks for in the file
 PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, g_methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
@@ -398,5 +399,6 @@ PyMODINIT_FUNC PyInit__binding(void) {
     Py_DECREF(f);
   }
   if (PyModule_AddObject(m, "calls", d) != 0) { Py_DECREF(d); Py_DECREF(m); return nullptr; }
+  if (PyModule_AddStringConstant(m, "built_for", built_for) != 0) { Py_DECREF(m); return nullptr; }
   return m;
 }

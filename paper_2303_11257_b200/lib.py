@@ -167,7 +167,14 @@ def _load() -> C.CDLL:
 
 
 _lib = _library = _load()
-from . import _binding                                        # noqa: E402  (links the library that has just been loaded)
+from .build import built_for                                  # noqa: E402
+try:
+    from . import _binding                                    # links the library that has just been loaded
+    if _binding.built_for != built_for():                     # torch's C++ interface is another one from version to version
+        raise ImportError(f"{_binding.built_for} {built_for()}")
+except ImportError as e:
+    raise ImportError(f"the Python binding is missing or was built for another Python or torch ({e}): build it with "
+                      "`python -m paper_2303_11257_b200.build`") from e
 
 _binding.register_types((us_mat, us_epilogue, us_batch, us_attention_batch, us_attention_bwd_batch, us_attention_bwd_all_batch, us_linear_call, C.c_float))
 
