@@ -28,17 +28,20 @@ struct LnArgs {
   const void* w; int w_dt;                  // [cols]
   const void* c; int c_dt;                  // [cols], forward only
   void* out; int out_dt; int64_t out_ld;    // Y (forward) or dX (backward)
-  void* q; int q_dt; int64_t q_ld;          // an FP8 copy of it (null: none)
+  void* q; int q_dt; int64_t q_ld;          // an FP8 copy of it (COPY variants)
   float* partial;                           // backward: [gridDim.x][2][cols]
   int64_t rows; int cols;
   int vec_ok;                               // all row starts 16-byte aligned and cols % 8 == 0
   float eps, beta_x;
 };
 
-// Eight results: stored, and the stored values once more in FP8 where the caller wants them as the operand of a matmul.
+// Eight results: stored, and (COPY) the stored values once more in FP8 for a caller that wants them as the operand of a matmul.  The
+// kernels have variants for it, because the code of the copy, never taken, cost the passes without one 2 to 4 % (backward 8192 x 1024
+// BF16 19.7 -> 20.3 us, forward 1000 x 1024 3.71 -> 3.82).
+template <bool COPY>
 __device__ __forceinline__ void ln_store8(const LnArgs& a, int64_t row, int col, bool vec, const float (&t)[8]) {
   store8(a.out, a.out_dt, row * a.out_ld, col, a.cols, vec, t);
-  if (a.q) {
+  if (COPY) {
     float r[8];
 #pragma unroll
     for (int i = 0; i < 8; i += 2) {
@@ -93,7 +96,7 @@ __device__ __forceinline__ void row_stats(const LnArgs& a, int64_t x_off, int la
 }
 
 // NCH > 0: rows of up to 256 * NCH elements, held in registers.  NCH == 0: any length, re-read.
-template <int NCH>
+template <int NCH, bool COPY>
 __global__ void __launch_bounds__(kLnThreads) ln_fwd_kernel(const LnArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * kLnWarps + (threadIdx.x >> 5);
@@ -119,12 +122,12 @@ __global__ void __launch_bounds__(kLnThreads) ln_fwd_kernel(const LnArgs a) {
     load8(a.c, a.c_dt, 0, col, a.cols, vec, 0.f, b);
 #pragma unroll
     for (int i = 0; i < 8; ++i) t[i] = fmaf(w[i], (t[i] - mu) * rstd, b[i]);
-    ln_store8(a, row, col, vec, t);
+    ln_store8<COPY>(a, row, col, vec, t);
   }
 }
 
 // Input gradient of the rows this warp walks, and the CTA's partial column sums of G * xhat and G.
-template <int NCH>
+template <int NCH, bool COPY>
 __global__ void __launch_bounds__(kLnThreads) ln_bwd_kernel(const LnArgs a) {
   extern __shared__ __align__(16) float ln_smem[];          // NCH > 0: [warps][cols] for the combine; NCH == 0: [warps][2][cols]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -200,7 +203,7 @@ __global__ void __launch_bounds__(kLnThreads) ln_bwd_kernel(const LnArgs a) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) d[i] = k * (g[i] * w[i] - mean_u - (t[i] - mu) * rstd * mean_ux);
       }
-      ln_store8(a, row, col, vec, d);
+      ln_store8<COPY>(a, row, col, vec, d);
     }
   }
   // ---- combine the CTA's warps in warp order; one partial row (G xhat sums, then G sums) per CTA
@@ -259,7 +262,7 @@ __device__ __forceinline__ void stats_regs(const float (&x)[NCH][8], int lane, i
   rstd = rsqrtf(warp_sum(q) / (float)cols + eps);
 }
 
-template <int NCH>
+template <int NCH, bool COPY>
 __global__ void __launch_bounds__(kLnThreads, NCH <= 4 ? 3 : 2) ln_fwd16_kernel(const LnArgs a) {
   extern __shared__ __align__(16) float ln_smem[];                         // w[cols], c[cols] as float32
   float* w_s = ln_smem;
@@ -290,7 +293,7 @@ __global__ void __launch_bounds__(kLnThreads, NCH <= 4 ? 3 : 2) ln_fwd16_kernel(
         float t[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) t[i] = fmaf(w[i], (x[c][i] - mu) * rstd, b[i]);
-        ln_store8(a, row, col, true, t);
+        ln_store8<COPY>(a, row, col, true, t);
       }
     }
 #pragma unroll
@@ -311,7 +314,7 @@ constexpr uint32_t kLnWaitLimit = 1u << 20;
 
 // XBF: X (and a 16-bit gradient) are BF16 rather than F16; fixed at compile time, because a run-time choice
 // in the unpacking costs more instructions than the arithmetic it feeds.
-template <int NCH, bool G32, bool XBF>
+template <int NCH, bool G32, bool XBF, bool COPY>
 __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
   extern __shared__ __align__(16) float ln_smem[];             // w[cols] as float32, [warps][cols] for the combine, the ring, its mbarriers
   float* w_s = ln_smem;                                        // NCH * 256 floats
@@ -494,7 +497,7 @@ __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
           const f32x2 t = fma2(mul2(g_pair(c, j), w2[j]), k2, c0);
           unpack2(fma2(xp[c][j], c1, t), d[2 * j], d[2 * j + 1]);
         }
-        ln_store8(a, row, col, true, d);
+        ln_store8<COPY>(a, row, col, true, d);
       }
     }
   }
@@ -603,6 +606,31 @@ static int ln_bwd_grid(int64_t rows, int warps = kLnWarps, int per_sm = 2) {
 }
 constexpr int kLnFastWarps = 4, kLnFastPerSm = 3;   // the 16-bit backward kernel: three CTAs of four warps per SM
 
+template <bool COPY>
+static us_status ln_fwd_launch(const LnArgs& a, cudaStream_t st) {
+  const int64_t grid64 = (a.rows + kLnWarps - 1) / kLnWarps;
+  if (grid64 > 0x7fffffff) return US_ERR_INVALID_ARG;
+  const int grid = (int)grid64, nch = (a.cols + 255) / 256;
+  if (a.vec_ok && (a.x_dt == US_BF16 || a.x_dt == US_F16) && nch <= 8) {
+    const int sms = host::sm_count();
+    if (sms <= 0) return US_ERR_CUDA;
+    // resident CTAs, warps walk the rows; three an SM where their registers fit (BF16, two -> three: 8192 x 1024 9.8 -> 9.4 us, 8192 x 256
+    // 4.6 -> 4.2, 32768 x 128 10.5 -> 9.0, 32768 x 1024 28.3 -> 28.2; up to 1000 rows, which are no more CTAs than SMs, equal)
+    const int most = (nch <= 4 ? 3 : 2) * sms, pgrid = grid < most ? grid : most;
+    const size_t smem = (size_t)2 * a.cols * sizeof(float);
+    if (nch <= 1) return host::launch(ln_fwd16_kernel<1, COPY>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
+    if (nch <= 2) return host::launch(ln_fwd16_kernel<2, COPY>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
+    if (nch <= 4) return host::launch(ln_fwd16_kernel<4, COPY>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
+    return host::launch(ln_fwd16_kernel<8, COPY>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
+  }
+  if (nch <= 1) ln_fwd_kernel<1, COPY><<<grid, kLnThreads, 0, st>>>(a);
+  else if (nch <= 2) ln_fwd_kernel<2, COPY><<<grid, kLnThreads, 0, st>>>(a);
+  else if (nch <= 4) ln_fwd_kernel<4, COPY><<<grid, kLnThreads, 0, st>>>(a);
+  else if (nch <= 8) ln_fwd_kernel<8, COPY><<<grid, kLnThreads, 0, st>>>(a);
+  else ln_fwd_kernel<0, COPY><<<grid, kLnThreads, 0, st>>>(a);
+  return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
+}
+
 static us_status ln_fwd(const us_mat* X, const us_mat* w, const us_mat* c, float eps, const us_mat* Y, const us_mat* Yq, void* stream) {
   us_status s = check_matrix(X, nullptr, true);
   if (s == US_OK) s = check_matrix(Y, X, false);
@@ -619,27 +647,50 @@ static us_status ln_fwd(const us_mat* X, const us_mat* w, const us_mat* c, float
   if (Yq) { a.q = Yq->ptr; a.q_dt = Yq->dtype; a.q_ld = Yq->ld; }
   a.rows = X->rows; a.cols = (int)X->cols; a.eps = eps; a.beta_x = 1.f;
   a.vec_ok = ln_rows_aligned(X) && ln_rows_aligned(Y) && ln_rows_aligned(w) && ln_rows_aligned(c) && copy_rows_aligned(Yq) && X->cols % 8 == 0;
-  const int64_t grid64 = (a.rows + kLnWarps - 1) / kLnWarps;
-  if (grid64 > 0x7fffffff) return US_ERR_INVALID_ARG;
-  const int grid = (int)grid64, nch = (a.cols + 255) / 256;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (a.vec_ok && (a.x_dt == US_BF16 || a.x_dt == US_F16) && nch <= 8) {
-    const int sms = host::sm_count();
-    if (sms <= 0) return US_ERR_CUDA;
-    // resident CTAs, warps walk the rows; three an SM where their registers fit (8192 x 1024 BF16: 9.7 -> 9.2 us)
-    const int most = (nch <= 4 ? 3 : 2) * sms, pgrid = grid < most ? grid : most;
-    const size_t smem = (size_t)2 * a.cols * sizeof(float);
-    if (nch <= 1) return host::launch(ln_fwd16_kernel<1>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
-    if (nch <= 2) return host::launch(ln_fwd16_kernel<2>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
-    if (nch <= 4) return host::launch(ln_fwd16_kernel<4>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
-    return host::launch(ln_fwd16_kernel<8>, nullptr, pgrid, kLnThreads, smem, 1, st, a);
+  return Yq ? ln_fwd_launch<true>(a, st) : ln_fwd_launch<false>(a, st);
+}
+
+template <bool COPY>
+static us_status ln_bwd_launch(const LnArgs& a, int grid, float beta_wc, const us_mat* dw, const us_mat* dc, cudaStream_t st) {
+  const int nch = (a.cols + 255) / 256;
+  int nparts = grid;
+  // With no rows the first kernel still runs (one CTA) and writes zero partials, so dw = dc = 0.
+  if (a.vec_ok && nch <= 4 && (a.x_dt == US_BF16 || a.x_dt == US_F16) && (a.g_dt == a.x_dt || a.g_dt == US_F32)) {
+    const bool g32 = a.g_dt == US_F32;
+    nparts = ln_bwd_grid(a.rows > 0 ? a.rows : 1, kLnFastWarps, kLnFastPerSm);
+    const size_t smem = ((size_t)(nch <= 1 ? 1 : nch <= 2 ? 2 : 4) * 256 + (size_t)kLnFastWarps * a.cols) * sizeof(float) +
+                        (g32 ? (size_t)0 : (size_t)kLnFastWarps * kLnStages * (a.cols * 4 + 8));
+    const bool xbf = a.x_dt == US_BF16;
+    const int n = nch <= 1 ? 1 : nch <= 2 ? 2 : 4;
+    void (*fn)(const LnArgs) = nullptr;
+#define US_LN_PICK(N)                                                                                   \
+  fn = g32 ? (xbf ? ln_bwd16_kernel<N, true, true, COPY> : ln_bwd16_kernel<N, true, false, COPY>)       \
+           : (xbf ? ln_bwd16_kernel<N, false, true, COPY> : ln_bwd16_kernel<N, false, false, COPY>)
+    if (n == 1) US_LN_PICK(1);
+    else if (n == 2) US_LN_PICK(2);
+    else US_LN_PICK(4);
+#undef US_LN_PICK
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return host::failed();
+    const us_status launched = host::launch(fn, nullptr, nparts, 32 * kLnFastWarps, smem, 1, st, a);
+    if (launched != US_OK) return launched;
+  } else if (nch <= 4) {
+    const size_t smem = (size_t)kLnWarps * a.cols * sizeof(float);
+    if (nch <= 1) ln_bwd_kernel<1, COPY><<<grid, kLnThreads, smem, st>>>(a);
+    else if (nch <= 2) ln_bwd_kernel<2, COPY><<<grid, kLnThreads, smem, st>>>(a);
+    else ln_bwd_kernel<4, COPY><<<grid, kLnThreads, smem, st>>>(a);
+  } else {
+    const size_t smem = (size_t)4 * 2 * a.cols * sizeof(float);
+    if (cudaFuncSetAttribute(ln_bwd_kernel<0, COPY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return host::failed();
+    ln_bwd_kernel<0, COPY><<<grid, 128, smem, st>>>(a);
   }
-  if (nch <= 1) ln_fwd_kernel<1><<<grid, kLnThreads, 0, st>>>(a);
-  else if (nch <= 2) ln_fwd_kernel<2><<<grid, kLnThreads, 0, st>>>(a);
-  else if (nch <= 4) ln_fwd_kernel<4><<<grid, kLnThreads, 0, st>>>(a);
-  else if (nch <= 8) ln_fwd_kernel<8><<<grid, kLnThreads, 0, st>>>(a);
-  else ln_fwd_kernel<0><<<grid, kLnThreads, 0, st>>>(a);
-  return cudaGetLastError() == cudaSuccess ? US_OK : US_ERR_CUDA;
+  if (cudaGetLastError() != cudaSuccess) return US_ERR_CUDA;
+  const int rgrid = (2 * a.cols + 31) / 32;
+  return host::launch(ln_bwd_reduce_kernel, nullptr, rgrid, 32 * kLnReduceGroups, 0, 1, st, a.partial, nparts, a.cols, beta_wc, dw->ptr,
+                      dw->dtype, dc->ptr, dc->dtype);
 }
 
 static us_status ln_bwd(const us_mat* X, const us_mat* w, const us_mat* G, float eps, float beta_x, float beta_wc, const us_mat* dX,
@@ -669,45 +720,8 @@ static us_status ln_bwd(const us_mat* X, const us_mat* w, const us_mat* G, float
   a.rows = X->rows; a.cols = (int)X->cols; a.eps = eps; a.beta_x = beta_x;
   a.vec_ok = ln_rows_aligned(X) && ln_rows_aligned(G) && ln_rows_aligned(dX) && ln_rows_aligned(w) &&
              copy_rows_aligned(dXq) && X->cols % 8 == 0;
-  const int nch = (a.cols + 255) / 256;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int nparts = grid;
-  // With no rows the first kernel still runs (one CTA) and writes zero partials, so dw = dc = 0.
-  if (a.vec_ok && nch <= 4 && (a.x_dt == US_BF16 || a.x_dt == US_F16) && (a.g_dt == a.x_dt || a.g_dt == US_F32)) {
-    const bool g32 = a.g_dt == US_F32;
-    nparts = ln_bwd_grid(X->rows > 0 ? X->rows : 1, kLnFastWarps, kLnFastPerSm);
-    const size_t smem = ((size_t)(nch <= 1 ? 1 : nch <= 2 ? 2 : 4) * 256 + (size_t)kLnFastWarps * a.cols) * sizeof(float) +
-                        (g32 ? (size_t)0 : (size_t)kLnFastWarps * kLnStages * (a.cols * 4 + 8));
-    const bool xbf = a.x_dt == US_BF16;
-    const int n = nch <= 1 ? 1 : nch <= 2 ? 2 : 4;
-    void (*fn)(const LnArgs) = nullptr;
-#define US_LN_PICK(N)                                                                                   \
-  fn = g32 ? (xbf ? ln_bwd16_kernel<N, true, true> : ln_bwd16_kernel<N, true, false>)                   \
-           : (xbf ? ln_bwd16_kernel<N, false, true> : ln_bwd16_kernel<N, false, false>)
-    if (n == 1) US_LN_PICK(1);
-    else if (n == 2) US_LN_PICK(2);
-    else US_LN_PICK(4);
-#undef US_LN_PICK
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return host::failed();
-    const us_status launched = host::launch(fn, nullptr, nparts, 32 * kLnFastWarps, smem, 1, st, a);
-    if (launched != US_OK) return launched;
-  } else if (nch <= 4) {
-    const size_t smem = (size_t)kLnWarps * a.cols * sizeof(float);
-    if (nch <= 1) ln_bwd_kernel<1><<<grid, kLnThreads, smem, st>>>(a);
-    else if (nch <= 2) ln_bwd_kernel<2><<<grid, kLnThreads, smem, st>>>(a);
-    else ln_bwd_kernel<4><<<grid, kLnThreads, smem, st>>>(a);
-  } else {
-    const size_t smem = (size_t)4 * 2 * a.cols * sizeof(float);
-    if (cudaFuncSetAttribute(ln_bwd_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return host::failed();
-    ln_bwd_kernel<0><<<grid, 128, smem, st>>>(a);
-  }
-  if (cudaGetLastError() != cudaSuccess) return US_ERR_CUDA;
-  const int rgrid = (2 * a.cols + 31) / 32;
-  return host::launch(ln_bwd_reduce_kernel, nullptr, rgrid, 32 * kLnReduceGroups, 0, 1, st, a.partial, nparts, a.cols, beta_wc, dw->ptr,
-                      dw->dtype, dc->ptr, dc->dtype);
+  return dXq ? ln_bwd_launch<true>(a, grid, beta_wc, dw, dc, st) : ln_bwd_launch<false>(a, grid, beta_wc, dw, dc, st);
 }
 
 }  // namespace us
