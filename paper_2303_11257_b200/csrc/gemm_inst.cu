@@ -110,9 +110,18 @@ us_status launch_gemm(const us_mat* A, const us_mat* B, GemmParams& p, const Epi
   const long long pair_tiles = (long long)((p.M + 2 * kBM - 1) / (2 * kBM)) * ((p.N + 255) / 256) * bd.nb0 * bd.nb1;
   const bool pair = p.N > 128 && p.M > kBM && (sms <= 0 || 4 * pair_tiles >= sms);
   // 128 x 64 tiles where the machine has an SM for each of them (or, batched, where the outputs are no wider): half the operand
-  // bytes and epilogue of a 128 x 128 tile per CTA.
+  // bytes and epilogue of a 128 x 128 tile per CTA.  us, 128 x 128 -> 128 x 64 tiles, outputs x contraction, FP8 unless said: 48 x 4096 x 512
+  // 4.1 -> 3.4, 200 x 4700 x 512 weight gradient 5.5 -> 5.1, 1000 x 528 x 512 4.2 -> 3.4, 9000 x 128 x 512 4.3 -> 4.0, 128 x 9472 x 2048
+  // 6.2 -> 6.2; batched 256 x (512 x 64) 13.4 -> 12.0.  Two exceptions:
+  //  - An MN-major A with rows shorter than a 128-byte box is fetched by every tile in pieces of its short rows, so fewer tiles are better
+  //    sooner.  Weight gradients, contraction of 2048, 32 / 48 / 64 / 96 tiles of 128 x 64 against the 128 x 128 ones: 16-byte rows
+  //    7.6 / 8.0 / 9.6 / 14.4 against 7.6 / 7.8 / 8.1 / 8.6, 48 bytes 8.6 / 8.8 / 9.6 / 13.5 against 8.8 / 8.9 / 9.1 / 9.2, 96 bytes (BF16)
+  //    7.8 / 7.8 / 8.0 / 9.9 against 9.4 / 9.4 / 9.4 / 9.5; 200 bytes 10.9 / 10.9 / 11.0 / 11.8 against 12.5 / 12.5 / 12.7 / 12.8.
+  //  - 65 to 95 columns are two tiles instead of one, the second mostly empty (9400 x 80 x 1024: 4.7 -> 5.3, 5000 x 100 4.9 -> 4.3).
   const long long narrow_tiles = (long long)((p.M + kBM - 1) / kBM) * ((p.N + 63) / 64);
-  const bool narrow = !pair && (bd.batched() ? p.N <= 64 : narrow_tiles <= sms);
+  const int short_a = A_MN ? p.M * ES : kStageKBytes;
+  const int most = short_a < 32 ? 32 : short_a < 96 ? 48 : short_a < kStageKBytes ? 64 : p.N > 64 && p.N < 96 ? sms * 3 / 4 : sms;
+  const bool narrow = !pair && (bd.batched() ? p.N <= 64 : narrow_tiles <= most);
   const int bn = pair ? 256 : narrow ? 64 : 128, cg = pair ? 2 : 1;
   using Narrow = GemmSmem<64, 1, 8>;
   p.a_bytes = (A_MN || p.M >= kBM ? kBM : (p.M + 7) / 8 * 8) * kStageKBytes;

@@ -92,3 +92,15 @@ def test_batched_outputs_of_at_most_64_columns(fmt, rows, k, cols):
         assert L.us_workspace_status(ws) == 0
         for i, p in enumerate(probs):
             U.assert_close_stored(out[i * rows:(i + 1) * rows], p[2], "f32", TOL * max(1.0, np.abs(p[2]).max() / 4), f"{op} problem {i}")
+
+
+@pytest.mark.parametrize("op,rows,cols", [("bwd_w", 16, 2048), ("bwd_w", 16, 2064), ("bwd_w", 40, 3072), ("bwd_w", 40, 3088), ("bwd_w", 50, 4096), ("bwd_w", 50, 4112),
+                                          ("bwd_w", 100, 4112), ("fwd", 7000, 80), ("fwd", 7100, 80)])
+@pytest.mark.parametrize("fmt", ["e4m3", "bf16"])
+def test_both_sides_of_the_lines_of_the_choice(op, rows, cols, fmt):
+    from paper_2303_11257_b200 import lib as L, synth
+    A, B, val, scale = _operands(L, synth, op, rows, 144, cols, 64, fmt, fmt)
+    ws, out = L.new_workspace(), U.empty(rows, cols, "f32", PAD(cols))
+    getattr(L, "us_linear_" + op)(A, B, scale, out, ws)
+    assert L.us_workspace_status(ws) == 0
+    U.assert_close_stored(out, val, "f32", TOL * max(1.0, np.abs(val).max() / 4), op)
