@@ -291,7 +291,8 @@ __device__ __forceinline__ void xent_unpack(const XentChunk<DT>& c, float (&v)[8
     unpack16x8(c.v[0], DT, v);
   }
 }
-// k (onehot - p) for eight consecutive classes, the target being number `at` of them: the comparison is made once for all eight.
+// k (onehot - p) for eight consecutive classes, the target being number `at` of them: the comparison is made once for all eight.  (A gain of 2
+// to 4 % with a warp per row and in the ring; the branch keeps the chunks of the register form apart, 1000 x 10752 float32 gradients 14.1 -> 15.4 us.)
 __device__ __forceinline__ void xent_grad(float (&p)[8], float k, unsigned at) {
   if (at < 8u) {
 #pragma unroll
@@ -365,8 +366,10 @@ __global__ void __launch_bounds__(1024) softmax_xent_row_kernel(const XentArgs a
   const int64_t out_off = row * a.out_ld;
   for_chunks([&](int col, float (&v)[8]) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = ex2_approx(fmaf(v[i], kLog2e, -mb)) * inv;
-    xent_grad(v, k, (unsigned)t - (unsigned)col);
+    for (int i = 0; i < 8; ++i) {
+      const float p = ex2_approx(fmaf(v[i], kLog2e, -mb)) * inv;
+      v[i] = k * ((col + i == t ? 1.0f : 0.f) - p);
+    }
     store8(a.out, a.out_dt, out_off, col, a.cols, a.vec_ok && col + 8 <= a.cols, v);
   });
 }
@@ -433,7 +436,8 @@ __global__ void __launch_bounds__(kXentStagedThreads, 3) softmax_xent_staged_ker
     for_chunks([&](int col, float (&v)[8]) {
 #pragma unroll
       for (int i = 0; i < 8; ++i) v[i] = ex2_approx(fmaf(v[i], kLog2e, -mb)) * inv;
-      xent_grad(v, k, (unsigned)t - (unsigned)col);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = k * ((col + i == t ? 1.0f : 0.f) - v[i]);
       store8(a.out, a.out_dt, out_off, col, a.cols, true, v);
     });
     if (tid < tail) {
@@ -449,7 +453,7 @@ __global__ void __launch_bounds__(kXentStagedThreads, 3) softmax_xent_staged_ker
 // memory is filled by bulk copies ahead of the row that is worked on, and a thread holds its (at most 32) elements of that
 // row in registers, widened, from the maximum to the write.  Each exponential is computed once (twice in the other forms, which the
 // ex2 unit bounds).  E5M2 gradient of 2048 rows of BF16 logits: 16384 classes 33.5 -> 27.1 us, 12000 24.6 -> 22.1, 8192 17.2 -> 14.0;
-// 4096 rows of 5000 22.0 -> 20.0.  Rows of up to 4096 classes gain nothing, longer ones than 16384 leave room for one CTA an SM and
+// 4096 rows of 5000 22.0 -> 20.0 (xent_launch_dt has the lines).  Rows of up to 4096 classes gain nothing, longer ones than 16384 leave room for one CTA an SM and
 // lose, and so does the forward pass, which has no second exponential to save.
 // A wait that runs out falls back to loads from global memory.
 constexpr int kXentRing = 3;
@@ -724,9 +728,17 @@ static us_status xent_launch_dt(const XentArgs& a, cudaStream_t st) {
   const int nch = (chunks + threads - 1) / threads;
   const int rows = (int)a.rows;
   if constexpr (DT != US_F32) {
-    if (BWD && a.vec_ok && a.cols > 4096 && a.cols <= 16384) {
+    // The ring: wherever every row has a CTA of its own; with more rows not for float32 gradients, whose writes bound both forms and are
+    // less even from fewer CTAs, not for 8193 to 10240 classes, where the register form has five chunks a thread and 256 threads, the
+    // ring 512 of which few have more than two, and not below 5000.  Registers against ring, times as fast, 4104 / 6000 / 8192 / 8200 / 10000 /
+    // 10752 / 16384 classes: 1 to 296 rows 1.2 to 1.6 at any; E5M2 or BF16 gradients of 1000 rows 0.97 / 1.08 / 1.14 / 0.91 / 0.93 / 1.00 / 1.05, of
+    // 4096 1.04 / 1.18 / 1.26 / 0.93 / 0.98 / 1.09 / 1.14; float32 of 592 rows 1.13 / 1.15 / 1.20 / 0.91 / 0.95 / 1.04 / 1.03, of 4096 0.86 / 0.97 /
+    // 0.97 / 0.78 / 0.83 / 0.95 / 0.87.
+    const int t = a.cols > 8192 ? 512 : 256, units = sms * (1024 / t);
+    const bool walks = a.out_dt != US_F32 && ((a.cols >= 5000 && a.cols <= 8192) || a.cols > 10240);
+    if (BWD && a.vec_ok && a.cols > 4096 && a.cols <= 16384 && (rows <= units || walks)) {
       static std::atomic<uint64_t> ring_set[2];
-      const int t = a.cols > 8192 ? 512 : 256, units = sms * (1024 / t), g = rows < units ? rows : units, max_smem = kXentRing * 64 * t;
+      const int g = rows < units ? rows : units, max_smem = kXentRing * 64 * t;
       const size_t smem = (size_t)kXentRing * (a.cols / 8) * 16;
       if (t == 512) return host::launch_plain(softmax_xent_ring_kernel<DT, 512>, &ring_set[0], g, t, max_smem, smem, st, a);
       return host::launch_plain(softmax_xent_ring_kernel<DT, 256>, &ring_set[1], g, t, max_smem, smem, st, a);

@@ -116,3 +116,17 @@ def test_softmax_xent_backward_of_rows_that_a_cta_walks(rows, cols, in_fmt, out_
     for i in np.flatnonzero((t[pick] < 0) | (t[pick] >= cols)):       # no one-hot term there
         ref[i, np.clip(t[pick[i]], 0, cols - 1)] -= 8.0 * np.float64(g[pick[i]])
     U.assert_close_stored(dX[torch.from_numpy(pick).cuda()], ref, out_fmt, 3e-6 * 8.0 * np.abs(g).max(), "xent bwd")
+
+
+@pytest.mark.parametrize("rows,cols,out_fmt", [(1, 4104, "f32"), (296, 8201, "e5m2"), (297, 8201, "e5m2"), (297, 10240, "bf16"), (1000, 10247, "bf16"), (296, 16384, "f32"),
+                                               (297, 16384, "f32"), (592, 8192, "f32"), (593, 8192, "f32"), (800, 4999, "e5m2"), (800, 5000, "e5m2")])
+def test_softmax_xent_backward_on_both_sides_of_the_ring(rows, cols, out_fmt):
+    L, synth = _mods()
+    ld = (cols + 15) // 16 * 16
+    x, g = synth.normal(36, cols, (rows, cols), 2.0), synth.normal(36, 1, (1, rows))[0]
+    t = (np.arange(rows) * 7919 % cols).astype(np.int32)
+    dX = U.empty(rows, cols, out_fmt, ld)
+    L.us_softmax_xent_bwd(U.to_device(x, "bf16", ld), torch.from_numpy(t).cuda(), torch.from_numpy(g).cuda(), 8.0, dX)
+    pick = np.unique(np.concatenate([np.arange(0, rows, 37), np.arange(max(0, rows - 3), rows)]))
+    ref = O.softmax_xent_bwd(U.values_of(x, "bf16")[pick], t[pick], g[pick].astype(np.float64), 8.0)
+    U.assert_close_stored(dX[torch.from_numpy(pick).cuda()], ref, out_fmt, 3e-6 * 8.0 * np.abs(g).max(), "xent bwd")
