@@ -84,6 +84,17 @@ def test_cast_of_padded_rows_with_several_chunks_per_thread(shape, ld, src):
         assert not dst.as_strided((shape[0], ld), (ld, 1)).view(torch.uint8)[:, shape[1]:].any()
 
 
+@pytest.mark.parametrize("src", ["f32", "bf16", "fp16"])
+@pytest.mark.parametrize("shape,ld", [((70, 32), 48), ((70, 33), 48), ((70, 100), 112), ((70, 101), 112), ((1, 100), 112), ((700, 101), 101), ((3, 20), 32)])
+def test_cast_on_both_sides_of_the_choice_of_kernel(shape, ld, src):
+    from paper_2303_11257_b200 import synth
+    L = _lib()
+    x = synth.normal(13, 0, shape)
+    dst = U.empty(*shape, "e5m2", ld)
+    L.us_cast_fp8(U.to_device(x, src, ld), 1.5, dst)
+    assert np.array_equal(U.codes_of(dst), F.scaled_cast(U.values_of(x, src).astype(np.float32), 1.5, F.E5M2))
+
+
 def test_cast_empty_and_errors():
     L = _lib()
     src = torch.zeros((0, 8), device="cuda")
