@@ -35,6 +35,32 @@ from . import lib as L
 E4, E5 = torch.float8_e4m3fn, torch.float8_e5m2
 
 
+def backward_in_one_launch(problems: int, slen: int, fp8: bool) -> bool:
+    """Whether the backward pass of fused attention over `problems` (sequence, head) pairs goes out as one launch instead of three.
+
+    Up to 128 keys a CTA holds a problem, and one launch is faster at any size (8192 tokens of 16 heads, 16 / 64 / 128 keys: the layer
+    takes 131 / 40 / 27 us less).  Up to 256 a cluster of two does, 74 of which run at once; beyond, one of four, 33 at once, that walks
+    the problem's query tiles one after another, while the three launches give each tile to one of 148 CTAs.  So the line depends on the
+    waves of both, and on the keys that a cluster's last CTA has.  Layers of 2 to 6 heads, us that one launch adds (a list: problems):
+      144 keys, 16-bit, 12 / 36 / 40 / 80 / 150 / 300: +1.1 -0.7 -1.3 -0.5 +0.4 +4.4; 192: +0.7 +0.5 -2.0 -0.4 0 +0.5 (12 heads, 252:
+      +1.3); 208: 0 -0.2 -2.5 -2.2 -2.9 -4.4; 256: 0 -0.7 -2.6 -2.0 -2.8 -9.2
+      144 keys, FP8: +0.8 -0.8 -1.6 -2.0 -2.5 -3.7; 256: 0 0 -1.5 -2.5 -3.5 -5.8
+      336 keys, 16-bit, 8 / 20 / 32 / 36 / 64 / 96 / 192 / 256: +0.7 -0.7 -1.8 +6.9 -1.9 +5.2 +10.5 +13.8; 448: +1.4 -0.7 -1.7 +8.1 -0.7 -3.0 -5.9 +3.2;
+      480: +0.7 -1.4 -3.1 +7.8 -3.4 -7.8 -15.3 -8.6; 512: +0.8 -1.0 -3.7 +6.3 -5.5 -11.0 -22.4 -16.3
+      336 keys, FP8: -0.2 -1.3 -1.9 +5.0 -0.5 +5.1 +15.8 +19.9; 448: +0.5 -1.2 -1.7 +7.6 -1.1 -0.4 +2.4 +11.5; 512: +0.7 -0.6 -1.6 +7.0 -1.8 -2.2 -1.4 +4.2
+      272 to 320 keys: within 1.4 up to 33 problems, +0.2 to +23 beyond"""
+    if slen <= 128:
+        return True
+    if slen <= 256:
+        return problems >= 37 and (fp8 or slen >= 208 or problems <= 80)
+    waves, waves_of_three = -(-problems // 33), -(-problems * -(-slen // 128) // 148)
+    if slen < 336 or problems < 20:
+        return False
+    if fp8:
+        return waves <= min(3, waves_of_three)
+    return waves * (0.8 if slen >= 480 else 0.92 if slen >= 448 else 1.0) <= waves_of_three
+
+
 class UnitScaledEncoderLayer:
     def __init__(self, nseq: int, slen: int, d: int, nhead: int, d_ff: int, tau: float = 0.5,
                  attention: str = "bf16", norm: str | None = None, eps: float = 1e-5, device="cuda",
@@ -97,10 +123,7 @@ class UnitScaledEncoderLayer:
         self.bt_fused = L.attention_batch(n, qkv, qkv, qkv, td, sq)
         self.bt_fused_bwd = L.attention_bwd_batch(n, td, sq, qkv, qkv, sq, qkv)
         self.bt_fused_all = L.attention_bwd_all_batch(n, td, sq, qkv, qkv, qkv, sq, qkv, qkv, qkv)
-        # The whole backward pass of attention as one launch where that was the faster way, against three (us, 8192 tokens of
-        # 16 heads): 16-bit operands, sequences of 32: 83 against 135, 128: 32 / 56, 256: 66 / 84, 400 (12 heads): 111 / 103,
-        # 512: 117 / 132; FP8 operands, 256: 53 / 60, 400 (12 heads): 97 / 85, 512: 99 / 95.
-        self._whole = slen <= 256 or (slen > 448 and attention != "fp8")
+        self._whole = backward_in_one_launch(nseq * nhead, slen, attention == "fp8")
 
     @property
     def whole_bwd(self) -> bool:

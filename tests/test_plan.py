@@ -174,3 +174,12 @@ def test_the_first_pass_issues_its_first_call_before_it_makes_what_later_ones_ne
     monkeypatch.setattr(L, "_lib", rec)
     layer.step(*x, stream=0)
     assert early and min(early) >= 2 and rec.names()[:2] == [CAST, "us_linear_fwd"]
+
+
+@pytest.mark.parametrize("slen,fp8,yes,no", [
+    (128, False, (1, 5000), ()), (144, False, (37, 80), (1, 36, 81)), (144, True, (37, 5000), (36,)), (192, False, (37, 80), (36, 81)), (208, False, (37, 5000), (36,)), (256, True, (37,), (36,)),
+    (272, False, (), (8, 33, 256)), (336, False, (20, 33, 50, 66), (19, 36, 96)), (448, False, (20, 40, 66, 192), (34, 36, 256)),
+    (480, False, (38, 256), (36, 68)), (512, False, (20, 66, 96, 256), (8, 36, 68)), (512, True, (20, 66, 96), (36, 128, 256)), (336, True, (33, 50), (49, 96))])
+def test_when_the_attention_backward_pass_is_one_launch(slen, fp8, yes, no):
+    assert all(encoder.backward_in_one_launch(p, slen, fp8) for p in yes)
+    assert not any(encoder.backward_in_one_launch(p, slen, fp8) for p in no)
