@@ -44,8 +44,8 @@ def _close(got, ref, fmt, what):
     assert ok.all(), f"{what}: {(~ok).sum()} elements out"
 
 
-# one key and one query; the edges of a query tile, of a key block, of a 128-key half and of a CTA's 256 keys; the partner CTA with
-# one key, an odd number of blocks and all of them; more problems than CTAs (clusters), so that every phase carries over
+# one key and one query; the edges of a query tile, of a key block, of a CTA's 128 keys and of a cluster of two; a last CTA of a cluster
+# with one key, none (384 keys or fewer of four CTAs) and all of them; more problems than CTAs (clusters), so that every phase carries over
 SHAPES = [(1, 1, 1, 1), (1, 2, 40, 72), (2, 1, 128, 128), (1, 1, 129, 136), (1, 2, 200, 256), (1, 1, 130, 257), (1, 1, 384, 330),
           (1, 2, 512, 512), (3, 60, 136, 200), (2, 40, 264, 272), (5, 20, 130, 64)]
 
@@ -132,3 +132,77 @@ def test_a_cluster_that_gives_up_drains_what_its_ctas_send_each_other(fmt, s_k, 
     with pytest.raises(L.UnitScaleError) as e:
         L.us_test_attention_bwd_all_starved(dC, P, Q, K, V, s_k, dS, *again, bt, ws, wait_limit=0, rank=0, tile=0)
     assert e.value.status == 1
+
+
+def _layer(s_q, s_k, fmt, out_fmt, n, seed, spoil=None):
+    """(dC, P, Q, K, V), the results' buffers and the two ways to the results, over the layout of an encoder layer: heads are column slices of
+    [tokens x 3 x heads x 64] matrices, P and dS have padded rows.  The buffers begin as ones, results' neighbours among them."""
+    from paper_2303_11257_b200 import lib as L
+    gfmt, h = "e5m2" if fmt == "e4m3" else fmt, 3
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    wide = lambda r, f, w: torch.randn(n * r, w * h * 64, generator=gen, device="cuda").to(U.TORCH_OF[f])
+    dC, q, kv, ld = wide(s_q, gfmt, 1), wide(s_q, fmt, 1), wide(s_k, fmt, 2), (s_k + 15) // 16 * 16
+    P = torch.zeros(n * h * s_q, ld, device="cuda")
+    P[:, :s_k] = s_k * torch.softmax(torch.randn(n * h * s_q, s_k, generator=gen, device="cuda"), 1)
+    P = P.to(U.TORCH_OF[fmt])[:, :s_k]
+    if spoil:
+        spoil(dC, kv)
+    ones = lambda r, c, f: torch.ones(r, c, device="cuda").to(U.TORCH_OF[f])
+    hs = lambda t, r, w, at=0: (t[:r, at * h * 64:at * h * 64 + 64], (r * w * h * 64, 64))       # head 0 of sequence 0, strides
+    (dc, sdc), (Q, sq), (K, sk), (V, _) = hs(dC, s_q, 1), hs(q, s_q, 1), hs(kv, s_k, 2), hs(kv, s_k, 2, 1)
+    sp, ws = (h * s_q * ld, s_q * ld), L.new_workspace()
+
+    def run(one):
+        dS, dq, dkv = ones(n * h * s_q, ld, gfmt)[:, :s_k], ones(n * s_q, h * 64 + 16, out_fmt), ones(n * s_k, 2 * h * 64 + 32, out_fmt)
+        dQ, dK, dV = dq[:s_q, :64], dkv[:s_k, :64], dkv[:s_k, h * 64 + 16:h * 64 + 80]
+        rq, rk = (s_q * dq.shape[1], 64), (s_k * dkv.shape[1], 64)
+        if one:
+            L.us_attention_bwd_all(dc, P[:s_q], Q, K, V, 0.125, s_k, s_k, 0.25, 0.125, 0.5, dS[:s_q], dQ, dK, dV,
+                                   L.attention_bwd_all_batch((n, h), sdc, sp, sq, sk, sk, sp, rq, rk, rk), ws)
+        else:
+            L.us_linear_bwd_w_batched(P[:s_q], dc, 0.5, dV, L.batch((n, h), sp, sdc, rk), ws)
+            L.us_attention_bwd(dc, P[:s_q], K, V, 0.125, s_k, s_k, 0.25, dS[:s_q], dQ, L.attention_bwd_batch((n, h), sdc, sp, sk, sk, sp, rq), ws)
+            L.us_linear_bwd_w_batched(dS[:s_q], Q, 0.125, dK, L.batch((n, h), sp, sq, rk), ws)
+        assert L.us_workspace_status(ws) == 0
+        return dS, dq, dkv
+
+    return (dC, P, q, kv), run
+
+
+@pytest.mark.parametrize("s_q,s_k", [(100, 112), (272, 272), (160, 304), (384, 384), (130, 400), (496, 496)])
+@pytest.mark.parametrize("fmt,out_fmt", [("bf16", "e5m2"), ("fp16", "f32"), ("e4m3", "bf16")])
+def test_strided_heads_and_what_lies_between_them(s_q, s_k, fmt, out_fmt):
+    """In the layout of a layer: dS within one code of the three launches' (their row sums have another order), dQ and dK against products of
+    the launch's own dS, dV bit for bit that of the batched GEMM; nothing written between the results."""
+    n, h = 2, 3
+    (dC, P, q, kv), run = _layer(s_q, s_k, fmt, out_fmt, n, 41)
+    (dS, dq, dkv), (dS3, dq3, dkv3) = run(True), run(False)
+    apart = (dS.float() - dS3.float()).abs()
+    # beside one code, 3e-6 of the largest dS and of dP (variance 1, below 16): a float32 difference of the mean where dP is close to it
+    tol = 3e-6 * (float(dS3.float().abs().max()) + 16.0)
+    assert bool(((apart <= tol).cpu() | torch.from_numpy(U.code_distance(U.codes_of(dS), U.codes_of(dS3), "e5m2" if fmt == "e4m3" else fmt) <= 1)).all())
+    pieces = lambda t, s, at: t.float().double().reshape(n, s, -1)[:, :, at:at + h * 64].reshape(n, s, h, 64).transpose(1, 2).cpu().numpy()
+    w = dS.float().double().reshape(n, h, s_q, s_k).cpu().numpy()
+    _close(pieces(dq, s_q, 0), 0.25 * w @ pieces(kv, s_k, 0), out_fmt, "dQ")
+    _close(pieces(dkv, s_k, 0), 0.125 * w.transpose(0, 1, 3, 2) @ pieces(q, s_q, 0), out_fmt, "dK")
+    at = h * 64 + 16
+    assert torch.equal(dkv[:, at:at + h * 64].contiguous().view(torch.uint8), dkv3[:, at:at + h * 64].contiguous().view(torch.uint8))
+    for t, gaps in ((dq, [slice(h * 64, None)]), (dkv, [slice(h * 64, at), slice(at + h * 64, None)])):
+        assert all(bool((t[:, g].float() == 1).all()) for g in gaps)
+
+
+@pytest.mark.parametrize("s_q,s_k", [(100, 100), (300, 208), (200, 336)])
+@pytest.mark.parametrize("fmt", ["bf16", "e4m3"])
+@pytest.mark.parametrize("what", ["inf in dC", "nan in dC", "nan in V", "nan in K"])
+def test_gradients_that_are_not_finite_spread_as_with_three_launches(s_q, s_k, fmt, what):
+    if fmt == "e4m3" and s_k % 16:
+        s_k = 112                                                        # FP8 rows of P start on 16 bytes
+    def spoil(dC, kv):
+        if what.endswith("dC"):
+            dC[37, 70] = float("inf") if what[0] == "i" else float("nan")           # sequence 0, head 1
+        else:
+            kv[s_k + 5, (3 if what.endswith("V") else 0) * 64 + 130] = float("nan")  # sequence 1, head 2
+    _, run = _layer(s_q, s_k, fmt, "f32", 2, 42, spoil)
+    finite = [[torch.isfinite(t.float()) for t in run(one)] for one in (True, False)]
+    assert not all(bool(t.all()) for t in finite[1]) and all(bool(t.any()) for t in finite[1])
+    assert all(torch.equal(a, b) for a, b in zip(*finite))

@@ -130,3 +130,27 @@ def test_softmax_xent_backward_on_both_sides_of_the_ring(rows, cols, out_fmt):
     pick = np.unique(np.concatenate([np.arange(0, rows, 37), np.arange(max(0, rows - 3), rows)]))
     ref = O.softmax_xent_bwd(U.values_of(x, "bf16")[pick], t[pick], g[pick].astype(np.float64), 8.0)
     U.assert_close_stored(dX[torch.from_numpy(pick).cuda()], ref, out_fmt, 3e-6 * 8.0 * np.abs(g).max(), "xent bwd")
+
+
+@pytest.mark.parametrize("rows,cols,out_fmt", [(700, 6000, "bf16"), (700, 6003, "e5m2"), (40, 12000, "f32"), (700, 3000, "bf16")])
+def test_softmax_xent_backward_of_rows_that_are_not_finite(rows, cols, out_fmt):
+    """A NaN, a row of -inf only and a +inf make their own row NaN, in the ring (the first three) as in registers, and no other."""
+    L, synth = _mods()
+    ld = (cols + 15) // 16 * 16
+    x = synth.normal(37, cols, (rows, cols), 2.0)
+    bad = {5: ("one", np.nan), 6: ("all", -np.inf), 7: ("one", np.inf), rows - 2: ("last", np.nan)}
+    for r, (where, v) in bad.items():
+        x[r, {"one": slice(cols // 3, cols // 3 + 1), "all": slice(None), "last": slice(cols - 1, cols)}[where]] = v
+    x[11, ::2] = -np.inf                                                 # finite: half of the weights are zero
+    t = (np.arange(rows) * 7919 % cols).astype(np.int32)
+    X = torch.zeros(rows, ld, device="cuda")
+    X[:, :cols] = torch.from_numpy(x).cuda()
+    X = X.to(torch.bfloat16)[:, :cols]
+    dX = U.empty(rows, cols, out_fmt, ld)
+    L.us_softmax_xent_bwd(X, torch.from_numpy(t).cuda(), None, 8.0, dX)
+    got = dX.float().cpu().numpy()
+    good = np.setdiff1d(np.arange(rows), list(bad))
+    assert np.isnan(got[list(bad)]).all() and np.isfinite(got[good]).all()
+    pick = np.unique(np.concatenate([good[:16], good[::37], good[-3:]]))
+    ref = O.softmax_xent_bwd(X.double().cpu().numpy()[pick], t[pick], np.ones(len(pick)), 8.0)
+    U.assert_close_stored(dX[torch.from_numpy(pick).cuda()], ref, out_fmt, 3e-6 * 8.0, "xent bwd")
