@@ -18,10 +18,12 @@
 // FP8: dC and dS are E5M2, P, Q, K, V E4M3.  A head row is then 64 bytes, and Q, K, V and dC tiles take the 64-byte swizzle.
 //
 // Bound: the serial chain of a tile (dP, row sums, the cluster's exchange, dS, dQ), of which two are under way in an SM, and beside it the
-// 16-bit conversions of the softmax warps; at 32 to 128 keys HBM (64 x 16 x 128: 185 MB in 32 us, 0.88 of a copy's rate).  128 keys a CTA, because
-// dP of two tiles and the sums of two problems fill tensor memory.  16-bit / FP8 operands, us against us_attention_bwd and the two
-// GEMMs (sequences x heads x length): 16 x 16 x 512 117 / 99 against 132 / 95; 20 x 12 x 400 111 / 97 against 103 / 85; 32 x 16 x 256
-// 66 / 53 against 84 / 60; 64 x 16 x 128 32 against 56; 64 x 8 x 128 14.7 (FP8) against 24.7; 256 x 16 x 32 83 against 135.
+// 16-bit conversions of the softmax warps; at 128 keys HBM (64 x 16 x 128: 159 MB in 28.8 us, 0.84 of a copy's rate); at shorter lengths the
+// same chain again, on tiles that are mostly empty rows (32: three quarters).  128 keys a CTA, because dP of two tiles and the sums of two
+// problems fill tensor memory.  16-bit / FP8 operands, E5M2 results of contiguous heads, us against us_attention_bwd and the two GEMMs
+// (sequences x heads x length): 16 x 16 x 512 104 / 93 against 130 / 91; 20 x 12 x 400 104 / 92 against 99 / 81; 24 x 16 x 320 123 / 117 against
+// 96 / 76; 32 x 16 x 256 57 / 50 against 80 / 58; 64 x 16 x 128 28.8 / 21.4 against 54 / 42; 256 x 16 x 32 64 / 71 against 128 / 129.  The
+// store of dS (dS = NULL leaves it out) is 7 / 2 us of 16 x 16 x 512, 4.5 / 3.3 of 32 x 16 x 256.
 //
 // Every wait is on an mbarrier and bounded, remote arrivals included, and no role waits at a hardware barrier between the
 // start and the end, so a wait that runs out (in any CTA of a cluster) only makes the others' waits run out too; the

@@ -317,6 +317,15 @@ __device__ __forceinline__ f32x2 gelu_grad_scaled2(f32x2 h, f32x2 g, f32x2 in2, 
   return mul2(mul2(os2, d), g);
 }
 
+// Eight results as the values that storage format dt holds of them (float32, BF16 or F16).
+__device__ __forceinline__ void as_stored8(int dt, const float (&y)[8], float (&r)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) {
+    const float2 v = dt == US_BF16 ? unpack_bf16x2(pack_bf16x2(y[i], y[i + 1])) : dt == US_F16 ? unpack_f16x2(pack_f16x2(y[i], y[i + 1])) : make_float2(y[i], y[i + 1]);
+    r[i] = v.x; r[i + 1] = v.y;
+  }
+}
+
 // Division of a non-negative int below 2^31 by a divisor fixed at launch: one multiply-high, one
 // add and one shift instead of the ~30-instruction sequence of a hardware-less integer divide, which
 // every epilogue warp would otherwise run several times per tile.  mul = floor(2^32 (2^shift - d) / d) + 1,

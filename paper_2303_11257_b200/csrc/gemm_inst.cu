@@ -132,8 +132,10 @@ us_status launch_gemm(const us_mat* A, const us_mat* B, GemmParams& p, const Epi
   // A (M x K operand) is re-read by every column of tiles: keep the plain order while it fits well
   // inside the 126 MB L2, switch to bands of 8 tile rows beyond that.
   p.band_m = ((long long)p.M * p.K * ES <= (80ll << 20)) ? p.tiles_m : 8;
-  // A short contraction mostly writes: tiles that run together then cover whole rows of a few bands (8192 x 8192 float32 with K = 512:
-  // 54.5 -> 50.5 us; 1024 x 30528 with K = 2048 loses that way from two bands down).
+  // A short contraction mostly writes: tiles that run together then cover whole rows of a few bands (us, FP8 operands, outputs x K: 8192 x
+  // 8192 float32 x 512 55.7 -> 49.7, repeated runs of either up to 8 apart; 16384 x 8192 BF16 x 1024 115 -> 108, 16384 x 1024 x 256 13.9 ->
+  // 11.7; 8192 x 4096 x 1024, 1024 x 30528 float32 x 512, 65536 x 512 x 128 and batched scores equal; 1024 x 30528 with K = 2048 loses that
+  // way from two bands down).
   if ((long long)p.K * ES <= 1024 && p.tiles_m > 4) p.band_m = 4;
   p.full_bands = p.tiles_m / p.band_m;
   p.d_problem = make_fast_div(p.tiles_m * p.tiles_n);

@@ -237,11 +237,7 @@ struct EpiCtx {
 // Four more codes of a lane's FP8 copy: eight results as the output format dt stores them, rounded once more.
 __device__ __forceinline__ void copy_codes(int dt, int copy_dt, const float (&y)[8], uint32_t* codes) {
   float r[8];
-#pragma unroll
-  for (int i = 0; i < 8; i += 2) {
-    const float2 v = dt == US_BF16 ? unpack_bf16x2(pack_bf16x2(y[i], y[i + 1])) : dt == US_F16 ? unpack_f16x2(pack_f16x2(y[i], y[i + 1])) : make_float2(y[i], y[i + 1]);
-    r[i] = v.x; r[i + 1] = v.y;
-  }
+  as_stored8(dt, y, r);
 #pragma unroll
   for (int i = 0; i < 2; ++i)
     codes[i] = copy_dt == US_E5M2 ? cvt_fp8x4<true>(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]) : cvt_fp8x4<false>(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
@@ -824,8 +820,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
       int stage = 0; uint32_t phase = 0;
       uint32_t local = 0;
       bool ok = true;
-      // The issuing thread is a single instruction stream that has to start four MMAs every ~500
-      // cycles, so the loop body is kept minimal: descriptors differ from stage to stage and from
+      // The issuing thread is a single instruction stream that has to start four MMAs every ~280
+      // cycles (commit and wait for the next barrier included), so the loop body is kept minimal: descriptors differ from stage to stage and from
       // k-step to k-step only in their 14-bit start-address field, i.e. by adding a constant to the
       // low word (no carry: shared memory addresses / 16 stay below 2^14).
       const uint64_t a_desc0 = A_MN ? ptx::smem_desc_sw128(smem_base, kChunkBytes, 1024) : ptx::smem_desc_sw128(smem_base, 16, 1024);

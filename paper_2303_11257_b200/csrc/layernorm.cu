@@ -43,12 +43,7 @@ __device__ __forceinline__ void ln_store8(const LnArgs& a, int64_t row, int col,
   store8(a.out, a.out_dt, row * a.out_ld, col, a.cols, vec, t);
   if (COPY) {
     float r[8];
-#pragma unroll
-    for (int i = 0; i < 8; i += 2) {
-      const float2 v = a.out_dt == US_BF16 ? unpack_bf16x2(pack_bf16x2(t[i], t[i + 1])) : a.out_dt == US_F16 ? unpack_f16x2(pack_f16x2(t[i], t[i + 1]))
-                                                                                                        : make_float2(t[i], t[i + 1]);
-      r[i] = v.x; r[i + 1] = v.y;
-    }
+    as_stored8(a.out_dt, t, r);
     store8(a.q, a.q_dt, row * a.q_ld, col, a.cols, vec, r);
   }
 }

@@ -7,7 +7,6 @@ compiled library: there is no fallback of any kind.
 from __future__ import annotations
 
 import ctypes as C
-import operator
 import os
 
 import torch
@@ -425,9 +424,7 @@ def us_workspace_status(ws: torch.Tensor, stream=None) -> int:
 
 def _linear(name, a, b, scale, ep, out, ws, stream):
     fn = _entry(name)
-    epp = ep if ep is not None else None
-    _check(name, fn(a, b, scale, epp, out,
-                    ws, ws, _stream(stream)))
+    _check(name, fn(a, b, scale, ep, out, ws, ws, _stream(stream)))
     return out
 
 
