@@ -99,11 +99,12 @@ def test_softmax_xent_forward_of_many_rows(rows, cols, in_fmt):
     assert np.abs(out.cpu().numpy() - ref).max() <= 4e-6 * (1 + np.abs(ref).max())
 
 
-@pytest.mark.parametrize("rows,cols", [(2400, 4104), (2400, 8192), (1300, 8201), (1000, 16384)])
+@pytest.mark.parametrize("rows,cols", [(2400, 4104), (2400, 8192), (1300, 8201), (1000, 16384), (2400, 5003), (1300, 10249), (1200, 16384)])
 @pytest.mark.parametrize("in_fmt,out_fmt", [("bf16", "e5m2"), ("fp16", "bf16")])
 def test_softmax_xent_backward_of_rows_that_a_cta_walks(rows, cols, in_fmt, out_fmt):
-    """16-bit rows of 4097 to 16384 classes: CTAs that walk four or more rows through their ring of three, at both CTA sizes, with
-    targets outside the row and a gradient per row; every 37th row and the last ones against the oracle."""
+    """16-bit rows of 4097 to 16384 classes: CTAs that walk four or more rows through their ring of three, at both CTA sizes and with
+    ragged ends (5000 to 8192 classes and from 10241 on; the other two sizes take the register form), with targets outside the row and a
+    gradient per row; every 37th row and the last ones against the oracle."""
     L, synth = _mods()
     ld = (cols + 15) // 16 * 16
     x, g = synth.normal(35, cols, (rows, cols), 2.0), synth.normal(35, 1, (1, rows))[0]
