@@ -17,6 +17,13 @@
 // for FP8 and two for 16-bit elements), instruction descriptor, scale, epilogue kind.
 // Measured, four separate launches -> this one, us: FP8 8192 x 1024 x 4096 122 -> 101; BF16 216 -> 199;
 // FP8 16384 x 2048 x 8192 (21 tiles per pair) 912 of kernel time, partly side by side, -> 809; FP8 256 x 128 x 512 26 -> 7.
+//
+// The run-time data are kernel parameters reached through an index: loads of 100 cycles and more, which a store or a wait
+// between two uses makes the compiler repeat.  So every role fetches a tile's fields once, the first tile's before it waits for the
+// previous kernel, and the epilogue takes its choices (skip type, output type) once per 32-column slice.  With the choices inside the
+// groups of eight columns a slice with a skip tensor took 1550 cycles after its data were there, and its reading another 800.
+// Captured steps, us: 256 x 128 x 512 9.5 -> 8.8, 512 x 512 x 1456 18.0 -> 16.8, 1000 x 528 x 2096 27.4 -> 25.2, 4096 x 256 x 704
+// 24.6 -> 23.4, 2048 x 1024 x 3008 55.1 -> 54.3; BF16 8192 x 1024 x 4096 412 -> 402.
 #pragma once
 
 #include "gemm_kernel.cuh"
@@ -126,7 +133,8 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
         group_decode(e, pi, tm, tn);
         const GroupProblem& P = g.prob[pi];
         const int m0 = tm * kTileM + rank * 128, n0 = tn / SPLIT * BN + rank * 128;
-        const int num_kb = (P.K + kBK - 1) / kBK;
+        const int num_kb = (P.K + kBK - 1) / kBK, a_mn = P.a_mn, b_mn = P.b_mn;
+        if (r == 0) { ptx::prefetch_tensormap(&P.ta); ptx::prefetch_tensormap(&P.tb); }
         for (int kb = 0; kb < num_kb; ++kb) {
           ok = wait_bounded(empty_bar(stage), phase ^ 1u, abort_flag, g.status, g.wait_limit);
           if (!ok) break;
@@ -146,8 +154,8 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
               load(dst, tmap, k0, mn0);
             }
           };
-          operand(a_dst, &P.ta, P.a_mn, m0);
-          operand(b_dst, &P.tb, P.b_mn, n0);
+          operand(a_dst, &P.ta, a_mn, m0);
+          operand(b_dst, &P.tb, b_mn, n0);
           ++issued;
           if (++stage == S::kStages) { stage = 0; phase ^= 1u; }
         }
@@ -164,7 +172,6 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA of a pair only)
     if (ptx::elect_one() && rank == 0) {
-      ptx::grid_wait_previous();                       // no operand comes earlier: the bounded waits begin when the loads do
       int stage = 0; uint32_t phase = 0, local = 0;
       bool ok = true;
       constexpr uint32_t kStageStep = S::kStageBytes >> 4;
@@ -183,6 +190,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
         const uint32_t a_step = (P.a_mn ? kChunkBytes / kKSteps : 32u) >> 4, b_step = (P.b_mn ? kChunkBytes / kKSteps : 32u) >> 4;
         const uint32_t idesc = P.idesc;
         const uint32_t acc = local & 1u, acc_phase = (local >> 1) & 1u;
+        if (local == 0) ptx::grid_wait_previous();       // no operand comes earlier: the bounded waits begin when the loads do
         ++local;
         ok = wait_bounded(acc_empty_bar(acc), acc_phase ^ 1u, abort_flag, g.status, g.wait_limit);
         if (!ok) break;
@@ -219,50 +227,55 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
     // Warp (quarter q, half) owns 32 rows x half of the columns of a tile, worked in 32-column slices.  Staging: box 0
     // (4 KB) receives the skip tensor's boxes by TMA, box 1 (4 KB) collects output and leaves by TMA store.
     const int q = warp & 3, half = (warp - 2) >> 2;
-    ptx::grid_wait_previous();
     const uint32_t buf_in = epi_base + (warp - 2) * epi_warp_bytes(kGroupEW), buf_out = buf_in + 4096u;
     const uint32_t in_bar = epi_in_bar(warp - 2);
     const uint32_t row_off = (uint32_t)lane * 128u, sw = (uint32_t)(lane & 7);
     uint32_t in_phase = 0, local = 0;
     bool in_pending = false, ok = true;
 
-    auto issue_in = [&](const GroupProblem& P, int col, int row0) {
+    auto issue_in = [&](const CUtensorMap* map, int col, int row0) {
       if (ptx::elect_one()) {
         ptx::mbar_expect_tx(in_bar, 4096);
-        ptx::tma_load_2d(buf_in, &P.tskip, in_bar, col, row0);
+        ptx::tma_load_2d(buf_in, map, in_bar, col, row0);
       }
       in_pending = true;
     };
-    // first box of the skip tensor for the first tile at or after round r that has one for this warp
-    auto prefetch_from = [&](int r) {
-      for (; r < g.rounds; ++r) {
-        const int32_t e = entry(r);
-        if (e < 0) continue;
-        int pi, tm, tn;
-        group_decode(e, pi, tm, tn);
-        const GroupProblem& P = g.prob[pi];
-        const int n_w = warp_col(tn, half);
-        if (P.has_skip && n_w < P.N) issue_in(P, n_w, tm * kTileM + rank * 128 + q * 32);
-        return;                                                // only the very next tile is looked at
-      }
-    };
-    prefetch_from(0);
-
-    for (int r = 0; ok && r < g.rounds; ++r) {
-      const int32_t e = entry(r);
-      if (e < 0) continue;
+    // The entry of a round, and the first box of the skip tensor that its tile has for this warp (map null: none).  A round is looked at
+    // while the one before waits for its accumulator, the first one before the previous kernel is waited for.
+    struct Next { int32_t e; const CUtensorMap* map; int col, row; };
+    auto look = [&](int r) {
+      Next n{r < g.rounds ? entry(r) : -1, nullptr, 0, 0};
+      if (n.e < 0) return n;
       int pi, tm, tn;
-      group_decode(e, pi, tm, tn);
+      group_decode(n.e, pi, tm, tn);
+      const GroupProblem& P = g.prob[pi];
+      n.col = warp_col(tn, half); n.row = tm * kTileM + rank * 128 + q * 32;
+      if (P.has_skip && n.col < P.N) n.map = &P.tskip;
+      return n;
+    };
+    Next next = look(0);
+    ptx::grid_wait_previous();
+    if (next.map) issue_in(next.map, next.col, next.row);
+
+    for (int r = 0; ok && next.e >= 0; ++r) {
+      int pi, tm, tn;
+      group_decode(next.e, pi, tm, tn);
       const GroupProblem& P = g.prob[pi];
       const uint32_t acc = local & 1u, acc_phase = (local >> 1) & 1u;
       ++local;
       const int row0 = tm * kTileM + rank * 128 + q * 32, n_w = warp_col(tn, half);
-      const bool skip = P.has_skip != 0;
-      const int in_es = dtype_size(P.skip_dt), out_es = dtype_size(P.out_dt);
+      // The problem's fields are fetched once per tile: a parameter reached through an index is a long load, and would be loaded again after
+      // every instruction that may write memory.
+      const bool skip = ptx::once(P.has_skip) != 0;
+      const int skip_dt = ptx::once(P.skip_dt), out_dt = ptx::once(P.out_dt), cols = ptx::once(P.N);
+      const float scale = __int_as_float(ptx::once(__float_as_int(P.scale))), skip_coef = __int_as_float(ptx::once(__float_as_int(P.skip_coef))),
+                  out_coef = __int_as_float(ptx::once(__float_as_int(P.out_coef)));
+      const int in_es = dtype_size(skip_dt), out_es = dtype_size(out_dt);
       // an output box holds 128-byte rows, or the fewer bytes that a warp's columns are (swizzled accordingly; 32-byte rows: not)
       const int out_row = min(128, kWarpCols * out_es);
       const int in_box_cols = 128 / in_es, out_box_cols = out_row / out_es;
       const uint32_t out_sw = out_row == 128 ? sw : out_row == 64 ? (uint32_t)((lane >> 1) & 3) : 0u;
+      next = look(r + 1);
       ok = wait_bounded(acc_full_bar(acc), acc_phase, abort_flag, g.status, g.wait_limit);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
@@ -277,13 +290,13 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
         }
       };
       bool released = false, looked_ahead = false;
-      if (n_w < P.N) {
-        const f32x2 scale2 = splat2(P.scale), skip2 = splat2(P.skip_coef), oc2 = splat2(P.out_coef);
+      if (n_w < cols) {
+        const f32x2 scale2 = splat2(scale), skip2 = splat2(skip_coef), oc2 = splat2(out_coef);
 #pragma unroll 1
         for (int sl = 0; sl < kWarpCols / 32; ++sl) {
           const int col = n_w + 32 * sl;
-          if (col >= P.N) break;
-          const bool last_slice = sl == kWarpCols / 32 - 1 || col + 32 >= P.N;
+          if (col >= cols) break;
+          const bool last_slice = sl == kWarpCols / 32 - 1 || col + 32 >= cols;
           uint4 raw[8];
           if (skip) {
             const int off = (32 * sl) & (in_box_cols - 1);
@@ -301,8 +314,8 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
               if (j < nchunk) raw[j] = ptx::lds128(buf_in + row_off + (((cb + j) ^ sw) << 4));
             if (off + 32 == in_box_cols || last_slice) {
               __syncwarp();                                    // every lane has read the box
-              if (!last_slice) issue_in(P, col + 32, row0);
-              else { prefetch_from(r + 1); looked_ahead = true; }
+              if (!last_slice) issue_in(&P.tskip, col + 32, row0);
+              else { if (next.map) issue_in(next.map, next.col, next.row); looked_ahead = true; }
             }
           }
           const int out_off = (32 * sl) & (out_box_cols - 1);
@@ -315,56 +328,59 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
           if (last_slice) { release_acc(); released = true; }
           const uint32_t out_cb = (uint32_t)(out_off * out_es) >> 4;
           const uint32_t dst = buf_out + (uint32_t)(lane * out_row);
-          uint32_t held[2], copy[8];
+          uint32_t copy[8];
+          float y[32];
+          // The choices of a tile are taken once per slice, not once per eight columns.
 #pragma unroll
-          for (int gi = 0; gi < 4; ++gi) {
-            f32x2 x[4];
+          for (int k = 0; k < 16; ++k) unpack2(mul2(pack2(v[2 * k], v[2 * k + 1]), scale2), y[2 * k], y[2 * k + 1]);
+          if (skip) {
+            if (skip_dt == US_F32) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) x[k] = mul2(pack2(v[8 * gi + 2 * k], v[8 * gi + 2 * k + 1]), scale2);
-            float y[8];
-            if (skip) {
-              float sk[8];
-              if (P.skip_dt == US_F32) {
-                sk[0] = __uint_as_float(raw[2 * gi].x); sk[1] = __uint_as_float(raw[2 * gi].y);
-                sk[2] = __uint_as_float(raw[2 * gi].z); sk[3] = __uint_as_float(raw[2 * gi].w);
-                sk[4] = __uint_as_float(raw[2 * gi + 1].x); sk[5] = __uint_as_float(raw[2 * gi + 1].y);
-                sk[6] = __uint_as_float(raw[2 * gi + 1].z); sk[7] = __uint_as_float(raw[2 * gi + 1].w);
-              } else {
-                const uint32_t w[4] = {raw[gi].x, raw[gi].y, raw[gi].z, raw[gi].w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  const float2 h = P.skip_dt == US_BF16 ? unpack_bf16x2(w[k]) : unpack_f16x2(w[k]);
-                  sk[2 * k] = h.x; sk[2 * k + 1] = h.y;
-                }
+              for (int k = 0; k < 8; ++k) {
+                unpack2(fma2(skip2, pack2(__uint_as_float(raw[k].x), __uint_as_float(raw[k].y)), mul2(oc2, pack2(y[4 * k], y[4 * k + 1]))), y[4 * k], y[4 * k + 1]);
+                unpack2(fma2(skip2, pack2(__uint_as_float(raw[k].z), __uint_as_float(raw[k].w)), mul2(oc2, pack2(y[4 * k + 2], y[4 * k + 3]))), y[4 * k + 2], y[4 * k + 3]);
               }
-#pragma unroll
-              for (int k = 0; k < 4; ++k)
-                unpack2(fma2(skip2, pack2(sk[2 * k], sk[2 * k + 1]), mul2(oc2, x[k])), y[2 * k], y[2 * k + 1]);
-              if (COPY && P.copy) copy_codes(P.out_dt, P.copy_dt, y, &copy[2 * gi]);
             } else {
 #pragma unroll
-              for (int k = 0; k < 4; ++k) unpack2(x[k], y[2 * k], y[2 * k + 1]);
+              for (int k = 0; k < 16; ++k) {
+                const uint32_t w = k % 4 == 0 ? raw[k / 4].x : k % 4 == 1 ? raw[k / 4].y : k % 4 == 2 ? raw[k / 4].z : raw[k / 4].w;
+                const float2 h = skip_dt == US_BF16 ? unpack_bf16x2(w) : unpack_f16x2(w);
+                unpack2(fma2(skip2, pack2(h.x, h.y), mul2(oc2, pack2(y[2 * k], y[2 * k + 1]))), y[2 * k], y[2 * k + 1]);
+              }
             }
-            if (P.out_dt == US_F32) {
-              ptx::sts128(dst + (((out_cb + 2 * gi) ^ out_sw) << 4),
-                          make_uint4(__float_as_uint(y[0]), __float_as_uint(y[1]), __float_as_uint(y[2]), __float_as_uint(y[3])));
-              ptx::sts128(dst + (((out_cb + 2 * gi + 1) ^ out_sw) << 4),
-                          make_uint4(__float_as_uint(y[4]), __float_as_uint(y[5]), __float_as_uint(y[6]), __float_as_uint(y[7])));
-            } else if (P.out_dt == US_BF16 || P.out_dt == US_F16) {
-              uint32_t w[4];
+            if (COPY && P.copy) {
 #pragma unroll
-              for (int k = 0; k < 4; ++k)
-                w[k] = P.out_dt == US_BF16 ? pack_bf16x2(y[2 * k], y[2 * k + 1]) : pack_f16x2(y[2 * k], y[2 * k + 1]);
-              ptx::sts128(dst + (((out_cb + gi) ^ out_sw) << 4), make_uint4(w[0], w[1], w[2], w[3]));
-            } else {
-              const uint32_t lo = P.out_dt == US_E5M2 ? cvt_fp8x4<true>(y[0], y[1], y[2], y[3]) : cvt_fp8x4<false>(y[0], y[1], y[2], y[3]);
-              const uint32_t hi = P.out_dt == US_E5M2 ? cvt_fp8x4<true>(y[4], y[5], y[6], y[7]) : cvt_fp8x4<false>(y[4], y[5], y[6], y[7]);
-              if ((gi & 1) == 0) { held[0] = lo; held[1] = hi; }
-              else ptx::sts128(dst + (((out_cb + (gi >> 1)) ^ out_sw) << 4), make_uint4(held[0], held[1], lo, hi));
+              for (int gi = 0; gi < 4; ++gi) {
+                const float y8[8] = {y[8 * gi], y[8 * gi + 1], y[8 * gi + 2], y[8 * gi + 3], y[8 * gi + 4], y[8 * gi + 5], y[8 * gi + 6], y[8 * gi + 7]};
+                copy_codes(out_dt, P.copy_dt, y8, &copy[2 * gi]);
+              }
             }
           }
+          auto stage = [&](int chunk, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+            ptx::sts128(dst + (((out_cb + chunk) ^ out_sw) << 4), make_uint4(a, b, c, d));
+          };
+          if (out_dt == US_F32) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+              stage(k, __float_as_uint(y[4 * k]), __float_as_uint(y[4 * k + 1]), __float_as_uint(y[4 * k + 2]), __float_as_uint(y[4 * k + 3]));
+          } else if (out_dt == US_BF16) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              stage(k, pack_bf16x2(y[8 * k], y[8 * k + 1]), pack_bf16x2(y[8 * k + 2], y[8 * k + 3]), pack_bf16x2(y[8 * k + 4], y[8 * k + 5]), pack_bf16x2(y[8 * k + 6], y[8 * k + 7]));
+          } else if (out_dt == US_F16) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              stage(k, pack_f16x2(y[8 * k], y[8 * k + 1]), pack_f16x2(y[8 * k + 2], y[8 * k + 3]), pack_f16x2(y[8 * k + 4], y[8 * k + 5]), pack_f16x2(y[8 * k + 6], y[8 * k + 7]));
+          } else {
+            uint32_t w[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+              w[k] = out_dt == US_E5M2 ? cvt_fp8x4<true>(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]) : cvt_fp8x4<false>(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]);
+            stage(0, w[0], w[1], w[2], w[3]);
+            stage(1, w[4], w[5], w[6], w[7]);
+          }
           if (COPY && skip && P.copy && row0 + lane < P.M)
-            copy_store(P.copy + (int64_t)(row0 + lane) * P.copy_ld + col, copy, P.N - col, P.copy_sectors != 0);
+            copy_store(P.copy + (int64_t)(row0 + lane) * P.copy_ld + col, copy, cols - col, P.copy_sectors != 0);
           if (out_off + 32 == out_box_cols || last_slice) {
             ptx::fence_proxy_async_smem();
             __syncwarp();
@@ -375,7 +391,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       if (!released) release_acc();
-      if (!looked_ahead) prefetch_from(r + 1);                 // plain tile, or no columns here: the input box is free, fetch for the next tile
+      if (!looked_ahead && next.map) issue_in(next.map, next.col, next.row);   // plain tile, or no columns here: the input box is free, fetch for the next tile
     }
     if (in_pending && lane == 0)
       for (uint32_t it = 0; it < g.wait_limit && !ptx::mbar_try_wait(in_bar, in_phase); ++it) {}

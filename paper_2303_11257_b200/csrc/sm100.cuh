@@ -24,6 +24,12 @@ __device__ __forceinline__ bool elect_one() {
   return pred != 0;
 }
 
+// A value that is kept in a register from here on: the compiler does not fetch it anew where it is used.
+__device__ __forceinline__ int once(int x) {
+  asm volatile("" : "+r"(x));
+  return x;
+}
+
 // ------------------------------------------------------------------ mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
