@@ -348,37 +348,9 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
                 unpack2(fma2(skip2, pack2(h.x, h.y), mul2(oc2, pack2(y[2 * k], y[2 * k + 1]))), y[2 * k], y[2 * k + 1]);
               }
             }
-            if (COPY && P.copy) {
-#pragma unroll
-              for (int gi = 0; gi < 4; ++gi) {
-                const float y8[8] = {y[8 * gi], y[8 * gi + 1], y[8 * gi + 2], y[8 * gi + 3], y[8 * gi + 4], y[8 * gi + 5], y[8 * gi + 6], y[8 * gi + 7]};
-                copy_codes(out_dt, P.copy_dt, y8, &copy[2 * gi]);
-              }
-            }
+            if (COPY && P.copy) copy_codes32(out_dt, P.copy_dt, y, copy);
           }
-          auto stage = [&](int chunk, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-            ptx::sts128(dst + (((out_cb + chunk) ^ out_sw) << 4), make_uint4(a, b, c, d));
-          };
-          if (out_dt == US_F32) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-              stage(k, __float_as_uint(y[4 * k]), __float_as_uint(y[4 * k + 1]), __float_as_uint(y[4 * k + 2]), __float_as_uint(y[4 * k + 3]));
-          } else if (out_dt == US_BF16) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              stage(k, pack_bf16x2(y[8 * k], y[8 * k + 1]), pack_bf16x2(y[8 * k + 2], y[8 * k + 3]), pack_bf16x2(y[8 * k + 4], y[8 * k + 5]), pack_bf16x2(y[8 * k + 6], y[8 * k + 7]));
-          } else if (out_dt == US_F16) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              stage(k, pack_f16x2(y[8 * k], y[8 * k + 1]), pack_f16x2(y[8 * k + 2], y[8 * k + 3]), pack_f16x2(y[8 * k + 4], y[8 * k + 5]), pack_f16x2(y[8 * k + 6], y[8 * k + 7]));
-          } else {
-            uint32_t w[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-              w[k] = out_dt == US_E5M2 ? cvt_fp8x4<true>(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]) : cvt_fp8x4<false>(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]);
-            stage(0, w[0], w[1], w[2], w[3]);
-            stage(1, w[4], w[5], w[6], w[7]);
-          }
+          stage_row32(out_dt, y, dst, out_cb, out_sw);
           if (COPY && skip && P.copy && row0 + lane < P.M)
             copy_store(P.copy + (int64_t)(row0 + lane) * P.copy_ld + col, copy, cols - col, P.copy_sectors != 0);
           if (out_off + 32 == out_box_cols || last_slice) {

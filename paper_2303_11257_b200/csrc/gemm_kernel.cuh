@@ -64,6 +64,7 @@ __host__ __device__ constexpr int epi_warp_bytes(int ew) { return ew == 16 ? 409
 // What the epilogue fuses, fixed at compile time so that each kernel carries one code path only.
 enum EpiKind {
   kEpiPlain = 0,     // scale, round, store
+  kEpiPlainF32 = 6,  // the same with float32 output, single problems (beside the code of the other types 48 x 1024 x 4096 takes 3.9 us instead of 3.8)
   kEpiGelu = 1,      // + scaled GELU, optionally keeping the 16-bit pre-activation
   kEpiGeluGrad = 2,  // + scaled GELU gradient from the stored pre-activation
   kEpiSkip = 3,      // + weighted skip tensor (residual)
@@ -256,6 +257,40 @@ __device__ __forceinline__ void copy_store(uint8_t* dst, const uint32_t (&codes)
   }
 }
 
+__device__ __forceinline__ void copy_codes32(int dt, int copy_dt, const float (&y)[32], uint32_t (&codes)[8]) {
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    const float y8[8] = {y[8 * g], y[8 * g + 1], y[8 * g + 2], y[8 * g + 3], y[8 * g + 4], y[8 * g + 5], y[8 * g + 6], y[8 * g + 7]};
+    copy_codes(dt, copy_dt, y8, &codes[2 * g]);
+  }
+}
+// A lane's 32 results, rounded to the output format dt, into its row dst of a staging box, from 16-byte chunk `chunk` on: chunk c at c ^ sw.
+// F32: dt may be float32.
+template <bool F32 = true>
+__device__ __forceinline__ void stage_row32(int dt, const float (&y)[32], uint32_t dst, uint32_t chunk, uint32_t sw) {
+  auto put = [&](int c, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3) { ptx::sts128(dst + (((chunk + c) ^ sw) << 4), make_uint4(x0, x1, x2, x3)); };
+  if (F32 && dt == US_F32) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      put(k, __float_as_uint(y[4 * k]), __float_as_uint(y[4 * k + 1]), __float_as_uint(y[4 * k + 2]), __float_as_uint(y[4 * k + 3]));
+  } else if (dt == US_BF16) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      put(k, pack_bf16x2(y[8 * k], y[8 * k + 1]), pack_bf16x2(y[8 * k + 2], y[8 * k + 3]), pack_bf16x2(y[8 * k + 4], y[8 * k + 5]), pack_bf16x2(y[8 * k + 6], y[8 * k + 7]));
+  } else if (dt == US_F16) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      put(k, pack_f16x2(y[8 * k], y[8 * k + 1]), pack_f16x2(y[8 * k + 2], y[8 * k + 3]), pack_f16x2(y[8 * k + 4], y[8 * k + 5]), pack_f16x2(y[8 * k + 6], y[8 * k + 7]));
+  } else {
+    uint32_t w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      w[k] = dt == US_E5M2 ? cvt_fp8x4<true>(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]) : cvt_fp8x4<false>(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]);
+    put(0, w[0], w[1], w[2], w[3]);
+    put(1, w[4], w[5], w[6], w[7]);
+  }
+}
+
 // Bytes per row of an output box of the eight-warp epilogue.
 __host__ __device__ constexpr int out_row_bytes(int bn, int es) { return bn / 2 * es < 128 ? bn / 2 * es : 128; }
 
@@ -280,7 +315,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
   const int in_es = in_kind ? dtype_size(in_dt) : 4;
   const CUtensorMap* tm_in = in_kind == 1 ? tm_aux : tm_skip;
   const bool aux_out = EPI == kEpiGelu && p.aux != nullptr;
-  const int out_es = dtype_size(p.out_dt);
+  const int out_dt = EPI == kEpiPlainF32 ? (int)US_F32 : p.out_dt, out_es = dtype_size(out_dt);
   // Boxes have rows of 128 bytes, or of the fewer bytes that a warp's columns are, swizzled with the pattern of that width (32-byte
   // rows: not): 16-byte chunk c of row r sits at c ^ (r & 7), 64-byte rows c ^ ((r >> 1) & 3).
   const int out_row = out_row_bytes(BN, out_es);
@@ -389,97 +424,68 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
         const f32x2 os2 = splat2(p.act_out * p.act_in), skip2 = splat2(p.skip_coef), oc2 = splat2(p.out_coef);
         const uint32_t aux_cb = (uint32_t)(aux_off * 2) >> 4, out_cb = (uint32_t)(out_off * out_es) >> 4;
         const uint32_t dst = buf_out + out_row_off;
-        uint32_t held[2];                                    // first half of a 16-byte chunk of FP8 codes
         uint32_t copy[8];                                    // the FP8 copy of this lane's 32 columns
-        // Eight values at a time run through the whole chain (scale, kept pre-activation, activation,
-        // residual, rounding, staging store), so that the different execution pipes overlap.
+        // The choices of a launch (types, activation) are taken once per slice: inside the groups of eight columns that the conversions
+        // work on they cost more than the arithmetic (us: BF16 8192 x 1024 x 1024 with GELU 26.1 -> 18.1, its gradient 30.5 -> 19.9; FP8 48 x 1024 x
+        // 4096 with GELU 5.9 -> 4.5; plain, 16 x 8192 x 8192 weight gradient in BF16 31.5 -> 23.9, 2048 x 128 x 8192 10.9 -> 8.9).
+        float y[32];
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          f32x2 x[4];
+        for (int k = 0; k < 16; ++k) unpack2(mul2(pack2(v[2 * k], v[2 * k + 1]), scale2), y[2 * k], y[2 * k + 1]);
+        if (EPI == kEpiGelu) {
+          if (aux_out) {
+            uint32_t w[16];
+            if (p.aux_dt == US_BF16) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) x[k] = mul2(pack2(v[8 * g + 2 * k], v[8 * g + 2 * k + 1]), scale2);
-          float y[8];
-          if (EPI == kEpiGelu) {
-            if (aux_out) {
-              uint32_t w[4];
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                float a, b;
-                unpack2(x[k], a, b);
-                w[k] = p.aux_dt == US_BF16 ? pack_bf16x2(a, b) : pack_f16x2(a, b);
-              }
-              ptx::sts128(buf_aux + aux_row_off + (((aux_cb + g) ^ aux_sw) << 4), make_uint4(w[0], w[1], w[2], w[3]));
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              if (BN == 64 && p.fn == US_FN_GELU && out_es == 1) {     // the form the 16-warp epilogue takes for FP8 outputs of larger tiles
-                gelu_scaled2<true>(x[k], tail_k, act_oi, y[2 * k], y[2 * k + 1]);
-              } else if (p.fn == US_FN_GELU) {
-                gelu_scaled2<false>(x[k], tail_k, act_oi, y[2 * k], y[2 * k + 1]);
-              } else {                                          // relu, tanh, sigmoid (table section "Activations")
-                float a, b;
-                unpack2(x[k], a, b);
-                y[2 * k] = act_scaled(p.fn, a, p.act_in, p.act_out); y[2 * k + 1] = act_scaled(p.fn, b, p.act_in, p.act_out);
-              }
-            }
-          } else if (EPI == kEpiGeluGrad) {
-            const uint32_t w[4] = {raw[g].x, raw[g].y, raw[g].z, raw[g].w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float2 h = in_dt == US_BF16 ? unpack_bf16x2(w[k]) : unpack_f16x2(w[k]);
-              if (p.fn == US_FN_GELU) {
-                unpack2(gelu_grad_scaled2(pack2(h.x, h.y), x[k], in2, os2), y[2 * k], y[2 * k + 1]);
-              } else {
-                float a, b;
-                unpack2(x[k], a, b);
-                y[2 * k] = act_grad_scaled(p.fn, h.x, a, p.act_in, p.act_out); y[2 * k + 1] = act_grad_scaled(p.fn, h.y, b, p.act_in, p.act_out);
-              }
-            }
-          } else if (in_kind == 2) {
-            float sk[8];
-            if (in_dt == US_F32) {
-              sk[0] = __uint_as_float(raw[2 * g].x); sk[1] = __uint_as_float(raw[2 * g].y);
-              sk[2] = __uint_as_float(raw[2 * g].z); sk[3] = __uint_as_float(raw[2 * g].w);
-              sk[4] = __uint_as_float(raw[2 * g + 1].x); sk[5] = __uint_as_float(raw[2 * g + 1].y);
-              sk[6] = __uint_as_float(raw[2 * g + 1].z); sk[7] = __uint_as_float(raw[2 * g + 1].w);
+              for (int k = 0; k < 16; ++k) w[k] = pack_bf16x2(y[2 * k], y[2 * k + 1]);
             } else {
-              const uint32_t w[4] = {raw[g].x, raw[g].y, raw[g].z, raw[g].w};
 #pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                const float2 h = in_dt == US_BF16 ? unpack_bf16x2(w[k]) : unpack_f16x2(w[k]);
-                sk[2 * k] = h.x; sk[2 * k + 1] = h.y;
-              }
+              for (int k = 0; k < 16; ++k) w[k] = pack_f16x2(y[2 * k], y[2 * k + 1]);
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-              unpack2(fma2(skip2, pack2(sk[2 * k], sk[2 * k + 1]), mul2(oc2, x[k])), y[2 * k], y[2 * k + 1]);
+            for (int g = 0; g < 4; ++g)
+              ptx::sts128(buf_aux + aux_row_off + (((aux_cb + g) ^ aux_sw) << 4), make_uint4(w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]));
+          }
+          if (p.fn == US_FN_GELU) {
+            if (BN == 64 && out_es == 1) {                     // the form the 16-warp epilogue takes for FP8 outputs of larger tiles
+#pragma unroll
+              for (int k = 0; k < 16; ++k) gelu_scaled2<true>(pack2(y[2 * k], y[2 * k + 1]), tail_k, act_oi, y[2 * k], y[2 * k + 1]);
+            } else {
+#pragma unroll
+              for (int k = 0; k < 16; ++k) gelu_scaled2<false>(pack2(y[2 * k], y[2 * k + 1]), tail_k, act_oi, y[2 * k], y[2 * k + 1]);
+            }
+          } else {                                              // relu, tanh, sigmoid (table section "Activations")
+#pragma unroll
+            for (int k = 0; k < 32; ++k) y[k] = act_scaled(p.fn, y[k], p.act_in, p.act_out);
+          }
+        } else if (EPI == kEpiGeluGrad) {
+          float h[32];
+          unpack16<32>(raw, in_dt, h);
+          if (p.fn == US_FN_GELU) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+              unpack2(gelu_grad_scaled2(pack2(h[2 * k], h[2 * k + 1]), pack2(y[2 * k], y[2 * k + 1]), in2, os2), y[2 * k], y[2 * k + 1]);
           } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) unpack2(x[k], y[2 * k], y[2 * k + 1]);
+            for (int k = 0; k < 32; ++k) y[k] = act_grad_scaled(p.fn, h[k], y[k], p.act_in, p.act_out);
           }
-          if (EPI == kEpiSkipCopy) copy_codes(p.out_dt, p.aux_dt, y, &copy[2 * g]);
-          // ---- rounding to the output format and staging store of these eight values
-          if (p.out_dt == US_F32) {
-            ptx::sts128(dst + (((out_cb + 2 * g) ^ out_sw) << 4),
-                        make_uint4(__float_as_uint(y[0]), __float_as_uint(y[1]), __float_as_uint(y[2]), __float_as_uint(y[3])));
-            ptx::sts128(dst + (((out_cb + 2 * g + 1) ^ out_sw) << 4),
-                        make_uint4(__float_as_uint(y[4]), __float_as_uint(y[5]), __float_as_uint(y[6]), __float_as_uint(y[7])));
-          } else if (p.out_dt == US_BF16 || p.out_dt == US_F16) {
-            uint32_t w[4];
+        } else if (in_kind == 2) {
+          float sk[32];
+          if (in_dt == US_F32) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-              w[k] = p.out_dt == US_BF16 ? pack_bf16x2(y[2 * k], y[2 * k + 1]) : pack_f16x2(y[2 * k], y[2 * k + 1]);
-            ptx::sts128(dst + (((out_cb + g) ^ out_sw) << 4), make_uint4(w[0], w[1], w[2], w[3]));
-          } else {
-            const uint32_t lo = p.out_dt == US_E5M2 ? cvt_fp8x4<true>(y[0], y[1], y[2], y[3]) : cvt_fp8x4<false>(y[0], y[1], y[2], y[3]);
-            const uint32_t hi = p.out_dt == US_E5M2 ? cvt_fp8x4<true>(y[4], y[5], y[6], y[7]) : cvt_fp8x4<false>(y[4], y[5], y[6], y[7]);
-            if ((g & 1) == 0) {
-              held[0] = lo; held[1] = hi;
-            } else {
-              ptx::sts128(dst + (((out_cb + (g >> 1)) ^ out_sw) << 4), make_uint4(held[0], held[1], lo, hi));
+            for (int k = 0; k < 8; ++k) {
+              sk[4 * k] = __uint_as_float(raw[k].x); sk[4 * k + 1] = __uint_as_float(raw[k].y);
+              sk[4 * k + 2] = __uint_as_float(raw[k].z); sk[4 * k + 3] = __uint_as_float(raw[k].w);
             }
+          } else {
+            unpack16<32>(raw, in_dt, sk);
           }
+#pragma unroll
+          for (int k = 0; k < 16; ++k)
+            unpack2(fma2(skip2, pack2(sk[2 * k], sk[2 * k + 1]), mul2(oc2, pack2(y[2 * k], y[2 * k + 1]))), y[2 * k], y[2 * k + 1]);
         }
+        if (EPI == kEpiSkipCopy) copy_codes32(p.out_dt, p.aux_dt, y, copy);
+        // ---- rounding to the output format and staging stores
+        stage_row32<EPI != kEpiPlain || BATCHED>(out_dt, y, dst, out_cb, out_sw);
         if (EPI == kEpiSkipCopy && row0 + lane < p.M)
           copy_store(static_cast<uint8_t*>(p.aux) + (int64_t)(row0 + lane) * p.aux_ld + col, copy, p.N - col, p.aux_sectors != 0);
         // ---- boxes completed by this slice go out
