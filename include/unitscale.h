@@ -111,6 +111,10 @@ typedef struct {
  * and columns need not be multiples of the tile sizes.  Alignment rule: see
  * us_mat (violations return US_ERR_ALIGNMENT).
  *
+ * Where an output has few tiles and the contraction is long (more than 2432 bytes of an operand's K, for
+ * weight gradients 6016) without a fused activation, up to eight SMs may share a tile: each sums a part of the
+ * contraction in float32 and one adds the parts in a fixed order.  Repeated calls give identical results.
+ *
  * ws: device workspace of at least us_workspace_bytes() bytes, 16-byte aligned,
  * zeroed once by the caller before its first use (cudaMemsetAsync).  It holds a
  * status word that a kernel sets if one of its bounded waits runs out.  The word
@@ -162,8 +166,9 @@ us_status us_linear_bwd_w_batched(const us_mat* X, const us_mat* G, float beta_w
  * us_linear_group: count (1..4) independent linear ops as ONE kernel launch.
  *
  * Each call is one of the three GEMMs of section "Example" with the same arithmetic, rounding and
- * scale handling as the single entry points (bit-identical results: a tile is always accumulated by
- * one accumulator over its whole K range).  The ops must not depend on one another (no output of one
+ * scale handling as the single entry points.  Here a tile is always accumulated by one accumulator
+ * over its whole K range; results are bit-identical to those of the single entry points wherever these
+ * do the same (they may share long contractions among several SMs, see us_linear_fwd).  The ops must not depend on one another (no output of one
  * is an operand, skip tensor or output of another).  Meant for the tail of a training step, where
  * several GEMMs of different shapes are ready at once -- for the FFN block the second forward GEMM,
  * both weight-gradient GEMMs and the first layer's input-gradient GEMM -- and separate launches

@@ -334,20 +334,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
 #pragma unroll
           for (int k = 0; k < 16; ++k) unpack2(mul2(pack2(v[2 * k], v[2 * k + 1]), scale2), y[2 * k], y[2 * k + 1]);
           if (skip) {
-            if (skip_dt == US_F32) {
-#pragma unroll
-              for (int k = 0; k < 8; ++k) {
-                unpack2(fma2(skip2, pack2(__uint_as_float(raw[k].x), __uint_as_float(raw[k].y)), mul2(oc2, pack2(y[4 * k], y[4 * k + 1]))), y[4 * k], y[4 * k + 1]);
-                unpack2(fma2(skip2, pack2(__uint_as_float(raw[k].z), __uint_as_float(raw[k].w)), mul2(oc2, pack2(y[4 * k + 2], y[4 * k + 3]))), y[4 * k + 2], y[4 * k + 3]);
-              }
-            } else {
-#pragma unroll
-              for (int k = 0; k < 16; ++k) {
-                const uint32_t w = k % 4 == 0 ? raw[k / 4].x : k % 4 == 1 ? raw[k / 4].y : k % 4 == 2 ? raw[k / 4].z : raw[k / 4].w;
-                const float2 h = skip_dt == US_BF16 ? unpack_bf16x2(w) : unpack_f16x2(w);
-                unpack2(fma2(skip2, pack2(h.x, h.y), mul2(oc2, pack2(y[2 * k], y[2 * k + 1]))), y[2 * k], y[2 * k + 1]);
-              }
-            }
+            residual_row32(skip_dt, raw, skip2, oc2, y);
             if (COPY && P.copy) copy_codes32(out_dt, P.copy_dt, y, copy);
           }
           stage_row32(out_dt, y, dst, out_cb, out_sw);

@@ -47,6 +47,7 @@ struct GemmParams {
   unsigned int* status;
   uint32_t wait_limit;                      // polls a bounded wait makes before it gives up (kWaitLimit unless a test shortens it)
   int no_loads;                             // test hook: the producer issues no operand loads, so that the waits run out
+  int splits;                               // CTAs (or pairs) that share a tile's contraction (gemm_split.cuh; 1: none)
   uint32_t a_bytes, stages;                 // narrow tiles (BN = 64): bytes of A in a stage, and the stages that fit
 };
 
@@ -291,6 +292,23 @@ __device__ __forceinline__ void stage_row32(int dt, const float (&y)[32], uint32
   }
 }
 
+// A lane's 32 scaled results y with its row's skip values, as read from a box: y = skip_coef * skip + out_coef * y.
+__device__ __forceinline__ void residual_row32(int skip_dt, const uint4 (&raw)[8], f32x2 skip2, f32x2 oc2, float (&y)[32]) {
+  float sk[32];
+  if (skip_dt == US_F32) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      sk[4 * k] = __uint_as_float(raw[k].x); sk[4 * k + 1] = __uint_as_float(raw[k].y);
+      sk[4 * k + 2] = __uint_as_float(raw[k].z); sk[4 * k + 3] = __uint_as_float(raw[k].w);
+    }
+  } else {
+    unpack16<32>(raw, skip_dt, sk);
+  }
+#pragma unroll
+  for (int k = 0; k < 16; ++k)
+    unpack2(fma2(skip2, pack2(sk[2 * k], sk[2 * k + 1]), mul2(oc2, pack2(y[2 * k], y[2 * k + 1]))), y[2 * k], y[2 * k + 1]);
+}
+
 // Bytes per row of an output box of the eight-warp epilogue.
 __host__ __device__ constexpr int out_row_bytes(int bn, int es) { return bn / 2 * es < 128 ? bn / 2 * es : 128; }
 
@@ -469,19 +487,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
             for (int k = 0; k < 32; ++k) y[k] = act_grad_scaled(p.fn, h[k], y[k], p.act_in, p.act_out);
           }
         } else if (in_kind == 2) {
-          float sk[32];
-          if (in_dt == US_F32) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              sk[4 * k] = __uint_as_float(raw[k].x); sk[4 * k + 1] = __uint_as_float(raw[k].y);
-              sk[4 * k + 2] = __uint_as_float(raw[k].z); sk[4 * k + 3] = __uint_as_float(raw[k].w);
-            }
-          } else {
-            unpack16<32>(raw, in_dt, sk);
-          }
-#pragma unroll
-          for (int k = 0; k < 16; ++k)
-            unpack2(fma2(skip2, pack2(sk[2 * k], sk[2 * k + 1]), mul2(oc2, pack2(y[2 * k], y[2 * k + 1]))), y[2 * k], y[2 * k + 1]);
+          residual_row32(in_dt, raw, skip2, oc2, y);
         }
         if (EPI == kEpiSkipCopy) copy_codes32(p.out_dt, p.aux_dt, y, copy);
         // ---- rounding to the output format and staging stores

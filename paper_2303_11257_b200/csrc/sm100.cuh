@@ -224,6 +224,10 @@ __device__ __forceinline__ void mbar_arrive_relaxed_cluster(uint32_t bar) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// Four floats to a CTA of the cluster (a shared::cluster address); ordered by the next cluster_sync.
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, const float* v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+}
 // Two words to a CTA of the cluster (a shared::cluster address); ordered by the next cluster_sync.
 __device__ __forceinline__ void st_cluster_v2(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");

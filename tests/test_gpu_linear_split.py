@@ -1,0 +1,70 @@
+"""Linear ops whose contraction is shared by the CTAs of a cluster (few output tiles, long K): two, four and eight CTAs on tiles of 128 x 64
+and 128 x 128, two and four CTA pairs on 256 x 256, with rows, columns and K blocks that do not divide.  A part of the contraction is a
+float32 sum like the whole, so the bounds are those of the unshared kernels."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import ops as O
+from tests import util as U
+from tests.test_gpu_linear_narrow import PAD, TOL, _operands
+
+pytestmark = pytest.mark.gpu
+
+# rows, contraction, columns
+SHAPES = [(1, 2576, 16), (48, 4096, 1024), (130, 5008, 700), (300, 5008, 690), (500, 6160, 1300), (2048, 6400, 1024), (1000, 8208, 700)]
+
+
+@pytest.mark.parametrize("op,fmt,out_fmt", [("fwd", "e4m3", "bf16"), ("fwd", "bf16", "f32"), ("fwd", "fp16", "e4m3"), ("bwd_x", "e4m3", "f32"),
+                                            ("bwd_x", "bf16", "bf16"), ("bwd_w", "e4m3", "f32"), ("bwd_w", "bf16", "f32")])
+@pytest.mark.parametrize("rows,k,cols", SHAPES)
+def test_shared_contraction(op, fmt, out_fmt, rows, k, cols):
+    from paper_2303_11257_b200 import lib as L, synth
+    fb = "e5m2" if fmt == "e4m3" and op != "fwd" else fmt
+    A, B, val, scale = _operands(L, synth, op, rows, k, cols, 81, fmt, fb)
+    ws, fn = L.new_workspace(), getattr(L, "us_linear_" + op)
+    out, again = U.empty(rows, cols, out_fmt, PAD(cols)), U.empty(rows, cols, out_fmt, PAD(cols))
+    tol = TOL * max(1.0, np.abs(val).max() / 4)
+    fn(A, B, scale, out, ws)
+    for _ in range(3):
+        fn(A, B, scale, again, ws)
+    assert L.us_workspace_status(ws) == 0
+    U.assert_close_stored(out, val, out_fmt, tol, f"{op} plain")
+    assert torch.equal(out.contiguous().view(torch.uint8), again.contiguous().view(torch.uint8))
+    if PAD(cols) > cols:
+        assert not out.as_strided((rows, PAD(cols)), (PAD(cols), 1))[:, cols:].contiguous().view(torch.uint8).any()
+    for skip_fmt in ("f32", "bf16"):
+        sk = synth.normal(81, 2, (rows, cols))
+        out = U.empty(rows, cols, out_fmt, PAD(cols))
+        fn(A, B, scale, out, ws, L.epilogue(skip=U.to_device(sk, skip_fmt, PAD(cols)), skip_coef=0.8, out_coef=0.6))
+        assert L.us_workspace_status(ws) == 0
+        U.assert_close_stored(out, O.weighted_add(U.values_of(sk, skip_fmt), val, np.float32(0.8), np.float32(0.6)), out_fmt, tol, f"{op} residual {skip_fmt}")
+
+
+@pytest.mark.parametrize("rows,k,cols", [(48, 4096, 1024), (2048, 6400, 1024)])
+def test_shared_contraction_with_a_copy_in_fp8(rows, k, cols):
+    from paper_2303_11257_b200 import lib as L, synth
+    X, W, val, scale = _operands(L, synth, "fwd", rows, k, cols, 82, "e4m3", "e4m3")
+    ws, out, q = L.new_workspace(), U.empty(rows, cols, "bf16"), U.empty(rows, cols, "e4m3")
+    sk = synth.normal(82, 2, (rows, cols))
+    plan = L.Plan((), ())
+    ep = L.epilogue(skip=U.to_device(sk, "f32"), skip_coef=0.8, out_coef=0.6)
+    L.Call("us_linear_fwd_cast", plan.mat(X), plan.mat(W), scale, ep, plan.mat(out), plan.mat(q), ws.data_ptr(), ws.numel())(L.current_stream())
+    assert L.us_workspace_status(ws) == 0
+    U.assert_close_stored(out, O.weighted_add(U.values_of(sk, "f32"), val, np.float32(0.8), np.float32(0.6)), "bf16", TOL * max(1.0, np.abs(val).max() / 4), "residual")
+    assert torch.equal(q.view(torch.uint8), out.float().clamp(-448, 448).to(torch.float8_e4m3fn).view(torch.uint8))
+
+
+def test_waits_that_run_out_in_a_cluster():
+    """Operand loads withheld: every CTA's waits run out, the cluster's barriers are passed all the same, the status says so, and
+    the next call is correct."""
+    from paper_2303_11257_b200 import lib as L, synth
+    for rows, k, cols in ((48, 4096, 1024), (2048, 6400, 1024)):
+        X, W, val, scale = _operands(L, synth, "fwd", rows, k, cols, 83, "e4m3", "e4m3")
+        ws, out = L.new_workspace(), U.empty(rows, cols, "bf16")
+        L.us_test_linear_fwd_starved(X, W, scale, out, ws, 2000)
+        assert L.us_workspace_status(ws) == L.US_ERR_TIMEOUT
+        ws.zero_()
+        L.us_linear_fwd(X, W, scale, out, ws)
+        assert L.us_workspace_status(ws) == 0
+        U.assert_close_stored(out, val, "bf16", TOL * max(1.0, np.abs(val).max() / 4), "after")
