@@ -334,6 +334,8 @@ typedef enum { US_FN_GELU = 0, US_FN_RELU = 1, US_FN_TANH = 2, US_FN_SIGMOID = 3
  *                  nothing is launched.  Tensors must not overlap.
  * us_cast_multi    the same launch with BF16 / F16 destinations allowed (the 16-bit alternative of a step's operands):
  *                  one rounding of scale[i] * src[i], as us_residual_add with tau = 0 rounds it.
+ * us_cast_multi_pitched  us_cast_multi whose destinations may have padded rows, of a multiple of 16 columns and
+ *                  starting on 16-byte boundaries (matmul operands are read fastest with rows on 128-byte ones).
  *
  * Inputs may be F32, BF16 or F16 (us_weighted_add also takes E4M3 / E5M2 inputs: partial results that travelled
  * in 8 bits); outputs any us_dtype (us_cast_fp8, us_cast_fp8_multi: E4M3 or E5M2 only).  0 <= tau <= 1.
@@ -352,6 +354,7 @@ us_status us_cast_fp8(const us_mat* src, float scale, const us_mat* dst, void* s
 us_status us_cast_fp8_multi(int count, const us_mat* src, const float* scale, const us_mat* dst,
                             void* stream);
 us_status us_cast_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, void* stream);
+us_status us_cast_multi_pitched(int count, const us_mat* src, const float* scale, const us_mat* dst, void* stream);
 
 /* ------------------------------------------------------------ fused scaled dot-product attention (forward)
  *

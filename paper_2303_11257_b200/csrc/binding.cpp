@@ -212,7 +212,7 @@ const Known kKnown[] = {
     US_CALL(us_linear_fwd), US_CALL(us_linear_bwd_x), US_CALL(us_linear_bwd_w), US_CALL(us_linear_fwd_batched), US_CALL(us_linear_bwd_x_batched),
     US_CALL(us_linear_bwd_w_batched), US_ARRAYS(us_linear_group, 1), US_ARRAYS(us_linear_group_any, 1), US_CALL(us_ffn_hidden), US_CALL(us_ffn_hidden_any),
     US_CALL(us_attention_fwd), US_CALL(us_attention_bwd), US_CALL(us_attention_bwd_all), US_CALL(us_cast_fp8), US_ARRAYS(us_cast_fp8_multi, 3),
-    US_ARRAYS(us_cast_multi, 3), US_CALL(us_residual_add), US_CALL(us_gelu_fwd), US_CALL(us_gelu_bwd), US_CALL(us_activation_fwd),
+    US_ARRAYS(us_cast_multi, 3), US_ARRAYS(us_cast_multi_pitched, 3), US_CALL(us_residual_add), US_CALL(us_gelu_fwd), US_CALL(us_gelu_bwd), US_CALL(us_activation_fwd),
     US_CALL(us_activation_bwd), US_ARRAYS(us_weighted_add, 2), US_CALL(us_softmax_fwd), US_CALL(us_softmax_bwd), US_CALL(us_softmax_xent_fwd),
     US_CALL(us_softmax_xent_bwd), US_CALL(us_layer_norm_fwd), US_CALL(us_layer_norm_bwd), US_CALL(us_linear_fwd_cast), US_ARRAYS(us_linear_group_cast, 2),
     US_CALL(us_layer_norm_fwd_cast), US_CALL(us_layer_norm_bwd_cast),

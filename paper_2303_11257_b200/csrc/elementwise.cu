@@ -152,11 +152,16 @@ struct MultiCastArgs {
   float scale[kMultiMax];
   int src_dt[kMultiMax], dst_dt[kMultiMax];
   int count;
+  // destinations with padded rows: chunks per row (0: no padding), its divisor, and elements from row to row
+  uint32_t row_chunks[kMultiMax];
+  FastDiv d_row[kMultiMax];
+  int64_t dst_ld[kMultiMax];
 };
 
 struct MultiChunk {
   const char* src; char* dst; float scale; int sdt, ddt, t; int64_t e0; bool full;
 };
+template <bool PITCHED>
 __device__ __forceinline__ MultiChunk multi_locate(const MultiCastArgs& p, int64_t c) {
   MultiChunk m;
   int t = 0;
@@ -166,6 +171,10 @@ __device__ __forceinline__ MultiChunk multi_locate(const MultiCastArgs& p, int64
   m.sdt = p.src_dt[t]; m.ddt = p.dst_dt[t];
   m.src = static_cast<const char*>(p.src[t]) + m.e0 * dtype_size(m.sdt);
   m.dst = static_cast<char*>(p.dst[t]) + m.e0 * dtype_size(m.ddt);
+  if (PITCHED && p.row_chunks[t]) {                      // whole chunks only: such rows are a multiple of one long
+    const int i = (int)(c - (t ? p.chunk_end[t - 1] : 0)), row = p.d_row[t].div(i);
+    m.dst = static_cast<char*>(p.dst[t]) + (row * p.dst_ld[t] + (int64_t)(i - row * (int)p.row_chunks[t]) * kVec) * dtype_size(m.ddt);
+  }
   m.scale = p.scale[t];
   m.full = m.e0 + kVec <= p.elems[t];
   return m;
@@ -182,13 +191,14 @@ __device__ __forceinline__ void multi_tail(const MultiCastArgs& p, const MultiCh
 }
 
 // Two chunks per thread and iteration, both loaded before either is stored, to keep more loads in flight.
+template <bool PITCHED>
 __global__ void __launch_bounds__(kThreads) multi_cast_kernel(const MultiCastArgs p) {
   const int64_t total = p.chunk_end[p.count - 1];
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   for (int64_t c = blockIdx.x * (int64_t)kThreads + threadIdx.x + ptx::grid_sync_previous(); c < total; c += 2 * stride) {
-    const MultiChunk m0 = multi_locate(p, c);
+    const MultiChunk m0 = multi_locate<PITCHED>(p, c);
     const bool two = c + stride < total;
-    const MultiChunk m1 = two ? multi_locate(p, c + stride) : m0;
+    const MultiChunk m1 = two ? multi_locate<PITCHED>(p, c + stride) : m0;
     float a[kVec], b[kVec];
     if (m0.full) load_vec<kVec>(m0.src, m0.sdt, a);
     if (two && m1.full) load_vec<kVec>(m1.src, m1.sdt, b);
@@ -330,11 +340,13 @@ extern "C" us_status us_cast_fp8(const us_mat* src, float scale, const us_mat* d
   return ew_launch<kCast>(src, nullptr, dst, scale, 0.f, stream);
 }
 
-static us_status cast_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, bool to16, void* stream) {
+// pitched: destinations may have padded rows.
+static us_status cast_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, bool to16, void* stream, bool pitched = false) {
   if (count < 1 || count > kMultiMax || !src || !scale || !dst) return US_ERR_INVALID_ARG;
   MultiCastArgs p{};
   int64_t chunks = 0;
   int used = 0;
+  bool padded = false;
   for (int i = 0; i < count; ++i) {
     us_status s = check_ew(&src[i], nullptr, &dst[i]);
     if (s != US_OK) return s;
@@ -343,7 +355,15 @@ static us_status cast_multi(int count, const us_mat* src, const float* scale, co
     const int64_t n = src[i].rows * src[i].cols;
     if (n == 0) continue;
     const bool dense = (src[i].ld == src[i].cols && dst[i].ld == dst[i].cols) || src[i].rows == 1;
-    if (!dense) return US_ERR_UNSUPPORTED;                               // padded rows: use us_cast_fp8
+    const bool rows = pitched && !dense && src[i].ld == src[i].cols && dst[i].cols % kVec == 0 && n / kVec < 0x7fffffffll;
+    if (!dense && !rows) return US_ERR_UNSUPPORTED;                      // padded rows: use us_cast_fp8
+    if (rows) {
+      if (dst[i].ld * dtype_size(dst[i].dtype) % 16) return US_ERR_ALIGNMENT;
+      p.row_chunks[used] = (uint32_t)(dst[i].cols / kVec);
+      p.d_row[used] = make_fast_div((int)p.row_chunks[used]);
+      p.dst_ld[used] = dst[i].ld;
+      padded = true;
+    }
     if (reinterpret_cast<uintptr_t>(src[i].ptr) % 16 || reinterpret_cast<uintptr_t>(dst[i].ptr) % 16) return US_ERR_ALIGNMENT;
     p.src[used] = src[i].ptr; p.dst[used] = dst[i].ptr; p.elems[used] = n; p.scale[used] = scale[i];
     p.src_dt[used] = src[i].dtype; p.dst_dt[used] = dst[i].dtype;
@@ -357,7 +377,7 @@ static us_status cast_multi(int count, const us_mat* src, const float* scale, co
   if (sms <= 0) return US_ERR_CUDA;
   const int64_t want = (chunks + kThreads - 1) / kThreads;
   const int64_t cap = (int64_t)sms * 8;
-  return host::launch(multi_cast_kernel, nullptr, (int)(want < cap ? want : cap), kThreads, 0, 1, static_cast<cudaStream_t>(stream), p);
+  return host::launch(padded ? multi_cast_kernel<true> : multi_cast_kernel<false>, nullptr, (int)(want < cap ? want : cap), kThreads, 0, 1, static_cast<cudaStream_t>(stream), p);
 }
 
 extern "C" us_status us_cast_fp8_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, void* stream) {
@@ -365,6 +385,9 @@ extern "C" us_status us_cast_fp8_multi(int count, const us_mat* src, const float
 }
 extern "C" us_status us_cast_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, void* stream) {
   return cast_multi(count, src, scale, dst, true, stream);
+}
+extern "C" us_status us_cast_multi_pitched(int count, const us_mat* src, const float* scale, const us_mat* dst, void* stream) {
+  return cast_multi(count, src, scale, dst, true, stream, true);
 }
 
 extern "C" us_status us_weighted_add(int count, const us_mat* src, const float* gamma, float alpha, const us_mat* out,

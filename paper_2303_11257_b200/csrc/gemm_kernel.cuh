@@ -294,19 +294,20 @@ __device__ __forceinline__ void stage_row32(int dt, const float (&y)[32], uint32
 
 // A lane's 32 scaled results y with its row's skip values, as read from a box: y = skip_coef * skip + out_coef * y.
 __device__ __forceinline__ void residual_row32(int skip_dt, const uint4 (&raw)[8], f32x2 skip2, f32x2 oc2, float (&y)[32]) {
-  float sk[32];
   if (skip_dt == US_F32) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      sk[4 * k] = __uint_as_float(raw[k].x); sk[4 * k + 1] = __uint_as_float(raw[k].y);
-      sk[4 * k + 2] = __uint_as_float(raw[k].z); sk[4 * k + 3] = __uint_as_float(raw[k].w);
+      unpack2(fma2(skip2, pack2(__uint_as_float(raw[k].x), __uint_as_float(raw[k].y)), mul2(oc2, pack2(y[4 * k], y[4 * k + 1]))), y[4 * k], y[4 * k + 1]);
+      unpack2(fma2(skip2, pack2(__uint_as_float(raw[k].z), __uint_as_float(raw[k].w)), mul2(oc2, pack2(y[4 * k + 2], y[4 * k + 3]))), y[4 * k + 2], y[4 * k + 3]);
     }
   } else {
-    unpack16<32>(raw, skip_dt, sk);
-  }
 #pragma unroll
-  for (int k = 0; k < 16; ++k)
-    unpack2(fma2(skip2, pack2(sk[2 * k], sk[2 * k + 1]), mul2(oc2, pack2(y[2 * k], y[2 * k + 1]))), y[2 * k], y[2 * k + 1]);
+    for (int k = 0; k < 16; ++k) {
+      const uint32_t w = k % 4 == 0 ? raw[k / 4].x : k % 4 == 1 ? raw[k / 4].y : k % 4 == 2 ? raw[k / 4].z : raw[k / 4].w;
+      const float2 h = skip_dt == US_BF16 ? unpack_bf16x2(w) : unpack_f16x2(w);
+      unpack2(fma2(skip2, pack2(h.x, h.y), mul2(oc2, pack2(y[2 * k], y[2 * k + 1]))), y[2 * k], y[2 * k + 1]);
+    }
+  }
 }
 
 // Bytes per row of an output box of the eight-warp epilogue.

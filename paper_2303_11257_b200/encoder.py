@@ -270,8 +270,8 @@ class UnitScaledEncoderLayer:
         f = self.ffn
         # every tensor that is known when the step starts goes to FP8 in one launch (with post-norm the FFN
         # block's incoming gradient is produced by the second norm's backward pass and is cast there)
-        L.us_cast_fp8_multi([Wqkv, Wo, X, W1, W2] + ([] if post else [G]), [1.0] * (5 if post else 6),
-                            [self.Wqkv_q, self.Wo_q, self.Xq, f.W1q, f.W2q] + ([] if post else [f.Gq]), stream)
+        dsts = [self.Wqkv_q, self.Wo_q, self.Xq, f.W1q, f.W2q] + ([] if post else [f.Gq])
+        (L.us_cast_multi_pitched if L._padded(dsts) else L.us_cast_fp8_multi)([Wqkv, Wo, X, W1, W2] + ([] if post else [G]), [1.0] * len(dsts), dsts, stream)
         L.us_linear_fwd(self.Xq, self.Wqkv_q, sc["alpha_qkv"], self.QKV, ws, None, stream)
         Q, K, V = (self._heads(self.QKV, i) for i in range(3))
         if self.fused_attention:

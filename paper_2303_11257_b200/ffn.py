@@ -72,10 +72,11 @@ class UnitScaledFFN:
         self.operand = operand
         act_dt, grad_dt = _OPERAND[operand]
         e = lambda r, c, dt: torch.empty((r, c), dtype=dt, device=device)
-        self.Xq, self.W1q, self.W2q, self.Gq = e(T, d, act_dt), e(d, f, act_dt), e(f, d, act_dt), e(T, d, grad_dt)
+        op = lambda r, c, dt: L.operand(r, c, dt, device)          # matmul operands: rows on 128-byte boundaries
+        self.Xq, self.W1q, self.W2q, self.Gq = op(T, d, act_dt), op(d, f, act_dt), op(f, d, act_dt), op(T, d, grad_dt)
         self.H = e(T, f, h_dtype)
-        self.Aq = e(T, f, act_dt)
-        self.dHq = e(T, f, grad_dt)
+        self.Aq = op(T, f, act_dt)
+        self.dHq = op(T, f, grad_dt)
         self.R, self.dX = e(T, d, io_dtype), e(T, d, io_dtype)
         self.dW1 = e(d, f, torch.float32)
         self.dW2 = e(f, d, torch.float32)
@@ -199,7 +200,8 @@ class UnitScaledFFN:
 
     def _cast_all(self, X, W1, W2, G, stream):
         try:
-            L.us_cast_multi([W1, W2, X, G], [1.0] * 4, [self.W1q, self.W2q, self.Xq, self.Gq], stream)
+            dsts = [self.W1q, self.W2q, self.Xq, self.Gq]
+            (L.us_cast_multi_pitched if L._padded(dsts) else L.us_cast_multi)([W1, W2, X, G], [1.0] * 4, dsts, stream)
         except L.UnitScaleError as e:
             if self.operand == "fp8" or e.status not in (L.US_ERR_UNSUPPORTED, L.US_ERR_ALIGNMENT):
                 raise

@@ -128,7 +128,7 @@ def _load() -> C.CDLL:
     lib.us_activation_fwd.argtypes = [C.c_int, MP, F, F, MP, V]
     lib.us_activation_bwd.argtypes = [C.c_int, MP, MP, F, F, MP, V]
     lib.us_activation_fwd.restype = lib.us_activation_bwd.restype = C.c_int
-    lib.us_cast_fp8_multi.argtypes = lib.us_cast_multi.argtypes = [C.c_int, MP, C.POINTER(C.c_float), MP, V]
+    lib.us_cast_fp8_multi.argtypes = lib.us_cast_multi.argtypes = lib.us_cast_multi_pitched.argtypes = [C.c_int, MP, C.POINTER(C.c_float), MP, V]
     lib.us_weighted_add.argtypes = [C.c_int, MP, C.POINTER(C.c_float), F, MP, V]
     lib.us_weighted_add.restype = C.c_int
     lib.us_softmax_fwd.argtypes = [MP, F, MP, V]
@@ -145,7 +145,7 @@ def _load() -> C.CDLL:
     lib.us_quant_stats_workspace_bytes.restype = SZ
     lib.us_quant_stats.argtypes = [MP, F, C.c_int, C.c_int, C.c_int, V, V, V, SZ, V]
     lib.us_quant_stats.restype = C.c_int
-    for name in ("us_gelu_fwd", "us_gelu_bwd", "us_residual_add", "us_cast_fp8", "us_cast_fp8_multi", "us_cast_multi", "us_softmax_fwd", "us_softmax_bwd"):
+    for name in ("us_gelu_fwd", "us_gelu_bwd", "us_residual_add", "us_cast_fp8", "us_cast_fp8_multi", "us_cast_multi", "us_cast_multi_pitched", "us_softmax_fwd", "us_softmax_bwd"):
         getattr(lib, name).restype = C.c_int
     FP = C.POINTER(C.c_float)
     lib.us_scales_linear.argtypes = [C.c_int64, C.c_int64, C.c_int64, C.c_int, FP, FP, FP]
@@ -328,7 +328,7 @@ class Plan:
         self.program = names, _binding.program(steps, slots)
 
     def cast_multi(self, srcs, dsts, padded=False):
-        """us_cast_multi at scale 1; an entry of srcs is a tensor or the name of an input.  padded: rows that it does not
+        """us_cast_multi (us_cast_multi_pitched where a destination has padded rows) at scale 1; an entry of srcs is a tensor or the name of an input.  padded: rows that it does not
         take (padded or unaligned ones) go out as one us_residual_add per tensor, for 16-bit destinations."""
         n = len(srcs)
         sm = (us_mat * n)()
@@ -343,7 +343,7 @@ class Plan:
             for s, d in zip(sm, dm):
                 _check("us_residual_add", _entry("us_residual_add")(s, s, 0.0, d, stream))
 
-        return Call("us_cast_multi", n, sm, (C.c_float * n)(*[1.0] * n), dm,
+        return Call("us_cast_multi_pitched" if _padded(dsts) else "us_cast_multi", n, sm, (C.c_float * n)(*[1.0] * n), dm,
                     instead=((US_ERR_UNSUPPORTED, US_ERR_ALIGNMENT) if padded else (), each))
 
     def residual(self, skip, coef):
@@ -669,6 +669,25 @@ def us_cast_fp8_multi(srcs, scales, dsts, stream=None, name="us_cast_fp8_multi")
 def us_cast_multi(srcs, scales, dsts, stream=None):
     """us_cast_fp8_multi with BF16 / F16 destinations allowed."""
     return us_cast_fp8_multi(srcs, scales, dsts, stream, "us_cast_multi")
+
+
+def us_cast_multi_pitched(srcs, scales, dsts, stream=None):
+    """us_cast_multi with destinations whose rows may be padded."""
+    return us_cast_fp8_multi(srcs, scales, dsts, stream, "us_cast_multi_pitched")
+
+
+def operand(rows: int, cols: int, dtype, device="cuda") -> torch.Tensor:
+    """An uninitialised matmul operand [rows x cols] with rows on 128-byte boundaries, the width of the boxes in which a GEMM fetches
+    it: a box of rows on 16-byte boundaries touches two lines a row and takes twice as long (1000 x 2096 x 2096, FP8, input gradient, rows
+    of 2096 / 2112 / 2176 bytes: 10.0 / 7.5 / 6.6 us; BF16 12.5 / 9.5 / 9.5).  Rows of less than 128 bytes, and columns that are no multiple
+    of 16, are not padded."""
+    per = 128 // dtype.itemsize
+    pitch = -(-cols // per) * per if cols % 16 == 0 and cols >= per else cols
+    return torch.empty((rows, pitch), dtype=dtype, device=device)[:, :cols]
+
+
+def _padded(dsts) -> bool:
+    return any(t.stride(0) != t.shape[1] for t in dsts)
 
 
 def us_softmax_fwd(S, alpha, P, stream=None):

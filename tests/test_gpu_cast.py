@@ -153,3 +153,31 @@ def test_cast_multi_errors_launch_nothing():
     assert e.value.status == 3
     torch.cuda.synchronize()
     assert not da.view(torch.uint8).any()                            # the valid first tensor was not written either
+
+
+@pytest.mark.parametrize("src_fmt", ["f32", "bf16"])
+def test_cast_multi_into_padded_rows(src_fmt):
+    """Destinations with padded rows beside dense ones, one row, more chunks than a grid takes at once: the codes of single casts, and
+    nothing written between the rows; what the other forms refuse stays refused."""
+    from paper_2303_11257_b200 import lib as L, synth
+    shapes = [(5, 16, 32, "e4m3"), (1, 144, 256, "e5m2"), (3000, 528, 640, "e4m3"), (64, 96, 96, "bf16"), (33, 272, 384, "fp16"), (70, 100, 100, "e4m3")]
+    srcs = [U.to_device(synth.normal(21, i, (r, c)), src_fmt) for i, (r, c, _, _) in enumerate(shapes)]
+    outs = [[U.empty(r, c, f, ld) for r, c, ld, f in shapes] for _ in range(2)]
+    L.us_cast_multi_pitched(srcs, [1.0, 0.5, 1.0, 1.0, 1.0, 2.0], outs[0])
+    for s, o, k, (r, c, ld, f) in zip(srcs, outs[1], [1.0, 0.5, 1.0, 1.0, 1.0, 2.0], shapes):
+        L.us_cast_fp8(s, k, o) if f[0] == "e" else L.us_residual_add(s, s, 0.0, o)
+    for a, b, (r, c, ld, f) in zip(*outs, shapes):
+        assert np.array_equal(U.codes_of(a), U.codes_of(b))
+        assert not a.as_strided((r, ld), (ld, 1))[:, c:].contiguous().view(torch.uint8).any()
+
+    def status(s, d):
+        with pytest.raises(L.UnitScaleError) as e:
+            L.us_cast_multi_pitched([s], [1.0], [d])
+        return e.value.status
+
+    padded = U.to_device(synth.normal(21, 9, (8, 32)), src_fmt, 48)
+    assert status(padded, U.empty(8, 32, "e4m3", 48)) == L.US_ERR_UNSUPPORTED                # padded sources
+    assert status(srcs[5], U.empty(70, 100, "e4m3", 112)) == L.US_ERR_UNSUPPORTED            # rows that end inside a chunk
+    assert status(srcs[0], U.empty(5, 16, "e4m3", 24)) == L.US_ERR_ALIGNMENT                 # row starts
+    with pytest.raises(L.UnitScaleError):
+        L.us_cast_multi([srcs[0]], [1.0], [outs[0][0]])
