@@ -195,7 +195,8 @@ typedef struct {
 us_status us_linear_group(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, void* stream);
 /* The same launch without those limits, for a training step that issues its GEMMs this way at every size: 16-bit operands
  * (all calls of a launch the same operand width) and outputs of any size are covered too; US_ERR_UNSUPPORTED remains for a
- * fused activation, mixed widths and more tiles than the work list holds (2048). */
+ * fused activation, mixed widths and more tiles than the work list holds (2048).  Calls of few tiles with far longer contractions
+ * than the others (the weight gradients of many tokens) share them among several SMs as in us_linear_fwd, in a second launch. */
 us_status us_linear_group_any(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, void* stream);
 /* us_linear_group_any with FP8 copies as in us_linear_fwd_cast: copies[i] (ptr NULL: none) of the output of call i, which has a skip
  * tensor. */

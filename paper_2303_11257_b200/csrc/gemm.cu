@@ -91,7 +91,7 @@ static us_status linear(Op op, const us_mat* A, const us_mat* B, float scale, co
   if (reinterpret_cast<uintptr_t>(ws) % 16) return US_ERR_ALIGNMENT;
   p.status = static_cast<unsigned int*>(ws);
 
-  EpiMats em{out, p.aux && !copy ? &ep->aux : nullptr, p.skip ? &ep->skip : nullptr};
+  EpiMats em{out, p.aux && !copy ? &ep->aux : nullptr, p.skip ? &ep->skip : nullptr, copy};
   // The specialised epilogues cover the combinations of the FFN path; anything else (an activation
   // together with a skip tensor) takes the general direct-access epilogue.
   int epi = kEpiLegacy;

@@ -107,6 +107,72 @@ bool deal(GroupParams& g, int es, int tile_m, int bn, int split, int units, int 
   return true;
 }
 
+// 256 x 256 tiles per CTA pair unless they would leave a quarter of the pairs idle (measured over FFN steps, FP8 / BF16,
+// us: 48 such tiles 14.3 / 19.2 against 10.7 / 17.1 with 128 x 128 tiles, 64 tiles 14.9 / 20.0 against 16.3 / 27.3).
+bool pair_tiles_pay(int64_t pair_tiles, int sms) { return 8 * pair_tiles >= 3 * sms; }
+
+// Estimated time, us, of the grouped launch of the calls in `which` (a bit each): the busiest unit's K blocks, an epilogue counted as eight.
+double group_time(const Shape* sh, int count, unsigned which, int es, int sms) {
+  int64_t pair_tiles = 0, blocks = 0, longest = 0;
+  for (int i = 0; i < count; ++i)
+    if (which >> i & 1) pair_tiles += ((sh[i].M + 255) / 256) * ((sh[i].N + 255) / 256);
+  if (pair_tiles == 0) return 0.0;
+  const bool pair = pair_tiles_pay(pair_tiles, sms);
+  const int tile = pair ? 256 : 128, kbk = 128 / es;
+  for (int i = 0; i < count; ++i) {
+    if (!(which >> i & 1)) continue;
+    const int64_t kb = (sh[i].K + kbk - 1) / kbk + 8;
+    blocks += ((sh[i].M + tile - 1) / tile) * ((sh[i].N + tile - 1) / tile) * kb;
+    longest = std::max(longest, kb);
+  }
+  const int units = pair ? sms / 2 : sms;
+  return 3.0 + std::max((double)longest, (double)blocks / units) * (pair ? 0.3 : 0.16);
+}
+
+// The calls (a bit each) whose contractions several CTAs share in a launch of their own, in tiles t; 0: none.  A few tiles with a far
+// longer contraction than the rest of the work per unit (the weight gradients of many tokens and a narrow block) leave the other
+// units of the grouped launch idle; a second launch costs what its estimate says and has to save 2 us beyond it.  Captured FFN steps,
+// one grouped launch -> two, us: FP8 8192 x 128 x 512 39.9 -> 31.6, 8192 x 256 x 768 44.6 -> 38.8, 16000 x 128 x 400 65.5 -> 44.3; BF16 4096 x 128
+// x 256 25.5 -> 18.5, 9000 x 256 x 768 74.6 -> 54.2; F16 16384 x 256 x 1024 141.9 -> 101.8; nothing of 14 such shapes slower.
+unsigned shared_calls(const us_linear_call* calls, const Shape* sh, int count, int es, int sms, Tiling* t) {
+  const int kbk = 128 / es;
+  int64_t longest = 0;
+  for (int i = 0; i < count; ++i) longest = std::max(longest, sh[i].K);
+  if (longest < 48ll * kbk) return 0;
+  const unsigned all = (1u << count) - 1;
+  double best = group_time(sh, count, all, es, sms) - 2.0;
+  unsigned pick = 0;
+  for (int k = 0; k < count; ++k) {                       // every call of at least sh[k].K
+    const int64_t K = sh[k].K;
+    if (K < 48ll * kbk || K > 8192ll * kbk) continue;
+    unsigned which = 0;
+    bool sectors = true;
+    int64_t most = 0;
+    for (int i = 0; i < count; ++i) {
+      if (sh[i].K < K) continue;
+      which |= 1u << i;
+      most = std::max(most, sh[i].K);
+      sectors = sectors && calls[i].a.ld * es % 32 == 0 && calls[i].b.ld * es % 32 == 0;
+    }
+    const double rest = group_time(sh, count, all & ~which, es, sms);
+    for (int form = 0; form < 3; ++form)
+      for (int s = 2; s * (form == 2 ? 2 : 1) <= 8; s *= 2) {
+        const Tiling c{form == 0 ? 64 : form == 1 ? 128 : 256, form == 2 ? 2 : 1, s};
+        int64_t tiles = 0;
+        int a_bytes = 0;
+        for (int i = 0; i < count; ++i)
+          if (which >> i & 1) {
+            tiles += ((sh[i].M + 128 * c.cg - 1) / (128 * c.cg)) * ((sh[i].N + c.bn - 1) / c.bn);
+            a_bytes = std::max(a_bytes, split_a_bytes(c.bn, calls[i].op == US_OP_BWD_W, sh[i].M));
+          }
+        if (tiles * c.cg * s > sms) continue;
+        const double time = rest + tiling_time(c, tiles, (int)((most + kbk - 1) / kbk), a_bytes, sectors, sms);
+        if (time < best && tiles <= split_capacity(es, c)) { best = time; pick = which; *t = c; }
+      }
+  }
+  return pick;
+}
+
 template <int ES, int BN, int CG, int SPLIT, bool COPY>
 us_status launch_variant(const GroupParams& g, cudaStream_t stream) {
   auto kern = gemm_group_kernel<ES, BN, CG, SPLIT, COPY>;
@@ -126,8 +192,6 @@ us_status group_impl(int count, const us_linear_call* calls, const us_mat* copie
   if (reinterpret_cast<uintptr_t>(ws) % 16) return US_ERR_ALIGNMENT;
   static_assert(sizeof(GroupParams) < 32000, "kernel parameter limit");
   Shape sh[kGroupMaxProblems];
-  int64_t pair_tiles = 0;
-  bool copy = false;
   for (int i = 0; i < count; ++i) {
     us_status s = check_call(&calls[i], any, &sh[i]);
     if (s != US_OK) return s;
@@ -135,26 +199,44 @@ us_status group_impl(int count, const us_linear_call* calls, const us_mat* copie
     if (copies && copies[i].ptr) {
       s = check_copy(&copies[i], &calls[i].out, calls[i].ep.skip.ptr != nullptr);
       if (s != US_OK) return s;
-      copy = true;
     }
-    pair_tiles += ((sh[i].M + 255) / 256) * ((sh[i].N + 255) / 256);
   }
   const int sms = host::sm_count();
   if (sms <= 0) return US_ERR_CUDA;
   const int es = dtype_size(calls[0].a.dtype);
-  // 256 x 256 tiles per CTA pair unless they would leave a quarter of the pairs idle (measured over FFN steps, FP8 / BF16,
-  // us: 48 such tiles 14.3 / 19.2 against 10.7 / 17.1 with 128 x 128 tiles, 64 tiles 14.9 / 20.0 against 16.3 / 27.3).
-  const bool pair = 8 * pair_tiles >= 3 * sms;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  Tiling t{};
+  const unsigned shared = any ? shared_calls(calls, sh, count, es, sms, &t) : 0;
+  SplitCall split_calls[kGroupMaxProblems];
+  int splits = 0, left = 0, at[kGroupMaxProblems];
+  int64_t pair_tiles = 0;
+  bool copy = false;
+  for (int i = 0; i < count; ++i) {
+    const us_linear_call& c = calls[i];
+    const us_mat* q = copies && copies[i].ptr ? &copies[i] : nullptr;
+    if (shared >> i & 1) {
+      const bool skip = c.ep.skip.ptr != nullptr;
+      split_calls[splits++] = SplitCall{&c.a, &c.b, &c.out, skip ? &c.ep.skip : nullptr, q, c.op == US_OP_BWD_W, c.op != US_OP_BWD_X, c.scale,
+                                        skip ? c.ep.skip_coef : 0.f, skip ? c.ep.out_coef : 1.f};
+      continue;
+    }
+    at[left++] = i;
+    copy = copy || q;
+    pair_tiles += ((sh[i].M + 255) / 256) * ((sh[i].N + 255) / 256);
+  }
+  if (left == 0) return launch_split(splits, split_calls, t, static_cast<unsigned int*>(ws), kWaitLimit, 0, st);
+  const bool pair = pair_tiles_pay(pair_tiles, sms);
   const int tile_m = pair ? 256 : 128, bn = pair ? 256 : 128;
   int64_t tiles = 0;
-  for (int i = 0; i < count; ++i) tiles += ((sh[i].M + tile_m - 1) / tile_m) * ((sh[i].N + bn - 1) / bn);
+  for (int j = 0; j < left; ++j) tiles += ((sh[at[j]].M + tile_m - 1) / tile_m) * ((sh[at[j]].N + bn - 1) / bn);
   const int most = std::min(pair ? sms / 2 : sms, kGroupMaxUnits);
   const int split = !pair && 2 * tiles <= most ? 2 : 1;
   const int units = (int)std::min<int64_t>(most, tiles * split);
   GroupParams g;
-  g.count = count;
-  for (int i = 0; i < count; ++i) {
-    GroupProblem& P = g.prob[i];
+  g.count = left;
+  for (int j = 0; j < left; ++j) {
+    const int i = at[j];
+    GroupProblem& P = g.prob[j];
     const us_linear_call& c = calls[i];
     P.M = (int)sh[i].M; P.N = (int)sh[i].N; P.K = (int)sh[i].K;
     P.a_mn = c.op == US_OP_BWD_W; P.b_mn = c.op != US_OP_BWD_X;
@@ -179,7 +261,10 @@ us_status group_impl(int count, const us_linear_call* calls, const us_mat* copie
   if (!deal(g, es, tile_m, bn, split, units, any ? kGroupMaxItems : 12)) return US_ERR_UNSUPPORTED;      // too many tiles per unit for the work list
   g.status = static_cast<unsigned int*>(ws);
   g.wait_limit = kWaitLimit;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (splits) {                                            // (a grouped launch that is refused has launched nothing)
+    const us_status s = launch_split(splits, split_calls, t, static_cast<unsigned int*>(ws), kWaitLimit, 0, st);
+    if (s != US_OK) return s;
+  }
   if (es == 1) return pair ? launch_group<1, 256, 2, 1>(g, copy, st) : split == 2 ? launch_group<1, 128, 1, 2>(g, copy, st) : launch_group<1, 128, 1, 1>(g, copy, st);
   return pair ? launch_group<2, 256, 2, 1>(g, copy, st) : split == 2 ? launch_group<2, 128, 1, 2>(g, copy, st) : launch_group<2, 128, 1, 1>(g, copy, st);
 }

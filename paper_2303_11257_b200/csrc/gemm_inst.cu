@@ -7,7 +7,6 @@
 
 #include "gemm_kernel.cuh"
 #include "gemm_launch.h"
-#include "gemm_split.cuh"
 #include "host.h"
 
 #ifndef US_INST_ES
@@ -101,36 +100,10 @@ static us_status pick_epilogue(const us_mat* A, const us_mat* B, const GemmParam
   }
 }
 
-// A launch with p.splits CTAs (or pairs) per tile.
-template <int ES, bool A_MN, bool B_MN, int BN, int CG>
-static us_status launch_split(const us_mat* A, const us_mat* B, const GemmParams& p, const EpiMats& em, cudaStream_t stream) {
-  constexpr int kBK = kStageKBytes / ES;
-  CUtensorMap ta, tb, t_out, t_skip;
-  if (!make_tmap(&ta, A, ES, A_MN ? kBK : BN == 64 ? (int)p.a_bytes / kStageKBytes : kBM)) return US_ERR_CUDA;
-  if (!make_tmap(&tb, B, ES, B_MN ? kBK : BN / CG, B_MN && BN / CG * ES < 128 ? 64 : 128)) return US_ERR_CUDA;
-  const int out_es = dtype_size(em.out->dtype);
-  if (!make_tmap(&t_out, em.out, out_es, 32, 32 * out_es)) return US_ERR_CUDA;
-  t_skip = t_out;
-  if (em.skip && !make_tmap(&t_skip, em.skip, dtype_size(em.skip->dtype), 32)) return US_ERR_CUDA;
-  static std::atomic<uint64_t> smem_set{0};
-  return host::launch(gemm_split_kernel<ES, A_MN, B_MN, BN, CG>, &smem_set, CG * p.splits * p.tiles_m * p.tiles_n, gemm_threads(8), GemmSmem<BN, CG, 8>::kTotal,
-                      CG * p.splits, stream, ta, tb, t_out, t_skip, p);
-}
-// Clusters of `splits` CTAs (pairs) that run at once.
-template <int ES, bool A_MN, bool B_MN, int BN, int CG>
-static int split_capacity(int splits) {
-  static host::ClusterCount count;
-  return host::resident_clusters(reinterpret_cast<const void*>(gemm_split_kernel<ES, A_MN, B_MN, BN, CG>), gemm_threads(8), GemmSmem<BN, CG, 8>::kTotal, CG * splits, count);
-}
-
-struct Tiling { int bn, cg, splits; };
-
 // Whether the contraction is shared by several CTAs, and in which tiles.  now: the tiles taken otherwise; sectors: the operands' rows
 // start on 32-byte boundaries (a box of other rows takes TMA about twice as long).
 //
-// A launch is estimated as a base and a time per K block, which is bound by the tensor core (128 x 128 and narrower tiles 0.152 us, pairs
-// 0.28) or by what the L2 cache hands to all CTAs together (15 bytes per ps).  The bases hold the exchange: partial sums cross between SMs at
-// some 25 bytes per ns.  Measured, us, FP8 into BF16, one CTA a tile / two / four / eight CTAs on tiles of 128 x 64 / the same on 128 x 128 /
+// Both ways are estimated by tiling_time.  Measured, us, FP8 into BF16, one CTA a tile / two / four / eight CTAs on tiles of 128 x 64 / the same on 128 x 128 /
 // two and four pairs on 256 x 256 (-: more CTAs than SMs, or more clusters than run at once), rows x K x columns:
 //     48 x 1920 x 1024    4.7 / 4.8 4.7 - / 6.0 6.2 7.1 / -           48 x 2560 x 1024   5.4 / 5.2 4.8 - / 6.4 6.2 7.4 / -
 //     48 x 4096 x 1024    7.3 / 6.0 5.2 - / 7.2 6.7 7.2 / -           48 x 8192 x 1024  12.2 / 8.2 6.4 - / 9.7 7.9 7.9 / -
@@ -144,14 +117,7 @@ static Tiling split_tiling(const GemmParams& p, Tiling now, bool sectors) {
   const int kb = (p.K + kStageKBytes / ES - 1) / (kStageKBytes / ES), sms = host::sm_count();
   if (kb < (A_MN ? 48 : 20) || kb > 8192 || sms <= 0) return now;
   const auto tiles = [&](const Tiling& t) { return (long long)((p.M + kBM * t.cg - 1) / (kBM * t.cg)) * ((p.N + t.bn - 1) / t.bn); };
-  const auto cost = [&](const Tiling& t) {
-    const double bytes = (t.bn == 64 ? (double)p.a_bytes : 16384.0) + t.bn / t.cg * 128;
-    const long long ctas = std::min<long long>(tiles(t) * t.cg * t.splits, sms), waves = (tiles(t) * t.cg * t.splits + sms - 1) / sms;
-    const double block = std::max(t.cg == 2 ? 0.28 : 0.152, std::max(ctas * bytes / 15e6, sectors ? 0.0 : bytes / 86e3));
-    const int s = t.splits;
-    const double base = s == 1 ? 2.4 : t.cg == 2 ? (s == 2 ? 7.0 : 8.2) : t.bn == 128 ? (s == 2 ? 4.8 : s == 4 ? 5.4 : 6.6) : s == 2 ? 3.4 : s == 4 ? 4.0 : 4.4;
-    return base + (ctas > 100 ? 0.8 : 0.0) + waves * ((kb + s - 1) / s) * block;
-  };
+  const auto cost = [&](const Tiling& t) { return tiling_time(t, tiles(t), kb, split_a_bytes(t.bn, A_MN, p.M), sectors, sms); };
   Tiling pick = now;
   double best = 0.92 * cost(now);
   for (int form = 0; form < 3; ++form) {
@@ -159,8 +125,7 @@ static Tiling split_tiling(const GemmParams& p, Tiling now, bool sectors) {
     if (t.cg == 2 && (p.M <= kBM || p.N <= 128)) continue;
     for (; t.splits * t.cg <= 8; t.splits *= 2) {
       if (kb < 4 * t.splits || tiles(t) * t.splits * t.cg > sms || cost(t) >= best) continue;
-      const int fit = form == 0 ? split_capacity<ES, A_MN, B_MN, 64, 1>(t.splits) : form == 1 ? split_capacity<ES, A_MN, B_MN, 128, 1>(t.splits) : split_capacity<ES, A_MN, B_MN, 256, 2>(t.splits);
-      if (tiles(t) > fit) continue;
+      if (tiles(t) > split_capacity(ES, t)) continue;
       best = cost(t);
       pick = t;
     }
@@ -201,7 +166,10 @@ us_status launch_gemm(const us_mat* A, const us_mat* B, GemmParams& p, const Epi
     t = split_tiling<ES, A_MN, B_MN>(p, t, sectors);
   }
   const int bn = t.bn, cg = t.cg;
-  p.splits = t.splits;
+  if (t.splits > 1) {
+    const SplitCall call{A, B, em.out, em.skip, em.copy, A_MN, B_MN, p.scale, p.skip_coef, p.out_coef};
+    return launch_split(1, &call, t, p.status, p.wait_limit, p.no_loads, stream);
+  }
   p.tiles_m = (p.M + kBM * cg - 1) / (kBM * cg);
   p.tiles_n = (p.N + bn - 1) / bn;
   p.nb0 = (int)bd.nb0; p.nb1 = (int)bd.nb1;
@@ -220,9 +188,6 @@ us_status launch_gemm(const us_mat* A, const us_mat* B, GemmParams& p, const Epi
   p.d_rows_last = make_fast_div(p.tiles_m % p.band_m ? p.tiles_m % p.band_m : 1);
   p.d_nb1 = make_fast_div(p.nb1);
   p.idesc = (p.idesc & ~((0x3fu << 17) | (0x1fu << 24))) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)((kBM * cg) >> 4) << 24);
-  if (t.splits > 1)
-    return bn == 256 ? launch_split<ES, A_MN, B_MN, 256, 2>(A, B, p, em, stream)
-         : bn == 128 ? launch_split<ES, A_MN, B_MN, 128, 1>(A, B, p, em, stream) : launch_split<ES, A_MN, B_MN, 64, 1>(A, B, p, em, stream);
   return pair ? pick_epilogue<ES, A_MN, B_MN, 256, 2>(A, B, p, em, epi, bd, stream)
        : narrow ? pick_epilogue<ES, A_MN, B_MN, 64, 1>(A, B, p, em, epi, bd, stream)
                 : pick_epilogue<ES, A_MN, B_MN, 128, 1>(A, B, p, em, epi, bd, stream);

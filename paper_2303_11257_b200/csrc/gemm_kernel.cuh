@@ -24,6 +24,8 @@
 // drained (bounded again), TMEM is freed and the kernel returns.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "sm100.cuh"
 
@@ -47,7 +49,6 @@ struct GemmParams {
   unsigned int* status;
   uint32_t wait_limit;                      // polls a bounded wait makes before it gives up (kWaitLimit unless a test shortens it)
   int no_loads;                             // test hook: the producer issues no operand loads, so that the waits run out
-  int splits;                               // CTAs (or pairs) that share a tile's contraction (gemm_split.cuh; 1: none)
   uint32_t a_bytes, stages;                 // narrow tiles (BN = 64): bytes of A in a stage, and the stages that fit
 };
 
@@ -115,6 +116,14 @@ __device__ __forceinline__ void tile_batch(const GemmParams& p, int tile, int& b
   const int b = p.d_problem.div(tile);
   b0 = p.d_nb1.div(b);
   b1 = b - b0 * p.nb1;
+}
+
+// Calls f with an operand layout of the linear ops as compile-time constants (A, B stored MN-major): forward, input gradient, weight gradient.
+template <class F>
+__device__ __forceinline__ void with_layout(bool a_mn, bool b_mn, F f) {
+  if (a_mn) f(std::true_type(), std::true_type());
+  else if (b_mn) f(std::false_type(), std::true_type());
+  else f(std::false_type(), std::false_type());
 }
 
 // Bounded mbarrier wait.  Returns false if the CTA is aborting (this wait or another one timed out).

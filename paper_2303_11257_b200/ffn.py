@@ -186,7 +186,8 @@ class UnitScaledFFN:
 
     @property
     def launches_per_step(self) -> int:
-        """Kernel launches of step(): the cast(s) plus gemm_launches."""
+        """Kernel launches of step(): the cast(s) plus gemm_launches (one more where the grouped launch shares the weight
+        gradients' contractions: many tokens, a narrow block)."""
         if self.fused_casts:
             return 1 + self.gemm_launches
         return 10

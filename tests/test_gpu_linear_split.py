@@ -68,3 +68,36 @@ def test_waits_that_run_out_in_a_cluster():
         L.us_linear_fwd(X, W, scale, out, ws)
         assert L.us_workspace_status(ws) == 0
         U.assert_close_stored(out, val, "bf16", TOL * max(1.0, np.abs(val).max() / 4), "after")
+
+
+@pytest.mark.parametrize("fmt", ["e4m3", "bf16"])
+@pytest.mark.parametrize("b,m,n", [(16000, 128, 400), (8200, 272, 144), (6500, 64, 80)])
+def test_grouped_launch_whose_long_contractions_are_shared(fmt, b, m, n):
+    """The weight gradients of many tokens beside the other two products of a step, with a residual and its copy in FP8: against the single
+    entry points, whose sums are float32 sums in another order (2e-6 of the largest result, one step of the stored format)."""
+    from paper_2303_11257_b200 import lib as L, synth
+    ws = L.new_workspace()
+    dev = lambda i, shape: U.to_device(synth.normal(90 + i, 0, shape), fmt, PAD(shape[1]))
+    X, W, G, skip = dev(0, (b, m)), dev(1, (m, n)), dev(2, (b, n)), U.to_device(synth.normal(93, 0, (b, m)), "f32")
+    ep = lambda: L.epilogue(skip=skip, skip_coef=0.8, out_coef=0.6)
+    s = b ** -0.5
+    outs = [[U.empty(m, n, "f32"), U.empty(b, n, "bf16", PAD(n)), U.empty(b, m, "bf16"), U.empty(m, n, "fp16", PAD(n))] for _ in range(3)]
+    q = U.empty(b, m, "e5m2")
+    for o in outs[:2]:
+        plan = L.Plan((), ())
+        plan.group([(L.US_OP_BWD_W, X, G, s, o[0], None, None), (L.US_OP_FWD, X, W, 0.1, o[1], None, None),
+                    (L.US_OP_BWD_X, G, W, 0.1, o[2], skip, (0.8, 0.6)), (L.US_OP_BWD_W, X, G, s, o[3], None, None)], ws, {2: q})(L.current_stream())
+    o = outs[2]
+    L.us_linear_bwd_w(X, G, s, o[0], ws)
+    L.us_linear_fwd(X, W, 0.1, o[1], ws)
+    L.us_linear_bwd_x(G, W, 0.1, o[2], ws, ep())
+    L.us_linear_bwd_w(X, G, s, o[3], ws)
+    assert L.us_workspace_status(ws) == 0
+    for a, r in zip(outs[0], outs[1]):
+        assert torch.equal(a.contiguous().view(torch.uint8), r.contiguous().view(torch.uint8))
+    ref = U.host_values(o[0])
+    assert np.abs(U.host_values(outs[0][0]) - ref).max() <= 2e-6 * np.abs(ref).max()
+    U.assert_close_stored(outs[0][3], ref, "fp16", 2e-6 * np.abs(ref).max(), "fp16 weight gradient")
+    for i in (1, 2):
+        assert torch.equal(outs[0][i].contiguous().view(torch.uint8), o[i].contiguous().view(torch.uint8))
+    assert torch.equal(q.view(torch.uint8), outs[0][2].float().clamp(-57344, 57344).to(torch.float8_e5m2).view(torch.uint8))
