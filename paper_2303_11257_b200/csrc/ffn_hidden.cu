@@ -23,6 +23,8 @@
 // (and the grouped launch over two) the whole three-launch step 16.4 -> 12.3.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include <type_traits>
 
 #include "gemm_kernel.cuh"
@@ -35,15 +37,18 @@ constexpr int kHidEW = 16;
 // Shared-memory plan: 32 KB operand stages (this CTA's 128 rows of A and 128 rows of B, 128 bytes of K each) and one
 // output box of 32 rows per epilogue warp, BN / 4 columns of OES bytes.  The kept pre-activation lives in registers,
 // which leaves room for six stages (five with 16-bit outputs and 256-column tiles).
-template <int BN, int OES>
+// NB: columns of the products a CTA computes, 64 where several share a tile; then 24 KB stages, or smaller ones with fewer
+// rows of A than 128, in as many as fit.
+template <int BN, int OES, int NB>
 struct HidSmem {
   static constexpr int kABytes = kBM * kStageKBytes;
-  static constexpr int kBBytes = 128 * kStageKBytes;
+  static constexpr int kBBytes = (NB == 64 ? 64 : 128) * kStageKBytes;
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr int kRowBytes = BN / 4 * OES;                     // of an output box: 32, 64 or 128
   static constexpr int kEpiWarpBytes = 32 * kRowBytes;
   static constexpr int kEpiBytes = kHidEW * kEpiWarpBytes;
   static constexpr int kStages = (229376 - kEpiBytes) / kStageBytes;
+  static constexpr int kMaxStages = NB == 64 ? 16 : kStages;
   static constexpr int kBarrierBytes = 512;
   static constexpr int kTotal = kStages * kStageBytes + kEpiBytes + kBarrierBytes + 1024;   // + alignment slack
 };
@@ -60,14 +65,16 @@ struct HiddenParams {
   uint8_t *a_ptr, *d_ptr; long long a_ld, d_ld;   // A and dH, for SPLIT > 1 (otherwise reached by TMA)
   unsigned int* status;
   uint32_t wait_limit;
+  uint32_t x_bytes; int stages;     // SPLIT > 1: bytes of X or G in a stage (the rows that exist), and the stages that fit
   int no_loads;                     // test hook: no operand loads are issued, so that the waits run out
 };
 
 // ES: operand bytes per element (1 = FP8, 2 = BF16 / F16).  BN, CG: tiles of 256 x 256 per CTA pair (256, 2), or of
 // 128 x 128 per CTA (128, 1) where the large ones would leave more than half of the pairs idle (hidden_impl).
-// SPLIT (128 x 128 tiles): CTAs that compute the same tile, each turning 128 / SPLIT of its columns into outputs.  In a
-// small problem the arithmetic of the epilogue (3700 + 2800 cycles of one SM's issue slots for a tile) is the longest part of
-// the launch while most SMs are idle; repeating the short main loop costs less than it.
+// SPLIT (128 x 128 tiles): CTAs that share a tile, each computing 64 of its columns (of four, two the same ones) and turning 128 / SPLIT
+// into outputs.  In a small problem the arithmetic of the epilogue (3700 + 2800 cycles of one SM's issue slots for a tile) is the
+// longest part of the launch while most SMs are idle.  With all 128 columns computed by each, the operands they fetched were twice
+// the bytes: captured steps, us, 48 x 1024 x 4096 30.7 -> 28.7, 16 x 1024 x 4096 32.4 -> 29.1, 512 x 512 x 1456 15.0 -> 14.8.
 // OUT_A, OUT_D: output formats of A and dH (us_dtype).  H_BF16: pre-activation rounded to BF16 (else F16).
 template <int ES, int BN, int CG, int SPLIT, int OUT_A, int OUT_D, bool H_BF16>
 __global__ void __launch_bounds__(gemm_threads(kHidEW), 1)
@@ -76,7 +83,8 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                   const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_dh,
                   const HiddenParams p) {
   constexpr int kOes = OUT_A == US_E4M3 || OUT_A == US_E5M2 ? 1 : 2;
-  using S = HidSmem<BN, kOes>;
+  constexpr int kNB = SPLIT > 1 ? 64 : BN;          // columns of an accumulator
+  using S = HidSmem<BN, kOes, kNB>;
   static_assert(BN / CG == 128, "128 rows of B per CTA");
   constexpr int kBK = 128 / ES;                     // K elements per stage
   constexpr int kTileM = kBM * CG;
@@ -85,7 +93,10 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   constexpr int kSliceCols = SPLIT > 1 ? 16 : 32, kSlices = kWarpCols / kSliceCols;   // worked in slices
   constexpr int kWarpsUsed = SPLIT > 1 ? 4 * (BN / SPLIT / kWarpCols) : kHidEW;
   constexpr uint32_t kChunkBytes = kBK * 128;       // a box of an MN-major operand tile: kBK rows of K x 128 bytes
-  constexpr uint32_t kTmemCols = 2 * BN;
+  constexpr uint32_t kTmemCols = 2 * kNB;
+  constexpr bool kHalfRowB = SPLIT > 1 && ES == 1;  // W1 in rows of 64 bytes
+  const uint32_t x_bytes = SPLIT > 1 ? p.x_bytes : (uint32_t)S::kABytes, stage_bytes = x_bytes + S::kBBytes;
+  const int stages = SPLIT > 1 ? p.stages : S::kStages;
 
   ptx::grid_release_next();
   extern __shared__ uint8_t smem_raw[];
@@ -94,26 +105,27 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   const uint32_t epi_base = smem_base + S::kStages * S::kStageBytes;
   const uint32_t bars = epi_base + S::kEpiBytes;
   auto full_bar = [&](int s) { return bars + 8u * s; };
-  auto empty_bar = [&](int s) { return bars + 8u * (S::kStages + s); };
-  auto acc_full_bar = [&](int a) { return bars + 8u * (2 * S::kStages + a); };
-  auto acc_empty_bar = [&](int a) { return bars + 8u * (2 * S::kStages + 2 + a); };
-  const uint32_t drained_bar = bars + 8u * (2 * S::kStages + 4);
-  static_assert(8 * (2 * S::kStages + 5) + 8 <= S::kBarrierBytes, "barrier area too small");
-  uint8_t* tail = smem_gen + S::kStages * S::kStageBytes + S::kEpiBytes + 8 * (2 * S::kStages + 5);
+  auto empty_bar = [&](int s) { return bars + 8u * (S::kMaxStages + s); };
+  auto acc_full_bar = [&](int a) { return bars + 8u * (2 * S::kMaxStages + a); };
+  auto acc_empty_bar = [&](int a) { return bars + 8u * (2 * S::kMaxStages + 2 + a); };
+  const uint32_t drained_bar = bars + 8u * (2 * S::kMaxStages + 4);
+  static_assert(8 * (2 * S::kMaxStages + 5) + 8 <= S::kBarrierBytes, "barrier area too small");
+  uint8_t* tail = smem_gen + S::kStages * S::kStageBytes + S::kEpiBytes + 8 * (2 * S::kMaxStages + 5);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(tail);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 4);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = CG == 2 ? (int)ptx::cluster_ctarank() : 0;
   const int pair = blockIdx.x / (CG * SPLIT), num_pairs = gridDim.x / (CG * SPLIT);      // tile-walking unit: CTA pair or CTA(s)
-  const int split_col = SPLIT > 1 ? (int)(blockIdx.x % SPLIT) * (BN / SPLIT) : 0;        // this CTA's columns of the tile
+  const int split_col = SPLIT > 1 ? (int)(blockIdx.x % SPLIT) * (BN / SPLIT) : 0;        // this CTA's first output column of the tile
+  const int split_acc = SPLIT > 1 ? split_col % 64 : 0;                                  // and where it is in the accumulators
   const int num_tiles = p.tiles_m * p.tiles_n;
   const int kb1 = (p.K1 + kBK - 1) / kBK, kb2 = (p.K2 + kBK - 1) / kBK;
   // column-major over the tiles: pairs that run side by side share a panel of W1 and of W2
   auto tile_mn2 = [&](int tile, int& tm, int& tn) { tn = p.d_tiles_m.div(tile); tm = tile - tn * p.tiles_m; };
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < S::kStages; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
+    for (int s = 0; s < stages; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
     for (int a = 0; a < 2; ++a) { ptx::mbar_init(acc_full_bar(a), 1); ptx::mbar_init(acc_empty_bar(a), CG * kWarpsUsed); }
     ptx::mbar_init(drained_bar, 1);
     *abort_flag = 0;
@@ -142,38 +154,38 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       for (int tile = pair; ok && !p.no_loads && tile < num_tiles; tile += num_pairs) {
         int tm, tn;
         tile_mn2(tile, tm, tn);
-        const int m0 = tm * kTileM + rank * 128, n0 = tn * BN + rank * 128;
+        const int m0 = tm * kTileM + rank * 128, n0 = tn * BN + rank * 128 + (split_col - split_acc);
         for (int sub = 0; ok && sub < 2; ++sub) {
           const int num_kb = sub ? kb2 : kb1;
           for (int kb = 0; kb < num_kb; ++kb) {
             ok = wait_bounded(empty_bar(stage), phase ^ 1u, abort_flag, p.status, p.wait_limit);
             if (!ok) break;
-            const uint32_t a_dst = smem_base + stage * S::kStageBytes, b_dst = a_dst + S::kABytes;
+            const uint32_t a_dst = smem_base + stage * stage_bytes, b_dst = a_dst + x_bytes;
             const int k0 = kb * kBK;
             if (issued == 0) ptx::grid_wait_previous();       // coordinates and barriers are ready: only the loads wait
             const uint32_t fb = CG == 2 ? ptx::in_even_cta(full_bar(stage)) : full_bar(stage);
-            if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), CG * S::kStageBytes);
+            if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), CG * stage_bytes);
             auto load = [&](uint32_t dst, const void* tmap, int x, int y) {
               if (CG == 2) ptx::tma_load_2d_pair(dst, tmap, fb, x, y); else ptx::tma_load_2d(dst, tmap, fb, x, y);
             };
             if (sub == 0) {
               load(a_dst, &tm_x, k0, m0);                           // X  [M x K1], K-major
 #pragma unroll
-              for (int c = 0; c < ES; ++c) load(b_dst + c * kChunkBytes, &tm_w1, n0 + c * kBK, k0);   // W1 [K1 x N], N-major, 128 / ES columns per box
+              for (int c = 0; c < (SPLIT > 1 ? 1 : ES); ++c) load(b_dst + c * kChunkBytes, &tm_w1, n0 + c * kBK, k0);   // W1 [K1 x N], N-major, 128 / ES columns per box
             } else {
               load(a_dst, &tm_g, k0, m0);                           // G  [M x K2], K-major
               load(b_dst, &tm_w2, k0, n0);                          // W2 [N x K2], K-major
             }
             ++issued;
-            if (++stage == S::kStages) { stage = 0; phase ^= 1u; }
+            if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
         }
       }
       if (*abort_flag && rank == 0) {
         // Let copies that are still in flight land before the CTA gives up its shared memory.
-        const uint32_t n = issued < (uint32_t)S::kStages ? issued : (uint32_t)S::kStages;
+        const uint32_t n = issued < (uint32_t)stages ? issued : (uint32_t)stages;
         for (uint32_t i = 0; i < n; ++i) {
-          if (stage == 0) { stage = S::kStages; phase ^= 1u; }
+          if (stage == 0) { stage = stages; phase ^= 1u; }
           --stage;
           for (uint32_t it = 0; it < p.wait_limit && !ptx::mbar_try_wait(full_bar(stage), phase); ++it) {}
         }
@@ -185,23 +197,24 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       ptx::grid_wait_previous();                       // no operand comes earlier: the bounded waits begin when the loads do
       int stage = 0; uint32_t phase = 0, local = 0;
       bool ok = true;
-      constexpr uint32_t kStageStep = S::kStageBytes >> 4;
+      const uint32_t stage_step = stage_bytes >> 4;
       const uint64_t a_desc = ptx::smem_desc_sw128(smem_base, 16, 1024);                              // K-major
-      const uint64_t b_desc_mn = ptx::smem_desc_sw128(smem_base + S::kABytes, kChunkBytes, 1024);     // W1: N-major
-      const uint64_t b_desc_k = ptx::smem_desc_sw128(smem_base + S::kABytes, 16, 1024);               // W2: K-major
+      const uint64_t b_desc_mn = kHalfRowB ? ptx::smem_desc_sw64(smem_base + x_bytes, 16, 512)
+                                           : ptx::smem_desc_sw128(smem_base + x_bytes, kChunkBytes, 1024);    // W1: N-major
+      const uint64_t b_desc_k = ptx::smem_desc_sw128(smem_base + x_bytes, 16, 1024);                  // W2: K-major
       const uint32_t a_hi = (uint32_t)(a_desc >> 32), a_lo0 = (uint32_t)a_desc;
       for (int tile = pair; ok && tile < num_tiles; tile += num_pairs, ++local) {
         const uint32_t acc_phase = local & 1u;
         for (int sub = 0; ok && sub < 2; ++sub) {
           const uint64_t b_desc = sub ? b_desc_k : b_desc_mn;
           const uint32_t b_hi = (uint32_t)(b_desc >> 32), b_lo0 = (uint32_t)b_desc;
-          const uint32_t b_step = (sub ? 32u : kChunkBytes / kKSteps) >> 4;
+          const uint32_t b_step = (sub ? 32u : (kHalfRowB ? kChunkBytes / 2 : kChunkBytes) / kKSteps) >> 4;
           const uint32_t idesc = sub ? p.idesc2 : p.idesc1;
           const int num_kb = sub ? kb2 : kb1;
           ok = wait_bounded(acc_empty_bar(sub), acc_phase ^ 1u, abort_flag, p.status, p.wait_limit);
           if (!ok) break;
           ptx::tc_fence_after_sync();
-          const uint32_t d_tmem = tmem_base + sub * BN;
+          const uint32_t d_tmem = tmem_base + sub * kNB;
           uint32_t accumulate = 0;
           for (int kb = 0; kb < num_kb; ++kb) {
             if (!ptx::mbar_try_wait(full_bar(stage), phase)) {
@@ -209,7 +222,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
               if (!ok) break;
             }
             ptx::tc_fence_after_sync();
-            const uint32_t a_lo = a_lo0 + stage * kStageStep, b_lo = b_lo0 + stage * kStageStep;
+            const uint32_t a_lo = a_lo0 + stage * stage_step, b_lo = b_lo0 + stage * stage_step;
 #pragma unroll
             for (int k = 0; k < kKSteps; ++k) {
               const uint64_t adesc = ((uint64_t)a_hi << 32) | (a_lo + k * 2u);
@@ -219,7 +232,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
               accumulate = 1;
             }
             if (CG == 2) ptx::mma_commit_pair(empty_bar(stage), 3); else ptx::mma_commit(empty_bar(stage));
-            if (++stage == S::kStages) { stage = 0; phase ^= 1u; }
+            if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
           if (ok) { if (CG == 2) ptx::mma_commit_pair(acc_full_bar(sub), 3); else ptx::mma_commit(acc_full_bar(sub)); }
         }
@@ -334,7 +347,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         ptx::tc_fence_after_sync();
-        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + sub * BN + split_col + part * kWarpCols;
+        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + sub * kNB + split_acc + part * kWarpCols;
         uint32_t r0[kSliceCols], r1[kSliceCols];
         if (SPLIT > 1) {
           const long long at = sub == 0 ? (long long)(row0 + lane) * p.a_ld : (long long)(row0 + lane) * p.d_ld;
@@ -440,7 +453,7 @@ bool is_fp8(int dt) { return dt == US_E4M3 || dt == US_E5M2; }
 template <int ES, int BN, int CG, int SPLIT, int OUT_A, int OUT_D, bool H_BF16>
 us_status launch_hidden(const CUtensorMap* t, const HiddenParams& p, int units, cudaStream_t stream) {
   auto kern = ffn_hidden_kernel<ES, BN, CG, SPLIT, OUT_A, OUT_D, H_BF16>;
-  constexpr int smem = HidSmem<BN, OUT_A == US_E4M3 || OUT_A == US_E5M2 ? 1 : 2>::kTotal;
+  constexpr int smem = HidSmem<BN, OUT_A == US_E4M3 || OUT_A == US_E5M2 ? 1 : 2, (SPLIT > 1 ? 64 : BN)>::kTotal;
   static std::atomic<uint64_t> smem_set{0};
   return host::launch(kern, &smem_set, CG * SPLIT * units, gemm_threads(kHidEW), smem, CG, stream, t[0], t[1], t[2], t[3], t[4], t[5], p);
 }
@@ -491,8 +504,18 @@ us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_m
   p.tiles_m = (int)((M + tile - 1) / tile); p.tiles_n = (int)((N + tile - 1) / tile);
   if ((int64_t)p.tiles_m * p.tiles_n >= (1ll << 30)) return US_ERR_UNSUPPORTED;
   p.d_tiles_m = make_fast_div(p.tiles_m);
-  p.idesc1 = make_idesc(X->dtype == one, W1->dtype == one, false, true, tile, tile);
-  p.idesc2 = make_idesc(G->dtype == one, W2->dtype == one, false, false, tile, tile);
+  const int tiles = p.tiles_m * p.tiles_n, most = pair ? sms / 2 : sms;
+  const int units = tiles < most ? tiles : most;
+  const int split = pair ? 1 : 4 * tiles <= sms ? 4 : 2 * tiles <= sms ? 2 : 1;
+  const int cols = split > 1 ? 64 : tile;                        // of an accumulator
+  p.idesc1 = make_idesc(X->dtype == one, W1->dtype == one, false, true, tile, cols);
+  p.idesc2 = make_idesc(G->dtype == one, W2->dtype == one, false, false, tile, cols);
+  // a short X or G: its rows in groups of eight.  The MMA still reads 128; what lies behind them ends up in rows that do not exist.
+  const int x_rows = split > 1 && M < 128 ? (int)((M + 7) / 8 * 8) : 128;
+  p.x_bytes = (uint32_t)x_rows * kStageKBytes;
+  using Half1 = HidSmem<128, 1, 64>;
+  using Half2 = HidSmem<128, 2, 64>;
+  p.stages = (int)std::min((uint32_t)Half1::kMaxStages, (uint32_t)(f8 ? Half1::kStages * Half1::kStageBytes : Half2::kStages * Half2::kStageBytes) / (p.x_bytes + (uint32_t)Half1::kBBytes));
   p.scale1 = alpha; p.scale2 = beta_x;
   p.act_in = act_in_scale; p.act_out = act_out_scale; p.grad_out = grad_out_scale;
   p.h_ptr = keep_h ? static_cast<uint8_t*>(H->ptr) : nullptr;
@@ -506,13 +529,10 @@ us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_m
 
   CUtensorMap t[6];
   const int out_box = tile / 4 * es;                             // bytes per row of an epilogue warp's output box
-  if (!make_tmap(&t[0], X, es, 128, 128) || !make_tmap(&t[1], W1, es, 128 / es, 128) || !make_tmap(&t[2], G, es, 128, 128) ||
-      !make_tmap(&t[3], W2, es, 128, 128) || !make_tmap(&t[4], A, es, 32, out_box) || !make_tmap(&t[5], dH, es, 32, out_box))
+  if (!make_tmap(&t[0], X, es, x_rows, 128) || !make_tmap(&t[1], W1, es, 128 / es, split > 1 && es == 1 ? 64 : 128) ||
+      !make_tmap(&t[2], G, es, x_rows, 128) || !make_tmap(&t[3], W2, es, split > 1 ? 64 : 128, 128) || !make_tmap(&t[4], A, es, 32, out_box) || !make_tmap(&t[5], dH, es, 32, out_box))
     return US_ERR_CUDA;
 
-  const int tiles = p.tiles_m * p.tiles_n, most = pair ? sms / 2 : sms;
-  const int units = tiles < most ? tiles : most;
-  const int split = pair ? 1 : 4 * tiles <= sms ? 4 : 2 * tiles <= sms ? 2 : 1;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const bool bf = h_dtype == US_BF16;
   if (!f8) return X->dtype == US_BF16 ? pick_hidden<2, US_BF16, US_BF16>(pair, split, bf, t, p, units, st) : pick_hidden<2, US_F16, US_F16>(pair, split, bf, t, p, units, st);
