@@ -255,10 +255,10 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     const f32x2 s1 = splat2(p.scale1), s2 = splat2(p.scale2), in2 = splat2(p.act_in), os2 = splat2(p.grad_out * p.act_in);
     const float tail_k = fabsf(p.act_in) * (1.0f / kTailRange), act_oi = p.act_out * p.act_in;
 
-    auto release_acc = [&](int a) {
+    auto release_acc = [&](int a, int tile) {                   // (where no later tile takes it nobody waits)
       ptx::tc_fence_before_sync();
       __syncwarp();
-      if (lane == 0) {
+      if (lane == 0 && tile + num_pairs < num_tiles) {
         if (CG == 2) ptx::mbar_arrive_cluster(ptx::in_even_cta(acc_empty_bar(a)));
         else ptx::mbar_arrive(acc_empty_bar(a));
       }
@@ -367,7 +367,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             ptx::tmem_ld_fence(r1);
           }
         }
-        release_acc(sub);                                       // the values are in registers
+        release_acc(sub, tile);                                       // the values are in registers
         if (active) {
           if (kSlices == 2) { if (sub == 0) slice_fwd(r1, 1); else slice_bwd(r1, 1); }
           else { if (sub == 0) slice_fwd(r0, 0); else slice_bwd(r0, 0); }
@@ -419,7 +419,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (CG == 2) ptx::cluster_sync();
+  if (CG == 2) ptx::cluster_meet();
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     if (CG == 2) ptx::tmem_dealloc_pair(tmem_base, kTmemCols); else ptx::tmem_dealloc(tmem_base, kTmemCols);

@@ -242,9 +242,11 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
     };
     // The entry of a round, and the first box of the skip tensor that its tile has for this warp (map null: none).  A round is looked at
     // while the one before waits for its accumulator, the first one before the previous kernel is waited for.
+    int mine = g.rounds;                                       // entries of this unit
+    while (mine > 0 && entry(mine - 1) < 0) --mine;
     struct Next { int32_t e; const CUtensorMap* map; int col, row; };
     auto look = [&](int r) {
-      Next n{r < g.rounds ? entry(r) : -1, nullptr, 0, 0};
+      Next n{r < mine ? entry(r) : -1, nullptr, 0, 0};
       if (n.e < 0) return n;
       int pi, tm, tn;
       group_decode(n.e, pi, tm, tn);
@@ -284,7 +286,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
       auto release_acc = [&]() {
         ptx::tc_fence_before_sync();
         __syncwarp();
-        if (lane == 0) {
+        if (lane == 0 && r + 2 < mine) {                     // (where no later tile takes it nobody waits)
           if (CG == 2) ptx::mbar_arrive_cluster(ptx::in_even_cta(acc_empty_bar(acc)));
           else ptx::mbar_arrive(acc_empty_bar(acc));
         }
@@ -360,7 +362,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
 
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (CG == 2) ptx::cluster_sync();
+  if (CG == 2) ptx::cluster_meet();
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     if (CG == 2) ptx::tmem_dealloc_pair(tmem_base, kTmemCols); else ptx::tmem_dealloc(tmem_base, kTmemCols);

@@ -374,11 +374,12 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
     in_pending = true;
   };
   // This warp is done reading accumulator a: its values are in registers, so the buffer is handed
-  // back to the MMA warp before the arithmetic and the stores of the last slice, not after them.
-  auto release_acc = [&](uint32_t a) {
+  // back to the MMA warp before the arithmetic and the stores of the last slice, not after them.  (Where no later tile takes it
+  // nobody is told: what the odd CTA of a pair signals to the even one has then been waited for before that leaves.)
+  auto release_acc = [&](uint32_t a, int tile) {
     ptx::tc_fence_before_sync();
     __syncwarp();
-    if (lane == 0) {
+    if (lane == 0 && tile + 2 * c.num_groups < c.num_tiles) {
       if (CG == 2) ptx::mbar_arrive_cluster(ptx::in_even_cta(c.acc_empty0 + 8u * a));
       else ptx::mbar_arrive(c.acc_empty0 + 8u * a);
     }
@@ -446,7 +447,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
         }
         float v[32];
         ptx::tmem_ld_32x32(t_row + 32 * sl, v);
-        if (last_slice) { release_acc(acc); released = true; }   // the MMA warp may refill it while this slice is worked on
+        if (last_slice) { release_acc(acc, tile); released = true; }   // the MMA warp may refill it while this slice is worked on
         const f32x2 scale2 = splat2(p.scale), in2 = splat2(p.act_in);
         const float tail_k = fabsf(p.act_in) * (1.0f / kTailRange), act_oi = p.act_out * p.act_in;
         const f32x2 os2 = splat2(p.act_out * p.act_in), skip2 = splat2(p.skip_coef), oc2 = splat2(p.out_coef);
@@ -523,7 +524,7 @@ __device__ __forceinline__ void epilogue_staged(const GemmParams& p, const CUten
     }
     ok = __all_sync(0xffffffffu, ok);
     if (!ok) break;
-    if (!released) release_acc(acc);                           // tile without columns for this warp
+    if (!released) release_acc(acc, tile);                     // tile without columns for this warp
   }
   // Leaving early (a wait ran out somewhere in the CTA): an input box may still be in flight; let it
   // land before the CTA may give up its shared memory.
@@ -574,10 +575,11 @@ __device__ __forceinline__ void epilogue_act16(const GemmParams& p, const CUtens
     ptx::mbar_expect_tx(bar, 2048);
     ptx::tma_load_2d(buf_aux + 2048u * half, tm_aux, bar, n_w + 32 * half, row0);
   };
-  auto release_acc = [&](uint32_t a) {
+  int tile = c.group;
+  auto release_acc = [&](uint32_t a) {                        // (as in epilogue_staged)
     ptx::tc_fence_before_sync();
     __syncwarp();
-    if (lane == 0) {
+    if (lane == 0 && tile + 2 * c.num_groups < c.num_tiles) {
       if (CG == 2) ptx::mbar_arrive_cluster(ptx::in_even_cta(c.acc_empty0 + 8u * a));
       else ptx::mbar_arrive(c.acc_empty0 + 8u * a);
     }
@@ -624,7 +626,7 @@ __device__ __forceinline__ void epilogue_act16(const GemmParams& p, const CUtens
     }
   };
 
-  int tile = c.group, row0 = 0, n_w = 0;
+  int row0 = 0, n_w = 0;
   bool pending[2] = {false, false};                          // an input box load is in flight
   if (tile < c.num_tiles) {
     coords(tile, row0, n_w);
@@ -947,7 +949,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
       }
       ptx::tc_fence_before_sync();
       __syncwarp();
-      if (lane == 0) {                               // the issuing (even) CTA owns the accumulator-free barrier
+      if (lane == 0 && tile + 2 * num_groups < num_tiles) {      // the issuing (even) CTA owns the accumulator-free barrier
         if (CG == 2) ptx::mbar_arrive_cluster(ptx::in_even_cta(acc_empty_bar(acc)));
         else ptx::mbar_arrive(acc_empty_bar(acc));
       }
@@ -956,7 +958,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
 
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (CG == 2) ptx::cluster_sync();                  // no CTA leaves while its partner may still signal it
+  if (CG == 2) ptx::cluster_meet();                  // no CTA leaves while its partner may still signal it
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     if (CG == 2) ptx::tmem_dealloc_pair(tmem_base, kTmemCols); else ptx::tmem_dealloc(tmem_base, kTmemCols);

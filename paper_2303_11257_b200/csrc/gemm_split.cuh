@@ -297,7 +297,7 @@ gemm_split_kernel(const __grid_constant__ SplitParams<MULTI ? kGroupMaxProblems 
 
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (CG == 2) ptx::cluster_sync();
+  if (CG == 2) ptx::cluster_meet();
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     if (CG == 2) ptx::tmem_dealloc_pair(tmem_base, BN); else ptx::tmem_dealloc(tmem_base, BN);

@@ -194,6 +194,12 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// The same without ordering memory: nobody goes on before all have arrived.  (A release also waits for the thread's earlier stores to
+// reach memory, about 1 us at the end of a kernel.)
+__device__ __forceinline__ void cluster_meet() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
 // A shared-memory address of this CTA re-addressed to the same offset in the pair's even CTA.
 // (clusters here have exactly two CTAs, so the even CTA is rank 0)
 __device__ __forceinline__ uint32_t in_even_cta(uint32_t addr) {
