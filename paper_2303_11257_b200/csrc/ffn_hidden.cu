@@ -141,7 +141,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   }
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (CG == 2) ptx::cluster_sync();
+  if (CG == 2) ptx::cluster_meet();
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
 

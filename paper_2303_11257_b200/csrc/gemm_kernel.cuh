@@ -777,7 +777,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   }
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (CG == 2) ptx::cluster_sync();                  // the partner's barriers and TMEM are ready too
+  if (CG == 2) ptx::cluster_meet();                  // the partner's barriers and TMEM are ready too
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
 

@@ -90,7 +90,7 @@ gemm_split_kernel(const __grid_constant__ SplitParams<MULTI ? kGroupMaxProblems 
   }
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (CG == 2) ptx::cluster_sync();                  // the partner's barriers and TMEM are ready too
+  if (CG == 2) ptx::cluster_meet();                  // the partner's barriers and TMEM are ready too
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
 

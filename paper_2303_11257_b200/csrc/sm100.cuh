@@ -194,8 +194,8 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// The same without ordering memory: nobody goes on before all have arrived.  (A release also waits for the thread's earlier stores to
-// reach memory, about 1 us at the end of a kernel.)
+// The same without a release: nobody goes on before all have arrived.  (A release also waits for the thread's earlier stores to reach
+// memory, about 1 us at the end of a kernel.)  After mbar_init_fence it publishes the barriers that the fencing thread has initialised.
 __device__ __forceinline__ void cluster_meet() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
