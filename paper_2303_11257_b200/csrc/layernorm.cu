@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(kLnThreads, NCH <= 4 ? 3 : 2) ln_fwd16_kernel(
   }
 }
 
-// G32: the gradient is float32 (the gradient of a layer's output often is) instead of the 16-bit type of X.
+// Rows beyond what L2 holds, with a gradient of X's 16-bit type: one warp per row.
 //
 // The rows reach the SM through a ring of kLnStages slots per warp in shared memory, filled by bulk
 // copies (cp.async.bulk, completion counted on one mbarrier per slot): with one row per warp in
@@ -309,18 +309,18 @@ constexpr uint32_t kLnWaitLimit = 1u << 20;
 
 // XBF: X (and a 16-bit gradient) are BF16 rather than F16; fixed at compile time, because a run-time choice
 // in the unpacking costs more instructions than the arithmetic it feeds.
-template <int NCH, bool G32, bool XBF, bool COPY>
+template <int NCH, bool XBF, bool COPY>
 __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
   extern __shared__ __align__(16) float ln_smem[];             // w[cols] as float32, [warps][cols] for the combine, the ring, its mbarriers
   float* w_s = ln_smem;                                        // NCH * 256 floats
   float* comb = ln_smem + NCH * 256;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const uint32_t xb = (uint32_t)a.cols * 2u, gb = (uint32_t)a.cols * (G32 ? 4u : 2u), slot = xb + gb;
+  const uint32_t xb = (uint32_t)a.cols * 2u, gb = xb, slot = xb + gb;
   char* ring_gen = reinterpret_cast<char*>(comb + (size_t)nw * a.cols) + (size_t)warp * kLnStages * slot;
   const uint32_t ring = ptx::smem_addr(ring_gen);
   const uint32_t bars = ptx::smem_addr(reinterpret_cast<char*>(comb + (size_t)nw * a.cols) + (size_t)nw * kLnStages * slot) +
                         8u * (uint32_t)(warp * kLnStages);
-  if (!G32 && lane == 0) {                                     // (no ring, hence no mbarriers, with a float32 gradient)
+  if (lane == 0) {
     for (int st = 0; st < kLnStages; ++st) ptx::mbar_init(bars + 8u * st, 1);
     ptx::mbar_init_fence();
   }
@@ -344,21 +344,17 @@ __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
     const uint32_t bar = bars + 8u * st;
     ptx::mbar_expect_tx(bar, slot);
     ptx::bulk_load_1d(ring + st * slot, static_cast<const char*>(a.x) + r * a.x_ld * 2, xb, bar);
-    ptx::bulk_load_1d(ring + st * slot + xb, static_cast<const char*>(a.g) + r * a.g_ld * (G32 ? 4 : 2), gb, bar);
+    ptx::bulk_load_1d(ring + st * slot + xb, static_cast<const char*>(a.g) + r * a.g_ld * 2, gb, bar);
   };
   int issued = 0;                                              // rows asked for so far (warp-uniform)
-  if (!G32)
-    for (; issued < kLnStages && row + issued * stride < a.rows; ++issued)
-      if (lane == 0) issue(row + issued * stride, issued);
-  // direct: ordinary loads instead of the ring -- after a wait ran out, and always for a float32 gradient
-  // (rows of 6 bytes per element: the ring then costs a CTA per SM and measured slower than plain loads)
-  bool direct = G32;
+  for (; issued < kLnStages && row + issued * stride < a.rows; ++issued)
+    if (lane == 0) issue(row + issued * stride, issued);
+  bool direct = false;                                         // ordinary loads instead of the ring, after a wait ran out
   int it = 0, unconsumed = 0;                                  // unconsumed: first row whose copy was never waited for
-  uint4 cx[NCH], cg[G32 ? 1 : NCH], nx[G32 ? NCH : 1];
+  uint4 cx[NCH], cg[NCH];
   for (; row < a.rows; row += stride, ++it) {
     const int st = it % kLnStages;
     const uint32_t parity = (uint32_t)(it / kLnStages) & 1u;
-    float gf[G32 ? NCH : 1][8];
     if (!direct) {
       bool ok = false;
       for (uint32_t k = 0; k < kLnWaitLimit && !(ok = ptx::mbar_try_wait(bars + 8u * st, parity)); ++k) {}
@@ -372,16 +368,10 @@ __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
         const int col = (c * 32 + lane) * 8;
         if (col < a.cols) {
           cx[c] = *reinterpret_cast<const uint4*>(sx + col * 2);
-          if (G32) {
-            const float4 g0 = *reinterpret_cast<const float4*>(sx + xb + col * 4), g1 = *reinterpret_cast<const float4*>(sx + xb + col * 4 + 16);
-            gf[G32 ? c : 0][0] = g0.x; gf[G32 ? c : 0][1] = g0.y; gf[G32 ? c : 0][2] = g0.z; gf[G32 ? c : 0][3] = g0.w;
-            gf[G32 ? c : 0][4] = g1.x; gf[G32 ? c : 0][5] = g1.y; gf[G32 ? c : 0][6] = g1.z; gf[G32 ? c : 0][7] = g1.w;
-          } else {
-            cg[G32 ? 0 : c] = *reinterpret_cast<const uint4*>(sx + xb + col * 2);
-          }
+          cg[c] = *reinterpret_cast<const uint4*>(sx + xb + col * 2);
         } else {
           cx[c] = make_uint4(0, 0, 0, 0);
-          if (!G32) cg[G32 ? 0 : c] = make_uint4(0, 0, 0, 0);
+          cg[c] = make_uint4(0, 0, 0, 0);
         }
       }
       __syncwarp();                                            // every lane holds its part: the slot can be refilled
@@ -391,23 +381,8 @@ __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
         ++issued;
       }
     } else {
-      if constexpr (G32) {
-        // X of this row was fetched one iteration ahead (packed, in registers); the float32 gradient is read now
-        if (it == 0) load_row16<NCH>(a.x, row * a.x_ld, lane, a.cols, cx);
-        else {
-#pragma unroll
-          for (int c = 0; c < NCH; ++c) cx[c] = nx[c];
-        }
-        if (row + stride < a.rows) load_row16<NCH>(a.x, (row + stride) * a.x_ld, lane, a.cols, nx);
-#pragma unroll
-        for (int c = 0; c < NCH; ++c) {
-          const int col = (c * 32 + lane) * 8;
-          if (col < a.cols) load_vec<8>(static_cast<const char*>(a.g) + (row * a.g_ld + col) * 4, US_F32, gf[c]);
-        }
-      } else {
-        load_row16<NCH>(a.x, row * a.x_ld, lane, a.cols, cx);
-        load_row16<NCH>(a.g, row * a.g_ld, lane, a.cols, cg);
-      }
+      load_row16<NCH>(a.x, row * a.x_ld, lane, a.cols, cx);
+      load_row16<NCH>(a.g, row * a.g_ld, lane, a.cols, cg);
     }
     // From here on the row is worked on as pairs of float32 in 64-bit registers (add / mul / fma .f32x2):
     // the kernel is bound by instruction issue, and the packed forms halve the arithmetic instructions.
@@ -422,8 +397,7 @@ __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
       }
     }
     auto g_pair = [&](int c, int j) -> f32x2 {                 // gradient values 2 j, 2 j + 1 of chunk c
-      if (G32) return pack2(gf[G32 ? c : 0][2 * j], gf[G32 ? c : 0][2 * j + 1]);
-      const uint4& r = cg[G32 ? 0 : c];
+      const uint4& r = cg[c];
       const uint32_t w = j == 0 ? r.x : j == 1 ? r.y : j == 2 ? r.z : r.w;
       const float2 f = XBF ? unpack_bf16x2(w) : unpack_f16x2(w);
       return pack2(f.x, f.y);
@@ -525,6 +499,181 @@ __global__ void __launch_bounds__(128, 3) ln_bwd16_kernel(const LnArgs a) {
   }
 }
 
+// Sums over the warp of four values per lane; lane l gets that of v[l & 3].  (Six shuffles instead of twenty.)
+__device__ __forceinline__ float warp_sum4(const float (&v)[4], int lane) {
+  const bool b0 = lane & 1, b1 = lane & 2;
+  float x = (b0 ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, b0 ? v[0] : v[1], 1);
+  const float z = (b0 ? v[3] : v[2]) + __shfl_xor_sync(0xffffffffu, b0 ? v[2] : v[3], 1);
+  x = (b1 ? z : x) + __shfl_xor_sync(0xffffffffu, b1 ? x : z, 2);
+#pragma unroll
+  for (int o = 4; o <= 16; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// The 16-bit cases of the backward pass (rows of at most 2048 elements): a row belongs to wpr = cols / 256 warps, eight columns a lane, so
+// that a lane's share of the column sums is 16 registers and three CTAs of eight warps fit an SM; the warps of a row take four rows at
+// a time, which hides the latency of their loads and shares two exchanges through shared memory among four rows: the means, then the
+// sums of (x - mu)^2, g w and g w (x - mu).  G32: the gradient is float32 (the gradient of a layer's output often is) instead of the 16-bit
+// type of X.  XBF: X (and a 16-bit gradient) are BF16 rather than F16.  Bound: latency of the exchanges, 16 warps an SM; beyond L2
+// memory.  us, a warp per row -> this, BF16 with an FP8 copy: 8192 x 1024 22.8 -> 17.9, its float32 gradient 25.6 -> 18.9, 2048 x 768 12.0 -> 7.8, 4096 x
+// 256 8.7 -> 5.6, 256 x 1024 8.9 -> 5.8; 2048 x 2048, which the general kernel took, 65 -> 13.
+constexpr int kLnBatch = 4, kLnRowsPerSm = 2;
+enum LnOut { kLnSame = 0, kLnSameE4 = 1, kLnSameE5 = 2, kLnAny = 3, kLnAnyCopy = 4 };   // dX of X's type (and its FP8 copy), or of any type
+template <bool G32, bool XBF, int OUT>
+__global__ void __launch_bounds__(kLnThreads, kLnRowsPerSm) ln_bwd_rows_kernel(const LnArgs a, const int wpr) {
+  extern __shared__ __align__(16) float ln_smem[];             // exchanges [warps][1 + 3][4], then the combine [groups][2][cols]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int groups = nw / wpr, group = warp / wpr, col = ((warp - group * wpr) * 32 + lane) * 8;
+  const bool has = col < a.cols;
+  float4* means = reinterpret_cast<float4*>(ln_smem) + group * wpr;                       // of this row group: one per warp
+  float4* sums = reinterpret_cast<float4*>(ln_smem) + nw + 3 * group * wpr;               // three per warp
+  float* comb = ln_smem + 16 * nw;
+  const float inv_n = 1.0f / (float)a.cols;
+  auto meet = [&]() { ptx::named_barrier_sync(1 + group, 32 * wpr); };
+  const int zero = ptx::grid_wait_previous();
+  f32x2 w2[4], sw[4], sc[4];                                   // weights; column sums of g * xhat and of g
+  {
+    float w[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (has) load8(a.w, a.w_dt, 0, col + zero, a.cols, true, 0.f, w);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { w2[j] = pack2(w[2 * j], w[2 * j + 1]); sw[j] = sc[j] = pack2(0.f, 0.f); }
+  }
+  auto unpack = [](uint32_t w) { const float2 f = XBF ? unpack_bf16x2(w) : unpack_f16x2(w); return pack2(f.x, f.y); };
+  // The rows stay packed between the exchanges: without this the compiler keeps what it has unpacked, and spills.
+  auto packed = [](uint4& r) { asm volatile("" : "+r"(r.x), "+r"(r.y), "+r"(r.z), "+r"(r.w)); };
+  auto word = [](const uint4& r, int j) { return j == 0 ? r.x : j == 1 ? r.y : j == 2 ? r.z : r.w; };
+  const int64_t stride = (int64_t)gridDim.x * groups;
+  for (int64_t row0 = (int64_t)blockIdx.x * groups + group + zero; row0 < a.rows; row0 += kLnBatch * stride) {
+    const int64_t rest = (a.rows - row0 + stride - 1) / stride;
+    const int here = rest < kLnBatch ? (int)rest : kLnBatch;   // rows of this turn
+    uint4 cx[kLnBatch], cg[kLnBatch], ch[G32 ? kLnBatch : 1];  // packed rows; a float32 gradient takes two vectors
+#pragma unroll
+    for (int b = 0; b < kLnBatch; ++b) {
+      const int64_t row = row0 + b * stride;
+      cx[b] = cg[b] = make_uint4(0, 0, 0, 0);
+      if (G32) ch[G32 ? b : 0] = make_uint4(0, 0, 0, 0);
+      if (has && b < here) {
+        cx[b] = __ldg(reinterpret_cast<const uint4*>(static_cast<const char*>(a.x) + (row * a.x_ld + col) * 2));
+        const uint4* g = reinterpret_cast<const uint4*>(static_cast<const char*>(a.g) + (row * a.g_ld + col) * (G32 ? 4 : 2));
+        cg[b] = __ldg(g);
+        if (G32) ch[G32 ? b : 0] = __ldg(g + 1);
+      }
+    }
+    auto g_pair = [&](int b, int j) -> f32x2 {                 // gradient values 2 j, 2 j + 1 of row b
+      if (!G32) return unpack(word(cg[b], j));
+      const uint4& r = j < 2 ? cg[b] : ch[G32 ? b : 0];
+      return j & 1 ? pack2(__uint_as_float(r.z), __uint_as_float(r.w)) : pack2(__uint_as_float(r.x), __uint_as_float(r.y));
+    };
+    // ---- means
+    float v[kLnBatch], lo, hi;
+#pragma unroll
+    for (int b = 0; b < kLnBatch; ++b) {
+      v[b] = 0.f;
+      if (b >= here) continue;
+      unpack2(add2(add2(unpack(cx[b].x), unpack(cx[b].y)), add2(unpack(cx[b].z), unpack(cx[b].w))), lo, hi);
+      v[b] = lo + hi;
+    }
+    const float m = warp_sum4(v, lane);
+    float mu[kLnBatch] = {0.f, 0.f, 0.f, 0.f};
+    if (wpr == 1) {
+#pragma unroll
+      for (int b = 0; b < kLnBatch; ++b) mu[b] = __shfl_sync(0xffffffffu, m, b);
+    } else {
+      if (lane < 4) reinterpret_cast<float*>(&means[warp - group * wpr])[lane] = m;
+      meet();
+      for (int k = 0; k < wpr; ++k) { const float4 t = means[k]; mu[0] += t.x; mu[1] += t.y; mu[2] += t.z; mu[3] += t.w; }
+    }
+#pragma unroll
+    for (int b = 0; b < kLnBatch; ++b) packed(cx[b]);
+    // ---- variance about the mean, sums of u = g w and of u (x - mu)
+    float q[kLnBatch], su[kLnBatch], sd[kLnBatch];
+#pragma unroll
+    for (int b = 0; b < kLnBatch; ++b) {
+      q[b] = su[b] = sd[b] = 0.f;
+      if (b >= here) continue;
+      mu[b] *= inv_n;
+      const f32x2 neg = splat2(-mu[b]);
+      f32x2 q2 = pack2(0.f, 0.f), u2 = q2, d2 = q2;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const f32x2 d = add2(unpack(word(cx[b], j)), neg), u = mul2(g_pair(b, j), w2[j]);
+        q2 = fma2(d, d, q2); u2 = add2(u2, u); d2 = fma2(u, d, d2);
+      }
+      unpack2(q2, lo, hi); q[b] = has ? lo + hi : 0.f;
+      unpack2(u2, lo, hi); su[b] = lo + hi;                    // (zero beyond the row's end: g and w are)
+      unpack2(d2, lo, hi); sd[b] = lo + hi;
+    }
+    const float rq = warp_sum4(q, lane), ru = warp_sum4(su, lane), rd = warp_sum4(sd, lane);
+    if (wpr == 1) {
+#pragma unroll
+      for (int b = 0; b < kLnBatch; ++b) { q[b] = __shfl_sync(0xffffffffu, rq, b); su[b] = __shfl_sync(0xffffffffu, ru, b); sd[b] = __shfl_sync(0xffffffffu, rd, b); }
+    } else {
+      if (lane < 4) {
+        float* t = reinterpret_cast<float*>(&sums[3 * (warp - group * wpr)]) + lane;
+        t[0] = rq; t[4] = ru; t[8] = rd;
+      }
+      meet();
+#pragma unroll
+      for (int b = 0; b < kLnBatch; ++b) q[b] = su[b] = sd[b] = 0.f;
+      for (int k = 0; k < wpr; ++k) {
+        const float4 t0 = sums[3 * k], t1 = sums[3 * k + 1], t2 = sums[3 * k + 2];
+        q[0] += t0.x; q[1] += t0.y; q[2] += t0.z; q[3] += t0.w;
+        su[0] += t1.x; su[1] += t1.y; su[2] += t1.z; su[3] += t1.w;
+        sd[0] += t2.x; sd[1] += t2.y; sd[2] += t2.z; sd[3] += t2.w;
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < kLnBatch; ++b) { packed(cx[b]); packed(cg[b]); }
+    // ---- dX = beta_x rstd (u - mean(u) - xhat mean(u xhat)), column sums
+#pragma unroll
+    for (int b = 0; b < kLnBatch; ++b) {
+      const int64_t row = row0 + b * stride;
+      if (b >= here) continue;
+      const float rstd = rsqrtf(q[b] * inv_n + a.eps), k = a.beta_x * rstd;
+      const f32x2 rstd2 = splat2(rstd), shift = splat2(-mu[b] * rstd), k2 = splat2(k), c0 = splat2(-k * (su[b] * inv_n)),
+                  c1 = splat2(-k * (sd[b] * rstd * inv_n));
+      float d[8];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const f32x2 g2 = g_pair(b, j), xh = fma2(unpack(word(cx[b], j)), rstd2, shift);
+        sw[j] = fma2(g2, xh, sw[j]);
+        sc[j] = add2(sc[j], g2);
+        unpack2(fma2(xh, c1, fma2(mul2(g2, w2[j]), k2, c0)), d[2 * j], d[2 * j + 1]);
+      }
+      if (OUT >= kLnAny) {
+        if (has) ln_store8<OUT == kLnAnyCopy>(a, row, col, true, d);
+      } else if (has) {
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = XBF ? pack_bf16x2(d[2 * j], d[2 * j + 1]) : pack_f16x2(d[2 * j], d[2 * j + 1]);
+        *reinterpret_cast<uint4*>(static_cast<char*>(a.out) + (row * a.out_ld + col) * 2) = make_uint4(w[0], w[1], w[2], w[3]);
+        if (OUT != kLnSame) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) { const float2 t = XBF ? unpack_bf16x2(w[j]) : unpack_f16x2(w[j]); d[2 * j] = t.x; d[2 * j + 1] = t.y; }
+          constexpr bool E5 = OUT == kLnSameE5;
+          *reinterpret_cast<uint2*>(static_cast<char*>(a.q) + row * a.q_ld + col) =
+              make_uint2(cvt_fp8x4<E5>(d[0], d[1], d[2], d[3]), cvt_fp8x4<E5>(d[4], d[5], d[6], d[7]));
+        }
+      }
+    }
+  }
+  // ---- combine the CTA's row groups in their order; one partial row (G xhat sums, then G sums) per CTA
+  if (has) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      *reinterpret_cast<f32x2*>(comb + (size_t)(2 * group) * a.cols + col + 2 * j) = sw[j];
+      *reinterpret_cast<f32x2*>(comb + (size_t)(2 * group + 1) * a.cols + col + 2 * j) = sc[j];
+    }
+  }
+  __syncthreads();
+  float* dst = a.partial + (size_t)blockIdx.x * 2 * a.cols;
+  for (int j = threadIdx.x; j < 2 * a.cols; j += blockDim.x) {
+    float t = 0.f;
+    for (int g = 0; g < groups; ++g) t += comb[(size_t)g * 2 * a.cols + j];
+    dst[j] = t;
+  }
+}
+
 // dw_j = beta * sum over CTAs of partial[cta][0][j], dc_j likewise from partial[cta][1][j].
 // One CTA per 32 columns of the 2 * cols sums: 32 groups of 32 threads each add every 32nd partial row
 // in order (four independent partial sums per thread, combined in a fixed order), then the groups are
@@ -599,7 +748,8 @@ static int ln_bwd_grid(int64_t rows, int warps = kLnWarps, int per_sm = 2) {
   const int64_t cap = (int64_t)sms * per_sm;
   return (int)(want < cap ? want : cap);
 }
-constexpr int kLnFastWarps = 4, kLnFastPerSm = 3;   // the 16-bit backward kernel: three CTAs of four warps per SM
+
+constexpr int kLnFastWarps = 4, kLnFastPerSm = 3;   // of ln_bwd16_kernel
 
 template <bool COPY>
 static us_status ln_fwd_launch(const LnArgs& a, cudaStream_t st) {
@@ -651,25 +801,42 @@ static us_status ln_bwd_launch(const LnArgs& a, int grid, float beta_wc, const u
   const int nch = (a.cols + 255) / 256;
   int nparts = grid;
   // With no rows the first kernel still runs (one CTA) and writes zero partials, so dw = dc = 0.
-  if (a.vec_ok && nch <= 4 && (a.x_dt == US_BF16 || a.x_dt == US_F16) && (a.g_dt == a.x_dt || a.g_dt == US_F32)) {
-    const bool g32 = a.g_dt == US_F32;
-    nparts = ln_bwd_grid(a.rows > 0 ? a.rows : 1, kLnFastWarps, kLnFastPerSm);
-    const size_t smem = ((size_t)(nch <= 1 ? 1 : nch <= 2 ? 2 : 4) * 256 + (size_t)kLnFastWarps * a.cols) * sizeof(float) +
-                        (g32 ? (size_t)0 : (size_t)kLnFastWarps * kLnStages * (a.cols * 4 + 8));
+  const bool rows16 = a.vec_ok && (a.x_dt == US_BF16 || a.x_dt == US_F16);
+  // Beyond 16 M elements (X and G no longer stay in L2) a warp per row with a ring of bulk copies keeps more of memory busy.  us, rows among
+  // warps / warp per row, BF16: 16384 x 1024 30.9 / 30.6, 24576 x 1024 46.4 / 40.9, 32768 x 768 53.2 / 42.1, 65536 x 512 56.5 / 53.4; a float32 gradient
+  // 32768 x 1024 66 / 89, rows of at most 256 131072 x 256 48 / 75.
+  if (rows16 && a.g_dt == a.x_dt && nch > 1 && nch <= 4 && a.rows * a.cols > (16 << 20)) {
+    nparts = ln_bwd_grid(a.rows, kLnFastWarps, kLnFastPerSm);
+    const size_t smem = ((size_t)(nch <= 2 ? 2 : 4) * 256 + (size_t)kLnFastWarps * a.cols) * sizeof(float) + (size_t)kLnFastWarps * kLnStages * (a.cols * 4 + 8);
     const bool xbf = a.x_dt == US_BF16;
-    const int n = nch <= 1 ? 1 : nch <= 2 ? 2 : 4;
-    void (*fn)(const LnArgs) = nullptr;
-#define US_LN_PICK(N)                                                                                   \
-  fn = g32 ? (xbf ? ln_bwd16_kernel<N, true, true, COPY> : ln_bwd16_kernel<N, true, false, COPY>)       \
-           : (xbf ? ln_bwd16_kernel<N, false, true, COPY> : ln_bwd16_kernel<N, false, false, COPY>)
-    if (n == 1) US_LN_PICK(1);
-    else if (n == 2) US_LN_PICK(2);
-    else US_LN_PICK(4);
-#undef US_LN_PICK
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return host::failed();
+    void (*fn)(const LnArgs) = nch <= 2 ? (xbf ? ln_bwd16_kernel<2, true, COPY> : ln_bwd16_kernel<2, false, COPY>)
+                                        : (xbf ? ln_bwd16_kernel<4, true, COPY> : ln_bwd16_kernel<4, false, COPY>);
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return host::failed();
     const us_status launched = host::launch(fn, nullptr, nparts, 32 * kLnFastWarps, smem, 1, st, a);
+    if (launched != US_OK) return launched;
+  } else if (rows16 && nch <= kLnWarps && (a.g_dt == a.x_dt || a.g_dt == US_F32)) {
+    const int groups = kLnWarps / nch;
+    // rows per group: four, fewer where that would be few CTAs (1000 x 384 5.4 / 5.4 / 6.2 us with 4 / 2 / 1, 256 x 1024 6.2 / 5.8 / 6.0, 300 x 128 4.8 /
+    // 4.6 / 4.4; 4096 x 256 5.6 / 6.2 / 6.6: each CTA is a partial row that the second kernel adds)
+    const int64_t turns = (a.rows + kLnBatch * groups - 1) / (kLnBatch * groups);
+    nparts = ln_bwd_grid(a.rows > 0 ? a.rows : 1, (turns >= 64 ? 4 : turns >= 16 ? 2 : 1) * groups, kLnRowsPerSm);
+    const size_t smem = ((size_t)16 * nch * groups + (size_t)2 * groups * a.cols) * sizeof(float);
+    const bool g32 = a.g_dt == US_F32, xbf = a.x_dt == US_BF16;
+    const int out = a.out_dt != a.x_dt ? (COPY ? kLnAnyCopy : kLnAny) : !COPY ? kLnSame : a.q_dt == US_E5M2 ? kLnSameE5 : kLnSameE4;
+    void (*fn)(const LnArgs, const int) = nullptr;
+#define US_LN_PICK(OUT)                                                                            \
+  fn = g32 ? (xbf ? ln_bwd_rows_kernel<true, true, OUT> : ln_bwd_rows_kernel<true, false, OUT>)    \
+           : (xbf ? ln_bwd_rows_kernel<false, true, OUT> : ln_bwd_rows_kernel<false, false, OUT>)
+    if constexpr (COPY) {
+      if (out == kLnAnyCopy) US_LN_PICK(kLnAnyCopy);
+      else if (out == kLnSameE5) US_LN_PICK(kLnSameE5);
+      else US_LN_PICK(kLnSameE4);
+    } else {
+      if (out == kLnAny) US_LN_PICK(kLnAny);
+      else US_LN_PICK(kLnSame);
+    }
+#undef US_LN_PICK
+    const us_status launched = host::launch(fn, nullptr, nparts, 32 * nch * groups, smem, 1, st, a, nch);
     if (launched != US_OK) return launched;
   } else if (nch <= 4) {
     const size_t smem = (size_t)kLnWarps * a.cols * sizeof(float);
@@ -725,7 +892,7 @@ using namespace us;
 
 extern "C" size_t us_layer_norm_bwd_workspace_bytes(int64_t rows, int64_t cols) {
   if (rows <= 0 || cols <= 0) return 0;
-  const int g0 = ln_bwd_grid(rows), g1 = ln_bwd_grid(rows, kLnFastWarps, kLnFastPerSm);
+  const int g0 = ln_bwd_grid(rows), g1 = ln_bwd_grid(rows, 1, 3);
   const int grid = g0 > g1 ? g0 : g1;                // whichever kernel the call takes
   return (size_t)(grid > 0 ? grid : 1) * 2 * (size_t)cols * sizeof(float);
 }

@@ -118,3 +118,30 @@ def test_layer_norm_backward_with_a_float32_gradient(rows, cols, ld):
     U.assert_close_stored(dX, rdX, "bf16", 3e-5 * max(1.0, scale), "dX")
     tol = 8 * (2e-6 * np.sqrt(rows) + 1e-6)
     assert np.abs(dw.cpu().numpy() - rdw.reshape(-1)).max() <= tol and np.abs(dc.cpu().numpy() - rdc.reshape(-1)).max() <= tol
+
+
+@pytest.mark.parametrize("x_fmt,g_fmt,out_fmt,q_fmt", [("bf16", "bf16", "bf16", "e5m2"), ("fp16", "f32", "fp16", "e4m3"), ("bf16", "f32", "f32", None), ("fp16", "fp16", "bf16", "e5m2")])
+@pytest.mark.parametrize("rows,cols", [(1, 8), (3, 264), (37, 256), (130, 776), (67, 1288), (9, 2048), (5000, 136)])
+def test_layer_norm_backward_with_rows_among_several_warps(rows, cols, x_fmt, g_fmt, out_fmt, q_fmt):
+    """Rows of one to eight warps, turns of one to four rows, every output kind: dX and its copy in FP8, dw and dc."""
+    from paper_2303_11257_b200 import lib as L, synth
+    X, G, w, _ = _inputs(8, rows, cols, x_fmt)
+    G = synth.normal(8, 4, (rows, cols), 1.0)
+    eps, beta_wc = 1e-5, float(np.float32(rows ** -0.5))
+    dX, q = U.empty(rows, cols, out_fmt, cols + 24), U.empty(rows, cols, q_fmt, cols + 8) if q_fmt else None
+    dw, dc = torch.empty(cols, device="cuda"), torch.empty(cols, device="cuda")
+    ws = torch.empty(max(16, L.us_layer_norm_bwd_workspace_bytes(rows, cols)), dtype=torch.uint8, device="cuda")
+    args = (U.to_device(X, x_fmt), U.to_device(w, "f32"), U.to_device(G, g_fmt))
+    tail = (L._vec(dw), L._vec(dc), ws.data_ptr(), ws.numel())
+    m = [L.mat(t) for t in (*args, dX)]
+    name = "us_layer_norm_bwd_cast" if q_fmt else "us_layer_norm_bwd"
+    L.Call(name, m[0], m[1], m[2], eps, 1.0, beta_wc, m[3], *([L.mat(q)] if q_fmt else []), *tail)(L.current_stream())
+    Xv, Gv = U.values_of(X, x_fmt), U.values_of(G, g_fmt)
+    rx, rw, rc = O.layer_norm_bwd(Xv, w.astype(np.float64), Gv, eps, 1.0, beta_wc)
+    scale = 1.0 / np.sqrt(Xv.var(axis=1).min() + eps)
+    U.assert_close_stored(dX, rx, out_fmt, 3e-5 * max(1.0, scale), "dX")
+    tol = 8 * (2e-6 * np.sqrt(rows) + 1e-6)
+    assert np.abs(U.host_values(dw) - rw.ravel()).max() <= tol and np.abs(U.host_values(dc) - rc.ravel()).max() <= tol
+    if q_fmt:
+        most = 448 if q_fmt == "e4m3" else 57344
+        assert torch.equal(q.contiguous().view(torch.uint8), dX.float().clamp(-most, most).to(U.TORCH_OF[q_fmt]).contiguous().view(torch.uint8))
