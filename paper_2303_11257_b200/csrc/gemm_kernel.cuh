@@ -61,12 +61,14 @@ constexpr int kEpilogueWarps = 8;           // default: two per TMEM lane quarte
 __host__ __device__ constexpr int gemm_threads(int ew) { return 64 + 32 * ew; }
 // Staging per epilogue warp: EW = 8: two 32-row x 128-byte boxes; EW = 16: one such box (stored
 // pre-activation in or out, 64 columns of 16 bits) and one 32-row x 64-byte box (64 FP8 outputs).
-__host__ __device__ constexpr int epi_warp_bytes(int ew) { return ew == 16 ? 4096 + 2048 : 8192; }
+// kEpiPlain16: one box of 32 rows x 64 FP8 columns (in twice the room that takes, which keeps the stages' alignment).
+__host__ __device__ constexpr int epi_warp_bytes(int ew, bool plain = false) { return ew == 16 ? (plain ? 4096 : 4096 + 2048) : 8192; }
 
 // What the epilogue fuses, fixed at compile time so that each kernel carries one code path only.
 enum EpiKind {
   kEpiPlain = 0,     // scale, round, store
   kEpiPlainF32 = 6,  // the same with float32 output, single problems (beside the code of the other types 48 x 1024 x 4096 takes 3.9 us instead of 3.8)
+  kEpiPlain16 = 7,   // the same by sixteen warps, FP8 outputs of 256 x 256 tiles
   kEpiGelu = 1,      // + scaled GELU, optionally keeping the 16-bit pre-activation
   kEpiGeluGrad = 2,  // + scaled GELU gradient from the stored pre-activation
   kEpiSkip = 3,      // + weighted skip tensor (residual)
@@ -78,12 +80,12 @@ constexpr unsigned int kStatusTimeout = 1;
 
 // Shared-memory plan of one CTA.  CG = CTAs cooperating on a tile (1, or 2 = cta_group::2 pair):
 // a pair computes 256 x BN, each CTA holding its 128 rows of A and its BN/2 rows of B.
-template <int BN, int CG, int EW>
+template <int BN, int CG, int EW, bool PLAIN = false>
 struct GemmSmem {
   static constexpr int kABytes = kBM * kStageKBytes;
   static constexpr int kBBytes = (BN / CG) * kStageKBytes;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kEpiBytes = EW * epi_warp_bytes(EW);          // 64 KB (EW = 8) or 96 KB (EW = 16)
+  static constexpr int kEpiBytes = EW * epi_warp_bytes(EW, PLAIN);          // 64 KB (EW = 8) or 96 KB (EW = 16)
   static constexpr int kStages = (229376 - kEpiBytes) / kStageBytes; // 32 KB stages: 5 (EW = 8) or 4 (EW = 16)
   // A narrow tile (BN = 64) of a short matrix holds only the rows of A that exist, in as many stages as fit: one such CTA is bound
   // by the latency of its loads.  The MMA still reads 128 rows; what lies behind those of A ends up in rows that do not exist.
@@ -710,6 +712,71 @@ __device__ __forceinline__ void epilogue_act16(const GemmParams& p, const CUtens
   __syncwarp();
 }
 
+// Plain FP8 outputs of 256 x 256 tiles by sixteen warps, 64 columns each as in epilogue_act16: the second slice is loaded while the
+// first is rounded, and a tile is one box and one store per warp.  With eight warps of 128 columns a tile's epilogue takes longer
+// than the main loop of a short contraction.  us, FP8 operands and outputs: 8192 x 128 x 3072 16.2 -> 8.8, 8192 x 512 x 4096 22.1 -> 15.6, 8192 x 1024
+// x 3072 21.7 -> 20.3, 8192 x 2048 x 4096 45.4 -> 44.0, 8192 x 8192 x 4096 186 -> 186; weight gradient 512 x 8192 x 8192 38.9 -> 27.0.
+template <int BN, int CG>
+__device__ __forceinline__ void epilogue_plain16(const GemmParams& p, const CUtensorMap* tm_out, const EpiCtx& c) {
+  const int q = c.warp & 3, part = (c.warp - 2) >> 2, lane = c.lane;
+  const uint32_t out_sw = (uint32_t)((lane >> 1) & 3), dst = c.buf0 + (uint32_t)lane * 64u;
+  const f32x2 scale2 = splat2(p.scale);
+  auto slice = [&](const uint32_t (&r)[32], uint32_t chunk) {
+    float y[32];
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      unpack2(mul2(pack2(__uint_as_float(r[2 * k]), __uint_as_float(r[2 * k + 1])), scale2), y[2 * k], y[2 * k + 1]);
+    uint32_t w[8];
+    if (p.out_dt == US_E5M2) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) w[k] = cvt_fp8x4<true>(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) w[k] = cvt_fp8x4<false>(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]);
+    }
+    ptx::sts128(dst + ((chunk ^ out_sw) << 4), make_uint4(w[0], w[1], w[2], w[3]));
+    ptx::sts128(dst + (((chunk + 1) ^ out_sw) << 4), make_uint4(w[4], w[5], w[6], w[7]));
+  };
+  uint32_t local = 0;
+  for (int tile = c.group; tile < c.num_tiles; tile += c.num_groups, ++local) {
+    const uint32_t acc = local & 1u, acc_phase = (local >> 1) & 1u;
+    int tm, tn;
+    tile_mn(p, tile, tm, tn);
+    const int row0 = tm * (kBM * CG) + c.rank * kBM + q * 32, n_w = tn * BN + part * 64;
+    bool ok = wait_bounded(c.acc_full0 + 8u * acc, acc_phase, c.abort_flag, p.status, p.wait_limit);
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok) break;
+    ptx::tc_fence_after_sync();
+    const uint32_t t_row = c.tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + part * 64;
+    const bool active = n_w < p.N;                            // warp-uniform
+    uint32_t r0[32], r1[32];
+    if (active) {
+      ptx::tmem_ld_32x32_issue(t_row, r0);
+      if (ptx::elect_one()) ptx::bulk_wait_group_read<0>();   // the previous tile's store has read the box
+      __syncwarp();
+      ptx::tmem_ld_fence(r0);
+      ptx::tmem_ld_32x32_issue(t_row + 32, r1);
+      slice(r0, 0);
+      ptx::tmem_ld_fence(r1);
+    }
+    ptx::tc_fence_before_sync();
+    __syncwarp();
+    if (lane == 0 && tile + 2 * c.num_groups < c.num_tiles) { // (as in epilogue_staged)
+      if (CG == 2) ptx::mbar_arrive_cluster(ptx::in_even_cta(c.acc_empty0 + 8u * acc));
+      else ptx::mbar_arrive(c.acc_empty0 + 8u * acc);
+    }
+    if (active) {
+      slice(r1, 2);
+      ptx::fence_proxy_async_smem();
+      __syncwarp();
+      if (ptx::elect_one()) { ptx::tma_store_2d(tm_out, c.buf0, n_w, row0); ptx::bulk_commit_group(); }
+    }
+  }
+  ptx::tmem_ld_wait_all();
+  if (ptx::elect_one()) ptx::bulk_wait_group_read<0>();       // stores have left shared memory before the CTA may exit
+  __syncwarp();
+}
+
 // ES: operand element size in bytes (1 = FP8, 2 = BF16 / F16).
 // A_MN / B_MN: operand stored MN-major ([K x M] resp. [K x N] row-major) instead of K-major.
 // EPI: the fused epilogue (EpiKind).  EW: number of epilogue warps (8 or 16).
@@ -720,9 +787,9 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
             const __grid_constant__ CUtensorMap tmap_out, const __grid_constant__ CUtensorMap tmap_aux,
             const __grid_constant__ CUtensorMap tmap_skip, const GemmParams p) {
-  using S = GemmSmem<BN, CG, EW>;
+  using S = GemmSmem<BN, CG, EW, EPI == kEpiPlain16>;
   static_assert(!BATCHED || EPI == kEpiPlain, "batched problems take the plain epilogue");
-  static_assert(EW == 8 || (EW == 16 && (EPI == kEpiGelu || EPI == kEpiGeluGrad)), "16 epilogue warps serve the GELU epilogues only");
+  static_assert(EW == 8 || (EW == 16 && (EPI == kEpiGelu || EPI == kEpiGeluGrad || EPI == kEpiPlain16)), "16 epilogue warps: GELU and plain");
   constexpr int kBK = kStageKBytes / ES;            // K elements per stage
   constexpr int kChunkElems = 128 / ES;             // MN elements per 128-byte row of an MN-major tile
   constexpr uint32_t kChunkBytes = kBK * 128;       // one MN-major chunk: kBK rows of 128 bytes
@@ -898,10 +965,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
     ptx::grid_wait_previous();
     EpiCtx c;
     c.tmem_base = tmem_base; c.acc_full0 = acc_full_bar(0); c.acc_empty0 = acc_empty_bar(0);
-    c.in_bar = epi_in_bar(2 * (warp - 2)); c.buf0 = epi_base + (warp - 2) * epi_warp_bytes(EW);
+    c.in_bar = epi_in_bar(2 * (warp - 2)); c.buf0 = epi_base + (warp - 2) * epi_warp_bytes(EW, EPI == kEpiPlain16);
     c.abort_flag = abort_flag; c.warp = warp; c.lane = lane; c.rank = rank;
     c.group = group; c.num_groups = num_groups; c.num_tiles = num_tiles;
-    if constexpr (EW == 16) {
+    if constexpr (EPI == kEpiPlain16) {
+      epilogue_plain16<BN, CG>(p, &tmap_out, c);
+    } else if constexpr (EW == 16) {
       const uint32_t in_bar1 = epi_in_bar(2 * (warp - 2) + 1);
       const bool e5 = p.out_dt == US_E5M2, bf = p.aux_dt == US_BF16;
       if (e5 && bf) epilogue_act16<BN, CG, EPI, true, true>(p, &tmap_out, &tmap_aux, c, in_bar1);

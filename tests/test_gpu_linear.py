@@ -221,3 +221,18 @@ def test_other_activations_as_epilogues(fn, shape):
         L.us_linear_bwd_x(U.to_device(G, "e5m2"), U.to_device(W, "e4m3"), float(bx), dH, ws, ep)
         U.assert_close_stored(dH, ref, out_fmt, TOL * float(beta_f), f"{fn} gradient -> {out_fmt}")
     assert L.us_workspace_status(ws) == 0
+
+
+@pytest.mark.parametrize("op", ["fwd", "bwd_x", "bwd_w"])
+@pytest.mark.parametrize("fmt,out_fmt", [("e4m3", "e4m3"), ("bf16", "e5m2")])
+@pytest.mark.parametrize("rows,k,cols", [(2500, 64, 2500), (4600, 272, 1100), (1300, 144, 9000)])
+def test_plain_fp8_outputs_of_many_large_tiles(op, fmt, out_fmt, rows, k, cols):
+    """Several 256 x 256 tiles per CTA pair, ragged rows and columns, a last warp without columns: FP8 codes within one step."""
+    from paper_2303_11257_b200 import lib as L, synth
+    from tests.test_gpu_linear_narrow import PAD, _operands
+    A, B, val, scale = _operands(L, synth, op, rows, k, cols, 91, fmt, fmt)
+    ws, out = L.new_workspace(), U.empty(rows, cols, out_fmt, PAD(cols) + 16)
+    getattr(L, "us_linear_" + op)(A, B, scale, out, ws)
+    assert L.us_workspace_status(ws) == 0
+    U.assert_close_stored(out, val, out_fmt, 2e-3, op)
+    assert not out.as_strided((rows, PAD(cols) + 16), (PAD(cols) + 16, 1))[:, cols:].contiguous().view(torch.uint8).any()
