@@ -101,6 +101,8 @@ struct CastArgs {
   FastDiv d_row;                   // by chunks_per_row
 };
 
+// F32: float32 rows that start on 32-byte boundaries, read in whole sectors (see multi_cast_kernel).
+template <bool F32>
 __global__ void __launch_bounds__(kThreads) cast_kernel(const CastArgs p) {
   const int zero = ptx::grid_wait_previous();
   const uint32_t stride = gridDim.x * kThreads;
@@ -118,7 +120,8 @@ __global__ void __launch_bounds__(kThreads) cast_kernel(const CastArgs p) {
       at[k] = (int64_t)row * p.dst_ld + col;
       n[k] = (int)min((int64_t)kVec, p.cols - col);
       if (n[k] == kVec) {
-        load_vec<kVec>(p.src + i0 * dtype_size(p.src_dt), p.src_dt, v[k]);
+        if (F32) { ptx::ldg256(p.src + i0 * 4, v[k]); ptx::ldg256(p.src + i0 * 4 + 32, v[k] + 8); }
+        else load_vec<kVec>(p.src + i0 * dtype_size(p.src_dt), p.src_dt, v[k]);
       } else {
 #pragma unroll
         for (int i = 0; i < kVec; ++i) v[k][i] = i < n[k] ? load_one(p.src, p.src_dt, i0 + i) : 0.f;
@@ -342,7 +345,8 @@ extern "C" us_status us_cast_fp8(const us_mat* src, float scale, const us_mat* d
     const int sms = host::sm_count();
     if (sms <= 0) return US_ERR_CUDA;
     const int64_t want = ((int64_t)p.total + kThreads - 1) / kThreads, cap = (int64_t)sms * 8;
-    return host::launch(cast_kernel, nullptr, (int)(want < cap ? want : cap), kThreads, 0, 1, static_cast<cudaStream_t>(stream), p);
+    const bool f32 = src->dtype == US_F32 && reinterpret_cast<uintptr_t>(src->ptr) % 32 == 0 && (dense || src->ld % 8 == 0);
+    return host::launch(f32 ? cast_kernel<true> : cast_kernel<false>, nullptr, (int)(want < cap ? want : cap), kThreads, 0, 1, static_cast<cudaStream_t>(stream), p);
   }
   return ew_launch<kCast>(src, nullptr, dst, scale, 0.f, stream);
 }
