@@ -379,7 +379,16 @@ __global__ void __launch_bounds__(1024) softmax_xent_row_kernel(const XentArgs a
 // runs under two others' reductions.  2048 rows of 30522 BF16 logits: forward 39 -> 31 us (4.1 TB/s), backward with an E5M2
 // gradient 66 -> 56 us (3.3 TB/s; two exponentials per class make 28 us of it).  A wait that runs out falls back to loads
 // from global memory.
+// The maximum of packed 16-bit values, sums and scalings of float32 pairs, one product a class instead of three operations, and the E5M2
+// store chosen once a row, us: 2048 x 30522 forward 29.7 -> 27.1, backward E5M2 55.8 -> 44.2, BF16 54.4 -> 48.3; 2048 x 16400 E5M2 36.8 -> 30.4.
 constexpr int kXentStagedThreads = 512;
+template <int DT>
+__device__ __forceinline__ uint32_t max16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  if (DT == US_BF16) asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  else asm("max.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
 constexpr uint32_t kXentWaitLimit = 1u << 20;
 template <bool BWD, int DT>
 __global__ void __launch_bounds__(kXentStagedThreads, 3) softmax_xent_staged_kernel(const XentArgs a) {
@@ -410,36 +419,63 @@ __global__ void __launch_bounds__(kXentStagedThreads, 3) softmax_xent_staged_ker
     for (int c = tid; c < full; c += kXentStagedThreads) {
       const uint4 raw = staged ? ptx::lds128(data + (uint32_t)c * 16u)
                                : __ldg(reinterpret_cast<const uint4*>(static_cast<const char*>(a.x) + x_off * 2) + c);
-      float v[8];
-      unpack16x8(raw, DT, v);
-      fn(8 * c, v);
+      const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+      fn(8 * c, w);
     }
   };
-  float m = last;
-  for_chunks([&](int, float (&v)[8]) {
+  auto pair = [](uint32_t w) { const float2 f = DT == US_BF16 ? unpack_bf16x2(w) : unpack_f16x2(w); return pack2(f.x, f.y); };
+  uint32_t m2 = DT == US_BF16 ? 0xff80ff80u : 0xfc00fc00u;    // the maximum of 16-bit values needs no widening
+  for_chunks([&](int, const uint32_t (&w)[4]) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) m = fmaxf(m, v[i]);
+    for (int i = 0; i < 4; ++i) m2 = max16x2<DT>(m2, w[i]);
   });
-  m = cta_reduce<true>(m, slots[0]);
+  float m, mo;
+  unpack2(pair(m2), m, mo);
+  m = cta_reduce<true>(fmaxf(last, fmaxf(m, mo)), slots[0]);
   const float mb = m * kLog2e;
-  float sum = tid < tail ? ex2_approx(fmaf(last, kLog2e, -mb)) : 0.f;
-  for_chunks([&](int, float (&v)[8]) {
+  const f32x2 l2 = splat2(kLog2e), neg = splat2(-mb);
+  f32x2 sum2 = pack2(tid < tail ? ex2_approx(fmaf(last, kLog2e, -mb)) : 0.f, 0.f);
+  for_chunks([&](int, const uint32_t (&w)[4]) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) sum += ex2_approx(fmaf(v[i], kLog2e, -mb));
+    for (int i = 0; i < 4; ++i) {
+      float a0, a1;
+      unpack2(fma2(pair(w[i]), l2, neg), a0, a1);
+      sum2 = add2(sum2, pack2(ex2_approx(a0), ex2_approx(a1)));
+    }
   });
-  sum = cta_reduce<false>(sum, slots[1]);
+  float sum, so;
+  unpack2(sum2, sum, so);
+  sum = cta_reduce<false>(sum + so, slots[1]);
   if (!BWD) {
     if (tid == 0) static_cast<float*>(a.out)[row] = (xt - m) - 0.6931471805599453f * __log2f(sum);
   } else {
     const float k = a.beta * gr, inv = 1.0f / sum;
     const int64_t out_off = row * a.out_ld;
-    for_chunks([&](int col, float (&v)[8]) {
+    const f32x2 c2 = splat2(-k * inv);
+    auto gradients = [&](auto&& put) {
+      for_chunks([&](int col, const uint32_t (&w)[4]) {
+        float v[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = ex2_approx(fmaf(v[i], kLog2e, -mb)) * inv;
+        for (int i = 0; i < 4; ++i) {
+          float a0, a1;
+          unpack2(fma2(pair(w[i]), l2, neg), a0, a1);
+          unpack2(mul2(pack2(ex2_approx(a0), ex2_approx(a1)), c2), v[2 * i], v[2 * i + 1]);
+        }
+        if ((unsigned)(t - col) < 8u) {                        // the target's class
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = k * ((col + i == t ? 1.0f : 0.f) - v[i]);
-      store8(a.out, a.out_dt, out_off, col, a.cols, true, v);
-    });
+          for (int i = 0; i < 8; ++i)
+            if (col + i == t) v[i] += k;
+        }
+        put(col, v);
+      });
+    };
+    if (a.out_dt == US_E5M2) {
+      gradients([&](int col, const float (&v)[8]) {
+        *reinterpret_cast<uint2*>(static_cast<char*>(a.out) + out_off + col) = make_uint2(cvt_fp8x4<true>(v[0], v[1], v[2], v[3]), cvt_fp8x4<true>(v[4], v[5], v[6], v[7]));
+      });
+    } else {
+      gradients([&](int col, const float (&v)[8]) { store8(a.out, a.out_dt, out_off, col, a.cols, true, v); });
+    }
     if (tid < tail) {
       const int col = 8 * full + tid;
       store_one(a.out, a.out_dt, out_off + col, k * ((col == t ? 1.0f : 0.f) - ex2_approx(fmaf(last, kLog2e, -mb)) * inv));
