@@ -530,7 +530,10 @@ us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_m
   CUtensorMap t[6];
   const int out_box = tile / 4 * es;                             // bytes per row of an epilogue warp's output box
   if (!make_tmap(&t[0], X, es, x_rows, 128) || !make_tmap(&t[1], W1, es, 128 / es, split > 1 && es == 1 ? 64 : 128) ||
-      !make_tmap(&t[2], G, es, x_rows, 128) || !make_tmap(&t[3], W2, es, split > 1 ? 64 : 128, 128) || !make_tmap(&t[4], A, es, 32, out_box) || !make_tmap(&t[5], dH, es, 32, out_box))
+      !make_tmap(&t[2], G, es, x_rows, 128) || !make_tmap(&t[3], W2, es, split > 1 ? 64 : 128, 128))
+    return US_ERR_CUDA;
+  t[4] = t[5] = t[0];                                            // (CTAs that share a tile store without them)
+  if (split == 1 && (!make_tmap(&t[4], A, es, 32, out_box) || !make_tmap(&t[5], dH, es, 32, out_box)))
     return US_ERR_CUDA;
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);

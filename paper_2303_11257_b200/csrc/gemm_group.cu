@@ -78,7 +78,6 @@ bool deal(GroupParams& g, int es, int tile_m, int bn, int split, int units, int 
   uint32_t heap[kGroupMaxUnits];                        // load << 8 | unit, a binary heap with the least on top
   int filled[kGroupMaxUnits] = {0};
   for (int u = 0; u < units; ++u) heap[u] = (uint32_t)u;
-  std::fill(g.table, g.table + kGroupMaxItems, -1);
   const auto more = [](uint32_t x, uint32_t y) { return x > y; };
   int rounds = 0;
   const int kbk = 128 / es;
@@ -96,8 +95,11 @@ bool deal(GroupParams& g, int es, int tile_m, int bn, int split, int units, int 
           const uint32_t top = heap[units - 1], unit = top & 0xffu;
           const int slot = filled[unit] * units + (int)unit;
           if (filled[unit] >= max_rounds || slot >= kGroupMaxItems || (top >> 8) + cost >= (1u << 24)) return false;
+          if (++filled[unit] > rounds) {                            // a new round: nobody has an entry yet
+            std::fill(g.table + rounds * units, g.table + std::min((rounds + 1) * units, kGroupMaxItems), -1);
+            ++rounds;
+          }
           g.table[slot] = (order[o] << 28) | (tm << 14) | tn;
-          rounds = std::max(rounds, ++filled[unit]);
           heap[units - 1] = (((top >> 8) + cost) << 8) | unit;
           std::push_heap(heap, heap + units, more);
         }

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "../../include/unitscale.h"
 
@@ -47,7 +48,9 @@ us_status launch(void (*kern)(P...), std::atomic<uint64_t>* smem_set, int grid, 
   attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = cluster > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kern, P(args)...) == cudaSuccess ? US_OK : failed();
+  static_assert((std::is_same_v<P, A> && ...), "parameters are handed over as they are, without a copy");
+  void* params[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+  return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kern), params) == cudaSuccess ? US_OK : failed();
 }
 
 // Number of SMs of the current device (cached per device), or -1 on error.

@@ -851,7 +851,7 @@ static us_status ln_bwd_launch(const LnArgs& a, int grid, float beta_wc, const u
   }
   if (cudaGetLastError() != cudaSuccess) return US_ERR_CUDA;
   const int rgrid = (2 * a.cols + 31) / 32;
-  return host::launch(ln_bwd_reduce_kernel, nullptr, rgrid, 32 * kLnReduceGroups, 0, 1, st, a.partial, nparts, a.cols, beta_wc, dw->ptr,
+  return host::launch(ln_bwd_reduce_kernel, nullptr, rgrid, 32 * kLnReduceGroups, 0, 1, st, static_cast<const float*>(a.partial), nparts, a.cols, beta_wc, dw->ptr,
                       dw->dtype, dc->ptr, dc->dtype);
 }
 
