@@ -292,7 +292,7 @@ __device__ __forceinline__ void xent_unpack(const XentChunk<DT>& c, float (&v)[8
   }
 }
 // k (onehot - p) for eight consecutive classes, the target being number `at` of them: the comparison is made once for all eight.  (A gain of 2
-// to 4 % with a warp per row and in the ring; the branch keeps the chunks of the register form apart, 1000 x 10752 float32 gradients 14.1 -> 15.4 us.)
+// to 4 % with a warp per row; the branch keeps the chunks of the register form apart, 1000 x 10752 float32 gradients 14.1 -> 15.4 us.)
 __device__ __forceinline__ void xent_grad(float (&p)[8], float k, unsigned at) {
   if (at < 8u) {
 #pragma unroll
@@ -546,8 +546,8 @@ __global__ void __launch_bounds__(kXentStagedThreads, 3) softmax_xent_staged_ker
 // Persistent CTAs of T threads, 1024 / T of them per SM, walk the rows of a 16-bit vocabulary: a ring of kXentRing rows in shared
 // memory is filled by bulk copies ahead of the row that is worked on, and a thread holds its (at most 32) elements of that
 // row in registers, widened, from the maximum to the write.  Each exponential is computed once (twice in the other forms, which the
-// ex2 unit bounds).  E5M2 gradient of 2048 rows of BF16 logits: 16384 classes 33.5 -> 27.1 us, 12000 24.6 -> 22.1, 8192 17.2 -> 14.0;
-// 4096 rows of 5000 22.0 -> 20.0 (xent_launch_dt has the lines).  Rows of up to 4096 classes gain nothing, longer ones than 16384 leave room for one CTA an SM and
+// ex2 unit bounds).  E5M2 gradient of 4096 rows of BF16 logits, the register form / this one: 16384 classes 59.8 / 46.1 us, 12000 45.7 / 39.0,
+// 8192 32.5 / 22.6, 5000 20.0 / 17.5 (xent_launch_dt has the lines).  Rows of up to 4096 classes gain nothing, longer ones than 16384 leave room for one CTA an SM and
 // lose, and so does the forward pass, which has no second exponential to save.
 // A wait that runs out falls back to loads from global memory.
 constexpr int kXentRing = 3;
@@ -836,10 +836,10 @@ static us_status xent_launch_dt(const XentArgs& a, cudaStream_t st) {
   if constexpr (DT != US_F32) {
     // The ring: wherever every row has a CTA of its own; with more rows not for float32 gradients, whose writes bound both forms and are
     // less even from fewer CTAs, not for 8193 to 10240 classes, where the register form has five chunks a thread and 256 threads, the
-    // ring 512 of which few have more than two, and not below 5000.  Registers against ring, times as fast, 4104 / 6000 / 8192 / 8200 / 10000 /
-    // 10752 / 16384 classes: 1 to 296 rows 1.2 to 1.6 at any; E5M2 or BF16 gradients of 1000 rows 0.97 / 1.08 / 1.14 / 0.91 / 0.93 / 1.00 / 1.05, of
-    // 4096 1.04 / 1.18 / 1.26 / 0.93 / 0.98 / 1.09 / 1.14; float32 of 592 rows 1.13 / 1.15 / 1.20 / 0.91 / 0.95 / 1.04 / 1.03, of 4096 0.86 / 0.97 /
-    // 0.97 / 0.78 / 0.83 / 0.95 / 0.87.
+    // ring 512 of which few have more than two, and not below 5000.  Registers over ring, BF16 logits, 4104 / 5000 / 6000 / 8192 / 8200 / 10000 /
+    // 10752 / 12000 / 16384 classes: 148 rows, E5M2 1.34 1.33 1.50 1.71 1.33 1.33 1.40 1.38 1.58, BF16 1.21 to 1.55, float32 1.18 1.20 1.23 1.34 1.01 0.96 1.00 0.98
+    // 1.01; 1000 rows, E5M2 1.03 1.06 1.12 1.32 0.95 1.04 1.07 1.07 1.19, BF16 0.94 0.97 1.05 1.18 0.88 0.95 1.00 1.00 1.08, float32 0.87 0.91 0.98 1.07 0.76 0.82
+    // 0.84 0.82 0.92; 4096 rows, E5M2 1.10 1.14 1.24 1.43 1.07 1.11 1.16 1.17 1.30, BF16 0.97 1.01 1.13 1.20 0.98 1.01 1.06 1.06 1.18, float32 0.81 to 1.00.
     const int t = a.cols > 8192 ? 512 : 256, units = sms * (1024 / t);
     const bool walks = a.out_dt != US_F32 && ((a.cols >= 5000 && a.cols <= 8192) || a.cols > 10240);
     if (BWD && a.vec_ok && a.cols > 4096 && a.cols <= 16384 && (rows <= units || walks)) {
