@@ -683,7 +683,7 @@ def operand(rows: int, cols: int, dtype, device="cuda") -> torch.Tensor:
     of 16, are not padded."""
     per = 128 // dtype.itemsize
     pitch = -(-cols // per) * per if cols % 16 == 0 and cols >= per else cols
-    return torch.empty((rows, pitch), dtype=dtype, device=device)[:, :cols]
+    return torch.empty_strided((rows, cols), (pitch, 1), dtype=dtype, device=device)   # (a slice of torch.empty: 5 us instead of 1.4)
 
 
 def _padded(dsts) -> bool:
