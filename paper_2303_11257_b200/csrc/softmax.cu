@@ -327,6 +327,16 @@ __device__ __forceinline__ f32x2 pair16(uint32_t w) {
   const float2 f = DT == US_BF16 ? unpack_bf16x2(w) : unpack_f16x2(w);
   return pack2(f.x, f.y);
 }
+// Factors of a row's gradients k (onehot - e / sum), e the exponential of a class: k (1 - e / sum) at the target, e (-k / sum) elsewhere, one
+// product a class.  (The target's is not the same product plus k: with an infinite k that would be NaN.  The zero that is added makes the
+// gradient of a class of weight zero +0, as k (0 - 0) is.)
+struct XentScale {
+  float k, inv;
+  f32x2 each;
+  __device__ __forceinline__ XentScale(float k, float inv) : k(k), inv(inv), each(splat2(-k * inv)) {}
+  __device__ __forceinline__ float target(float e) const { return k * (1.0f - e * inv); }
+  __device__ __forceinline__ f32x2 others(f32x2 e) const { return fma2(e, each, splat2(0.f)); }
+};
 // Eight gradients into a row at a column that is a multiple of eight, all of them in the row.
 __device__ __forceinline__ void xent_put(const XentArgs& a, int64_t out_off, int col, const float (&v)[8]) {
   if (a.out_dt == US_E5M2)
@@ -345,6 +355,10 @@ __global__ void __launch_bounds__(1024) softmax_xent_row_kernel(const XentArgs a
   const int t = a.t[row];
   const bool valid = t >= 0 && t < a.cols;                   // a target outside the row: NaN forward, no one-hot term backward
   float xt = __int_as_float(0x7fc00000), gr = 1.0f;
+  // kPairs: float32 pairs, and one product a gradient; gradients of one or two chunks a thread, of float32 rows up to three, stay scalar (2048 x
+  // 1500 BF16 logits 6.4 us, in pairs 6.8; 2048 x 3000 8.4 -> 7.9, 4000 x 12000 44.1 -> 38.6, forward 25.3 -> 21.1; float32 logits and gradients
+  // 4000 x 12000 74, in pairs 76 to 79).
+  constexpr bool kPairs = !BWD || NCH == 0 || NCH > (DT == US_F32 ? 3 : 2);
   if (!BWD && threadIdx.x == 0 && valid) xt = load_one(a.x, DT, x_off + t);
   if (BWD && a.g) gr = a.g[row];
   XentChunk<DT> keep[NCH > 0 ? NCH : 1];
@@ -386,9 +400,6 @@ __global__ void __launch_bounds__(1024) softmax_xent_row_kernel(const XentArgs a
   }
   m = cta_reduce<true>(m, slots[0]);
   const float mb = m * kLog2e;
-  // Float32 pairs, and one product a gradient; gradients of one or two chunks a thread stay scalar (2048 x 1500 BF16 logits 6.4 us, in pairs
-  // 6.8; 2048 x 3000 8.4 -> 7.9, 4000 x 12000 44.1 -> 38.6, forward 25.3 -> 21.1).
-  constexpr bool kPairs = !BWD || NCH == 0 || NCH > 2;
   const f32x2 l2 = splat2(kLog2e), neg = splat2(-mb);
   f32x2 sum2 = pack2(0.f, 0.f);
   float sum = 0.f;
@@ -417,8 +428,12 @@ __global__ void __launch_bounds__(1024) softmax_xent_row_kernel(const XentArgs a
   }
   const float k = a.beta * gr;
   const float inv = 1.0f / sum;
-  const f32x2 c2 = splat2(-k * inv);
+  const XentScale f(k, inv);
   const int64_t out_off = row * a.out_ld;
+  // The target's gradient is written over what the same thread has put there: chosen among its chunk's eight in the loop it takes registers that
+  // the longest rows lack (us, in the loop / behind it: 2048 x 9000 in BF16 18.7 / 17.2, 2048 x 4500 into E5M2 12.2 / 11.0).
+  const bool mine = kPairs && valid && (t >> 3) % (int)blockDim.x == (int)threadIdx.x;        // the target is in a chunk of this thread
+  if (mine) xt = load_one(a.x, DT, x_off + t);
   for_chunks([&](int col, float (&v)[8]) {
     if constexpr (!kPairs) {
 #pragma unroll
@@ -431,13 +446,12 @@ __global__ void __launch_bounds__(1024) softmax_xent_row_kernel(const XentArgs a
       for (int i = 0; i < 4; ++i) {
         float a0, a1;
         unpack2(fma2(pack2(v[2 * i], v[2 * i + 1]), l2, neg), a0, a1);
-        unpack2(mul2(pack2(ex2_approx(a0), ex2_approx(a1)), c2), v[2 * i], v[2 * i + 1]);
+        unpack2(f.others(pack2(ex2_approx(a0), ex2_approx(a1))), v[2 * i], v[2 * i + 1]);
       }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] += col + i == t ? k : 0.f;
     }
     store8(a.out, a.out_dt, out_off, col, a.cols, a.vec_ok && col + 8 <= a.cols, v);
   });
+  if (mine) store_one(a.out, a.out_dt, out_off + t, f.target(ex2_approx(fmaf(xt, kLog2e, -mb))));
 }
 
 // One CTA per row of 16-bit logits staged in shared memory by one bulk copy, for vocabularies whose rows the register form
@@ -466,7 +480,7 @@ __global__ void __launch_bounds__(kXentStagedThreads, 3) softmax_xent_staged_ker
   const int t = a.t[row];
   const bool valid = t >= 0 && t < a.cols;                   // a target outside the row: NaN forward, no one-hot term backward
   float xt = __int_as_float(0x7fc00000), gr = 1.0f;
-  if (!BWD && tid == 0 && valid) xt = load_one(a.x, DT, x_off + t);
+  if ((BWD || tid == 0) && valid) xt = load_one(a.x, DT, x_off + t);
   if (BWD && a.g) gr = a.g[row];
   const float last = tid < tail ? load_one(a.x, DT, x_off + 8 * full + tid) : -INFINITY;
   __syncthreads();
@@ -509,7 +523,8 @@ __global__ void __launch_bounds__(kXentStagedThreads, 3) softmax_xent_staged_ker
   } else {
     const float k = a.beta * gr, inv = 1.0f / sum;
     const int64_t out_off = row * a.out_ld;
-    const f32x2 c2 = splat2(-k * inv);
+    const XentScale f(k, inv);
+    const float gt = f.target(ex2_approx(fmaf(xt, kLog2e, -mb)));
     auto gradients = [&](auto&& put) {
       for_chunks([&](int col, const uint32_t (&w)[4]) {
         float v[8];
@@ -517,12 +532,12 @@ __global__ void __launch_bounds__(kXentStagedThreads, 3) softmax_xent_staged_ker
         for (int i = 0; i < 4; ++i) {
           float a0, a1;
           unpack2(fma2(pair(w[i]), l2, neg), a0, a1);
-          unpack2(mul2(pack2(ex2_approx(a0), ex2_approx(a1)), c2), v[2 * i], v[2 * i + 1]);
+          unpack2(f.others(pack2(ex2_approx(a0), ex2_approx(a1))), v[2 * i], v[2 * i + 1]);
         }
-        if ((unsigned)(t - col) < 8u) {                        // the target's class
+        if ((unsigned)t - (unsigned)col < 8u) {                // the target's class
 #pragma unroll
           for (int i = 0; i < 8; ++i)
-            if (col + i == t) v[i] += k;
+            if (col + i == t) v[i] = gt;
         }
         put(col, v);
       });
@@ -634,7 +649,7 @@ __global__ void __launch_bounds__(T, 1024 / T) softmax_xent_ring_kernel(const Xe
     unpack2(sum2, sum, so);
     sum = ring_reduce<false, T>(sum + so, slots[i & 1][1]);
     const float k = a.beta * gr, inv = 1.0f / sum;
-    const f32x2 c2 = splat2(-k * inv);
+    const XentScale f(k, inv);
     const int64_t out_off = row * a.out_ld;
 #pragma unroll
     for (int c = 0; c < kCh; ++c) {
@@ -642,11 +657,14 @@ __global__ void __launch_bounds__(T, 1024 / T) softmax_xent_ring_kernel(const Xe
       if (tid + c * T < full) {
         float g[8];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) unpack2(mul2(v[c][e], c2), g[2 * e], g[2 * e + 1]);
-        if ((unsigned)(t - col) < 8u) {                        // the target's class
+        for (int e = 0; e < 4; ++e) unpack2(f.others(v[c][e]), g[2 * e], g[2 * e + 1]);
+        if ((unsigned)t - (unsigned)col < 8u) {                // the target's class
 #pragma unroll
-          for (int e = 0; e < 8; ++e)
-            if (col + e == t) g[e] += k;
+          for (int e = 0; e < 8; ++e) {
+            float lo, hi;
+            unpack2(v[c][e / 2], lo, hi);
+            if (col + e == t) g[e] = f.target(e & 1 ? hi : lo);
+          }
         }
         xent_put(a, out_off, col, g);
       }

@@ -155,3 +155,27 @@ def test_softmax_xent_backward_of_rows_that_are_not_finite(rows, cols, out_fmt):
     pick = np.unique(np.concatenate([good[:16], good[::37], good[-3:]]))
     ref = O.softmax_xent_bwd(X.double().cpu().numpy()[pick], t[pick], np.ones(len(pick)), 8.0)
     U.assert_close_stored(dX[torch.from_numpy(pick).cuda()], ref, out_fmt, 3e-6 * 8.0, "xent bwd")
+
+
+@pytest.mark.parametrize("rows,cols,out_fmt", [(700, 3000, "bf16"), (700, 5000, "f32"), (700, 6003, "bf16"), (700, 9000, "f32"), (300, 12001, "e5m2"), (9, 20003, "f32"), (9, 40001, "bf16")])
+@pytest.mark.parametrize("in_fmt", ["bf16", "fp16"])
+def test_softmax_xent_backward_of_an_infinite_gradient(rows, cols, out_fmt, in_fmt):
+    """beta g (onehot - p) with an infinite g (a loss that overflowed): infinite at the target and of the other sign elsewhere (saturated
+    in FP8), not NaN; with a finite one a class of weight zero gets +0.  In registers, the ring, staged and read again."""
+    L, synth = _mods()
+    ld = (cols + 15) // 16 * 16
+    x, g = synth.normal(38, cols, (rows, cols), 2.0), np.ones(rows, np.float32)
+    t = (np.arange(rows) * 7919 % cols).astype(np.int32)
+    t[8] = cols - 1
+    g[[2, 8]], g[5] = np.inf, -np.inf
+    x[3, ::2] = -np.inf
+    dX = U.empty(rows, cols, out_fmt, ld)
+    L.us_softmax_xent_bwd(U.to_device(x, in_fmt, ld), torch.from_numpy(t).cuda(), torch.from_numpy(g).cuda(), 8.0, dX)
+    got = dX.float().cpu().numpy()
+    most = 57344.0 if out_fmt == "e5m2" else np.inf
+    for r in (2, 5, 8):
+        want = np.full(cols, -most if g[r] > 0 else most)
+        want[t[r]] *= -1
+        assert np.array_equal(got[r], want)
+    off = np.setdiff1d(np.arange(0, cols, 2), t[3])
+    assert not got[3, off].any() and not np.signbit(got[3, off]).any()
