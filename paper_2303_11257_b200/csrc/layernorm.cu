@@ -528,7 +528,9 @@ __global__ void __launch_bounds__(kLnThreads, kLnRowsPerSm) ln_bwd_rows_kernel(c
   float4* means = reinterpret_cast<float4*>(ln_smem) + group * wpr;                       // of this row group: one per warp
   float4* sums = reinterpret_cast<float4*>(ln_smem) + nw + 3 * group * wpr;               // three per warp
   float* comb = ln_smem + 16 * nw;
-  const float inv_n = 1.0f / (float)a.cols;
+  const float inv_n = 1.0f / (float)a.cols, inv_rest = fmaf(-inv_n, (float)a.cols, 1.0f) * inv_n;
+  // s / cols as a division rounds it, or the value next to that
+  auto mean = [&](float s) { return fmaf(s, inv_n, isinf(s) ? 0.f : s * inv_rest); };
   auto meet = [&]() { ptx::named_barrier_sync(1 + group, 32 * wpr); };
   const int zero = ptx::grid_wait_previous();
   f32x2 w2[4], sw[4], sc[4];                                   // weights; column sums of g * xhat and of g
@@ -591,7 +593,7 @@ __global__ void __launch_bounds__(kLnThreads, kLnRowsPerSm) ln_bwd_rows_kernel(c
     for (int b = 0; b < kLnBatch; ++b) {
       q[b] = su[b] = sd[b] = 0.f;
       if (b >= here) continue;
-      mu[b] *= inv_n;
+      mu[b] = mean(mu[b]);
       const f32x2 neg = splat2(-mu[b]);
       f32x2 q2 = pack2(0.f, 0.f), u2 = q2, d2 = q2;
 #pragma unroll
@@ -629,13 +631,13 @@ __global__ void __launch_bounds__(kLnThreads, kLnRowsPerSm) ln_bwd_rows_kernel(c
     for (int b = 0; b < kLnBatch; ++b) {
       const int64_t row = row0 + b * stride;
       if (b >= here) continue;
-      const float rstd = rsqrtf(q[b] * inv_n + a.eps), k = a.beta_x * rstd;
-      const f32x2 rstd2 = splat2(rstd), shift = splat2(-mu[b] * rstd), k2 = splat2(k), c0 = splat2(-k * (su[b] * inv_n)),
+      const float rstd = rsqrtf(mean(q[b]) + a.eps), k = a.beta_x * rstd;
+      const f32x2 rstd2 = splat2(rstd), neg = splat2(-mu[b]), k2 = splat2(k), c0 = splat2(-k * (su[b] * inv_n)),
                   c1 = splat2(-k * (sd[b] * rstd * inv_n));
       float d[8];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const f32x2 g2 = g_pair(b, j), xh = fma2(unpack(word(cx[b], j)), rstd2, shift);
+        const f32x2 g2 = g_pair(b, j), xh = mul2(add2(unpack(word(cx[b], j)), neg), rstd2);     // (exact where the mean is far above the spread)
         sw[j] = fma2(g2, xh, sw[j]);
         sc[j] = add2(sc[j], g2);
         unpack2(fma2(xh, c1, fma2(mul2(g2, w2[j]), k2, c0)), d[2 * j], d[2 * j + 1]);
@@ -750,7 +752,6 @@ static int ln_bwd_grid(int64_t rows, int warps = kLnWarps, int per_sm = 2) {
 }
 
 constexpr int kLnFastWarps = 4, kLnFastPerSm = 3;   // of ln_bwd16_kernel
-
 template <bool COPY>
 static us_status ln_fwd_launch(const LnArgs& a, cudaStream_t st) {
   const int64_t grid64 = (a.rows + kLnWarps - 1) / kLnWarps;

@@ -145,3 +145,42 @@ def test_layer_norm_backward_with_rows_among_several_warps(rows, cols, x_fmt, g_
     if q_fmt:
         most = 448 if q_fmt == "e4m3" else 57344
         assert torch.equal(q.contiguous().view(torch.uint8), dX.float().clamp(-most, most).to(U.TORCH_OF[q_fmt]).contiguous().view(torch.uint8))
+
+
+@pytest.mark.parametrize("cols", [512, 1024, 2048])
+@pytest.mark.parametrize("g_fmt", ["fp16", "f32"])
+def test_layer_norm_backward_of_rows_far_from_zero(cols, g_fmt):
+    """Rows of whole numbers about 1500 with a spread of 1.4 and a gradient that goes along with them: sums and means are exact in float32, so
+    that x - mu is.  What is left is 1 / sigma and the products: 2^-22 relative in every term of dX (at most 8 of up to 4), and in the 16
+    terms of dw.  (A normalised input formed as x / sigma - mu / sigma rounds at 1060: 6e-5 in dX, 8e-4 in dw.)"""
+    from paper_2303_11257_b200 import lib as L
+    rows, rng = 16, np.random.default_rng(cols)
+    D = rng.integers(-2, 3, (rows, cols))
+    X, G, w = (1500 + D).astype(np.float32), (1 + D + rng.integers(-1, 2, (rows, cols))).astype(np.float32), np.ones((1, cols), np.float32)
+    dX, dw, dc = U.empty(rows, cols, "f32"), torch.empty(cols, device="cuda"), torch.empty(cols, device="cuda")
+    ws = torch.empty(max(L.us_layer_norm_bwd_workspace_bytes(rows, cols), 16), dtype=torch.uint8, device="cuda")
+    L.us_layer_norm_bwd(U.to_device(X, "fp16"), torch.from_numpy(w[0]).cuda(), U.to_device(G, g_fmt), 1e-5, 1.0, 1.0, dX, dw, dc, ws)
+    rdX, rdw, rdc = O.layer_norm_bwd(X, w, G, np.float32(1e-5), 1.0, 1.0)
+    assert np.abs(U.host_values(dX) - rdX).max() <= 1e-5
+    assert np.abs(dw.cpu().numpy() - rdw.reshape(-1)).max() <= 5e-5
+    assert np.array_equal(dc.cpu().numpy(), rdc.reshape(-1).astype(np.float32))
+
+
+@pytest.mark.parametrize("rows,cols", [(37, 256), (70, 1000), (70, 1536), (300, 2048)])
+@pytest.mark.parametrize("g_fmt", ["bf16", "f32"])
+def test_layer_norm_backward_of_rows_that_are_not_finite(rows, cols, g_fmt):
+    """A NaN or an infinity makes its own row of dX NaN and no other; a row whose squares overflow float32 has 1 / sigma = 0 and a gradient of 0."""
+    from paper_2303_11257_b200 import lib as L
+    X, G, w, _ = _inputs(10, rows, cols, "bf16")
+    bad = [5, rows // 2, rows - 1]
+    for r, v in zip(bad, (np.nan, np.inf, -np.inf)):
+        X[r, cols // 3] = v
+    X[7] = np.float32(2.0 ** 70) * np.where(np.arange(cols) % 3, 1, -1)
+    dX, dw, dc = U.empty(rows, cols, "f32"), torch.empty(cols, device="cuda"), torch.empty(cols, device="cuda")
+    ws = torch.empty(max(L.us_layer_norm_bwd_workspace_bytes(rows, cols), 16), dtype=torch.uint8, device="cuda")
+    Xt = torch.from_numpy(X).cuda().bfloat16()
+    L.us_layer_norm_bwd(Xt, torch.from_numpy(w[0]).cuda(), U.to_device(G, g_fmt), 1e-5, 1.0, 1.0, dX, dw, dc, ws)
+    got, good = dX.cpu().numpy(), np.setdiff1d(np.arange(rows), bad + [7])
+    assert np.isnan(got[bad]).all() and not got[7].any()
+    ref = O.layer_norm_bwd(X[good], w, G[good], np.float32(1e-5), 1.0, 1.0)[0]
+    assert np.abs(got[good] - ref).max() <= 3e-5 * max(1.0, 1.0 / np.sqrt(X[good].var(axis=1).min() + 1e-5))
