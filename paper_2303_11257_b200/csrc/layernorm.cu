@@ -11,6 +11,8 @@
 // the rows its warp walks, combines the warps of a CTA in a fixed order and writes one partial row
 // per CTA to the caller's workspace; a second kernel adds the CTAs' partials in a fixed order and
 // applies beta.  No atomics: results do not depend on scheduling.
+#include <algorithm>
+
 #include "common.cuh"
 #include "host.h"
 #include "rowwise.cuh"
@@ -517,10 +519,10 @@ __device__ __forceinline__ float warp_sum4(const float (&v)[4], int lane) {
 // type of X.  XBF: X (and a 16-bit gradient) are BF16 rather than F16.  Bound: latency of the exchanges, 16 warps an SM; beyond L2
 // memory.  us, a warp per row -> this, BF16 with an FP8 copy: 8192 x 1024 22.8 -> 17.9, its float32 gradient 25.6 -> 18.9, 2048 x 768 12.0 -> 7.8, 4096 x
 // 256 8.7 -> 5.6, 256 x 1024 8.9 -> 5.8; 2048 x 2048, which the general kernel took, 65 -> 13.
-constexpr int kLnBatch = 4, kLnRowsPerSm = 2;
+constexpr int kLnBatch = 4, kLnCtasPerSm = 2;
 enum LnOut { kLnSame = 0, kLnSameE4 = 1, kLnSameE5 = 2, kLnAny = 3, kLnAnyCopy = 4 };   // dX of X's type (and its FP8 copy), or of any type
 template <bool G32, bool XBF, int OUT>
-__global__ void __launch_bounds__(kLnThreads, kLnRowsPerSm) ln_bwd_rows_kernel(const LnArgs a, const int wpr) {
+__global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) ln_bwd_rows_kernel(const LnArgs a, const int wpr) {
   extern __shared__ __align__(16) float ln_smem[];             // exchanges [warps][1 + 3][4], then the combine [groups][2][cols]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int groups = nw / wpr, group = warp / wpr, col = ((warp - group * wpr) * 32 + lane) * 8;
@@ -742,16 +744,19 @@ static us_status check_vector(const us_mat* v, int64_t cols, bool input) {
   return US_OK;
 }
 
-// CTAs of the backward kernel: `warps` rows in flight per CTA, at most `per_sm` CTAs per SM.
-static int ln_bwd_grid(int64_t rows, int warps = kLnWarps, int per_sm = 2) {
+// CTAs of a backward kernel: `rows_each` rows in flight per CTA, at most `per_sm` CTAs per SM.
+static int ln_bwd_grid(int64_t rows, int rows_each = kLnWarps, int per_sm = 2) {
   const int sms = host::sm_count();
   if (sms <= 0) return 0;
-  const int64_t want = (rows + warps - 1) / warps;
+  const int64_t want = (rows + rows_each - 1) / rows_each;
   const int64_t cap = (int64_t)sms * per_sm;
   return (int)(want < cap ? want : cap);
 }
 
 constexpr int kLnFastWarps = 4, kLnFastPerSm = 3;   // of ln_bwd16_kernel
+// Rows of partial sums that a workspace holds, whichever kernel the call takes: a CTA writes one.
+static int ln_bwd_partials(int64_t rows) { return std::max(ln_bwd_grid(rows), ln_bwd_grid(rows, kLnFastWarps, kLnFastPerSm)); }
+
 template <bool COPY>
 static us_status ln_fwd_launch(const LnArgs& a, cudaStream_t st) {
   const int64_t grid64 = (a.rows + kLnWarps - 1) / kLnWarps;
@@ -818,9 +823,10 @@ static us_status ln_bwd_launch(const LnArgs& a, int grid, float beta_wc, const u
   } else if (rows16 && nch <= kLnWarps && (a.g_dt == a.x_dt || a.g_dt == US_F32)) {
     const int groups = kLnWarps / nch;
     // rows per group: four, fewer where that would be few CTAs (1000 x 384 5.4 / 5.4 / 6.2 us with 4 / 2 / 1, 256 x 1024 6.2 / 5.8 / 6.0, 300 x 128 4.8 /
-    // 4.6 / 4.4; 4096 x 256 5.6 / 6.2 / 6.6: each CTA is a partial row that the second kernel adds)
+    // 4.6 / 4.4; 4096 x 256 5.6 / 6.2 / 6.6: each CTA is a partial row that the second kernel adds), and never more CTAs than the workspace has
+    // partial rows (which binds few long rows: 16 x 2048 6.3 us with a CTA a row, 6.7 with one for four)
     const int64_t turns = (a.rows + kLnBatch * groups - 1) / (kLnBatch * groups);
-    nparts = ln_bwd_grid(a.rows > 0 ? a.rows : 1, (turns >= 64 ? 4 : turns >= 16 ? 2 : 1) * groups, kLnRowsPerSm);
+    nparts = std::min(ln_bwd_grid(a.rows > 0 ? a.rows : 1, (turns >= 64 ? 4 : turns >= 16 ? 2 : 1) * groups, kLnCtasPerSm), ln_bwd_partials(a.rows > 0 ? a.rows : 1));
     const size_t smem = ((size_t)16 * nch * groups + (size_t)2 * groups * a.cols) * sizeof(float);
     const bool g32 = a.g_dt == US_F32, xbf = a.x_dt == US_BF16;
     const int out = a.out_dt != a.x_dt ? (COPY ? kLnAnyCopy : kLnAny) : !COPY ? kLnSame : a.q_dt == US_E5M2 ? kLnSameE5 : kLnSameE4;
@@ -893,8 +899,7 @@ using namespace us;
 
 extern "C" size_t us_layer_norm_bwd_workspace_bytes(int64_t rows, int64_t cols) {
   if (rows <= 0 || cols <= 0) return 0;
-  const int g0 = ln_bwd_grid(rows), g1 = ln_bwd_grid(rows, 1, 3);
-  const int grid = g0 > g1 ? g0 : g1;                // whichever kernel the call takes
+  const int grid = ln_bwd_partials(rows);
   return (size_t)(grid > 0 ? grid : 1) * 2 * (size_t)cols * sizeof(float);
 }
 

@@ -184,3 +184,26 @@ def test_layer_norm_backward_of_rows_that_are_not_finite(rows, cols, g_fmt):
     assert np.isnan(got[bad]).all() and not got[7].any()
     ref = O.layer_norm_bwd(X[good], w, G[good], np.float32(1e-5), 1.0, 1.0)[0]
     assert np.abs(got[good] - ref).max() <= 3e-5 * max(1.0, 1.0 / np.sqrt(X[good].var(axis=1).min() + 1e-5))
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 2048), (60, 2048), (300, 128), (200, 1288), (1000, 768), (5000, 136)])
+def test_layer_norm_backward_workspace_of_one_partial_row_per_eight_or_four_rows(rows, cols):
+    """The workspace is a row of 2 x cols partial sums per CTA of the widest grid: rows / 8 up to two per SM, or rows / 4 up to three.  A
+    buffer of that size is enough and nothing is written beyond it; a smaller one is refused."""
+    L = _lib()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    need = 8 * cols * max(min(-(-rows // 8), 2 * sms), min(-(-rows // 4), 3 * sms))
+    assert L.us_layer_norm_bwd_workspace_bytes(rows, cols) == need
+    X, G, w, _ = _inputs(9, rows, cols, "bf16")
+    dX, dw, dc = U.empty(rows, cols, "f32"), torch.empty(cols, device="cuda"), torch.empty(cols, device="cuda")
+    buf = torch.full((need + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    args = (U.to_device(X, "bf16"), torch.from_numpy(w[0]).cuda(), U.to_device(G, "bf16"), 1e-5, 1.0, 1.0, dX, dw, dc)
+    L.us_layer_norm_bwd(*args, buf[:need])
+    rdX, rdw, rdc = O.layer_norm_bwd(X, w, G, np.float32(1e-5), 1.0, 1.0)
+    assert (buf[need:] == 0xA5).all()
+    assert np.abs(U.host_values(dX) - rdX).max() <= 3e-5 * max(1.0, 1.0 / np.sqrt(X.var(axis=1).min() + 1e-5))
+    tol = 8 * (2e-6 * np.sqrt(rows) + 1e-6) * np.sqrt(rows)
+    assert np.abs(dw.cpu().numpy() - rdw.reshape(-1)).max() <= tol and np.abs(dc.cpu().numpy() - rdc.reshape(-1)).max() <= tol
+    with pytest.raises(L.UnitScaleError) as e:
+        L.us_layer_norm_bwd(*args, buf[:need - 16])
+    assert e.value.status == L.US_ERR_WORKSPACE
