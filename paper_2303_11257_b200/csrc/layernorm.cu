@@ -808,10 +808,13 @@ static us_status ln_bwd_launch(const LnArgs& a, int grid, float beta_wc, const u
   int nparts = grid;
   // With no rows the first kernel still runs (one CTA) and writes zero partials, so dw = dc = 0.
   const bool rows16 = a.vec_ok && (a.x_dt == US_BF16 || a.x_dt == US_F16);
-  // Beyond 16 M elements (X and G no longer stay in L2) a warp per row with a ring of bulk copies keeps more of memory busy.  us, rows among
-  // warps / warp per row, BF16: 16384 x 1024 30.9 / 30.6, 24576 x 1024 46.4 / 40.9, 32768 x 768 53.2 / 42.1, 65536 x 512 56.5 / 53.4; a float32 gradient
+  // Large 16-bit cases (X and G no longer stay in L2), a warp per row with a ring of bulk copies, which keeps more of memory busy: from 16 M
+  // elements on, with 513 to 1024 columns, whose CTAs hold two rows, from 14 M, up to 768 of them, six warps, from 7.5 M.  us, rows among warps / warp per
+  // row, BF16: 10000 x 640 18.0 / 18.0, 12288 x 640 20.5 / 19.9, 14000 x 768 21.7 / 22.1, 20000 x 768 34.0 / 30.4, 26000 x 640 41.3 / 34.7; 14000 x 1024
+  // 27.5 / 28.5, 16384 x 896 29.0 / 28.1, 16384 x 1024 32.1 / 31.0; 26000 x 512 24.1 / 25.8, 65536 x 512 56.5 / 53.4; a float32 gradient
   // 32768 x 1024 66 / 89, rows of at most 256 131072 x 256 48 / 75.
-  if (rows16 && a.g_dt == a.x_dt && nch > 1 && nch <= 4 && a.rows * a.cols > (16 << 20)) {
+  const int64_t ring_from = nch == 2 ? 32 : nch == 3 ? 15 : 28;          // in half millions of elements
+  if (rows16 && a.g_dt == a.x_dt && nch > 1 && nch <= 4 && a.rows * a.cols >= ring_from << 19) {
     nparts = ln_bwd_grid(a.rows, kLnFastWarps, kLnFastPerSm);
     const size_t smem = ((size_t)(nch <= 2 ? 2 : 4) * 256 + (size_t)kLnFastWarps * a.cols) * sizeof(float) + (size_t)kLnFastWarps * kLnStages * (a.cols * 4 + 8);
     const bool xbf = a.x_dt == US_BF16;

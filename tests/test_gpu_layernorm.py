@@ -207,3 +207,29 @@ def test_layer_norm_backward_workspace_of_one_partial_row_per_eight_or_four_rows
     with pytest.raises(L.UnitScaleError) as e:
         L.us_layer_norm_bwd(*args, buf[:need - 16])
     assert e.value.status == L.US_ERR_WORKSPACE
+
+
+@pytest.mark.parametrize("rows,cols,q_fmt", [(16400, 1024, None), (16384, 896, "e4m3"), (12289, 640, "e5m2"), (33000, 512, None), (12000, 640, "e5m2")])
+def test_layer_norm_backward_beyond_what_l2_holds(rows, cols, q_fmt):
+    """The warp-per-row kernel with its ring of bulk copies, several rows a slot, and its FP8 copy (the last shape is on the other side of
+    the line): all of dX, dw and dc against float64."""
+    from paper_2303_11257_b200 import lib as L
+    torch.manual_seed(rows)
+    X, G = (torch.randn(rows, cols, device="cuda") * 1.5 + 0.5).bfloat16(), torch.randn(rows, cols, device="cuda").bfloat16()
+    w = 1 + 0.25 * torch.randn(1, cols, device="cuda")
+    dX, q = torch.empty_like(X), U.empty(rows, cols, q_fmt) if q_fmt else None
+    dw, dc = torch.empty(1, cols, device="cuda"), torch.empty(1, cols, device="cuda")
+    ws = torch.empty(L.us_layer_norm_bwd_workspace_bytes(rows, cols), dtype=torch.uint8, device="cuda")
+    name, bw = ("us_layer_norm_bwd_cast" if q_fmt else "us_layer_norm_bwd"), rows ** -0.5
+    m = [L.mat(t) for t in (X, w, G, dX)]
+    L.Call(name, *m[:3], 1e-5, 1.0, bw, m[3], *([L.mat(q)] if q_fmt else []), L.mat(dw), L.mat(dc), ws.data_ptr(), ws.numel())(L.current_stream())
+    x, g, u = X.double(), G.double(), G.double() * w.double()
+    d = x - x.mean(1, keepdim=True)
+    r = (d.square().mean(1, keepdim=True) + 1e-5).rsqrt()
+    ref = r * (u - u.mean(1, keepdim=True) - d * r * (u * d * r).mean(1, keepdim=True))
+    assert ((dX.double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 3e-5).all()             # half a BF16 step, rounded up, and float32 sums
+    tol = 8 * (2e-6 * rows ** 0.5 + 1e-6)
+    assert (dw.double() - bw * (g * d * r).sum(0)).abs().max() <= tol and (dc.double() - bw * g.sum(0)).abs().max() <= tol
+    if q_fmt:
+        most = 448 if q_fmt == "e4m3" else 57344
+        assert torch.equal(q.view(torch.uint8), dX.float().clamp(-most, most).to(U.TORCH_OF[q_fmt]).view(torch.uint8))
