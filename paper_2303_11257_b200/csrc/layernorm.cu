@@ -512,16 +512,21 @@ __device__ __forceinline__ float warp_sum4(const float (&v)[4], int lane) {
   return x;
 }
 
+// The same for the B rows of a turn, four or one.
+__device__ __forceinline__ float sum_rows(const float (&v)[4], int lane) { return warp_sum4(v, lane); }
+__device__ __forceinline__ float sum_rows(const float (&v)[1], int) { return warp_sum(v[0]); }
+
 // The 16-bit cases of the backward pass (rows of at most 2048 elements): a row belongs to wpr = cols / 256 warps, eight columns a lane, so
 // that a lane's share of the column sums is 16 registers and three CTAs of eight warps fit an SM; the warps of a row take four rows at
 // a time, which hides the latency of their loads and shares two exchanges through shared memory among four rows: the means, then the
-// sums of (x - mu)^2, g w and g w (x - mu).  G32: the gradient is float32 (the gradient of a layer's output often is) instead of the 16-bit
+// sums of (x - mu)^2, g w and g w (x - mu).  B: rows of a turn, four, or one where each group has but one row (300 x 128 4.4 -> 3.9 us, 100 x 512
+// 5.3 -> 4.6: less code to fetch).  G32: the gradient is float32 (the gradient of a layer's output often is) instead of the 16-bit
 // type of X.  XBF: X (and a 16-bit gradient) are BF16 rather than F16.  Bound: latency of the exchanges, 16 warps an SM; beyond L2
 // memory.  us, a warp per row -> this, BF16 with an FP8 copy: 8192 x 1024 22.8 -> 17.9, its float32 gradient 25.6 -> 18.9, 2048 x 768 12.0 -> 7.8, 4096 x
 // 256 8.7 -> 5.6, 256 x 1024 8.9 -> 5.8; 2048 x 2048, which the general kernel took, 65 -> 13.
 constexpr int kLnBatch = 4, kLnCtasPerSm = 2;
 enum LnOut { kLnSame = 0, kLnSameE4 = 1, kLnSameE5 = 2, kLnAny = 3, kLnAnyCopy = 4 };   // dX of X's type (and its FP8 copy), or of any type
-template <bool G32, bool XBF, int OUT>
+template <bool G32, bool XBF, int OUT, int B>
 __global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) ln_bwd_rows_kernel(const LnArgs a, const int wpr) {
   extern __shared__ __align__(16) float ln_smem[];             // exchanges [warps][1 + 3][4], then the combine [groups][2][cols]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -547,12 +552,12 @@ __global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) ln_bwd_rows_kernel(c
   auto packed = [](uint4& r) { asm volatile("" : "+r"(r.x), "+r"(r.y), "+r"(r.z), "+r"(r.w)); };
   auto word = [](const uint4& r, int j) { return j == 0 ? r.x : j == 1 ? r.y : j == 2 ? r.z : r.w; };
   const int64_t stride = (int64_t)gridDim.x * groups;
-  for (int64_t row0 = (int64_t)blockIdx.x * groups + group + zero; row0 < a.rows; row0 += kLnBatch * stride) {
+  for (int64_t row0 = (int64_t)blockIdx.x * groups + group + zero; row0 < a.rows; row0 += B * stride) {
     const int64_t rest = (a.rows - row0 + stride - 1) / stride;
-    const int here = rest < kLnBatch ? (int)rest : kLnBatch;   // rows of this turn
-    uint4 cx[kLnBatch], cg[kLnBatch], ch[G32 ? kLnBatch : 1];  // packed rows; a float32 gradient takes two vectors
+    const int here = rest < B ? (int)rest : B;   // rows of this turn
+    uint4 cx[B], cg[B], ch[G32 ? B : 1];  // packed rows; a float32 gradient takes two vectors
 #pragma unroll
-    for (int b = 0; b < kLnBatch; ++b) {
+    for (int b = 0; b < B; ++b) {
       const int64_t row = row0 + b * stride;
       cx[b] = cg[b] = make_uint4(0, 0, 0, 0);
       if (G32) ch[G32 ? b : 0] = make_uint4(0, 0, 0, 0);
@@ -569,30 +574,34 @@ __global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) ln_bwd_rows_kernel(c
       return j & 1 ? pack2(__uint_as_float(r.z), __uint_as_float(r.w)) : pack2(__uint_as_float(r.x), __uint_as_float(r.y));
     };
     // ---- means
-    float v[kLnBatch], lo, hi;
+    float v[B], lo, hi;
 #pragma unroll
-    for (int b = 0; b < kLnBatch; ++b) {
+    for (int b = 0; b < B; ++b) {
       v[b] = 0.f;
       if (b >= here) continue;
       unpack2(add2(add2(unpack(cx[b].x), unpack(cx[b].y)), add2(unpack(cx[b].z), unpack(cx[b].w))), lo, hi);
       v[b] = lo + hi;
     }
-    const float m = warp_sum4(v, lane);
-    float mu[kLnBatch] = {0.f, 0.f, 0.f, 0.f};
+    const float m = sum_rows(v, lane);
+    float mu[B] = {};
     if (wpr == 1) {
 #pragma unroll
-      for (int b = 0; b < kLnBatch; ++b) mu[b] = __shfl_sync(0xffffffffu, m, b);
+      for (int b = 0; b < B; ++b) mu[b] = __shfl_sync(0xffffffffu, m, b);
     } else {
-      if (lane < 4) reinterpret_cast<float*>(&means[warp - group * wpr])[lane] = m;
+      if (lane < B) reinterpret_cast<float*>(&means[warp - group * wpr])[lane] = m;
       meet();
-      for (int k = 0; k < wpr; ++k) { const float4 t = means[k]; mu[0] += t.x; mu[1] += t.y; mu[2] += t.z; mu[3] += t.w; }
+      for (int k = 0; k < wpr; ++k) {
+        const float4 t = means[k];
+        mu[0] += t.x;
+        if constexpr (B == 4) { mu[1] += t.y; mu[2] += t.z; mu[3] += t.w; }
+      }
     }
 #pragma unroll
-    for (int b = 0; b < kLnBatch; ++b) packed(cx[b]);
+    for (int b = 0; b < B; ++b) packed(cx[b]);
     // ---- variance about the mean, sums of u = g w and of u (x - mu)
-    float q[kLnBatch], su[kLnBatch], sd[kLnBatch];
+    float q[B], su[B], sd[B];
 #pragma unroll
-    for (int b = 0; b < kLnBatch; ++b) {
+    for (int b = 0; b < B; ++b) {
       q[b] = su[b] = sd[b] = 0.f;
       if (b >= here) continue;
       mu[b] = mean(mu[b]);
@@ -607,30 +616,33 @@ __global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) ln_bwd_rows_kernel(c
       unpack2(u2, lo, hi); su[b] = lo + hi;                    // (zero beyond the row's end: g and w are)
       unpack2(d2, lo, hi); sd[b] = lo + hi;
     }
-    const float rq = warp_sum4(q, lane), ru = warp_sum4(su, lane), rd = warp_sum4(sd, lane);
+    const float rq = sum_rows(q, lane), ru = sum_rows(su, lane), rd = sum_rows(sd, lane);
     if (wpr == 1) {
 #pragma unroll
-      for (int b = 0; b < kLnBatch; ++b) { q[b] = __shfl_sync(0xffffffffu, rq, b); su[b] = __shfl_sync(0xffffffffu, ru, b); sd[b] = __shfl_sync(0xffffffffu, rd, b); }
+      for (int b = 0; b < B; ++b) { q[b] = __shfl_sync(0xffffffffu, rq, b); su[b] = __shfl_sync(0xffffffffu, ru, b); sd[b] = __shfl_sync(0xffffffffu, rd, b); }
     } else {
-      if (lane < 4) {
+      if (lane < B) {
         float* t = reinterpret_cast<float*>(&sums[3 * (warp - group * wpr)]) + lane;
         t[0] = rq; t[4] = ru; t[8] = rd;
       }
       meet();
 #pragma unroll
-      for (int b = 0; b < kLnBatch; ++b) q[b] = su[b] = sd[b] = 0.f;
+      for (int b = 0; b < B; ++b) q[b] = su[b] = sd[b] = 0.f;
       for (int k = 0; k < wpr; ++k) {
         const float4 t0 = sums[3 * k], t1 = sums[3 * k + 1], t2 = sums[3 * k + 2];
-        q[0] += t0.x; q[1] += t0.y; q[2] += t0.z; q[3] += t0.w;
-        su[0] += t1.x; su[1] += t1.y; su[2] += t1.z; su[3] += t1.w;
-        sd[0] += t2.x; sd[1] += t2.y; sd[2] += t2.z; sd[3] += t2.w;
+        q[0] += t0.x; su[0] += t1.x; sd[0] += t2.x;
+        if constexpr (B == 4) {
+          q[1] += t0.y; q[2] += t0.z; q[3] += t0.w;
+          su[1] += t1.y; su[2] += t1.z; su[3] += t1.w;
+          sd[1] += t2.y; sd[2] += t2.z; sd[3] += t2.w;
+        }
       }
     }
 #pragma unroll
-    for (int b = 0; b < kLnBatch; ++b) { packed(cx[b]); packed(cg[b]); }
+    for (int b = 0; b < B; ++b) { packed(cx[b]); packed(cg[b]); }
     // ---- dX = beta_x rstd (u - mean(u) - xhat mean(u xhat)), column sums
 #pragma unroll
-    for (int b = 0; b < kLnBatch; ++b) {
+    for (int b = 0; b < B; ++b) {
       const int64_t row = row0 + b * stride;
       if (b >= here) continue;
       const float rstd = rsqrtf(mean(q[b]) + a.eps), k = a.beta_x * rstd;
@@ -825,18 +837,20 @@ static us_status ln_bwd_launch(const LnArgs& a, int grid, float beta_wc, const u
     if (launched != US_OK) return launched;
   } else if (rows16 && nch <= kLnWarps && (a.g_dt == a.x_dt || a.g_dt == US_F32)) {
     const int groups = kLnWarps / nch;
-    // rows per group: four, fewer where that would be few CTAs (1000 x 384 5.4 / 5.4 / 6.2 us with 4 / 2 / 1, 256 x 1024 6.2 / 5.8 / 6.0, 300 x 128 4.8 /
-    // 4.6 / 4.4; 4096 x 256 5.6 / 6.2 / 6.6: each CTA is a partial row that the second kernel adds), and never more CTAs than the workspace has
-    // partial rows (which binds few long rows: 16 x 2048 6.3 us with a CTA a row, 6.7 with one for four)
+    // Rows per group: four, fewer where that would be few CTAs, each of which is a partial row that the second kernel adds (us with 4 / 2 / 1: 1000 x
+    // 384 5.4 / 5.4 / 6.2, 4096 x 256 5.6 / 6.2 / 6.6; with 2 / 1: 300 x 384 5.3 / 4.6, 600 x 256 4.8 / 4.2, 1200 x 256 4.9 / 5.1), and never more CTAs
+    // than the workspace has partial rows (which binds few long rows: 16 x 2048 6.3 us with a CTA a row, 6.7 with one for four).
     const int64_t turns = (a.rows + kLnBatch * groups - 1) / (kLnBatch * groups);
-    nparts = std::min(ln_bwd_grid(a.rows > 0 ? a.rows : 1, (turns >= 64 ? 4 : turns >= 16 ? 2 : 1) * groups, kLnCtasPerSm), ln_bwd_partials(a.rows > 0 ? a.rows : 1));
+    nparts = std::min(ln_bwd_grid(a.rows > 0 ? a.rows : 1, (turns >= 64 ? 4 : turns >= 32 ? 2 : 1) * groups, kLnCtasPerSm), ln_bwd_partials(a.rows > 0 ? a.rows : 1));
     const size_t smem = ((size_t)16 * nch * groups + (size_t)2 * groups * a.cols) * sizeof(float);
-    const bool g32 = a.g_dt == US_F32, xbf = a.x_dt == US_BF16;
+    const bool g32 = a.g_dt == US_F32, xbf = a.x_dt == US_BF16, one = (int64_t)nparts * groups >= a.rows;      // (a row for each group: no turns of four)
     const int out = a.out_dt != a.x_dt ? (COPY ? kLnAnyCopy : kLnAny) : !COPY ? kLnSame : a.q_dt == US_E5M2 ? kLnSameE5 : kLnSameE4;
     void (*fn)(const LnArgs, const int) = nullptr;
 #define US_LN_PICK(OUT)                                                                            \
-  fn = g32 ? (xbf ? ln_bwd_rows_kernel<true, true, OUT> : ln_bwd_rows_kernel<true, false, OUT>)    \
-           : (xbf ? ln_bwd_rows_kernel<false, true, OUT> : ln_bwd_rows_kernel<false, false, OUT>)
+  fn = one ? (g32 ? (xbf ? ln_bwd_rows_kernel<true, true, OUT, 1> : ln_bwd_rows_kernel<true, false, OUT, 1>)                       \
+                  : (xbf ? ln_bwd_rows_kernel<false, true, OUT, 1> : ln_bwd_rows_kernel<false, false, OUT, 1>))                    \
+           : (g32 ? (xbf ? ln_bwd_rows_kernel<true, true, OUT, kLnBatch> : ln_bwd_rows_kernel<true, false, OUT, kLnBatch>)         \
+                  : (xbf ? ln_bwd_rows_kernel<false, true, OUT, kLnBatch> : ln_bwd_rows_kernel<false, false, OUT, kLnBatch>))
     if constexpr (COPY) {
       if (out == kLnAnyCopy) US_LN_PICK(kLnAnyCopy);
       else if (out == kLnSameE5) US_LN_PICK(kLnSameE5);
