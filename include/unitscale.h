@@ -293,6 +293,15 @@ us_status us_linear_fwd_static_ws(const us_mat* X, const us_mat* W, float alpha,
  */
 us_status us_test_linear_fwd_starved(const us_mat* X, const us_mat* W, float alpha, const us_mat* Y, void* ws,
                                      size_t ws_bytes, unsigned int wait_limit, void* stream);
+/* The same with loads withheld from some CTAs only, and in the middle of their work: `cta` -1: from every CTA, else from that one
+ * of each cluster (0 .. 7; of a CTA pair the odd one, whose copies the even one waits for), once it has had those of `tiles` output
+ * tiles (0 .. 1024; a launch with shared contractions has one tile per CTA: 0).  us_test_linear_group_starved: for us_linear_group_any. */
+us_status us_test_linear_fwd_starved_cta(const us_mat* X, const us_mat* W, float alpha, const us_mat* Y, void* ws, size_t ws_bytes,
+                                         unsigned int wait_limit, int cta, int tiles, void* stream);
+us_status us_test_ffn_hidden_starved_cta(const us_mat* X, const us_mat* W1, const us_mat* G, const us_mat* W2, const us_mat* A, const us_mat* dH,
+                                         void* ws, size_t ws_bytes, unsigned int wait_limit, int cta, int tiles, void* stream);
+us_status us_test_linear_group_starved(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, unsigned int wait_limit, int cta,
+                                       int tiles, void* stream);
 
 /* Activations of the table "Table of unit scaling factors", section Activations. */
 typedef enum { US_FN_GELU = 0, US_FN_RELU = 1, US_FN_TANH = 2, US_FN_SIGMOID = 3 } us_fn;

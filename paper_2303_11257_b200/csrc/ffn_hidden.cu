@@ -66,7 +66,7 @@ struct HiddenParams {
   unsigned int* status;
   uint32_t wait_limit;
   uint32_t x_bytes; int stages;     // SPLIT > 1: bytes of X or G in a stage (the rows that exist), and the stages that fit
-  int no_loads;                     // test hook: no operand loads are issued, so that the waits run out
+  int starved, served;              // test hook (starved_cta)
 };
 
 // ES: operand bytes per element (1 = FP8, 2 = BF16 / F16).  BN, CG: tiles of 256 x 256 per CTA pair (256, 2), or of
@@ -151,7 +151,8 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       uint32_t issued = 0;
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
-      for (int tile = pair; ok && !p.no_loads && tile < num_tiles; tile += num_pairs) {
+      const int end = starved_cta(p.starved, rank) ? min(num_tiles, pair + p.served * num_pairs) : num_tiles;
+      for (int tile = pair; ok && tile < end; tile += num_pairs) {
         int tm, tn;
         tile_mn2(tile, tm, tn);
         const int m0 = tm * kTileM + rank * 128, n0 = tn * BN + rank * 128 + (split_col - split_acc);
@@ -419,7 +420,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (CG == 2) ptx::cluster_meet();
+  if (CG == 2) ptx::cluster_part(*abort_flag != 0);
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     if (CG == 2) ptx::tmem_dealloc_pair(tmem_base, kTmemCols); else ptx::tmem_dealloc(tmem_base, kTmemCols);
@@ -473,7 +474,7 @@ us_status pick_hidden(bool pair, int split, bool h_bf16, const CUtensorMap* t, c
 us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_mat* G, const us_mat* W2, float beta_x,
                       float act_in_scale, float act_out_scale, float grad_out_scale, int h_dtype, const us_mat* H,
                       const us_mat* A, const us_mat* dH, void* ws, size_t ws_bytes, void* stream, uint32_t wait_limit,
-                      int no_loads, bool any) {
+                      int starved, int served, bool any) {
   if (!valid_mat(X) || !valid_mat(W1) || !valid_mat(G) || !valid_mat(W2) || !valid_mat(A) || !valid_mat(dH)) return US_ERR_INVALID_ARG;
   const bool keep_h = H && H->ptr;
   if (keep_h && !valid_mat(H)) return US_ERR_INVALID_ARG;
@@ -525,7 +526,7 @@ us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_m
   p.d_ptr = static_cast<uint8_t*>(dH->ptr); p.d_ld = dH->ld;
   p.status = static_cast<unsigned int*>(ws);
   p.wait_limit = wait_limit;
-  p.no_loads = no_loads;
+  p.starved = starved; p.served = served;
 
   CUtensorMap t[6];
   const int out_box = tile / 4 * es;                             // bytes per row of an epilogue warp's output box
@@ -554,7 +555,7 @@ extern "C" us_status us_ffn_hidden(const us_mat* X, const us_mat* W1, float alph
                                    int32_t h_dtype, const us_mat* H, const us_mat* A, const us_mat* dH, void* ws,
                                    size_t ws_bytes, void* stream) {
   return us::hidden_impl(X, W1, alpha, G, W2, beta_x, act_in_scale, act_out_scale, grad_out_scale, h_dtype, H, A, dH, ws,
-                         ws_bytes, stream, us::kWaitLimit, 0, false);
+                         ws_bytes, stream, us::kWaitLimit, 0, 0, false);
 }
 
 extern "C" us_status us_ffn_hidden_any(const us_mat* X, const us_mat* W1, float alpha, const us_mat* G, const us_mat* W2,
@@ -562,12 +563,17 @@ extern "C" us_status us_ffn_hidden_any(const us_mat* X, const us_mat* W1, float 
                                        int32_t h_dtype, const us_mat* H, const us_mat* A, const us_mat* dH, void* ws,
                                        size_t ws_bytes, void* stream) {
   return us::hidden_impl(X, W1, alpha, G, W2, beta_x, act_in_scale, act_out_scale, grad_out_scale, h_dtype, H, A, dH, ws,
-                         ws_bytes, stream, us::kWaitLimit, 0, true);
+                         ws_bytes, stream, us::kWaitLimit, 0, 0, true);
 }
 
 extern "C" us_status us_test_ffn_hidden_starved(const us_mat* X, const us_mat* W1, const us_mat* G, const us_mat* W2,
                                                 const us_mat* A, const us_mat* dH, void* ws, size_t ws_bytes,
                                                 uint32_t wait_limit, void* stream) {
   if (wait_limit == 0 || wait_limit > (1u << 16)) return US_ERR_INVALID_ARG;
-  return us::hidden_impl(X, W1, 1.f, G, W2, 1.f, 1.f, 1.f, 1.f, US_BF16, nullptr, A, dH, ws, ws_bytes, stream, wait_limit, 1, false);
+  return us::hidden_impl(X, W1, 1.f, G, W2, 1.f, 1.f, 1.f, 1.f, US_BF16, nullptr, A, dH, ws, ws_bytes, stream, wait_limit, 1, 0, false);
+}
+extern "C" us_status us_test_ffn_hidden_starved_cta(const us_mat* X, const us_mat* W1, const us_mat* G, const us_mat* W2, const us_mat* A, const us_mat* dH,
+                                                    void* ws, size_t ws_bytes, uint32_t wait_limit, int cta, int tiles, void* stream) {
+  if (wait_limit == 0 || wait_limit > (1u << 16) || cta < -1 || cta > 1 || tiles < 0 || tiles > 1024) return US_ERR_INVALID_ARG;
+  return us::hidden_impl(X, W1, 1.f, G, W2, 1.f, 1.f, 1.f, 1.f, US_BF16, nullptr, A, dH, ws, ws_bytes, stream, wait_limit, cta + 2, tiles, false);
 }

@@ -26,10 +26,10 @@ us_status check_copy(const us_mat* q, const us_mat* out, bool residual) {
   return aligned16(q) ? US_OK : US_ERR_ALIGNMENT;
 }
 
-// Failure-path test settings of one call: a short wait limit, and a producer that issues no loads.
+// Failure-path test settings of one call: a short wait limit, and which CTAs get no operands (starved_cta).
 struct WaitTest {
   uint32_t wait_limit;
-  int no_loads;
+  int starved, served;
 };
 
 // A, B: the two operands in call order; out [M x N].
@@ -56,7 +56,8 @@ static us_status linear(Op op, const us_mat* A, const us_mat* B, float scale, co
   p.out = out->ptr; p.out_dt = out->dtype; p.out_ld = out->ld;
   p.out_coef = 1.f;
   p.wait_limit = wt ? wt->wait_limit : kWaitLimit;
-  p.no_loads = wt ? wt->no_loads : 0;
+  p.starved = wt ? wt->starved : 0;
+  p.served = wt ? wt->served : 0;
   if (ep) {
     if (ep->act < US_ACT_NONE || ep->act > US_ACT_SIGMOID_GRAD) return US_ERR_INVALID_ARG;
     // the activation's class (forward: value from the accumulator; gradient: slope from the stored pre-activation)
@@ -182,7 +183,13 @@ extern "C" us_status us_linear_fwd_check(const us_mat* X, const us_mat* W, const
 extern "C" us_status us_test_linear_fwd_starved(const us_mat* X, const us_mat* W, float alpha, const us_mat* Y, void* ws,
                                                 size_t ws_bytes, unsigned int wait_limit, void* stream) {
   if (wait_limit < 1 || wait_limit > (1u << 16)) return US_ERR_INVALID_ARG;
-  const us::WaitTest wt = {wait_limit, 1};
+  const us::WaitTest wt = {wait_limit, 1, 0};
+  return us::linear(us::kFwd, X, W, alpha, nullptr, Y, ws, ws_bytes, stream, nullptr, &wt);
+}
+extern "C" us_status us_test_linear_fwd_starved_cta(const us_mat* X, const us_mat* W, float alpha, const us_mat* Y, void* ws, size_t ws_bytes,
+                                                    unsigned int wait_limit, int cta, int tiles, void* stream) {
+  if (wait_limit < 1 || wait_limit > (1u << 16) || cta < -1 || cta > 7 || tiles < 0 || tiles > 1024) return US_ERR_INVALID_ARG;
+  const us::WaitTest wt = {wait_limit, cta + 2, tiles};
   return us::linear(us::kFwd, X, W, alpha, nullptr, Y, ws, ws_bytes, stream, nullptr, &wt);
 }
 

@@ -188,7 +188,10 @@ us_status launch_group(const GroupParams& g, bool copy, cudaStream_t stream) {
 }
 
 // copies: NULL, or for each call the FP8 copy of its output (ptr NULL: none).
-us_status group_impl(int count, const us_linear_call* calls, const us_mat* copies, bool any, void* ws, size_t ws_bytes, void* stream) {
+// test: NULL, or a short wait limit and which CTAs get no operands.
+struct GroupTest { uint32_t wait_limit; int starved, served; };
+us_status group_impl(int count, const us_linear_call* calls, const us_mat* copies, bool any, void* ws, size_t ws_bytes, void* stream,
+                     const GroupTest* test = nullptr) {
   if (count < 1 || count > kGroupMaxProblems || !calls) return count >= 1 && calls ? US_ERR_UNSUPPORTED : US_ERR_INVALID_ARG;
   if (!ws || ws_bytes < us_workspace_bytes()) return US_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(ws) % 16) return US_ERR_ALIGNMENT;
@@ -207,6 +210,8 @@ us_status group_impl(int count, const us_linear_call* calls, const us_mat* copie
   if (sms <= 0) return US_ERR_CUDA;
   const int es = dtype_size(calls[0].a.dtype);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const GroupTest tt = test ? *test : GroupTest{kWaitLimit, 0, 0};
+  const int starved = tt.served ? 0 : tt.starved;         // of a launch in which a CTA has one tile
   Tiling t{};
   const unsigned shared = any ? shared_calls(calls, sh, count, es, sms, &t) : 0;
   SplitCall split_calls[kGroupMaxProblems];
@@ -226,7 +231,7 @@ us_status group_impl(int count, const us_linear_call* calls, const us_mat* copie
     copy = copy || q;
     pair_tiles += ((sh[i].M + 255) / 256) * ((sh[i].N + 255) / 256);
   }
-  if (left == 0) return launch_split(splits, split_calls, t, static_cast<unsigned int*>(ws), kWaitLimit, 0, st);
+  if (left == 0) return launch_split(splits, split_calls, t, static_cast<unsigned int*>(ws), tt.wait_limit, starved, st);
   const bool pair = pair_tiles_pay(pair_tiles, sms);
   const int tile_m = pair ? 256 : 128, bn = pair ? 256 : 128;
   int64_t tiles = 0;
@@ -262,9 +267,9 @@ us_status group_impl(int count, const us_linear_call* calls, const us_mat* copie
   }
   if (!deal(g, es, tile_m, bn, split, units, any ? kGroupMaxItems : 12)) return US_ERR_UNSUPPORTED;      // too many tiles per unit for the work list
   g.status = static_cast<unsigned int*>(ws);
-  g.wait_limit = kWaitLimit;
+  g.wait_limit = tt.wait_limit; g.starved = tt.starved; g.served = tt.served;
   if (splits) {                                            // (a grouped launch that is refused has launched nothing)
-    const us_status s = launch_split(splits, split_calls, t, static_cast<unsigned int*>(ws), kWaitLimit, 0, st);
+    const us_status s = launch_split(splits, split_calls, t, static_cast<unsigned int*>(ws), tt.wait_limit, starved, st);
     if (s != US_OK) return s;
   }
   if (es == 1) return pair ? launch_group<1, 256, 2, 1>(g, copy, st) : split == 2 ? launch_group<1, 128, 1, 2>(g, copy, st) : launch_group<1, 128, 1, 1>(g, copy, st);
@@ -282,4 +287,10 @@ extern "C" us_status us_linear_group_any(int count, const us_linear_call* calls,
 }
 extern "C" us_status us_linear_group_cast(int count, const us_linear_call* calls, const us_mat* copies, void* ws, size_t ws_bytes, void* stream) {
   return copies ? us::group_impl(count, calls, copies, true, ws, ws_bytes, stream) : US_ERR_INVALID_ARG;
+}
+extern "C" us_status us_test_linear_group_starved(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, unsigned int wait_limit, int cta, int tiles,
+                                                  void* stream) {
+  if (wait_limit < 1 || wait_limit > (1u << 16) || cta < -1 || cta > 7 || tiles < 0 || tiles > 1024) return US_ERR_INVALID_ARG;
+  const us::GroupTest test = {wait_limit, cta + 2, tiles};
+  return us::group_impl(count, calls, nullptr, true, ws, ws_bytes, stream, &test);
 }

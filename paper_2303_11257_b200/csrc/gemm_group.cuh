@@ -52,6 +52,7 @@ struct GroupParams {
   int count, rounds, units;             // units: CTA pairs, or CTAs with single-CTA tiles
   unsigned int* status;
   uint32_t wait_limit;
+  int starved, served;                  // test hook (starved_cta)
   // work list: entry [round * units + unit] = problem << 28 | tile row << 14 | tile column, or -1
   int32_t table[kGroupMaxItems];
 };
@@ -126,7 +127,8 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
       uint32_t issued = 0;
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
-      for (int r = 0; ok && r < g.rounds; ++r) {
+      const int end = starved_cta(g.starved, rank) ? min(g.rounds, g.served) : g.rounds;
+      for (int r = 0; ok && r < end; ++r) {
         const int32_t e = entry(r);
         if (e < 0) continue;
         int pi, tm, tn;
@@ -362,7 +364,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams g) {
 
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (CG == 2) ptx::cluster_meet();
+  if (CG == 2) ptx::cluster_part(*abort_flag != 0);
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     if (CG == 2) ptx::tmem_dealloc_pair(tmem_base, kTmemCols); else ptx::tmem_dealloc(tmem_base, kTmemCols);

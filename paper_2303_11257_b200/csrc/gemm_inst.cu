@@ -173,7 +173,7 @@ us_status launch_gemm(const us_mat* A, const us_mat* B, GemmParams& p, const Epi
   const int bn = t.bn, cg = t.cg;
   if (t.splits > 1) {
     const SplitCall call{A, B, em.out, em.skip, em.copy, A_MN, B_MN, p.scale, p.skip_coef, p.out_coef};
-    return launch_split(1, &call, t, p.status, p.wait_limit, p.no_loads, stream);
+    return launch_split(1, &call, t, p.status, p.wait_limit, p.served ? 0 : p.starved, stream);
   }
   p.tiles_m = (p.M + kBM * cg - 1) / (kBM * cg);
   p.tiles_n = (p.N + bn - 1) / bn;

@@ -48,7 +48,7 @@ struct GemmParams {
   const void* skip; int skip_dt; int64_t skip_ld; float skip_coef, out_coef;
   unsigned int* status;
   uint32_t wait_limit;                      // polls a bounded wait makes before it gives up (kWaitLimit unless a test shortens it)
-  int no_loads;                             // test hook: the producer issues no operand loads, so that the waits run out
+  int starved, served;                      // test hook (starved_cta)
   uint32_t a_bytes, stages;                 // narrow tiles (BN = 64): bytes of A in a stage, and the stages that fit
 };
 
@@ -127,6 +127,10 @@ __device__ __forceinline__ void with_layout(bool a_mn, bool b_mn, F f) {
   else if (b_mn) f(std::false_type(), std::true_type());
   else f(std::false_type(), std::false_type());
 }
+
+// Test hook: whether CTA `cta` of a cluster gets no operands after its first `served` tiles, so that the waits run out (0: none, 1: every
+// one, r + 2: CTA r).
+__device__ __forceinline__ bool starved_cta(int starved, int cta) { return starved == 1 || starved == cta + 2; }
 
 // Bounded mbarrier wait.  Returns false if the CTA is aborting (this wait or another one timed out).
 // (Each attempt already suspends the thread in hardware for a while, so polling costs few issue
@@ -854,7 +858,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
       uint32_t issued = 0;
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
-      for (int tile = group; ok && !p.no_loads && tile < num_tiles; tile += num_groups) {
+      const int end = starved_cta(p.starved, rank) ? min(num_tiles, group + p.served * num_groups) : num_tiles;
+      for (int tile = group; ok && tile < end; tile += num_groups) {
         const int m0 = tile_m(p, tile) * (kBM * CG) + rank * kBM;
         const int n0 = tile_n(p, tile) * BN + rank * kBRows;
         int b0 = 0, b1 = 0;
@@ -1027,7 +1032,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
 
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (CG == 2) ptx::cluster_meet();                  // no CTA leaves while its partner may still signal it
+  if (CG == 2) ptx::cluster_part(*abort_flag != 0);    // no CTA leaves while its partner may still signal it
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     if (CG == 2) ptx::tmem_dealloc_pair(tmem_base, kTmemCols); else ptx::tmem_dealloc(tmem_base, kTmemCols);

@@ -38,7 +38,7 @@ struct SplitCall {
   float scale, skip_coef, out_coef;
 };
 // Tiles of the calls' outputs all t; t.splits is 2, 4 or 8 and t.splits * t.cg at most 8.
-us_status launch_split(int count, const SplitCall* calls, const Tiling& t, unsigned int* status, uint32_t wait_limit, int no_loads, cudaStream_t stream);
+us_status launch_split(int count, const SplitCall* calls, const Tiling& t, unsigned int* status, uint32_t wait_limit, int starved, cudaStream_t stream);
 int split_a_bytes(int bn, bool a_mn, int64_t rows);
 // Estimated time, us, of a launch of `tiles` tiles of kb K blocks.  sectors: the operands' rows start on 32-byte boundaries.
 double tiling_time(const Tiling& t, long long tiles, int kb, int a_bytes, bool sectors, int sms);

@@ -35,9 +35,9 @@ int capacity(int splits) {
   return host::resident_clusters(reinterpret_cast<const void*>(gemm_split_kernel<ES, BN, CG, false>), gemm_threads(8), GemmSmem<BN, CG, 8>::kTotal, CG * splits, count);
 }
 template <int PROBLEMS>
-us_status launch_problems(int count, const SplitCall* calls, const Tiling& t, unsigned int* status, uint32_t wait_limit, int no_loads, cudaStream_t stream) {
+us_status launch_problems(int count, const SplitCall* calls, const Tiling& t, unsigned int* status, uint32_t wait_limit, int starved, cudaStream_t stream) {
   SplitParams<PROBLEMS> p;
-  p.splits = t.splits; p.status = status; p.wait_limit = wait_limit; p.no_loads = no_loads;
+  p.splits = t.splits; p.status = status; p.wait_limit = wait_limit; p.starved = starved;
   const int es = dtype_size(calls[0].a->dtype), one = es == 1 ? US_E5M2 : US_BF16;      // the format the descriptor numbers 1
   int tiles = 0;
   for (int i = 0; i < count; ++i) {
@@ -97,9 +97,9 @@ int split_capacity(int es, const Tiling& t) {
   return t.bn == 64 ? capacity<2, 64, 1>(t.splits) : t.bn == 128 ? capacity<2, 128, 1>(t.splits) : capacity<2, 256, 2>(t.splits);
 }
 
-us_status launch_split(int count, const SplitCall* calls, const Tiling& t, unsigned int* status, uint32_t wait_limit, int no_loads, cudaStream_t stream) {
-  return count == 1 ? launch_problems<1>(count, calls, t, status, wait_limit, no_loads, stream)
-                    : launch_problems<kGroupMaxProblems>(count, calls, t, status, wait_limit, no_loads, stream);
+us_status launch_split(int count, const SplitCall* calls, const Tiling& t, unsigned int* status, uint32_t wait_limit, int starved, cudaStream_t stream) {
+  return count == 1 ? launch_problems<1>(count, calls, t, status, wait_limit, starved, stream)
+                    : launch_problems<kGroupMaxProblems>(count, calls, t, status, wait_limit, starved, stream);
 }
 
 }  // namespace us

@@ -25,7 +25,7 @@ struct SplitParams {
   int splits;                               // CTAs (pairs) per tile: 2, 4 or 8
   unsigned int* status;
   uint32_t wait_limit;
-  int no_loads;
+  int starved;                              // test hook (starved_cta)
 };
 
 // MULTI: several problems; the parameters of one alone are at fixed addresses and need not be fetched ahead.
@@ -124,7 +124,8 @@ gemm_split_kernel(const __grid_constant__ SplitParams<MULTI ? kGroupMaxProblems 
       ptx::grid_wait_previous();
       with_layout(a_mn, b_mn, [&](auto amn, auto bmn) {
         constexpr bool A_MN = decltype(amn)::value, B_MN = decltype(bmn)::value;
-        for (int kb = 0; ok && !p.no_loads && kb < num_kb; ++kb) {
+        const int end = starved_cta(p.starved, cluster_rank) ? 0 : num_kb;
+        for (int kb = 0; ok && kb < end; ++kb) {
           ok = wait_bounded(empty_bar(stage), phase ^ 1u, abort_flag, p.status, p.wait_limit);
           if (!ok) break;
           const uint32_t a_dst = smem_base + stage * stage_bytes, b_dst = a_dst + a_bytes;
@@ -297,7 +298,7 @@ gemm_split_kernel(const __grid_constant__ SplitParams<MULTI ? kGroupMaxProblems 
 
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (CG == 2) ptx::cluster_meet();
+  if (CG == 2) ptx::cluster_meet();                  // (nothing has been signalled since the barriers above)
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     if (CG == 2) ptx::tmem_dealloc_pair(tmem_base, BN); else ptx::tmem_dealloc(tmem_base, BN);

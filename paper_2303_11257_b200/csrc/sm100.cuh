@@ -205,6 +205,14 @@ __device__ __forceinline__ void cluster_meet() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 }
+// The end of a kernel: nobody leaves before all have arrived.  Where everything that the CTAs signal to one another has been waited for, as it
+// has when no wait ran out, nothing is left to be ordered.  A CTA that gave up (the same for all of its threads) may have signalled what
+// nobody waited for: it releases, so that this has landed when its partner, which acquires, leaves.
+__device__ __forceinline__ void cluster_part(bool gave_up) {
+  if (gave_up) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  else asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 // A shared-memory address of this CTA re-addressed to the same offset in the pair's even CTA.
 // (clusters here have exactly two CTAs, so the even CTA is rank 0)
 __device__ __forceinline__ uint32_t in_even_cta(uint32_t addr) {

@@ -117,6 +117,11 @@ def _load() -> C.CDLL:
     lib.us_ffn_hidden.restype = lib.us_ffn_hidden_any.restype = C.c_int
     lib.us_test_ffn_hidden_starved.argtypes = [MP, MP, MP, MP, MP, MP, V, SZ, C.c_uint, V]
     lib.us_test_ffn_hidden_starved.restype = C.c_int
+    lib.us_test_linear_fwd_starved_cta.argtypes = [MP, MP, F, MP, V, SZ, C.c_uint, C.c_int, C.c_int, V]
+    lib.us_test_ffn_hidden_starved_cta.argtypes = [MP] * 6 + [V, SZ, C.c_uint, C.c_int, C.c_int, V]
+    lib.us_test_linear_group_starved.argtypes = [C.c_int, C.POINTER(us_linear_call), V, SZ, C.c_uint, C.c_int, C.c_int, V]
+    for name in ("us_test_linear_fwd_starved_cta", "us_test_ffn_hidden_starved_cta", "us_test_linear_group_starved"):
+        getattr(lib, name).restype = C.c_int
     lib.us_workspace_bytes.argtypes = []
     lib.us_workspace_bytes.restype = SZ
     lib.us_workspace_status.argtypes = [V, V]
@@ -605,6 +610,24 @@ def us_test_ffn_hidden_starved(X, W1, G, W2, A, dH, ws, wait_limit: int, stream=
            _lib.us_test_ffn_hidden_starved(C.byref(mat(X)), C.byref(mat(W1)), C.byref(mat(G)), C.byref(mat(W2)),
                                            C.byref(mat(A)), C.byref(mat(dH)), ws.data_ptr(),
                                            ws.numel() * ws.element_size(), wait_limit, _stream(stream)))
+
+
+def us_test_linear_fwd_starved_cta(X, W, alpha, Y, ws, wait_limit: int, cta: int, tiles: int, stream=None):
+    """us_test_linear_fwd_starved with loads withheld from one CTA of each cluster (-1: every CTA) after its first `tiles` tiles."""
+    _check("us_test_linear_fwd_starved_cta",
+           _lib.us_test_linear_fwd_starved_cta(C.byref(mat(X)), C.byref(mat(W)), alpha, C.byref(mat(Y)), ws.data_ptr(), ws.numel(), wait_limit, cta, tiles, _stream(stream)))
+
+
+def us_test_ffn_hidden_starved_cta(X, W1, G, W2, A, dH, ws, wait_limit: int, cta: int, tiles: int, stream=None):
+    """us_test_linear_fwd_starved_cta for the kernel of us_ffn_hidden."""
+    _check("us_test_ffn_hidden_starved_cta",
+           _lib.us_test_ffn_hidden_starved_cta(*(C.byref(mat(t)) for t in (X, W1, G, W2, A, dH)), ws.data_ptr(), ws.numel(), wait_limit, cta, tiles, _stream(stream)))
+
+
+def us_test_linear_group_starved(calls, ws, wait_limit: int, cta: int, tiles: int, stream=None):
+    """us_test_linear_fwd_starved_cta for the kernels of us_linear_group_any."""
+    _check("us_test_linear_group_starved",
+           _lib.us_test_linear_group_starved(len(calls), (us_linear_call * len(calls))(*calls), ws.data_ptr(), ws.numel(), wait_limit, cta, tiles, _stream(stream)))
 
 
 def us_workspace_status_ptr(ws_ptr: int, stream=None) -> int:

@@ -61,6 +61,67 @@ def test_starved_launch_argument_checks():
     assert L.us_workspace_status(ws) == 0
 
 
+def _bytes(*ts):
+    return [t.contiguous().view(torch.uint8).clone() for t in ts]
+
+
+def _starve_and_repeat(L, ws, starve, run, outs):
+    """The results of a call before and after launches that starved are the same bits, and each of those is reported."""
+    run()
+    want = _bytes(*outs)
+    for cta, tiles in ((-1, 1), (-1, 2), (1, 0), (1, 1), (1, 2)):
+        starve(cta, tiles)
+        assert L.us_workspace_status(ws) == US_ERR_TIMEOUT, (cta, tiles)
+        ws.zero_()
+        for t in outs:
+            t.view(torch.uint8).zero_()
+        run()
+        assert L.us_workspace_status(ws) == 0, (cta, tiles)
+        assert all(torch.equal(a, b) for a, b in zip(_bytes(*outs), want)), (cta, tiles)
+
+
+@pytest.mark.parametrize("out_fmt", ["e4m3", "bf16", "f32"])
+def test_pairs_whose_operands_stop_after_some_tiles(out_fmt):
+    """240 tiles of 256 x 256, three or four per CTA pair: a pair gives up with accumulators handed back that nobody takes any more, or
+    because only its odd CTA gets no operands; both CTAs leave in order and the next call is correct."""
+    from paper_2303_11257_b200 import lib as L, synth
+    X, W, _ = synth.linear_tensors(3840, 144, 4096, 33)
+    X, W, ws, out = U.to_device(X, "e4m3"), U.to_device(W, "e4m3"), L.new_workspace(), U.empty(3840, 4096, out_fmt)
+    _starve_and_repeat(L, ws, lambda cta, tiles: L.us_test_linear_fwd_starved_cta(X, W, 1 / 12, out, ws, 2000, cta, tiles),
+                       lambda: L.us_linear_fwd(X, W, 1 / 12, out, ws), [out])
+
+
+def test_hidden_pairs_whose_operands_stop_after_some_tiles():
+    from paper_2303_11257_b200 import lib as L, synth
+    d = lambda i, shape, fmt: U.to_device(synth.normal(34, i, shape), fmt)
+    X, W1, G, W2 = d(0, (3840, 144), "e4m3"), d(1, (144, 4096), "e4m3"), d(2, (3840, 144), "e5m2"), d(3, (4096, 144), "e4m3")
+    ws, A, dH = L.new_workspace(), U.empty(3840, 4096, "e4m3"), U.empty(3840, 4096, "e5m2")
+    _starve_and_repeat(L, ws, lambda cta, tiles: L.us_test_ffn_hidden_starved_cta(X, W1, G, W2, A, dH, ws, 2000, cta, tiles),
+                       lambda: L.us_ffn_hidden(X, W1, 1 / 12, G, W2, 1 / 12, 1.0, 1.7, 1.5, A, dH, ws), [A, dH])
+
+
+@pytest.mark.parametrize("fmt", ["e4m3", "bf16"])
+def test_grouped_pairs_whose_operands_stop_after_some_tiles(fmt):
+    from paper_2303_11257_b200 import lib as L, synth
+    d = lambda i, shape: U.to_device(synth.normal(35, i, shape), fmt)
+    X, W, G, skip = d(0, (3840, 144)), d(1, (144, 4096)), d(2, (3840, 4096)), U.to_device(synth.normal(35, 3, (3840, 144)), "f32")
+    ws, Y, dX = L.new_workspace(), U.empty(3840, 4096, "bf16"), U.empty(3840, 144, "bf16")
+    calls = [L.linear_call(L.US_OP_FWD, X, W, 1 / 12, Y), L.linear_call(L.US_OP_BWD_X, G, W, 1 / 64, dX, L.epilogue(skip=skip, skip_coef=0.8, out_coef=0.6))]
+    _starve_and_repeat(L, ws, lambda cta, tiles: L.us_test_linear_group_starved(calls, ws, 2000, cta, tiles),
+                       lambda: L.us_linear_group_any(calls, ws), [Y, dX])
+
+
+def test_partly_starved_launch_argument_checks():
+    from paper_2303_11257_b200 import lib as L
+    ws = L.new_workspace()
+    X, W, Y = U.empty(32, 64, "e4m3"), U.empty(64, 48, "e4m3"), U.empty(32, 48, "f32")
+    for limit, cta, tiles in ((0, -1, 0), (1 << 17, -1, 0), (100, -2, 0), (100, 8, 0), (100, 0, -1), (100, 0, 1025)):
+        with pytest.raises(L.UnitScaleError) as e:
+            L.us_test_linear_fwd_starved_cta(X, W, 1.0, Y, ws, limit, cta, tiles)
+        assert e.value.status == 1
+    assert L.us_workspace_status(ws) == 0
+
+
 def _starve_linear(L, ws):
     X, W, Y = U.empty(96, 64, "e4m3"), U.empty(64, 80, "e4m3"), U.empty(96, 80, "f32")
     return lambda: L.us_test_linear_fwd_starved(X, W, 1.0, Y, ws, wait_limit=500)
