@@ -146,7 +146,7 @@ unsigned shared_calls(const us_linear_call* calls, const Shape* sh, int count, i
   unsigned pick = 0;
   for (int k = 0; k < count; ++k) {                       // every call of at least sh[k].K
     const int64_t K = sh[k].K;
-    if (K < 48ll * kbk || K > 8192ll * kbk) continue;
+    if (K < 48ll * kbk) continue;
     unsigned which = 0;
     bool sectors = true;
     int64_t most = 0;
@@ -156,18 +156,21 @@ unsigned shared_calls(const us_linear_call* calls, const Shape* sh, int count, i
       most = std::max(most, sh[i].K);
       sectors = sectors && calls[i].a.ld * es % 32 == 0 && calls[i].b.ld * es % 32 == 0;
     }
+    if (most > (int64_t)kSplitMostBlocks * kbk) continue;
     const double rest = group_time(sh, count, all & ~which, es, sms);
     for (int form = 0; form < 3; ++form)
       for (int s = 2; s * (form == 2 ? 2 : 1) <= 8; s *= 2) {
         const Tiling c{form == 0 ? 64 : form == 1 ? 128 : 256, form == 2 ? 2 : 1, s};
         int64_t tiles = 0;
         int a_bytes = 0;
+        bool fits = true;
         for (int i = 0; i < count; ++i)
           if (which >> i & 1) {
+            fits = fits && split_form_fits(c, sh[i].M, sh[i].N);
             tiles += ((sh[i].M + 128 * c.cg - 1) / (128 * c.cg)) * ((sh[i].N + c.bn - 1) / c.bn);
             a_bytes = std::max(a_bytes, split_a_bytes(c.bn, calls[i].op == US_OP_BWD_W, sh[i].M));
           }
-        if (tiles * c.cg * s > sms) continue;
+        if (!fits || tiles * c.cg * s > sms) continue;
         const double time = rest + tiling_time(c, tiles, (int)((most + kbk - 1) / kbk), a_bytes, sectors, sms);
         if (time < best && tiles <= split_capacity(es, c)) { best = time; pick = which; *t = c; }
       }

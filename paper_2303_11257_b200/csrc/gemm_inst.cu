@@ -120,14 +120,14 @@ static us_status pick_epilogue(const us_mat* A, const us_mat* B, const GemmParam
 template <int ES, bool A_MN, bool B_MN>
 static Tiling split_tiling(const GemmParams& p, Tiling now, bool sectors) {
   const int kb = (p.K + kStageKBytes / ES - 1) / (kStageKBytes / ES), sms = host::sm_count();
-  if (kb < (A_MN ? 48 : 20) || kb > 8192 || sms <= 0) return now;
+  if (kb < (A_MN ? 48 : 20) || kb > kSplitMostBlocks || sms <= 0) return now;
   const auto tiles = [&](const Tiling& t) { return (long long)((p.M + kBM * t.cg - 1) / (kBM * t.cg)) * ((p.N + t.bn - 1) / t.bn); };
   const auto cost = [&](const Tiling& t) { return tiling_time(t, tiles(t), kb, split_a_bytes(t.bn, A_MN, p.M), sectors, sms); };
   Tiling pick = now;
   double best = 0.92 * cost(now);
   for (int form = 0; form < 3; ++form) {
     Tiling t{form == 0 ? 64 : form == 1 ? 128 : 256, form == 2 ? 2 : 1, 2};
-    if (t.cg == 2 && (p.M <= kBM || p.N <= 128)) continue;
+    if (!split_form_fits(t, p.M, p.N)) continue;
     for (; t.splits * t.cg <= 8; t.splits *= 2) {
       if (kb < 4 * t.splits || tiles(t) * t.splits * t.cg > sms || cost(t) >= best) continue;
       if (tiles(t) > split_capacity(ES, t)) continue;

@@ -40,6 +40,10 @@ struct SplitCall {
 // Tiles of the calls' outputs all t; t.splits is 2, 4 or 8 and t.splits * t.cg at most 8.
 us_status launch_split(int count, const SplitCall* calls, const Tiling& t, unsigned int* status, uint32_t wait_limit, int starved, cudaStream_t stream);
 int split_a_bytes(int bn, bool a_mn, int64_t rows);
+// Contractions that may be shared have at most this many K blocks (128 bytes of an operand's K): what was measured.
+constexpr int kSplitMostBlocks = 8192;
+// Whether an M x N output can be tiled that way: pairs only where both halves of a tile have rows and columns.
+inline bool split_form_fits(const Tiling& t, int64_t M, int64_t N) { return t.cg == 1 || (M > 128 && N > 128); }
 // Estimated time, us, of a launch of `tiles` tiles of kb K blocks.  sectors: the operands' rows start on 32-byte boundaries.
 double tiling_time(const Tiling& t, long long tiles, int kb, int a_bytes, bool sectors, int sms);
 // Clusters of such a launch that run at once.

@@ -101,3 +101,19 @@ def test_grouped_launch_whose_long_contractions_are_shared(fmt, b, m, n):
     for i in (1, 2):
         assert torch.equal(outs[0][i].contiguous().view(torch.uint8), o[i].contiguous().view(torch.uint8))
     assert torch.equal(q.view(torch.uint8), outs[0][2].float().clamp(-57344, 57344).to(torch.float8_e5m2).view(torch.uint8))
+
+
+def test_grouped_launch_leaves_longer_contractions_than_were_measured_alone():
+    """Beyond 8192 K blocks a contraction is not shared, nor is one beside it: the bits are those of the single entry point, one accumulator
+    per tile."""
+    from paper_2303_11257_b200 import lib as L
+    ws = L.new_workspace()
+    torch.manual_seed(84)
+    long, short = (8192 + 40) * 128, 120 * 128
+    A, B = ((torch.randn(long, 16, device="cuda")).to(torch.float8_e4m3fn) for _ in range(2))
+    one, two, alone = (torch.empty(16, 16, device="cuda") for _ in range(3))
+    L.us_linear_group_any([L.linear_call(L.US_OP_BWD_W, A, B, long ** -0.5, one), L.linear_call(L.US_OP_BWD_W, A[:short], B[:short], short ** -0.5, two)], ws)
+    L.us_linear_bwd_w(A, B, long ** -0.5, alone, ws)
+    assert L.us_workspace_status(ws) == 0
+    assert torch.equal(one, alone)
+    assert (two - (A[:short].float().T @ B[:short].float()) * short ** -0.5).abs().max() <= 1e-3
