@@ -201,6 +201,9 @@ us_status us_linear_group_any(int count, const us_linear_call* calls, void* ws, 
 /* us_linear_group_any with FP8 copies as in us_linear_fwd_cast: copies[i] (ptr NULL: none) of the output of call i, which has a skip
  * tensor. */
 us_status us_linear_group_cast(int count, const us_linear_call* calls, const us_mat* copies, void* ws, size_t ws_bytes, void* stream);
+/* Number of kernels that us_linear_group_any launches for these calls on the current device (1 or 2); host only, nothing is launched.
+ * Errors as there. */
+us_status us_linear_group_launches(int count, const us_linear_call* calls, int* launches);
 
 /*
  * us_ffn_hidden: both GEMMs that end in the hidden layer of the FFN block, as ONE kernel launch.

@@ -191,12 +191,12 @@ us_status launch_group(const GroupParams& g, bool copy, cudaStream_t stream) {
 }
 
 // copies: NULL, or for each call the FP8 copy of its output (ptr NULL: none).
-// test: NULL, or a short wait limit and which CTAs get no operands.
+// test: NULL, or a short wait limit and which CTAs get no operands.  launches: NULL, or receives the number of kernels, and nothing is launched.
 struct GroupTest { uint32_t wait_limit; int starved, served; };
 us_status group_impl(int count, const us_linear_call* calls, const us_mat* copies, bool any, void* ws, size_t ws_bytes, void* stream,
-                     const GroupTest* test = nullptr) {
+                     const GroupTest* test = nullptr, int* launches = nullptr) {
   if (count < 1 || count > kGroupMaxProblems || !calls) return count >= 1 && calls ? US_ERR_UNSUPPORTED : US_ERR_INVALID_ARG;
-  if (!ws || ws_bytes < us_workspace_bytes()) return US_ERR_WORKSPACE;
+  if (!launches && (!ws || ws_bytes < us_workspace_bytes())) return US_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(ws) % 16) return US_ERR_ALIGNMENT;
   static_assert(sizeof(GroupParams) < 32000, "kernel parameter limit");
   Shape sh[kGroupMaxProblems];
@@ -234,7 +234,8 @@ us_status group_impl(int count, const us_linear_call* calls, const us_mat* copie
     copy = copy || q;
     pair_tiles += ((sh[i].M + 255) / 256) * ((sh[i].N + 255) / 256);
   }
-  if (left == 0) return launch_split(splits, split_calls, t, static_cast<unsigned int*>(ws), tt.wait_limit, starved, st);
+  if (launches) *launches = (splits > 0) + (left > 0);
+  if (left == 0) return launches ? US_OK : launch_split(splits, split_calls, t, static_cast<unsigned int*>(ws), tt.wait_limit, starved, st);
   const bool pair = pair_tiles_pay(pair_tiles, sms);
   const int tile_m = pair ? 256 : 128, bn = pair ? 256 : 128;
   int64_t tiles = 0;
@@ -262,6 +263,7 @@ us_status group_impl(int count, const us_linear_call* calls, const us_mat* copie
     P.copy_ld = P.copy ? copies[i].ld : 0;
     P.copy_dt = P.copy ? copies[i].dtype : US_E4M3;
     P.copy_sectors = reinterpret_cast<uintptr_t>(P.copy) % 32 == 0 && P.copy_ld % 32 == 0;
+    if (launches) continue;
     if (!make_tmap(&P.ta, &c.a, es, P.a_mn ? 128 / es : 128) || !make_tmap(&P.tb, &c.b, es, P.b_mn ? 128 / es : 128)) return US_ERR_CUDA;
     const int oes = dtype_size(c.out.dtype);
     if (!make_tmap(&P.tout, &c.out, oes, 32, std::min(128, bn / 2 / split * oes))) return US_ERR_CUDA;
@@ -269,6 +271,7 @@ us_status group_impl(int count, const us_linear_call* calls, const us_mat* copie
     if (P.has_skip && !make_tmap(&P.tskip, &c.ep.skip, dtype_size(c.ep.skip.dtype), 32)) return US_ERR_CUDA;
   }
   if (!deal(g, es, tile_m, bn, split, units, any ? kGroupMaxItems : 12)) return US_ERR_UNSUPPORTED;      // too many tiles per unit for the work list
+  if (launches) return US_OK;
   g.status = static_cast<unsigned int*>(ws);
   g.wait_limit = tt.wait_limit; g.starved = tt.starved; g.served = tt.served;
   if (splits) {                                            // (a grouped launch that is refused has launched nothing)
@@ -290,6 +293,10 @@ extern "C" us_status us_linear_group_any(int count, const us_linear_call* calls,
 }
 extern "C" us_status us_linear_group_cast(int count, const us_linear_call* calls, const us_mat* copies, void* ws, size_t ws_bytes, void* stream) {
   return copies ? us::group_impl(count, calls, copies, true, ws, ws_bytes, stream) : US_ERR_INVALID_ARG;
+}
+extern "C" us_status us_linear_group_launches(int count, const us_linear_call* calls, int* launches) {
+  if (!launches) return US_ERR_INVALID_ARG;
+  return us::group_impl(count, calls, nullptr, true, nullptr, 0, nullptr, nullptr, launches);
 }
 extern "C" us_status us_test_linear_group_starved(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, unsigned int wait_limit, int cta, int tiles,
                                                   void* stream) {

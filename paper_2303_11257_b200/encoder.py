@@ -139,10 +139,24 @@ class UnitScaledEncoderLayer:
 
     @property
     def kernel_launches(self) -> int:
-        """Kernel launches of one step while the grouped launches hold its tiles: launches_per_step less one for each
-        projection, with layer norms the three GEMMs that end the FFN block's backward pass as one, the fused backward pass of
-        attention as one, and the casts that their tensors' producers make."""
-        return self.launches_per_step - 2 - (2 if self.norm is not None and self.ffn.grouped else 0) - (2 if self.whole_bwd else 0) - (2 if self.norm is None else 3)
+        """Kernel launches of one step: launches_per_step with the two gradient GEMMs of a projection, with layer norms the three
+        GEMMs that end the FFN block's backward pass, and the fused backward pass of attention as the launches they make, and
+        less the casts that their tensors' producers make."""
+        together = sum(2 - L.us_linear_group_launches(calls) for calls in (self._out_grads(), self._qkv_grads()))
+        if self.norm is not None and self.ffn.grouped:
+            together += 3 - self.ffn._group_launches(forward=False)
+        return self.launches_per_step - together - (2 if self.whole_bwd else 0) - (2 if self.norm is None else 3)
+
+    def _out_grads(self):
+        """Gradient GEMMs of the output projection."""
+        sc = self.sc
+        return [L.linear_call(L.US_OP_BWD_W, self.Cq, self.g1q, sc["beta_w"], self.dWo), L.linear_call(L.US_OP_BWD_X, self.g1q, self.Wo_q, sc["beta_o"], self.dC)]
+
+    def _qkv_grads(self, ep=None):
+        """Gradient GEMMs of the query, key and value projections."""
+        sc = self.sc
+        return [L.linear_call(L.US_OP_BWD_W, self.Xq, self.dQKVq, sc["beta_w"], self.dWqkv),
+                L.linear_call(L.US_OP_BWD_X, self.dQKVq, self.Wqkv_q, sc["beta_qkv"], self.dX, ep)]
 
     def _heads(self, M, which):
         """Problem (0, 0) of a [T x 3d] matrix: rows of the first sequence, columns of head 0 of Q / K / V."""
@@ -318,8 +332,7 @@ class UnitScaledEncoderLayer:
             fn(side)
 
         L.us_cast_fp8(g1, 1.0, self.g1q, cur)
-        L.linear_together([L.linear_call(L.US_OP_BWD_W, self.Cq, self.g1q, sc["beta_w"], self.dWo),
-                           L.linear_call(L.US_OP_BWD_X, self.g1q, self.Wo_q, sc["beta_o"], self.dC)], ws, cur)
+        L.linear_together(self._out_grads(), ws, cur)
         dC_h = self.dC[:s, : self.hd]
         if self.whole_bwd:
             L.us_attention_bwd_all(dC_h, self.P[:s], Q, K, V, sc["beta_P"], sc["sm"], sc["sm"], sc["beta_Q"], sc["beta_K"], sc["beta_V"],
@@ -341,8 +354,7 @@ class UnitScaledEncoderLayer:
         if self.dQKV is not self.dQKVq:
             L.us_cast_fp8(self.dQKV, 1.0, self.dQKVq, cur)
         ep = L.epilogue(skip=g1, skip_coef=self.c_skip, out_coef=self.c_branch)
-        L.linear_together([L.linear_call(L.US_OP_BWD_W, self.Xq, self.dQKVq, sc["beta_w"], self.dWqkv),
-                           L.linear_call(L.US_OP_BWD_X, self.dQKVq, self.Wqkv_q, sc["beta_qkv"], self.dX, ep)], ws, cur)
+        L.linear_together(self._qkv_grads(ep), ws, cur)
         return self.dX
 
     def check(self) -> None:

@@ -181,13 +181,22 @@ class UnitScaledFFN:
 
     @property
     def gemm_launches(self) -> int:
-        """Launches step_from_casts() makes for the six GEMMs."""
-        return 6 - ((3 + (1 if self.fused_hidden else 0)) if self.grouped else 0)
+        """Launches step_from_casts() makes for the six GEMMs: the grouped launch is two where it shares the weight gradients'
+        contractions (many tokens, a narrow block)."""
+        if not self.grouped:
+            return 6
+        return (1 if self.fused_hidden else 2) + self._group_launches(forward=True)
+
+    def _group_launches(self, forward: bool) -> int:
+        """Launches of the GEMMs that follow the GELU-gradient GEMM, with the second forward GEMM among them or not."""
+        sc = self.sc
+        calls = [L.linear_call(L.US_OP_BWD_W, self.Aq, self.Gq, sc.beta_w, self.dW2), L.linear_call(L.US_OP_BWD_W, self.Xq, self.dHq, sc.beta_w, self.dW1),
+                 L.linear_call(L.US_OP_BWD_X, self.dHq, self.W1q, sc.beta_x1, self.dX)]
+        return L.us_linear_group_launches(calls + ([L.linear_call(L.US_OP_FWD, self.Aq, self.W2q, sc.alpha2, self.R)] if forward else []))
 
     @property
     def launches_per_step(self) -> int:
-        """Kernel launches of step(): the cast(s) plus gemm_launches (one more where the grouped launch shares the weight
-        gradients' contractions: many tokens, a narrow block)."""
+        """Kernel launches of step(): the cast(s) plus gemm_launches."""
         if self.fused_casts:
             return 1 + self.gemm_launches
         return 10

@@ -106,6 +106,8 @@ def _load() -> C.CDLL:
     lib.us_linear_group.argtypes = [C.c_int, C.POINTER(us_linear_call), V, SZ, V]
     lib.us_linear_group_any.argtypes = lib.us_linear_group.argtypes
     lib.us_linear_group.restype = lib.us_linear_group_any.restype = C.c_int
+    lib.us_linear_group_launches.argtypes = [C.c_int, C.POINTER(us_linear_call), C.POINTER(C.c_int)]
+    lib.us_linear_group_launches.restype = C.c_int
     lib.us_linear_fwd_cast.argtypes = [MP, MP, F, EP, MP, MP, V, SZ, V]
     lib.us_linear_group_cast.argtypes = [C.c_int, C.POINTER(us_linear_call), MP, V, SZ, V]
     lib.us_layer_norm_fwd_cast.argtypes = [MP, MP, MP, F, MP, MP, V]
@@ -466,6 +468,16 @@ def us_linear_group(calls, ws, stream=None, name="us_linear_group"):
 def us_linear_group_any(calls, ws, stream=None):
     """us_linear_group for 16-bit operands and outputs of any size, too."""
     us_linear_group(calls, ws, stream, "us_linear_group_any")
+
+
+def us_linear_group_launches(calls) -> int:
+    """Number of kernels us_linear_group_any launches for these calls; one each where it refuses them (linear_together)."""
+    n = C.c_int()
+    status = _lib.us_linear_group_launches(len(calls), (us_linear_call * len(calls))(*calls), C.byref(n))
+    if status == US_ERR_UNSUPPORTED:
+        return len(calls)
+    _check("us_linear_group_launches", status)
+    return n.value
 
 
 def linear_each(calls, ws, stream=None):
