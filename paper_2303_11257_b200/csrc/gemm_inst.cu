@@ -100,7 +100,9 @@ static us_status pick_epilogue(const us_mat* A, const us_mat* B, const GemmParam
                                      : launch<ES, A_MN, B_MN, BN, CG, kEpiPlain, 8>(A, B, p, em, stream);
     case kEpiGelu:     return launch<ES, A_MN, B_MN, BN, CG, kEpiGelu, 8>(A, B, p, em, stream);
     case kEpiGeluGrad: return launch<ES, A_MN, B_MN, BN, CG, kEpiGeluGrad, 8>(A, B, p, em, stream);
-    case kEpiSkip:     return launch<ES, A_MN, B_MN, BN, CG, kEpiSkip, 8>(A, B, p, em, stream);
+    case kEpiSkip:
+      return em.out->dtype == US_F32 ? launch<ES, A_MN, B_MN, BN, CG, kEpiSkipF32, 8>(A, B, p, em, stream)
+                                     : launch<ES, A_MN, B_MN, BN, CG, kEpiSkip, 8>(A, B, p, em, stream);
     default:           return launch<ES, A_MN, B_MN, BN, CG, kEpiLegacy, 8>(A, B, p, em, stream);
   }
 }
