@@ -306,6 +306,12 @@ us_status us_test_ffn_hidden_starved_cta(const us_mat* X, const us_mat* W1, cons
 us_status us_test_linear_group_starved(int count, const us_linear_call* calls, void* ws, size_t ws_bytes, unsigned int wait_limit, int cta,
                                        int tiles, void* stream);
 
+/* us_test_linear_tiling: how the output of a linear op would be tiled on the current device (host only, nothing is launched): columns of
+ * a tile (64, 128 or 256), CTAs that work on it as a pair (1 or 2), and CTAs or pairs that share its contraction (1, 2, 4 or 8).  op: a
+ * us_linear_op; arguments and errors as for the single entry point. */
+us_status us_test_linear_tiling(int op, const us_mat* A, const us_mat* B, const us_epilogue* ep, const us_mat* out, void* ws, size_t ws_bytes,
+                                int* cols, int* ctas, int* shares);
+
 /* Activations of the table "Table of unit scaling factors", section Activations. */
 typedef enum { US_FN_GELU = 0, US_FN_RELU = 1, US_FN_TANH = 2, US_FN_SIGMOID = 3 } us_fn;
 

@@ -35,7 +35,7 @@ struct WaitTest {
 // A, B: the two operands in call order; out [M x N].
 static us_status linear(Op op, const us_mat* A, const us_mat* B, float scale, const us_epilogue* ep, const us_mat* out,
                         void* ws, size_t ws_bytes, void* stream, const us_batch* batch = nullptr,
-                        const WaitTest* wt = nullptr, bool validate_only = false, const us_mat* copy = nullptr) {
+                        const WaitTest* wt = nullptr, bool validate_only = false, const us_mat* copy = nullptr, Tiling* tiling = nullptr) {
   if (!valid_mat(A) || !valid_mat(B) || !valid_mat(out)) return US_ERR_INVALID_ARG;
   int64_t M, N, K;
   bool shapes_ok;
@@ -128,15 +128,15 @@ static us_status linear(Op op, const us_mat* A, const us_mat* B, float scale, co
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (f8) {
     switch (op) {
-      case kFwd:  return launch_gemm<1, false, true>(A, B, p, em, epi, bd, st);
-      case kBwdX: return launch_gemm<1, false, false>(A, B, p, em, epi, bd, st);
-      default:    return launch_gemm<1, true, true>(A, B, p, em, epi, bd, st);
+      case kFwd:  return launch_gemm<1, false, true>(A, B, p, em, epi, bd, st, tiling);
+      case kBwdX: return launch_gemm<1, false, false>(A, B, p, em, epi, bd, st, tiling);
+      default:    return launch_gemm<1, true, true>(A, B, p, em, epi, bd, st, tiling);
     }
   }
   switch (op) {
-    case kFwd:  return launch_gemm<2, false, true>(A, B, p, em, epi, bd, st);
-    case kBwdX: return launch_gemm<2, false, false>(A, B, p, em, epi, bd, st);
-    default:    return launch_gemm<2, true, true>(A, B, p, em, epi, bd, st);
+    case kFwd:  return launch_gemm<2, false, true>(A, B, p, em, epi, bd, st, tiling);
+    case kBwdX: return launch_gemm<2, false, false>(A, B, p, em, epi, bd, st, tiling);
+    default:    return launch_gemm<2, true, true>(A, B, p, em, epi, bd, st, tiling);
   }
 }
 
@@ -178,6 +178,16 @@ extern "C" us_status us_linear_bwd_w_batched(const us_mat* X, const us_mat* G, f
 extern "C" us_status us_linear_fwd_check(const us_mat* X, const us_mat* W, const us_epilogue* ep, const us_mat* Y,
                                          const void* ws, size_t ws_bytes) {
   return us::linear(us::kFwd, X, W, 1.f, ep, Y, const_cast<void*>(ws), ws_bytes, nullptr, nullptr, nullptr, true);
+}
+
+extern "C" us_status us_test_linear_tiling(int op, const us_mat* A, const us_mat* B, const us_epilogue* ep, const us_mat* out, void* ws, size_t ws_bytes, int* cols,
+                                           int* ctas, int* shares) {
+  if (op < US_OP_FWD || op > US_OP_BWD_W || !cols || !ctas || !shares) return US_ERR_INVALID_ARG;
+  us::Tiling t{};
+  const us_status s = us::linear(op == US_OP_FWD ? us::kFwd : op == US_OP_BWD_X ? us::kBwdX : us::kBwdW, A, B, 1.f, ep, out, ws, ws_bytes, nullptr, nullptr, nullptr,
+                                 false, nullptr, &t);
+  *cols = t.bn; *ctas = t.cg; *shares = t.splits;
+  return s;
 }
 
 extern "C" us_status us_test_linear_fwd_starved(const us_mat* X, const us_mat* W, float alpha, const us_mat* Y, void* ws,

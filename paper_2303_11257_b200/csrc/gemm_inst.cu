@@ -144,7 +144,7 @@ static Tiling split_tiling(const GemmParams& p, Tiling now, bool sectors) {
 
 template <int ES, bool A_MN, bool B_MN>
 us_status launch_gemm(const us_mat* A, const us_mat* B, GemmParams& p, const EpiMats& em, int epi, const BatchDesc& bd,
-                      cudaStream_t stream) {
+                      cudaStream_t stream, Tiling* only) {
   // CTA pairs with 256 x 256 tiles whenever such a tile is not mostly empty and there are enough of them to occupy at
   // least half of the machine's CTA pairs; 128 x 128 tiles otherwise (a 1024 x 1024 output is 16 pair tiles on 74
   // pairs, but 64 single-CTA tiles).
@@ -171,6 +171,10 @@ us_status launch_gemm(const us_mat* A, const us_mat* B, GemmParams& p, const Epi
   if (!bd.batched() && (epi == kEpiPlain || epi == kEpiSkip || epi == kEpiSkipCopy)) {
     const bool sectors = A->ld * ES % 32 == 0 && B->ld * ES % 32 == 0;
     t = split_tiling<ES, A_MN, B_MN>(p, t, sectors);
+  }
+  if (only) {
+    *only = t;
+    return US_OK;
   }
   const int bn = t.bn, cg = t.cg;
   if (t.splits > 1) {
@@ -201,6 +205,6 @@ us_status launch_gemm(const us_mat* A, const us_mat* B, GemmParams& p, const Epi
 }
 
 template us_status launch_gemm<US_INST_ES, (US_INST_AMN != 0), (US_INST_BMN != 0)>(const us_mat*, const us_mat*, GemmParams&,
-                                                                                 const EpiMats&, int, const BatchDesc&, cudaStream_t);
+                                                                                 const EpiMats&, int, const BatchDesc&, cudaStream_t, Tiling*);
 
 }  // namespace us

@@ -50,9 +50,10 @@ double tiling_time(const Tiling& t, long long tiles, int kb, int a_bytes, bool s
 int split_capacity(int es, const Tiling& t);
 
 // Builds the tensor maps, picks the tile configuration and launches the kernel for
-// ES-byte operands (1 = FP8, 2 = BF16 / F16) with the given operand layouts and epilogue kind.
+// ES-byte operands (1 = FP8, 2 = BF16 / F16) with the given operand layouts and epilogue kind.  only: NULL, or takes the configuration, and
+// nothing is launched.
 template <int ES, bool A_MN, bool B_MN>
 us_status launch_gemm(const us_mat* A, const us_mat* B, GemmParams& p, const EpiMats& em, int epi, const BatchDesc& bd,
-                      cudaStream_t stream);
+                      cudaStream_t stream, Tiling* only);
 
 }  // namespace us

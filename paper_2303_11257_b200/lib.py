@@ -106,6 +106,8 @@ def _load() -> C.CDLL:
     lib.us_linear_group.argtypes = [C.c_int, C.POINTER(us_linear_call), V, SZ, V]
     lib.us_linear_group_any.argtypes = lib.us_linear_group.argtypes
     lib.us_linear_group.restype = lib.us_linear_group_any.restype = C.c_int
+    lib.us_test_linear_tiling.argtypes = [C.c_int, MP, MP, EP, MP, V, SZ] + [C.POINTER(C.c_int)] * 3
+    lib.us_test_linear_tiling.restype = C.c_int
     lib.us_linear_group_launches.argtypes = [C.c_int, C.POINTER(us_linear_call), C.POINTER(C.c_int)]
     lib.us_linear_group_launches.restype = C.c_int
     lib.us_linear_fwd_cast.argtypes = [MP, MP, F, EP, MP, MP, V, SZ, V]
@@ -628,6 +630,14 @@ def us_test_linear_fwd_starved_cta(X, W, alpha, Y, ws, wait_limit: int, cta: int
     """us_test_linear_fwd_starved with loads withheld from one CTA of each cluster (-1: every CTA) after its first `tiles` tiles."""
     _check("us_test_linear_fwd_starved_cta",
            _lib.us_test_linear_fwd_starved_cta(C.byref(mat(X)), C.byref(mat(W)), alpha, C.byref(mat(Y)), ws.data_ptr(), ws.numel(), wait_limit, cta, tiles, _stream(stream)))
+
+
+def us_test_linear_tiling(op: int, a, b, out, ws, ep=None) -> tuple[int, int, int]:
+    """Columns of a tile, CTAs that work on it as a pair, CTAs or pairs that share its contraction."""
+    r = [C.c_int() for _ in range(3)]
+    _check("us_test_linear_tiling", _lib.us_test_linear_tiling(op, C.byref(mat(a)), C.byref(mat(b)), C.byref(ep) if ep is not None else None, C.byref(mat(out)),
+                                                               ws.data_ptr(), ws.numel(), *(C.byref(x) for x in r)))
+    return tuple(x.value for x in r)
 
 
 def us_test_ffn_hidden_starved_cta(X, W1, G, W2, A, dH, ws, wait_limit: int, cta: int, tiles: int, stream=None):

@@ -1,5 +1,5 @@
 """Linear ops whose contraction is shared by the CTAs of a cluster (few output tiles, long K): two, four and eight CTAs on tiles of 128 x 64
-and 128 x 128, two and four CTA pairs on 256 x 256, with rows, columns and K blocks that do not divide.  A part of the contraction is a
+and 128 x 128, two and four CTA pairs on 256 x 256 (test_every_form says which call takes which), with rows, columns and K blocks that do not divide.  A part of the contraction is a
 float32 sum like the whole, so the bounds are those of the unshared kernels."""
 import numpy as np
 import pytest
@@ -55,19 +55,53 @@ def test_shared_contraction_with_a_copy_in_fp8(rows, k, cols):
     assert torch.equal(q.view(torch.uint8), out.float().clamp(-448, 448).to(torch.float8_e4m3fn).view(torch.uint8))
 
 
-def test_waits_that_run_out_in_a_cluster():
-    """Operand loads withheld: every CTA's waits run out, the cluster's barriers are passed all the same, the status says so, and
-    the next call is correct."""
+# Every form: (columns of a tile, CTAs of a pair, shares) on 148 SMs, and a forward call that takes it.
+FORMS = {(64, 1, 2): ("e4m3", 300, 5024, 690), (64, 1, 4): ("e4m3", 48, 4096, 1024), (64, 1, 8): ("bf16", 1, 2576, 16), (128, 1, 2): ("bf16", 500, 6160, 1300),
+         (128, 1, 4): ("bf16", 300, 5008, 690), (128, 1, 8): ("e4m3", 128, 32768, 1280), (256, 2, 2): ("e4m3", 2048, 6400, 1024), (256, 2, 4): ("bf16", 1000, 8208, 700)}
+
+
+@pytest.mark.parametrize("form", list(FORMS), ids=str)
+def test_every_form(form):
+    """The form is the one that is meant; its result; its waits when they run out in every CTA, and in one CTA only (of a pair the odd one):
+    the cluster's barriers are passed all the same, the status says so, and the next call has the bits of the first."""
     from paper_2303_11257_b200 import lib as L, synth
-    for rows, k, cols in ((48, 4096, 1024), (2048, 6400, 1024)):
-        X, W, val, scale = _operands(L, synth, "fwd", rows, k, cols, 83, "e4m3", "e4m3")
-        ws, out = L.new_workspace(), U.empty(rows, cols, "bf16")
-        L.us_test_linear_fwd_starved(X, W, scale, out, ws, 2000)
-        assert L.us_workspace_status(ws) == L.US_ERR_TIMEOUT
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the choice depends on the number of SMs")
+    fmt, rows, k, cols = FORMS[form]
+    X, W, val, scale = _operands(L, synth, "fwd", rows, k, cols, 83, fmt, fmt)
+    ws, out = L.new_workspace(), U.empty(rows, cols, "f32", PAD(cols))
+    assert L.us_test_linear_tiling(L.US_OP_FWD, X, W, out, ws) == form
+    L.us_linear_fwd(X, W, scale, out, ws)
+    assert L.us_workspace_status(ws) == 0
+    U.assert_close_stored(out, val, "f32", TOL * max(1.0, np.abs(val).max() / 4), "first")
+    first = out.clone()
+    ctas = form[1] * form[2]
+    for cta in (-1, 1, ctas - 1):
+        L.us_test_linear_fwd_starved_cta(X, W, scale, out, ws, 2000, cta, 0)
+        assert L.us_workspace_status(ws) == L.US_ERR_TIMEOUT, cta
         ws.zero_()
         L.us_linear_fwd(X, W, scale, out, ws)
-        assert L.us_workspace_status(ws) == 0
-        U.assert_close_stored(out, val, "bf16", TOL * max(1.0, np.abs(val).max() / 4), "after")
+        assert L.us_workspace_status(ws) == 0 and torch.equal(out, first), cta
+
+
+@pytest.mark.parametrize("fmt,b,m,n", [("e4m3", 16000, 128, 400), ("bf16", 9008, 256, 768)])
+def test_waits_that_run_out_in_the_shared_launch_of_a_group(fmt, b, m, n):
+    from paper_2303_11257_b200 import lib as L, synth
+    dev = lambda i, shape: U.to_device(synth.normal(95 + i, 0, shape), fmt, PAD(shape[1]))
+    X, W, G, ws = dev(0, (b, m)), dev(1, (m, n)), dev(2, (b, n)), L.new_workspace()
+    outs = [U.empty(m, n, "f32"), U.empty(m, n, "bf16", PAD(n)), U.empty(b, n, "bf16", PAD(n)), U.empty(b, m, "bf16")]
+    calls = [L.linear_call(L.US_OP_BWD_W, X, G, b ** -0.5, outs[0]), L.linear_call(L.US_OP_BWD_W, X, G, b ** -0.5, outs[1]), L.linear_call(L.US_OP_FWD, X, W, 0.1, outs[2]),
+             L.linear_call(L.US_OP_BWD_X, G, W, 0.1, outs[3])]
+    assert L.us_linear_group_launches(calls) == 2
+    L.us_linear_group_any(calls, ws)
+    assert L.us_workspace_status(ws) == 0
+    first = [t.clone() for t in outs]
+    for cta in (-1, 1, 3):
+        L.us_test_linear_group_starved(calls, ws, 2000, cta, 0)
+        assert L.us_workspace_status(ws) == L.US_ERR_TIMEOUT, cta
+        ws.zero_()
+        L.us_linear_group_any(calls, ws)
+        assert L.us_workspace_status(ws) == 0 and all(torch.equal(t.view(torch.uint8), f.view(torch.uint8)) for t, f in zip(outs, first)), cta
 
 
 @pytest.mark.parametrize("fmt", ["e4m3", "bf16"])

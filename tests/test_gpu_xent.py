@@ -157,6 +157,38 @@ def test_softmax_xent_backward_of_rows_that_are_not_finite(rows, cols, out_fmt):
     U.assert_close_stored(dX[torch.from_numpy(pick).cuda()], ref, out_fmt, 3e-6 * 8.0, "xent bwd")
 
 
+@pytest.mark.parametrize("rows,cols", [(2400, 700), (700, 3000), (700, 9001), (300, 12000), (40, 16390), (40, 30522), (12, 40000)])
+@pytest.mark.parametrize("in_fmt", ["bf16", "fp16"])
+def test_softmax_xent_of_rows_that_are_not_finite_in_every_form(rows, cols, in_fmt):
+    """A warp per row, registers, the ring, staged rows, rows that are read again: a NaN, a +inf and a row of -inf only make the row's
+    log-likelihood and gradient NaN, in the maximum of packed pairs as well; classes of -inf or of the type's lowest value (masks) have
+    weight zero."""
+    L, synth = _mods()
+    ld = (cols + 15) // 16 * 16
+    x = U.values_of(synth.normal(39, cols, (rows, cols), 2.0), in_fmt).astype(np.float32)
+    bad = {3: (cols // 3, np.nan), 4: (cols - 1, np.nan), 5: (0, np.inf), 6: (slice(None), -np.inf)}
+    for r, (where, v) in bad.items():
+        x[r, where] = v
+    x[8, 1::2] = -np.inf
+    # (some classes, not all: the row's maximum times log2 e is rounded before it is subtracted, by up to 2^-8 at 65504, and overflows in BF16)
+    x[9, 1::3] = -65504.0 if in_fmt == "fp16" else -3.3895314e38
+    X = torch.zeros(rows, ld, device="cuda", dtype=U.TORCH_OF[in_fmt])[:, :cols]
+    X.copy_(torch.from_numpy(x))
+    t = (np.arange(rows) * 7919 % cols).astype(np.int32)
+    t[8] = t[8] // 2 * 2
+    tt, out, dX = torch.from_numpy(t).cuda(), torch.empty(rows, device="cuda"), U.empty(rows, cols, "bf16", ld)
+    L.us_softmax_xent_fwd(X, tt, out)
+    L.us_softmax_xent_bwd(X, tt, None, 8.0, dX)
+    got, ll, good = dX.float().cpu().numpy(), out.cpu().numpy(), np.setdiff1d(np.arange(rows), list(bad))
+    assert np.isnan(got[list(bad)]).all() and np.isfinite(got[good]).all()
+    assert np.isnan(ll[list(bad)]).all() and np.isfinite(ll[good]).all()
+    pick = np.unique(np.concatenate([good[:8], good[::53]]))
+    v = X.double().cpu().numpy()[pick]
+    ref = O.softmax_xent_fwd(v, t[pick])
+    assert np.abs(ll[pick] - ref).max() <= 4e-6 * (1 + np.abs(ref).max())
+    U.assert_close_stored(dX[torch.from_numpy(pick).cuda()], O.softmax_xent_bwd(v, t[pick], np.ones(len(pick)), 8.0), "bf16", 3e-6 * 8.0, "xent bwd")
+
+
 @pytest.mark.parametrize("rows,cols,out_fmt", [(700, 3000, "bf16"), (700, 5000, "f32"), (700, 6003, "bf16"), (700, 9000, "f32"), (300, 12001, "e5m2"), (9, 20003, "f32"), (9, 40001, "bf16")])
 @pytest.mark.parametrize("in_fmt", ["bf16", "fp16"])
 def test_softmax_xent_backward_of_an_infinite_gradient(rows, cols, out_fmt, in_fmt):
