@@ -389,7 +389,9 @@ static us_status cast_multi(int count, const us_mat* src, const float* scale, co
   if (sms <= 0) return US_ERR_CUDA;
   const int64_t want = (chunks + kThreads - 1) / kThreads;
   const int64_t cap = (int64_t)sms * 8;
-  return host::launch(padded ? (f32 ? multi_cast_kernel<true, true> : multi_cast_kernel<true, false>) : f32 ? multi_cast_kernel<false, true> : multi_cast_kernel<false, false>, nullptr, (int)(want < cap ? want : cap), kThreads, 0, 1, static_cast<cudaStream_t>(stream), p);
+  void (*kern)(const MultiCastArgs) = padded ? (f32 ? multi_cast_kernel<true, true> : multi_cast_kernel<true, false>)
+                                             : (f32 ? multi_cast_kernel<false, true> : multi_cast_kernel<false, false>);
+  return host::launch(kern, nullptr, (int)(want < cap ? want : cap), kThreads, 0, 1, static_cast<cudaStream_t>(stream), p);
 }
 
 extern "C" us_status us_cast_fp8_multi(int count, const us_mat* src, const float* scale, const us_mat* dst, void* stream) {

@@ -427,20 +427,7 @@ ffn_hidden_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   }
 }
 
-// Row-major [rows x cols] matrix of es-byte elements, boxes of box_rows rows x box_bytes, swizzled with the
-// pattern of that width; out-of-range parts of a box read as zero and are not written.
-bool make_tmap(CUtensorMap* tm, const us_mat* m, int es, int box_rows, int box_bytes) {
-  host::EncodeTiledFn fn = host::encode_tiled_fn();
-  if (!fn) return false;
-  const CUtensorMapDataType type = es == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_UINT16;
-  cuuint64_t dims[2] = {(cuuint64_t)m->cols, (cuuint64_t)m->rows};
-  cuuint64_t strides[1] = {(cuuint64_t)m->ld * es};
-  cuuint32_t box[2] = {(cuuint32_t)(box_bytes / es), (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(tm, type, 2, m->ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            box_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_NONE : box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
+using host::make_tmap;
 
 bool aligned16(const us_mat* m) {
   return reinterpret_cast<uintptr_t>(m->ptr) % 16 == 0 && (m->ld * dtype_size(m->dtype)) % 16 == 0;
@@ -516,7 +503,8 @@ us_status hidden_impl(const us_mat* X, const us_mat* W1, float alpha, const us_m
   p.x_bytes = (uint32_t)x_rows * kStageKBytes;
   using Half1 = HidSmem<128, 1, 64>;
   using Half2 = HidSmem<128, 2, 64>;
-  p.stages = (int)std::min((uint32_t)Half1::kMaxStages, (uint32_t)(f8 ? Half1::kStages * Half1::kStageBytes : Half2::kStages * Half2::kStageBytes) / (p.x_bytes + (uint32_t)Half1::kBBytes));
+  const int room = f8 ? Half1::kStages * Half1::kStageBytes : Half2::kStages * Half2::kStageBytes;
+  p.stages = std::min(Half1::kMaxStages, room / ((int)p.x_bytes + Half1::kBBytes));
   p.scale1 = alpha; p.scale2 = beta_x;
   p.act_in = act_in_scale; p.act_out = act_out_scale; p.grad_out = grad_out_scale;
   p.h_ptr = keep_h ? static_cast<uint8_t*>(H->ptr) : nullptr;

@@ -16,33 +16,22 @@
 namespace us {
 namespace {
 
-// Tensor map over a row-major matrix [rows x cols] of ES-byte elements with a box of `box_rows` rows
-// and `box_bytes` (128, 64 or 32) bytes per row, swizzled with the pattern of that width (32: not).  Out-of-range parts of a box read as zero.
+// host::make_tmap, or with a batch (bstride: elements between problems) a map of rank 4: column, row, inner batch index, outer batch
+// index; a box never spans problems.
 static bool make_tmap(CUtensorMap* tm, const us_mat* m, int es, int box_rows, int box_bytes = 128,
                       const BatchDesc* bd = nullptr, const int64_t* bstride = nullptr) {
+  if (!bd) return host::make_tmap(tm, m, es, box_rows, box_bytes);
   host::EncodeTiledFn fn = host::encode_tiled_fn();
   if (!fn) return false;
   const CUtensorMapDataType type = es == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8
                                  : es == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_UINT32;
-  const CUtensorMapSwizzle swz = box_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_NONE : box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
-  CUresult r;
-  if (!bd) {
-    cuuint64_t dims[2] = {(cuuint64_t)m->cols, (cuuint64_t)m->rows};
-    cuuint64_t strides[1] = {(cuuint64_t)m->ld * es};
-    cuuint32_t box[2] = {(cuuint32_t)(box_bytes / es), (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    r = fn(tm, type, 2, m->ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
-           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  } else {
-    // rank 4: (column, row, inner batch index, outer batch index); a box never spans problems
-    cuuint64_t dims[4] = {(cuuint64_t)m->cols, (cuuint64_t)m->rows, (cuuint64_t)bd->nb1, (cuuint64_t)bd->nb0};
-    cuuint64_t strides[3] = {(cuuint64_t)m->ld * es, (cuuint64_t)bstride[1] * es, (cuuint64_t)bstride[0] * es};
-    cuuint32_t box[4] = {(cuuint32_t)(box_bytes / es), (cuuint32_t)box_rows, 1, 1};
-    cuuint32_t estr[4] = {1, 1, 1, 1};
-    r = fn(tm, type, 4, m->ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
-           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  }
-  return r == CUDA_SUCCESS;
+  cuuint64_t dims[4] = {(cuuint64_t)m->cols, (cuuint64_t)m->rows, (cuuint64_t)bd->nb1, (cuuint64_t)bd->nb0};
+  cuuint64_t strides[3] = {(cuuint64_t)m->ld * es, (cuuint64_t)bstride[1] * es, (cuuint64_t)bstride[0] * es};
+  cuuint32_t box[4] = {(cuuint32_t)(box_bytes / es), (cuuint32_t)box_rows, 1, 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(tm, type, 4, m->ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            box_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_NONE : box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <int ES, bool A_MN, bool B_MN, int BN, int CG, int EPI, int EW, bool BATCHED = false>
@@ -92,9 +81,11 @@ static us_status pick_epilogue(const us_mat* A, const us_mat* B, const GemmParam
   switch (epi) {
     case kEpiPlain:
       if constexpr (CG == 2) {
-        // FP8 outputs of contractions of up to 32 K blocks: sixteen epilogue warps (beyond, equal or, at 64, 2 % slower).  Not 16-bit ones, whose tiles are bound by the bytes they write (FP8 operands into BF16, eight / sixteen
-        // warps, us: 8192 x 128 x 3072 12.1 / 11.3, x 1024 x 3072 22.6 / 23.8, 2048 x 1024 x 30528 57.6 / 60.2).
-        if ((em.out->dtype == US_E4M3 || em.out->dtype == US_E5M2) && (long long)p.K * ES <= 4096) return launch<ES, A_MN, B_MN, BN, CG, kEpiPlain16, 16>(A, B, p, em, stream);
+        // FP8 outputs of contractions of up to 32 K blocks: sixteen epilogue warps (beyond, equal or, at 64, 2 % slower).  Not 16-bit ones,
+        // whose tiles are bound by the bytes they write (FP8 operands into BF16, eight / sixteen warps, us: 8192 x 128 x 3072 12.1 / 11.3,
+        // x 1024 x 3072 22.6 / 23.8, 2048 x 1024 x 30528 57.6 / 60.2).
+        if ((em.out->dtype == US_E4M3 || em.out->dtype == US_E5M2) && (long long)p.K * ES <= 4096)
+          return launch<ES, A_MN, B_MN, BN, CG, kEpiPlain16, 16>(A, B, p, em, stream);
       }
       return em.out->dtype == US_F32 ? launch<ES, A_MN, B_MN, BN, CG, kEpiPlainF32, 8>(A, B, p, em, stream)
                                      : launch<ES, A_MN, B_MN, BN, CG, kEpiPlain, 8>(A, B, p, em, stream);

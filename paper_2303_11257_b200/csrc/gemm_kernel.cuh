@@ -293,11 +293,13 @@ __device__ __forceinline__ void stage_row32(int dt, const float (&y)[32], uint32
   } else if (dt == US_BF16) {
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      put(k, pack_bf16x2(y[8 * k], y[8 * k + 1]), pack_bf16x2(y[8 * k + 2], y[8 * k + 3]), pack_bf16x2(y[8 * k + 4], y[8 * k + 5]), pack_bf16x2(y[8 * k + 6], y[8 * k + 7]));
+      put(k, pack_bf16x2(y[8 * k], y[8 * k + 1]), pack_bf16x2(y[8 * k + 2], y[8 * k + 3]),
+          pack_bf16x2(y[8 * k + 4], y[8 * k + 5]), pack_bf16x2(y[8 * k + 6], y[8 * k + 7]));
   } else if (dt == US_F16) {
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      put(k, pack_f16x2(y[8 * k], y[8 * k + 1]), pack_f16x2(y[8 * k + 2], y[8 * k + 3]), pack_f16x2(y[8 * k + 4], y[8 * k + 5]), pack_f16x2(y[8 * k + 6], y[8 * k + 7]));
+      put(k, pack_f16x2(y[8 * k], y[8 * k + 1]), pack_f16x2(y[8 * k + 2], y[8 * k + 3]),
+          pack_f16x2(y[8 * k + 4], y[8 * k + 5]), pack_f16x2(y[8 * k + 6], y[8 * k + 7]));
   } else {
     uint32_t w[8];
 #pragma unroll

@@ -10,24 +10,13 @@
 namespace us {
 namespace {
 
-bool make_tmap(CUtensorMap* tm, const us_mat* m, int es, int box_rows, int box_bytes = 128) {
-  host::EncodeTiledFn fn = host::encode_tiled_fn();
-  if (!fn) return false;
-  const CUtensorMapDataType type = es == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8
-                                 : es == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_UINT32;
-  cuuint64_t dims[2] = {(cuuint64_t)m->cols, (cuuint64_t)m->rows};
-  cuuint64_t strides[1] = {(cuuint64_t)m->ld * es};
-  cuuint32_t box[2] = {(cuuint32_t)(box_bytes / es), (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(tm, type, 2, m->ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            box_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_NONE : box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
+using host::make_tmap;
 
 template <int ES, int BN, int CG, int PROBLEMS>
 us_status launch(const SplitParams<PROBLEMS>& p, int tiles, cudaStream_t stream) {
   static std::atomic<uint64_t> smem_set{0};
-  return host::launch(gemm_split_kernel<ES, BN, CG, (PROBLEMS > 1)>, &smem_set, CG * p.splits * tiles, gemm_threads(8), GemmSmem<BN, CG, 8>::kTotal, CG * p.splits, stream, p);
+  return host::launch(gemm_split_kernel<ES, BN, CG, (PROBLEMS > 1)>, &smem_set, CG * p.splits * tiles, gemm_threads(8), GemmSmem<BN, CG, 8>::kTotal,
+                      CG * p.splits, stream, p);
 }
 template <int ES, int BN, int CG>
 int capacity(int splits) {
@@ -57,9 +46,9 @@ us_status launch_problems(int count, const SplitCall* calls, const Tiling& t, un
     P.copy_dt = c.copy ? c.copy->dtype : US_E4M3;
     P.copy_sectors = reinterpret_cast<uintptr_t>(P.copy) % 32 == 0 && P.copy_ld % 32 == 0;
     s.a_bytes = (uint32_t)us::split_a_bytes(t.bn, c.a_mn, c.out->rows);
-    const uint32_t b_bytes = (uint32_t)(t.bn / t.cg * kStageKBytes);
-    s.stages = t.bn == 64 ? (int)std::min((uint32_t)GemmSmem<64, 1, 8>::kMaxStages, (uint32_t)(GemmSmem<64, 1, 8>::kStages * GemmSmem<64, 1, 8>::kStageBytes) / (s.a_bytes + b_bytes))
-              : t.bn == 128 ? GemmSmem<128, 1, 8>::kStages : GemmSmem<256, 2, 8>::kStages;
+    using Narrow = GemmSmem<64, 1, 8>;
+    s.stages = t.bn == 64    ? std::min((int)Narrow::kMaxStages, Narrow::kStages * Narrow::kStageBytes / ((int)s.a_bytes + Narrow::kBBytes))
+               : t.bn == 128 ? GemmSmem<128, 1, 8>::kStages : GemmSmem<256, 2, 8>::kStages;
     s.tiles_m = (P.M + kBM * t.cg - 1) / (kBM * t.cg);
     tiles += s.tiles_m * ((P.N + t.bn - 1) / t.bn);
     s.tile_end = tiles;

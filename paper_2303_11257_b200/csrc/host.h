@@ -65,6 +65,9 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn encode_tiled_fn();
+// Tensor map of a row-major matrix of es-byte elements in boxes of box_rows rows x box_bytes, swizzled with the pattern of that width (32
+// bytes: none); out-of-range parts of a box read as zero and are not written.
+bool make_tmap(CUtensorMap* tm, const us_mat* m, int es, int box_rows, int box_bytes = 128);
 // A launch without that overlap, of a kernel that may take up to max_smem bytes of dynamic shared memory.
 template <class... P, class... A>
 us_status launch_plain(void (*kern)(P...), std::atomic<uint64_t>* smem_set, int grid, int threads, int max_smem, size_t smem,

@@ -337,8 +337,9 @@ class Plan:
         self.program = names, _binding.program(steps, slots)
 
     def cast_multi(self, srcs, dsts, padded=False):
-        """us_cast_multi (us_cast_multi_pitched where a destination has padded rows) at scale 1; an entry of srcs is a tensor or the name of an input.  padded: rows that it does not
-        take (padded or unaligned ones) go out as one us_residual_add per tensor, for 16-bit destinations."""
+        """us_cast_multi (us_cast_multi_pitched where a destination has padded rows) at scale 1; an entry of srcs is a tensor or
+        the name of an input.  padded: rows that it does not take (padded or unaligned ones) go out as one us_residual_add per
+        tensor, for 16-bit destinations."""
         n = len(srcs)
         sm = (us_mat * n)()
         for i, s in enumerate(srcs):
@@ -629,7 +630,8 @@ def us_test_ffn_hidden_starved(X, W1, G, W2, A, dH, ws, wait_limit: int, stream=
 def us_test_linear_fwd_starved_cta(X, W, alpha, Y, ws, wait_limit: int, cta: int, tiles: int, stream=None):
     """us_test_linear_fwd_starved with loads withheld from one CTA of each cluster (-1: every CTA) after its first `tiles` tiles."""
     _check("us_test_linear_fwd_starved_cta",
-           _lib.us_test_linear_fwd_starved_cta(C.byref(mat(X)), C.byref(mat(W)), alpha, C.byref(mat(Y)), ws.data_ptr(), ws.numel(), wait_limit, cta, tiles, _stream(stream)))
+           _lib.us_test_linear_fwd_starved_cta(C.byref(mat(X)), C.byref(mat(W)), alpha, C.byref(mat(Y)), ws.data_ptr(), ws.numel(), wait_limit, cta, tiles,
+                                               _stream(stream)))
 
 
 def us_test_linear_tiling(op: int, a, b, out, ws, ep=None) -> tuple[int, int, int]:

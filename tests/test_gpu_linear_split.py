@@ -1,5 +1,6 @@
 """Linear ops whose contraction is shared by the CTAs of a cluster (few output tiles, long K): two, four and eight CTAs on tiles of 128 x 64
-and 128 x 128, two and four CTA pairs on 256 x 256 (test_every_form says which call takes which), with rows, columns and K blocks that do not divide.  A part of the contraction is a
+and 128 x 128, two and four CTA pairs on 256 x 256 (test_every_form says which call takes which), with rows, columns and K blocks that do
+not divide.  A part of the contraction is a
 float32 sum like the whole, so the bounds are those of the unshared kernels."""
 import numpy as np
 import pytest
@@ -90,8 +91,8 @@ def test_waits_that_run_out_in_the_shared_launch_of_a_group(fmt, b, m, n):
     dev = lambda i, shape: U.to_device(synth.normal(95 + i, 0, shape), fmt, PAD(shape[1]))
     X, W, G, ws = dev(0, (b, m)), dev(1, (m, n)), dev(2, (b, n)), L.new_workspace()
     outs = [U.empty(m, n, "f32"), U.empty(m, n, "bf16", PAD(n)), U.empty(b, n, "bf16", PAD(n)), U.empty(b, m, "bf16")]
-    calls = [L.linear_call(L.US_OP_BWD_W, X, G, b ** -0.5, outs[0]), L.linear_call(L.US_OP_BWD_W, X, G, b ** -0.5, outs[1]), L.linear_call(L.US_OP_FWD, X, W, 0.1, outs[2]),
-             L.linear_call(L.US_OP_BWD_X, G, W, 0.1, outs[3])]
+    calls = [L.linear_call(L.US_OP_BWD_W, X, G, b ** -0.5, outs[0]), L.linear_call(L.US_OP_BWD_W, X, G, b ** -0.5, outs[1]),
+             L.linear_call(L.US_OP_FWD, X, W, 0.1, outs[2]), L.linear_call(L.US_OP_BWD_X, G, W, 0.1, outs[3])]
     assert L.us_linear_group_launches(calls) == 2
     L.us_linear_group_any(calls, ws)
     assert L.us_workspace_status(ws) == 0
