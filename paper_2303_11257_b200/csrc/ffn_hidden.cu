@@ -73,8 +73,8 @@ struct HiddenParams {
 // 128 x 128 per CTA (128, 1) where the large ones would leave more than half of the pairs idle (hidden_impl).
 // SPLIT (128 x 128 tiles): CTAs that share a tile, each computing 64 of its columns (of four, two the same ones) and turning 128 / SPLIT
 // into outputs.  In a small problem the arithmetic of the epilogue (3700 + 2800 cycles of one SM's issue slots for a tile) is the
-// longest part of the launch while most SMs are idle.  With all 128 columns computed by each, the operands they fetched were twice
-// the bytes: captured steps, us, 48 x 1024 x 4096 30.7 -> 28.7, 16 x 1024 x 4096 32.4 -> 29.1, 512 x 512 x 1456 15.0 -> 14.8.
+// longest part of the launch while most SMs are idle.  With all 128 columns computed by each they fetched a third more bytes (32 KB a K block
+// instead of 24, with few rows twice as many): captured steps, us, 48 x 1024 x 4096 30.7 -> 28.7, 16 x 1024 x 4096 32.4 -> 29.1, 512 x 512 x 1456 15.0 -> 14.8.
 // OUT_A, OUT_D: output formats of A and dH (us_dtype).  H_BF16: pre-activation rounded to BF16 (else F16).
 template <int ES, int BN, int CG, int SPLIT, int OUT_A, int OUT_D, bool H_BF16>
 __global__ void __launch_bounds__(gemm_threads(kHidEW), 1)

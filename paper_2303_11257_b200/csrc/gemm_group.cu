@@ -100,6 +100,10 @@ bool deal(GroupParams& g, int es, int tile_m, int bn, int split, int units, int 
 bool pair_tiles_pay(int64_t pair_tiles, int sms) { return 8 * pair_tiles >= 3 * sms; }
 
 // Estimated time, us, of the grouped launch of the calls in `which` (a bit each): the busiest unit's K blocks, an epilogue counted as eight.
+// Measured / estimated, FP8, all four GEMMs of a step or the two that are not weight gradients: 2048 x 256 x 1024 7.0 / 6.8, 4.7 / 5.6; 4096 x 256 x
+// 1024 10.0 / 9.4, 5.8 / 5.6; 1500 x 768 x 2304 12.9 / 11.2, 7.9 / 7.2; 8192 x 144 x 512 23.1 / 24.6, 7.2 / 6.6; 8192 x 256 x 768 23.0 / 24.6, 8.1 / 7.2;
+// 16384 x 256 x 512 41.2 / 43.8, 11.1 / 9.2; low with much output, whose bytes it leaves
+// out (8192 x 512 x 2048 29.2 / 24.8, 20.1 / 15.5), and for few tiles of very long contractions (16000 x 144 x 400 56.7 / 42.9, 30000 x 144 x 288 99 / 76).
 double group_time(const Shape* sh, int count, unsigned which, int es, int sms) {
   int64_t pair_tiles = 0, blocks = 0, longest = 0;
   for (int i = 0; i < count; ++i)
@@ -119,9 +123,12 @@ double group_time(const Shape* sh, int count, unsigned which, int es, int sms) {
 
 // The calls (a bit each) whose contractions several CTAs share in a launch of their own, in tiles t; 0: none.  A few tiles with a far
 // longer contraction than the rest of the work per unit (the weight gradients of many tokens and a narrow block) leave the other
-// units of the grouped launch idle; a second launch costs what its estimate says and has to save 2 us beyond it.  Captured FFN steps,
-// one grouped launch -> two, us: FP8 8192 x 128 x 512 39.9 -> 31.6, 8192 x 256 x 768 44.6 -> 38.8, 16000 x 128 x 400 65.5 -> 44.3; BF16 4096 x 128
-// x 256 25.5 -> 18.5, 9000 x 256 x 768 74.6 -> 54.2; F16 16384 x 256 x 1024 141.9 -> 101.8; nothing of 14 such shapes slower.
+// units of the grouped launch idle; a second launch costs what its estimate says and has to save 2 us, about what the estimates are off, beyond
+// it.  Captured FFN steps, one grouped launch -> two, us: FP8 8192 x 128 x 512 39.9 -> 31.6, 8192 x 256 x 768 44.6 -> 38.8, 16000 x 128 x 400 65.5 ->
+// 44.3; BF16 4096 x 128 x 256 25.5 -> 18.5, 9000 x 256 x 768 74.6 -> 54.2; F16 16384 x 256 x 1024 141.9 -> 101.8.  Of 260 drawn groups that go out in two
+// launches (2900 to 46000 tokens; of a whole step or of a backward pass alone) the geometric mean is 1.6 times as fast, the best 4.8; eleven are 2
+// to 12 % slower (7520 x 336 x 656 25.9 -> 29.6, 5200 x 448 x 1360 in BF16 28.9 -> 31.4), all with two shares or pairs; a margin that spares them costs
+// as many others up to 1.3 times.
 unsigned shared_calls(const us_linear_call* calls, const Shape* sh, int count, int es, int sms, Tiling* t) {
   const int kbk = 128 / es;
   int64_t longest = 0;

@@ -1,7 +1,7 @@
 // GEMMs whose contractions are shared by the CTAs of a cluster (one, or up to four in a launch).
 //
-// An output of few tiles with a long contraction leaves most SMs idle, and the ones at work are bound by what an SM can take in
-// (about 86 bytes per ns: a K block of 128 x 128 FP8 operands, 32 KB, every 380 ns).  Here p.splits CTAs (or CTA pairs, CG = 2) of a
+// An output of few tiles with a long contraction leaves most SMs idle, and the ones at work are bound by what an SM can take in (a K
+// block of 128 x 128 operands, 32 KB, every 150 ns; every 380 ns, 86 bytes per ns, where rows start inside a 32-byte sector).  Here p.splits CTAs (or CTA pairs, CG = 2) of a
 // cluster compute the same tile over consecutive parts of K.  When all have finished, every block of 32 rows x 32 columns belongs to
 // one of them: the others store their partial sums into its operand ring through distributed shared memory, and it adds them to its
 // own in float32, in a fixed order, and finishes the block.  One tile per cluster, no workspace, no atomics: results do not depend on scheduling.

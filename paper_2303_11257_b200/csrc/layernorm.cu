@@ -2,7 +2,8 @@
 // factors", row layer_norm: alpha = 1, beta_x = 1, beta_w = beta_c = b^-1/2 for a b x n input).
 //
 // Forward and the input gradient are row-wise: one warp per row, 128-bit loads and stores, warp-shuffle
-// reductions, the row held in registers when it has at most 1024 elements (re-read from cache otherwise).
+// reductions, the row held in registers when it has at most 1024 elements (re-read from cache otherwise).  The
+// backward pass of 16-bit rows of up to 2048 elements shares a row among several warps (ln_bwd_rows_kernel).
 // The variance is taken about the mean (sum of (x - mu)^2), which equals the table's
 // mean(x^2) - mu^2 without its cancellation in float32.
 //
@@ -235,9 +236,9 @@ __global__ void __launch_bounds__(kLnThreads) ln_bwd_kernel(const LnArgs a) {
 }
 
 // ---------------------------------------------------------------- 16-bit inputs, rows in registers
-// The common case (BF16 / F16 activations and gradients, rows of at most 2048 / 1024 elements, aligned)
+// The common case (BF16 / F16 activations and gradients, rows of at most 2048 elements, aligned) of the forward pass
 // gets persistent warps that fetch their next row, still packed, before working on the current one,
-// and read the weight (and bias) from a float32 copy in shared memory.
+// and read the weight (and bias) from a float32 copy in shared memory; the backward pass has two kernels further down.
 
 // Mean and reciprocal standard deviation of a row held as floats (zeros beyond the row's end).
 template <int NCH>
@@ -517,13 +518,13 @@ __device__ __forceinline__ float sum_rows(const float (&v)[4], int lane) { retur
 __device__ __forceinline__ float sum_rows(const float (&v)[1], int) { return warp_sum(v[0]); }
 
 // The 16-bit cases of the backward pass (rows of at most 2048 elements): a row belongs to wpr = cols / 256 warps, eight columns a lane, so
-// that a lane's share of the column sums is 16 registers and three CTAs of eight warps fit an SM; the warps of a row take four rows at
+// that a lane's share of the column sums is 16 registers and two CTAs of eight warps fit an SM; the warps of a row take four rows at
 // a time, which hides the latency of their loads and shares two exchanges through shared memory among four rows: the means, then the
 // sums of (x - mu)^2, g w and g w (x - mu).  B: rows of a turn, four, or one where each group has but one row (300 x 128 4.4 -> 3.9 us, 100 x 512
 // 5.3 -> 4.6: less code to fetch).  G32: the gradient is float32 (the gradient of a layer's output often is) instead of the 16-bit
 // type of X.  XBF: X (and a 16-bit gradient) are BF16 rather than F16.  Bound: latency of the exchanges, 16 warps an SM; beyond L2
-// memory.  us, a warp per row -> this, BF16 with an FP8 copy: 8192 x 1024 22.8 -> 17.9, its float32 gradient 25.6 -> 18.9, 2048 x 768 12.0 -> 7.8, 4096 x
-// 256 8.7 -> 5.6, 256 x 1024 8.9 -> 5.8; 2048 x 2048, which the general kernel took, 65 -> 13.
+// memory.  us, a warp per row -> this, BF16 with an FP8 copy: 8192 x 1024 22.9 -> 18.3, its float32 gradient 25.9 -> 19.0, 2048 x 768 12.2 -> 8.2, 4096 x
+// 256 9.1 -> 5.8, 256 x 1024 9.1 -> 6.3; 2048 x 2048, which the general kernel took, 65 -> 13.
 constexpr int kLnBatch = 4, kLnCtasPerSm = 2;
 enum LnOut { kLnSame = 0, kLnSameE4 = 1, kLnSameE5 = 2, kLnAny = 3, kLnAnyCopy = 4 };   // dX of X's type (and its FP8 copy), or of any type
 template <bool G32, bool XBF, int OUT, int B>
