@@ -56,6 +56,21 @@ def test_shared_contraction_with_a_copy_in_fp8(rows, k, cols):
     assert torch.equal(q.view(torch.uint8), out.float().clamp(-448, 448).to(torch.float8_e4m3fn).view(torch.uint8))
 
 
+def test_waits_that_run_out_in_a_cluster():
+    """Operand loads withheld: every CTA's waits run out, the cluster's barriers are passed all the same, the status says so, and
+    the next call is correct."""
+    from paper_2303_11257_b200 import lib as L, synth
+    for rows, k, cols in ((48, 4096, 1024), (2048, 6400, 1024)):
+        X, W, val, scale = _operands(L, synth, "fwd", rows, k, cols, 83, "e4m3", "e4m3")
+        ws, out = L.new_workspace(), U.empty(rows, cols, "bf16")
+        L.us_test_linear_fwd_starved(X, W, scale, out, ws, 2000)
+        assert L.us_workspace_status(ws) == L.US_ERR_TIMEOUT
+        ws.zero_()
+        L.us_linear_fwd(X, W, scale, out, ws)
+        assert L.us_workspace_status(ws) == 0
+        U.assert_close_stored(out, val, "bf16", TOL * max(1.0, np.abs(val).max() / 4), "after")
+
+
 # Every form: (columns of a tile, CTAs of a pair, shares) on 148 SMs, and a forward call that takes it.
 FORMS = {(64, 1, 2): ("e4m3", 300, 5024, 690), (64, 1, 4): ("e4m3", 48, 4096, 1024), (64, 1, 8): ("bf16", 1, 2576, 16), (128, 1, 2): ("bf16", 500, 6160, 1300),
          (128, 1, 4): ("bf16", 300, 5008, 690), (128, 1, 8): ("e4m3", 128, 32768, 1280), (256, 2, 2): ("e4m3", 2048, 6400, 1024), (256, 2, 4): ("bf16", 1000, 8208, 700)}
